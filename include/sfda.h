@@ -138,8 +138,9 @@ SFDA_API int sfda_forward_partition(int B, int T, int H, int d_k, int d_v, int c
  * chunk size named (they do not depend on where a sequence is cut) at the cost per
  * token of chunk = 64; workspace, partition and slicing rules are those of chunk = 64.
  * bf16 inputs with d_k = d_v = 128 and chunk >= 64 take the tensor-core path
- * (bf16 operands, fp32 accumulation and state); everything else runs in fp32 on
- * the CUDA cores.  The tensor-core path forms 1/gamma_t inside a chunk and so
+ * (bf16 operands, fp32 accumulation and state); everything else runs at fp32
+ * precision (products of operands split into two fp16 parts, 22 bits, summed in
+ * fp32; any alpha in [0, 1]).  The bf16 tensor-core path forms 1/gamma_t inside a chunk and so
  * additionally assumes prod_{t in chunk} alpha_{t,j} >= exp(-80) for every
  * coordinate j; beyond that results lose accuracy but stay finite.
  */
@@ -455,7 +456,7 @@ SFDA_API int sfda_frontend_backward(const float *a_raw, const float *b_raw, cons
  * s = 1 / (|k_raw| + eps), is the recurrence on k_raw with beta s^2 for beta and v / s for v (Eq. "sfda"), and
  * |k_raw|^2 is read off the diagonal of the chunk's Gram matrix, i.e. from the bf16 operands (relative error of
  * s about 2e-4).  |k_raw| + eps below 1e-18 is treated as 1e-18; |k_raw|^2 must be finite in fp32.  The workspace
- * is the one of sfda_forward.  Other shapes run sfda_frontend into the workspace and the CUDA-core forward from
+ * is the one of sfda_forward.  Other shapes run sfda_frontend into the workspace and the fp32 forward from
  * there.  sfda_forward_fused_workspace_bytes gives the size for full speed in
  * both cases (the tensor-core path again runs with as little as 256 bytes; the other shapes need it all).
  */

@@ -243,7 +243,7 @@ int sfda_forward(const void *q, const void *k, const void *v, const float *alpha
         sfda::forward_ws_supported(a)
             ? sfda::launch_forward_ws(a, workspace, workspace_bytes, static_cast<cudaStream_t>(stream),
                                       &g_last_launches)
-            : sfda::launch_forward_simt(a, static_cast<cudaStream_t>(stream), &g_last_launches);
+            : sfda::launch_forward_f32(a, static_cast<cudaStream_t>(stream), &g_last_launches);
     return e == cudaSuccess ? SFDA_OK : SFDA_ERR_CUDA;
 }
 
@@ -672,7 +672,7 @@ int sfda_forward_fused(const void *q, const void *k_raw, const void *v, const fl
     f.alpha_min = alpha_min; f.alpha_max = alpha_max; f.theta_max = theta_max; f.eps = eps;
     if (sfda::launch_frontend(f, s, &g_last_launches) != cudaSuccess) return SFDA_ERR_CUDA;
     a.alpha = f.alpha; a.theta = f.theta; a.beta = f.beta; a.k = f.k;
-    return sfda::launch_forward_simt(a, s, &g_last_launches) == cudaSuccess ? SFDA_OK : SFDA_ERR_CUDA;
+    return sfda::launch_forward_f32(a, s, &g_last_launches) == cudaSuccess ? SFDA_OK : SFDA_ERR_CUDA;
 }
 
 size_t sfda_backward_workspace_bytes(int B, int T, int H, int d_k, int d_v, int dtype)

@@ -1,4 +1,5 @@
-// fp32 CUDA-core chunk-WY forward.
+// fp32 CUDA-core chunk-WY forward: the library's cross-check (sfda_forward_simt); calls for speed take
+// sfda_forward_f32.cu.
 //
 // What is computed per chunk (C tokens, one (batch, head) pair, gamma_t = prod_{s<=t} lambda_s inside
 // the chunk, written gamma_t = a_t e^{i phi_t}):

@@ -91,6 +91,8 @@ struct DecoupledArgs {
 
 // Each returns a cudaError_t from configuring / launching; *launches is incremented per kernel.
 cudaError_t launch_forward_simt(const ForwardArgs &a, cudaStream_t stream, int *launches);
+// fp32 forward on the tensor cores (split fp16 operands), every supported d_k, d_v and dtype.
+cudaError_t launch_forward_f32(const ForwardArgs &a, cudaStream_t stream, int *launches);
 // Tensor-core path (bf16, d_k = d_v = 128, chunk = 64): warp-specialised, chunk-pipelined tcgen05 kernel.
 // `status` is one device word the kernel sets when a bounded wait runs out; it is cleared on the stream
 // before the launch.
