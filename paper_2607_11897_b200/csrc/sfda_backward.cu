@@ -1,86 +1,44 @@
-// sfda_backward: reverse-mode derivative of the recurrence of Section 3 (Eq. "sfda") with o_t = S_t^* q_t, token by
-// token in fp32 on the CUDA cores.  (The paper asks for the backward pass only as something to be timed, App. E; what
-// it computes is the adjoint of Eq. "sfda".)  This is the first correct path: one CTA per (batch, head) pair and
-// block of value columns (the columns of the state and of its cotangent never interact; with many sequences a block
-// is all d_v columns, with few it is 64 or 32 of them so that every SM has work) walks the sequence three times --
+// sfda_backward: reverse-mode derivative of the recurrence of Section 3 (Eq. "sfda") with o_t = S_t^* q_t, chunk by
+// chunk (16 tokens) at fp32 precision on the tensor cores.  (The paper asks for the backward pass only as something to
+// be timed, App. E; what it computes is the adjoint of Eq. "sfda".)  Complex cotangents Xb mean dL = Re sum conj(Xb) dX,
+// i.e. the ordinary gradient with respect to the (Re, Im) pair; yb_t = do_re + i do_im.
 //
-//   1. forward, keeping the state at the start of every segment of kSeg tokens (checkpoints in the workspace);
-//   2. per segment, last to first: forward again from the checkpoint, keeping S_{t-1} of every token of the segment;
-//   3. backward through the segment.
+// Per chunk, with W, Y, Q, M, A^{qk} of sfda_chunk16.cuh, S_0 the state before the chunk and G_C the cotangent of the
+// state after it:
 //
-// The state (sweeps 1, 2) and its cotangent G (sweep 3) live in registers, a tile of rows x columns per thread;
-// S_{t-1} of the backward step arrives from the scratch by cp.async, one token ahead.
+//   forward    U = M (V - W^* S_0)  (rows u_t^T = v_t^T - k_t^* Lambda_t S_{t-1}),   S_C = gamma_C S_0 + Y U
+//   backward   Bc = M^H (Y^* G_C + (A^{qk} D_beta)^H Yb^*)   (rows beta_t p_t^*, p_t = G_t^* k_t),   dv_t = Re Bc_t
+//              G_0 = conj(gamma_C) G_C + Q^T Yb^* - W^T Bc
+//   gradients  dq_t = S_t yb_t,   f_t = G_t conj(u_t),   z_t = Lambda_t S_{t-1} (beta_t p_t),
+//              dk_t = beta_t f_t - z_t,   dbeta_t = Re(f_t^* k_t),
+//              D_t = D_{t+1} + q_t conj(dq_t) - beta_t conj(k_t) f_t - k_t conj(z_t)    (D_{T+1} = rowdot(S_T, G_T)),
+//              dalpha_t = Re D_t / alpha_t,   dtheta_t = Im D_t
 //
-// One backward step, with Z = Lambda_t S_{t-1}, u^T = v_t^T - k_t^* Z (so S_t = Z + beta_t k_t u^T) and
-// yb_t = do_re + i do_im:
+// where S_t, G_t inside a chunk are S_0, G_C plus rank-16 corrections, so dq, f, z come from three products with the
+// boundary matrices (S_0 Yb^T, S_0 B^T, G_C U^H), two 16 x 16 matrices U Yb^T, U B^T and triangular products with the
+// decayed keys and queries.  Where alpha_t < 1/16 the division would lose digits: dalpha comes from its definition,
+// sum_c conj(S_{t-1,jc}) Zb_jc, rebuilt for that (token, coordinate) alone.
 //
-//   G += q yb^*                    p = G^* k                     dv = beta Re p            dbeta = Re(u^T p)
-//   dq = Z yb + beta k (u^T yb)    dk = beta (G conj(u) - Z p)   Zb = G - beta k p^*
-//   lamb_j = sum_c conj(S_{t-1,jc}) Zb_jc      dalpha = Re(conj(lamb) e^{i theta})     dtheta = -Im(conj(lamb) lam)
-//   G <- conj(lam) Zb   (row-wise: the cotangent of S_{t-1})
-//
-// Complex cotangents Xb mean dL = Re sum conj(Xb) dX, i.e. the ordinary gradient with respect to the (Re, Im) pair.
-// dq, dk, dalpha, dtheta, dbeta are sums over the value columns: with more than one column block every block writes
-// its share as fp32 to the workspace and a second kernel adds the shares in a fixed order, so the result is
-// deterministic either way.
-#include "sfda_common.cuh"
+// One CTA per (batch, head) pair and block of value columns (all of them, or with few sequences 64 or 32: the columns
+// never interact, and a second kernel adds the blocks' shares of the sums over the columns in a fixed order).  The
+// CHAIN warps walk the sequence forward once, keeping the state every 64 tokens, then per segment of 64 tokens, last to
+// first: forward again from the checkpoint, backward through it.  They leave S_0, U, G_C, Bc of a chunk in a scratch
+// ring as the operand registers of the gradients' products.  The AUX warps prepare the chunks' operand tiles and turn
+// what the chain leaves into gradients one chunk behind it.  The two meet at hardware barriers, one per slot:
+//   FULL  operand tile ready       DONE  the chain is through with a chunk       FREE  its gradients are written
+#include <type_traits>
+
+#include "sfda_chunk16.cuh"
 #include "sfda_internal.h"
 
 namespace sfda {
 namespace {
 
-constexpr int kBwdThreads = 512;
-constexpr int kSeg = 64;     // tokens between checkpoints
+using namespace c16;
 
-// Thread mapping: warp w owns TR consecutive rows of the (complex) state, lane l owns TC consecutive value columns,
-// so a thread keeps a TR x TC tile of the cotangent G -- and of the state, while a step needs it -- in registers.
-// Sums over rows (per column) cross the warps through shared memory; sums over columns (per row) stay inside a warp.
-template <int DK, int DV>
-struct BwdSmem {
-    static constexpr int M = DK / 2, NW = kBwdThreads / 32;
-    static constexpr int TR = M / NW, TC = DV / 32;
-    static_assert(M % NW == 0 && DV % 32 == 0 && (TC == 1 || TC == 2 || TC == 4), "tile shape");
-    // two buffers of S_{t-1} (interleaved complex [M][DV]), the warps' partial column sums [NW][DV] float4, two
-    // sets of token vectors (row vectors 2 float4 [M], column vectors float2 + float [DV], beta), and the
-    // per-column results of a step (p, u / e: 2 float2 [DV]) with the warps' scalar sums
-    static constexpr int state = M * DV * 2;                           // floats
-    static constexpr int tokvec = 8 * M + 3 * DV + 4;                  // floats, one set
-    static constexpr size_t bytes = (size_t)(2 * state + NW * DV * 4 + 2 * tokvec + 4 * DV + 64) * 4;
-};
-
-__device__ __forceinline__ void cp_async16(float *dst_smem, const float *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst_smem)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// N consecutive float2 (N = 1, 2, 4) with the widest accesses; p is aligned to 8 N bytes (16 for N = 4)
-template <int N>
-__device__ __forceinline__ void ld_row(const float2 *p, float2 (&x)[N])
-{
-    if constexpr (N == 1) {
-        x[0] = *p;
-    } else {
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i) {
-            const float4 t = reinterpret_cast<const float4 *>(p)[i];
-            x[2 * i] = make_float2(t.x, t.y);
-            x[2 * i + 1] = make_float2(t.z, t.w);
-        }
-    }
-}
-template <int N>
-__device__ __forceinline__ void st_row(float2 *p, const float2 (&x)[N])
-{
-    if constexpr (N == 1) {
-        *p = x[0];
-    } else {
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i)
-            reinterpret_cast<float4 *>(p)[i] = make_float4(x[2 * i].x, x[2 * i].y, x[2 * i + 1].x, x[2 * i + 1].y);
-    }
-}
+constexpr int kSeg = 64;                    // tokens between checkpoints
+constexpr int kSegChunks = kSeg / kC;
+static_assert(kSegChunks == kSlots, "a segment's operand tiles fill the ring");
 
 struct BwdArgsDev {
     const void *q, *k, *v, *d_o, *d_o_im;
@@ -88,375 +46,99 @@ struct BwdArgsDev {
     void *dq, *dk, *dv;
     float *dalpha, *dtheta, *dbeta, *dS0;
     float *dq_p, *dk_p, *dalpha_p, *dtheta_p, *dbeta_p;   // shares of the column blocks: [blocks][rows][...] fp32
-    float *check, *scratch;      // [BH][blocks][NS][M][cols][2], [BH][blocks][kSeg][M][cols][2] (interleaved complex)
-    size_t rows;                 // B * T * H
+    float *check, *scratch;
+    size_t rows;
     int T, H, NS;
 };
 
-// DVT value columns per state, DV of them per CTA
-template <int DK, int DVT, int DV, typename T>
-__global__ void __launch_bounds__(kBwdThreads, 1)
-sfda_backward_kernel(const BwdArgsDev a)
+// One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
+// S_0, G_C as B operands [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U, Bc as A operands
+// [chain warp][plane][lane] uint4; then the chunk's rotated keys and queries, decays and phases, 8 floats per
+// (token, key).
+template <int DK, int NB>
+struct BwdScratch {
+    static constexpr int NCW = NB / 16, KT = DK / 16, M = DK / 2;
+    static constexpr int oS = 0, oU = oS + NCW * KT * 1024, oG = oU + NCW * 2048, oB = oG + NCW * KT * 1024;
+    static constexpr int oV = oB + NCW * 2048, slot = oV + 16 * M * 32;
+    static_assert((size_t)slot * kSlots <= (size_t)kSeg * DK * NB * 4, "the scratch ring must fit the workspace");
+};
+
+template <int DK, int NB>
+struct BwdSmem {
+    static constexpr int NCW = NB / 16, M = DK / 2;
+    static constexpr int frag_bytes = 3 * NCW * 2048;             // Yb, Bc, U of the chunk as A operands
+    static constexpr int stage = kSlots * Tile<DK>::bytes;        // PREP's staging and the gradients' operands share a place
+    static constexpr int stage_bytes = frag_bytes > PrepSmem<DK>::stage_bytes ? frag_bytes : PrepSmem<DK>::stage_bytes;
+    static constexpr int small = stage + stage_bytes;
+    static constexpr int tri = small + PrepSmem<DK>::small_bytes; // the triangular factors of the corrections, 8 x 4 uint4 [32]
+    static constexpr int uy = tri + 8 * 4 * 512;                  // U Yb^T, U B^T: float2 [2][16][17]
+    static constexpr int scal = uy + 2 * 16 * 17 * 8;             // inverse scales [slot][NCW] (S, U, G, B), [NCW] Yb
+    static constexpr int rg = scal + kSlots * NCW * 16 + NCW * 4 + (16 - NCW * 4 % 16) % 16;   // rowdot(S, G): float2 [2][NCW][M]
+    static constexpr int db = rg + 2 * NCW * M * 8;               // dbeta: [8][16] floats
+    static constexpr int flag = db + 8 * 16 * 4;                  // fast flag per slot
+    static constexpr int bytes = flag + 16;
+};
+
+__device__ __forceinline__ int ring_slot(int r, int c) { return (r & 1) ? kSlots - 1 - c : c; }
+
+// d += a (bh + bl); the head of `a` alone where its values are exact in fp16 (kExact)
+template <bool kExact>
+__device__ __forceinline__ void mma3x(float (&d)[4], const uint32_t (&ah)[4], const uint32_t (&al)[4], uint32_t bh0,
+                                      uint32_t bh1, uint32_t bl0, uint32_t bl1)
 {
-    constexpr int NSL = DVT / DV;                  // column blocks per state
-    static_assert(DVT % DV == 0, "the value columns split into equal blocks");
-    using L = BwdSmem<DK, DV>;
-    constexpr int M = L::M, NW = L::NW, TR = L::TR, TC = L::TC;
-    static_assert(M + DV + 1 <= kBwdThreads, "one thread per staged value");
-    extern __shared__ __align__(16) float sm[];
-    float2 *const Sbuf0 = reinterpret_cast<float2 *>(sm);                        // S_{t-1}, two buffers [M][DV]
-    float4 *const red = reinterpret_cast<float4 *>(sm + 2 * L::state);           // [NW][DV] partial column sums
-    float *const tok0 = sm + 2 * L::state + NW * DV * 4;                         // two sets of token vectors
-    float2 *const v_p = reinterpret_cast<float2 *>(tok0 + 2 * L::tokvec);        // p per column (backward)
-    float2 *const v_u = v_p + DV;                                                // u (backward) / e = beta u (forward)
-    float *const scal = reinterpret_cast<float *>(v_u + DV);                     // [4 w + x]: scalar sums of warp w
-    auto Sbuf = [&](int i) { return Sbuf0 + i * (M * DV); };
-    // token vectors of set i: per row (lam re, lam im, k re, k im), (q re, q im, cos theta, sin theta); per column
-    // yb (re, im) and v; beta
-    auto t_lk = [&](int i) { return reinterpret_cast<float4 *>(tok0 + i * L::tokvec); };
-    auto t_qc = [&](int i) { return reinterpret_cast<float4 *>(tok0 + i * L::tokvec) + M; };
-    auto t_y = [&](int i) { return reinterpret_cast<float2 *>(tok0 + i * L::tokvec + 8 * M); };
-    auto t_v = [&](int i) { return tok0 + i * L::tokvec + 8 * M + 2 * DV; };
-    auto t_beta = [&](int i) { return tok0 + i * L::tokvec + 8 * M + 3 * DV; };
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bh = blockIdx.x, h = bh % a.H, b = bh / a.H, slice = blockIdx.y, c0 = slice * DV;
-    const int T_ = a.T, H = a.H;
-    const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k), *v = static_cast<const T *>(a.v);
-    const T *d_o = static_cast<const T *>(a.d_o), *d_oi = static_cast<const T *>(a.d_o_im);
-    float *check = a.check + ((size_t)bh * NSL + slice) * a.NS * 2 * M * DV;
-    float *scratch = a.scratch + ((size_t)bh * NSL + slice) * kSeg * 2 * M * DV;
-    const int j0 = warp * TR, cl = lane * TC;      // this thread's tile: rows j0 + r, columns cl + x
-
-    // ---- token vectors: global -> registers (issued a step ahead) -> one of the two sets in shared memory
-    // (staged by the last M + DV + 1 threads: the first DV are the ones that reduce the column sums meanwhile)
-    const int sid = kBwdThreads - 1 - tid;
-    float r0 = 0.f, r1 = 0.f, r2 = 0.f, r3 = 0.f, r4 = 0.f, r5 = 0.f;
-    auto load_tok = [&](int t, bool back) {
-        if (t < 0 || t >= T_) return;
-        const size_t row = ((size_t)b * T_ + t) * H + h;
-        if (sid < M) {
-            r0 = a.alpha[row * M + sid];
-            r1 = a.theta[row * M + sid];
-            r2 = ld_val(k, row * DK + 2 * sid);
-            r3 = ld_val(k, row * DK + 2 * sid + 1);
-            if (back) {
-                r4 = ld_val(q, row * DK + 2 * sid);
-                r5 = ld_val(q, row * DK + 2 * sid + 1);
-            }
-        } else if (sid < M + DV) {
-            const int cc = sid - M;
-            r0 = ld_val(v, row * DVT + c0 + cc);
-            if (back) {
-                r1 = ld_val(d_o, row * DVT + c0 + cc);
-                r2 = d_oi ? ld_val(d_oi, row * DVT + c0 + cc) : 0.f;
-            }
-        } else if (sid == M + DV) {
-            r0 = a.beta[row];
-        }
-    };
-    auto stage_tok = [&](int set, bool back) {
-        if (sid < M) {
-            float sn, cs;
-            sincosf(r1, &sn, &cs);
-            t_lk(set)[sid] = make_float4(r0 * cs, r0 * sn, r2, r3);
-            if (back) t_qc(set)[sid] = make_float4(r4, r5, cs, sn);
-        } else if (sid < M + DV) {
-            const int cc = sid - M;
-            t_v(set)[cc] = r0;
-            if (back) t_y(set)[cc] = make_float2(r1, r2);
-        } else if (sid == M + DV) {
-            t_beta(set)[0] = r0;
-        }
-    };
-
-    // ---- one forward step on the tile s (registers).  Set `set` holds the token's vectors (visible to all); the
-    // next token's vectors, already in registers, are staged into the other set on the way.
-    auto fwd_step = [&](float2 (&s)[TR][TC], int set, bool stage_next) {
-        const float4 *lkv = t_lk(set);
-        float2 kz[TC];
+    if constexpr (!kExact) mma_f16(d, al, bh0, bh1);
+    mma_f16(d, ah, bl0, bl1);
+    mma_f16(d, ah, bh0, bh1);
+}
+template <bool kExact>
+__device__ __forceinline__ void product_small_conj(float (&re)[2][4], float (&im)[2][4], const TokFrag &a, const TokFrag &b,
+                                                   float f, bool has_im)
+{
 #pragma unroll
-        for (int x = 0; x < TC; ++x) kz[x] = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int r = 0; r < TR; ++r) {
-            const float4 lk = lkv[j0 + r];
-#pragma unroll
-            for (int x = 0; x < TC; ++x) {
-                const float zr = lk.x * s[r][x].x - lk.y * s[r][x].y, zi = lk.x * s[r][x].y + lk.y * s[r][x].x;   // Z = Lambda S
-                s[r][x] = make_float2(zr, zi);
-                kz[x].x += lk.z * zr + lk.w * zi;                                  // conj(k) z
-                kz[x].y += lk.z * zi - lk.w * zr;
-            }
+    for (int n = 0; n < 2; ++n) {
+        float rr[4] = {0.f, 0.f, 0.f, 0.f}, ir[4] = {0.f, 0.f, 0.f, 0.f}, ri[4] = {0.f, 0.f, 0.f, 0.f};
+        mma3x<kExact>(rr, a.rh, a.rl, b.rh[2 * n], b.rh[2 * n + 1], b.rl[2 * n], b.rl[2 * n + 1]);
+        mma3x<kExact>(ri, a.rh, a.rl, b.ih[2 * n], b.ih[2 * n + 1], b.il[2 * n], b.il[2 * n + 1]);
+        if (has_im) {
+            mma3x<kExact>(rr, a.ih, a.il, b.ih[2 * n], b.ih[2 * n + 1], b.il[2 * n], b.il[2 * n + 1]);
+            mma3x<kExact>(ir, a.ih, a.il, b.rh[2 * n], b.rh[2 * n + 1], b.rl[2 * n], b.rl[2 * n + 1]);
         }
 #pragma unroll
-        for (int x = 0; x < TC; ++x) reinterpret_cast<float2 *>(red)[(warp * TC + x) * 32 + lane] = kz[x];
-        __syncthreads();
-        if (tid < DV) {                     // warp x' of these sums column x' of every lane's tile
-            const int c = lane * TC + warp;
-            float sr_ = 0.f, si_ = 0.f;
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                const float2 x = reinterpret_cast<const float2 *>(red)[(w * TC + warp) * 32 + lane];
-                sr_ += x.x;
-                si_ += x.y;
-            }
-            const float bt = t_beta(set)[0];
-            v_u[c] = make_float2(bt * (t_v(set)[c] - sr_), -bt * si_);              // e = beta u, u = v - k^* Z
-        }
-        if (stage_next) stage_tok(set ^ 1, false);
-        __syncthreads();
-        float2 e[TC];
-        ld_row<TC>(v_u + cl, e);
-#pragma unroll
-        for (int r = 0; r < TR; ++r) {
-            const float4 lk = lkv[j0 + r];
-#pragma unroll
-            for (int x = 0; x < TC; ++x) {
-                s[r][x].x += lk.z * e[x].x - lk.w * e[x].y;
-                s[r][x].y += lk.z * e[x].y + lk.w * e[x].x;
-            }
-        }
-    };
-
-    // ---- a tile between registers and global memory (workspace format: interleaved complex [M][DV])
-    auto store_tile = [&](const float2 (&s)[TR][TC], float *dst) {
-#pragma unroll
-        for (int r = 0; r < TR; ++r) st_row<TC>(reinterpret_cast<float2 *>(dst) + (size_t)(j0 + r) * DV + cl, s[r]);
-    };
-    auto load_tile = [&](float2 (&s)[TR][TC], const float *src) {
-#pragma unroll
-        for (int r = 0; r < TR; ++r) ld_row<TC>(reinterpret_cast<const float2 *>(src) + (size_t)(j0 + r) * DV + cl, s[r]);
-    };
-    auto load_state_async = [&](float2 *S, const float *src) {
-        for (int idx = tid; idx < M * DV / 2; idx += kBwdThreads) cp_async16(reinterpret_cast<float *>(S) + 4 * idx, src + 4 * idx);
-        cp_async_commit();
-    };
-
-    // ---- sweep 1: forward, checkpoints at the start of every segment (nothing is needed beyond the last one)
-    float2 s[TR][TC];
-#pragma unroll
-    for (int r = 0; r < TR; ++r)
-#pragma unroll
-        for (int x = 0; x < TC; ++x) {
-            const size_t at = ((size_t)bh * DK + 2 * (j0 + r)) * DVT + c0 + cl + x;
-            s[r][x] = a.S0 ? make_float2(a.S0[at], a.S0[at + DVT]) : make_float2(0.f, 0.f);
-        }
-    const int t_last_check = (a.NS - 1) * kSeg;
-    int set = 0;
-    load_tok(0, false);
-    stage_tok(set, false);
-    __syncthreads();
-    for (int t = 0; t < t_last_check; ++t) {
-        if (t % kSeg == 0) store_tile(s, check + (size_t)(t / kSeg) * 2 * M * DV);
-        load_tok(t + 1, false);
-        fwd_step(s, set, true);
-        set ^= 1;
-    }
-    store_tile(s, check + (size_t)(a.NS - 1) * 2 * M * DV);
-
-    // ---- cotangent of the final state
-    float2 G[TR][TC];
-#pragma unroll
-    for (int r = 0; r < TR; ++r)
-#pragma unroll
-        for (int x = 0; x < TC; ++x) {
-            const size_t at = ((size_t)bh * DK + 2 * (j0 + r)) * DVT + c0 + cl + x;
-            G[r][x] = a.dS_T ? make_float2(a.dS_T[at], a.dS_T[at + DVT]) : make_float2(0.f, 0.f);
-        }
-
-    T *dq = static_cast<T *>(a.dq), *dk = static_cast<T *>(a.dk), *dv = static_cast<T *>(a.dv);
-    float *dq_p = a.dq_p + (size_t)slice * a.rows * DK, *dk_p = a.dk_p + (size_t)slice * a.rows * DK;
-    float *dal_p = a.dalpha_p + (size_t)slice * a.rows * M, *dth_p = a.dtheta_p + (size_t)slice * a.rows * M;
-    float *dbe_p = a.dbeta_p + (size_t)slice * a.rows;
-    for (int si = a.NS - 1; si >= 0; --si) {
-        const int t0 = si * kSeg, t1 = min(t0 + kSeg, T_);
-        // ---- sweep 2: forward again from the checkpoint (this thread wrote the tile it reads), S_{t-1} of every
-        // token to the scratch
-        __syncthreads();                  // every reader of the token vectors and of v_u is done
-        load_tile(s, check + (size_t)si * 2 * M * DV);
-        set = 0;
-        load_tok(t0, false);
-        stage_tok(set, false);
-        __syncthreads();
-        for (int t = t0; t < t1; ++t) {
-            store_tile(s, scratch + (size_t)(t - t0) * 2 * M * DV);
-            if (t + 1 < t1) {                                   // the state after the last token is not needed
-                load_tok(t + 1, false);
-                fwd_step(s, set, true);
-                set ^= 1;
-            }
-        }
-        __syncthreads();      // the scratch stores of this CTA are visible to its own later loads
-
-        // ---- sweep 3: backward through the segment; S_{t-1} arrives one token ahead in the other buffer
-        int buf = 0;
-        set = 0;
-        load_state_async(Sbuf(buf), scratch + (size_t)(t1 - 1 - t0) * 2 * M * DV);
-        load_tok(t1 - 1, true);
-        stage_tok(set, true);
-        cp_async_wait_all();
-        __syncthreads();
-        for (int t = t1 - 1; t >= t0; --t) {
-            if (t > t0) {
-                load_state_async(Sbuf(buf ^ 1), scratch + (size_t)(t - 1 - t0) * 2 * M * DV);
-                load_tok(t - 1, true);
-            }
-            const float4 *lkv = t_lk(set), *qcv = t_qc(set);
-            const float bt = t_beta(set)[0];
-            const size_t row = ((size_t)b * T_ + t) * H + h;
-            float2 y[TC];
-            ld_row<TC>(t_y(set) + cl, y);
-
-            // step 1: G += q yb^*; partial sums over this warp's rows of p = G^* k and k^* Z
-            {
-                float4 acc[TC];
-#pragma unroll
-                for (int x = 0; x < TC; ++x) acc[x] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int r = 0; r < TR; ++r) {
-                    const float4 lk = lkv[j0 + r], qc = qcv[j0 + r];
-                    ld_row<TC>(Sbuf(buf) + (j0 + r) * DV + cl, s[r]);
-#pragma unroll
-                    for (int x = 0; x < TC; ++x) {
-                        const float gr = G[r][x].x + qc.x * y[x].x + qc.y * y[x].y;          // G + q conj(yb)
-                        const float gi = G[r][x].y + qc.y * y[x].x - qc.x * y[x].y;
-                        G[r][x] = make_float2(gr, gi);
-                        acc[x].x += gr * lk.z + gi * lk.w;                                  // conj(G) k
-                        acc[x].y += gr * lk.w - gi * lk.z;
-                        const float zr = lk.x * s[r][x].x - lk.y * s[r][x].y, zi = lk.x * s[r][x].y + lk.y * s[r][x].x;
-                        acc[x].z += lk.z * zr + lk.w * zi;                                  // conj(k) z
-                        acc[x].w += lk.z * zi - lk.w * zr;
-                    }
-                }
-#pragma unroll
-                for (int x = 0; x < TC; ++x) red[(warp * TC + x) * 32 + lane] = acc[x];     // [warp][x][lane]: no bank conflicts
-            }
-            __syncthreads();
-            // step 2: p, u per column; dv; the sums over columns u^T p and u^T yb (one set per warp of columns)
-            if (tid < DV) {                 // warp x' of these sums column x' of every lane's tile
-                const int c = lane * TC + warp;
-                float pr = 0.f, pi = 0.f, zr = 0.f, zi = 0.f;
-#pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    const float4 x = red[(w * TC + warp) * 32 + lane];
-                    pr += x.x;  pi += x.y;  zr += x.z;  zi += x.w;
-                }
-                const float ur = t_v(set)[c] - zr, ui = -zi;
-                const float2 yy = t_y(set)[c];
-                v_p[c] = make_float2(pr, pi);
-                v_u[c] = make_float2(ur, ui);
-                st_val(dv, row * DVT + c0 + c, bt * pr);
-                float s0 = ur * pr - ui * pi;                                   // Re(u p)
-                float s1 = ur * yy.x - ui * yy.y, s2 = ur * yy.y + ui * yy.x;   // u yb
-#pragma unroll
-                for (int d = 16; d >= 1; d >>= 1) {
-                    s0 += __shfl_xor_sync(0xffffffffu, s0, d);
-                    s1 += __shfl_xor_sync(0xffffffffu, s1, d);
-                    s2 += __shfl_xor_sync(0xffffffffu, s2, d);
-                }
-                if (lane == 0) { scal[4 * warp] = s0; scal[4 * warp + 1] = s1; scal[4 * warp + 2] = s2; }
-            }
-            if (t > t0) stage_tok(set ^ 1, true);
-            cp_async_wait_all();
-            __syncthreads();
-            // step 3: this warp's rows: shares of dq, dk, dalpha, dtheta; G <- conj(lam) (G - beta k p^*)
-            {
-                float uy_r = 0.f, uy_i = 0.f, dbe = 0.f;
-#pragma unroll
-                for (int w = 0; w < DV / 32; ++w) { dbe += scal[4 * w]; uy_r += scal[4 * w + 1]; uy_i += scal[4 * w + 2]; }
-                if (tid == 0) (NSL == 1 ? a.dbeta : dbe_p)[row] = dbe;
-                float2 pp[TC], uu[TC];
-                ld_row<TC>(v_p + cl, pp);
-                ld_row<TC>(v_u + cl, uu);
-                // per row: dq re, im; dk re, im (before the factor beta); dalpha; dtheta; two unused
-                constexpr int NV = 8 * TR;
-                float val[NV];
-#pragma unroll
-                for (int r = 0; r < TR; ++r) {
-                    const float4 lk = lkv[j0 + r], qc = qcv[j0 + r];
-                    const float lr = lk.x, li = lk.y, kr = lk.z, ki = lk.w;
-                    float qzr = 0.f, qzi = 0.f, dkr = 0.f, dki = 0.f, lbr = 0.f, lbi = 0.f;
-#pragma unroll
-                    for (int x = 0; x < TC; ++x) {
-                        const float gr = G[r][x].x, gi = G[r][x].y, sr = s[r][x].x, si2 = s[r][x].y;
-                        const float yr = y[x].x, yi = y[x].y, ur = uu[x].x, ui = uu[x].y, pr = pp[x].x, pi = pp[x].y;
-                        const float zr = lr * sr - li * si2, zi = lr * si2 + li * sr;
-                        qzr += zr * yr - zi * yi;  qzi += zr * yi + zi * yr;                 // Z yb
-                        dkr += gr * ur + gi * ui - (zr * pr - zi * pi);                      // G conj(u) - Z p
-                        dki += gi * ur - gr * ui - (zr * pi + zi * pr);
-                        // Zb = G - beta k conj(p)
-                        const float br = gr - bt * (kr * pr + ki * pi), bi = gi - bt * (ki * pr - kr * pi);
-                        lbr += sr * br + si2 * bi;  lbi += sr * bi - si2 * br;               // conj(S_{t-1}) Zb
-                        G[r][x] = make_float2(lr * br + li * bi, lr * bi - li * br);         // conj(lam) Zb
-                    }
-                    val[8 * r + 0] = qzr;
-                    val[8 * r + 1] = qzi;
-                    val[8 * r + 2] = bt * dkr;
-                    val[8 * r + 3] = bt * dki;
-                    val[8 * r + 4] = lbr * qc.z + lbi * qc.w;                                // Re(conj(lamb) e^{i theta})
-                    val[8 * r + 5] = lbi * lr - lbr * li;                                    // -Im(conj(lamb) lam)
-                    val[8 * r + 6] = 0.f;
-                    val[8 * r + 7] = 0.f;
-                }
-                // sums over the warp's lanes (= columns): every exchange halves the values a lane still carries, so
-                // that lane l ends with the total of value l (NV = 32) or l / 2 (NV = 16)
-                int n = NV;
-#pragma unroll
-                for (int d = 16; d >= 1; d >>= 1) {
-                    if (n > 1) {
-                        const int half = n / 2;
-                        const bool up = (lane & d) != 0;
-#pragma unroll
-                        for (int i = 0; i < NV / 2; ++i) {
-                            if (i < half) {
-                                const float send = up ? val[i] : val[i + half];
-                                const float keep = up ? val[i + half] : val[i];
-                                val[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
-                            }
-                        }
-                        n = half;
-                    } else {
-                        val[0] += __shfl_xor_sync(0xffffffffu, val[0], d);
-                    }
-                }
-                const int vi = NV == 32 ? lane : lane >> 1;
-                const int rr = vi >> 3, qq = vi & 7, j = j0 + rr;
-                if (qq < 6 && (NV == 32 || !(lane & 1))) {
-                    float out = val[0];
-                    if (qq < 2) {
-                        const float4 lk = lkv[j];
-                        out += qq == 0 ? bt * (lk.z * uy_r - lk.w * uy_i) : bt * (lk.z * uy_i + lk.w * uy_r);   // + beta k (u^T yb)
-                    }
-                    if constexpr (NSL == 1) {
-                        if (qq < 2) st_val(dq, row * DK + 2 * j + qq, out);
-                        else if (qq < 4) st_val(dk, row * DK + 2 * j + qq - 2, out);
-                        else if (qq == 4) a.dalpha[row * M + j] = out;
-                        else a.dtheta[row * M + j] = out;
-                    } else {      // this column block's share of the sums over the columns
-                        if (qq < 2) dq_p[row * DK + 2 * j + qq] = out;
-                        else if (qq < 4) dk_p[row * DK + 2 * j + qq - 2] = out;
-                        else if (qq == 4) dal_p[row * M + j] = out;
-                        else dth_p[row * M + j] = out;
-                    }
-                }
-            }
-            buf ^= 1;
-            set ^= 1;
+        for (int i = 0; i < 4; ++i) {
+            re[n][i] = fmaf(f, rr[i], re[n][i]);
+            im[n][i] = fmaf(f, ir[i] - ri[i], im[n][i]);
         }
     }
-#pragma unroll
-    for (int r = 0; r < TR; ++r)
-#pragma unroll
-        for (int x = 0; x < TC; ++x) {
-            const size_t at = ((size_t)bh * DK + 2 * (j0 + r)) * DVT + c0 + cl + x;
-            a.dS0[at] = G[r][x].x;
-            a.dS0[at + DVT] = G[r][x].y;
-        }
 }
 
-// ---- the sums over the column blocks: out[i] = share_0[i] + share_1[i] + ... in that order, one thread per four
-// consecutive elements.  HBM-bound and small beside the sweeps.
-constexpr int kSumThreads = 256;
+// the [value x token] operand as the A operand (token, value) of products over the value columns
+__device__ __forceinline__ void publish_frag(uint4 *p, const TokFrag &f, int lane)
+{
+    p[0 * 32 + lane] = make_uint4(transpose8x8(f.rh[0]), transpose8x8(f.rh[2]), transpose8x8(f.rh[1]), transpose8x8(f.rh[3]));
+    p[1 * 32 + lane] = make_uint4(transpose8x8(f.rl[0]), transpose8x8(f.rl[2]), transpose8x8(f.rl[1]), transpose8x8(f.rl[3]));
+    p[2 * 32 + lane] = make_uint4(transpose8x8(f.ih[0]), transpose8x8(f.ih[2]), transpose8x8(f.ih[1]), transpose8x8(f.ih[3]));
+    p[3 * 32 + lane] = make_uint4(transpose8x8(f.il[0]), transpose8x8(f.il[2]), transpose8x8(f.il[1]), transpose8x8(f.il[3]));
+}
+
+template <int KT>
+__device__ __forceinline__ void store_state(float4 *p, const float (&sr)[KT][4], const float (&si)[KT][4], int lane)
+{
+#pragma unroll
+    for (int n = 0; n < KT; ++n) {
+        p[(2 * n) * 32 + lane] = make_float4(sr[n][0], sr[n][1], sr[n][2], sr[n][3]);
+        p[(2 * n + 1) * 32 + lane] = make_float4(si[n][0], si[n][1], si[n][2], si[n][3]);
+    }
+}
+template <int KT>
+__device__ __forceinline__ void load_state(const float4 *p, float (&sr)[KT][4], float (&si)[KT][4], int lane)
+{
+#pragma unroll
+    for (int n = 0; n < KT; ++n) {
+        const float4 x = p[(2 * n) * 32 + lane], y = p[(2 * n + 1) * 32 + lane];
+        sr[n][0] = x.x; sr[n][1] = x.y; sr[n][2] = x.z; sr[n][3] = x.w;
+        si[n][0] = y.x; si[n][1] = y.y; si[n][2] = y.z; si[n][3] = y.w;
+    }
+}
 
 __device__ __forceinline__ void st_val4(float *p, float4 x) { *reinterpret_cast<float4 *>(p) = x; }
 __device__ __forceinline__ void st_val4(__nv_bfloat16 *p, float4 x)
@@ -464,6 +146,697 @@ __device__ __forceinline__ void st_val4(__nv_bfloat16 *p, float4 x)
     const __nv_bfloat162 lo = __floats2bfloat162_rn(x.x, x.y), hi = __floats2bfloat162_rn(x.z, x.w);
     *reinterpret_cast<uint2 *>(p) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
 }
+
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
+__device__ __forceinline__ float2 cmulc(float2 a, float2 b) { return make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }   // conj(a) b
+
+// one 16-bit half of the head and of the tail, added
+__device__ __forceinline__ float join_half(uint32_t h, uint32_t l, int half)
+{
+    const float2 x = unpack_f16(h), y = unpack_f16(l);
+    return half ? x.y + y.y : x.x + y.x;
+}
+
+// ---- AUX: the gradients of one chunk --------------------------------------------------------------
+template <int DK, int DVT, int NB, typename T>
+__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, int slot, int rpar,
+                                             bool first, int t0, size_t row0, float2 (&carry)[2], int tid)
+{
+    using L = BwdSmem<DK, NB>;
+    using SC = BwdScratch<DK, NB>;
+    constexpr int NCW = L::NCW, M = L::M, KT = M / 8, NSL = DVT / NB;
+    constexpr bool kExact = sizeof(T) == 2;
+    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3, c0 = blockIdx.y * NB;
+    const bool has_im = a.d_o_im != nullptr;
+    uint4 *frag = reinterpret_cast<uint4 *>(smem + L::stage);                     // [Yb, Bc, U][NCW][4][32]
+    uint4 *tri = reinterpret_cast<uint4 *>(smem + L::tri);
+    float2 *uy = reinterpret_cast<float2 *>(smem + L::uy);
+    float *scal = reinterpret_cast<float *>(smem + L::scal), *yscal = scal + kSlots * NCW * 4;
+    const float *sc = scal + slot * NCW * 4;
+    float *db = reinterpret_cast<float *>(smem + L::db);
+    const uint4 *pS = reinterpret_cast<const uint4 *>(scr + SC::oS), *pG = reinterpret_cast<const uint4 *>(scr + SC::oG);
+    const float4 *vals = reinterpret_cast<const float4 *>(scr + SC::oV);
+
+    // operands over the value columns: Yb from the caller's arrays, Bc and U from the ring
+    for (int w = warp; w < NCW; w += kAuxWarps) {
+        float2 y[2][4];
+        uint32_t m = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int t = t0 + g + 8 * (i & 1);
+            y[0][i] = y[1][i] = make_float2(0.f, 0.f);
+            if (t < a.T) {
+                const size_t at = (row0 + (size_t)t * a.H) * DVT + c0 + 16 * w + 2 * t4 + 8 * (i >> 1);
+                y[0][i] = ld_pair(static_cast<const T *>(a.d_o), at);
+                if (has_im) y[1][i] = ld_pair(static_cast<const T *>(a.d_o_im), at);
+            }
+            m = max(m, max(max(abs_bits(y[0][i].x), abs_bits(y[0][i].y)), max(abs_bits(y[1][i].x), abs_bits(y[1][i].y))));
+        }
+        const uint4 *pB = reinterpret_cast<const uint4 *>(scr + SC::oB) + w * 128, *pU = reinterpret_cast<const uint4 *>(scr + SC::oU) + w * 128;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            frag[((NCW + w) * 4 + p) * 32 + lane] = pB[p * 32 + lane];
+            frag[((2 * NCW + w) * 4 + p) * 32 + lane] = pU[p * 32 + lane];
+        }
+        float inv;
+        const float s = scale_for(__reduce_max_sync(0xffffffffu, m), inv);
+        if (lane == 0) yscal[w] = inv;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            uint32_t h[4], l[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) split_f16(y[c][i].x * s, y[c][i].y * s, h[i], l[i]);
+            frag[(w * 4 + 2 * c) * 32 + lane] = make_uint4(h[0], h[1], h[2], h[3]);
+            frag[(w * 4 + 2 * c + 1) * 32 + lane] = make_uint4(l[0], l[1], l[2], l[3]);
+        }
+    }
+    bar_sync(kBarAux, kAux);
+
+    // U Yb^T (index [i][t]: u_i . yb_t) and U B^T (b_t = beta_t p_t = conj of the rows of Bc): warp = (matrix, half of
+    // the columns, Re / Im); the A-operand registers of tokens 0-7 / 8-15 are the B operand of that half
+    {
+        const int mat = warp & 1, nt = (warp >> 1) & 1, part = warp >> 2;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        const float sx = (mat && part) ? -1.f : 1.f, sz = (!mat && !part) ? -1.f : 1.f;
+#pragma unroll 2
+        for (int w = 0; w < NCW; ++w) {
+            const uint4 *fu = frag + (2 * NCW + w) * 128 + lane, *fx = frag + (mat * NCW + w) * 128 + lane;
+            const uint4 urh = fu[0], url = fu[32], uih = fu[64], uil = fu[96];
+            const uint4 xh = fx[part * 64], xl = fx[part * 64 + 32], zh = fx[64 - part * 64], zl = fx[96 - part * 64];
+            const uint32_t ar[4] = {urh.x, urh.y, urh.z, urh.w}, arl[4] = {url.x, url.y, url.z, url.w};
+            const uint32_t ai[4] = {uih.x, uih.y, uih.z, uih.w}, ail[4] = {uil.x, uil.y, uil.z, uil.w};
+            float p[4] = {0.f, 0.f, 0.f, 0.f}, z[4] = {0.f, 0.f, 0.f, 0.f};
+            mma3(p, ar, arl, nt ? xh.y : xh.x, nt ? xh.w : xh.z, nt ? xl.y : xl.x, nt ? xl.w : xl.z);
+            mma3(z, ai, ail, nt ? zh.y : zh.x, nt ? zh.w : zh.z, nt ? zl.y : zl.x, nt ? zl.w : zl.z);
+            const float f = sc[4 * w + 1] * (mat ? sc[4 * w + 3] : yscal[w]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] = fmaf(f, fmaf(sx, p[i], sz * z[i]), acc[i]);
+        }
+        float *dst = reinterpret_cast<float *>(uy + mat * 16 * 17) + part;
+        const int t = 8 * nt + 2 * t4;
+        dst[2 * (g * 17 + t)] = acc[0];
+        dst[2 * (g * 17 + t + 1)] = acc[1];
+        dst[2 * ((g + 8) * 17 + t)] = acc[2];
+        dst[2 * ((g + 8) * 17 + t + 1)] = acc[3];
+    }
+
+    // X1 = S_0 yb_t, X2 = S_0 b_t, X3 = G_C conj(u_t) for the keys of tile `warp` (accumulator layout: token g (+ 8),
+    // keys 2 t4, + 1); every chain warp's 16 columns come with scales of their own
+    float x1r[4] = {0.f, 0.f, 0.f, 0.f}, x1i[4] = {0.f, 0.f, 0.f, 0.f}, x2r[4] = {0.f, 0.f, 0.f, 0.f};
+    float x2i[4] = {0.f, 0.f, 0.f, 0.f}, x3r[4] = {0.f, 0.f, 0.f, 0.f}, x3i[4] = {0.f, 0.f, 0.f, 0.f};
+    if (warp < KT) {
+#pragma unroll 1
+        for (int w = 0; w < NCW; ++w) {
+            const uint4 s0 = pS[((w * KT + warp) * 2) * 32 + lane], s1 = pS[((w * KT + warp) * 2 + 1) * 32 + lane];
+            const uint4 g0 = pG[((w * KT + warp) * 2) * 32 + lane], g1 = pG[((w * KT + warp) * 2 + 1) * 32 + lane];
+            {
+                const uint4 *fy = frag + w * 128 + lane;
+                const uint4 h = fy[0], l = fy[32];
+                const uint32_t ah[4] = {h.x, h.y, h.z, h.w}, al[4] = {l.x, l.y, l.z, l.w};
+                float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mr[4] = {0.f, 0.f, 0.f, 0.f};
+                mma3x<kExact>(pr, ah, al, s0.x, s0.y, s0.z, s0.w);
+                mma3x<kExact>(pi, ah, al, s1.x, s1.y, s1.z, s1.w);
+                if (has_im) {
+                    const uint4 h2 = fy[64], l2 = fy[96];
+                    const uint32_t bh[4] = {h2.x, h2.y, h2.z, h2.w}, bl[4] = {l2.x, l2.y, l2.z, l2.w};
+                    mma3x<kExact>(mr, bh, bl, s1.x, s1.y, s1.z, s1.w);
+                    mma3x<kExact>(pi, bh, bl, s0.x, s0.y, s0.z, s0.w);
+                }
+                const float f = sc[4 * w] * yscal[w];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    x1r[i] = fmaf(f, pr[i] - mr[i], x1r[i]);
+                    x1i[i] = fmaf(f, pi[i], x1i[i]);
+                }
+            }
+            auto conj_product = [&](const uint4 *fx, const uint4 &b0, const uint4 &b1, float f, float (&xr)[4], float (&xi)[4]) {
+                const uint4 h = fx[0], l = fx[32], h2 = fx[64], l2 = fx[96];
+                const uint32_t rh[4] = {h.x, h.y, h.z, h.w}, rl[4] = {l.x, l.y, l.z, l.w};
+                const uint32_t ih[4] = {h2.x, h2.y, h2.z, h2.w}, il[4] = {l2.x, l2.y, l2.z, l2.w};
+                float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mi[4] = {0.f, 0.f, 0.f, 0.f};
+                mma3(pr, rh, rl, b0.x, b0.y, b0.z, b0.w);
+                mma3(pi, rh, rl, b1.x, b1.y, b1.z, b1.w);
+                mma3(mi, ih, il, b0.x, b0.y, b0.z, b0.w);
+                mma3(pr, ih, il, b1.x, b1.y, b1.z, b1.w);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    xr[i] = fmaf(f, pr[i], xr[i]);
+                    xi[i] = fmaf(f, pi[i] - mi[i], xi[i]);
+                }
+            };
+            conj_product(frag + (NCW + w) * 128 + lane, s0, s1, sc[4 * w] * sc[4 * w + 3], x2r, x2i);
+            conj_product(frag + (2 * NCW + w) * 128 + lane, g0, g1, sc[4 * w + 2] * sc[4 * w + 1], x3r, x3i);
+        }
+    }
+    bar_sync(kBarAux, kAux);
+
+    // the triangular factors of the corrections as TF32 A operands: warp = (sum, step of eight tokens); the k index of
+    // a step runs over tokens 4 t4 + 2 step (slot t4) and + 1 (slot t4 + 4), PREP's order of tokens
+    const float *beta_row = a.beta + row0;
+    {
+        const int sum = warp >> 1, i0 = 4 * t4 + 2 * (warp & 1);
+        uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int t = g + 8 * (e & 1), i = i0 + (e >> 1);
+            float2 x = make_float2(0.f, 0.f);
+            if (sum < 2) {
+                if (sum == 0 ? i <= t : i < t) {
+                    const float be = t0 + i < a.T ? beta_row[(size_t)(t0 + i) * a.H] : 0.f;
+                    x = uy[sum * 272 + i * 17 + t];
+                    x = make_float2(be * x.x, be * x.y);
+                }
+            } else if (sum == 2 ? i >= t : i > t) {
+                x = uy[(sum - 2) * 272 + t * 17 + i];
+                x = sum == 2 ? make_float2(x.x, -x.y) : make_float2(-x.x, x.y);
+            }
+            split_tf32(x.x, rh[e], rl[e]);
+            split_tf32(x.y, ih[e], il[e]);
+        }
+        uint4 *p = tri + warp * 128 + lane;
+        p[0] = make_uint4(rh[0], rh[1], rh[2], rh[3]);
+        p[32] = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+        p[64] = make_uint4(ih[0], ih[1], ih[2], ih[3]);
+        p[96] = make_uint4(il[0], il[1], il[2], il[3]);
+    }
+    bar_sync(kBarAux, kAux);
+
+    if (warp < KT) {
+        const bool fast = reinterpret_cast<const int *>(smem + L::flag)[slot] != 0;
+        float z1r[4] = {0.f, 0.f, 0.f, 0.f}, z1i[4] = {0.f, 0.f, 0.f, 0.f}, z2r[4] = {0.f, 0.f, 0.f, 0.f};
+        float z2i[4] = {0.f, 0.f, 0.f, 0.f}, z3r[4] = {0.f, 0.f, 0.f, 0.f}, z3i[4] = {0.f, 0.f, 0.f, 0.f};
+        if (fast) {
+            auto tri_product = [&](int sum, int step, const float2 &b0, const float2 &b1, float (&zr)[4], float (&zi)[4]) {
+                const uint4 *p = tri + (2 * sum + step) * 128 + lane;
+                const uint4 h = p[0], l = p[32], h2 = p[64], l2 = p[96];
+                const uint32_t rh[4] = {h.x, h.y, h.z, h.w}, rl[4] = {l.x, l.y, l.z, l.w};
+                const uint32_t ih[4] = {h2.x, h2.y, h2.z, h2.w}, il[4] = {l2.x, l2.y, l2.z, l2.w};
+                uint32_t brh[2], brl[2], bih[2], bil[2], nih[2], nil[2];
+                split_tf32(b0.x, brh[0], brl[0]);
+                split_tf32(b1.x, brh[1], brl[1]);
+                split_tf32(b0.y, bih[0], bil[0]);
+                split_tf32(b1.y, bih[1], bil[1]);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    nih[i] = bih[i] ^ 0x80000000u;
+                    nil[i] = bil[i] ^ 0x80000000u;
+                }
+                mma3_tf32(zr, rh, rl, brh, brl);
+                mma3_tf32(zi, rh, rl, bih, bil);
+                mma3_tf32(zr, ih, il, nih, nil);
+                mma3_tf32(zi, ih, il, brh, brl);
+            };
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                float2 kh[2], qw[2], wv[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float4 *p = vals + ((4 * t4 + 2 * s + e) * M + 8 * warp + g) * 2;
+                    const float4 x = p[0], y = p[1];
+                    const float ia = __frcp_rn(y.x);
+                    kh[e] = make_float2(x.x * ia, x.y * ia);
+                    wv[e] = make_float2(x.x * y.x, x.y * y.x);
+                    qw[e] = make_float2(x.z * y.x, x.w * y.x);
+                }
+                tri_product(0, s, kh[0], kh[1], z1r, z1i);
+                tri_product(1, s, kh[0], kh[1], z2r, z2i);
+                tri_product(2, s, qw[0], qw[1], z3r, z3i);
+                tri_product(3, s, wv[0], wv[1], z3r, z3i);
+            }
+        }
+        float2 dqv[4], dkv[4], dd[4];
+        float al[4], dbp[2] = {0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = i >> 1, e = i & 1, tl = g + 8 * r, t = t0 + tl, key = 8 * warp + 2 * t4 + e;
+            const size_t row = row0 + (size_t)t * a.H;
+            const float4 x = vals[(tl * M + key) * 2], y = vals[(tl * M + key) * 2 + 1];
+            const float4 last = vals[(15 * M + key) * 2 + 1];                     // e^{i phi_C}
+            const float2 kp = make_float2(x.x, x.y), qp = make_float2(x.z, x.w), ph = make_float2(y.z, y.w);
+            const float be = t < a.T ? a.beta[row] : 0.f;
+            al[i] = t < a.T ? a.alpha[row * M + key] : 1.f;
+            const float2 x3 = cmulc(make_float2(last.z, last.w), make_float2(x3r[i], x3i[i]));
+            float2 qb, zb, fb;
+            if (fast) {
+                const float ia = __frcp_rn(y.x);
+                qb = make_float2(y.x * (x1r[i] + z1r[i]), y.x * (x1i[i] + z1i[i]));
+                zb = make_float2(y.x * (x2r[i] + z2r[i]), y.x * (x2i[i] + z2i[i]));
+                fb = make_float2(fmaf(y.y, x3.x, ia * z3r[i]), fmaf(y.y, x3.y, ia * z3i[i]));
+            } else {
+                // decays too strong to divide by: running products, token by token
+                float w = 1.f;
+                qb = zb = fb = make_float2(0.f, 0.f);
+                for (int j = tl; j >= 0; --j) {
+                    const size_t rj = row0 + (size_t)(t0 + j) * a.H;
+                    const float4 kj = vals[(j * M + key) * 2];
+                    const float bj = t0 + j < a.T ? w * a.beta[rj] : 0.f;
+                    const float2 kk = make_float2(bj * kj.x, bj * kj.y);
+                    const float2 p = cmul(kk, uy[j * 17 + tl]), s = cmul(kk, uy[272 + j * 17 + tl]);
+                    qb = make_float2(qb.x + p.x, qb.y + p.y);
+                    if (j < tl) zb = make_float2(zb.x + s.x, zb.y + s.y);
+                    w *= t0 + j < a.T ? a.alpha[rj * M + key] : 1.f;
+                }
+                qb = make_float2(fmaf(w, x1r[i], qb.x), fmaf(w, x1i[i], qb.y));
+                zb = make_float2(fmaf(w, x2r[i], zb.x), fmaf(w, x2i[i], zb.y));
+                w = 1.f;
+                for (int l = tl; l < 16; ++l) {
+                    const float4 kl = vals[(l * M + key) * 2];
+                    const float2 p = cmulc(uy[tl * 17 + l], make_float2(w * kl.z, w * kl.w));
+                    fb = make_float2(fb.x + p.x, fb.y + p.y);
+                    if (l > tl) {
+                        const float2 s = cmulc(uy[272 + tl * 17 + l], make_float2(w * kl.x, w * kl.y));
+                        fb = make_float2(fb.x - s.x, fb.y - s.y);
+                    }
+                    if (l < 15 && t0 + l + 1 < a.T) w *= a.alpha[(row0 + (size_t)(t0 + l + 1) * a.H) * M + key];
+                }
+                fb = make_float2(fmaf(w, x3.x, fb.x), fmaf(w, x3.y, fb.y));
+            }
+            const float2 dkp = make_float2(be * fb.x - zb.x, be * fb.y - zb.y);
+            dqv[i] = cmul(ph, qb);
+            dkv[i] = cmul(ph, dkp);
+            dbp[r] += fb.x * kp.x + fb.y * kp.y;
+            const float2 p = cmulc(qb, qp), s = cmulc(kp, make_float2(be * fb.x, be * fb.y)), z = cmulc(zb, kp);
+            dd[i] = make_float2(p.x - s.x - z.x, p.y - s.y - z.y);
+        }
+        // D: sums over the tokens behind, down to each token (tokens 8-15 in i = 2, 3, tokens 0-7 in i = 0, 1)
+        if (first) {
+            const float2 *rg = reinterpret_cast<const float2 *>(smem + L::rg) + rpar * NCW * M;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                carry[e] = make_float2(0.f, 0.f);
+                for (int w = 0; w < NCW; ++w) {
+                    const float2 x = rg[w * M + 8 * warp + 2 * t4 + e];
+                    carry[e] = make_float2(carry[e].x + x.x, carry[e].y + x.y);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int d = 4; d < 32; d <<= 1) {
+                const float ox = __shfl_down_sync(0xffffffffu, dd[i].x, d), oy = __shfl_down_sync(0xffffffffu, dd[i].y, d);
+                if (lane + d < 32) dd[i] = make_float2(dd[i].x + ox, dd[i].y + oy);
+            }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            dd[2 + e] = make_float2(dd[2 + e].x + carry[e].x, dd[2 + e].y + carry[e].y);
+            dd[e] = make_float2(dd[e].x + __shfl_sync(0xffffffffu, dd[2 + e].x, t4), dd[e].y + __shfl_sync(0xffffffffu, dd[2 + e].y, t4));
+            carry[e] = make_float2(__shfl_sync(0xffffffffu, dd[e].x, t4), __shfl_sync(0xffffffffu, dd[e].y, t4));
+        }
+        float dal[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) dal[i] = __fdiv_rn(dd[i].x, al[i]);
+        // small alpha: from the definition, one (token, key) at a time
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+            unsigned todo = __ballot_sync(0xffffffffu, (i == 0 ? al[0] : i == 1 ? al[1] : i == 2 ? al[2] : al[3]) < 0.0625f);
+            while (todo) {
+                const int src = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const int tl = (src >> 2) + 8 * (i >> 1), kl = 2 * (src & 3) + (i & 1), key = 8 * warp + kl;
+                float sum = 0.f;
+                float cst = 1.f, snt = 0.f;
+                for (int val = lane; val < NB; val += 32) {
+                    const int w = val >> 4, vl = val & 15, hf = vl & 1;
+                    auto state = [&](const uint4 *base, float inv) {
+                        const uint32_t *p = reinterpret_cast<const uint32_t *>(base + ((w * KT + warp) * 2) * 32 + 4 * kl + ((vl & 7) >> 1)) + (vl >> 3);
+                        return make_float2(inv * join_half(p[0], p[2], hf), inv * join_half(p[128], p[130], hf));
+                    };
+                    auto token = [&](int mat, int tok, float inv) {
+                        const uint32_t *p = reinterpret_cast<const uint32_t *>(frag + (mat * NCW + w) * 128 + 4 * (tok & 7) + ((vl & 7) >> 1)) + (tok >> 3) + 2 * (vl >> 3);
+                        return make_float2(inv * join_half(p[0], p[128], hf), inv * join_half(p[256], p[384], hf));
+                    };
+                    float2 s = state(pS, sc[4 * w]), z = state(pG, sc[4 * w + 2]);
+                    for (int j = 0; j < 16; ++j) {           // S_{t-1}
+                        if (j >= tl) break;
+                        const size_t rj = row0 + (size_t)(t0 + j) * a.H;
+                        const float4 x = vals[(j * M + key) * 2], y = vals[(j * M + key) * 2 + 1];
+                        float sn, cs;
+                        sincosf(a.theta[rj * M + key], &sn, &cs);
+                        const float aj = a.alpha[rj * M + key], bj = a.beta[rj];
+                        const float2 kj = cmul(make_float2(y.z, y.w), make_float2(bj * x.x, bj * x.y)), u = token(2, j, sc[4 * w + 1]);
+                        s = cmul(make_float2(aj * cs, aj * sn), s);
+                        const float2 p = cmul(kj, u);
+                        s = make_float2(s.x + p.x, s.y + p.y);
+                    }
+                    for (int l = 15; l >= tl; --l) {         // the cotangent of Lambda_t S_{t-1}
+                        if (t0 + l >= a.T) continue;
+                        const size_t rl = row0 + (size_t)(t0 + l) * a.H;
+                        const float4 x = vals[(l * M + key) * 2], y = vals[(l * M + key) * 2 + 1];
+                        const float2 ph = make_float2(y.z, y.w), ql = cmul(ph, make_float2(x.z, x.w)), kj = cmul(ph, make_float2(x.x, x.y));
+                        const float2 yb = token(0, l, yscal[w]), bc = token(1, l, sc[4 * w + 3]);
+                        const float2 p = cmulc(yb, ql), m = cmul(kj, bc);
+                        z = make_float2(z.x + p.x - m.x, z.y + p.y - m.y);
+                        float sn, cs;
+                        sincosf(a.theta[rl * M + key], &sn, &cs);
+                        if (l > tl) {
+                            const float aj = a.alpha[rl * M + key];
+                            z = cmulc(make_float2(aj * cs, aj * sn), z);
+                        } else {
+                            cst = cs;
+                            snt = sn;
+                        }
+                    }
+                    const float2 lb = cmulc(s, z);
+                    sum += lb.x * cst + lb.y * snt;          // Re(conj(lambda bar) e^{i theta})
+                }
+#pragma unroll
+                for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+                if (lane == src) {
+                    if (i == 0) dal[0] = sum;
+                    else if (i == 1) dal[1] = sum;
+                    else if (i == 2) dal[2] = sum;
+                    else dal[3] = sum;
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int t = t0 + g + 8 * r;
+            if (t < a.T) {
+                const size_t row = row0 + (size_t)t * a.H;
+                const size_t ak = row * DK + 2 * (8 * warp + 2 * t4), am = row * M + 8 * warp + 2 * t4;
+                const float4 q4 = make_float4(dqv[2 * r].x, dqv[2 * r].y, dqv[2 * r + 1].x, dqv[2 * r + 1].y);
+                const float4 k4 = make_float4(dkv[2 * r].x, dkv[2 * r].y, dkv[2 * r + 1].x, dkv[2 * r + 1].y);
+                const float2 a2 = make_float2(dal[2 * r], dal[2 * r + 1]), th2 = make_float2(dd[2 * r].y, dd[2 * r + 1].y);
+                if constexpr (NSL == 1) {
+                    st_val4(static_cast<T *>(a.dq) + ak, q4);
+                    st_val4(static_cast<T *>(a.dk) + ak, k4);
+                    *reinterpret_cast<float2 *>(a.dalpha + am) = a2;
+                    *reinterpret_cast<float2 *>(a.dtheta + am) = th2;
+                } else {
+                    const size_t off = (size_t)blockIdx.y * a.rows;
+                    st_val4(a.dq_p + off * DK + ak, q4);
+                    st_val4(a.dk_p + off * DK + ak, k4);
+                    *reinterpret_cast<float2 *>(a.dalpha_p + off * M + am) = a2;
+                    *reinterpret_cast<float2 *>(a.dtheta_p + off * M + am) = th2;
+                }
+            }
+            float x = dbp[r];
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            x += __shfl_xor_sync(0xffffffffu, x, 2);
+            if (t4 == 0) db[warp * 16 + g + 8 * r] = x;
+        }
+    }
+    bar_sync(kBarAux, kAux);
+    if (tid < 16 && t0 + tid < a.T) {
+        float x = 0.f;
+#pragma unroll
+        for (int w = 0; w < KT; ++w) x += db[w * 16 + tid];
+        const size_t row = row0 + (size_t)(t0 + tid) * a.H;
+        if constexpr (NSL == 1) a.dbeta[row] = x;
+        else a.dbeta_p[(size_t)blockIdx.y * a.rows + row] = x;
+    }
+}
+
+template <int DK, int DVT, int NB, typename T>
+__global__ void __launch_bounds__(kAux + 2 * NB, 1) sfda_backward_kernel(const BwdArgsDev a)
+{
+    using TL = Tile<DK>;
+    using L = BwdSmem<DK, NB>;
+    using SC = BwdScratch<DK, NB>;
+    constexpr int kAll = kAux + 2 * NB, NCW = NB / 16, M = DK / 2, KT = TL::KT;
+    constexpr bool kExact = sizeof(T) == 2;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
+    const size_t row0 = (size_t)b * a.T * a.H + h;                       // row of token t: row0 + t H
+    const int nch = (a.T + kC - 1) / kC, NS = a.NS;
+    unsigned char *ring = reinterpret_cast<unsigned char *>(a.scratch + ((size_t)bh * DVT + c0) * kSeg * DK);
+    const int last_nch = nch - (NS - 1) * kSegChunks;                    // chunks of the last segment
+
+    if (tid < kAux) {
+        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+        const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3, key = 8 * warp + g;
+        const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
+        float2 *stage = reinterpret_cast<float2 *>(smem + L::stage);
+        int par = 0;
+        for (int c = 0; c < nch; ++c) {                                  // first sweep: keys only
+            const int slot = c % kSlots;
+            if (c >= kSlots) bar_sync(kBarDone + slot, kAll);
+            PrepIn in;
+            PrepVals pv;
+            prep_load<DK, T>(in, nullptr, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, key, t4);
+            prep_chunk<DK, false>(in, pv, smem + slot * TL::bytes, stage, smem + L::small, par, tid);
+            bar_arrive(kBarFull + slot, kAll);
+            par ^= 1;
+        }
+        for (int c = max(nch - kSlots, 0); c < nch; ++c) bar_sync(kBarDone + c % kSlots, kAll);
+        // Second sweep.  Chunks are prepared in the order the chain goes forward through the segments (last segment
+        // first) and their gradients follow in the order it comes back; the ring's slots are assigned so that the
+        // p-th chunk prepared takes the slot of gradient p - 4.
+        float2 carry[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        for (int p = 0; p < nch + kSlots; ++p) {
+            if (p >= kSlots) {
+                const int n = p - kSlots, r = n < last_nch ? 0 : 1 + (n - last_nch) / kSegChunks;
+                const int nc = r == 0 ? last_nch : kSegChunks, at = r == 0 ? n : (n - last_nch) % kSegChunks, c = nc - 1 - at;
+                const int slot = ring_slot(r, c);
+                bar_sync(kBarDone + slot, kAll);
+                chunk_gradients<DK, DVT, NB, T>(a, smem, ring + (size_t)slot * SC::slot, slot, r & 1, at == 0,
+                                                (NS - 1 - r) * kSeg + c * kC, row0, carry, tid);
+                if (p < nch) bar_arrive(kBarFree + slot, kAll);
+            }
+            if (p < nch) {
+                const int r = p < last_nch ? 0 : 1 + (p - last_nch) / kSegChunks, c = r == 0 ? p : (p - last_nch) % kSegChunks;
+                const int slot = ring_slot(r, c);
+                PrepIn in;
+                PrepVals pv;
+                prep_load<DK, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, (NS - 1 - r) * kSeg + c * kC, a.T, key, t4);
+                const bool fast = prep_chunk<DK, true>(in, pv, smem + slot * TL::bytes, stage, smem + L::small, par, tid);
+                bar_arrive(kBarFull + slot, kAll);
+                par ^= 1;
+                if (tid == 0) reinterpret_cast<int *>(smem + L::flag)[slot] = fast;
+                if (key < M) {
+                    float4 *vals = reinterpret_cast<float4 *>(ring + (size_t)slot * SC::slot + SC::oV) + (4 * t4 * M + key) * 2;
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        vals[x * M * 2] = make_float4(pv.kr[x], pv.ki[x], pv.qr[x], pv.qi[x]);
+                        vals[x * M * 2 + 1] = make_float4(pv.a[x], pv.sfx[x], pv.cs[x], pv.sn[x]);
+                    }
+                }
+            }
+        }
+        return;
+    }
+
+    if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+    const int lane = tid & 31, w = (tid - kAux) >> 5, g = lane >> 2, t4 = lane & 3;
+    const int col = c0 + 16 * w + g;                                     // and col + 8
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+    float *scal = reinterpret_cast<float *>(smem + L::scal);
+    auto checkpoint = [&](int s) {
+        return reinterpret_cast<float4 *>(a.check + (((size_t)bh * NS + s) * DVT + c0 + 16 * w) * DK);
+    };
+    auto state_at = [&](int n, int i) {                                  // Re of (key, column) of accumulator element (n, i)
+        return ((size_t)bh * DK + 2 * (8 * n + 2 * t4 + (i & 1))) * DVT + col + 8 * (i >> 1);
+    };
+    auto load_tokens = [&](const void *p, int t0, float sign, float (&x)[2][4]) {
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int t = t0 + 8 * n + 2 * t4 + (i & 1);
+                x[n][i] = p && t < a.T ? sign * ld_val(static_cast<const T *>(p), (row0 + (size_t)t * a.H) * DVT + col + 8 * (i >> 1)) : 0.f;
+            }
+    };
+    float sr[KT][4], si[KT][4];
+#pragma unroll
+    for (int n = 0; n < KT; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            sr[n][i] = a.S0 ? a.S0[state_at(n, i)] : 0.f;
+            si[n][i] = a.S0 ? a.S0[state_at(n, i) + DVT] : 0.f;
+        }
+
+    // forward through one chunk: U = M (V - W^* S), S <- gamma_C S + Y U
+    auto forward_chunk = [&](int slot, int t0, auto pub, bool update) {
+        constexpr bool kPub = decltype(pub)::value;
+        unsigned char *scr = ring + (size_t)slot * SC::slot;
+        float rr[2][4], ri[2][4];
+        load_tokens(a.v, t0, 1.f, rr);
+        bar_sync(kBarFull + slot, kAll);
+        const uint32_t tile = base + slot * TL::bytes;
+        const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
+        float isv;
+        const float ss = scale_for(__reduce_max_sync(0xffffffffu, max(max_bits4(sr), max_bits4(si))), isv);
+        float acc[1][3][2][4];
+        const uint32_t tiles[1] = {tile + TL::oW};
+        product_over_keys<DK, 1, kPub>(acc, sr, si, ss, tiles, lane, reinterpret_cast<uint4 *>(scr + SC::oS) + w * KT * 64);
+        const float fw = isv * inv[0];
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
+                ri[n][i] = -fw * (acc[0][1][n][i] - acc[0][2][n][i]);
+            }
+        TokFrag fr, fb;
+        const float ir = make_frag(fr, rr, ri);
+        load_small<false>(fb, tile + TL::oM, lane);
+        product_small<false>(rr, ri, fr, fb, ir * inv[3]);
+        const float iu = make_frag(fr, rr, ri);
+        if constexpr (kPub) {
+            publish_frag(reinterpret_cast<uint4 *>(scr + SC::oU) + w * 128, fr, lane);
+            if (lane == 0) {
+                scal[(slot * NCW + w) * 4] = isv;
+                scal[(slot * NCW + w) * 4 + 1] = iu;
+            }
+        }
+        if (update)
+            state_update<DK>(sr, si, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
+    };
+
+    for (int c = 0; c < nch; ++c) {
+        if (c % kSegChunks == 0) store_state<KT>(checkpoint(c / kSegChunks), sr, si, lane);
+        forward_chunk(c % kSlots, c * kC, std::false_type{}, true);
+        bar_arrive(kBarDone + c % kSlots, kAll);
+    }
+
+    float gr[KT][4], gi[KT][4];
+    for (int r = 0; r < NS; ++r) {
+        const int s = NS - 1 - r, nc = r == 0 ? last_nch : kSegChunks, p0 = r == 0 ? 0 : last_nch + kSegChunks * (r - 1);
+        // rowdot(conj S, G) at the segment's end, this warp's columns; G then waits where that state was kept
+        {
+            float2 *rg = reinterpret_cast<float2 *>(smem + L::rg) + ((r & 1) * NCW + w) * M;
+            if (r == 0) {
+#pragma unroll
+                for (int n = 0; n < KT; ++n)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        gr[n][i] = a.dS_T ? a.dS_T[state_at(n, i)] : 0.f;
+                        gi[n][i] = a.dS_T ? a.dS_T[state_at(n, i) + DVT] : 0.f;
+                    }
+            } else {
+                load_state<KT>(checkpoint(s + 1), sr, si, lane);
+            }
+#pragma unroll
+            for (int n = 0; n < KT; ++n)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    float x = sr[n][e] * gr[n][e] + si[n][e] * gi[n][e] + sr[n][e + 2] * gr[n][e + 2] + si[n][e + 2] * gi[n][e + 2];
+                    float y = sr[n][e] * gi[n][e] - si[n][e] * gr[n][e] + sr[n][e + 2] * gi[n][e + 2] - si[n][e + 2] * gr[n][e + 2];
+#pragma unroll
+                    for (int d = 4; d < 32; d <<= 1) {
+                        x += __shfl_xor_sync(0xffffffffu, x, d);
+                        y += __shfl_xor_sync(0xffffffffu, y, d);
+                    }
+                    if (g == 0) rg[8 * n + 2 * t4 + e] = make_float2(x, y);
+                }
+            if (r > 0) store_state<KT>(checkpoint(s + 1), gr, gi, lane);
+        }
+        load_state<KT>(checkpoint(s), sr, si, lane);
+        for (int c = 0; c < nc; ++c) {
+            const int slot = ring_slot(r, c);
+            if (p0 + c >= kSlots) bar_sync(kBarFree + slot, kAll);
+            forward_chunk(slot, s * kSeg + c * kC, std::true_type{}, c + 1 < nc);
+        }
+        if (r == 0) {
+#pragma unroll
+            for (int n = 0; n < KT; ++n)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    gr[n][i] = a.dS_T ? a.dS_T[state_at(n, i)] : 0.f;
+                    gi[n][i] = a.dS_T ? a.dS_T[state_at(n, i) + DVT] : 0.f;
+                }
+        } else {
+            load_state<KT>(checkpoint(s + 1), gr, gi, lane);
+        }
+        for (int c = nc - 1; c >= 0; --c) {
+            const int slot = ring_slot(r, c), t0 = s * kSeg + c * kC;
+            unsigned char *scr = ring + (size_t)slot * SC::slot;
+            const bool has_im = a.d_o_im != nullptr;
+            float yr[2][4], yi[2][4];
+            load_tokens(a.d_o, t0, 1.f, yr);
+            load_tokens(a.d_o_im, t0, -1.f, yi);
+            const uint32_t tile = base + slot * TL::bytes;
+            const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
+            float ig;
+            const float sg = scale_for(__reduce_max_sync(0xffffffffu, max(max_bits4(gr), max_bits4(gi))), ig);
+            float acc[1][3][2][4];
+            const uint32_t tiles[1] = {tile + TL::oY};
+            product_over_keys<DK, 1, true>(acc, gr, gi, sg, tiles, lane, reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64);
+            TokFrag fy, fp, fb;
+            const float iy = make_frag(fy, yr, yi);
+            float pr[2][4], pi[2][4];
+            const float fg = ig * inv[1];
+#pragma unroll
+            for (int n = 0; n < 2; ++n)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    pr[n][i] = fg * acc[0][0][n][i];
+                    pi[n][i] = fg * (acc[0][1][n][i] - acc[0][2][n][i]);
+                }
+            load_small<true>(fb, tile + TL::oA, lane);
+            product_small_conj<kExact>(pr, pi, fy, fb, iy * inv[4], has_im);
+            const float ip = make_frag(fp, pr, pi);
+            load_small<true>(fb, tile + TL::oM, lane);
+            product_small<true>(pr, pi, fp, fb, ip * inv[3]);
+#pragma unroll
+            for (int n = 0; n < 2; ++n)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int t = t0 + 8 * n + 2 * t4 + (i & 1);
+                    if (t < a.T) st_val(static_cast<T *>(a.dv), (row0 + (size_t)t * a.H) * DVT + col + 8 * (i >> 1), pr[n][i]);
+                }
+            const float ib = make_frag(fp, pr, pi);
+            publish_frag(reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, fp, lane);
+            if (lane == 0) {
+                scal[(slot * NCW + w) * 4 + 2] = ig;
+                scal[(slot * NCW + w) * 4 + 3] = ib;
+            }
+            // G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc
+            const float fq = iy * inv[2], fw = ib * inv[0];
+            const float4 *gamma = reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG);
+            const uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
+#pragma unroll
+            for (int np = 0; np < KT; np += 2) {
+                uint32_t qrh[4], qrl[4], qih[4], qil[4], wrh[4], wrl[4], wih[4], wil[4];
+                ldsm_t(qrh, at + TL::oQ + np * 16);
+                ldsm_t(qrl, at + TL::oQ + np * 16 + TL::PL);
+                ldsm_t(qih, at + TL::oQ + np * 16 + 2 * TL::PL);
+                ldsm_t(qil, at + TL::oQ + np * 16 + 3 * TL::PL);
+                ldsm_t(wrh, at + TL::oW + np * 16);
+                ldsm_t(wrl, at + TL::oW + np * 16 + TL::PL);
+                ldsm_t(wih, at + TL::oW + np * 16 + 2 * TL::PL);
+                ldsm_t(wil, at + TL::oW + np * 16 + 3 * TL::PL);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int n = np + e;
+                    float qr_[4] = {0.f, 0.f, 0.f, 0.f}, qn[4] = {0.f, 0.f, 0.f, 0.f}, qm[4] = {0.f, 0.f, 0.f, 0.f};
+                    float wr_[4] = {0.f, 0.f, 0.f, 0.f}, wn[4] = {0.f, 0.f, 0.f, 0.f}, wm[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma3(wr_, fp.rh, fp.rl, wrh[2 * e], wrh[2 * e + 1], wrl[2 * e], wrl[2 * e + 1]);
+                    mma3(wm, fp.ih, fp.il, wrh[2 * e], wrh[2 * e + 1], wrl[2 * e], wrl[2 * e + 1]);
+                    mma3(wn, fp.ih, fp.il, wih[2 * e], wih[2 * e + 1], wil[2 * e], wil[2 * e + 1]);
+                    mma3x<kExact>(qr_, fy.rh, fy.rl, qrh[2 * e], qrh[2 * e + 1], qrl[2 * e], qrl[2 * e + 1]);
+                    mma3x<kExact>(qm, fy.rh, fy.rl, qih[2 * e], qih[2 * e + 1], qil[2 * e], qil[2 * e + 1]);
+                    mma3(wm, fp.rh, fp.rl, wih[2 * e], wih[2 * e + 1], wil[2 * e], wil[2 * e + 1]);
+                    if (has_im) {
+                        mma3x<kExact>(qn, fy.ih, fy.il, qih[2 * e], qih[2 * e + 1], qil[2 * e], qil[2 * e + 1]);
+                        mma3x<kExact>(qm, fy.ih, fy.il, qrh[2 * e], qrh[2 * e + 1], qrl[2 * e], qrl[2 * e + 1]);
+                    }
+                    const float4 gm = gamma[4 * n + t4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float cr = (i & 1) ? gm.z : gm.x, ci = (i & 1) ? gm.w : gm.y, x = gr[n][i], y = gi[n][i];
+                        gr[n][i] = fmaf(fq, qr_[i] - qn[i], fmaf(-fw, wr_[i] - wn[i], cr * x + ci * y));
+                        gi[n][i] = fmaf(fq, qm[i], fmaf(-fw, wm[i], cr * y - ci * x));
+                    }
+                }
+            }
+            bar_arrive(kBarDone + slot, kAll);
+        }
+    }
+#pragma unroll
+    for (int n = 0; n < KT; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            a.dS0[state_at(n, i)] = gr[n][i];
+            a.dS0[state_at(n, i) + DVT] = gi[n][i];
+        }
+}
+
+// ---- the sums over the column blocks: out[i] = share_0[i] + share_1[i] + ... in that order, one thread per four
+// consecutive elements.  HBM-bound and small beside the sweeps.
+constexpr int kSumThreads = 256;
 
 template <int NSL, typename T>
 __global__ void __launch_bounds__(kSumThreads)
@@ -557,7 +930,7 @@ cudaError_t launch_cols(const BackwardArgs &x, void *workspace, cudaStream_t str
     a.rows = bhn * x.T;
     a.check = ws + w.check; a.scratch = ws + w.scratch;
     a.dq_p = ws + w.dq; a.dk_p = ws + w.dk; a.dalpha_p = ws + w.dalpha; a.dtheta_p = ws + w.dtheta; a.dbeta_p = ws + w.dbeta;
-    kern<<<dim3((unsigned)bhn, NSL), kBwdThreads, L::bytes, stream>>>(a);
+    kern<<<dim3((unsigned)bhn, NSL), kAux + 2 * DV, L::bytes, stream>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (launches) ++*launches;
     if constexpr (NSL > 1) {
