@@ -3,7 +3,7 @@
 // be timed, App. E; what it computes is the adjoint of Eq. "sfda".)  Complex cotangents Xb mean dL = Re sum conj(Xb) dX,
 // i.e. the ordinary gradient with respect to the (Re, Im) pair; yb_t = do_re + i do_im.
 //
-// Per chunk, with W, Y, Q, M, A^{qk} of sfda_chunk16.cuh, S_0 the state before the chunk and G_C the cotangent of the
+// Per chunk, with W, Y, Q, M, A^{qk} of sfda_chunk16_unrolled.cuh, S_0 the state before the chunk and G_C the cotangent of the
 // state after it:
 //
 //   forward    U = M (V - W^* S_0)  (rows u_t^T = v_t^T - k_t^* Lambda_t S_{t-1}),   S_C = gamma_C S_0 + Y U
@@ -28,7 +28,7 @@
 //   FULL  operand tile ready       DONE  the chain is through with a chunk       FREE  its gradients are written
 #include <type_traits>
 
-#include "sfda_chunk16.cuh"
+#include "sfda_chunk16_unrolled.cuh"
 #include "sfda_internal.h"
 
 namespace sfda {

@@ -6,16 +6,23 @@
 // products (323 effective) are twice as fast as 3 x TF32 (161) and 2.5 times the fp32 pipe (128), at the same 22 bits.
 // fp16's exponent range is covered by scaling every operand tile by a power of two that puts its largest magnitude
 // at 2^14: entries down to 2^-16 of the largest keep all 22 bits, smaller ones an absolute error of 2^-39 of it.
-// Where an operand's range is not bounded (keys divided by the cumulative decay) 3 x TF32 is used instead.
 //
 // Why chunks of 16: the state-sized products cost the same per token at any chunk size, the products inside a chunk
-// grow with it, and inside 16 tokens the decays divide safely unless a coordinate loses more than 2^-80, which is
+// grow with it, and inside 16 tokens the decays divide safely unless a coordinate loses more than 2^-16, which is
 // checked per chunk (a slow exact path takes over then).
 //
-// Roles in a CTA: eight AUX warps prepare the operand tiles of a chunk (PREP) into a ring of shared-memory slots;
-// CHAIN warps own 16 value columns of the state each, for all keys, in the accumulator layout of m16n8 with the value
-// channel as the row.  That layout is also the A-operand layout of the next product, so a chain warp goes
-// R = V - W^* S -> U = M R -> S = gamma_C S + Y U with no exchange with other warps at all.
+// Roles in a CTA: PREP warps make the operand tiles of a chunk into a ring of shared-memory slots, SOLVE warps the two
+// Gram matrices and the inverse of the triangular system, and each CHAIN warp owns 16 value columns of the state, for
+// all keys, in the accumulator layout of m16n8 with the value channel as the row.  That layout is also the A-operand
+// layout of the next product, so a chain warp goes R = V - W^* S -> U = M R -> S = gamma_C S + Y U with no exchange
+// with other warps at all.
+//
+// Code counts: mma.sync holds its scheduler (sfda_forward_f32.cu), so every other instruction adds to the time, and
+// unrolled code streams from the instruction caches (the first version was 93 KB for the forward).  So the operands of
+// the Gram products come from the planes by ldmatrix instead of being split again, and every loop over key tiles is
+// rolled.  Registers cannot be indexed at run time, hence the state lives in tensor memory -- a thread's accumulator
+// fragment in consecutive columns of its lane -- and passes through registers 16 columns at a time, requested one step
+// ahead; that also frees the 64 registers per thread it took.
 #pragma once
 #include "sfda_common.cuh"
 
@@ -23,7 +30,6 @@ namespace sfda {
 namespace c16 {
 
 constexpr int kC = 16;                       // tokens per chunk
-constexpr int kAuxWarps = 8, kAux = 32 * kAuxWarps;
 constexpr int kSlots = 4;                    // operand tiles in flight
 constexpr int kBarAux = 1, kBarFull = 2, kBarDone = 6, kBarFree = 10;   // hardware barriers; the last three: + slot
 
@@ -37,26 +43,12 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+// d = a b
+__device__ __forceinline__ void mma_f16_z(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// d += (ah + al)(bh + bl) without the product of the tails, smallest terms first
-__device__ __forceinline__ void mma3(float (&d)[4], const uint32_t (&ah)[4], const uint32_t (&al)[4], uint32_t bh0,
-                                     uint32_t bh1, uint32_t bl0, uint32_t bl1)
-{
-    mma_f16(d, al, bh0, bh1);
-    mma_f16(d, ah, bl0, bl1);
-    mma_f16(d, ah, bh0, bh1);
-}
-__device__ __forceinline__ void mma3_tf32(float (&d)[4], const uint32_t (&ah)[4], const uint32_t (&al)[4],
-                                          const uint32_t (&bh)[2], const uint32_t (&bl)[2])
-{
-    mma_tf32(d, al, bh[0], bh[1]);
-    mma_tf32(d, ah, bl[0], bl[1]);
-    mma_tf32(d, ah, bh[0], bh[1]);
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 __device__ __forceinline__ void ldsm(uint32_t (&r)[4], uint32_t addr)
 {
@@ -93,37 +85,83 @@ __device__ __forceinline__ void split_f16(float x, float y, uint32_t &h, uint32_
     const float2 f = unpack_f16(h);
     l = pack_f16(x - f.x, y - f.y);
 }
-// TF32 head = the value cut to ten mantissa bits; the tail is passed as it is (the tensor core reads its leading bits)
-__device__ __forceinline__ void split_tf32(float x, uint32_t &h, uint32_t &l)
+// Power of two that brings this magnitude into [2^14, 2^15), and its inverse.
+__device__ __forceinline__ float scale_for(float largest, float &inv)
 {
-    h = __float_as_uint(x) & 0xffffe000u;
-    l = __float_as_uint(x - __uint_as_float(h));
-}
-// Power of two that brings a magnitude with these bits into [2^14, 2^15), and its inverse.
-__device__ __forceinline__ float scale_for(uint32_t max_bits, float &inv)
-{
-    const int e = max((int)(max_bits >> 23) - 127, -100);
+    const int e = max((int)(__float_as_uint(largest) >> 23) - 127, -100);
     inv = __uint_as_float((uint32_t)(113 + e) << 23);
     return __uint_as_float((uint32_t)(141 - e) << 23);
 }
-__device__ __forceinline__ uint32_t abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ float warp_max(float x) { return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x))); }   // x >= 0
 template <int N>
-__device__ __forceinline__ uint32_t max_bits4(const float (&x)[N][4])
+__device__ __forceinline__ float max_abs(const float (&x)[N][4])
 {
-    uint32_t m = 0;
+    float m = 0.f;
 #pragma unroll
     for (int n = 0; n < N; ++n)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) m = max(m, abs_bits(x[n][i]));
+        for (int i = 0; i < 4; ++i) m = fmaxf(m, fabsf(x[n][i]));
     return m;
 }
 // A-operand registers (16 x 16) of two neighbouring accumulator tiles, scaled and split
-__device__ __forceinline__ void split_tiles(const float (&x)[4], const float (&y)[4], float s, uint32_t (&h)[4], uint32_t (&l)[4])
+__device__ __forceinline__ void split_tiles(const float *x, const float *y, float s, uint32_t (&h)[4], uint32_t (&l)[4])
 {
     split_f16(x[0] * s, x[1] * s, h[0], l[0]);
     split_f16(x[2] * s, x[3] * s, h[1], l[1]);
     split_f16(y[0] * s, y[1] * s, h[2], l[2]);
     split_f16(y[2] * s, y[3] * s, h[3], l[3]);
+}
+// cos / sin of a phase in 2^-32 turns: the quadrant is the two leading bits, the rest lies in [-pi/4, pi/4], where the
+// Taylor polynomials to x^9 and x^10 are off by 2e-9 (half the code of sincospif, and code is what costs here)
+__device__ __forceinline__ void cos_sin(uint32_t turns, float &c, float &s)
+{
+    const uint32_t q = (turns + 0x20000000u) >> 30;
+    const float x = (float)(int32_t)(turns - (q << 30)) * 1.4629180792671596e-9f, y = x * x;
+    float p = fmaf(y, 2.7557319e-6f, -1.9841270e-4f), r = fmaf(y, -2.7557319e-7f, 2.4801587e-5f);
+    p = fmaf(y, p, 8.3333333e-3f);
+    r = fmaf(y, r, -1.3888889e-3f);
+    p = fmaf(y, p, -0.16666667f);
+    r = fmaf(y, r, 4.1666667e-2f);
+    p = fmaf(x * y, p, x);
+    r = fmaf(y, fmaf(y, r, -0.5f), 1.f);
+    const float cc = q & 1 ? p : r, ss = q & 1 ? r : p;
+    c = (q + 1) & 2 ? -cc : cc;
+    s = q & 2 ? -ss : ss;
+}
+
+// ---- the state in tensor memory: 16 columns of the thread's lane = two key tiles, [re 4, im 4] each ------------------
+__device__ __forceinline__ void tm_load(float (&x)[16], uint32_t addr)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7]), "=f"(x[8]),
+                   "=f"(x[9]), "=f"(x[10]), "=f"(x[11]), "=f"(x[12]), "=f"(x[13]), "=f"(x[14]), "=f"(x[15])
+                 : "r"(addr));
+}
+// the loaded registers pass through the wait, so that no use of them can be moved in front of it
+__device__ __forceinline__ void tm_wait_load(float (&x)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(x[0]), "+f"(x[1]), "+f"(x[2]), "+f"(x[3]), "+f"(x[4]), "+f"(x[5]), "+f"(x[6]), "+f"(x[7]), "+f"(x[8]),
+                   "+f"(x[9]), "+f"(x[10]), "+f"(x[11]), "+f"(x[12]), "+f"(x[13]), "+f"(x[14]), "+f"(x[15])
+                 :
+                 : "memory");
+}
+__device__ __forceinline__ void tm_store(uint32_t addr, const float (&x)[16])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+                 ::"r"(addr), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7]), "f"(x[8]),
+                 "f"(x[9]), "f"(x[10]), "f"(x[11]), "f"(x[12]), "f"(x[13]), "f"(x[14]), "f"(x[15])
+                 : "memory");
+}
+__device__ __forceinline__ void tm_wait_store() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tm_alloc(uint32_t *where, int columns)     // one warp; columns: a power of two >= 32
+{
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(where)), "r"(columns) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tm_free(uint32_t base, int columns)
+{
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(columns));
 }
 
 // ---- operand tiles of a chunk in shared memory --------------------------------------------------
@@ -138,17 +176,17 @@ struct Tile {
     static constexpr int PL = 16 * LDB, BIG = 4 * PL;
     static constexpr int LDS = 48, PS = 16 * LDS, SMALL = 4 * PS;
     static constexpr int oW = 0, oY = BIG, oQ = 2 * BIG, oM = 3 * BIG, oA = oM + SMALL, oG = oA + SMALL, oS = oG + 8 * M;
-    static constexpr int bytes = (oS + 32 + 127) / 128 * 128;     // oG: gamma_C float2 [M]; oS: inverse scales W Y Q M A
+    // oG: gamma_C float2 [M]; oS: inverse scales of W, Y, Q, M, A, Kb, then whether the chunk is fast
+    static constexpr int bytes = (oS + 32 + 127) / 128 * 128;
 };
 
 // ---- CHAIN --------------------------------------------------------------------------------------
-// acc[x] = products conj(X_x)^T S of NX tiles with the state, value channels in rows, tokens in columns, for each of
-// two token tiles: [0] = Xr Sr + Xi Si, [1] = Xr Si, [2] = Xi Sr (Im = [1] - [2]); scaled by s and the tiles' scales.
-// With kPub the split state is also left in `pub` as the B operand (value channel, key) of products over the columns.
-template <int DK, int NX, bool kPub>
-__device__ __forceinline__ void product_over_keys(float (&acc)[NX][3][2][4], const float (&sr)[DK / 16][4],
-                                                  const float (&si)[DK / 16][4], float s, const uint32_t (&tile)[NX],
-                                                  int lane, uint4 *pub)
+// acc[x] = products conj(X_x)^T S of NX tiles with the state at `st`, value channels in rows, tokens in columns, for
+// each of two token tiles: [0] = Xr Sr + Xi Si, [1] = Xr Si, [2] = Xi Sr (Im = [1] - [2]); scaled by s and the tiles'
+// scales.  pub(kk, rh, rl, ih, il) sees the split state of every step.
+template <int DK, int NX, typename Pub>
+__device__ __forceinline__ void keys_product(float (&acc)[NX][3][2][4], uint32_t st, float s, const uint32_t (&tile)[NX],
+                                             int lane, Pub pub)
 {
     using TL = Tile<DK>;
 #pragma unroll
@@ -159,37 +197,44 @@ __device__ __forceinline__ void product_over_keys(float (&acc)[NX][3][2][4], con
             for (int n = 0; n < 2; ++n)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc[x][c][n][i] = 0.f;
-    const uint32_t at = (uint32_t)(((lane & 7) + ((lane >> 4) << 3)) * TL::LDB + ((lane >> 3) & 1) * 16);
-#pragma unroll
-    for (int kk = 0; kk < TL::KS; ++kk) {
+    uint32_t at = (uint32_t)(((lane & 7) + ((lane >> 4) << 3)) * TL::LDB + ((lane >> 3) & 1) * 16);
+    float x[16];
+    tm_load(x, st);
+    tm_wait_load(x);
+#pragma unroll 1
+    for (int kk = 0; kk < TL::KS; ++kk, at += 32) {
         uint32_t rh[4], rl[4], ih[4], il[4];
-        split_tiles(sr[2 * kk], sr[2 * kk + 1], s, rh, rl);
-        split_tiles(si[2 * kk], si[2 * kk + 1], s, ih, il);
-        if constexpr (kPub) {
+        split_tiles(x, x + 8, s, rh, rl);
+        split_tiles(x + 4, x + 12, s, ih, il);
+        const bool more = kk + 1 < TL::KS;
+        if (more) tm_load(x, st + 16 * (kk + 1));
+        pub(kk, rh, rl, ih, il);
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                pub[((2 * kk + e) * 2 + 0) * 32 + lane] = make_uint4(transpose8x8(rh[2 * e]), transpose8x8(rh[2 * e + 1]),
-                                                                   transpose8x8(rl[2 * e]), transpose8x8(rl[2 * e + 1]));
-                pub[((2 * kk + e) * 2 + 1) * 32 + lane] = make_uint4(transpose8x8(ih[2 * e]), transpose8x8(ih[2 * e + 1]),
-                                                                   transpose8x8(il[2 * e]), transpose8x8(il[2 * e + 1]));
-            }
-        }
-#pragma unroll
-        for (int x = 0; x < NX; ++x) {
+        for (int t = 0; t < NX; ++t) {
             uint32_t brh[4], brl[4], bih[4], bil[4];
-            const uint32_t p = tile[x] + at + kk * 32;
+            const uint32_t p = tile[t] + at;
             ldsm(brh, p);
-            ldsm(brl, p + TL::PL);
             ldsm(bih, p + 2 * TL::PL);
+            ldsm(brl, p + TL::PL);
             ldsm(bil, p + 3 * TL::PL);
+            // an accumulator's next product is four instructions away
 #pragma unroll
-            for (int n = 0; n < 2; ++n) {
-                mma3(acc[x][0][n], rh, rl, brh[2 * n], brh[2 * n + 1], brl[2 * n], brl[2 * n + 1]);
-                mma3(acc[x][1][n], ih, il, brh[2 * n], brh[2 * n + 1], brl[2 * n], brl[2 * n + 1]);
-                mma3(acc[x][2][n], rh, rl, bih[2 * n], bih[2 * n + 1], bil[2 * n], bil[2 * n + 1]);
-                mma3(acc[x][0][n], ih, il, bih[2 * n], bih[2 * n + 1], bil[2 * n], bil[2 * n + 1]);
+            for (int k = 0; k < 3; ++k) {
+                const uint32_t(&ar)[4] = k == 0 ? rl : rh;
+                const uint32_t(&ai)[4] = k == 0 ? il : ih;
+                const uint32_t(&br)[4] = k == 1 ? brl : brh;
+                const uint32_t(&bi)[4] = k == 1 ? bil : bih;
+#pragma unroll
+                for (int n = 0; n < 2; ++n) mma_f16(acc[t][0][n], ar, br[2 * n], br[2 * n + 1]);
+#pragma unroll
+                for (int n = 0; n < 2; ++n) mma_f16(acc[t][1][n], ai, br[2 * n], br[2 * n + 1]);
+#pragma unroll
+                for (int n = 0; n < 2; ++n) mma_f16(acc[t][0][n], ai, bi[2 * n], bi[2 * n + 1]);
+#pragma unroll
+                for (int n = 0; n < 2; ++n) mma_f16(acc[t][2][n], ar, bi[2 * n], bi[2 * n + 1]);
             }
         }
+        if (more) tm_wait_load(x);
     }
 }
 
@@ -222,449 +267,570 @@ __device__ __forceinline__ void load_small(TokFrag &b, uint32_t tile, int lane)
 template <bool kConj>
 __device__ __forceinline__ void product_small(float (&re)[2][4], float (&im)[2][4], const TokFrag &a, const TokFrag &b, float f)
 {
+    float rr[2][4], ii[2][4], ir[2][4], ri[2][4];
 #pragma unroll
-    for (int n = 0; n < 2; ++n) {
-        float rr[4] = {0.f, 0.f, 0.f, 0.f}, ii[4] = {0.f, 0.f, 0.f, 0.f}, ir[4] = {0.f, 0.f, 0.f, 0.f}, ri[4] = {0.f, 0.f, 0.f, 0.f};
-        mma3(rr, a.rh, a.rl, b.rh[2 * n], b.rh[2 * n + 1], b.rl[2 * n], b.rl[2 * n + 1]);
-        mma3(ii, a.ih, a.il, b.ih[2 * n], b.ih[2 * n + 1], b.il[2 * n], b.il[2 * n + 1]);
-        mma3(ir, a.ih, a.il, b.rh[2 * n], b.rh[2 * n + 1], b.rl[2 * n], b.rl[2 * n + 1]);
-        mma3(ri, a.rh, a.rl, b.ih[2 * n], b.ih[2 * n + 1], b.il[2 * n], b.il[2 * n + 1]);
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t(&ar)[4] = k == 0 ? a.rl : a.rh;
+        const uint32_t(&ai)[4] = k == 0 ? a.il : a.ih;
+        const uint32_t(&br)[4] = k == 1 ? b.rl : b.rh;
+        const uint32_t(&bi)[4] = k == 1 ? b.il : b.ih;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            re[n][i] = f * (kConj ? rr[i] + ii[i] : rr[i] - ii[i]);
-            im[n][i] = f * (kConj ? ir[i] - ri[i] : ir[i] + ri[i]);
+        for (int n = 0; n < 2; ++n) {
+            if (k == 0) {
+                mma_f16_z(rr[n], ar, br[2 * n], br[2 * n + 1]);
+                mma_f16_z(ii[n], ai, bi[2 * n], bi[2 * n + 1]);
+                mma_f16_z(ir[n], ai, br[2 * n], br[2 * n + 1]);
+                mma_f16_z(ri[n], ar, bi[2 * n], bi[2 * n + 1]);
+            } else {
+                mma_f16(rr[n], ar, br[2 * n], br[2 * n + 1]);
+                mma_f16(ii[n], ai, bi[2 * n], bi[2 * n + 1]);
+                mma_f16(ir[n], ai, br[2 * n], br[2 * n + 1]);
+                mma_f16(ri[n], ar, bi[2 * n], bi[2 * n + 1]);
+            }
         }
     }
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            re[n][i] = f * (kConj ? rr[n][i] + ii[n][i] : rr[n][i] - ii[n][i]);
+            im[n][i] = f * (kConj ? ir[n][i] - ri[n][i] : ir[n][i] + ri[n][i]);
+        }
 }
 
 // scale and split a [value x 16 tokens] matrix; returns the inverse scale
 __device__ __forceinline__ float make_frag(TokFrag &f, const float (&re)[2][4], const float (&im)[2][4])
 {
     float inv;
-    const float s = scale_for(__reduce_max_sync(0xffffffffu, max(max_bits4(re), max_bits4(im))), inv);
+    const float s = scale_for(warp_max(fmaxf(max_abs(re), max_abs(im))), inv);
     split_tiles(re[0], re[1], s, f.rh, f.rl);
     split_tiles(im[0], im[1], s, f.ih, f.il);
     return inv;
 }
 
-// S <- gamma_C S + sum_t a[., t] X[t][.]   (X: W-like tile read with tokens as k), unscaled by f
+// re, im (two key tiles of eight) = a X with tokens as k: X the tile at `at` (B operand by transposed loads);
+// nih, nil = the imaginary registers of `a` negated
 template <int DK>
-__device__ __forceinline__ void state_update(float (&sr)[DK / 16][4], float (&si)[DK / 16][4], const TokFrag &a, float f,
-                                             uint32_t tile, const float4 *__restrict__ gamma, int lane)
+__device__ __forceinline__ void tokens_product(float (&re)[2][4], float (&im)[2][4], const TokFrag &a, const uint32_t (&nih)[4],
+                                               const uint32_t (&nil)[4], uint32_t at)
 {
     using TL = Tile<DK>;
-    const uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
+    uint32_t brh[4], brl[4], bih[4], bil[4];
+    ldsm_t(brh, at);
+    ldsm_t(bih, at + 2 * TL::PL);
+    ldsm_t(brl, at + TL::PL);
+    ldsm_t(bil, at + 3 * TL::PL);
 #pragma unroll
-    for (int np = 0; np < TL::KT; np += 2) {
-        uint32_t brh[4], brl[4], bih[4], bil[4];
-        ldsm_t(brh, at + np * 16);
-        ldsm_t(brl, at + np * 16 + TL::PL);
-        ldsm_t(bih, at + np * 16 + 2 * TL::PL);
-        ldsm_t(bil, at + np * 16 + 3 * TL::PL);
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t(&ar)[4] = k == 0 ? a.rl : a.rh;
+        const uint32_t(&ai)[4] = k == 0 ? a.il : a.ih;
+        const uint32_t(&an)[4] = k == 0 ? nil : nih;
+        const uint32_t(&br)[4] = k == 1 ? brl : brh;
+        const uint32_t(&bi)[4] = k == 1 ? bil : bih;
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            float rr[4] = {0.f, 0.f, 0.f, 0.f}, ii[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
-            mma3(rr, a.rh, a.rl, brh[2 * e], brh[2 * e + 1], brl[2 * e], brl[2 * e + 1]);
-            mma3(im, a.ih, a.il, brh[2 * e], brh[2 * e + 1], brl[2 * e], brl[2 * e + 1]);
-            mma3(ii, a.ih, a.il, bih[2 * e], bih[2 * e + 1], bil[2 * e], bil[2 * e + 1]);
-            mma3(im, a.rh, a.rl, bih[2 * e], bih[2 * e + 1], bil[2 * e], bil[2 * e + 1]);
-            const int n = np + e;
-            const float4 g = gamma[4 * n + (lane & 3)];           // gamma_C of keys 8 n + 2 (lane & 3), + 1
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float gr = (i & 1) ? g.z : g.x, gi = (i & 1) ? g.w : g.y;
-                const float x = sr[n][i], y = si[n][i];
-                sr[n][i] = fmaf(f, rr[i] - ii[i], gr * x - gi * y);
-                si[n][i] = fmaf(f, im[i], gr * y + gi * x);
-            }
+        for (int n = 0; n < 2; ++n) {
+            if (k == 0) mma_f16_z(re[n], ar, br[2 * n], br[2 * n + 1]);
+            else mma_f16(re[n], ar, br[2 * n], br[2 * n + 1]);
         }
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            if (k == 0) mma_f16_z(im[n], ai, br[2 * n], br[2 * n + 1]);
+            else mma_f16(im[n], ai, br[2 * n], br[2 * n + 1]);
+        }
+#pragma unroll
+        for (int n = 0; n < 2; ++n) mma_f16(re[n], an, bi[2 * n], bi[2 * n + 1]);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) mma_f16(im[n], ar, bi[2 * n], bi[2 * n + 1]);
     }
 }
 
-// ---- PREP ---------------------------------------------------------------------------------------
-// Thread of AUX warp w: key 8 w + (lane >> 2), tokens 4 (lane & 3) .. + 3 of a chunk.
-struct PrepIn {
-    float kr[4], ki[4], qr[4], qi[4], al[4], th[4], be[4];
-};
-struct PrepVals {                             // what the gradients of a chunk need again
-    float kr[4], ki[4], qr[4], qi[4];         // rotated key and query (phases inside the chunk)
-    float a[4], sfx[4], cs[4], sn[4];         // prod alpha up to the token / after it; e^{i phi}
-};
-
-__device__ __forceinline__ float2 ld_pair(const float *p, size_t i) { return *reinterpret_cast<const float2 *>(p + i); }
-__device__ __forceinline__ float2 ld_pair(const __nv_bfloat16 *p, size_t i)
+// The thread's 16 elements (token 8 n + (i & 1), column + 8 (i >> 1)) of a [token][column] array: `p` points at the
+// first, `step` is a token's distance, `left` the number of tokens from p's on.
+template <typename T>
+__device__ __forceinline__ void load_rows(float (&x)[2][4], const T *p, size_t step, int left)
 {
-    const uint32_t u = *reinterpret_cast<const uint32_t *>(p + i);
-    return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+#pragma unroll
+    for (int n = 0; n < 2; ++n, p += 8 * step)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const T *r = p + (e ? step : 0);
+            const bool on = 8 * n + e < left;
+            x[n][e] = on ? ld_val(r, 0) : 0.f;
+            x[n][e + 2] = on ? ld_val(r, 8) : 0.f;
+        }
+}
+template <typename T>
+__device__ __forceinline__ void store_rows(T *p, const float (&x)[2][4], size_t step, int left)
+{
+#pragma unroll
+    for (int n = 0; n < 2; ++n, p += 8 * step)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            T *r = p + (e ? step : 0);
+            if (8 * n + e < left) {
+                st_val(r, 0, x[n][e]);
+                st_val(r, 8, x[n][e + 2]);
+            }
+        }
 }
 
-// q may be NULL (keys only)
-template <int DK, typename T>
-__device__ __forceinline__ void prep_load(PrepIn &in, const T *__restrict__ q, const T *__restrict__ k,
-                                          const float *__restrict__ alpha, const float *__restrict__ theta,
-                                          const float *__restrict__ beta, size_t row0, int H, int t0, int T_, int key, int t4)
+// The thread's fragment of a state [d_k][dv] (paired rows) at `p` (its key pair 2 (lane & 3), its column); returns the
+// largest magnitude.  p = NULL: zeros.
+template <int DK>
+__device__ __forceinline__ float state_from_memory(uint32_t st, const float *p, int dv)
 {
-    constexpr int M = DK / 2;
+    float largest = 0.f;
+#pragma unroll 1
+    for (int n = 0; n < Tile<DK>::KS; ++n) {
+        float x[16];
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
-        const int t = t0 + 4 * t4 + x;
-        in.kr[x] = in.ki[x] = in.qr[x] = in.qi[x] = in.th[x] = in.be[x] = 0.f;
-        in.al[x] = 1.f;
-        if (t < T_ && key < M) {
-            const size_t row = row0 + (size_t)t * H;
-            const float2 kk = ld_pair(k, row * DK + 2 * key);
-            in.kr[x] = kk.x;
-            in.ki[x] = kk.y;
-            if (q) {
-                const float2 qq = ld_pair(q, row * DK + 2 * key);
-                in.qr[x] = qq.x;
-                in.qi[x] = qq.y;
+        for (int i = 0; i < 16; ++i) {                            // [key tile][Re / Im][column half][key]
+            x[i] = p ? p[(size_t)(32 * n + 16 * (i >> 3) + 2 * (i & 1) + ((i >> 2) & 1)) * dv + 8 * ((i >> 1) & 1)] : 0.f;
+            largest = fmaxf(largest, fabsf(x[i]));
+        }
+        tm_store(st + 16 * n, x);
+    }
+    tm_wait_store();
+    return largest;
+}
+template <int DK>
+__device__ __forceinline__ void state_to_memory(uint32_t st, float *p, int dv)
+{
+#pragma unroll 1
+    for (int n = 0; n < Tile<DK>::KS; ++n) {
+        float x[16];
+        tm_load(x, st + 16 * n);
+        tm_wait_load(x);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) p[(size_t)(32 * n + 16 * (i >> 3) + 2 * (i & 1) + ((i >> 2) & 1)) * dv + 8 * ((i >> 1) & 1)] = x[i];
+    }
+}
+
+// S <- gamma_C S + f a Y, the state at `st`; returns the thread's largest magnitude of the new state
+template <int DK>
+__device__ __forceinline__ float state_update(uint32_t st, const TokFrag &a, float f, uint32_t tile, const float4 *gamma, int lane)
+{
+    using TL = Tile<DK>;
+    uint32_t nih[4], nil[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        nih[i] = a.ih[i] ^ 0x80008000u;
+        nil[i] = a.il[i] ^ 0x80008000u;
+    }
+    uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
+    gamma += lane & 3;
+    float largest = 0.f;
+#pragma unroll 1
+    for (int np = 0; np < TL::KS; ++np, at += 32, gamma += 8, st += 16) {
+        float x[16], re[2][4], im[2][4];
+        tm_load(x, st);
+        tokens_product<DK>(re, im, a, nih, nil, at);
+        tm_wait_load(x);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const float4 g = gamma[4 * n];                       // gamma_C of keys 8 n + 2 (lane & 3), + 1
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float gr = (i & 1) ? g.z : g.x, gi = (i & 1) ? g.w : g.y, u = x[8 * n + i], v = x[8 * n + 4 + i];
+                x[8 * n + i] = fmaf(f, re[n][i], gr * u - gi * v);
+                x[8 * n + 4 + i] = fmaf(f, im[n][i], gr * v + gi * u);
+                largest = fmaxf(largest, fmaxf(fabsf(x[8 * n + i]), fabsf(x[8 * n + 4 + i])));
             }
-            in.al[x] = alpha[row * M + key];
-            in.th[x] = theta[row * M + key];
+        }
+        tm_store(st, x);
+    }
+    tm_wait_store();
+    return largest;
+}
+
+// ---- PREP and SOLVE ------------------------------------------------------------------------------
+// PREP (PW warps): a thread owns two neighbouring keys and kC / NG consecutive tokens, so that global rows are read and
+// operand rows written in whole words.  The decays' products and the phases' sums cross the token groups through
+// shared memory.  SOLVE: one warp per Gram matrix, straight from the operand planes.
+template <int DK, int PW>
+struct PrepMap {
+    static constexpr int M = DK / 2, PAIRS = M / 2, NG = 32 * PW / PAIRS, TPT = kC / NG;
+    static_assert(NG * PAIRS == 32 * PW && TPT * NG == kC && TPT >= 1, "token groups must tile the chunk");
+    static constexpr int scan_bytes = NG * PAIRS * 16 + 4 * PW * 4;          // products, phase sums, the warps' maxima
+    static constexpr int slow_bytes = kC * (M + 4) * 8 * 3;                 // k', q', alpha of a chunk that is not fast
+};
+
+template <typename T> struct KeyPair;
+template <> struct KeyPair<float> {
+    float4 v;
+    __device__ __forceinline__ void zero() { v = make_float4(0.f, 0.f, 0.f, 0.f); }
+    __device__ __forceinline__ void load(const float *p) { v = *reinterpret_cast<const float4 *>(p); }
+    __device__ __forceinline__ float4 get() const { return v; }
+};
+template <> struct KeyPair<__nv_bfloat16> {
+    uint2 v;
+    __device__ __forceinline__ void zero() { v = make_uint2(0u, 0u); }
+    __device__ __forceinline__ void load(const __nv_bfloat16 *p) { v = *reinterpret_cast<const uint2 *>(p); }
+    __device__ __forceinline__ float4 get() const
+    {
+        return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                           __uint_as_float(v.y & 0xffff0000u));
+    }
+};
+
+template <int TPT, typename T>
+struct PrepRaw {
+    KeyPair<T> k[TPT], q[TPT];
+    float2 al[TPT], th[TPT];
+    float be[TPT];
+};
+
+template <int DK, int PW, bool kNeedQ, typename T>
+__device__ __forceinline__ void prep_fetch(PrepRaw<PrepMap<DK, PW>::TPT, T> &in, const T *__restrict__ q, const T *__restrict__ k,
+                                           const float *__restrict__ alpha, const float *__restrict__ theta,
+                                           const float *__restrict__ beta, size_t row0, int H, int t0, int T_, int tid)
+{
+    using PM = PrepMap<DK, PW>;
+    const int pair = tid % PM::PAIRS, t1 = t0 + tid / PM::PAIRS * PM::TPT;
+#pragma unroll
+    for (int x = 0; x < PM::TPT; ++x) {
+        in.k[x].zero();
+        in.q[x].zero();
+        in.al[x] = make_float2(1.f, 1.f);
+        in.th[x] = make_float2(0.f, 0.f);
+        in.be[x] = 0.f;
+        if (t1 + x < T_) {
+            const size_t row = row0 + (size_t)(t1 + x) * H;
+            in.k[x].load(k + row * DK + 4 * pair);
+            if constexpr (kNeedQ) in.q[x].load(q + row * DK + 4 * pair);
+            in.al[x] = *reinterpret_cast<const float2 *>(alpha + row * PM::M + 2 * pair);
+            in.th[x] = *reinterpret_cast<const float2 *>(theta + row * PM::M + 2 * pair);
             in.be[x] = beta[row];
         }
     }
 }
 
-// Scratch of PREP: fp32 copies of W, K = k' / a, Q for the Gram products, the two Gram matrices, the warps' maxima.
-template <int DK>
-struct PrepSmem {
-    static constexpr int M = DK / 2, LDF = M + 4;                 // float2 per token row
-    static constexpr int gram = 16 * 17;                          // float2
-    static constexpr int stage_bytes = 3 * 16 * LDF * 8;
-    static constexpr int small_bytes = 2 * (2 * gram * 8 + 4 * kAuxWarps * 4 + 16 * 4);   // two chunks deep
-};
-
-// Inverse of I + N (16 x 16 complex, N strictly lower, [17] float2 rows) by one warp: the two 8 x 8 diagonal blocks by
-// substitution (a lane owns half -- Re or Im -- of one column), then X21 = -X22 N21 X11.  The result replaces N.
-__device__ __forceinline__ void invert_unit_lower16(float2 *N, int lane)
-{
-    const int blk = (lane >> 3) & 1, c = lane & 7, part = lane >> 4;
-    float2 *B = N + blk * 8 * 17 + blk * 8;
-    float xr[8], xi[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-        for (int i = 0; i < t; ++i) {
-            const float2 n = B[t * 17 + i];
-            // Re: nr xr - ni xi; Im: nr xi + ni xr
-            s0 = fmaf(n.x, part ? xi[i] : xr[i], s0);
-            s1 = fmaf(part ? n.y : -n.y, part ? xr[i] : xi[i], s1);
-        }
-        const float own = ((t == c && part == 0) ? 1.f : 0.f) - (s0 + s1);
-        const float other = __shfl_xor_sync(0xffffffffu, own, 16);
-        xr[t] = part ? other : own;
-        xi[t] = part ? own : other;
-    }
-    __syncwarp();
-    if (part == 0) {
-#pragma unroll
-        for (int t = 0; t < 8; ++t) B[t * 17 + c] = make_float2(xr[t], xi[t]);
-    }
-    __syncwarp();
-    // T = N21 X11, then X21 = -X22 T: a lane owns row lane >> 2, columns 2 (lane & 3), + 1
-    const int r = lane >> 2, c0 = 2 * (lane & 3);
-    float2 acc[2];
-#pragma unroll
-    for (int pass = 0; pass < 2; ++pass) {
-        acc[0] = acc[1] = make_float2(0.f, 0.f);
-        const float2 *L = pass == 0 ? N + (8 + r) * 17 : N + (8 + r) * 17 + 8;
-        const float2 *R = pass == 0 ? N : N + 8 * 17;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float2 l = L[i];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const float2 x = R[i * 17 + c0 + e];
-                acc[e].x += l.x * x.x - l.y * x.y;
-                acc[e].y += l.x * x.y + l.y * x.x;
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-            N[(8 + r) * 17 + c0 + e] = pass == 0 ? acc[e] : make_float2(-acc[e].x, -acc[e].y);
-        __syncwarp();
-    }
-}
-
-// Splits a [16][16] matrix held by one warp ([17] float2 rows) into the four planes of a small tile.  Element (t, i)
-// is kept for i < t (strict == true) or i <= t, multiplied by w[i] when w is given.
-__device__ __forceinline__ void store_small(unsigned char *tile, const float2 *A, const float *w, bool mask, float *inv_out, int lane)
-{
-    // lane: column pair 2 (lane & 7), rows 4 (lane >> 3) .. + 3
-    const int i0 = 2 * (lane & 7), r0 = 4 * (lane >> 3);
-    float2 v[4][2];
-    uint32_t m = 0;
-#pragma unroll
-    for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            float2 a = A[(r0 + x) * 17 + i0 + e];
-            if (mask) {
-                const float f = w[i0 + e];
-                const bool keep = i0 + e <= r0 + x;
-                a = keep ? make_float2(a.x * f, a.y * f) : make_float2(0.f, 0.f);
-            }
-            v[x][e] = a;
-            m = max(m, max(abs_bits(a.x), abs_bits(a.y)));
-        }
-    float inv;
-    const float s = scale_for(__reduce_max_sync(0xffffffffu, m), inv);
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-        uint32_t h, l;
-        unsigned char *p = tile + (r0 + x) * 48 + i0 * 2;
-        split_f16(v[x][0].x * s, v[x][1].x * s, h, l);
-        *reinterpret_cast<uint32_t *>(p) = h;
-        *reinterpret_cast<uint32_t *>(p + 768) = l;
-        split_f16(v[x][0].y * s, v[x][1].y * s, h, l);
-        *reinterpret_cast<uint32_t *>(p + 2 * 768) = h;
-        *reinterpret_cast<uint32_t *>(p + 3 * 768) = l;
-    }
-    if (lane == 0) *inv_out = inv;
-}
-
-// One value pair (keys 2 p, 2 p + 1 of a token) would need an exchange between lanes; single 16-bit stores instead.
-__device__ __forceinline__ void store_planes(unsigned char *p, int pl, float re, float im)
+// two keys of one token into the four planes
+__device__ __forceinline__ void put_planes(unsigned char *p, int pl, float r0, float i0, float r1, float i1)
 {
     uint32_t h, l;
-    split_f16(re, im, h, l);
-    *reinterpret_cast<uint16_t *>(p) = (uint16_t)h;
-    *reinterpret_cast<uint16_t *>(p + pl) = (uint16_t)l;
-    *reinterpret_cast<uint16_t *>(p + 2 * pl) = (uint16_t)(h >> 16);
-    *reinterpret_cast<uint16_t *>(p + 3 * pl) = (uint16_t)(l >> 16);
+    split_f16(r0, r1, h, l);
+    *reinterpret_cast<uint32_t *>(p) = h;
+    *reinterpret_cast<uint32_t *>(p + pl) = l;
+    split_f16(i0, i1, h, l);
+    *reinterpret_cast<uint32_t *>(p + 2 * pl) = h;
+    *reinterpret_cast<uint32_t *>(p + 3 * pl) = l;
 }
 
-// Builds the operand tile of one chunk.  All AUX threads call it; the caller announces the slot afterwards.  `stage`
-// and `small` are PrepSmem; par alternates from chunk to chunk.  kNeedQ == false: W, Y, M only.
-// Returns whether the chunk took the fast path (no coordinate decays below 2^-80 inside it).
-template <int DK, bool kNeedQ>
-__device__ __forceinline__ bool prep_chunk(const PrepIn &in, PrepVals &pv, unsigned char *slot, float2 *stage,
-                                           unsigned char *small, int par, int tid)
+// Operand planes of one chunk: W, Y (and Q) into the slot, Kb_i = beta_i k_i / gamma_i into `kb` for the Gram products.
+// `vals` (or NULL) receives what the gradients need again, two float4 per (token, key): rotated key and query; prod
+// alpha up to the token and after it, e^{i phi}.  Called by all 32 PW threads; the planes are complete for other
+// threads only after a barrier of the caller's.
+//
+// The division by gamma_i is bounded by 2^16 inside a fast chunk (every coordinate keeps at least 2^-16 over the 16
+// tokens): Kb's entries then reach 2^16, the smaller ones keep an absolute error of 2^-39 of that, 2^-23 beside the
+// unit-sized entries of W they meet.  Stronger decays take slow_gram.  Returns whether the chunk is fast (the same
+// value in every thread).
+template <int DK, int PW, bool kNeedQ, typename T>
+__device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, T> &in, float4 *vals, unsigned char *slot,
+                                            unsigned char *kb, unsigned char *scan, int tid)
 {
+    using PM = PrepMap<DK, PW>;
     using TL = Tile<DK>;
-    using PS = PrepSmem<DK>;
-    constexpr int M = TL::M;
-    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3, key = 8 * warp + g;
-    const bool own = key < M;
-    unsigned char *sm = small + par * (PS::small_bytes / 2);
-    float2 *gk = reinterpret_cast<float2 *>(sm), *gq = gk + PS::gram;
-    float *red = reinterpret_cast<float *>(gq + PS::gram), *bsm = red + 4 * kAuxWarps;
-    float2 *sW = stage, *sK = stage + 16 * PS::LDF, *sQ = stage + 32 * PS::LDF;
+    constexpr int M = PM::M, PAIRS = PM::PAIRS, NG = PM::NG, TPT = PM::TPT;
+    const int pair = tid % PAIRS, grp = tid / PAIRS, lane = tid & 31, warp = tid >> 5;
+    float2 *sp = reinterpret_cast<float2 *>(scan);
+    uint2 *su = reinterpret_cast<uint2 *>(scan + NG * PAIRS * 8);
+    uint32_t *red = reinterpret_cast<uint32_t *>(scan + NG * PAIRS * 16);
 
-    // products of alpha and sums of the phase: inside the thread's four tokens, then over the key's four lanes
-    float p[4], sf[4];
-    uint32_t u[4];
-    p[0] = in.al[0];
-    u[0] = phase_to_turns(in.th[0]);
+    float2 p[TPT], sf[TPT];
+    uint2 u[TPT];
 #pragma unroll
-    for (int x = 1; x < 4; ++x) {
-        p[x] = p[x - 1] * in.al[x];
-        u[x] = u[x - 1] + phase_to_turns(in.th[x]);
-    }
-    sf[3] = 1.f;
-#pragma unroll
-    for (int x = 2; x >= 0; --x) sf[x] = sf[x + 1] * in.al[x + 1];
-    float inc = p[3], dec = p[3];
-    uint32_t ut = u[3];
-#pragma unroll
-    for (int d = 1; d < 4; d <<= 1) {
-        const float up = __shfl_up_sync(0xffffffffu, inc, d, 4), dn = __shfl_down_sync(0xffffffffu, dec, d, 4);
-        const uint32_t uu = __shfl_up_sync(0xffffffffu, ut, d, 4);
-        if (t4 >= d) {
-            inc *= up;
-            ut += uu;
+    for (int x = 0; x < TPT; ++x) {
+        p[x] = in.al[x];
+        u[x] = make_uint2(phase_to_turns(in.th[x].x), phase_to_turns(in.th[x].y));
+        if (x) {
+            p[x] = make_float2(p[x - 1].x * p[x].x, p[x - 1].y * p[x].y);
+            u[x] = make_uint2(u[x - 1].x + u[x].x, u[x - 1].y + u[x].y);
         }
-        if (t4 + d < 4) dec *= dn;
     }
-    float pre = __shfl_up_sync(0xffffffffu, inc, 1, 4), suf = __shfl_down_sync(0xffffffffu, dec, 1, 4);
-    uint32_t ub = __shfl_up_sync(0xffffffffu, ut, 1, 4);
-    if (t4 == 0) {
-        pre = 1.f;
-        ub = 0u;
-    }
-    if (t4 == 3) suf = 1.f;
-    const float aC = __shfl_sync(0xffffffffu, inc, 3, 4);
-
-    float Wr[4], Wi[4], Qr[4], Qi[4];
-    uint32_t mk = 0, my = 0, mq = 0;
+    sf[TPT - 1] = make_float2(1.f, 1.f);
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
-        pv.a[x] = pre * p[x];
-        pv.sfx[x] = sf[x] * suf;
-        turns_to_cos_sin(ub + u[x], &pv.cs[x], &pv.sn[x]);
-        pv.kr[x] = in.kr[x] * pv.cs[x] + in.ki[x] * pv.sn[x];
-        pv.ki[x] = in.ki[x] * pv.cs[x] - in.kr[x] * pv.sn[x];
-        Wr[x] = pv.a[x] * pv.kr[x];
-        Wi[x] = pv.a[x] * pv.ki[x];
-        mk = max(mk, max(abs_bits(Wr[x]), abs_bits(Wi[x])));
+    for (int x = TPT - 2; x >= 0; --x) sf[x] = make_float2(sf[x + 1].x * in.al[x + 1].x, sf[x + 1].y * in.al[x + 1].y);
+    sp[grp * PAIRS + pair] = p[TPT - 1];
+    su[grp * PAIRS + pair] = u[TPT - 1];
+    bar_sync(kBarAux, 32 * PW);
+    float2 pre = make_float2(1.f, 1.f), suf = pre, aC = pre;
+    uint2 ub = make_uint2(0u, 0u), uc = ub;
+#pragma unroll 2
+    for (int gg = 0; gg < NG; ++gg) {                              // the same order in every thread: aC decides `fast`
+        const float2 f = sp[gg * PAIRS + pair];
+        const uint2 v = su[gg * PAIRS + pair];
+        aC = make_float2(aC.x * f.x, aC.y * f.y);
+        uc = make_uint2(uc.x + v.x, uc.y + v.y);
+        if (gg < grp) {
+            pre = make_float2(pre.x * f.x, pre.y * f.y);
+            ub = make_uint2(ub.x + v.x, ub.y + v.y);
+        }
+        if (gg > grp) suf = make_float2(suf.x * f.x, suf.y * f.y);
+    }
+    const bool fast = __reduce_min_sync(0xffffffffu, __float_as_uint(fminf(aC.x, aC.y))) >= 0x37800000u;   // 2^-16
+    float2 gc0, gc1;                                              // e^{i phi_C}
+    cos_sin(uc.x, gc0.x, gc0.y);
+    cos_sin(uc.y, gc1.x, gc1.y);
+    if (grp == 0)
+        reinterpret_cast<float4 *>(slot + TL::oG)[pair] = make_float4(aC.x * gc0.x, aC.x * gc0.y, aC.y * gc1.x, aC.y * gc1.y);
+
+    float4 kk[TPT], qq[TPT];
+    float2 av[TPT], yf[TPT], bi[TPT];
+    float mw = 0.f, my = 0.f, mq = 0.f, mb = 0.f;
+#pragma unroll
+    for (int x = 0; x < TPT; ++x) {
+        const int t = grp * TPT + x;
+        av[x] = make_float2(pre.x * p[x].x, pre.y * p[x].y);
+        sf[x] = make_float2(sf[x].x * suf.x, sf[x].y * suf.y);
+        yf[x] = make_float2(sf[x].x * in.be[x], sf[x].y * in.be[x]);
+        float c0, s0, c1, s1;
+        cos_sin(ub.x + u[x].x, c0, s0);
+        cos_sin(ub.y + u[x].y, c1, s1);
+        float4 r = in.k[x].get();
+        kk[x] = make_float4(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0, r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
         if constexpr (kNeedQ) {
-            pv.qr[x] = in.qr[x] * pv.cs[x] + in.qi[x] * pv.sn[x];
-            pv.qi[x] = in.qi[x] * pv.cs[x] - in.qr[x] * pv.sn[x];
-            Qr[x] = pv.a[x] * pv.qr[x];
-            Qi[x] = pv.a[x] * pv.qi[x];
-            mq = max(mq, max(abs_bits(Qr[x]), abs_bits(Qi[x])));
+            r = in.q[x].get();
+            qq[x] = make_float4(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0, r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
+            if (vals) {
+                float4 *o = vals + (t * M + 2 * pair) * 2;
+                o[0] = make_float4(kk[x].x, kk[x].y, qq[x].x, qq[x].y);
+                o[1] = make_float4(av[x].x, sf[x].x, c0, s0);
+                o[2] = make_float4(kk[x].z, kk[x].w, qq[x].z, qq[x].w);
+                o[3] = make_float4(av[x].y, sf[x].y, c1, s1);
+            }
+            qq[x] = make_float4(av[x].x * qq[x].x, av[x].x * qq[x].y, av[x].y * qq[x].z, av[x].y * qq[x].w);
+            mq = fmaxf(fmaxf(mq, fmaxf(fabsf(qq[x].x), fabsf(qq[x].y))), fmaxf(fabsf(qq[x].z), fabsf(qq[x].w)));
         }
+        bi[x] = fast ? make_float2(__fdividef(in.be[x], av[x].x), __fdividef(in.be[x], av[x].y)) : make_float2(0.f, 0.f);
+        const float n0 = fabsf(kk[x].x) + fabsf(kk[x].y), n1 = fabsf(kk[x].z) + fabsf(kk[x].w);   // bounds both parts
+        mw = fmaxf(mw, fmaxf(av[x].x * n0, av[x].y * n1));
+        my = fmaxf(my, fmaxf(fabsf(yf[x].x) * n0, fabsf(yf[x].y) * n1));
+        mb = fmaxf(mb, fmaxf(fabsf(bi[x].x) * n0, fabsf(bi[x].y) * n1));
     }
-    const float gcs = __shfl_sync(0xffffffffu, pv.cs[3], 3, 4), gsn = __shfl_sync(0xffffffffu, pv.sn[3], 3, 4);
-    float Yr[4], Yi[4];
+    uint32_t m[4] = {__float_as_uint(mw), __float_as_uint(my), __float_as_uint(mq), __float_as_uint(mb)};   // all >= 0
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
-        const float f = pv.sfx[x] * in.be[x];
-        Yr[x] = f * (gcs * pv.kr[x] - gsn * pv.ki[x]);
-        Yi[x] = f * (gcs * pv.ki[x] + gsn * pv.kr[x]);
-        my = max(my, max(abs_bits(Yr[x]), abs_bits(Yi[x])));
+    for (int i = 0; i < 4; ++i)
+        if (kNeedQ || i != 2) m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+    if (lane == 0) *reinterpret_cast<uint4 *>(red + 4 * warp) = make_uint4(m[0], m[1], m[2], m[3]);
+    bar_sync(kBarAux, 32 * PW);
+#pragma unroll 2
+    for (int w = 0; w < PW; ++w) {
+        const uint4 r = *reinterpret_cast<const uint4 *>(red + 4 * w);
+        m[0] = max(m[0], r.x);
+        m[1] = max(m[1], r.y);
+        m[2] = max(m[2], r.z);
+        m[3] = max(m[3], r.w);
     }
-    if (own) {
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const int t = 4 * t4 + x;
-            const float ia = __frcp_rn(pv.a[x]);
-            sW[t * PS::LDF + key] = make_float2(Wr[x], Wi[x]);
-            sK[t * PS::LDF + key] = make_float2(pv.kr[x] * ia, pv.ki[x] * ia);
-            if constexpr (kNeedQ) sQ[t * PS::LDF + key] = make_float2(Qr[x], Qi[x]);
-        }
-        if (t4 == 3) reinterpret_cast<float2 *>(slot + TL::oG)[key] = make_float2(aC * gcs, aC * gsn);
-    }
-    if (warp == 0 && g == 0) {
-#pragma unroll
-        for (int x = 0; x < 4; ++x) bsm[4 * t4 + x] = in.be[x];
-    }
-    mk = __reduce_max_sync(0xffffffffu, mk);
-    my = __reduce_max_sync(0xffffffffu, my);
-    mq = __reduce_max_sync(0xffffffffu, mq);
-    const uint32_t lo = __reduce_min_sync(0xffffffffu, own ? __float_as_uint(aC) : 0x3f800000u);
-    if (lane == 0) {
-        red[warp] = __uint_as_float(mk);
-        red[8 + warp] = __uint_as_float(my);
-        red[16 + warp] = __uint_as_float(mq);
-        red[24 + warp] = __uint_as_float(lo);
-    }
-    bar_sync(kBarAux, kAux);
-    mk = my = mq = 0;
-    float amin = 1.f;
-#pragma unroll
-    for (int w = 0; w < kAuxWarps; ++w) {
-        mk = max(mk, __float_as_uint(red[w]));
-        my = max(my, __float_as_uint(red[8 + w]));
-        mq = max(mq, __float_as_uint(red[16 + w]));
-        amin = fminf(amin, red[24 + w]);
-    }
-    const bool fast = amin >= 0x1p-80f;
-    float *inv = reinterpret_cast<float *>(slot + TL::oS);
-    float ik, iy, iq;
-    const float sk = scale_for(mk, ik), sy = scale_for(my, iy), sq = scale_for(mq, iq);
+    float iw, iy, iq, ib;
+    const float sw = scale_for(__uint_as_float(m[0]), iw), sy = scale_for(__uint_as_float(m[1]), iy);
+    const float sq = scale_for(__uint_as_float(m[2]), iq), sb = scale_for(__uint_as_float(m[3]), ib);
     if (tid == 0) {
-        inv[0] = ik;
+        float *inv = reinterpret_cast<float *>(slot + TL::oS);
+        inv[0] = iw;
         inv[1] = iy;
         inv[2] = iq;
+        inv[5] = ib;
+        reinterpret_cast<int *>(inv)[6] = fast;
     }
-    if (own) {
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            unsigned char *row = slot + (4 * t4 + x) * TL::LDB + 2 * key;
-            store_planes(row + TL::oW, TL::PL, Wr[x] * sk, Wi[x] * sk);
-            store_planes(row + TL::oY, TL::PL, Yr[x] * sy, Yi[x] * sy);
-            if constexpr (kNeedQ) store_planes(row + TL::oQ, TL::PL, Qr[x] * sq, Qi[x] * sq);
+    for (int x = 0; x < TPT; ++x) {
+        const int at = (grp * TPT + x) * TL::LDB + 4 * pair;
+        const float w0 = av[x].x * sw, w1 = av[x].y * sw, y0 = yf[x].x * sy, y1 = yf[x].y * sy;
+        put_planes(slot + TL::oW + at, TL::PL, w0 * kk[x].x, w0 * kk[x].y, w1 * kk[x].z, w1 * kk[x].w);
+        put_planes(slot + TL::oY + at, TL::PL, y0 * (gc0.x * kk[x].x - gc0.y * kk[x].y), y0 * (gc0.x * kk[x].y + gc0.y * kk[x].x),
+                   y1 * (gc1.x * kk[x].z - gc1.y * kk[x].w), y1 * (gc1.x * kk[x].w + gc1.y * kk[x].z));
+        if constexpr (kNeedQ) put_planes(slot + TL::oQ + at, TL::PL, sq * qq[x].x, sq * qq[x].y, sq * qq[x].z, sq * qq[x].w);
+        if (fast) {
+            const float b0 = bi[x].x * sb, b1 = bi[x].y * sb;
+            put_planes(kb + at, TL::PL, b0 * kk[x].x, b0 * kk[x].y, b1 * kk[x].z, b1 * kk[x].w);
         }
-    }
-    if (fast) {
-        // K[t][i] = W_t^* K_i and A[t][i] = Q_t^* K_i, 3 x TF32: warp = (matrix, half of the columns, Re / Im)
-        const int which = warp & 1, nt = (warp >> 1) & 1, part = warp >> 2;
-        if (kNeedQ || which == 0) {
-            const float2 *A = which ? sQ : sW;
-            float acc0[4] = {0.f, 0.f, 0.f, 0.f}, acc1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int kk = 0; kk < TL::KT; ++kk) {
-                const float2 a0 = A[g * PS::LDF + 8 * kk + t4], a1 = A[(g + 8) * PS::LDF + 8 * kk + t4];
-                const float2 a2 = A[g * PS::LDF + 8 * kk + t4 + 4], a3 = A[(g + 8) * PS::LDF + 8 * kk + t4 + 4];
-                const float2 b0 = sK[(8 * nt + g) * PS::LDF + 8 * kk + t4], b1 = sK[(8 * nt + g) * PS::LDF + 8 * kk + t4 + 4];
-                uint32_t rh[4], rl[4], ih[4], il[4], ch[2], cl[2], dh[2], dl[2];
-                split_tf32(a0.x, rh[0], rl[0]);
-                split_tf32(a1.x, rh[1], rl[1]);
-                split_tf32(a2.x, rh[2], rl[2]);
-                split_tf32(a3.x, rh[3], rl[3]);
-                split_tf32(a0.y, ih[0], il[0]);
-                split_tf32(a1.y, ih[1], il[1]);
-                split_tf32(a2.y, ih[2], il[2]);
-                split_tf32(a3.y, ih[3], il[3]);
-                // Re: Ar Kr + Ai Ki;  Im: Ar Ki - Ai Kr
-                split_tf32(part ? b0.y : b0.x, ch[0], cl[0]);
-                split_tf32(part ? b1.y : b1.x, ch[1], cl[1]);
-                split_tf32(part ? -b0.x : b0.y, dh[0], dl[0]);
-                split_tf32(part ? -b1.x : b1.y, dh[1], dl[1]);
-                mma3_tf32(acc0, rh, rl, ch, cl);
-                mma3_tf32(acc1, ih, il, dh, dl);
-            }
-            float *dst = reinterpret_cast<float *>(which ? gq : gk) + part;
-            const int i = 8 * nt + 2 * t4;
-            dst[2 * (g * 17 + i)] = acc0[0] + acc1[0];
-            dst[2 * (g * 17 + i + 1)] = acc0[1] + acc1[1];
-            dst[2 * ((g + 8) * 17 + i)] = acc0[2] + acc1[2];
-            dst[2 * ((g + 8) * 17 + i + 1)] = acc0[3] + acc1[3];
-        }
-    } else {
-        // A coordinate decays too far to divide: every pair's decay as a running product.  The staging now takes k',
-        // q' and alpha; a warp does rows warp and warp + 8, a lane keys lane, lane + 32.
-        bar_sync(kBarAux, kAux);
-        if (own) {
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                const int t = 4 * t4 + x;
-                sW[t * PS::LDF + key] = make_float2(pv.kr[x], pv.ki[x]);
-                sK[t * PS::LDF + key] = make_float2(in.al[x], 0.f);
-                if constexpr (kNeedQ) sQ[t * PS::LDF + key] = make_float2(pv.qr[x], pv.qi[x]);
-            }
-        }
-        bar_sync(kBarAux, kAux);
-        for (int t = warp; t < 16; t += 8) {
-            float w[2] = {1.f, 1.f};
-            for (int i = t; i >= 0; --i) {
-                float s[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int e = 0; e < M / 32; ++e) {
-                    const int j = lane + 32 * e;
-                    const float2 b = sW[i * PS::LDF + j], x = sW[t * PS::LDF + j];
-                    const float br = w[e] * b.x, bi = w[e] * b.y;
-                    s[0] += x.x * br + x.y * bi;
-                    s[1] += x.x * bi - x.y * br;
-                    if constexpr (kNeedQ) {
-                        const float2 y = sQ[t * PS::LDF + j];
-                        s[2] += y.x * br + y.y * bi;
-                        s[3] += y.x * bi - y.y * br;
-                    }
-                    w[e] *= sK[i * PS::LDF + j].x;
-                }
-#pragma unroll
-                for (int d = 16; d >= 1; d >>= 1)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) s[e] += __shfl_xor_sync(0xffffffffu, s[e], d);
-                if (lane == 0) {
-                    gk[t * 17 + i] = make_float2(s[0], s[1]);
-                    if constexpr (kNeedQ) gq[t * 17 + i] = make_float2(s[2], s[3]);
-                }
-            }
-        }
-    }
-    bar_sync(kBarAux, kAux);
-    if (warp == 0) {
-        // N = K D_beta, strictly lower; only its lower part is read
-        for (int e = lane; e < 256; e += 32) {
-            const int t = e >> 4, i = e & 15;
-            const float2 x = gk[t * 17 + i];
-            const float f = i < t ? bsm[i] : 0.f;
-            gk[t * 17 + i] = i < t ? make_float2(x.x * f, x.y * f) : make_float2(0.f, 0.f);
-        }
-        __syncwarp();
-        invert_unit_lower16(gk, lane);
-        store_small(slot + TL::oM, gk, nullptr, false, inv + 3, lane);
-    } else if (kNeedQ && warp == 1) {
-        store_small(slot + TL::oA, gq, bsm, true, inv + 4, lane);
     }
     return fast;
+}
+
+// The Gram matrices of a chunk whose decays are too strong to divide by: every pair's decay as a running product.  Called
+// by all 32 PW threads after prep_planes returned false; `slow` is a scratch of PrepMap::slow_bytes nobody else uses.
+// Reads its inputs again: passed on, they would not stay in registers on the common path.
+template <int DK, int PW, bool kNeedQ, typename T>
+__device__ __noinline__ void slow_gram(const T *q, const T *k, const float *alpha, const float *theta, const float *beta,
+                                       size_t row0, int H, int t0, int T_, unsigned char *slow, const unsigned char *scan,
+                                       float2 *gk, float2 *gq, int tid)
+{
+    using PM = PrepMap<DK, PW>;
+    PrepRaw<PM::TPT, T> in;
+    prep_fetch<DK, PW, kNeedQ, T>(in, q, k, alpha, theta, beta, row0, H, t0, T_, tid);
+    constexpr int M = PM::M, PAIRS = PM::PAIRS, TPT = PM::TPT, LD = M + 4;
+    const int pair = tid % PAIRS, grp = tid / PAIRS, lane = tid & 31, warp = tid >> 5;
+    const uint2 *su = reinterpret_cast<const uint2 *>(scan + PM::NG * PAIRS * 8);
+    float2 *sk = reinterpret_cast<float2 *>(slow), *sq = sk + kC * LD, *sa = sq + kC * LD;   // sa: (alpha, beta)
+    uint2 ub = make_uint2(0u, 0u);
+    for (int gg = 0; gg < grp; ++gg) ub = make_uint2(ub.x + su[gg * PAIRS + pair].x, ub.y + su[gg * PAIRS + pair].y);
+#pragma unroll
+    for (int x = 0; x < TPT; ++x) {
+        const int at = (grp * TPT + x) * LD + 2 * pair;
+        ub = make_uint2(ub.x + phase_to_turns(in.th[x].x), ub.y + phase_to_turns(in.th[x].y));
+        float c0, s0, c1, s1;
+        cos_sin(ub.x, c0, s0);
+        cos_sin(ub.y, c1, s1);
+        float4 r = in.k[x].get();
+        sk[at] = make_float2(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0);
+        sk[at + 1] = make_float2(r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
+        if constexpr (kNeedQ) {
+            r = in.q[x].get();
+            sq[at] = make_float2(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0);
+            sq[at + 1] = make_float2(r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
+        }
+        sa[at] = make_float2(in.al[x].x, in.be[x]);
+        sa[at + 1] = make_float2(in.al[x].y, in.be[x]);
+    }
+    bar_sync(kBarAux, 32 * PW);
+    for (int t = warp; t < kC; t += PW) {
+        float w[M / 32];
+#pragma unroll
+        for (int e = 0; e < M / 32; ++e) w[e] = 1.f;
+        for (int i = t; i >= 0; --i) {
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+            float be = 0.f;
+#pragma unroll
+            for (int e = 0; e < M / 32; ++e) {
+                const int j = lane + 32 * e;
+                const float2 b = sk[i * LD + j], x = sk[t * LD + j], ab = sa[i * LD + j];
+                const float br = w[e] * b.x, bim = w[e] * b.y;
+                s[0] += x.x * br + x.y * bim;
+                s[1] += x.x * bim - x.y * br;
+                if constexpr (kNeedQ) {
+                    const float2 y = sq[t * LD + j];
+                    s[2] += y.x * br + y.y * bim;
+                    s[3] += y.x * bim - y.y * br;
+                }
+                w[e] *= ab.x;
+                be = ab.y;
+            }
+#pragma unroll
+            for (int d = 16; d >= 1; d >>= 1)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[e] += __shfl_xor_sync(0xffffffffu, s[e], d);
+            if (lane == 0) {
+                gk[t * 17 + i] = make_float2(be * s[0], be * s[1]);
+                if constexpr (kNeedQ) gq[t * 17 + i] = make_float2(be * s[2], be * s[3]);
+            }
+        }
+    }
+}
+
+// X^* Kb (X = W or Q) for the columns 8 nt0 .. of NT tiles of eight, by one warp, into [17] float2 rows
+template <int DK, int NT>
+__device__ __forceinline__ void gram_tiles(uint32_t x, uint32_t kb, float f, float2 *out, int nt0, int lane)
+{
+    using TL = Tile<DK>;
+    const int g = lane >> 2, t4 = lane & 3;
+    uint32_t pa = x + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
+    // B registers of both halves of a k-step for the heads (lanes 0-15) and the tails (lanes 16-31)
+    uint32_t pb = kb + (uint32_t)((8 * nt0 + (lane & 7)) * TL::LDB + ((lane >> 3) & 1) * 16 + (lane >> 4) * TL::PL);
+    float re[NT][4], im[NT][4], ni[NT][4];
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) re[n][i] = im[n][i] = ni[n][i] = 0.f;
+#pragma unroll 1
+    for (int kk = 0; kk < TL::KS; ++kk, pa += 32, pb += 32) {
+        uint32_t rh[4], rl[4], ih[4], il[4], br[NT][4], bi[NT][4];
+        ldsm(rh, pa);
+        ldsm(ih, pa + 2 * TL::PL);
+        ldsm(rl, pa + TL::PL);
+        ldsm(il, pa + 3 * TL::PL);
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            ldsm(br[n], pb + n * 8 * TL::LDB);
+            ldsm(bi[n], pb + n * 8 * TL::LDB + 2 * TL::PL);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t(&ar)[4] = k == 0 ? rl : rh;
+            const uint32_t(&ai)[4] = k == 0 ? il : ih;
+            const int o = k == 1 ? 2 : 0;
+#pragma unroll
+            for (int n = 0; n < NT; ++n) mma_f16(re[n], ar, br[n][o], br[n][o + 1]);
+#pragma unroll
+            for (int n = 0; n < NT; ++n) mma_f16(im[n], ar, bi[n][o], bi[n][o + 1]);
+#pragma unroll
+            for (int n = 0; n < NT; ++n) mma_f16(re[n], ai, bi[n][o], bi[n][o + 1]);
+#pragma unroll
+            for (int n = 0; n < NT; ++n) mma_f16(ni[n], ai, br[n][o], br[n][o + 1]);
+        }
+    }
+    out += g * 17 + 8 * nt0 + 2 * t4;
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) out[8 * 17 * (i >> 1) + 8 * n + (i & 1)] = make_float2(f * re[n][i], f * (im[n][i] - ni[n][i]));
+}
+
+// Inverse of I + N (16 x 16 complex, [17] float2 rows, only the strictly lower part of N is read) by one warp, in place:
+// X21 = -X22 N21 X11 for blocks of 1, 2, 4, 8 rows, one short loop for all of them.
+__device__ __forceinline__ void invert_unit_lower16(float2 *N, int lane)
+{
+#pragma unroll 1
+    for (int e = lane; e < 256; e += 32) {
+        const int t = e >> 4, i = e & 15;
+        if (i >= t) N[t * 17 + i] = make_float2(i == t ? 1.f : 0.f, 0.f);
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int lg = 0; lg < 4; ++lg) {
+        const int n = 1 << lg;                                    // 8 n elements of X21 altogether; n = 8: two per lane
+        const int first = (lane >> (2 * lg)) << (lg + 1), c = first + (lane & (n - 1)), r = first + n + ((lane >> lg) & (n - 1));
+        const bool on = lane < 8 * n, two = n == 8;
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {
+            const float2 *L = N + r * 17 + first + pass * n, *R = N + (first + pass * n) * 17 + c;
+            float2 x = make_float2(0.f, 0.f), y = x;
+            if (on) {
+#pragma unroll 1
+                for (int i = 0; i < n; ++i, ++L, R += 17) {
+                    const float2 u = *R, l = *L;
+                    x.x += l.x * u.x - l.y * u.y;
+                    x.y += l.x * u.y + l.y * u.x;
+                    if (two) {
+                        const float2 l2 = L[4 * 17];
+                        y.x += l2.x * u.x - l2.y * u.y;
+                        y.y += l2.x * u.y + l2.y * u.x;
+                    }
+                }
+            }
+            __syncwarp();
+            const float sg = pass ? -1.f : 1.f;
+            if (on) N[r * 17 + c] = make_float2(sg * x.x, sg * x.y);
+            if (two) N[(r + 4) * 17 + c] = make_float2(sg * y.x, sg * y.y);
+            __syncwarp();
+        }
+    }
+}
+
+// The lower triangle (diagonal included) of a [17] float2 matrix into the four planes of a small tile, by one warp
+__device__ __forceinline__ void store_lower(unsigned char *tile, const float2 *A, float *inv_out, int lane)
+{
+    const int i0 = 2 * (lane & 7), r0 = lane >> 3;                            // a lane: two columns, every fourth row
+    const float2 *p = A + r0 * 17 + i0;
+    float m = 0.f;
+#pragma unroll
+    for (int r = 0; r < 16; r += 4) {
+        const float2 x = p[r * 17], y = p[r * 17 + 1];
+        if (i0 <= r0 + r) m = fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.y)));
+        if (i0 + 1 <= r0 + r) m = fmaxf(m, fmaxf(fabsf(y.x), fabsf(y.y)));
+    }
+    float inv;
+    const float s = scale_for(warp_max(m), inv);
+    tile += r0 * 48 + i0 * 2;
+#pragma unroll 1
+    for (int r = 0; r < 16; r += 4, tile += 4 * 48) {
+        const float2 zero = make_float2(0.f, 0.f);
+        const float2 x = i0 <= r0 + r ? p[r * 17] : zero, y = i0 + 1 <= r0 + r ? p[r * 17 + 1] : zero;
+        put_planes(tile, 768, x.x * s, x.y * s, y.x * s, y.y * s);
+    }
+    if (lane == 0) *inv_out = inv;
 }
 
 }  // namespace c16

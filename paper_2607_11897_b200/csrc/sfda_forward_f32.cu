@@ -7,10 +7,9 @@
 // One CTA per (batch, head) pair and block of value columns; sfda_chunk16.cuh describes the arithmetic (split fp16 on
 // the tensor cores) and the two roles, which are pipelined over a ring of operand tiles.
 //
-// What bounds it: the latency of a chunk's dependent steps (scan, Gram products, inverse in the AUX warps; the three
-// products in the chain warps), not memory.  B = 2, T = 2001, H = 16, d = 128, fp32: 3154 us with the CUDA-core
-// kernel (an exponential per pair and coordinate, loops over shared memory), 665 us with this one; B = 1, T = 256,
-// H = 2, d = 64: 201 -> 61 us.
+// What bounds it: the schedulers' issue slots, which mma.sync holds (see Roles).  Measured in cycles per 16 tokens:
+// 6.4 k with 32 value columns per CTA (B = 2, T = 2001, H = 16, d = 128, fp32: 422 us; the unrolled first version 665 us,
+// the CUDA-core kernel 3154 us), 11.4 k with 128 columns; B = 1, T = 256, H = 2, d = 64: 43 us (61, 201).
 #include "sfda_chunk16.cuh"
 #include "sfda_internal.h"
 
@@ -27,129 +26,166 @@ struct FwdArgsDev {
     int T, H, dv;
 };
 
-template <int DK>
+constexpr int kPrepWarps = 8, kPrep = 32 * kPrepWarps, kSolve = 128;
+constexpr int kBarPlanes = kBarFree;                             // + slot: planes ready (the forward needs no FREE)
+
+// Which warp does what.  A warp runs on scheduler (warp % 4), and mma.sync holds its scheduler: measured, 8.2 cycles each
+// and 0.7 more for every other instruction issued meanwhile.  With 32 columns the two chain warps would share theirs
+// with a quarter of PREP each (7.2 k cycles per chunk); so PREP goes to schedulers 2 and 3, chain and SOLVE to 0 and 1.
+template <int NB>
+struct Roles {
+    static constexpr int threads = NB == 32 ? 512 : kPrep + kSolve + 2 * NB;
+    int prep = -1, solve = -1, chain = -1;                       // thread index inside the role, or -1
+    __device__ explicit Roles(int tid)
+    {
+        if constexpr (NB == 32) {
+            const int w = tid >> 5, lane = tid & 31;
+            if (w & 2) prep = ((w >> 2) * 2 + (w & 1)) * 32 + lane;
+            else if (w < 2) chain = tid;
+            else if (w < 12) solve = (((w >> 2) - 1) * 2 + (w & 1)) * 32 + lane;
+        } else {
+            if (tid < kPrep) prep = tid;
+            else if (tid < kPrep + kSolve) solve = tid - kPrep;
+            else chain = tid - kPrep - kSolve;
+        }
+    }
+};
+
+template <int DK, int NB>
 struct FwdSmem {
-    static constexpr int stage = kSlots * Tile<DK>::bytes;
-    static constexpr int small = stage + PrepSmem<DK>::stage_bytes;
-    static constexpr int bytes = small + PrepSmem<DK>::small_bytes;
+    using PM = PrepMap<DK, kPrepWarps>;
+    static constexpr int kb = kSlots * Tile<DK>::bytes;          // Kb planes, a slot each
+    static constexpr int gram = kb + kSlots * Tile<DK>::BIG;     // the two Gram matrices, a slot each
+    static constexpr int gram_bytes = 2 * 16 * 17 * 8;
+    static constexpr int scan = gram + kSlots * gram_bytes;
+    static constexpr int slow = scan + (PM::scan_bytes + 127) / 128 * 128;
+    static constexpr int bytes = slow + PM::slow_bytes;          // its first word also passes the tensor-memory address on
+    static constexpr int columns = (NB + 63) / 64 * DK / 2 < 32 ? 32 : (NB + 63) / 64 * DK / 2;
 };
 
 template <int DK, int NB, typename T>
-__global__ void __launch_bounds__(kAux + 2 * NB, 1) sfda_forward_f32_kernel(const FwdArgsDev a)
+__global__ void __launch_bounds__(Roles<NB>::threads, 1) sfda_forward_f32_kernel(const FwdArgsDev a)
 {
     using TL = Tile<DK>;
-    constexpr int kAll = kAux + 2 * NB;
+    using L = FwdSmem<DK, NB>;
+    constexpr int kChain = 2 * NB;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
     const size_t row0 = (size_t)b * a.T * a.H + h;               // row of token t: row0 + t H
     const int nch = (a.T + kC - 1) / kC;
+    if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::slow), L::columns);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::slow);
+    __syncthreads();
 
-    if (tid < kAux) {
-        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
-        const int key = 8 * (tid >> 5) + ((tid & 31) >> 2), t4 = tid & 3;
+    const Roles<NB> role(tid);
+    if (role.prep >= 0) {
+        // register shares with all 128 value columns: 256 x 88 + 128 x 72 + 256 x 112 of the launch's 640 x 96
+        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
         const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
-        PrepIn in;
-        prep_load<DK, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, 0, a.T, key, t4);
+        PrepRaw<L::PM::TPT, T> in;
+        prep_fetch<DK, kPrepWarps, true, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, 0, a.T, role.prep);
         for (int c = 0; c < nch; ++c) {
             const int slot = c % kSlots;
-            if (c >= kSlots) bar_sync(kBarDone + slot, kAll);
-            PrepIn next = in;
-            if (c + 1 < nch) prep_load<DK, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, (c + 1) * kC, a.T, key, t4);
-            PrepVals pv;
-            prep_chunk<DK, true>(in, pv, smem + slot * TL::bytes, reinterpret_cast<float2 *>(smem + FwdSmem<DK>::stage),
-                                 smem + FwdSmem<DK>::small, c & 1, tid);
-            bar_arrive(kBarFull + slot, kAll);
+            if (c >= kSlots) bar_sync(kBarDone + slot, kPrep + kChain);
+            PrepRaw<L::PM::TPT, T> next;
+            prep_fetch<DK, kPrepWarps, true, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, (c + 1) * kC, a.T, role.prep);
+            float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes);
+            if (!prep_planes<DK, kPrepWarps, true, T>(in, nullptr, smem + slot * TL::bytes, smem + L::kb + slot * TL::BIG, smem + L::scan, role.prep))
+                slow_gram<DK, kPrepWarps, true, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, smem + L::slow, smem + L::scan,
+                                                   gk, gk + 16 * 17, role.prep);
+            bar_arrive(kBarPlanes + slot, kPrep + 64);
             in = next;
         }
-        return;
-    }
-
-    if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
-    const int lane = tid & 31, w = (tid - kAux) >> 5, g = lane >> 2, t4 = lane & 3;
-    const int col = c0 + 16 * w + g;                             // and col + 8
-    const T *v = static_cast<const T *>(a.v);
-    float sr[TL::KT][4], si[TL::KT][4];
-#pragma unroll
-    for (int n = 0; n < TL::KT; ++n)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const size_t at = ((size_t)bh * DK + 2 * (8 * n + 2 * t4 + (i & 1))) * a.dv + col + 8 * (i >> 1);
-            sr[n][i] = a.S0 ? a.S0[at] : 0.f;
-            si[n][i] = a.S0 ? a.S0[at + a.dv] : 0.f;
+    } else if (role.solve >= 0) {
+        // warps 0, 1: the system's inverse of even / odd chunks; warps 2, 3: the outputs' Gram matrix of them
+        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        const int lane = tid & 31, w = role.solve >> 5, out = w >> 1;
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+        for (int c = w & 1; c < nch; c += 2) {
+            const int slot = c % kSlots;
+            unsigned char *tile = smem + slot * TL::bytes;
+            float *inv = reinterpret_cast<float *>(tile + TL::oS);
+            float2 *gm = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes) + out * 16 * 17;
+            bar_sync(kBarPlanes + slot, kPrep + 64);
+            if (reinterpret_cast<const int *>(inv)[6])
+                gram_tiles<DK, 2>(base + slot * TL::bytes + (out ? TL::oQ : TL::oW), base + L::kb + slot * TL::BIG, inv[out ? 2 : 0] * inv[5], gm, 0, lane);
+            __syncwarp();
+            if (!out) invert_unit_lower16(gm, lane);
+            store_lower(tile + (out ? TL::oA : TL::oM), gm, inv + 3 + out, lane);
+            bar_arrive(kBarFull + slot, 64 + kChain);
         }
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
-    for (int c = 0; c < nch; ++c) {
-        const int slot = c % kSlots;
-        float rr[2][4], ri[2][4];
+    } else if (role.chain >= 0) {
+        if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+        const int lane = tid & 31, w = role.chain >> 5, g = lane >> 2, t4 = lane & 3;
+        const int col = c0 + 16 * w + g;                         // and col + 8
+        const uint32_t st = tmem + ((uint32_t)(w & 3) << 21) + (w >> 2) * 8 * TL::KT;    // this warp's lanes and columns
+        const size_t state_at = ((size_t)bh * DK + 4 * t4) * a.dv + col;
+        float largest = state_from_memory<DK>(st, a.S0 ? a.S0 + state_at : nullptr, a.dv);
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+        const size_t step = (size_t)a.H * a.dv;
+        size_t at = (row0 + (size_t)(2 * t4) * a.H) * a.dv + col;
+        for (int c = 0; c < nch; ++c, at += 16 * step) {
+            const int slot = c % kSlots, left = a.T - c * kC - 2 * t4;
+            float rr[2][4], ri[2][4];
+            load_rows(rr, static_cast<const T *>(a.v) + at, step, left);
+            float isv;
+            const float ss = scale_for(warp_max(largest), isv);
+            bar_sync(kBarFull + slot, 64 + kChain);
+            const uint32_t tile = base + slot * TL::bytes;
+            const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
+            float acc[2][3][2][4];
+            const uint32_t tiles[2] = {tile + TL::oW, tile + TL::oQ};
+            keys_product<DK, 2>(acc, st, ss, tiles, lane, [](int, const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4]) {});
+            const float fw = isv * inv[0], fq = isv * inv[2];
 #pragma unroll
-        for (int n = 0; n < 2; ++n)
+            for (int n = 0; n < 2; ++n)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int t = c * kC + 8 * n + 2 * t4 + (i & 1);
-                rr[n][i] = t < a.T ? ld_val(v, (row0 + (size_t)t * a.H) * a.dv + col + 8 * (i >> 1)) : 0.f;
-            }
-        bar_sync(kBarFull + slot, kAll);
-        const uint32_t tile = base + slot * TL::bytes;
-        const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
-        float isv;
-        const float ss = scale_for(__reduce_max_sync(0xffffffffu, max(max_bits4(sr), max_bits4(si))), isv);
-        float acc[2][3][2][4];
-        const uint32_t tiles[2] = {tile + TL::oW, tile + TL::oQ};
-        product_over_keys<DK, 2, false>(acc, sr, si, ss, tiles, lane, nullptr);
-        const float fw = isv * inv[0], fq = isv * inv[2];
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
-                ri[n][i] = -fw * (acc[0][1][n][i] - acc[0][2][n][i]);
-            }
-        TokFrag fr, fb;
-        const float ir = make_frag(fr, rr, ri);
-        load_small<false>(fb, tile + TL::oM, lane);
-        float ur[2][4], ui[2][4];
-        product_small<false>(ur, ui, fr, fb, ir * inv[3]);
-        const float iu = make_frag(fr, ur, ui);
-        load_small<false>(fb, tile + TL::oA, lane);
-        product_small<false>(rr, ri, fr, fb, iu * inv[4]);
-        state_update<DK>(sr, si, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
-        if (c + kSlots < nch) bar_arrive(kBarDone + slot, kAll);
-        T *o = static_cast<T *>(a.o), *oi = static_cast<T *>(a.o_im);
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int t = c * kC + 8 * n + 2 * t4 + (i & 1);
-                if (t < a.T) {
-                    const size_t at = (row0 + (size_t)t * a.H) * a.dv + col + 8 * (i >> 1);
-                    st_val(o, at, fmaf(fq, acc[1][0][n][i], rr[n][i]));
-                    if (oi) st_val(oi, at, -fmaf(fq, acc[1][1][n][i] - acc[1][2][n][i], ri[n][i]));
+                for (int i = 0; i < 4; ++i) {
+                    rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
+                    ri[n][i] = -fw * (acc[0][1][n][i] - acc[0][2][n][i]);
                 }
+            TokFrag fr;
+            float iu;
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {               // U = M R, then (A^{qk} D_beta) U
+                TokFrag fb;
+                iu = make_frag(fr, rr, ri);
+                load_small<false>(fb, tile + (pass ? TL::oA : TL::oM), lane);
+                product_small<false>(rr, ri, fr, fb, iu * inv[3 + pass]);
             }
-    }
-    if (a.S_T) {
+            largest = state_update<DK>(st, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
+            if (c + kSlots < nch) bar_arrive(kBarDone + slot, kPrep + kChain);
 #pragma unroll
-        for (int n = 0; n < TL::KT; ++n)
+            for (int n = 0; n < 2; ++n)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const size_t at = ((size_t)bh * DK + 2 * (8 * n + 2 * t4 + (i & 1))) * a.dv + col + 8 * (i >> 1);
-                a.S_T[at] = sr[n][i];
-                a.S_T[at + a.dv] = si[n][i];
-            }
+                for (int i = 0; i < 4; ++i) {
+                    rr[n][i] = fmaf(fq, acc[1][0][n][i], rr[n][i]);
+                    ri[n][i] = -fmaf(fq, acc[1][1][n][i] - acc[1][2][n][i], ri[n][i]);
+                }
+            store_rows(static_cast<T *>(a.o) + at, rr, step, left);
+            if (a.o_im) store_rows(static_cast<T *>(a.o_im) + at, ri, step, left);
+        }
+        if (a.S_T) state_to_memory<DK>(st, a.S_T + state_at, a.dv);
     }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid < 32) tm_free(tmem, L::columns);
 }
 
 template <int DK, int NB, typename T>
 cudaError_t launch_nb(const ForwardArgs &x, cudaStream_t stream)
 {
     auto kern = sfda_forward_f32_kernel<DK, NB, T>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<DK>::bytes);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<DK, NB>::bytes);
     if (e != cudaSuccess) return e;
     FwdArgsDev a;
     a.q = x.q; a.k = x.k; a.v = x.v; a.alpha = x.alpha; a.theta = x.theta; a.beta = x.beta; a.S0 = x.S0;
     a.o = x.o; a.o_im = x.o_im; a.S_T = x.S_T;
     a.T = x.T; a.H = x.H; a.dv = x.d_v;
-    kern<<<dim3((unsigned)(x.B * x.H), (unsigned)(x.d_v / NB)), kAux + 2 * NB, FwdSmem<DK>::bytes, stream>>>(a);
+    kern<<<dim3((unsigned)(x.B * x.H), (unsigned)(x.d_v / NB)), Roles<NB>::threads, FwdSmem<DK, NB>::bytes, stream>>>(a);
     return cudaGetLastError();
 }
 
