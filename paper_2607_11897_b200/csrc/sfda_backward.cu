@@ -24,11 +24,10 @@
 // CHAIN warps walk the sequence forward once, keeping the state every 64 tokens, then per segment of 64 tokens, last to
 // first: forward again from the checkpoint, backward through it.  They leave S_0, U, G_C, Bc of a chunk in a scratch
 // ring as the operand registers of the gradients' products.  The AUX warps prepare the chunks' operand tiles and turn
-// what the chain leaves into gradients one chunk behind it.  The two meet at hardware barriers, one per slot:
-//   FULL  operand tile ready       DONE  the chain is through with a chunk       FREE  its gradients are written
-#include <type_traits>
-
-#include "sfda_chunk16_unrolled.cuh"
+// what the chain leaves into gradients one chunk behind it; SOLVE warps make the Gram matrices and the inverse.  They
+// meet at hardware barriers: PLANES (operand planes ready), FULL (the tile is complete), DONE (the chain is
+// through with the chunk); AUX prepares a slot again only after it has written that slot's gradients.
+#include "sfda_chunk16.cuh"
 #include "sfda_internal.h"
 
 namespace sfda {
@@ -39,6 +38,10 @@ using namespace c16;
 constexpr int kSeg = 64;                    // tokens between checkpoints
 constexpr int kSegChunks = kSeg / kC;
 static_assert(kSegChunks == kSlots, "a segment's operand tiles fill the ring");
+constexpr int kAuxWarps = 8, kAux = 32 * kAuxWarps, kSolve = 128;
+// PLANES goes by the order of preparation, modulo 4 (the ring turns round at every segment, so that neighbours share a
+// slot; AUX is at most two chunks ahead of SOLVE); SOLVED: SOLVE is through with a chunk's Kb planes, modulo 2.
+constexpr int kBarPlanes = 10, kBarSolved = 14;
 
 struct BwdArgsDev {
     const void *q, *k, *v, *d_o, *d_o_im;
@@ -54,29 +57,38 @@ struct BwdArgsDev {
 // One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
 // S_0, G_C as B operands [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U, Bc as A operands
 // [chain warp][plane][lane] uint4; then the chunk's rotated keys and queries, decays and phases, 8 floats per
-// (token, key).
+// (token, key).  Behind the ring: rowdot(S, G) [2][chain warp][key] and the final state.
 template <int DK, int NB>
 struct BwdScratch {
     static constexpr int NCW = NB / 16, KT = DK / 16, M = DK / 2;
     static constexpr int oS = 0, oU = oS + NCW * KT * 1024, oG = oU + NCW * 2048, oB = oG + NCW * KT * 1024;
     static constexpr int oV = oB + NCW * 2048, slot = oV + 16 * M * 32;
-    static_assert((size_t)slot * kSlots <= (size_t)kSeg * DK * NB * 4, "the scratch ring must fit the workspace");
+    static constexpr int oRg = slot * kSlots, oEnd = oRg + 2 * NCW * M * 8;
+    static_assert((size_t)oEnd + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "the scratch must fit the workspace");
 };
 
 template <int DK, int NB>
 struct BwdSmem {
+    using PM = PrepMap<DK, kAuxWarps>;
     static constexpr int NCW = NB / 16, M = DK / 2;
-    static constexpr int frag_bytes = 3 * NCW * 2048;             // Yb, Bc, U of the chunk as A operands
-    static constexpr int stage = kSlots * Tile<DK>::bytes;        // PREP's staging and the gradients' operands share a place
-    static constexpr int stage_bytes = frag_bytes > PrepSmem<DK>::stage_bytes ? frag_bytes : PrepSmem<DK>::stage_bytes;
-    static constexpr int small = stage + stage_bytes;
-    static constexpr int tri = small + PrepSmem<DK>::small_bytes; // the triangular factors of the corrections, 8 x 4 uint4 [32]
-    static constexpr int uy = tri + 8 * 4 * 512;                  // U Yb^T, U B^T: float2 [2][16][17]
-    static constexpr int scal = uy + 2 * 16 * 17 * 8;             // inverse scales [slot][NCW] (S, U, G, B), [NCW] Yb
-    static constexpr int rg = scal + kSlots * NCW * 16 + NCW * 4 + (16 - NCW * 4 % 16) % 16;   // rowdot(S, G): float2 [2][NCW][M]
-    static constexpr int db = rg + 2 * NCW * M * 8;               // dbeta: [8][16] floats
-    static constexpr int flag = db + 8 * 16 * 4;                  // fast flag per slot
-    static constexpr int bytes = flag + 16;
+    static constexpr int up(int x) { return (x + 127) / 128 * 128; }
+    static constexpr int gram_bytes = 2 * 16 * 17 * 8;
+    static constexpr int kb = kSlots * Tile<DK>::bytes;           // Kb planes, two chunks
+    static constexpr int gram = kb + 2 * Tile<DK>::BIG;           // the two Gram matrices, two chunks
+    // Yb, Bc, U of the chunk as A operands; slow_gram's scratch while a tile is prepared
+    static constexpr int frag = up(gram + 2 * gram_bytes);
+    static constexpr int frag_bytes = 3 * NCW * 2048 > PM::slow_bytes ? 3 * NCW * 2048 : PM::slow_bytes;
+    // U Yb^T, U B^T in two halves over the columns: float2 [2][2][16][17]; the scan's scratch while a tile is prepared
+    static constexpr int uy = up(frag + frag_bytes);
+    static constexpr int uy_bytes = 4 * 16 * 17 * 8;
+    static_assert(PM::scan_bytes <= uy_bytes, "the scan's scratch");
+    static constexpr int tri = uy + uy_bytes;                     // the corrections' triangular factors: 4 x 4 uint4 [32]
+    static constexpr int scal = tri + 4 * 4 * 512;                // inverse scales [slot][NCW] (S, U, G, B), [NCW] Yb, [4] tri
+    static constexpr int db = scal + kSlots * NCW * 16 + 48;      // dbeta: [8][16] floats
+    static constexpr int word = db + 8 * 16 * 4;                  // tensor-memory address
+    static constexpr int bytes = word + 16;
+    static_assert(bytes <= 232448, "shared memory");
+    static constexpr int columns = (NB + 63) / 64 * DK < 32 ? 32 : (NB + 63) / 64 * DK;   // S and G
 };
 
 __device__ __forceinline__ int ring_slot(int r, int c) { return (r & 1) ? kSlots - 1 - c : c; }
@@ -90,54 +102,17 @@ __device__ __forceinline__ void mma3x(float (&d)[4], const uint32_t (&ah)[4], co
     mma_f16(d, ah, bl0, bl1);
     mma_f16(d, ah, bh0, bh1);
 }
-template <bool kExact>
-__device__ __forceinline__ void product_small_conj(float (&re)[2][4], float (&im)[2][4], const TokFrag &a, const TokFrag &b,
-                                                   float f, bool has_im)
-{
-#pragma unroll
-    for (int n = 0; n < 2; ++n) {
-        float rr[4] = {0.f, 0.f, 0.f, 0.f}, ir[4] = {0.f, 0.f, 0.f, 0.f}, ri[4] = {0.f, 0.f, 0.f, 0.f};
-        mma3x<kExact>(rr, a.rh, a.rl, b.rh[2 * n], b.rh[2 * n + 1], b.rl[2 * n], b.rl[2 * n + 1]);
-        mma3x<kExact>(ri, a.rh, a.rl, b.ih[2 * n], b.ih[2 * n + 1], b.il[2 * n], b.il[2 * n + 1]);
-        if (has_im) {
-            mma3x<kExact>(rr, a.ih, a.il, b.ih[2 * n], b.ih[2 * n + 1], b.il[2 * n], b.il[2 * n + 1]);
-            mma3x<kExact>(ir, a.ih, a.il, b.rh[2 * n], b.rh[2 * n + 1], b.rl[2 * n], b.rl[2 * n + 1]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            re[n][i] = fmaf(f, rr[i], re[n][i]);
-            im[n][i] = fmaf(f, ir[i] - ri[i], im[n][i]);
-        }
-    }
-}
 
 // the [value x token] operand as the A operand (token, value) of products over the value columns
 __device__ __forceinline__ void publish_frag(uint4 *p, const TokFrag &f, int lane)
 {
-    p[0 * 32 + lane] = make_uint4(transpose8x8(f.rh[0]), transpose8x8(f.rh[2]), transpose8x8(f.rh[1]), transpose8x8(f.rh[3]));
-    p[1 * 32 + lane] = make_uint4(transpose8x8(f.rl[0]), transpose8x8(f.rl[2]), transpose8x8(f.rl[1]), transpose8x8(f.rl[3]));
-    p[2 * 32 + lane] = make_uint4(transpose8x8(f.ih[0]), transpose8x8(f.ih[2]), transpose8x8(f.ih[1]), transpose8x8(f.ih[3]));
-    p[3 * 32 + lane] = make_uint4(transpose8x8(f.il[0]), transpose8x8(f.il[2]), transpose8x8(f.il[1]), transpose8x8(f.il[3]));
-}
-
-template <int KT>
-__device__ __forceinline__ void store_state(float4 *p, const float (&sr)[KT][4], const float (&si)[KT][4], int lane)
-{
-#pragma unroll
-    for (int n = 0; n < KT; ++n) {
-        p[(2 * n) * 32 + lane] = make_float4(sr[n][0], sr[n][1], sr[n][2], sr[n][3]);
-        p[(2 * n + 1) * 32 + lane] = make_float4(si[n][0], si[n][1], si[n][2], si[n][3]);
-    }
-}
-template <int KT>
-__device__ __forceinline__ void load_state(const float4 *p, float (&sr)[KT][4], float (&si)[KT][4], int lane)
-{
-#pragma unroll
-    for (int n = 0; n < KT; ++n) {
-        const float4 x = p[(2 * n) * 32 + lane], y = p[(2 * n + 1) * 32 + lane];
-        sr[n][0] = x.x; sr[n][1] = x.y; sr[n][2] = x.z; sr[n][3] = x.w;
-        si[n][0] = y.x; si[n][1] = y.y; si[n][2] = y.z; si[n][3] = y.w;
-    }
+    auto put = [&](int plane, const uint32_t(&x)[4]) {
+        p[plane * 32 + lane] = make_uint4(transpose8x8(x[0]), transpose8x8(x[2]), transpose8x8(x[1]), transpose8x8(x[3]));
+    };
+    put(0, f.rh);
+    put(1, f.rl);
+    put(2, f.ih);
+    put(3, f.il);
 }
 
 __device__ __forceinline__ void st_val4(float *p, float4 x) { *reinterpret_cast<float4 *>(p) = x; }
@@ -158,48 +133,155 @@ __device__ __forceinline__ float join_half(uint32_t h, uint32_t l, int half)
 }
 
 // ---- AUX: the gradients of one chunk --------------------------------------------------------------
+// The corrections of one (token, key) where the decays are too strong to divide by: running products, token by token.
+// uy: U Yb^T and U B^T (two halves each); x1, x2, x3: the products with the boundary matrices.
+struct SlowOut {
+    float2 qb, zb, fb;
+};
+__device__ __noinline__ SlowOut slow_corrections(const float4 *vals, int M, const float2 *uy, const float *alpha, const float *beta,
+                                                 size_t row0, int H, int t0, int T_, int tl, int key, float2 x1, float2 x2, float2 x3)
+{
+    auto at = [&](int mat, int i, int t) {
+        const float2 x = uy[mat * 272 + i * 17 + t], y = uy[544 + mat * 272 + i * 17 + t];
+        return make_float2(x.x + y.x, x.y + y.y);
+    };
+    SlowOut o;
+    float w = 1.f;
+    o.qb = o.zb = o.fb = make_float2(0.f, 0.f);
+    for (int j = tl; j >= 0; --j) {
+        const size_t rj = row0 + (size_t)(t0 + j) * H;
+        const float4 kj = vals[(j * M + key) * 2];
+        const float bj = t0 + j < T_ ? w * beta[rj] : 0.f;
+        const float2 kk = make_float2(bj * kj.x, bj * kj.y);
+        const float2 p = cmul(kk, at(0, j, tl)), s = cmul(kk, at(1, j, tl));
+        o.qb = make_float2(o.qb.x + p.x, o.qb.y + p.y);
+        if (j < tl) o.zb = make_float2(o.zb.x + s.x, o.zb.y + s.y);
+        w *= t0 + j < T_ ? alpha[rj * M + key] : 1.f;
+    }
+    o.qb = make_float2(fmaf(w, x1.x, o.qb.x), fmaf(w, x1.y, o.qb.y));
+    o.zb = make_float2(fmaf(w, x2.x, o.zb.x), fmaf(w, x2.y, o.zb.y));
+    w = 1.f;
+    for (int l = tl; l < 16; ++l) {
+        const float4 kl = vals[(l * M + key) * 2];
+        const float2 p = cmulc(at(0, tl, l), make_float2(w * kl.z, w * kl.w));
+        o.fb = make_float2(o.fb.x + p.x, o.fb.y + p.y);
+        if (l > tl) {
+            const float2 s = cmulc(at(1, tl, l), make_float2(w * kl.x, w * kl.y));
+            o.fb = make_float2(o.fb.x - s.x, o.fb.y - s.y);
+        }
+        if (l < 15 && t0 + l + 1 < T_) w *= alpha[(row0 + (size_t)(t0 + l + 1) * H) * M + key];
+    }
+    o.fb = make_float2(fmaf(w, x3.x, o.fb.x), fmaf(w, x3.y, o.fb.y));
+    return o;
+}
+
+// dalpha of one (token tl, key) from its definition, by one warp: S_{t-1} and the cotangent of Lambda_t S_{t-1} rebuilt
+// from the boundary matrices, value column by value column.
+template <int DK, int NB>
+__device__ __noinline__ float small_alpha(const float4 *vals, const uint4 *frag, const uint4 *pS, const uint4 *pG, const float *sc,
+                                          const float *yscal, const float *alpha, const float *theta, const float *beta,
+                                          size_t row0, int H, int t0, int T_, int tl, int kt, int kl, int lane)
+{
+    constexpr int NCW = NB / 16, M = DK / 2, KT = M / 8;
+    const int key = 8 * kt + kl;
+    float sum = 0.f, cst = 1.f, snt = 0.f;
+    for (int val = lane; val < NB; val += 32) {
+        const int w = val >> 4, vl = val & 15, hf = vl & 1;
+        auto state = [&](const uint4 *base, float inv) {
+            const uint32_t *p = reinterpret_cast<const uint32_t *>(base + ((w * KT + kt) * 2) * 32 + 4 * kl + ((vl & 7) >> 1)) + (vl >> 3);
+            return make_float2(inv * join_half(p[0], p[2], hf), inv * join_half(p[128], p[130], hf));
+        };
+        auto token = [&](int mat, int tok, float inv) {
+            const uint32_t *p = reinterpret_cast<const uint32_t *>(frag + (mat * NCW + w) * 128 + 4 * (tok & 7) + ((vl & 7) >> 1)) + (tok >> 3) + 2 * (vl >> 3);
+            return make_float2(inv * join_half(p[0], p[128], hf), inv * join_half(p[256], p[384], hf));
+        };
+        float2 s = state(pS, sc[4 * w]), z = state(pG, sc[4 * w + 2]);
+        for (int j = 0; j < tl; ++j) {               // S_{t-1}
+            const size_t rj = row0 + (size_t)(t0 + j) * H;
+            const float4 x = vals[(j * M + key) * 2], y = vals[(j * M + key) * 2 + 1];
+            float sn, cs;
+            sincosf(theta[rj * M + key], &sn, &cs);
+            const float aj = alpha[rj * M + key], bj = beta[rj];
+            const float2 kj = cmul(make_float2(y.z, y.w), make_float2(bj * x.x, bj * x.y)), u = token(2, j, sc[4 * w + 1]);
+            s = cmul(make_float2(aj * cs, aj * sn), s);
+            const float2 p = cmul(kj, u);
+            s = make_float2(s.x + p.x, s.y + p.y);
+        }
+        for (int l = min(15, T_ - 1 - t0); l >= tl; --l) {     // the cotangent of Lambda_t S_{t-1}
+            const size_t rl = row0 + (size_t)(t0 + l) * H;
+            const float4 x = vals[(l * M + key) * 2], y = vals[(l * M + key) * 2 + 1];
+            const float2 ph = make_float2(y.z, y.w), ql = cmul(ph, make_float2(x.z, x.w)), kj = cmul(ph, make_float2(x.x, x.y));
+            const float2 yb = token(0, l, yscal[w]), bc = token(1, l, sc[4 * w + 3]);
+            const float2 p = cmulc(yb, ql), m = cmul(kj, bc);
+            z = make_float2(z.x + p.x - m.x, z.y + p.y - m.y);
+            float sn, cs;
+            sincosf(theta[rl * M + key], &sn, &cs);
+            if (l > tl) {
+                const float aj = alpha[rl * M + key];
+                z = cmulc(make_float2(aj * cs, aj * sn), z);
+            } else {
+                cst = cs;
+                snt = sn;
+            }
+        }
+        const float2 lb = cmulc(s, z);
+        sum += lb.x * cst + lb.y * snt;              // Re(conj(lambda bar) e^{i theta})
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+    return sum;
+}
+
 template <int DK, int DVT, int NB, typename T>
-__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, int slot, int rpar,
-                                             bool first, int t0, size_t row0, float2 (&carry)[2], int tid)
+__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, const float2 *rg, int slot,
+                                                bool first, int t0, size_t row0, float2 (&carry)[2], int tid)
 {
     using L = BwdSmem<DK, NB>;
     using SC = BwdScratch<DK, NB>;
+    using TL = Tile<DK>;
     constexpr int NCW = L::NCW, M = L::M, KT = M / 8, NSL = DVT / NB;
     constexpr bool kExact = sizeof(T) == 2;
     const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3, c0 = blockIdx.y * NB;
     const bool has_im = a.d_o_im != nullptr;
-    uint4 *frag = reinterpret_cast<uint4 *>(smem + L::stage);                     // [Yb, Bc, U][NCW][4][32]
+    uint4 *frag = reinterpret_cast<uint4 *>(smem + L::frag);                      // [Yb, Bc, U][NCW][4][32]
     uint4 *tri = reinterpret_cast<uint4 *>(smem + L::tri);
     float2 *uy = reinterpret_cast<float2 *>(smem + L::uy);
-    float *scal = reinterpret_cast<float *>(smem + L::scal), *yscal = scal + kSlots * NCW * 4;
+    float *scal = reinterpret_cast<float *>(smem + L::scal), *yscal = scal + kSlots * NCW * 4, *tscal = yscal + 8;
     const float *sc = scal + slot * NCW * 4;
     float *db = reinterpret_cast<float *>(smem + L::db);
     const uint4 *pS = reinterpret_cast<const uint4 *>(scr + SC::oS), *pG = reinterpret_cast<const uint4 *>(scr + SC::oG);
     const float4 *vals = reinterpret_cast<const float4 *>(scr + SC::oV);
 
     // operands over the value columns: Yb from the caller's arrays, Bc and U from the ring
-    for (int w = warp; w < NCW; w += kAuxWarps) {
+    if (warp < NCW) {
+        const int w = warp;
+        const uint4 *pB = reinterpret_cast<const uint4 *>(scr + SC::oB) + w * 128 + lane, *pU = reinterpret_cast<const uint4 *>(scr + SC::oU) + w * 128 + lane;
+        uint4 x[8];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            x[p] = pB[p * 32];
+            x[4 + p] = pU[p * 32];
+        }
         float2 y[2][4];
-        uint32_t m = 0;
+        float m = 0.f;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int t = t0 + g + 8 * (i & 1);
             y[0][i] = y[1][i] = make_float2(0.f, 0.f);
             if (t < a.T) {
                 const size_t at = (row0 + (size_t)t * a.H) * DVT + c0 + 16 * w + 2 * t4 + 8 * (i >> 1);
-                y[0][i] = ld_pair(static_cast<const T *>(a.d_o), at);
-                if (has_im) y[1][i] = ld_pair(static_cast<const T *>(a.d_o_im), at);
+                y[0][i] = make_float2(ld_val(static_cast<const T *>(a.d_o), at), ld_val(static_cast<const T *>(a.d_o), at + 1));
+                if (has_im) y[1][i] = make_float2(ld_val(static_cast<const T *>(a.d_o_im), at), ld_val(static_cast<const T *>(a.d_o_im), at + 1));
             }
-            m = max(m, max(max(abs_bits(y[0][i].x), abs_bits(y[0][i].y)), max(abs_bits(y[1][i].x), abs_bits(y[1][i].y))));
+            m = fmaxf(fmaxf(m, fmaxf(fabsf(y[0][i].x), fabsf(y[0][i].y))), fmaxf(fabsf(y[1][i].x), fabsf(y[1][i].y)));
         }
-        const uint4 *pB = reinterpret_cast<const uint4 *>(scr + SC::oB) + w * 128, *pU = reinterpret_cast<const uint4 *>(scr + SC::oU) + w * 128;
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
-            frag[((NCW + w) * 4 + p) * 32 + lane] = pB[p * 32 + lane];
-            frag[((2 * NCW + w) * 4 + p) * 32 + lane] = pU[p * 32 + lane];
+            frag[((NCW + w) * 4 + p) * 32 + lane] = x[p];
+            frag[((2 * NCW + w) * 4 + p) * 32 + lane] = x[4 + p];
         }
         float inv;
-        const float s = scale_for(__reduce_max_sync(0xffffffffu, m), inv);
+        const float s = scale_for(warp_max(m), inv);
         if (lane == 0) yscal[w] = inv;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
@@ -213,31 +295,44 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     bar_sync(kBarAux, kAux);
 
     // U Yb^T (index [i][t]: u_i . yb_t) and U B^T (b_t = beta_t p_t = conj of the rows of Bc): warp = (matrix, half of
-    // the columns, Re / Im); the A-operand registers of tokens 0-7 / 8-15 are the B operand of that half
+    // the tokens t, half of the value columns); the A-operand registers of tokens 0-7 / 8-15 are that half's B operand
     {
-        const int mat = warp & 1, nt = (warp >> 1) & 1, part = warp >> 2;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        const float sx = (mat && part) ? -1.f : 1.f, sz = (!mat && !part) ? -1.f : 1.f;
-#pragma unroll 2
-        for (int w = 0; w < NCW; ++w) {
+        const int mat = warp & 1, nt = (warp >> 1) & 1, wh = warp >> 2;
+        float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
+        const float sg = mat ? 1.f : -1.f;
+#pragma unroll 1
+        for (int w = wh; w < NCW; w += 2) {
             const uint4 *fu = frag + (2 * NCW + w) * 128 + lane, *fx = frag + (mat * NCW + w) * 128 + lane;
-            const uint4 urh = fu[0], url = fu[32], uih = fu[64], uil = fu[96];
-            const uint4 xh = fx[part * 64], xl = fx[part * 64 + 32], zh = fx[64 - part * 64], zl = fx[96 - part * 64];
-            const uint32_t ar[4] = {urh.x, urh.y, urh.z, urh.w}, arl[4] = {url.x, url.y, url.z, url.w};
-            const uint32_t ai[4] = {uih.x, uih.y, uih.z, uih.w}, ail[4] = {uil.x, uil.y, uil.z, uil.w};
-            float p[4] = {0.f, 0.f, 0.f, 0.f}, z[4] = {0.f, 0.f, 0.f, 0.f};
-            mma3(p, ar, arl, nt ? xh.y : xh.x, nt ? xh.w : xh.z, nt ? xl.y : xl.x, nt ? xl.w : xl.z);
-            mma3(z, ai, ail, nt ? zh.y : zh.x, nt ? zh.w : zh.z, nt ? zl.y : zl.x, nt ? zl.w : zl.z);
+            const uint4 u0 = fu[0], u1 = fu[32], u2 = fu[64], u3 = fu[96], x0 = fx[0], x1 = fx[32], x2 = fx[64], x3 = fx[96];
+            const uint32_t rh[4] = {u0.x, u0.y, u0.z, u0.w}, rl[4] = {u1.x, u1.y, u1.z, u1.w};
+            const uint32_t ih[4] = {u2.x, u2.y, u2.z, u2.w}, il[4] = {u3.x, u3.y, u3.z, u3.w};
+            const uint32_t xr[2] = {nt ? x0.y : x0.x, nt ? x0.w : x0.z}, xrl[2] = {nt ? x1.y : x1.x, nt ? x1.w : x1.z};
+            const uint32_t xi[2] = {nt ? x2.y : x2.x, nt ? x2.w : x2.z}, xil[2] = {nt ? x3.y : x3.x, nt ? x3.w : x3.z};
+            float rr[4], ii[4], ri[4], ir[4];
+            mma_f16_z(rr, rl, xr[0], xr[1]);
+            mma_f16_z(ii, il, xi[0], xi[1]);
+            mma_f16_z(ri, rl, xi[0], xi[1]);
+            mma_f16_z(ir, il, xr[0], xr[1]);
+            mma_f16(rr, rh, xrl[0], xrl[1]);
+            mma_f16(ii, ih, xil[0], xil[1]);
+            mma_f16(ri, rh, xil[0], xil[1]);
+            mma_f16(ir, ih, xrl[0], xrl[1]);
+            mma_f16(rr, rh, xr[0], xr[1]);
+            mma_f16(ii, ih, xi[0], xi[1]);
+            mma_f16(ri, rh, xi[0], xi[1]);
+            mma_f16(ir, ih, xr[0], xr[1]);
             const float f = sc[4 * w + 1] * (mat ? sc[4 * w + 3] : yscal[w]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) acc[i] = fmaf(f, fmaf(sx, p[i], sz * z[i]), acc[i]);
+            for (int i = 0; i < 4; ++i) {
+                re[i] = fmaf(f, fmaf(sg, ii[i], rr[i]), re[i]);
+                im[i] = fmaf(f, fmaf(-sg, ri[i], ir[i]), im[i]);
+            }
         }
-        float *dst = reinterpret_cast<float *>(uy + mat * 16 * 17) + part;
-        const int t = 8 * nt + 2 * t4;
-        dst[2 * (g * 17 + t)] = acc[0];
-        dst[2 * (g * 17 + t + 1)] = acc[1];
-        dst[2 * ((g + 8) * 17 + t)] = acc[2];
-        dst[2 * ((g + 8) * 17 + t + 1)] = acc[3];
+        float2 *dst = uy + (wh * 2 + mat) * 272 + g * 17 + 8 * nt + 2 * t4;
+        dst[0] = make_float2(re[0], im[0]);
+        dst[1] = make_float2(re[1], im[1]);
+        dst[8 * 17] = make_float2(re[2], im[2]);
+        dst[8 * 17 + 1] = make_float2(re[3], im[3]);
     }
 
     // X1 = S_0 yb_t, X2 = S_0 b_t, X3 = G_C conj(u_t) for the keys of tile `warp` (accumulator layout: token g (+ 8),
@@ -245,123 +340,172 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     float x1r[4] = {0.f, 0.f, 0.f, 0.f}, x1i[4] = {0.f, 0.f, 0.f, 0.f}, x2r[4] = {0.f, 0.f, 0.f, 0.f};
     float x2i[4] = {0.f, 0.f, 0.f, 0.f}, x3r[4] = {0.f, 0.f, 0.f, 0.f}, x3i[4] = {0.f, 0.f, 0.f, 0.f};
     if (warp < KT) {
-#pragma unroll 1
-        for (int w = 0; w < NCW; ++w) {
-            const uint4 s0 = pS[((w * KT + warp) * 2) * 32 + lane], s1 = pS[((w * KT + warp) * 2 + 1) * 32 + lane];
-            const uint4 g0 = pG[((w * KT + warp) * 2) * 32 + lane], g1 = pG[((w * KT + warp) * 2 + 1) * 32 + lane];
-            {
-                const uint4 *fy = frag + w * 128 + lane;
-                const uint4 h = fy[0], l = fy[32];
-                const uint32_t ah[4] = {h.x, h.y, h.z, h.w}, al[4] = {l.x, l.y, l.z, l.w};
-                float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mr[4] = {0.f, 0.f, 0.f, 0.f};
-                mma3x<kExact>(pr, ah, al, s0.x, s0.y, s0.z, s0.w);
-                mma3x<kExact>(pi, ah, al, s1.x, s1.y, s1.z, s1.w);
-                if (has_im) {
-                    const uint4 h2 = fy[64], l2 = fy[96];
-                    const uint32_t bh[4] = {h2.x, h2.y, h2.z, h2.w}, bl[4] = {l2.x, l2.y, l2.z, l2.w};
-                    mma3x<kExact>(mr, bh, bl, s1.x, s1.y, s1.z, s1.w);
-                    mma3x<kExact>(pi, bh, bl, s0.x, s0.y, s0.z, s0.w);
-                }
-                const float f = sc[4 * w] * yscal[w];
+        auto conj_product = [&](const uint4 *fx, const uint4 &b0, const uint4 &b1, float f, float (&xr)[4], float (&xi)[4]) {
+            const uint4 h = fx[0], l = fx[32], h2 = fx[64], l2 = fx[96];
+            const uint32_t rh[4] = {h.x, h.y, h.z, h.w}, rl[4] = {l.x, l.y, l.z, l.w};
+            const uint32_t ih[4] = {h2.x, h2.y, h2.z, h2.w}, il[4] = {l2.x, l2.y, l2.z, l2.w};
+            float pr[4], pi[4], qr[4], mi[4];
+            mma_f16_z(pr, rl, b0.x, b0.y);
+            mma_f16_z(pi, rl, b1.x, b1.y);
+            mma_f16_z(mi, il, b0.x, b0.y);
+            mma_f16_z(qr, il, b1.x, b1.y);
+            mma_f16(pr, rh, b0.z, b0.w);
+            mma_f16(pi, rh, b1.z, b1.w);
+            mma_f16(mi, ih, b0.z, b0.w);
+            mma_f16(qr, ih, b1.z, b1.w);
+            mma_f16(pr, rh, b0.x, b0.y);
+            mma_f16(pi, rh, b1.x, b1.y);
+            mma_f16(mi, ih, b0.x, b0.y);
+            mma_f16(qr, ih, b1.x, b1.y);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    x1r[i] = fmaf(f, pr[i] - mr[i], x1r[i]);
-                    x1i[i] = fmaf(f, pi[i], x1i[i]);
-                }
+            for (int i = 0; i < 4; ++i) {
+                xr[i] = fmaf(f, pr[i] + qr[i], xr[i]);
+                xi[i] = fmaf(f, pi[i] - mi[i], xi[i]);
             }
-            auto conj_product = [&](const uint4 *fx, const uint4 &b0, const uint4 &b1, float f, float (&xr)[4], float (&xi)[4]) {
-                const uint4 h = fx[0], l = fx[32], h2 = fx[64], l2 = fx[96];
-                const uint32_t rh[4] = {h.x, h.y, h.z, h.w}, rl[4] = {l.x, l.y, l.z, l.w};
-                const uint32_t ih[4] = {h2.x, h2.y, h2.z, h2.w}, il[4] = {l2.x, l2.y, l2.z, l2.w};
-                float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mi[4] = {0.f, 0.f, 0.f, 0.f};
-                mma3(pr, rh, rl, b0.x, b0.y, b0.z, b0.w);
-                mma3(pi, rh, rl, b1.x, b1.y, b1.z, b1.w);
-                mma3(mi, ih, il, b0.x, b0.y, b0.z, b0.w);
-                mma3(pr, ih, il, b1.x, b1.y, b1.z, b1.w);
+        };
+        // the ring's operands are requested two steps ahead: they come from L2
+        uint4 n[2][2];
+        const uint4 *p = pS + warp * 64 + lane;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    xr[i] = fmaf(f, pr[i], xr[i]);
-                    xi[i] = fmaf(f, pi[i] - mi[i], xi[i]);
+        for (int e = 0; e < 2; ++e) {
+            n[e][0] = p[e * KT * 64];
+            n[e][1] = p[e * KT * 64 + 32];
+        }
+#pragma unroll 1
+        for (int w2 = 0; w2 < NCW; w2 += 2) {
+            p += 2 * KT * 64;
+            if (w2 + 2 >= NCW) p = pG + warp * 64 + lane;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int w = w2 + e;
+                const uint4 s0 = n[e][0], s1 = n[e][1];
+                n[e][0] = p[e * KT * 64];
+                n[e][1] = p[e * KT * 64 + 32];
+                {
+                    const uint4 *fy = frag + w * 128 + lane;
+                    const uint4 h = fy[0], l = fy[32];
+                    const uint32_t ah[4] = {h.x, h.y, h.z, h.w}, al[4] = {l.x, l.y, l.z, l.w};
+                    float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mr[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma3x<kExact>(pr, ah, al, s0.x, s0.y, s0.z, s0.w);
+                    mma3x<kExact>(pi, ah, al, s1.x, s1.y, s1.z, s1.w);
+                    if (has_im) {
+                        const uint4 h2 = fy[64], l2 = fy[96];
+                        const uint32_t bh[4] = {h2.x, h2.y, h2.z, h2.w}, bl[4] = {l2.x, l2.y, l2.z, l2.w};
+                        mma3x<kExact>(mr, bh, bl, s1.x, s1.y, s1.z, s1.w);
+                        mma3x<kExact>(pi, bh, bl, s0.x, s0.y, s0.z, s0.w);
+                    }
+                    const float f = sc[4 * w] * yscal[w];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        x1r[i] = fmaf(f, pr[i] - mr[i], x1r[i]);
+                        x1i[i] = fmaf(f, pi[i], x1i[i]);
+                    }
                 }
-            };
-            conj_product(frag + (NCW + w) * 128 + lane, s0, s1, sc[4 * w] * sc[4 * w + 3], x2r, x2i);
-            conj_product(frag + (2 * NCW + w) * 128 + lane, g0, g1, sc[4 * w + 2] * sc[4 * w + 1], x3r, x3i);
+                conj_product(frag + (NCW + w) * 128 + lane, s0, s1, sc[4 * w] * sc[4 * w + 3], x2r, x2i);
+            }
+        }
+#pragma unroll 1
+        for (int w2 = 0; w2 < NCW; w2 += 2) {
+            p += 2 * KT * 64;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int w = w2 + e;
+                const uint4 g0 = n[e][0], g1 = n[e][1];
+                if (w2 + 2 < NCW) {
+                    n[e][0] = p[e * KT * 64];
+                    n[e][1] = p[e * KT * 64 + 32];
+                }
+                conj_product(frag + (2 * NCW + w) * 128 + lane, g0, g1, sc[4 * w + 2] * sc[4 * w + 1], x3r, x3i);
+            }
         }
     }
     bar_sync(kBarAux, kAux);
 
-    // the triangular factors of the corrections as TF32 A operands: warp = (sum, step of eight tokens); the k index of
-    // a step runs over tokens 4 t4 + 2 step (slot t4) and + 1 (slot t4 + 4), PREP's order of tokens
-    const float *beta_row = a.beta + row0;
-    {
-        const int sum = warp >> 1, i0 = 4 * t4 + 2 * (warp & 1);
-        uint32_t rh[4], rl[4], ih[4], il[4];
+    // the triangular factors of the corrections as A operands (t, i), a warp each:
+    //   0: u_i . yb_t (i <= t)   1: u_i . b_t (i < t)   2: conj(u_t . yb_i) (i >= t)   3: -conj(u_t . b_i) (i > t)
+    if (warp < 4) {
+        float2 x[4][2];
+        float m = 0.f;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int t = g + 8 * (e & 1), i = i0 + (e >> 1);
-            float2 x = make_float2(0.f, 0.f);
-            if (sum < 2) {
-                if (sum == 0 ? i <= t : i < t) {
-                    const float be = t0 + i < a.T ? beta_row[(size_t)(t0 + i) * a.H] : 0.f;
-                    x = uy[sum * 272 + i * 17 + t];
-                    x = make_float2(be * x.x, be * x.y);
-                }
-            } else if (sum == 2 ? i >= t : i > t) {
-                x = uy[(sum - 2) * 272 + t * 17 + i];
-                x = sum == 2 ? make_float2(x.x, -x.y) : make_float2(-x.x, x.y);
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int t = g + 8 * (e & 1), i = 2 * t4 + 8 * (e >> 1) + j;
+                const float2 *p = uy + (warp & 1) * 272 + (warp < 2 ? i * 17 + t : t * 17 + i);
+                const bool on = (warp & 1) ? (warp < 2 ? i < t : i > t) : (warp < 2 ? i <= t : i >= t);
+                const float2 u = p[0], v = p[544];
+                const float sr = warp == 3 ? -1.f : 1.f, si = warp == 2 ? -1.f : 1.f;
+                x[e][j] = on ? make_float2(sr * (u.x + v.x), si * (u.y + v.y)) : make_float2(0.f, 0.f);
+                m = fmaxf(m, fmaxf(fabsf(x[e][j].x), fabsf(x[e][j].y)));
             }
-            split_tf32(x.x, rh[e], rl[e]);
-            split_tf32(x.y, ih[e], il[e]);
-        }
+        float inv;
+        const float s = scale_for(warp_max(m), inv);
+        if (lane == 0) tscal[warp] = inv;
+        uint32_t h[4], l[4];
         uint4 *p = tri + warp * 128 + lane;
-        p[0] = make_uint4(rh[0], rh[1], rh[2], rh[3]);
-        p[32] = make_uint4(rl[0], rl[1], rl[2], rl[3]);
-        p[64] = make_uint4(ih[0], ih[1], ih[2], ih[3]);
-        p[96] = make_uint4(il[0], il[1], il[2], il[3]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) split_f16(x[e][0].x * s, x[e][1].x * s, h[e], l[e]);
+        p[0] = make_uint4(h[0], h[1], h[2], h[3]);
+        p[32] = make_uint4(l[0], l[1], l[2], l[3]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) split_f16(x[e][0].y * s, x[e][1].y * s, h[e], l[e]);
+        p[64] = make_uint4(h[0], h[1], h[2], h[3]);
+        p[96] = make_uint4(l[0], l[1], l[2], l[3]);
     }
     bar_sync(kBarAux, kAux);
 
     if (warp < KT) {
-        const bool fast = reinterpret_cast<const int *>(smem + L::flag)[slot] != 0;
-        float z1r[4] = {0.f, 0.f, 0.f, 0.f}, z1i[4] = {0.f, 0.f, 0.f, 0.f}, z2r[4] = {0.f, 0.f, 0.f, 0.f};
-        float z2i[4] = {0.f, 0.f, 0.f, 0.f}, z3r[4] = {0.f, 0.f, 0.f, 0.f}, z3i[4] = {0.f, 0.f, 0.f, 0.f};
+        const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
+        const bool fast = reinterpret_cast<const int *>(inv)[6] != 0;
+        float z1r[4], z1i[4], z2r[4], z2i[4], z3r[4], z3i[4];
         if (fast) {
-            auto tri_product = [&](int sum, int step, const float2 &b0, const float2 &b1, float (&zr)[4], float (&zi)[4]) {
-                const uint4 *p = tri + (2 * sum + step) * 128 + lane;
+            // B operand: tokens as k, the warp's eight keys; heads in registers 0, 1 and tails in 2, 3
+            const uint32_t tile = (uint32_t)__cvta_generic_to_shared(smem) + slot * TL::bytes + (uint32_t)((lane & 15) * TL::LDB + warp * 16 + (lane >> 4) * TL::PL);
+            auto tri_product = [&](int sum, const uint32_t(&br)[4], const uint32_t(&bi)[4], float (&zr)[4], float (&zi)[4]) {
+                const uint4 *p = tri + sum * 128 + lane;
                 const uint4 h = p[0], l = p[32], h2 = p[64], l2 = p[96];
                 const uint32_t rh[4] = {h.x, h.y, h.z, h.w}, rl[4] = {l.x, l.y, l.z, l.w};
                 const uint32_t ih[4] = {h2.x, h2.y, h2.z, h2.w}, il[4] = {l2.x, l2.y, l2.z, l2.w};
-                uint32_t brh[2], brl[2], bih[2], bil[2], nih[2], nil[2];
-                split_tf32(b0.x, brh[0], brl[0]);
-                split_tf32(b1.x, brh[1], brl[1]);
-                split_tf32(b0.y, bih[0], bil[0]);
-                split_tf32(b1.y, bih[1], bil[1]);
+                float nr[4], ni[4];
+                mma_f16_z(zr, rl, br[0], br[1]);
+                mma_f16_z(zi, rl, bi[0], bi[1]);
+                mma_f16_z(nr, il, bi[0], bi[1]);
+                mma_f16_z(ni, il, br[0], br[1]);
+                mma_f16(zr, rh, br[2], br[3]);
+                mma_f16(zi, rh, bi[2], bi[3]);
+                mma_f16(nr, ih, bi[2], bi[3]);
+                mma_f16(ni, ih, br[2], br[3]);
+                mma_f16(zr, rh, br[0], br[1]);
+                mma_f16(zi, rh, bi[0], bi[1]);
+                mma_f16(nr, ih, bi[0], bi[1]);
+                mma_f16(ni, ih, br[0], br[1]);
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    nih[i] = bih[i] ^ 0x80000000u;
-                    nil[i] = bil[i] ^ 0x80000000u;
+                for (int i = 0; i < 4; ++i) {
+                    zr[i] -= nr[i];
+                    zi[i] += ni[i];
                 }
-                mma3_tf32(zr, rh, rl, brh, brl);
-                mma3_tf32(zi, rh, rl, bih, bil);
-                mma3_tf32(zr, ih, il, nih, nil);
-                mma3_tf32(zi, ih, il, brh, brl);
             };
+            uint32_t br[4], bi[4];
+            ldsm_t(br, tile + TL::oY);
+            ldsm_t(bi, tile + TL::oY + 2 * TL::PL);
+            tri_product(0, br, bi, z1r, z1i);
+            tri_product(1, br, bi, z2r, z2i);
+            ldsm_t(br, tile + TL::oQ);
+            ldsm_t(bi, tile + TL::oQ + 2 * TL::PL);
+            tri_product(2, br, bi, z3r, z3i);
+            float wr[4], wi[4];
+            ldsm_t(br, tile + TL::oW);
+            ldsm_t(bi, tile + TL::oW + 2 * TL::PL);
+            tri_product(3, br, bi, wr, wi);
+            const float f0 = tscal[0] * inv[1], f1 = tscal[1] * inv[1], f2 = tscal[2] * inv[2], f3 = tscal[3] * inv[0];
 #pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                float2 kh[2], qw[2], wv[2];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const float4 *p = vals + ((4 * t4 + 2 * s + e) * M + 8 * warp + g) * 2;
-                    const float4 x = p[0], y = p[1];
-                    const float ia = __frcp_rn(y.x);
-                    kh[e] = make_float2(x.x * ia, x.y * ia);
-                    wv[e] = make_float2(x.x * y.x, x.y * y.x);
-                    qw[e] = make_float2(x.z * y.x, x.w * y.x);
-                }
-                tri_product(0, s, kh[0], kh[1], z1r, z1i);
-                tri_product(1, s, kh[0], kh[1], z2r, z2i);
-                tri_product(2, s, qw[0], qw[1], z3r, z3i);
-                tri_product(3, s, wv[0], wv[1], z3r, z3i);
+            for (int i = 0; i < 4; ++i) {
+                z1r[i] *= f0;
+                z1i[i] *= f0;
+                z2r[i] *= f1;
+                z2i[i] *= f1;
+                z3r[i] = fmaf(f2, z3r[i], f3 * wr[i]);
+                z3i[i] = fmaf(f2, z3i[i], f3 * wi[i]);
             }
         }
         float2 dqv[4], dkv[4], dd[4];
@@ -371,45 +515,24 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             const int r = i >> 1, e = i & 1, tl = g + 8 * r, t = t0 + tl, key = 8 * warp + 2 * t4 + e;
             const size_t row = row0 + (size_t)t * a.H;
             const float4 x = vals[(tl * M + key) * 2], y = vals[(tl * M + key) * 2 + 1];
-            const float4 last = vals[(15 * M + key) * 2 + 1];                     // e^{i phi_C}
-            const float2 kp = make_float2(x.x, x.y), qp = make_float2(x.z, x.w), ph = make_float2(y.z, y.w);
+            const float4 last = vals[(15 * M + key) * 2 + 1];                     // a_C, -, e^{i phi_C}
+            const float2 kp = make_float2(x.x, x.y), qp = make_float2(x.z, x.w), ph = make_float2(y.z, y.w), pc = make_float2(last.z, last.w);
             const float be = t < a.T ? a.beta[row] : 0.f;
             al[i] = t < a.T ? a.alpha[row * M + key] : 1.f;
-            const float2 x3 = cmulc(make_float2(last.z, last.w), make_float2(x3r[i], x3i[i]));
+            const float2 x3 = cmulc(pc, make_float2(x3r[i], x3i[i]));
             float2 qb, zb, fb;
             if (fast) {
-                const float ia = __frcp_rn(y.x);
-                qb = make_float2(y.x * (x1r[i] + z1r[i]), y.x * (x1i[i] + z1i[i]));
-                zb = make_float2(y.x * (x2r[i] + z2r[i]), y.x * (x2i[i] + z2i[i]));
-                fb = make_float2(fmaf(y.y, x3.x, ia * z3r[i]), fmaf(y.y, x3.y, ia * z3i[i]));
+                const float up = __fdividef(y.x, last.x), down = __frcp_rn(y.x);   // a_t / a_C, 1 / a_t: at most 2^16
+                const float2 c1 = cmulc(pc, make_float2(z1r[i], z1i[i])), c2 = cmulc(pc, make_float2(z2r[i], z2i[i]));
+                qb = make_float2(fmaf(y.x, x1r[i], up * c1.x), fmaf(y.x, x1i[i], up * c1.y));
+                zb = make_float2(fmaf(y.x, x2r[i], up * c2.x), fmaf(y.x, x2i[i], up * c2.y));
+                fb = make_float2(fmaf(y.y, x3.x, down * z3r[i]), fmaf(y.y, x3.y, down * z3i[i]));
             } else {
-                // decays too strong to divide by: running products, token by token
-                float w = 1.f;
-                qb = zb = fb = make_float2(0.f, 0.f);
-                for (int j = tl; j >= 0; --j) {
-                    const size_t rj = row0 + (size_t)(t0 + j) * a.H;
-                    const float4 kj = vals[(j * M + key) * 2];
-                    const float bj = t0 + j < a.T ? w * a.beta[rj] : 0.f;
-                    const float2 kk = make_float2(bj * kj.x, bj * kj.y);
-                    const float2 p = cmul(kk, uy[j * 17 + tl]), s = cmul(kk, uy[272 + j * 17 + tl]);
-                    qb = make_float2(qb.x + p.x, qb.y + p.y);
-                    if (j < tl) zb = make_float2(zb.x + s.x, zb.y + s.y);
-                    w *= t0 + j < a.T ? a.alpha[rj * M + key] : 1.f;
-                }
-                qb = make_float2(fmaf(w, x1r[i], qb.x), fmaf(w, x1i[i], qb.y));
-                zb = make_float2(fmaf(w, x2r[i], zb.x), fmaf(w, x2i[i], zb.y));
-                w = 1.f;
-                for (int l = tl; l < 16; ++l) {
-                    const float4 kl = vals[(l * M + key) * 2];
-                    const float2 p = cmulc(uy[tl * 17 + l], make_float2(w * kl.z, w * kl.w));
-                    fb = make_float2(fb.x + p.x, fb.y + p.y);
-                    if (l > tl) {
-                        const float2 s = cmulc(uy[272 + tl * 17 + l], make_float2(w * kl.x, w * kl.y));
-                        fb = make_float2(fb.x - s.x, fb.y - s.y);
-                    }
-                    if (l < 15 && t0 + l + 1 < a.T) w *= a.alpha[(row0 + (size_t)(t0 + l + 1) * a.H) * M + key];
-                }
-                fb = make_float2(fmaf(w, x3.x, fb.x), fmaf(w, x3.y, fb.y));
+                const SlowOut o = slow_corrections(vals, M, uy, a.alpha, a.beta, row0, a.H, t0, a.T, tl, key, make_float2(x1r[i], x1i[i]),
+                                                   make_float2(x2r[i], x2i[i]), x3);
+                qb = o.qb;
+                zb = o.zb;
+                fb = o.fb;
             }
             const float2 dkp = make_float2(be * fb.x - zb.x, be * fb.y - zb.y);
             dqv[i] = cmul(ph, qb);
@@ -420,10 +543,10 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         }
         // D: sums over the tokens behind, down to each token (tokens 8-15 in i = 2, 3, tokens 0-7 in i = 0, 1)
         if (first) {
-            const float2 *rg = reinterpret_cast<const float2 *>(smem + L::rg) + rpar * NCW * M;
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 carry[e] = make_float2(0.f, 0.f);
+#pragma unroll 1
                 for (int w = 0; w < NCW; ++w) {
                     const float2 x = rg[w * M + 8 * warp + 2 * t4 + e];
                     carry[e] = make_float2(carry[e].x + x.x, carry[e].y + x.y);
@@ -431,9 +554,9 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int d = 4; d < 32; d <<= 1)
 #pragma unroll
-            for (int d = 4; d < 32; d <<= 1) {
+            for (int i = 0; i < 4; ++i) {
                 const float ox = __shfl_down_sync(0xffffffffu, dd[i].x, d), oy = __shfl_down_sync(0xffffffffu, dd[i].y, d);
                 if (lane + d < 32) dd[i] = make_float2(dd[i].x + ox, dd[i].y + oy);
             }
@@ -447,66 +570,21 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
 #pragma unroll
         for (int i = 0; i < 4; ++i) dal[i] = __fdiv_rn(dd[i].x, al[i]);
         // small alpha: from the definition, one (token, key) at a time
+        if (__any_sync(0xffffffffu, fminf(fminf(al[0], al[1]), fminf(al[2], al[3])) < 0.0625f)) {
 #pragma unroll 1
-        for (int i = 0; i < 4; ++i) {
-            unsigned todo = __ballot_sync(0xffffffffu, (i == 0 ? al[0] : i == 1 ? al[1] : i == 2 ? al[2] : al[3]) < 0.0625f);
-            while (todo) {
-                const int src = __ffs(todo) - 1;
-                todo &= todo - 1;
-                const int tl = (src >> 2) + 8 * (i >> 1), kl = 2 * (src & 3) + (i & 1), key = 8 * warp + kl;
-                float sum = 0.f;
-                float cst = 1.f, snt = 0.f;
-                for (int val = lane; val < NB; val += 32) {
-                    const int w = val >> 4, vl = val & 15, hf = vl & 1;
-                    auto state = [&](const uint4 *base, float inv) {
-                        const uint32_t *p = reinterpret_cast<const uint32_t *>(base + ((w * KT + warp) * 2) * 32 + 4 * kl + ((vl & 7) >> 1)) + (vl >> 3);
-                        return make_float2(inv * join_half(p[0], p[2], hf), inv * join_half(p[128], p[130], hf));
-                    };
-                    auto token = [&](int mat, int tok, float inv) {
-                        const uint32_t *p = reinterpret_cast<const uint32_t *>(frag + (mat * NCW + w) * 128 + 4 * (tok & 7) + ((vl & 7) >> 1)) + (tok >> 3) + 2 * (vl >> 3);
-                        return make_float2(inv * join_half(p[0], p[128], hf), inv * join_half(p[256], p[384], hf));
-                    };
-                    float2 s = state(pS, sc[4 * w]), z = state(pG, sc[4 * w + 2]);
-                    for (int j = 0; j < 16; ++j) {           // S_{t-1}
-                        if (j >= tl) break;
-                        const size_t rj = row0 + (size_t)(t0 + j) * a.H;
-                        const float4 x = vals[(j * M + key) * 2], y = vals[(j * M + key) * 2 + 1];
-                        float sn, cs;
-                        sincosf(a.theta[rj * M + key], &sn, &cs);
-                        const float aj = a.alpha[rj * M + key], bj = a.beta[rj];
-                        const float2 kj = cmul(make_float2(y.z, y.w), make_float2(bj * x.x, bj * x.y)), u = token(2, j, sc[4 * w + 1]);
-                        s = cmul(make_float2(aj * cs, aj * sn), s);
-                        const float2 p = cmul(kj, u);
-                        s = make_float2(s.x + p.x, s.y + p.y);
+            for (int i = 0; i < 4; ++i) {
+                unsigned todo = __ballot_sync(0xffffffffu, (i == 0 ? al[0] : i == 1 ? al[1] : i == 2 ? al[2] : al[3]) < 0.0625f);
+                while (todo) {
+                    const int src = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    const float sum = small_alpha<DK, NB>(vals, frag, pS, pG, sc, yscal, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T,
+                                                          (src >> 2) + 8 * (i >> 1), warp, 2 * (src & 3) + (i & 1), lane);
+                    if (lane == src) {
+                        if (i == 0) dal[0] = sum;
+                        else if (i == 1) dal[1] = sum;
+                        else if (i == 2) dal[2] = sum;
+                        else dal[3] = sum;
                     }
-                    for (int l = 15; l >= tl; --l) {         // the cotangent of Lambda_t S_{t-1}
-                        if (t0 + l >= a.T) continue;
-                        const size_t rl = row0 + (size_t)(t0 + l) * a.H;
-                        const float4 x = vals[(l * M + key) * 2], y = vals[(l * M + key) * 2 + 1];
-                        const float2 ph = make_float2(y.z, y.w), ql = cmul(ph, make_float2(x.z, x.w)), kj = cmul(ph, make_float2(x.x, x.y));
-                        const float2 yb = token(0, l, yscal[w]), bc = token(1, l, sc[4 * w + 3]);
-                        const float2 p = cmulc(yb, ql), m = cmul(kj, bc);
-                        z = make_float2(z.x + p.x - m.x, z.y + p.y - m.y);
-                        float sn, cs;
-                        sincosf(a.theta[rl * M + key], &sn, &cs);
-                        if (l > tl) {
-                            const float aj = a.alpha[rl * M + key];
-                            z = cmulc(make_float2(aj * cs, aj * sn), z);
-                        } else {
-                            cst = cs;
-                            snt = sn;
-                        }
-                    }
-                    const float2 lb = cmulc(s, z);
-                    sum += lb.x * cst + lb.y * snt;          // Re(conj(lambda bar) e^{i theta})
-                }
-#pragma unroll
-                for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-                if (lane == src) {
-                    if (i == 0) dal[0] = sum;
-                    else if (i == 1) dal[1] = sum;
-                    else if (i == 2) dal[2] = sum;
-                    else dal[3] = sum;
                 }
             }
         }
@@ -549,289 +627,362 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     }
 }
 
+// ---- CHAIN helpers -----------------------------------------------------------------------------------
+// the state's 16-column pieces to and from the checkpoint [piece][4][lane] float4
+template <int DK>
+__device__ __forceinline__ void keep_state(float4 *p, uint32_t st)
+{
+#pragma unroll 1
+    for (int n = 0; n < Tile<DK>::KS; ++n, p += 128) {
+        float x[16];
+        tm_load(x, st + 16 * n);
+        tm_wait_load(x);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[32 * j] = make_float4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
+    }
+}
+__device__ __forceinline__ void read_piece(const float4 *p, float (&x)[16])
+{
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float4 v = p[32 * j];
+        x[4 * j] = v.x;
+        x[4 * j + 1] = v.y;
+        x[4 * j + 2] = v.z;
+        x[4 * j + 3] = v.w;
+    }
+}
+
 template <int DK, int DVT, int NB, typename T>
-__global__ void __launch_bounds__(kAux + 2 * NB, 1) sfda_backward_kernel(const BwdArgsDev a)
+__global__ void __launch_bounds__(kAux + kSolve + 2 * NB, 1) sfda_backward_kernel(const BwdArgsDev a)
 {
     using TL = Tile<DK>;
     using L = BwdSmem<DK, NB>;
     using SC = BwdScratch<DK, NB>;
-    constexpr int kAll = kAux + 2 * NB, NCW = NB / 16, M = DK / 2, KT = TL::KT;
+    constexpr int kChain = 2 * NB, NCW = NB / 16, M = DK / 2, KT = TL::KT;
     constexpr bool kExact = sizeof(T) == 2;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
     const size_t row0 = (size_t)b * a.T * a.H + h;                       // row of token t: row0 + t H
     const int nch = (a.T + kC - 1) / kC, NS = a.NS;
     unsigned char *ring = reinterpret_cast<unsigned char *>(a.scratch + ((size_t)bh * DVT + c0) * kSeg * DK);
+    float2 *rgs = reinterpret_cast<float2 *>(ring + SC::oRg);
     const int last_nch = nch - (NS - 1) * kSegChunks;                    // chunks of the last segment
+    // position n of the second sweep (segments last to first): segment from the end, place in it, its chunks
+    auto segment_of = [&](int n, int &r, int &at, int &nc) {
+        r = n < last_nch ? 0 : 1 + (n - last_nch) / kSegChunks;
+        at = r == 0 ? n : (n - last_nch) % kSegChunks;
+        nc = r == 0 ? last_nch : kSegChunks;
+    };
+    if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::word), L::columns);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::word);
 
     if (tid < kAux) {
-        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
-        const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3, key = 8 * warp + g;
+        // register shares with all 128 value columns: 256 x 112 + 128 x 56 + 256 x 100 rounded to 8: 112, 56, 96 of 640 x 96
+        if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
         const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
-        float2 *stage = reinterpret_cast<float2 *>(smem + L::stage);
-        int par = 0;
-        for (int c = 0; c < nch; ++c) {                                  // first sweep: keys only
-            const int slot = c % kSlots;
-            if (c >= kSlots) bar_sync(kBarDone + slot, kAll);
-            PrepIn in;
-            PrepVals pv;
-            prep_load<DK, T>(in, nullptr, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, key, t4);
-            prep_chunk<DK, false>(in, pv, smem + slot * TL::bytes, stage, smem + L::small, par, tid);
-            bar_arrive(kBarFull + slot, kAll);
-            par ^= 1;
-        }
-        for (int c = max(nch - kSlots, 0); c < nch; ++c) bar_sync(kBarDone + c % kSlots, kAll);
-        // Second sweep.  Chunks are prepared in the order the chain goes forward through the segments (last segment
-        // first) and their gradients follow in the order it comes back; the ring's slots are assigned so that the
-        // p-th chunk prepared takes the slot of gradient p - 4.
+        // Chunks are prepared in the order the chain goes forward through them (second sweep: last segment first) and
+        // their gradients follow in the order it comes back; the p-th chunk prepared takes the slot of gradient p - 4.
         float2 carry[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        for (int p = 0; p < nch + kSlots; ++p) {
-            if (p >= kSlots) {
-                const int n = p - kSlots, r = n < last_nch ? 0 : 1 + (n - last_nch) / kSegChunks;
-                const int nc = r == 0 ? last_nch : kSegChunks, at = r == 0 ? n : (n - last_nch) % kSegChunks, c = nc - 1 - at;
-                const int slot = ring_slot(r, c);
-                bar_sync(kBarDone + slot, kAll);
-                chunk_gradients<DK, DVT, NB, T>(a, smem, ring + (size_t)slot * SC::slot, slot, r & 1, at == 0,
-                                                (NS - 1 - r) * kSeg + c * kC, row0, carry, tid);
-                if (p < nch) bar_arrive(kBarFree + slot, kAll);
-            }
-            if (p < nch) {
-                const int r = p < last_nch ? 0 : 1 + (p - last_nch) / kSegChunks, c = r == 0 ? p : (p - last_nch) % kSegChunks;
-                const int slot = ring_slot(r, c);
-                PrepIn in;
-                PrepVals pv;
-                prep_load<DK, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, (NS - 1 - r) * kSeg + c * kC, a.T, key, t4);
-                const bool fast = prep_chunk<DK, true>(in, pv, smem + slot * TL::bytes, stage, smem + L::small, par, tid);
-                bar_arrive(kBarFull + slot, kAll);
-                par ^= 1;
-                if (tid == 0) reinterpret_cast<int *>(smem + L::flag)[slot] = fast;
-                if (key < M) {
-                    float4 *vals = reinterpret_cast<float4 *>(ring + (size_t)slot * SC::slot + SC::oV) + (4 * t4 * M + key) * 2;
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        vals[x * M * 2] = make_float4(pv.kr[x], pv.ki[x], pv.qr[x], pv.qi[x]);
-                        vals[x * M * 2 + 1] = make_float4(pv.a[x], pv.sfx[x], pv.cs[x], pv.sn[x]);
-                    }
+        int made = 0;
+#pragma unroll 1
+        for (int sweep = 0; sweep < 2; ++sweep) {
+#pragma unroll 1
+            for (int p = 0; p < nch + kSlots; ++p) {
+                int r, at, nc;
+                const int n = p - kSlots;
+                if (n >= 0 && n < nch) {
+                    segment_of(n, r, at, nc);
+                    const int c = nc - 1 - at, slot = sweep ? ring_slot(r, c) : n % kSlots;
+                    bar_sync(kBarDone + slot, kAux + kChain);
+                    if (sweep)
+                        chunk_gradients<DK, DVT, NB, T>(a, smem, ring + (size_t)slot * SC::slot, rgs + (r & 1) * NCW * M, slot, at == 0,
+                                                        (NS - 1 - r) * kSeg + c * kC, row0, carry, tid);
+                }
+                if (p < nch) {
+                    segment_of(p, r, at, nc);
+                    const int slot = sweep ? ring_slot(r, at) : p % kSlots, t0 = sweep ? (NS - 1 - r) * kSeg + at * kC : p * kC;
+                    const bool needq = sweep;
+                    PrepRaw<L::PM::TPT, T> in;
+                    prep_fetch<DK, kAuxWarps, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, needq, tid);
+                    if (made >= 2) bar_sync(kBarSolved + (made & 1), kAux + 64);
+                    float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + (made & 1) * L::gram_bytes);
+                    float4 *vals = sweep ? reinterpret_cast<float4 *>(ring + (size_t)slot * SC::slot + SC::oV) : nullptr;
+                    if (!prep_planes<DK, kAuxWarps, T>(in, vals, smem + slot * TL::bytes, smem + L::kb + (made & 1) * TL::BIG, smem + L::uy, needq, tid))
+                        slow_gram<DK, kAuxWarps, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, smem + L::frag, smem + L::uy, gk,
+                                                    gk + 16 * 17, needq, tid);
+                    bar_arrive(kBarPlanes + (made & 3), kAux + 64);
+                    ++made;
                 }
             }
         }
-        return;
-    }
-
-    if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
-    const int lane = tid & 31, w = (tid - kAux) >> 5, g = lane >> 2, t4 = lane & 3;
-    const int col = c0 + 16 * w + g;                                     // and col + 8
-    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
-    float *scal = reinterpret_cast<float *>(smem + L::scal);
-    auto checkpoint = [&](int s) {
-        return reinterpret_cast<float4 *>(a.check + (((size_t)bh * NS + s) * DVT + c0 + 16 * w) * DK);
-    };
-    auto state_at = [&](int n, int i) {                                  // Re of (key, column) of accumulator element (n, i)
-        return ((size_t)bh * DK + 2 * (8 * n + 2 * t4 + (i & 1))) * DVT + col + 8 * (i >> 1);
-    };
-    auto load_tokens = [&](const void *p, int t0, float sign, float (&x)[2][4]) {
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int t = t0 + 8 * n + 2 * t4 + (i & 1);
-                x[n][i] = p && t < a.T ? sign * ld_val(static_cast<const T *>(p), (row0 + (size_t)t * a.H) * DVT + col + 8 * (i >> 1)) : 0.f;
+    } else if (tid < kAux + kSolve) {
+        // warps 0, 1: the system's inverse of every other chunk; warps 2, 3: the outputs' Gram matrix of them
+        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        const int lane = tid & 31, w = (tid - kAux) >> 5, out = w >> 1;
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+#pragma unroll 1
+        for (int j = w & 1; j < 2 * nch; j += 2) {
+            const bool second = j >= nch;
+            int r, at, nc;
+            segment_of(j - nch, r, at, nc);
+            const int slot = second ? ring_slot(r, at) : j % kSlots;
+            unsigned char *tile = smem + slot * TL::bytes;
+            float *inv = reinterpret_cast<float *>(tile + TL::oS);
+            float2 *gm = reinterpret_cast<float2 *>(smem + L::gram + (j & 1) * L::gram_bytes) + out * 16 * 17;
+            bar_sync(kBarPlanes + (j & 3), kAux + 64);
+            if (second || !out) {
+                if (reinterpret_cast<const int *>(inv)[6])
+                    gram_tiles<DK, 2>(base + slot * TL::bytes + (out ? TL::oQ : TL::oW), base + L::kb + (j & 1) * TL::BIG, inv[out ? 2 : 0] * inv[5], gm, 0, lane);
+                __syncwarp();
+                if (!out) invert_unit_lower16(gm, lane);
+                store_lower(tile + (out ? TL::oA : TL::oM), gm, inv + 3 + out, lane);
             }
-    };
-    float sr[KT][4], si[KT][4];
-#pragma unroll
-    for (int n = 0; n < KT; ++n)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            sr[n][i] = a.S0 ? a.S0[state_at(n, i)] : 0.f;
-            si[n][i] = a.S0 ? a.S0[state_at(n, i) + DVT] : 0.f;
+            bar_arrive(kBarFull + slot, 64 + kChain);
+            if (j + 2 < 2 * nch) bar_arrive(kBarSolved + (j & 1), kAux + 64);
         }
-
-    // forward through one chunk: U = M (V - W^* S), S <- gamma_C S + Y U
-    auto forward_chunk = [&](int slot, int t0, auto pub, bool update) {
-        constexpr bool kPub = decltype(pub)::value;
-        unsigned char *scr = ring + (size_t)slot * SC::slot;
-        float rr[2][4], ri[2][4];
-        load_tokens(a.v, t0, 1.f, rr);
-        bar_sync(kBarFull + slot, kAll);
-        const uint32_t tile = base + slot * TL::bytes;
-        const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
-        float isv;
-        const float ss = scale_for(__reduce_max_sync(0xffffffffu, max(max_bits4(sr), max_bits4(si))), isv);
-        float acc[1][3][2][4];
-        const uint32_t tiles[1] = {tile + TL::oW};
-        product_over_keys<DK, 1, kPub>(acc, sr, si, ss, tiles, lane, reinterpret_cast<uint4 *>(scr + SC::oS) + w * KT * 64);
-        const float fw = isv * inv[0];
+    } else {
+        const int lane = tid & 31, w = (tid - kAux - kSolve) >> 5, g = lane >> 2, t4 = lane & 3;
+        const int col = c0 + 16 * w + g;                                 // and col + 8
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+        const uint32_t ss = tmem + ((uint32_t)(w & 3) << 21) + (w >> 2) * 16 * KT, sg = ss + 8 * KT;   // S and G
+        float *scal = reinterpret_cast<float *>(smem + L::scal);
+        const size_t step = (size_t)a.H * DVT, state_at = ((size_t)bh * DK + 4 * t4) * DVT + col;
+        auto checkpoint = [&](int s) {                                   // s = NS: the final state
+            float *p = s < NS ? a.check + (((size_t)bh * NS + s) * DVT + c0 + 16 * w) * DK : reinterpret_cast<float *>(ring + SC::oEnd) + 16 * w * DK;
+            return reinterpret_cast<float4 *>(p) + lane;
+        };
+        float big_s = state_from_memory<DK>(ss, a.S0 ? a.S0 + state_at : nullptr, DVT), big_g = 0.f;
+#pragma unroll 1
+        for (int r = -1; r < NS; ++r) {                                  // -1: the first sweep over the whole sequence
+            const int s = NS - 1 - r, nc = r < 0 ? nch : r == 0 ? last_nch : kSegChunks;
+            if (r >= 0) {
+                if (r == 0) {
+                    keep_state<DK>(checkpoint(NS), ss);
+                    big_g = state_from_memory<DK>(sg, a.dS_T ? a.dS_T + state_at : nullptr, DVT);
+                }
+                // rowdot(conj S, G) at the segment's end, this warp's columns; then S at its start
+                float2 *rg = rgs + ((r & 1) * NCW + w) * M + 2 * t4;
+                const float4 *end = checkpoint(s + 1), *start = checkpoint(s);
+                big_s = 0.f;
+#pragma unroll 1
+                for (int n = 0; n < TL::KS; ++n, rg += 16, end += 128, start += 128) {
+                    float x[16], y[16];
+                    tm_load(x, sg + 16 * n);
+                    read_piece(end, y);
+                    tm_wait_load(x);
 #pragma unroll
-        for (int n = 0; n < 2; ++n)
+                    for (int u = 0; u < 4; ++u) {                        // (tile, key)
+                        const int o = 8 * (u >> 1) + (u & 1);
+                        float re = y[o] * x[o] + y[o + 4] * x[o + 4] + y[o + 2] * x[o + 2] + y[o + 6] * x[o + 6];
+                        float im = y[o] * x[o + 4] - y[o + 4] * x[o] + y[o + 2] * x[o + 6] - y[o + 6] * x[o + 2];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
-                ri[n][i] = -fw * (acc[0][1][n][i] - acc[0][2][n][i]);
+                        for (int d = 4; d < 32; d <<= 1) {
+                            re += __shfl_xor_sync(0xffffffffu, re, d);
+                            im += __shfl_xor_sync(0xffffffffu, im, d);
+                        }
+                        if (g == 0) rg[8 * (u >> 1) + (u & 1)] = make_float2(re, im);
+                    }
+                    read_piece(start, y);
+                    tm_store(ss + 16 * n, y);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) big_s = fmaxf(big_s, fabsf(y[i]));
+                }
+                tm_wait_store();
             }
-        TokFrag fr, fb;
-        const float ir = make_frag(fr, rr, ri);
-        load_small<false>(fb, tile + TL::oM, lane);
-        product_small<false>(rr, ri, fr, fb, ir * inv[3]);
-        const float iu = make_frag(fr, rr, ri);
-        if constexpr (kPub) {
-            publish_frag(reinterpret_cast<uint4 *>(scr + SC::oU) + w * 128, fr, lane);
-            if (lane == 0) {
-                scal[(slot * NCW + w) * 4] = isv;
-                scal[(slot * NCW + w) * 4 + 1] = iu;
-            }
-        }
-        if (update)
-            state_update<DK>(sr, si, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
-    };
-
-    for (int c = 0; c < nch; ++c) {
-        if (c % kSegChunks == 0) store_state<KT>(checkpoint(c / kSegChunks), sr, si, lane);
-        forward_chunk(c % kSlots, c * kC, std::false_type{}, true);
-        bar_arrive(kBarDone + c % kSlots, kAll);
-    }
-
-    float gr[KT][4], gi[KT][4];
-    for (int r = 0; r < NS; ++r) {
-        const int s = NS - 1 - r, nc = r == 0 ? last_nch : kSegChunks, p0 = r == 0 ? 0 : last_nch + kSegChunks * (r - 1);
-        // rowdot(conj S, G) at the segment's end, this warp's columns; G then waits where that state was kept
-        {
-            float2 *rg = reinterpret_cast<float2 *>(smem + L::rg) + ((r & 1) * NCW + w) * M;
-            if (r == 0) {
+            // forward: U = M (V - W^* S), S <- gamma_C S + Y U; the second sweep leaves S and U for the gradients
+#pragma unroll 1
+            for (int c = 0; c < nc; ++c) {
+                const int slot = r < 0 ? c % kSlots : ring_slot(r, c), t0 = (r < 0 ? 0 : s * kSeg) + c * kC;
+                const bool pub = r >= 0;
+                if (!pub && c % kSegChunks == 0) keep_state<DK>(checkpoint(c / kSegChunks), ss);
+                unsigned char *scr = ring + (size_t)slot * SC::slot;
+                uint4 *ps = reinterpret_cast<uint4 *>(scr + SC::oS) + w * KT * 64 + lane;
+                float rr[2][4], ri[2][4];
+                load_rows(rr, static_cast<const T *>(a.v) + (row0 + (size_t)(t0 + 2 * t4) * a.H) * DVT + col, step, a.T - t0 - 2 * t4);
+                float isv;
+                const float sv = scale_for(warp_max(big_s), isv);
+                bar_sync(kBarFull + slot, 64 + kChain);
+                const uint32_t tile = base + slot * TL::bytes;
+                const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
+                float acc[1][3][2][4];
+                const uint32_t tiles[1] = {tile + TL::oW};
+                keys_product<DK, 1>(acc, ss, sv, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+                    if (pub) {
 #pragma unroll
-                for (int n = 0; n < KT; ++n)
+                        for (int e = 0; e < 2; ++e) {
+                            ps[(4 * kk + 2 * e) * 32] = make_uint4(transpose8x8(rh[2 * e]), transpose8x8(rh[2 * e + 1]), transpose8x8(rl[2 * e]), transpose8x8(rl[2 * e + 1]));
+                            ps[(4 * kk + 2 * e + 1) * 32] = make_uint4(transpose8x8(ih[2 * e]), transpose8x8(ih[2 * e + 1]), transpose8x8(il[2 * e]), transpose8x8(il[2 * e + 1]));
+                        }
+                    }
+                });
+                const float fw = isv * inv[0];
+#pragma unroll
+                for (int n = 0; n < 2; ++n)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        gr[n][i] = a.dS_T ? a.dS_T[state_at(n, i)] : 0.f;
-                        gi[n][i] = a.dS_T ? a.dS_T[state_at(n, i) + DVT] : 0.f;
+                        rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
+                        ri[n][i] = -fw * (acc[0][1][n][i] - acc[0][2][n][i]);
                     }
-            } else {
-                load_state<KT>(checkpoint(s + 1), sr, si, lane);
-            }
-#pragma unroll
-            for (int n = 0; n < KT; ++n)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    float x = sr[n][e] * gr[n][e] + si[n][e] * gi[n][e] + sr[n][e + 2] * gr[n][e + 2] + si[n][e + 2] * gi[n][e + 2];
-                    float y = sr[n][e] * gi[n][e] - si[n][e] * gr[n][e] + sr[n][e + 2] * gi[n][e + 2] - si[n][e + 2] * gr[n][e + 2];
-#pragma unroll
-                    for (int d = 4; d < 32; d <<= 1) {
-                        x += __shfl_xor_sync(0xffffffffu, x, d);
-                        y += __shfl_xor_sync(0xffffffffu, y, d);
+                TokFrag fr;
+                {
+                    TokFrag fb;
+                    const float ir = make_frag(fr, rr, ri);
+                    load_small<false>(fb, tile + TL::oM, lane);
+                    product_small<false>(rr, ri, fr, fb, ir * inv[3]);
+                }
+                const float iu = make_frag(fr, rr, ri);
+                if (pub) {
+                    publish_frag(reinterpret_cast<uint4 *>(scr + SC::oU) + w * 128, fr, lane);
+                    if (lane == 0) {
+                        scal[(slot * NCW + w) * 4] = isv;
+                        scal[(slot * NCW + w) * 4 + 1] = iu;
                     }
-                    if (g == 0) rg[8 * n + 2 * t4 + e] = make_float2(x, y);
                 }
-            if (r > 0) store_state<KT>(checkpoint(s + 1), gr, gi, lane);
-        }
-        load_state<KT>(checkpoint(s), sr, si, lane);
-        for (int c = 0; c < nc; ++c) {
-            const int slot = ring_slot(r, c);
-            if (p0 + c >= kSlots) bar_sync(kBarFree + slot, kAll);
-            forward_chunk(slot, s * kSeg + c * kC, std::true_type{}, c + 1 < nc);
-        }
-        if (r == 0) {
-#pragma unroll
-            for (int n = 0; n < KT; ++n)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    gr[n][i] = a.dS_T ? a.dS_T[state_at(n, i)] : 0.f;
-                    gi[n][i] = a.dS_T ? a.dS_T[state_at(n, i) + DVT] : 0.f;
-                }
-        } else {
-            load_state<KT>(checkpoint(s + 1), gr, gi, lane);
-        }
-        for (int c = nc - 1; c >= 0; --c) {
-            const int slot = ring_slot(r, c), t0 = s * kSeg + c * kC;
-            unsigned char *scr = ring + (size_t)slot * SC::slot;
-            const bool has_im = a.d_o_im != nullptr;
-            float yr[2][4], yi[2][4];
-            load_tokens(a.d_o, t0, 1.f, yr);
-            load_tokens(a.d_o_im, t0, -1.f, yi);
-            const uint32_t tile = base + slot * TL::bytes;
-            const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
-            float ig;
-            const float sg = scale_for(__reduce_max_sync(0xffffffffu, max(max_bits4(gr), max_bits4(gi))), ig);
-            float acc[1][3][2][4];
-            const uint32_t tiles[1] = {tile + TL::oY};
-            product_over_keys<DK, 1, true>(acc, gr, gi, sg, tiles, lane, reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64);
-            TokFrag fy, fp, fb;
-            const float iy = make_frag(fy, yr, yi);
-            float pr[2][4], pi[2][4];
-            const float fg = ig * inv[1];
-#pragma unroll
-            for (int n = 0; n < 2; ++n)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    pr[n][i] = fg * acc[0][0][n][i];
-                    pi[n][i] = fg * (acc[0][1][n][i] - acc[0][2][n][i]);
-                }
-            load_small<true>(fb, tile + TL::oA, lane);
-            product_small_conj<kExact>(pr, pi, fy, fb, iy * inv[4], has_im);
-            const float ip = make_frag(fp, pr, pi);
-            load_small<true>(fb, tile + TL::oM, lane);
-            product_small<true>(pr, pi, fp, fb, ip * inv[3]);
-#pragma unroll
-            for (int n = 0; n < 2; ++n)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int t = t0 + 8 * n + 2 * t4 + (i & 1);
-                    if (t < a.T) st_val(static_cast<T *>(a.dv), (row0 + (size_t)t * a.H) * DVT + col + 8 * (i >> 1), pr[n][i]);
-                }
-            const float ib = make_frag(fp, pr, pi);
-            publish_frag(reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, fp, lane);
-            if (lane == 0) {
-                scal[(slot * NCW + w) * 4 + 2] = ig;
-                scal[(slot * NCW + w) * 4 + 3] = ib;
+                if (!pub || c + 1 < nc)
+                    big_s = state_update<DK>(ss, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
+                if (!pub) bar_arrive(kBarDone + slot, kAux + kChain);
             }
-            // G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc
-            const float fq = iy * inv[2], fw = ib * inv[0];
-            const float4 *gamma = reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG);
-            const uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
+            if (r < 0) continue;
+#pragma unroll 1
+            for (int c = nc - 1; c >= 0; --c) {
+                const int slot = ring_slot(r, c), t0 = s * kSeg + c * kC, left = a.T - t0 - 2 * t4;
+                const size_t at0 = (row0 + (size_t)(t0 + 2 * t4) * a.H) * DVT + col;
+                unsigned char *scr = ring + (size_t)slot * SC::slot;
+                uint4 *ps = reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64 + lane;
+                const bool has_im = a.d_o_im != nullptr;
+                TokFrag fy;                                              // Yb^*
+                float iy;
+                {
+                    float yr[2][4], yi[2][4];
+                    load_rows(yr, static_cast<const T *>(a.d_o) + at0, step, left);
+                    load_rows(yi, static_cast<const T *>(a.d_o_im) + at0, step, has_im ? left : 0);
 #pragma unroll
-            for (int np = 0; np < KT; np += 2) {
-                uint32_t qrh[4], qrl[4], qih[4], qil[4], wrh[4], wrl[4], wih[4], wil[4];
-                ldsm_t(qrh, at + TL::oQ + np * 16);
-                ldsm_t(qrl, at + TL::oQ + np * 16 + TL::PL);
-                ldsm_t(qih, at + TL::oQ + np * 16 + 2 * TL::PL);
-                ldsm_t(qil, at + TL::oQ + np * 16 + 3 * TL::PL);
-                ldsm_t(wrh, at + TL::oW + np * 16);
-                ldsm_t(wrl, at + TL::oW + np * 16 + TL::PL);
-                ldsm_t(wih, at + TL::oW + np * 16 + 2 * TL::PL);
-                ldsm_t(wil, at + TL::oW + np * 16 + 3 * TL::PL);
+                    for (int n = 0; n < 2; ++n)
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int n = np + e;
-                    float qr_[4] = {0.f, 0.f, 0.f, 0.f}, qn[4] = {0.f, 0.f, 0.f, 0.f}, qm[4] = {0.f, 0.f, 0.f, 0.f};
-                    float wr_[4] = {0.f, 0.f, 0.f, 0.f}, wn[4] = {0.f, 0.f, 0.f, 0.f}, wm[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma3(wr_, fp.rh, fp.rl, wrh[2 * e], wrh[2 * e + 1], wrl[2 * e], wrl[2 * e + 1]);
-                    mma3(wm, fp.ih, fp.il, wrh[2 * e], wrh[2 * e + 1], wrl[2 * e], wrl[2 * e + 1]);
-                    mma3(wn, fp.ih, fp.il, wih[2 * e], wih[2 * e + 1], wil[2 * e], wil[2 * e + 1]);
-                    mma3x<kExact>(qr_, fy.rh, fy.rl, qrh[2 * e], qrh[2 * e + 1], qrl[2 * e], qrl[2 * e + 1]);
-                    mma3x<kExact>(qm, fy.rh, fy.rl, qih[2 * e], qih[2 * e + 1], qil[2 * e], qil[2 * e + 1]);
-                    mma3(wm, fp.rh, fp.rl, wih[2 * e], wih[2 * e + 1], wil[2 * e], wil[2 * e + 1]);
+                        for (int i = 0; i < 4; ++i) yi[n][i] = -yi[n][i];
+                    iy = make_frag(fy, yr, yi);
+                }
+                const uint32_t tile = base + slot * TL::bytes;
+                const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
+                float ig;
+                const float sv = scale_for(warp_max(big_g), ig);
+                float acc[1][3][2][4];
+                const uint32_t tiles[1] = {tile + TL::oY};
+                keys_product<DK, 1>(acc, sg, sv, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        ps[(4 * kk + 2 * e) * 32] = make_uint4(transpose8x8(rh[2 * e]), transpose8x8(rh[2 * e + 1]), transpose8x8(rl[2 * e]), transpose8x8(rl[2 * e + 1]));
+                        ps[(4 * kk + 2 * e + 1) * 32] = make_uint4(transpose8x8(ih[2 * e]), transpose8x8(ih[2 * e + 1]), transpose8x8(il[2 * e]), transpose8x8(il[2 * e + 1]));
+                    }
+                });
+                float pr[2][4], pi[2][4];
+                {                                                        // + (A D_beta)^H Yb^*
+                    TokFrag fb;
+                    load_small<true>(fb, tile + TL::oA, lane);
+                    const float fg = ig * inv[1], fa = iy * inv[4];
+#pragma unroll
+                    for (int n = 0; n < 2; ++n) {
+                        float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f}, ni[4] = {0.f, 0.f, 0.f, 0.f};
+                        mma3x<kExact>(re, fy.rh, fy.rl, fb.rh[2 * n], fb.rh[2 * n + 1], fb.rl[2 * n], fb.rl[2 * n + 1]);
+                        mma3x<kExact>(ni, fy.rh, fy.rl, fb.ih[2 * n], fb.ih[2 * n + 1], fb.il[2 * n], fb.il[2 * n + 1]);
+                        if (has_im) {
+                            mma3x<kExact>(re, fy.ih, fy.il, fb.ih[2 * n], fb.ih[2 * n + 1], fb.il[2 * n], fb.il[2 * n + 1]);
+                            mma3x<kExact>(im, fy.ih, fy.il, fb.rh[2 * n], fb.rh[2 * n + 1], fb.rl[2 * n], fb.rl[2 * n + 1]);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            pr[n][i] = fmaf(fa, re[i], fg * acc[0][0][n][i]);
+                            pi[n][i] = fmaf(fa, im[i] - ni[i], fg * (acc[0][1][n][i] - acc[0][2][n][i]));
+                        }
+                    }
+                }
+                TokFrag fp;
+                {
+                    TokFrag fb;
+                    const float ip = make_frag(fp, pr, pi);
+                    load_small<true>(fb, tile + TL::oM, lane);
+                    product_small<true>(pr, pi, fp, fb, ip * inv[3]);
+                }
+                store_rows(static_cast<T *>(a.dv) + at0, pr, step, left);
+                const float ib = make_frag(fp, pr, pi);
+                publish_frag(reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, fp, lane);
+                if (lane == 0) {
+                    scal[(slot * NCW + w) * 4 + 2] = ig;
+                    scal[(slot * NCW + w) * 4 + 3] = ib;
+                }
+                // G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc
+                const float fq = iy * inv[2], fw = -ib * inv[0];
+                const float4 *gamma = reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG) + t4;
+                uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
+                uint32_t nih[4], nil[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    nih[i] = fp.ih[i] ^ 0x80008000u;
+                    nil[i] = fp.il[i] ^ 0x80008000u;
+                }
+                big_g = 0.f;
+#pragma unroll 1
+                for (int np = 0; np < TL::KS; ++np, at += 32, gamma += 8) {
+                    float x[16];
+                    tm_load(x, sg + 16 * np);
+                    uint32_t qh[4], ql[4], jh[4], jl[4];
+                    ldsm_t(qh, at + TL::oQ);
+                    ldsm_t(jh, at + TL::oQ + 2 * TL::PL);
+                    ldsm_t(ql, at + TL::oQ + TL::PL);
+                    ldsm_t(jl, at + TL::oQ + 3 * TL::PL);
+                    float qr[2][4], qi[2][4];
+#pragma unroll
+                    for (int n = 0; n < 2; ++n) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) qr[n][i] = qi[n][i] = 0.f;
+                        mma3x<kExact>(qr[n], fy.rh, fy.rl, qh[2 * n], qh[2 * n + 1], ql[2 * n], ql[2 * n + 1]);
+                        mma3x<kExact>(qi[n], fy.rh, fy.rl, jh[2 * n], jh[2 * n + 1], jl[2 * n], jl[2 * n + 1]);
+                    }
                     if (has_im) {
-                        mma3x<kExact>(qn, fy.ih, fy.il, qih[2 * e], qih[2 * e + 1], qil[2 * e], qil[2 * e + 1]);
-                        mma3x<kExact>(qm, fy.ih, fy.il, qrh[2 * e], qrh[2 * e + 1], qrl[2 * e], qrl[2 * e + 1]);
-                    }
-                    const float4 gm = gamma[4 * n + t4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float cr = (i & 1) ? gm.z : gm.x, ci = (i & 1) ? gm.w : gm.y, x = gr[n][i], y = gi[n][i];
-                        gr[n][i] = fmaf(fq, qr_[i] - qn[i], fmaf(-fw, wr_[i] - wn[i], cr * x + ci * y));
-                        gi[n][i] = fmaf(fq, qm[i], fmaf(-fw, wm[i], cr * y - ci * x));
+                        for (int n = 0; n < 2; ++n) {
+                            float ni[4] = {0.f, 0.f, 0.f, 0.f};
+                            mma3x<kExact>(ni, fy.ih, fy.il, jh[2 * n], jh[2 * n + 1], jl[2 * n], jl[2 * n + 1]);
+                            mma3x<kExact>(qi[n], fy.ih, fy.il, qh[2 * n], qh[2 * n + 1], ql[2 * n], ql[2 * n + 1]);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) qr[n][i] -= ni[i];
+                        }
                     }
+                    tm_wait_load(x);
+#pragma unroll
+                    for (int n = 0; n < 2; ++n) {
+                        const float4 gm = gamma[4 * n];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float cr = (i & 1) ? gm.z : gm.x, ci = (i & 1) ? gm.w : gm.y, u = x[8 * n + i], v = x[8 * n + 4 + i];
+                            x[8 * n + i] = fmaf(fq, qr[n][i], cr * u + ci * v);
+                            x[8 * n + 4 + i] = fmaf(fq, qi[n][i], cr * v - ci * u);
+                        }
+                    }
+                    tokens_product<DK>(qr, qi, fp, nih, nil, at + TL::oW);
+#pragma unroll
+                    for (int n = 0; n < 2; ++n)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            x[8 * n + i] = fmaf(fw, qr[n][i], x[8 * n + i]);
+                            x[8 * n + 4 + i] = fmaf(fw, qi[n][i], x[8 * n + 4 + i]);
+                            big_g = fmaxf(big_g, fmaxf(fabsf(x[8 * n + i]), fabsf(x[8 * n + 4 + i])));
+                        }
+                    tm_store(sg + 16 * np, x);
                 }
+                tm_wait_store();
+                bar_arrive(kBarDone + slot, kAux + kChain);
             }
-            bar_arrive(kBarDone + slot, kAll);
         }
+        state_to_memory<DK>(sg, a.dS0 + state_at, DVT);
     }
-#pragma unroll
-    for (int n = 0; n < KT; ++n)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            a.dS0[state_at(n, i)] = gr[n][i];
-            a.dS0[state_at(n, i) + DVT] = gi[n][i];
-        }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid < 32) tm_free(tmem, L::columns);
 }
 
 // ---- the sums over the column blocks: out[i] = share_0[i] + share_1[i] + ... in that order, one thread per four
@@ -930,7 +1081,7 @@ cudaError_t launch_cols(const BackwardArgs &x, void *workspace, cudaStream_t str
     a.rows = bhn * x.T;
     a.check = ws + w.check; a.scratch = ws + w.scratch;
     a.dq_p = ws + w.dq; a.dk_p = ws + w.dk; a.dalpha_p = ws + w.dalpha; a.dtheta_p = ws + w.dtheta; a.dbeta_p = ws + w.dbeta;
-    kern<<<dim3((unsigned)bhn, NSL), kAux + 2 * DV, L::bytes, stream>>>(a);
+    kern<<<dim3((unsigned)bhn, NSL), kAux + kSolve + 2 * DV, L::bytes, stream>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (launches) ++*launches;
     if constexpr (NSL > 1) {

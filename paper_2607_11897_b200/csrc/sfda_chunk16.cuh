@@ -480,10 +480,10 @@ struct PrepRaw {
     float be[TPT];
 };
 
-template <int DK, int PW, bool kNeedQ, typename T>
+template <int DK, int PW, typename T>
 __device__ __forceinline__ void prep_fetch(PrepRaw<PrepMap<DK, PW>::TPT, T> &in, const T *__restrict__ q, const T *__restrict__ k,
                                            const float *__restrict__ alpha, const float *__restrict__ theta,
-                                           const float *__restrict__ beta, size_t row0, int H, int t0, int T_, int tid)
+                                           const float *__restrict__ beta, size_t row0, int H, int t0, int T_, bool needq, int tid)
 {
     using PM = PrepMap<DK, PW>;
     const int pair = tid % PM::PAIRS, t1 = t0 + tid / PM::PAIRS * PM::TPT;
@@ -497,7 +497,7 @@ __device__ __forceinline__ void prep_fetch(PrepRaw<PrepMap<DK, PW>::TPT, T> &in,
         if (t1 + x < T_) {
             const size_t row = row0 + (size_t)(t1 + x) * H;
             in.k[x].load(k + row * DK + 4 * pair);
-            if constexpr (kNeedQ) in.q[x].load(q + row * DK + 4 * pair);
+            if (needq) in.q[x].load(q + row * DK + 4 * pair);
             in.al[x] = *reinterpret_cast<const float2 *>(alpha + row * PM::M + 2 * pair);
             in.th[x] = *reinterpret_cast<const float2 *>(theta + row * PM::M + 2 * pair);
             in.be[x] = beta[row];
@@ -517,7 +517,7 @@ __device__ __forceinline__ void put_planes(unsigned char *p, int pl, float r0, f
     *reinterpret_cast<uint32_t *>(p + 3 * pl) = l;
 }
 
-// Operand planes of one chunk: W, Y (and Q) into the slot, Kb_i = beta_i k_i / gamma_i into `kb` for the Gram products.
+// Operand planes of one chunk: W, Y (and Q, with needq) into the slot, Kb_i = beta_i k_i / gamma_i into `kb` for the Gram products.
 // `vals` (or NULL) receives what the gradients need again, two float4 per (token, key): rotated key and query; prod
 // alpha up to the token and after it, e^{i phi}.  Called by all 32 PW threads; the planes are complete for other
 // threads only after a barrier of the caller's.
@@ -526,9 +526,9 @@ __device__ __forceinline__ void put_planes(unsigned char *p, int pl, float r0, f
 // tokens): Kb's entries then reach 2^16, the smaller ones keep an absolute error of 2^-39 of that, 2^-23 beside the
 // unit-sized entries of W they meet.  Stronger decays take slow_gram.  Returns whether the chunk is fast (the same
 // value in every thread).
-template <int DK, int PW, bool kNeedQ, typename T>
+template <int DK, int PW, typename T>
 __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, T> &in, float4 *vals, unsigned char *slot,
-                                            unsigned char *kb, unsigned char *scan, int tid)
+                                            unsigned char *kb, unsigned char *scan, bool needq, int tid)
 {
     using PM = PrepMap<DK, PW>;
     using TL = Tile<DK>;
@@ -590,7 +590,8 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
         cos_sin(ub.y + u[x].y, c1, s1);
         float4 r = in.k[x].get();
         kk[x] = make_float4(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0, r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
-        if constexpr (kNeedQ) {
+        qq[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (needq) {
             r = in.q[x].get();
             qq[x] = make_float4(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0, r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
             if (vals) {
@@ -612,7 +613,7 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
     uint32_t m[4] = {__float_as_uint(mw), __float_as_uint(my), __float_as_uint(mq), __float_as_uint(mb)};   // all >= 0
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-        if (kNeedQ || i != 2) m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+        m[i] = __reduce_max_sync(0xffffffffu, m[i]);
     if (lane == 0) *reinterpret_cast<uint4 *>(red + 4 * warp) = make_uint4(m[0], m[1], m[2], m[3]);
     bar_sync(kBarAux, 32 * PW);
 #pragma unroll 2
@@ -641,7 +642,7 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
         put_planes(slot + TL::oW + at, TL::PL, w0 * kk[x].x, w0 * kk[x].y, w1 * kk[x].z, w1 * kk[x].w);
         put_planes(slot + TL::oY + at, TL::PL, y0 * (gc0.x * kk[x].x - gc0.y * kk[x].y), y0 * (gc0.x * kk[x].y + gc0.y * kk[x].x),
                    y1 * (gc1.x * kk[x].z - gc1.y * kk[x].w), y1 * (gc1.x * kk[x].w + gc1.y * kk[x].z));
-        if constexpr (kNeedQ) put_planes(slot + TL::oQ + at, TL::PL, sq * qq[x].x, sq * qq[x].y, sq * qq[x].z, sq * qq[x].w);
+        if (needq) put_planes(slot + TL::oQ + at, TL::PL, sq * qq[x].x, sq * qq[x].y, sq * qq[x].z, sq * qq[x].w);
         if (fast) {
             const float b0 = bi[x].x * sb, b1 = bi[x].y * sb;
             put_planes(kb + at, TL::PL, b0 * kk[x].x, b0 * kk[x].y, b1 * kk[x].z, b1 * kk[x].w);
@@ -653,14 +654,14 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
 // The Gram matrices of a chunk whose decays are too strong to divide by: every pair's decay as a running product.  Called
 // by all 32 PW threads after prep_planes returned false; `slow` is a scratch of PrepMap::slow_bytes nobody else uses.
 // Reads its inputs again: passed on, they would not stay in registers on the common path.
-template <int DK, int PW, bool kNeedQ, typename T>
+template <int DK, int PW, typename T>
 __device__ __noinline__ void slow_gram(const T *q, const T *k, const float *alpha, const float *theta, const float *beta,
                                        size_t row0, int H, int t0, int T_, unsigned char *slow, const unsigned char *scan,
-                                       float2 *gk, float2 *gq, int tid)
+                                       float2 *gk, float2 *gq, bool needq, int tid)
 {
     using PM = PrepMap<DK, PW>;
     PrepRaw<PM::TPT, T> in;
-    prep_fetch<DK, PW, kNeedQ, T>(in, q, k, alpha, theta, beta, row0, H, t0, T_, tid);
+    prep_fetch<DK, PW, T>(in, q, k, alpha, theta, beta, row0, H, t0, T_, needq, tid);
     constexpr int M = PM::M, PAIRS = PM::PAIRS, TPT = PM::TPT, LD = M + 4;
     const int pair = tid % PAIRS, grp = tid / PAIRS, lane = tid & 31, warp = tid >> 5;
     const uint2 *su = reinterpret_cast<const uint2 *>(scan + PM::NG * PAIRS * 8);
@@ -677,7 +678,7 @@ __device__ __noinline__ void slow_gram(const T *q, const T *k, const float *alph
         float4 r = in.k[x].get();
         sk[at] = make_float2(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0);
         sk[at + 1] = make_float2(r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
-        if constexpr (kNeedQ) {
+        if (needq) {
             r = in.q[x].get();
             sq[at] = make_float2(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0);
             sq[at + 1] = make_float2(r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
@@ -700,7 +701,7 @@ __device__ __noinline__ void slow_gram(const T *q, const T *k, const float *alph
                 const float br = w[e] * b.x, bim = w[e] * b.y;
                 s[0] += x.x * br + x.y * bim;
                 s[1] += x.x * bim - x.y * br;
-                if constexpr (kNeedQ) {
+                if (needq) {
                     const float2 y = sq[t * LD + j];
                     s[2] += y.x * br + y.y * bim;
                     s[3] += y.x * bim - y.y * br;
@@ -714,7 +715,7 @@ __device__ __noinline__ void slow_gram(const T *q, const T *k, const float *alph
                 for (int e = 0; e < 4; ++e) s[e] += __shfl_xor_sync(0xffffffffu, s[e], d);
             if (lane == 0) {
                 gk[t * 17 + i] = make_float2(be * s[0], be * s[1]);
-                if constexpr (kNeedQ) gq[t * 17 + i] = make_float2(be * s[2], be * s[3]);
+                if (needq) gq[t * 17 + i] = make_float2(be * s[2], be * s[3]);
             }
         }
     }

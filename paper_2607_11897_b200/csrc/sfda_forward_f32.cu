@@ -86,16 +86,16 @@ __global__ void __launch_bounds__(Roles<NB>::threads, 1) sfda_forward_f32_kernel
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
         const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
         PrepRaw<L::PM::TPT, T> in;
-        prep_fetch<DK, kPrepWarps, true, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, 0, a.T, role.prep);
+        prep_fetch<DK, kPrepWarps, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, 0, a.T, true, role.prep);
         for (int c = 0; c < nch; ++c) {
             const int slot = c % kSlots;
             if (c >= kSlots) bar_sync(kBarDone + slot, kPrep + kChain);
             PrepRaw<L::PM::TPT, T> next;
-            prep_fetch<DK, kPrepWarps, true, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, (c + 1) * kC, a.T, role.prep);
+            prep_fetch<DK, kPrepWarps, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, (c + 1) * kC, a.T, true, role.prep);
             float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes);
-            if (!prep_planes<DK, kPrepWarps, true, T>(in, nullptr, smem + slot * TL::bytes, smem + L::kb + slot * TL::BIG, smem + L::scan, role.prep))
-                slow_gram<DK, kPrepWarps, true, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, smem + L::slow, smem + L::scan,
-                                                   gk, gk + 16 * 17, role.prep);
+            if (!prep_planes<DK, kPrepWarps, T>(in, nullptr, smem + slot * TL::bytes, smem + L::kb + slot * TL::BIG, smem + L::scan, true, role.prep))
+                slow_gram<DK, kPrepWarps, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, smem + L::slow, smem + L::scan,
+                                                   gk, gk + 16 * 17, true, role.prep);
             bar_arrive(kBarPlanes + slot, kPrep + 64);
             in = next;
         }
