@@ -482,14 +482,12 @@ SFDA_API int sfda_forward_fused(const void *q, const void *k_raw, const void *v,
  *               to its two real numbers), dv [B][T][H][d_v] dtype, dalpha, dtheta [B][T][H][m] float,
  *               dbeta [B][T][H] float, dS0 [B][H][d_k][d_v] float.  All are required and overwritten.
  *  workspace:   sfda_backward_workspace_bytes(...) bytes of device scratch (per (batch, head) pair the state at the
- *               start of every 64 tokens and the 64 states of one such segment; with few sequences also fp32
- *               shares of dq, dk, dalpha, dtheta, dbeta per block of value columns); clobbered.
+ *               start of every 64 tokens and room for 64 states; with few sequences more); clobbered.
  *
- * d_k, d_v in {64, 128}; no chunk argument (the derivative does not depend on the chunking).  fp32 arithmetic on
- * the CUDA cores, token by token: a first correct path, not a fast one.  One CTA per (batch, head) pair; when
- * B * H is at most half (a quarter) of the 148 SMs of a B200, the value columns -- which never interact -- are split
- * into blocks of 64 (32) with a CTA each, and a second kernel adds the blocks' shares of the sums over the
- * columns in a fixed order.  The result is deterministic either way.
+ * d_k, d_v in {64, 128}; no chunk argument (the derivative does not depend on the chunking).  fp32 precision on the
+ * tensor cores in chunks of 16 tokens, as the fp32 forward.  One launch, one CTA per (batch, head) pair; when B * H is
+ * at most half of the 148 SMs of a B200, two: the chains of the state and of its cotangent by themselves, then every
+ * segment of 64 tokens as a unit of its own.  The result is deterministic either way.
  */
 SFDA_API size_t sfda_backward_workspace_bytes(int B, int T, int H, int d_k, int d_v, int dtype);
 SFDA_API int sfda_backward(const void *q, const void *k, const void *v,

@@ -19,14 +19,13 @@
 // decayed keys and queries.  Where alpha_t < 1/16 the division would lose digits: dalpha comes from its definition,
 // sum_c conj(S_{t-1,jc}) Zb_jc, rebuilt for that (token, coordinate) alone.
 //
-// One CTA per (batch, head) pair and block of value columns (all of them, or with few sequences 64 or 32: the columns
-// never interact, and a second kernel adds the blocks' shares of the sums over the columns in a fixed order).  The
-// CHAIN warps walk the sequence forward once, keeping the state every 64 tokens, then per segment of 64 tokens, last to
-// first: forward again from the checkpoint, backward through it.  They leave S_0, U, G_C, Bc of a chunk in a scratch
-// ring as the operand registers of the gradients' products.  The AUX warps prepare the chunks' operand tiles and turn
-// what the chain leaves into gradients one chunk behind it; SOLVE warps make the Gram matrices and the inverse.  They
-// meet at hardware barriers: PLANES (operand planes ready), FULL (the tile is complete), DONE (the chain is
-// through with the chunk); AUX prepares a slot again only after it has written that slot's gradients.
+// One CTA per (batch, head) pair walks the sequence forward once, keeping the state every 64 tokens, then per segment of
+// 64 tokens, last to first: forward again from the kept state, backward through it.  With few sequences the two chains
+// run by themselves first, in blocks of value columns, and every segment is then a unit of its own.  The CHAIN warps leave
+// S_0, U, G_C, Bc of a chunk in a scratch ring as the operand registers of the gradients' products.  PREP warps prepare
+// the chunks' operand tiles; GRAD warps turn what the chain leaves into gradients one chunk behind it (they are what
+// bounds the kernel, so nothing else is theirs).  They meet at hardware barriers, one per slot: FULL (a tile is
+// complete), DONE (the chain came back through the chunk), FREE (the slot may be prepared again).
 #include "sfda_chunk16.cuh"
 #include "sfda_internal.h"
 
@@ -38,50 +37,47 @@ using namespace c16;
 constexpr int kSeg = 64;                    // tokens between checkpoints
 constexpr int kSegChunks = kSeg / kC;
 static_assert(kSegChunks == kSlots, "a segment's operand tiles fill the ring");
-constexpr int kAuxWarps = 8, kAux = 32 * kAuxWarps, kSolve = 128;
-// PLANES goes by the order of preparation, modulo 4 (the ring turns round at every segment, so that neighbours share a
-// slot; AUX is at most two chunks ahead of SOLVE); SOLVED: SOLVE is through with a chunk's Kb planes, modulo 2.
-constexpr int kBarPlanes = 10, kBarSolved = 14;
+constexpr int kGradWarps = 8, kGrad = 32 * kGradWarps;
+constexpr int kBarGrad = kBarAux, kBarPrep = 14;
 
 struct BwdArgsDev {
     const void *q, *k, *v, *d_o, *d_o_im;
     const float *alpha, *theta, *beta, *S0, *dS_T;
     void *dq, *dk, *dv;
     float *dalpha, *dtheta, *dbeta, *dS0;
-    float *dq_p, *dk_p, *dalpha_p, *dtheta_p, *dbeta_p;   // shares of the column blocks: [blocks][rows][...] fp32
-    float *check, *scratch;
-    size_t rows;
-    int T, H, NS;
+    // kept states: S at the start of segment s of pair bh at keep_s + (bh * pitch + s) * d_k * d_v, the final state in the
+    // place after the last; G at the end of segment s likewise at keep_g (few sequences only)
+    float *keep_s, *keep_g;
+    unsigned char *ring;      // the CTAs' scratch rings, ring_bytes apart
+    size_t ring_bytes;
+    int T, H, NS, pitch, units;
 };
 
 // One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
 // S_0, G_C as B operands [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U, Bc as A operands
 // [chain warp][plane][lane] uint4; then the chunk's rotated keys and queries, decays and phases, 8 floats per
-// (token, key).  Behind the ring: rowdot(S, G) [2][chain warp][key] and the final state.
+// (token, key).  Behind the ring: rowdot(S, G) [2][chain warp][key] and slow_gram's scratch.
 template <int DK, int NB>
 struct BwdScratch {
     static constexpr int NCW = NB / 16, KT = DK / 16, M = DK / 2;
     static constexpr int oS = 0, oU = oS + NCW * KT * 1024, oG = oU + NCW * 2048, oB = oG + NCW * KT * 1024;
     static constexpr int oV = oB + NCW * 2048, slot = oV + 16 * M * 32;
-    static constexpr int oRg = slot * kSlots, oEnd = oRg + 2 * NCW * M * 8;
-    static_assert((size_t)oEnd + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "the scratch must fit the workspace");
+    static constexpr int oRg = slot * kSlots, oSlow = oRg + 2 * NCW * M * 8;
+    static constexpr size_t bytes = (oSlow + PrepMap<DK, kPrepWarps>::slow_bytes + 255) / 256 * 256;
+    static_assert(bytes + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "ring and final state must fit a pair's scratch");
 };
 
 template <int DK, int NB>
 struct BwdSmem {
-    using PM = PrepMap<DK, kAuxWarps>;
+    using PM = PrepMap<DK, kPrepWarps>;
     static constexpr int NCW = NB / 16, M = DK / 2;
     static constexpr int up(int x) { return (x + 127) / 128 * 128; }
-    static constexpr int gram_bytes = 2 * 16 * 17 * 8;
-    static constexpr int kb = kSlots * Tile<DK>::bytes;           // Kb planes, two chunks
-    static constexpr int gram = kb + 2 * Tile<DK>::BIG;           // the two Gram matrices, two chunks
-    // Yb, Bc, U of the chunk as A operands; slow_gram's scratch while a tile is prepared
-    static constexpr int frag = up(gram + 2 * gram_bytes);
-    static constexpr int frag_bytes = 3 * NCW * 2048 > PM::slow_bytes ? 3 * NCW * 2048 : PM::slow_bytes;
-    // U Yb^T, U B^T in two halves over the columns: float2 [2][2][16][17]; the scan's scratch while a tile is prepared
-    static constexpr int uy = up(frag + frag_bytes);
+    static constexpr int kb = kSlots * Tile<DK>::bytes;           // PREP: Kb planes,
+    static constexpr int gram = kb + Tile<DK>::BIG;               // the two Gram matrices,
+    static constexpr int scan = gram + 2 * 16 * 17 * 8;           // the scan's scratch
+    static constexpr int frag = up(scan + PM::scan_bytes);        // GRAD: Yb, Bc, U of the chunk as A operands,
+    static constexpr int uy = up(frag + 3 * NCW * 2048);          // U Yb^T, U B^T in two halves over the columns: float2 [2][2][16][17]
     static constexpr int uy_bytes = 4 * 16 * 17 * 8;
-    static_assert(PM::scan_bytes <= uy_bytes, "the scan's scratch");
     static constexpr int tri = uy + uy_bytes;                     // the corrections' triangular factors: 4 x 4 uint4 [32]
     static constexpr int scal = tri + 4 * 4 * 512;                // inverse scales [slot][NCW] (S, U, G, B), [NCW] Yb, [4] tri
     static constexpr int db = scal + kSlots * NCW * 16 + 48;      // dbeta: [8][16] floats
@@ -232,16 +228,16 @@ __device__ __noinline__ float small_alpha(const float4 *vals, const uint4 *frag,
     return sum;
 }
 
-template <int DK, int DVT, int NB, typename T>
+template <int DK, int NB, typename T>
 __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, const float2 *rg, int slot,
                                                 bool first, int t0, size_t row0, float2 (&carry)[2], int tid)
 {
     using L = BwdSmem<DK, NB>;
     using SC = BwdScratch<DK, NB>;
     using TL = Tile<DK>;
-    constexpr int NCW = L::NCW, M = L::M, KT = M / 8, NSL = DVT / NB;
+    constexpr int NCW = L::NCW, M = L::M, KT = M / 8;
     constexpr bool kExact = sizeof(T) == 2;
-    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3, c0 = blockIdx.y * NB;
+    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3;
     const bool has_im = a.d_o_im != nullptr;
     uint4 *frag = reinterpret_cast<uint4 *>(smem + L::frag);                      // [Yb, Bc, U][NCW][4][32]
     uint4 *tri = reinterpret_cast<uint4 *>(smem + L::tri);
@@ -269,7 +265,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             const int t = t0 + g + 8 * (i & 1);
             y[0][i] = y[1][i] = make_float2(0.f, 0.f);
             if (t < a.T) {
-                const size_t at = (row0 + (size_t)t * a.H) * DVT + c0 + 16 * w + 2 * t4 + 8 * (i >> 1);
+                const size_t at = (row0 + (size_t)t * a.H) * NB + 16 * w + 2 * t4 + 8 * (i >> 1);
                 y[0][i] = make_float2(ld_val(static_cast<const T *>(a.d_o), at), ld_val(static_cast<const T *>(a.d_o), at + 1));
                 if (has_im) y[1][i] = make_float2(ld_val(static_cast<const T *>(a.d_o_im), at), ld_val(static_cast<const T *>(a.d_o_im), at + 1));
             }
@@ -292,7 +288,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             frag[(w * 4 + 2 * c + 1) * 32 + lane] = make_uint4(l[0], l[1], l[2], l[3]);
         }
     }
-    bar_sync(kBarAux, kAux);
+    bar_sync(kBarGrad, kGrad);
 
     // U Yb^T (index [i][t]: u_i . yb_t) and U B^T (b_t = beta_t p_t = conj of the rows of Bc): warp = (matrix, half of
     // the tokens t, half of the value columns); the A-operand registers of tokens 0-7 / 8-15 are that half's B operand
@@ -419,7 +415,26 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             }
         }
     }
-    bar_sync(kBarAux, kAux);
+    // what the elements need besides, requested here: it comes from L2 and memory
+    float4 vk[4], vp[4], last[2];
+    float2 al2[2];
+    float be2[2];
+    if (warp < KT) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int t = t0 + g + 8 * r;
+            const size_t row = row0 + (size_t)t * a.H;
+            const float4 *p = vals + ((g + 8 * r) * M + 8 * warp + 2 * t4) * 2;
+            vk[2 * r] = p[0];
+            vp[2 * r] = p[1];
+            vk[2 * r + 1] = p[2];
+            vp[2 * r + 1] = p[3];
+            last[r] = vals[(15 * M + 8 * warp + 2 * t4 + r) * 2 + 1];              // a_C, -, e^{i phi_C} of key r
+            al2[r] = t < a.T ? *reinterpret_cast<const float2 *>(a.alpha + row * M + 8 * warp + 2 * t4) : make_float2(1.f, 1.f);
+            be2[r] = t < a.T ? a.beta[row] : 0.f;
+        }
+    }
+    bar_sync(kBarGrad, kGrad);
 
     // the triangular factors of the corrections as A operands (t, i), a warp each:
     //   0: u_i . yb_t (i <= t)   1: u_i . b_t (i < t)   2: conj(u_t . yb_i) (i >= t)   3: -conj(u_t . b_i) (i > t)
@@ -452,7 +467,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         p[64] = make_uint4(h[0], h[1], h[2], h[3]);
         p[96] = make_uint4(l[0], l[1], l[2], l[3]);
     }
-    bar_sync(kBarAux, kAux);
+    bar_sync(kBarGrad, kGrad);
 
     if (warp < KT) {
         const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
@@ -512,17 +527,15 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         float al[4], dbp[2] = {0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int r = i >> 1, e = i & 1, tl = g + 8 * r, t = t0 + tl, key = 8 * warp + 2 * t4 + e;
-            const size_t row = row0 + (size_t)t * a.H;
-            const float4 x = vals[(tl * M + key) * 2], y = vals[(tl * M + key) * 2 + 1];
-            const float4 last = vals[(15 * M + key) * 2 + 1];                     // a_C, -, e^{i phi_C}
-            const float2 kp = make_float2(x.x, x.y), qp = make_float2(x.z, x.w), ph = make_float2(y.z, y.w), pc = make_float2(last.z, last.w);
-            const float be = t < a.T ? a.beta[row] : 0.f;
-            al[i] = t < a.T ? a.alpha[row * M + key] : 1.f;
+            const int r = i >> 1, e = i & 1, tl = g + 8 * r, key = 8 * warp + 2 * t4 + e;
+            const float4 x = vk[i], y = vp[i];
+            const float2 kp = make_float2(x.x, x.y), qp = make_float2(x.z, x.w), ph = make_float2(y.z, y.w), pc = make_float2(last[e].z, last[e].w);
+            const float be = be2[r];
+            al[i] = e ? al2[r].y : al2[r].x;
             const float2 x3 = cmulc(pc, make_float2(x3r[i], x3i[i]));
             float2 qb, zb, fb;
             if (fast) {
-                const float up = __fdividef(y.x, last.x), down = __frcp_rn(y.x);   // a_t / a_C, 1 / a_t: at most 2^16
+                const float up = __fdividef(y.x, last[e].x), down = __frcp_rn(y.x);   // a_t / a_C, 1 / a_t: at most 2^16
                 const float2 c1 = cmulc(pc, make_float2(z1r[i], z1i[i])), c2 = cmulc(pc, make_float2(z2r[i], z2i[i]));
                 qb = make_float2(fmaf(y.x, x1r[i], up * c1.x), fmaf(y.x, x1i[i], up * c1.y));
                 zb = make_float2(fmaf(y.x, x2r[i], up * c2.x), fmaf(y.x, x2i[i], up * c2.y));
@@ -568,7 +581,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         }
         float dal[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) dal[i] = __fdiv_rn(dd[i].x, al[i]);
+        for (int i = 0; i < 4; ++i) dal[i] = __fdividef(dd[i].x, al[i]);
         // small alpha: from the definition, one (token, key) at a time
         if (__any_sync(0xffffffffu, fminf(fminf(al[0], al[1]), fminf(al[2], al[3])) < 0.0625f)) {
 #pragma unroll 1
@@ -597,18 +610,10 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 const float4 q4 = make_float4(dqv[2 * r].x, dqv[2 * r].y, dqv[2 * r + 1].x, dqv[2 * r + 1].y);
                 const float4 k4 = make_float4(dkv[2 * r].x, dkv[2 * r].y, dkv[2 * r + 1].x, dkv[2 * r + 1].y);
                 const float2 a2 = make_float2(dal[2 * r], dal[2 * r + 1]), th2 = make_float2(dd[2 * r].y, dd[2 * r + 1].y);
-                if constexpr (NSL == 1) {
-                    st_val4(static_cast<T *>(a.dq) + ak, q4);
-                    st_val4(static_cast<T *>(a.dk) + ak, k4);
-                    *reinterpret_cast<float2 *>(a.dalpha + am) = a2;
-                    *reinterpret_cast<float2 *>(a.dtheta + am) = th2;
-                } else {
-                    const size_t off = (size_t)blockIdx.y * a.rows;
-                    st_val4(a.dq_p + off * DK + ak, q4);
-                    st_val4(a.dk_p + off * DK + ak, k4);
-                    *reinterpret_cast<float2 *>(a.dalpha_p + off * M + am) = a2;
-                    *reinterpret_cast<float2 *>(a.dtheta_p + off * M + am) = th2;
-                }
+                st_val4(static_cast<T *>(a.dq) + ak, q4);
+                st_val4(static_cast<T *>(a.dk) + ak, k4);
+                *reinterpret_cast<float2 *>(a.dalpha + am) = a2;
+                *reinterpret_cast<float2 *>(a.dtheta + am) = th2;
             }
             float x = dbp[r];
             x += __shfl_xor_sync(0xffffffffu, x, 1);
@@ -616,14 +621,13 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             if (t4 == 0) db[warp * 16 + g + 8 * r] = x;
         }
     }
-    bar_sync(kBarAux, kAux);
+    bar_sync(kBarGrad, kGrad);
     if (tid < 16 && t0 + tid < a.T) {
         float x = 0.f;
 #pragma unroll
         for (int w = 0; w < KT; ++w) x += db[w * 16 + tid];
         const size_t row = row0 + (size_t)(t0 + tid) * a.H;
-        if constexpr (NSL == 1) a.dbeta[row] = x;
-        else a.dbeta_p[(size_t)blockIdx.y * a.rows + row] = x;
+        a.dbeta[row] = x;
     }
 }
 
@@ -653,8 +657,304 @@ __device__ __forceinline__ void read_piece(const float4 *p, float (&x)[16])
     }
 }
 
+// The split state of a step of keys_product as the B operand (value channel, key) of the gradients' products
+__device__ __forceinline__ void publish_state(uint4 *p, int kk, const uint32_t (&rh)[4], const uint32_t (&rl)[4], const uint32_t (&ih)[4], const uint32_t (&il)[4])
+{
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        p[(4 * kk + 2 * e) * 32] = make_uint4(transpose8x8(rh[2 * e]), transpose8x8(rh[2 * e + 1]), transpose8x8(rl[2 * e]), transpose8x8(rl[2 * e + 1]));
+        p[(4 * kk + 2 * e + 1) * 32] = make_uint4(transpose8x8(ih[2 * e]), transpose8x8(ih[2 * e + 1]), transpose8x8(il[2 * e]), transpose8x8(il[2 * e + 1]));
+    }
+}
+
+// Where a chain warp leaves a chunk's operands for the gradients; ps = NULL: nowhere
+struct Publish {
+    uint4 *ps, *pt;           // the state's (offset by the lane), the [value x token] operand's
+    float *scale;             // two inverse scales
+};
+
+// forward through one chunk whose tile is at `slot` (shared memory): U = M (V - W^* S), S <- gamma_C S + Y U unless
+// `update` is false.  rr: the chunk's rows of v.  Returns the largest magnitude of S.
+template <int DK, int BARN>
+__device__ __forceinline__ float forward_step(uint32_t st, float big, unsigned char *slot, int bar, float (&rr)[2][4], const Publish &pub, bool update, int lane)
+{
+    using TL = Tile<DK>;
+    float isv;
+    const float sv = scale_for(warp_max(big), isv);
+    bar_sync(bar, BARN);
+    const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot);
+    const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
+    float acc[1][3][2][4], ri[2][4];
+    const uint32_t tiles[1] = {tile + TL::oW};
+    keys_product<DK, 1>(acc, st, sv, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+        if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il);
+    });
+    const float fw = isv * inv[0];
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
+            ri[n][i] = -fw * (acc[0][1][n][i] - acc[0][2][n][i]);
+        }
+    TokFrag fr;
+    {
+        TokFrag fb;
+        const float ir = make_frag(fr, rr, ri);
+        load_small<false>(fb, tile + TL::oM, lane);
+        product_small<false>(rr, ri, fr, fb, ir * inv[3]);
+    }
+    const float iu = make_frag(fr, rr, ri);
+    if (pub.ps) {
+        publish_frag(pub.pt, fr, lane);
+        if (lane == 0) {
+            pub.scale[0] = isv;
+            pub.scale[1] = iu;
+        }
+    }
+    return update ? state_update<DK>(st, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(slot + TL::oG), lane) : big;
+}
+
+// backward through one chunk: Bc = M^H (Y^* G + (A D_beta)^H Yb^*), G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc.  yr, yi: the
+// chunk's rows of Yb^* (yi only with has_im).  Leaves Re Bc (the rows of dv) in pr; returns the largest magnitude of G.
+template <int DK, bool kExact>
+__device__ __forceinline__ float backward_step(uint32_t sg, float big, unsigned char *slot, float (&yr)[2][4], float (&yi)[2][4], bool has_im,
+                                               float (&pr)[2][4], const Publish &pub, int lane)
+{
+    using TL = Tile<DK>;
+    const int t4 = lane & 3;
+    TokFrag fy;
+    const float iy = make_frag(fy, yr, yi);
+    const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot);
+    const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
+    float ig;
+    const float sv = scale_for(warp_max(big), ig);
+    float acc[1][3][2][4];
+    const uint32_t tiles[1] = {tile + TL::oY};
+    keys_product<DK, 1>(acc, sg, sv, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+        if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il);
+    });
+    float pi[2][4];
+    {
+        TokFrag fb;
+        load_small<true>(fb, tile + TL::oA, lane);
+        const float fg = ig * inv[1], fa = iy * inv[4];
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f}, ni[4] = {0.f, 0.f, 0.f, 0.f};
+            mma3x<kExact>(re, fy.rh, fy.rl, fb.rh[2 * n], fb.rh[2 * n + 1], fb.rl[2 * n], fb.rl[2 * n + 1]);
+            mma3x<kExact>(ni, fy.rh, fy.rl, fb.ih[2 * n], fb.ih[2 * n + 1], fb.il[2 * n], fb.il[2 * n + 1]);
+            if (has_im) {
+                mma3x<kExact>(re, fy.ih, fy.il, fb.ih[2 * n], fb.ih[2 * n + 1], fb.il[2 * n], fb.il[2 * n + 1]);
+                mma3x<kExact>(im, fy.ih, fy.il, fb.rh[2 * n], fb.rh[2 * n + 1], fb.rl[2 * n], fb.rl[2 * n + 1]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                pr[n][i] = fmaf(fa, re[i], fg * acc[0][0][n][i]);
+                pi[n][i] = fmaf(fa, im[i] - ni[i], fg * (acc[0][1][n][i] - acc[0][2][n][i]));
+            }
+        }
+    }
+    TokFrag fp;
+    {
+        TokFrag fb;
+        const float ip = make_frag(fp, pr, pi);
+        load_small<true>(fb, tile + TL::oM, lane);
+        product_small<true>(pr, pi, fp, fb, ip * inv[3]);
+    }
+    const float ib = make_frag(fp, pr, pi);
+    if (pub.ps) {
+        publish_frag(pub.pt, fp, lane);
+        if (lane == 0) {
+            pub.scale[0] = ig;
+            pub.scale[1] = ib;
+        }
+    }
+    const float fq = iy * inv[2], fw = -ib * inv[0];
+    const float4 *gamma = reinterpret_cast<const float4 *>(slot + TL::oG) + t4;
+    uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
+    uint32_t nih[4], nil[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        nih[i] = fp.ih[i] ^ 0x80008000u;
+        nil[i] = fp.il[i] ^ 0x80008000u;
+    }
+    big = 0.f;
+#pragma unroll 1
+    for (int np = 0; np < TL::KS; ++np, at += 32, gamma += 8) {
+        float x[16];
+        tm_load(x, sg + 16 * np);
+        uint32_t qh[4], ql[4], jh[4], jl[4];
+        ldsm_t(qh, at + TL::oQ);
+        ldsm_t(jh, at + TL::oQ + 2 * TL::PL);
+        ldsm_t(ql, at + TL::oQ + TL::PL);
+        ldsm_t(jl, at + TL::oQ + 3 * TL::PL);
+        float qr[2][4], qi[2][4];
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) qr[n][i] = qi[n][i] = 0.f;
+            mma3x<kExact>(qr[n], fy.rh, fy.rl, qh[2 * n], qh[2 * n + 1], ql[2 * n], ql[2 * n + 1]);
+            mma3x<kExact>(qi[n], fy.rh, fy.rl, jh[2 * n], jh[2 * n + 1], jl[2 * n], jl[2 * n + 1]);
+        }
+        if (has_im) {
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                float ni[4] = {0.f, 0.f, 0.f, 0.f};
+                mma3x<kExact>(ni, fy.ih, fy.il, jh[2 * n], jh[2 * n + 1], jl[2 * n], jl[2 * n + 1]);
+                mma3x<kExact>(qi[n], fy.ih, fy.il, qh[2 * n], qh[2 * n + 1], ql[2 * n], ql[2 * n + 1]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) qr[n][i] -= ni[i];
+            }
+        }
+        tm_wait_load(x);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const float4 gm = gamma[4 * n];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float cr = (i & 1) ? gm.z : gm.x, ci = (i & 1) ? gm.w : gm.y, u = x[8 * n + i], v = x[8 * n + 4 + i];
+                x[8 * n + i] = fmaf(fq, qr[n][i], cr * u + ci * v);
+                x[8 * n + 4 + i] = fmaf(fq, qi[n][i], cr * v - ci * u);
+            }
+        }
+        tokens_product<DK>(qr, qi, fp, nih, nil, at + TL::oW);
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                x[8 * n + i] = fmaf(fw, qr[n][i], x[8 * n + i]);
+                x[8 * n + 4 + i] = fmaf(fw, qi[n][i], x[8 * n + 4 + i]);
+                big = fmaxf(big, fmaxf(fabsf(x[8 * n + i]), fabsf(x[8 * n + 4 + i])));
+            }
+        tm_store(sg + 16 * np, x);
+    }
+    tm_wait_store();
+    return big;
+}
+
+// the rows of Yb^* of a chunk
+template <typename T>
+__device__ __forceinline__ void load_cotangents(float (&yr)[2][4], float (&yi)[2][4], const void *re, const void *im, size_t at, size_t step, int left)
+{
+    load_rows(yr, static_cast<const T *>(re) + at, step, left);
+    load_rows(yi, static_cast<const T *>(im) + at, step, im ? left : 0);
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) yi[n][i] = -yi[n][i];
+}
+
+// a chain warp's part of a kept state: [piece][4][lane] float4
+template <int DK>
+__device__ __forceinline__ float4 *kept(float *keep, int bh, int pitch, int s, int dv, int col0, int lane)
+{
+    return reinterpret_cast<float4 *>(keep + (((size_t)bh * pitch + s) * dv + col0) * DK) + lane;
+}
+
+// ---- few sequences: the two chains alone, side by side (blockIdx.z) -------------------------------------
+// With less than half as many sequences as SMs the walk of one CTA per sequence leaves the device idle.  But the
+// cotangent's chain needs neither S nor U: so S walks forward and G backward at the same time, each in blocks of value
+// columns (NB), both kept every 64 tokens; then every segment's gradients are a unit of their own (kUnits below).
 template <int DK, int DVT, int NB, typename T>
-__global__ void __launch_bounds__(kAux + kSolve + 2 * NB, 1) sfda_backward_kernel(const BwdArgsDev a)
+__global__ void __launch_bounds__(ChainRoles<NB>::threads, 1) sfda_backward_chain_kernel(const BwdArgsDev a)
+{
+    using TL = Tile<DK>;
+    using L = ChainSmem<DK, NB>;
+    constexpr int kChain = 2 * NB;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
+    const bool back = blockIdx.z != 0;
+    const size_t row0 = (size_t)b * a.T * a.H + h;
+    const int nch = (a.T + kC - 1) / kC;
+    if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::slow), L::columns);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::slow);
+    __syncthreads();
+
+    const ChainRoles<NB> role(tid);
+    if (role.prep >= 0) {
+        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+        const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
+        PrepRaw<L::PM::TPT, T> in;
+        prep_fetch<DK, kPrepWarps, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, (back ? nch - 1 : 0) * kC, a.T, back, role.prep);
+#pragma unroll 1
+        for (int c = 0; c < nch; ++c) {
+            const int slot = c % kSlots, at = back ? nch - 1 - c : c, nx = back ? max(at - 1, 0) : at + 1;
+            if (c >= kSlots) bar_sync(kBarDone + slot, kPrep + kChain);
+            PrepRaw<L::PM::TPT, T> next;
+            prep_fetch<DK, kPrepWarps, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, nx * kC, a.T, back, role.prep);
+            float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes);
+            if (!prep_planes<DK, kPrepWarps, kBarAux, T>(in, nullptr, smem + slot * TL::bytes, smem + L::kb + slot * TL::BIG, smem + L::scan, back, role.prep))
+                slow_gram<DK, kPrepWarps, kBarAux, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, at * kC, a.T, smem + L::slow, smem + L::scan,
+                                                      gk, gk + 16 * 17, back, role.prep);
+            bar_arrive(kBarPlanes + slot, kPrep + 64);
+            in = next;
+        }
+    } else if (role.solve >= 0) {
+        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        const int lane = tid & 31, w = role.solve >> 5, out = w >> 1;
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+#pragma unroll 1
+        for (int c = w & 1; c < nch; c += 2) {
+            const int slot = c % kSlots;
+            unsigned char *tile = smem + slot * TL::bytes;
+            float *inv = reinterpret_cast<float *>(tile + TL::oS);
+            float2 *gm = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes) + out * 16 * 17;
+            bar_sync(kBarPlanes + slot, kPrep + 64);
+            if (back || !out) {
+                if (reinterpret_cast<const int *>(inv)[6])
+                    gram_tiles<DK, 2>(base + slot * TL::bytes + (out ? TL::oQ : TL::oW), base + L::kb + slot * TL::BIG, inv[out ? 2 : 0] * inv[5], gm, 0, lane);
+                __syncwarp();
+                if (!out) invert_unit_lower16(gm, lane);
+                store_lower(tile + (out ? TL::oA : TL::oM), gm, inv + 3 + out, lane);
+            }
+            bar_arrive(kBarFull + slot, 64 + kChain);
+        }
+    } else if (role.chain >= 0) {
+        if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+        const int lane = tid & 31, w = role.chain >> 5, g = lane >> 2, t4 = lane & 3, col0 = c0 + 16 * w, col = col0 + g;
+        const uint32_t st = tmem + ((uint32_t)(w & 3) << 21) + (w >> 2) * 8 * TL::KT;
+        const size_t state_at = ((size_t)bh * DK + 4 * t4) * DVT + col, step = (size_t)a.H * DVT;
+        const Publish none = {nullptr, nullptr, nullptr};
+        const float *from = back ? a.dS_T : a.S0;
+        float big = state_from_memory<DK>(st, from ? from + state_at : nullptr, DVT);
+#pragma unroll 1
+        for (int c = 0; c < nch; ++c) {
+            const int slot = c % kSlots, cc = back ? nch - 1 - c : c, left = a.T - cc * kC - 2 * t4;
+            unsigned char *tile = smem + slot * TL::bytes;
+            const size_t at = (row0 + (size_t)(cc * kC + 2 * t4) * a.H) * DVT + col;
+            if (!back) {
+                if (cc % kSegChunks == 0) keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, cc / kSegChunks, DVT, col0, lane), st);
+                float rr[2][4];
+                load_rows(rr, static_cast<const T *>(a.v) + at, step, left);
+                big = forward_step<DK, 64 + kChain>(st, big, tile, kBarFull + slot, rr, none, true, lane);
+            } else {
+                if (c == 0 || cc % kSegChunks == kSegChunks - 1) keep_state<DK>(kept<DK>(a.keep_g, bh, a.pitch, cc / kSegChunks, DVT, col0, lane), st);
+                float yr[2][4], yi[2][4], pr[2][4];
+                load_cotangents<T>(yr, yi, a.d_o, a.d_o_im, at, step, left);
+                bar_sync(kBarFull + slot, 64 + kChain);
+                big = backward_step<DK, sizeof(T) == 2>(st, big, tile, yr, yi, a.d_o_im != nullptr, pr, none, lane);
+            }
+            if (c + kSlots < nch) bar_arrive(kBarDone + slot, kPrep + kChain);
+        }
+        if (back) state_to_memory<DK>(st, a.dS0 + state_at, DVT);
+        else keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, a.NS, DVT, col0, lane), st);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid < 32) tm_free(tmem, L::columns);
+}
+
+// ---- the walk with gradients ------------------------------------------------------------------------------
+// kUnits == false: one CTA per pair walks the sequence forward (keeping S), then its segments last to first.
+// kUnits == true: S and G are kept already; a CTA takes units (pair, segment) blockIdx.x, + gridDim.x, ...
+// Either way the second sweep is a list of segments, each of kSegChunks chunks (a ragged last one is completed with
+// neutral tokens), pipelined over its borders.
+template <int DK, int NB, typename T, bool kUnits>
+__global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kernel(const BwdArgsDev a)
 {
     using TL = Tile<DK>;
     using L = BwdSmem<DK, NB>;
@@ -662,118 +962,128 @@ __global__ void __launch_bounds__(kAux + kSolve + 2 * NB, 1) sfda_backward_kerne
     constexpr int kChain = 2 * NB, NCW = NB / 16, M = DK / 2, KT = TL::KT;
     constexpr bool kExact = sizeof(T) == 2;
     extern __shared__ __align__(128) unsigned char smem[];
-    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
-    const size_t row0 = (size_t)b * a.T * a.H + h;                       // row of token t: row0 + t H
-    const int nch = (a.T + kC - 1) / kC, NS = a.NS;
-    unsigned char *ring = reinterpret_cast<unsigned char *>(a.scratch + ((size_t)bh * DVT + c0) * kSeg * DK);
+    const int tid = threadIdx.x, NS = a.NS, nch = (a.T + kC - 1) / kC;
+    unsigned char *ring = a.ring + blockIdx.x * a.ring_bytes;
     float2 *rgs = reinterpret_cast<float2 *>(ring + SC::oRg);
-    const int last_nch = nch - (NS - 1) * kSegChunks;                    // chunks of the last segment
-    // position n of the second sweep (segments last to first): segment from the end, place in it, its chunks
-    auto segment_of = [&](int n, int &r, int &at, int &nc) {
-        r = n < last_nch ? 0 : 1 + (n - last_nch) / kSegChunks;
-        at = r == 0 ? n : (n - last_nch) % kSegChunks;
-        nc = r == 0 ? last_nch : kSegChunks;
+    const int segments = kUnits ? (a.units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : NS;
+    // the r-th segment of this CTA's list: pair and segment; row of token t of a pair: row0 + t H
+    auto segment = [&](int r, int &bh, int &s) {
+        if constexpr (kUnits) {
+            const int u = blockIdx.x + r * gridDim.x;
+            bh = u / NS;
+            s = u - bh * NS;
+        } else {
+            bh = blockIdx.x;
+            s = NS - 1 - r;
+        }
     };
+    auto row_of = [&](int bh) { return (size_t)(bh / a.H) * a.T * a.H + bh % a.H; };
     if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::word), L::columns);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::word);
 
-    if (tid < kAux) {
-        // register shares with all 128 value columns: 256 x 112 + 128 x 56 + 256 x 100 rounded to 8: 112, 56, 96 of 640 x 96
-        if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
-        const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
-        // Chunks are prepared in the order the chain goes forward through them (second sweep: last segment first) and
-        // their gradients follow in the order it comes back; the p-th chunk prepared takes the slot of gradient p - 4.
+    // register shares: 256 x (96 + 56 + 88) of 768 x 80 with 128 value columns; 256 x (112 + 72) + 128 x 112 of 640 x 96
+    // with 64
+    if (tid < kGrad) {
+        if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
+        if constexpr (NB == 64) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
         float2 carry[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        int made = 0;
 #pragma unroll 1
-        for (int sweep = 0; sweep < 2; ++sweep) {
-#pragma unroll 1
-            for (int p = 0; p < nch + kSlots; ++p) {
-                int r, at, nc;
-                const int n = p - kSlots;
-                if (n >= 0 && n < nch) {
-                    segment_of(n, r, at, nc);
-                    const int c = nc - 1 - at, slot = sweep ? ring_slot(r, c) : n % kSlots;
-                    bar_sync(kBarDone + slot, kAux + kChain);
-                    if (sweep)
-                        chunk_gradients<DK, DVT, NB, T>(a, smem, ring + (size_t)slot * SC::slot, rgs + (r & 1) * NCW * M, slot, at == 0,
-                                                        (NS - 1 - r) * kSeg + c * kC, row0, carry, tid);
-                }
-                if (p < nch) {
-                    segment_of(p, r, at, nc);
-                    const int slot = sweep ? ring_slot(r, at) : p % kSlots, t0 = sweep ? (NS - 1 - r) * kSeg + at * kC : p * kC;
-                    const bool needq = sweep;
-                    PrepRaw<L::PM::TPT, T> in;
-                    prep_fetch<DK, kAuxWarps, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, needq, tid);
-                    if (made >= 2) bar_sync(kBarSolved + (made & 1), kAux + 64);
-                    float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + (made & 1) * L::gram_bytes);
-                    float4 *vals = sweep ? reinterpret_cast<float4 *>(ring + (size_t)slot * SC::slot + SC::oV) : nullptr;
-                    if (!prep_planes<DK, kAuxWarps, T>(in, vals, smem + slot * TL::bytes, smem + L::kb + (made & 1) * TL::BIG, smem + L::uy, needq, tid))
-                        slow_gram<DK, kAuxWarps, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, smem + L::frag, smem + L::uy, gk,
-                                                    gk + 16 * 17, needq, tid);
-                    bar_arrive(kBarPlanes + (made & 3), kAux + 64);
-                    ++made;
-                }
-            }
+        for (int n = 0; n < segments * kSegChunks; ++n) {
+            const int r = n / kSegChunks, at = n % kSegChunks, c = kSegChunks - 1 - at, slot = ring_slot(r, c);
+            int bh, s;
+            segment(r, bh, s);
+            bar_sync(kBarDone + slot, kGrad + kChain);
+            chunk_gradients<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, rgs + (r & 1) * NCW * M, slot, at == 0,
+                                       s * kSeg + c * kC, row_of(bh), carry, tid);
+            if (r + 1 < segments) bar_arrive(kBarFree + slot, kGrad + kPrep);
         }
-    } else if (tid < kAux + kSolve) {
-        // warps 0, 1: the system's inverse of every other chunk; warps 2, 3: the outputs' Gram matrix of them
+    } else if (tid < kGrad + kPrep) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        const int lane = tid & 31, w = (tid - kAux) >> 5, out = w >> 1;
+        if constexpr (NB == 64) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
+        const int ptid = tid - kGrad, lane = tid & 31, w = ptid >> 5;
         const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+        float2 *gram = reinterpret_cast<float2 *>(smem + L::gram);
+        // Chunks are prepared in the order the chain goes forward through them; a slot is prepared again when the chain
+        // (first sweep) or the gradients (second sweep) are through with it.
 #pragma unroll 1
-        for (int j = w & 1; j < 2 * nch; j += 2) {
-            const bool second = j >= nch;
-            int r, at, nc;
-            segment_of(j - nch, r, at, nc);
-            const int slot = second ? ring_slot(r, at) : j % kSlots;
-            unsigned char *tile = smem + slot * TL::bytes;
-            float *inv = reinterpret_cast<float *>(tile + TL::oS);
-            float2 *gm = reinterpret_cast<float2 *>(smem + L::gram + (j & 1) * L::gram_bytes) + out * 16 * 17;
-            bar_sync(kBarPlanes + (j & 3), kAux + 64);
-            if (second || !out) {
-                if (reinterpret_cast<const int *>(inv)[6])
-                    gram_tiles<DK, 2>(base + slot * TL::bytes + (out ? TL::oQ : TL::oW), base + L::kb + (j & 1) * TL::BIG, inv[out ? 2 : 0] * inv[5], gm, 0, lane);
-                __syncwarp();
-                if (!out) invert_unit_lower16(gm, lane);
-                store_lower(tile + (out ? TL::oA : TL::oM), gm, inv + 3 + out, lane);
+        for (int sweep = kUnits ? 1 : 0; sweep < 2; ++sweep) {
+            const int np = sweep ? segments * kSegChunks : nch;
+#pragma unroll 1
+            for (int p = 0; p < np + (sweep ? 0 : kSlots); ++p) {
+                const int r = p / kSegChunks, at = p % kSegChunks, slot = sweep ? ring_slot(r, at) : at;
+                if (p >= kSlots && p - kSlots < np) bar_sync(kBarFree + slot, (sweep ? kGrad : kChain) + kPrep);
+                if (p >= np) continue;
+                int bh, s;
+                segment(sweep ? r : 0, bh, s);
+                const size_t row0 = row_of(bh);
+                const int t0 = sweep ? s * kSeg + at * kC : p * kC;
+                const bool needq = sweep;
+                unsigned char *tile = smem + slot * TL::bytes;
+                float *inv = reinterpret_cast<float *>(tile + TL::oS);
+                PrepRaw<L::PM::TPT, T> in;
+                prep_fetch<DK, kPrepWarps, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, needq, ptid);
+                float4 *vals = sweep ? reinterpret_cast<float4 *>(ring + (size_t)slot * SC::slot + SC::oV) : nullptr;
+                const bool fast = prep_planes<DK, kPrepWarps, kBarPrep, T>(in, vals, tile, smem + L::kb, smem + L::scan, needq, ptid);
+                if (!fast)
+                    slow_gram<DK, kPrepWarps, kBarPrep, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, ring + SC::oSlow,
+                                                           smem + L::scan, gram, gram + 16 * 17, needq, ptid);
+                bar_sync(kBarPrep, kPrep);
+                if (w == 0 || (needq && w == 1)) {               // the system's inverse; the outputs' Gram matrix
+                    float2 *gm = gram + w * 16 * 17;
+                    if (fast)
+                        gram_tiles<DK, 2>(base + slot * TL::bytes + (w ? TL::oQ : TL::oW), base + L::kb, inv[w ? 2 : 0] * inv[5], gm, 0, lane);
+                    __syncwarp();
+                    if (!w) invert_unit_lower16(gm, lane);
+                    store_lower(tile + (w ? TL::oA : TL::oM), gm, inv + 3 + w, lane);
+                }
+                bar_arrive(kBarFull + slot, kPrep + kChain);
             }
-            bar_arrive(kBarFull + slot, 64 + kChain);
-            if (j + 2 < 2 * nch) bar_arrive(kBarSolved + (j & 1), kAux + 64);
         }
     } else {
-        const int lane = tid & 31, w = (tid - kAux - kSolve) >> 5, g = lane >> 2, t4 = lane & 3;
-        const int col = c0 + 16 * w + g;                                 // and col + 8
-        const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+        if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
+        if constexpr (NB == 64) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+        const int lane = tid & 31, w = (tid - kGrad - kPrep) >> 5, g = lane >> 2, t4 = lane & 3;
+        const int col = 16 * w + g;                                      // and col + 8
         const uint32_t ss = tmem + ((uint32_t)(w & 3) << 21) + (w >> 2) * 16 * KT, sg = ss + 8 * KT;   // S and G
         float *scal = reinterpret_cast<float *>(smem + L::scal);
-        const size_t step = (size_t)a.H * DVT, state_at = ((size_t)bh * DK + 4 * t4) * DVT + col;
-        auto checkpoint = [&](int s) {                                   // s = NS: the final state
-            float *p = s < NS ? a.check + (((size_t)bh * NS + s) * DVT + c0 + 16 * w) * DK : reinterpret_cast<float *>(ring + SC::oEnd) + 16 * w * DK;
-            return reinterpret_cast<float4 *>(p) + lane;
-        };
-        float big_s = state_from_memory<DK>(ss, a.S0 ? a.S0 + state_at : nullptr, DVT), big_g = 0.f;
+        const size_t step = (size_t)a.H * NB;
+        float big_s = 0.f, big_g = 0.f;
 #pragma unroll 1
-        for (int r = -1; r < NS; ++r) {                                  // -1: the first sweep over the whole sequence
-            const int s = NS - 1 - r, nc = r < 0 ? nch : r == 0 ? last_nch : kSegChunks;
-            if (r >= 0) {
-                if (r == 0) {
-                    keep_state<DK>(checkpoint(NS), ss);
-                    big_g = state_from_memory<DK>(sg, a.dS_T ? a.dS_T + state_at : nullptr, DVT);
+        for (int r = kUnits ? 0 : -1; r < segments; ++r) {               // -1: the first sweep over the whole sequence
+            int bh, s;
+            segment(max(r, 0), bh, s);
+            const size_t state_at = ((size_t)bh * DK + 4 * t4) * NB + col, row0 = row_of(bh);
+            if (r < 0) {
+                big_s = state_from_memory<DK>(ss, a.S0 ? a.S0 + state_at : nullptr, NB);
+            } else {
+                if (!kUnits && r == 0) {
+                    keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), ss);
+                    big_g = state_from_memory<DK>(sg, a.dS_T ? a.dS_T + state_at : nullptr, NB);
                 }
                 // rowdot(conj S, G) at the segment's end, this warp's columns; then S at its start
                 float2 *rg = rgs + ((r & 1) * NCW + w) * M + 2 * t4;
-                const float4 *end = checkpoint(s + 1), *start = checkpoint(s);
+                const float4 *end = kept<DK>(a.keep_s, bh, a.pitch, s + 1, NB, 16 * w, lane), *start = kept<DK>(a.keep_s, bh, a.pitch, s, NB, 16 * w, lane);
+                const float4 *kg = kept<DK>(a.keep_g, bh, a.pitch, s, NB, 16 * w, lane);
                 big_s = 0.f;
+                if (kUnits) big_g = 0.f;
 #pragma unroll 1
-                for (int n = 0; n < TL::KS; ++n, rg += 16, end += 128, start += 128) {
+                for (int n = 0; n < TL::KS; ++n, rg += 16, end += 128, start += 128, kg += 128) {
                     float x[16], y[16];
-                    tm_load(x, sg + 16 * n);
-                    read_piece(end, y);
-                    tm_wait_load(x);
+                    if constexpr (kUnits) {
+                        read_piece(kg, x);
+                        tm_store(sg + 16 * n, x);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) big_g = fmaxf(big_g, fabsf(x[i]));
+                        read_piece(end, y);
+                    } else {
+                        tm_load(x, sg + 16 * n);
+                        read_piece(end, y);
+                        tm_wait_load(x);
+                    }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {                        // (tile, key)
                         const int o = 8 * (u >> 1) + (u & 1);
@@ -793,243 +1103,41 @@ __global__ void __launch_bounds__(kAux + kSolve + 2 * NB, 1) sfda_backward_kerne
                 }
                 tm_wait_store();
             }
-            // forward: U = M (V - W^* S), S <- gamma_C S + Y U; the second sweep leaves S and U for the gradients
 #pragma unroll 1
-            for (int c = 0; c < nc; ++c) {
+            for (int c = 0; c < (r < 0 ? nch : kSegChunks); ++c) {
                 const int slot = r < 0 ? c % kSlots : ring_slot(r, c), t0 = (r < 0 ? 0 : s * kSeg) + c * kC;
-                const bool pub = r >= 0;
-                if (!pub && c % kSegChunks == 0) keep_state<DK>(checkpoint(c / kSegChunks), ss);
+                if (r < 0 && c % kSegChunks == 0) keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, c / kSegChunks, NB, 16 * w, lane), ss);
                 unsigned char *scr = ring + (size_t)slot * SC::slot;
-                uint4 *ps = reinterpret_cast<uint4 *>(scr + SC::oS) + w * KT * 64 + lane;
-                float rr[2][4], ri[2][4];
-                load_rows(rr, static_cast<const T *>(a.v) + (row0 + (size_t)(t0 + 2 * t4) * a.H) * DVT + col, step, a.T - t0 - 2 * t4);
-                float isv;
-                const float sv = scale_for(warp_max(big_s), isv);
-                bar_sync(kBarFull + slot, 64 + kChain);
-                const uint32_t tile = base + slot * TL::bytes;
-                const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
-                float acc[1][3][2][4];
-                const uint32_t tiles[1] = {tile + TL::oW};
-                keys_product<DK, 1>(acc, ss, sv, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
-                    if (pub) {
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            ps[(4 * kk + 2 * e) * 32] = make_uint4(transpose8x8(rh[2 * e]), transpose8x8(rh[2 * e + 1]), transpose8x8(rl[2 * e]), transpose8x8(rl[2 * e + 1]));
-                            ps[(4 * kk + 2 * e + 1) * 32] = make_uint4(transpose8x8(ih[2 * e]), transpose8x8(ih[2 * e + 1]), transpose8x8(il[2 * e]), transpose8x8(il[2 * e + 1]));
-                        }
-                    }
-                });
-                const float fw = isv * inv[0];
-#pragma unroll
-                for (int n = 0; n < 2; ++n)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
-                        ri[n][i] = -fw * (acc[0][1][n][i] - acc[0][2][n][i]);
-                    }
-                TokFrag fr;
-                {
-                    TokFrag fb;
-                    const float ir = make_frag(fr, rr, ri);
-                    load_small<false>(fb, tile + TL::oM, lane);
-                    product_small<false>(rr, ri, fr, fb, ir * inv[3]);
-                }
-                const float iu = make_frag(fr, rr, ri);
-                if (pub) {
-                    publish_frag(reinterpret_cast<uint4 *>(scr + SC::oU) + w * 128, fr, lane);
-                    if (lane == 0) {
-                        scal[(slot * NCW + w) * 4] = isv;
-                        scal[(slot * NCW + w) * 4 + 1] = iu;
-                    }
-                }
-                if (!pub || c + 1 < nc)
-                    big_s = state_update<DK>(ss, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
-                if (!pub) bar_arrive(kBarDone + slot, kAux + kChain);
+                Publish pub = {nullptr, nullptr, nullptr};
+                if (r >= 0) pub = {reinterpret_cast<uint4 *>(scr + SC::oS) + w * KT * 64 + lane, reinterpret_cast<uint4 *>(scr + SC::oU) + w * 128, scal + (slot * NCW + w) * 4};
+                float rr[2][4];
+                load_rows(rr, static_cast<const T *>(a.v) + (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col, step, a.T - t0 - 2 * t4);
+                big_s = forward_step<DK, kPrep + kChain>(ss, big_s, smem + slot * TL::bytes, kBarFull + slot, rr, pub, r < 0 || c + 1 < kSegChunks, lane);
+                if (r < 0) bar_arrive(kBarFree + slot, kPrep + kChain);
             }
             if (r < 0) continue;
 #pragma unroll 1
-            for (int c = nc - 1; c >= 0; --c) {
+            for (int c = kSegChunks - 1; c >= 0; --c) {
                 const int slot = ring_slot(r, c), t0 = s * kSeg + c * kC, left = a.T - t0 - 2 * t4;
-                const size_t at0 = (row0 + (size_t)(t0 + 2 * t4) * a.H) * DVT + col;
+                const size_t at = (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col;
                 unsigned char *scr = ring + (size_t)slot * SC::slot;
-                uint4 *ps = reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64 + lane;
-                const bool has_im = a.d_o_im != nullptr;
-                TokFrag fy;                                              // Yb^*
-                float iy;
-                {
-                    float yr[2][4], yi[2][4];
-                    load_rows(yr, static_cast<const T *>(a.d_o) + at0, step, left);
-                    load_rows(yi, static_cast<const T *>(a.d_o_im) + at0, step, has_im ? left : 0);
-#pragma unroll
-                    for (int n = 0; n < 2; ++n)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) yi[n][i] = -yi[n][i];
-                    iy = make_frag(fy, yr, yi);
-                }
-                const uint32_t tile = base + slot * TL::bytes;
-                const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
-                float ig;
-                const float sv = scale_for(warp_max(big_g), ig);
-                float acc[1][3][2][4];
-                const uint32_t tiles[1] = {tile + TL::oY};
-                keys_product<DK, 1>(acc, sg, sv, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        ps[(4 * kk + 2 * e) * 32] = make_uint4(transpose8x8(rh[2 * e]), transpose8x8(rh[2 * e + 1]), transpose8x8(rl[2 * e]), transpose8x8(rl[2 * e + 1]));
-                        ps[(4 * kk + 2 * e + 1) * 32] = make_uint4(transpose8x8(ih[2 * e]), transpose8x8(ih[2 * e + 1]), transpose8x8(il[2 * e]), transpose8x8(il[2 * e + 1]));
-                    }
-                });
-                float pr[2][4], pi[2][4];
-                {                                                        // + (A D_beta)^H Yb^*
-                    TokFrag fb;
-                    load_small<true>(fb, tile + TL::oA, lane);
-                    const float fg = ig * inv[1], fa = iy * inv[4];
-#pragma unroll
-                    for (int n = 0; n < 2; ++n) {
-                        float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f}, ni[4] = {0.f, 0.f, 0.f, 0.f};
-                        mma3x<kExact>(re, fy.rh, fy.rl, fb.rh[2 * n], fb.rh[2 * n + 1], fb.rl[2 * n], fb.rl[2 * n + 1]);
-                        mma3x<kExact>(ni, fy.rh, fy.rl, fb.ih[2 * n], fb.ih[2 * n + 1], fb.il[2 * n], fb.il[2 * n + 1]);
-                        if (has_im) {
-                            mma3x<kExact>(re, fy.ih, fy.il, fb.ih[2 * n], fb.ih[2 * n + 1], fb.il[2 * n], fb.il[2 * n + 1]);
-                            mma3x<kExact>(im, fy.ih, fy.il, fb.rh[2 * n], fb.rh[2 * n + 1], fb.rl[2 * n], fb.rl[2 * n + 1]);
-                        }
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            pr[n][i] = fmaf(fa, re[i], fg * acc[0][0][n][i]);
-                            pi[n][i] = fmaf(fa, im[i] - ni[i], fg * (acc[0][1][n][i] - acc[0][2][n][i]));
-                        }
-                    }
-                }
-                TokFrag fp;
-                {
-                    TokFrag fb;
-                    const float ip = make_frag(fp, pr, pi);
-                    load_small<true>(fb, tile + TL::oM, lane);
-                    product_small<true>(pr, pi, fp, fb, ip * inv[3]);
-                }
-                store_rows(static_cast<T *>(a.dv) + at0, pr, step, left);
-                const float ib = make_frag(fp, pr, pi);
-                publish_frag(reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, fp, lane);
-                if (lane == 0) {
-                    scal[(slot * NCW + w) * 4 + 2] = ig;
-                    scal[(slot * NCW + w) * 4 + 3] = ib;
-                }
-                // G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc
-                const float fq = iy * inv[2], fw = -ib * inv[0];
-                const float4 *gamma = reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG) + t4;
-                uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
-                uint32_t nih[4], nil[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    nih[i] = fp.ih[i] ^ 0x80008000u;
-                    nil[i] = fp.il[i] ^ 0x80008000u;
-                }
-                big_g = 0.f;
-#pragma unroll 1
-                for (int np = 0; np < TL::KS; ++np, at += 32, gamma += 8) {
-                    float x[16];
-                    tm_load(x, sg + 16 * np);
-                    uint32_t qh[4], ql[4], jh[4], jl[4];
-                    ldsm_t(qh, at + TL::oQ);
-                    ldsm_t(jh, at + TL::oQ + 2 * TL::PL);
-                    ldsm_t(ql, at + TL::oQ + TL::PL);
-                    ldsm_t(jl, at + TL::oQ + 3 * TL::PL);
-                    float qr[2][4], qi[2][4];
-#pragma unroll
-                    for (int n = 0; n < 2; ++n) {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) qr[n][i] = qi[n][i] = 0.f;
-                        mma3x<kExact>(qr[n], fy.rh, fy.rl, qh[2 * n], qh[2 * n + 1], ql[2 * n], ql[2 * n + 1]);
-                        mma3x<kExact>(qi[n], fy.rh, fy.rl, jh[2 * n], jh[2 * n + 1], jl[2 * n], jl[2 * n + 1]);
-                    }
-                    if (has_im) {
-#pragma unroll
-                        for (int n = 0; n < 2; ++n) {
-                            float ni[4] = {0.f, 0.f, 0.f, 0.f};
-                            mma3x<kExact>(ni, fy.ih, fy.il, jh[2 * n], jh[2 * n + 1], jl[2 * n], jl[2 * n + 1]);
-                            mma3x<kExact>(qi[n], fy.ih, fy.il, qh[2 * n], qh[2 * n + 1], ql[2 * n], ql[2 * n + 1]);
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) qr[n][i] -= ni[i];
-                        }
-                    }
-                    tm_wait_load(x);
-#pragma unroll
-                    for (int n = 0; n < 2; ++n) {
-                        const float4 gm = gamma[4 * n];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float cr = (i & 1) ? gm.z : gm.x, ci = (i & 1) ? gm.w : gm.y, u = x[8 * n + i], v = x[8 * n + 4 + i];
-                            x[8 * n + i] = fmaf(fq, qr[n][i], cr * u + ci * v);
-                            x[8 * n + 4 + i] = fmaf(fq, qi[n][i], cr * v - ci * u);
-                        }
-                    }
-                    tokens_product<DK>(qr, qi, fp, nih, nil, at + TL::oW);
-#pragma unroll
-                    for (int n = 0; n < 2; ++n)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            x[8 * n + i] = fmaf(fw, qr[n][i], x[8 * n + i]);
-                            x[8 * n + 4 + i] = fmaf(fw, qi[n][i], x[8 * n + 4 + i]);
-                            big_g = fmaxf(big_g, fmaxf(fabsf(x[8 * n + i]), fabsf(x[8 * n + 4 + i])));
-                        }
-                    tm_store(sg + 16 * np, x);
-                }
-                tm_wait_store();
-                bar_arrive(kBarDone + slot, kAux + kChain);
+                const Publish pub = {reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64 + lane, reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, scal + (slot * NCW + w) * 4 + 2};
+                float yr[2][4], yi[2][4], pr[2][4];
+                load_cotangents<T>(yr, yi, a.d_o, a.d_o_im, at, step, left);
+                big_g = backward_step<DK, kExact>(sg, big_g, smem + slot * TL::bytes, yr, yi, a.d_o_im != nullptr, pr, pub, lane);
+                store_rows(static_cast<T *>(a.dv) + at, pr, step, left);
+                bar_arrive(kBarDone + slot, kGrad + kChain);
             }
+            if (!kUnits && r + 1 == segments) state_to_memory<DK>(sg, a.dS0 + state_at, NB);
         }
-        state_to_memory<DK>(sg, a.dS0 + state_at, DVT);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (tid < 32) tm_free(tmem, L::columns);
 }
 
-// ---- the sums over the column blocks: out[i] = share_0[i] + share_1[i] + ... in that order, one thread per four
-// consecutive elements.  HBM-bound and small beside the sweeps.
-constexpr int kSumThreads = 256;
-
-template <int NSL, typename T>
-__global__ void __launch_bounds__(kSumThreads)
-sfda_backward_sum_kernel(const float *__restrict__ dq_p, const float *__restrict__ dk_p, const float *__restrict__ dal_p,
-                         const float *__restrict__ dth_p, const float *__restrict__ dbe_p, T *__restrict__ dq,
-                         T *__restrict__ dk, float *__restrict__ dalpha, float *__restrict__ dtheta,
-                         float *__restrict__ dbeta, size_t n_key, size_t n_coord, size_t rows)
-{
-    // work items in float4 units: [dq | dk | dalpha | dtheta] then dbeta one by one
-    const size_t q4 = n_key / 4, c4 = n_coord / 4, total = 2 * q4 + 2 * c4 + rows;
-    for (size_t i = (size_t)blockIdx.x * kSumThreads + threadIdx.x; i < total; i += (size_t)gridDim.x * kSumThreads) {
-        if (i < 2 * q4 + 2 * c4) {
-            const float *src;
-            size_t n, at;
-            int which;
-            if (i < q4) { src = dq_p; n = n_key; at = i; which = 0; }
-            else if (i < 2 * q4) { src = dk_p; n = n_key; at = i - q4; which = 1; }
-            else if (i < 2 * q4 + c4) { src = dal_p; n = n_coord; at = i - 2 * q4; which = 2; }
-            else { src = dth_p; n = n_coord; at = i - 2 * q4 - c4; which = 3; }
-            float4 acc = *reinterpret_cast<const float4 *>(src + 4 * at);
-#pragma unroll
-            for (int sl = 1; sl < NSL; ++sl) {
-                const float4 x = *reinterpret_cast<const float4 *>(src + (size_t)sl * n + 4 * at);
-                acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
-            }
-            if (which >= 2) {
-                *reinterpret_cast<float4 *>((which == 2 ? dalpha : dtheta) + 4 * at) = acc;
-            } else {
-                st_val4((which == 0 ? dq : dk) + 4 * at, acc);
-            }
-        } else {
-            const size_t at = i - 2 * q4 - 2 * c4;
-            float acc = dbe_p[at];
-#pragma unroll
-            for (int sl = 1; sl < NSL; ++sl) acc += dbe_p[(size_t)sl * rows + at];
-            dbeta[at] = acc;
-        }
-    }
-}
-
-// Value columns per CTA: all of them while the (batch, head) pairs alone fill the SMs; halved (down to 32) while the
-// grid still fits the SMs of a B200, so that few sequences use the whole device.  (A fixed count rather than the
+// Blocks of value columns of the two chains: all of them while the (batch, head) pairs alone fill the SMs (then there is
+// only the walk with gradients, one CTA per pair); with few sequences 64 or 32.  (A fixed count rather than the
 // device's: the workspace size must not depend on where it is asked for.)
 constexpr int kBwdTargetCtas = 148;
 
@@ -1040,80 +1148,79 @@ int bwd_cols(int B, int H, int d_v)
     return cols;
 }
 
-// workspace: checkpoints, the S_{t-1} of one segment, then (more than one column block only) the blocks' shares of
-// dq, dk, dalpha, dtheta, dbeta
-struct BwdWorkspace {
-    size_t check, scratch, dq, dk, dalpha, dtheta, dbeta, total;   // offsets and size in floats
-};
-
-BwdWorkspace bwd_workspace(int B, int T, int H, int d_k, int d_v)
+// Workspace in floats: with many sequences the kept states (one per segment of 64 tokens and pair) and 64 states per
+// pair, which hold a CTA's ring and the final state.  With few sequences as much again and 3 d_k + 1 floats per row and
+// block of columns: room for both chains' kept states and one ring for as many CTAs as fit (never less than one).
+size_t bwd_workspace(int B, int T, int H, int d_k, int d_v)
 {
     const size_t bhn = (size_t)B * H, ns = (size_t)(T + kSeg - 1) / kSeg, state = (size_t)d_k * d_v;
     const size_t rows = bhn * T, nsl = (size_t)(d_v / bwd_cols(B, H, d_v)), shares = nsl > 1 ? nsl * rows : 0;
-    BwdWorkspace w;
-    w.check = 0;
-    w.scratch = w.check + bhn * ns * state;
-    w.dq = w.scratch + bhn * kSeg * state;
-    w.dk = w.dq + shares * d_k;
-    w.dalpha = w.dk + shares * d_k;
-    w.dtheta = w.dalpha + shares * (d_k / 2);
-    w.dbeta = w.dtheta + shares * (d_k / 2);
-    w.total = w.dbeta + ((shares + 3) & ~(size_t)3);
-    return w;
+    return bhn * (ns + kSeg) * state + shares * 3 * d_k + ((shares + 3) & ~(size_t)3);
 }
 
-template <int DK, int DVT, int DV, typename T>
-cudaError_t launch_cols(const BackwardArgs &x, void *workspace, cudaStream_t stream, int *launches)
+template <int DK, int DV, typename T, bool kUnits>
+cudaError_t launch_walk(const BwdArgsDev &a, int grid, cudaStream_t stream, int *launches)
 {
-    using L = BwdSmem<DK, DV>;
-    constexpr int NSL = DVT / DV;
-    auto kern = sfda_backward_kernel<DK, DVT, DV, T>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
+    auto kern = sfda_backward_kernel<DK, DV, T, kUnits>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BwdSmem<DK, DV>::bytes);
     if (e != cudaSuccess) return e;
-    const BwdWorkspace w = bwd_workspace(x.B, x.T, x.H, DK, DVT);
+    kern<<<grid, kGrad + kPrep + 2 * DV, BwdSmem<DK, DV>::bytes, stream>>>(a);
+    if (launches) ++*launches;
+    return cudaGetLastError();
+}
+
+template <int DK, int DV, int NB, typename T>
+cudaError_t launch_chains(const BwdArgsDev &a, int pairs, cudaStream_t stream, int *launches)
+{
+    auto kern = sfda_backward_chain_kernel<DK, DV, NB, T>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainSmem<DK, NB>::bytes);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3((unsigned)pairs, DV / NB, 2), ChainRoles<NB>::threads, ChainSmem<DK, NB>::bytes, stream>>>(a);
+    if (launches) ++*launches;
+    return cudaGetLastError();
+}
+
+template <int DK, int DV, typename T>
+cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t stream, int *launches)
+{
+    using SC = BwdScratch<DK, DV>;
+    const size_t state = (size_t)DK * DV;
+    const int pairs = x.B * x.H, cols = bwd_cols(x.B, x.H, DV);
     float *ws = static_cast<float *>(workspace);
     BwdArgsDev a;
     a.q = x.q; a.k = x.k; a.v = x.v; a.d_o = x.d_o; a.d_o_im = x.d_o_im;
     a.alpha = x.alpha; a.theta = x.theta; a.beta = x.beta; a.S0 = x.S0; a.dS_T = x.dS_T;
     a.dq = x.dq; a.dk = x.dk; a.dv = x.dv; a.dalpha = x.dalpha; a.dtheta = x.dtheta; a.dbeta = x.dbeta; a.dS0 = x.dS0;
     a.T = x.T; a.H = x.H; a.NS = (x.T + kSeg - 1) / kSeg;
-    const size_t bhn = (size_t)x.B * x.H;
-    a.rows = bhn * x.T;
-    a.check = ws + w.check; a.scratch = ws + w.scratch;
-    a.dq_p = ws + w.dq; a.dk_p = ws + w.dk; a.dalpha_p = ws + w.dalpha; a.dtheta_p = ws + w.dtheta; a.dbeta_p = ws + w.dbeta;
-    kern<<<dim3((unsigned)bhn, NSL), kAux + kSolve + 2 * DV, L::bytes, stream>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (launches) ++*launches;
-    if constexpr (NSL > 1) {
-        const size_t n_key = a.rows * DK, n_coord = a.rows * (DK / 2);
-        const size_t items = n_key / 2 + n_coord / 2 + a.rows;
-        size_t blocks = (items + kSumThreads - 1) / kSumThreads;
-        if (blocks > 148 * 8 * 8) blocks = 148 * 8 * 8;
-        sfda_backward_sum_kernel<NSL, T><<<(unsigned)blocks, kSumThreads, 0, stream>>>(
-            a.dq_p, a.dk_p, a.dalpha_p, a.dtheta_p, a.dbeta_p, static_cast<T *>(x.dq), static_cast<T *>(x.dk), x.dalpha,
-            x.dtheta, x.dbeta, n_key, n_coord, a.rows);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (launches) ++*launches;
+    a.units = pairs * a.NS;
+    a.keep_s = ws;
+    a.pitch = a.NS + 1;
+    a.keep_g = ws + (size_t)pairs * a.pitch * state;
+    a.ring_bytes = SC::bytes;
+    if (cols == DV) {
+        a.ring = reinterpret_cast<unsigned char *>(a.keep_g);
+        return launch_walk<DK, DV, T, false>(a, pairs, stream, launches);
     }
-    return cudaSuccess;
-}
-
-template <int DK, int DV, typename T>
-cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t stream, int *launches)
-{
-    const int cols = bwd_cols(x.B, x.H, DV);
-    if (cols == DV) return launch_cols<DK, DV, DV, T>(x, workspace, stream, launches);
-    if constexpr (DV > 64) {
-        if (cols == 64) return launch_cols<DK, DV, 64, T>(x, workspace, stream, launches);
-    }
-    return launch_cols<DK, DV, 32, T>(x, workspace, stream, launches);
+    float *rings = a.keep_g + (size_t)pairs * a.pitch * state;
+    a.ring = reinterpret_cast<unsigned char *>(rings);
+    const size_t room = (bwd_workspace(x.B, x.T, x.H, DK, DV) - (size_t)(rings - ws)) * sizeof(float) / SC::bytes;
+    int grid = a.units < kBwdTargetCtas ? a.units : kBwdTargetCtas;
+    if ((size_t)grid > room) grid = (int)room;
+    // both chains of all pairs at once: the columns are cut while that still fits the SMs
+    int nb = DV;
+    while (nb > 32 && 2LL * pairs * (DV / (nb / 2)) <= kBwdTargetCtas) nb /= 2;
+    cudaError_t e;
+    if (nb == DV) e = launch_chains<DK, DV, DV, T>(a, pairs, stream, launches);
+    else if (nb == 32) e = launch_chains<DK, DV, 32, T>(a, pairs, stream, launches);
+    else e = launch_chains<DK, DV, 64, T>(a, pairs, stream, launches);
+    return e == cudaSuccess ? launch_walk<DK, DV, T, true>(a, grid, stream, launches) : e;
 }
 
 }  // namespace
 
 size_t backward_workspace_bytes(int B, int T, int H, int d_k, int d_v)
 {
-    return bwd_workspace(B, T, H, d_k, d_v).total * sizeof(float);
+    return bwd_workspace(B, T, H, d_k, d_v) * sizeof(float);
 }
 
 cudaError_t launch_backward(const BackwardArgs &a, void *workspace, cudaStream_t stream, int *launches)

@@ -519,14 +519,14 @@ __device__ __forceinline__ void put_planes(unsigned char *p, int pl, float r0, f
 
 // Operand planes of one chunk: W, Y (and Q, with needq) into the slot, Kb_i = beta_i k_i / gamma_i into `kb` for the Gram products.
 // `vals` (or NULL) receives what the gradients need again, two float4 per (token, key): rotated key and query; prod
-// alpha up to the token and after it, e^{i phi}.  Called by all 32 PW threads; the planes are complete for other
-// threads only after a barrier of the caller's.
+// alpha up to the token and after it, e^{i phi}.  Called by all 32 PW threads (BAR: their barrier); the planes are
+// complete for other threads only after a barrier of the caller's.
 //
 // The division by gamma_i is bounded by 2^16 inside a fast chunk (every coordinate keeps at least 2^-16 over the 16
 // tokens): Kb's entries then reach 2^16, the smaller ones keep an absolute error of 2^-39 of that, 2^-23 beside the
 // unit-sized entries of W they meet.  Stronger decays take slow_gram.  Returns whether the chunk is fast (the same
 // value in every thread).
-template <int DK, int PW, typename T>
+template <int DK, int PW, int BAR, typename T>
 __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, T> &in, float4 *vals, unsigned char *slot,
                                             unsigned char *kb, unsigned char *scan, bool needq, int tid)
 {
@@ -554,7 +554,7 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
     for (int x = TPT - 2; x >= 0; --x) sf[x] = make_float2(sf[x + 1].x * in.al[x + 1].x, sf[x + 1].y * in.al[x + 1].y);
     sp[grp * PAIRS + pair] = p[TPT - 1];
     su[grp * PAIRS + pair] = u[TPT - 1];
-    bar_sync(kBarAux, 32 * PW);
+    bar_sync(BAR, 32 * PW);
     float2 pre = make_float2(1.f, 1.f), suf = pre, aC = pre;
     uint2 ub = make_uint2(0u, 0u), uc = ub;
 #pragma unroll 2
@@ -615,7 +615,7 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
     for (int i = 0; i < 4; ++i)
         m[i] = __reduce_max_sync(0xffffffffu, m[i]);
     if (lane == 0) *reinterpret_cast<uint4 *>(red + 4 * warp) = make_uint4(m[0], m[1], m[2], m[3]);
-    bar_sync(kBarAux, 32 * PW);
+    bar_sync(BAR, 32 * PW);
 #pragma unroll 2
     for (int w = 0; w < PW; ++w) {
         const uint4 r = *reinterpret_cast<const uint4 *>(red + 4 * w);
@@ -654,7 +654,7 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
 // The Gram matrices of a chunk whose decays are too strong to divide by: every pair's decay as a running product.  Called
 // by all 32 PW threads after prep_planes returned false; `slow` is a scratch of PrepMap::slow_bytes nobody else uses.
 // Reads its inputs again: passed on, they would not stay in registers on the common path.
-template <int DK, int PW, typename T>
+template <int DK, int PW, int BAR, typename T>
 __device__ __noinline__ void slow_gram(const T *q, const T *k, const float *alpha, const float *theta, const float *beta,
                                        size_t row0, int H, int t0, int T_, unsigned char *slow, const unsigned char *scan,
                                        float2 *gk, float2 *gq, bool needq, int tid)
@@ -686,7 +686,7 @@ __device__ __noinline__ void slow_gram(const T *q, const T *k, const float *alph
         sa[at] = make_float2(in.al[x].x, in.be[x]);
         sa[at + 1] = make_float2(in.al[x].y, in.be[x]);
     }
-    bar_sync(kBarAux, 32 * PW);
+    bar_sync(BAR, 32 * PW);
     for (int t = warp; t < kC; t += PW) {
         float w[M / 32];
 #pragma unroll
@@ -770,43 +770,73 @@ __device__ __forceinline__ void gram_tiles(uint32_t x, uint32_t kb, float f, flo
 }
 
 // Inverse of I + N (16 x 16 complex, [17] float2 rows, only the strictly lower part of N is read) by one warp, in place:
-// X21 = -X22 N21 X11 for blocks of 1, 2, 4, 8 rows, one short loop for all of them.
+// the 4 x 4 diagonal blocks by substitution, then X21 = -X22 N21 X11 twice (4 -> 8 -> 16).  A rolled loop over block
+// sizes 1 to 8 is a quarter of the code and took 3.5 k cycles instead of 1.7 k.
 __device__ __forceinline__ void invert_unit_lower16(float2 *N, int lane)
 {
-#pragma unroll 1
-    for (int e = lane; e < 256; e += 32) {
-        const int t = e >> 4, i = e & 15;
-        if (i >= t) N[t * 17 + i] = make_float2(i == t ? 1.f : 0.f, 0.f);
+    {
+        const int blk = lane >> 3, c = (lane >> 1) & 3, part = lane & 1;      // a lane: half (Re / Im) of one column
+        float2 *B = N + blk * 4 * 18;
+        const float2 n10 = B[17], n20 = B[34], n21 = B[35], n30 = B[51], n31 = B[52], n32 = B[53];
+        float x[4][2];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            float s = (t == c && part == 0) ? 1.f : 0.f;
+#pragma unroll
+            for (int i = 0; i < t; ++i) {
+                const float2 n = t == 1 ? n10 : t == 2 ? (i ? n21 : n20) : (i == 0 ? n30 : i == 1 ? n31 : n32);
+                s -= part ? n.x * x[i][1] + n.y * x[i][0] : n.x * x[i][0] - n.y * x[i][1];
+            }
+            const float o = __shfl_xor_sync(0xffffffffu, s, 1);
+            x[t][0] = part ? o : s;
+            x[t][1] = part ? s : o;
+        }
+        __syncwarp();
+        if (part == 0) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) B[t * 17 + c] = make_float2(x[t][0], x[t][1]);
+        } else if ((blk & 1) == 0) {                                          // the block right of it is zero
+#pragma unroll
+            for (int t = 0; t < 4; ++t) B[t * 17 + 4 + c] = make_float2(0.f, 0.f);
+        }
+        __syncwarp();
     }
-    __syncwarp();
-#pragma unroll 1
-    for (int lg = 0; lg < 4; ++lg) {
-        const int n = 1 << lg;                                    // 8 n elements of X21 altogether; n = 8: two per lane
-        const int first = (lane >> (2 * lg)) << (lg + 1), c = first + (lane & (n - 1)), r = first + n + ((lane >> lg) & (n - 1));
-        const bool on = lane < 8 * n, two = n == 8;
+    {
+        const int r = (lane >> 2) & 3, c = lane & 3;
+        float2 *B = N + (lane >> 4) * 8 * 18;
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
-            const float2 *L = N + r * 17 + first + pass * n, *R = N + (first + pass * n) * 17 + c;
-            float2 x = make_float2(0.f, 0.f), y = x;
-            if (on) {
-#pragma unroll 1
-                for (int i = 0; i < n; ++i, ++L, R += 17) {
-                    const float2 u = *R, l = *L;
-                    x.x += l.x * u.x - l.y * u.y;
-                    x.y += l.x * u.y + l.y * u.x;
-                    if (two) {
-                        const float2 l2 = L[4 * 17];
-                        y.x += l2.x * u.x - l2.y * u.y;
-                        y.y += l2.x * u.y + l2.y * u.x;
-                    }
-                }
+            float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 l = B[(4 + r) * 17 + 4 * pass + i], x = B[(4 * pass + i) * 17 + c];
+                acc.x += l.x * x.x - l.y * x.y;
+                acc.y += l.x * x.y + l.y * x.x;
             }
             __syncwarp();
-            const float sg = pass ? -1.f : 1.f;
-            if (on) N[r * 17 + c] = make_float2(sg * x.x, sg * x.y);
-            if (two) N[(r + 4) * 17 + c] = make_float2(sg * y.x, sg * y.y);
+            B[(4 + r) * 17 + c] = pass ? make_float2(-acc.x, -acc.y) : acc;
             __syncwarp();
         }
+    }
+    const int r = lane >> 2, c0 = 2 * (lane & 3);
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        float2 acc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        const float2 *L = N + (8 + r) * 17 + 8 * pass, *R = N + 8 * 17 * pass;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float2 l = L[i];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float2 x = R[i * 17 + c0 + e];
+                acc[e].x += l.x * x.x - l.y * x.y;
+                acc[e].y += l.x * x.y + l.y * x.x;
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < 2; ++e) N[(8 + r) * 17 + c0 + e] = pass ? make_float2(-acc[e].x, -acc[e].y) : acc[e];
+        __syncwarp();
     }
 }
 
@@ -833,6 +863,44 @@ __device__ __forceinline__ void store_lower(unsigned char *tile, const float2 *A
     }
     if (lane == 0) *inv_out = inv;
 }
+
+// ---- kernels that run a chain and nothing else: PREP, SOLVE, CHAIN -----------------------------------
+constexpr int kPrepWarps = 8, kPrep = 32 * kPrepWarps, kSolve = 128;
+constexpr int kBarPlanes = kBarFree;                             // + slot: planes ready (a chain alone needs no FREE)
+
+// Which warp does what.  A warp runs on scheduler (warp % 4), and mma.sync holds its scheduler: measured, 8.2 cycles each
+// and 0.7 more for every other instruction issued meanwhile.  With 32 columns the two chain warps would share theirs
+// with a quarter of PREP each (7.2 k cycles per chunk); so PREP goes to schedulers 2 and 3, chain and SOLVE to 0 and 1.
+template <int NB>
+struct ChainRoles {
+    static constexpr int threads = NB == 32 ? 512 : kPrep + kSolve + 2 * NB;
+    int prep = -1, solve = -1, chain = -1;                       // thread index inside the role, or -1
+    __device__ explicit ChainRoles(int tid)
+    {
+        if constexpr (NB == 32) {
+            const int w = tid >> 5, lane = tid & 31;
+            if (w & 2) prep = ((w >> 2) * 2 + (w & 1)) * 32 + lane;
+            else if (w < 2) chain = tid;
+            else if (w < 12) solve = (((w >> 2) - 1) * 2 + (w & 1)) * 32 + lane;
+        } else {
+            if (tid < kPrep) prep = tid;
+            else if (tid < kPrep + kSolve) solve = tid - kPrep;
+            else chain = tid - kPrep - kSolve;
+        }
+    }
+};
+
+template <int DK, int NB>
+struct ChainSmem {
+    using PM = PrepMap<DK, kPrepWarps>;
+    static constexpr int kb = kSlots * Tile<DK>::bytes;          // Kb planes, a slot each
+    static constexpr int gram = kb + kSlots * Tile<DK>::BIG;     // the two Gram matrices, a slot each
+    static constexpr int gram_bytes = 2 * 16 * 17 * 8;
+    static constexpr int scan = gram + kSlots * gram_bytes;
+    static constexpr int slow = scan + (PM::scan_bytes + 127) / 128 * 128;
+    static constexpr int bytes = slow + PM::slow_bytes;          // its first word also passes the tensor-memory address on
+    static constexpr int columns = (NB + 63) / 64 * DK / 2 < 32 ? 32 : (NB + 63) / 64 * DK / 2;
+};
 
 }  // namespace c16
 }  // namespace sfda

@@ -7,7 +7,7 @@
 // One CTA per (batch, head) pair and block of value columns; sfda_chunk16.cuh describes the arithmetic (split fp16 on
 // the tensor cores) and the two roles, which are pipelined over a ring of operand tiles.
 //
-// What bounds it: the schedulers' issue slots, which mma.sync holds (see Roles).  Measured in cycles per 16 tokens:
+// What bounds it: the schedulers' issue slots, which mma.sync holds (see ChainRoles).  Measured in cycles per 16 tokens:
 // 6.4 k with 32 value columns per CTA (B = 2, T = 2001, H = 16, d = 128, fp32: 422 us; the unrolled first version 665 us,
 // the CUDA-core kernel 3154 us), 11.4 k with 128 columns; B = 1, T = 256, H = 2, d = 64: 43 us (61, 201).
 #include "sfda_chunk16.cuh"
@@ -26,48 +26,11 @@ struct FwdArgsDev {
     int T, H, dv;
 };
 
-constexpr int kPrepWarps = 8, kPrep = 32 * kPrepWarps, kSolve = 128;
-constexpr int kBarPlanes = kBarFree;                             // + slot: planes ready (the forward needs no FREE)
-
-// Which warp does what.  A warp runs on scheduler (warp % 4), and mma.sync holds its scheduler: measured, 8.2 cycles each
-// and 0.7 more for every other instruction issued meanwhile.  With 32 columns the two chain warps would share theirs
-// with a quarter of PREP each (7.2 k cycles per chunk); so PREP goes to schedulers 2 and 3, chain and SOLVE to 0 and 1.
-template <int NB>
-struct Roles {
-    static constexpr int threads = NB == 32 ? 512 : kPrep + kSolve + 2 * NB;
-    int prep = -1, solve = -1, chain = -1;                       // thread index inside the role, or -1
-    __device__ explicit Roles(int tid)
-    {
-        if constexpr (NB == 32) {
-            const int w = tid >> 5, lane = tid & 31;
-            if (w & 2) prep = ((w >> 2) * 2 + (w & 1)) * 32 + lane;
-            else if (w < 2) chain = tid;
-            else if (w < 12) solve = (((w >> 2) - 1) * 2 + (w & 1)) * 32 + lane;
-        } else {
-            if (tid < kPrep) prep = tid;
-            else if (tid < kPrep + kSolve) solve = tid - kPrep;
-            else chain = tid - kPrep - kSolve;
-        }
-    }
-};
-
-template <int DK, int NB>
-struct FwdSmem {
-    using PM = PrepMap<DK, kPrepWarps>;
-    static constexpr int kb = kSlots * Tile<DK>::bytes;          // Kb planes, a slot each
-    static constexpr int gram = kb + kSlots * Tile<DK>::BIG;     // the two Gram matrices, a slot each
-    static constexpr int gram_bytes = 2 * 16 * 17 * 8;
-    static constexpr int scan = gram + kSlots * gram_bytes;
-    static constexpr int slow = scan + (PM::scan_bytes + 127) / 128 * 128;
-    static constexpr int bytes = slow + PM::slow_bytes;          // its first word also passes the tensor-memory address on
-    static constexpr int columns = (NB + 63) / 64 * DK / 2 < 32 ? 32 : (NB + 63) / 64 * DK / 2;
-};
-
 template <int DK, int NB, typename T>
-__global__ void __launch_bounds__(Roles<NB>::threads, 1) sfda_forward_f32_kernel(const FwdArgsDev a)
+__global__ void __launch_bounds__(ChainRoles<NB>::threads, 1) sfda_forward_f32_kernel(const FwdArgsDev a)
 {
     using TL = Tile<DK>;
-    using L = FwdSmem<DK, NB>;
+    using L = ChainSmem<DK, NB>;
     constexpr int kChain = 2 * NB;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
@@ -80,7 +43,7 @@ __global__ void __launch_bounds__(Roles<NB>::threads, 1) sfda_forward_f32_kernel
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::slow);
     __syncthreads();
 
-    const Roles<NB> role(tid);
+    const ChainRoles<NB> role(tid);
     if (role.prep >= 0) {
         // register shares with all 128 value columns: 256 x 88 + 128 x 72 + 256 x 112 of the launch's 640 x 96
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
@@ -93,8 +56,8 @@ __global__ void __launch_bounds__(Roles<NB>::threads, 1) sfda_forward_f32_kernel
             PrepRaw<L::PM::TPT, T> next;
             prep_fetch<DK, kPrepWarps, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, (c + 1) * kC, a.T, true, role.prep);
             float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes);
-            if (!prep_planes<DK, kPrepWarps, T>(in, nullptr, smem + slot * TL::bytes, smem + L::kb + slot * TL::BIG, smem + L::scan, true, role.prep))
-                slow_gram<DK, kPrepWarps, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, smem + L::slow, smem + L::scan,
+            if (!prep_planes<DK, kPrepWarps, kBarAux, T>(in, nullptr, smem + slot * TL::bytes, smem + L::kb + slot * TL::BIG, smem + L::scan, true, role.prep))
+                slow_gram<DK, kPrepWarps, kBarAux, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, smem + L::slow, smem + L::scan,
                                                    gk, gk + 16 * 17, true, role.prep);
             bar_arrive(kBarPlanes + slot, kPrep + 64);
             in = next;
@@ -179,13 +142,13 @@ template <int DK, int NB, typename T>
 cudaError_t launch_nb(const ForwardArgs &x, cudaStream_t stream)
 {
     auto kern = sfda_forward_f32_kernel<DK, NB, T>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdSmem<DK, NB>::bytes);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainSmem<DK, NB>::bytes);
     if (e != cudaSuccess) return e;
     FwdArgsDev a;
     a.q = x.q; a.k = x.k; a.v = x.v; a.alpha = x.alpha; a.theta = x.theta; a.beta = x.beta; a.S0 = x.S0;
     a.o = x.o; a.o_im = x.o_im; a.S_T = x.S_T;
     a.T = x.T; a.H = x.H; a.dv = x.d_v;
-    kern<<<dim3((unsigned)(x.B * x.H), (unsigned)(x.d_v / NB)), Roles<NB>::threads, FwdSmem<DK, NB>::bytes, stream>>>(a);
+    kern<<<dim3((unsigned)(x.B * x.H), (unsigned)(x.d_v / NB)), ChainRoles<NB>::threads, ChainSmem<DK, NB>::bytes, stream>>>(a);
     return cudaGetLastError();
 }
 
