@@ -38,7 +38,7 @@ constexpr int kSeg = 64;                    // tokens between checkpoints
 constexpr int kSegChunks = kSeg / kC;
 static_assert(kSegChunks == kSlots, "a segment's operand tiles fill the ring");
 constexpr int kGradWarps = 8, kGrad = 32 * kGradWarps;
-constexpr int kBarGrad = kBarAux, kBarPrep = 14;
+constexpr int kBarGrad = kBarAux, kBarPrep = 14, kBarReady = 10, kBarTaken = 12, kBarStaged = 13, kBarTri = 15;   // READY: + parity
 
 struct BwdArgsDev {
     const void *q, *k, *v, *d_o, *d_o_im;
@@ -128,7 +128,7 @@ __device__ __forceinline__ float join_half(uint32_t h, uint32_t l, int half)
     return half ? x.y + y.y : x.x + y.x;
 }
 
-// ---- AUX: the gradients of one chunk --------------------------------------------------------------
+// ---- the gradients where decays are too strong to divide by, or alpha too small -----------------------------
 // The corrections of one (token, key) where the decays are too strong to divide by: running products, token by token.
 // uy: U Yb^T and U B^T (two halves each); x1, x2, x3: the products with the boundary matrices.
 struct SlowOut {
@@ -228,15 +228,14 @@ __device__ __noinline__ float small_alpha(const float4 *vals, const uint4 *frag,
     return sum;
 }
 
+// ---- PREP, second task: what the gradients of a chunk need of its tokens -----------------------------------
+// Yb, Bc, U into shared memory (STAGED), U Yb^T and U B^T, and the triangular factors of the corrections (TRI).
 template <int DK, int NB, typename T>
-__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, const float2 *rg, int slot,
-                                                bool first, int t0, size_t row0, float2 (&carry)[2], int tid)
+__device__ __forceinline__ void stage_tokens(const BwdArgsDev &a, unsigned char *smem, const unsigned char *scr, int slot, int t0, size_t row0, int tid)
 {
     using L = BwdSmem<DK, NB>;
     using SC = BwdScratch<DK, NB>;
-    using TL = Tile<DK>;
-    constexpr int NCW = L::NCW, M = L::M, KT = M / 8;
-    constexpr bool kExact = sizeof(T) == 2;
+    constexpr int NCW = L::NCW;
     const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3;
     const bool has_im = a.d_o_im != nullptr;
     uint4 *frag = reinterpret_cast<uint4 *>(smem + L::frag);                      // [Yb, Bc, U][NCW][4][32]
@@ -244,9 +243,6 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     float2 *uy = reinterpret_cast<float2 *>(smem + L::uy);
     float *scal = reinterpret_cast<float *>(smem + L::scal), *yscal = scal + kSlots * NCW * 4, *tscal = yscal + 8;
     const float *sc = scal + slot * NCW * 4;
-    float *db = reinterpret_cast<float *>(smem + L::db);
-    const uint4 *pS = reinterpret_cast<const uint4 *>(scr + SC::oS), *pG = reinterpret_cast<const uint4 *>(scr + SC::oG);
-    const float4 *vals = reinterpret_cast<const float4 *>(scr + SC::oV);
 
     // operands over the value columns: Yb from the caller's arrays, Bc and U from the ring
     if (warp < NCW) {
@@ -288,7 +284,8 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             frag[(w * 4 + 2 * c + 1) * 32 + lane] = make_uint4(l[0], l[1], l[2], l[3]);
         }
     }
-    bar_sync(kBarGrad, kGrad);
+    bar_sync(kBarPrep, kPrep);
+    bar_arrive(kBarStaged, kPrep + kGrad);
 
     // U Yb^T (index [i][t]: u_i . yb_t) and U B^T (b_t = beta_t p_t = conj of the rows of Bc): warp = (matrix, half of
     // the tokens t, half of the value columns); the A-operand registers of tokens 0-7 / 8-15 are that half's B operand
@@ -330,6 +327,65 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         dst[8 * 17] = make_float2(re[2], im[2]);
         dst[8 * 17 + 1] = make_float2(re[3], im[3]);
     }
+
+    bar_sync(kBarPrep, kPrep);
+
+    // the triangular factors of the corrections as A operands (t, i), a warp each:
+    //   0: u_i . yb_t (i <= t)   1: u_i . b_t (i < t)   2: conj(u_t . yb_i) (i >= t)   3: -conj(u_t . b_i) (i > t)
+    if (warp < 4) {
+        float2 x[4][2];
+        float m = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int t = g + 8 * (e & 1), i = 2 * t4 + 8 * (e >> 1) + j;
+                const float2 *p = uy + (warp & 1) * 272 + (warp < 2 ? i * 17 + t : t * 17 + i);
+                const bool on = (warp & 1) ? (warp < 2 ? i < t : i > t) : (warp < 2 ? i <= t : i >= t);
+                const float2 u = p[0], v = p[544];
+                const float sr = warp == 3 ? -1.f : 1.f, si = warp == 2 ? -1.f : 1.f;
+                x[e][j] = on ? make_float2(sr * (u.x + v.x), si * (u.y + v.y)) : make_float2(0.f, 0.f);
+                m = fmaxf(m, fmaxf(fabsf(x[e][j].x), fabsf(x[e][j].y)));
+            }
+        float inv;
+        const float s = scale_for(warp_max(m), inv);
+        if (lane == 0) tscal[warp] = inv;
+        uint32_t h[4], l[4];
+        uint4 *p = tri + warp * 128 + lane;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) split_f16(x[e][0].x * s, x[e][1].x * s, h[e], l[e]);
+        p[0] = make_uint4(h[0], h[1], h[2], h[3]);
+        p[32] = make_uint4(l[0], l[1], l[2], l[3]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) split_f16(x[e][0].y * s, x[e][1].y * s, h[e], l[e]);
+        p[64] = make_uint4(h[0], h[1], h[2], h[3]);
+        p[96] = make_uint4(l[0], l[1], l[2], l[3]);
+    }
+    bar_arrive(kBarTri, kPrep + kGrad);
+}
+
+// ---- GRAD: the gradients of one chunk -----------------------------------------------------------------
+template <int DK, int NB, typename T>
+__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, const float2 *rg, int slot,
+                                                bool first, bool last_one, int t0, size_t row0, float2 (&carry)[2], int tid)
+{
+    using L = BwdSmem<DK, NB>;
+    using SC = BwdScratch<DK, NB>;
+    using TL = Tile<DK>;
+    constexpr int NCW = L::NCW, M = L::M, KT = M / 8;
+    constexpr bool kExact = sizeof(T) == 2;
+    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3;
+    const bool has_im = a.d_o_im != nullptr;
+    uint4 *frag = reinterpret_cast<uint4 *>(smem + L::frag);                      // [Yb, Bc, U][NCW][4][32]
+    uint4 *tri = reinterpret_cast<uint4 *>(smem + L::tri);
+    float2 *uy = reinterpret_cast<float2 *>(smem + L::uy);
+    float *scal = reinterpret_cast<float *>(smem + L::scal), *yscal = scal + kSlots * NCW * 4, *tscal = yscal + 8;
+    const float *sc = scal + slot * NCW * 4;
+    float *db = reinterpret_cast<float *>(smem + L::db);
+    const uint4 *pS = reinterpret_cast<const uint4 *>(scr + SC::oS), *pG = reinterpret_cast<const uint4 *>(scr + SC::oG);
+    const float4 *vals = reinterpret_cast<const float4 *>(scr + SC::oV);
+
+    bar_sync(kBarStaged, kPrep + kGrad);
 
     // X1 = S_0 yb_t, X2 = S_0 b_t, X3 = G_C conj(u_t) for the keys of tile `warp` (accumulator layout: token g (+ 8),
     // keys 2 t4, + 1); every chain warp's 16 columns come with scales of their own
@@ -434,40 +490,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             be2[r] = t < a.T ? a.beta[row] : 0.f;
         }
     }
-    bar_sync(kBarGrad, kGrad);
-
-    // the triangular factors of the corrections as A operands (t, i), a warp each:
-    //   0: u_i . yb_t (i <= t)   1: u_i . b_t (i < t)   2: conj(u_t . yb_i) (i >= t)   3: -conj(u_t . b_i) (i > t)
-    if (warp < 4) {
-        float2 x[4][2];
-        float m = 0.f;
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int t = g + 8 * (e & 1), i = 2 * t4 + 8 * (e >> 1) + j;
-                const float2 *p = uy + (warp & 1) * 272 + (warp < 2 ? i * 17 + t : t * 17 + i);
-                const bool on = (warp & 1) ? (warp < 2 ? i < t : i > t) : (warp < 2 ? i <= t : i >= t);
-                const float2 u = p[0], v = p[544];
-                const float sr = warp == 3 ? -1.f : 1.f, si = warp == 2 ? -1.f : 1.f;
-                x[e][j] = on ? make_float2(sr * (u.x + v.x), si * (u.y + v.y)) : make_float2(0.f, 0.f);
-                m = fmaxf(m, fmaxf(fabsf(x[e][j].x), fabsf(x[e][j].y)));
-            }
-        float inv;
-        const float s = scale_for(warp_max(m), inv);
-        if (lane == 0) tscal[warp] = inv;
-        uint32_t h[4], l[4];
-        uint4 *p = tri + warp * 128 + lane;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) split_f16(x[e][0].x * s, x[e][1].x * s, h[e], l[e]);
-        p[0] = make_uint4(h[0], h[1], h[2], h[3]);
-        p[32] = make_uint4(l[0], l[1], l[2], l[3]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) split_f16(x[e][0].y * s, x[e][1].y * s, h[e], l[e]);
-        p[64] = make_uint4(h[0], h[1], h[2], h[3]);
-        p[96] = make_uint4(l[0], l[1], l[2], l[3]);
-    }
-    bar_sync(kBarGrad, kGrad);
+    bar_sync(kBarTri, kPrep + kGrad);
 
     if (warp < KT) {
         const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
@@ -523,6 +546,9 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 z3i[i] = fmaf(f2, z3i[i], f3 * wi[i]);
             }
         }
+        // the staged operands are needed further only where a slow path rebuilds something from them
+        const bool keep = !fast || __any_sync(0xffffffffu, fminf(fminf(al2[0].x, al2[0].y), fminf(al2[1].x, al2[1].y)) < 0.0625f);
+        if (!last_one && !keep) bar_arrive(kBarTaken, kGrad + kPrep);
         float2 dqv[4], dkv[4], dd[4];
         float al[4], dbp[2] = {0.f, 0.f};
 #pragma unroll
@@ -620,6 +646,9 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             x += __shfl_xor_sync(0xffffffffu, x, 2);
             if (t4 == 0) db[warp * 16 + g + 8 * r] = x;
         }
+        if (!last_one && keep) bar_arrive(kBarTaken, kGrad + kPrep);
+    } else if (!last_one) {
+        bar_arrive(kBarTaken, kGrad + kPrep);
     }
     bar_sync(kBarGrad, kGrad);
     if (tid < 16 && t0 + tid < a.T) {
@@ -984,40 +1013,53 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::word);
 
-    // register shares: 256 x (96 + 56 + 88) of 768 x 80 with 128 value columns; 256 x (112 + 72) + 128 x 112 of 640 x 96
+    // register shares: 256 x (88 + 64 + 88) of 768 x 80 with 128 value columns; 256 x (104 + 80) + 128 x 112 of 640 x 96
     // with 64
+    const int total = segments * kSegChunks;
     if (tid < kGrad) {
-        if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
-        if constexpr (NB == 64) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+        if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
+        if constexpr (NB == 64) asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
         float2 carry[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll 1
-        for (int n = 0; n < segments * kSegChunks; ++n) {
+        for (int n = 0; n < total; ++n) {
             const int r = n / kSegChunks, at = n % kSegChunks, c = kSegChunks - 1 - at, slot = ring_slot(r, c);
             int bh, s;
             segment(r, bh, s);
-            bar_sync(kBarDone + slot, kGrad + kChain);
-            chunk_gradients<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, rgs + (r & 1) * NCW * M, slot, at == 0,
+            chunk_gradients<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, rgs + (r & 1) * NCW * M, slot, at == 0, n + 1 == total,
                                        s * kSeg + c * kC, row_of(bh), carry, tid);
-            if (r + 1 < segments) bar_arrive(kBarFree + slot, kGrad + kPrep);
+            if (n + kSlots < total) bar_arrive(kBarReady + (n & 1), kGrad + kPrep);
         }
     } else if (tid < kGrad + kPrep) {
-        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        if constexpr (NB == 64) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+        if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        if constexpr (NB == 64) asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
         const int ptid = tid - kGrad, lane = tid & 31, w = ptid >> 5;
         const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
         float2 *gram = reinterpret_cast<float2 *>(smem + L::gram);
-        // Chunks are prepared in the order the chain goes forward through them; a slot is prepared again when the chain
-        // (first sweep) or the gradients (second sweep) are through with it.
+        // One list of steps, two tasks each.  First sweep: chunk p is prepared once the chain is through with chunk p - 4.
+        // Second sweep: the tokens of chunk m = p - 3 (in the order the chain comes back) are staged for the gradients
+        // and chunk p (in the order it goes forward) is prepared once those of chunk p - 4 are written.  The chain needs
+        // a whole segment prepared before it can come back, so that a segment's first chunk is staged second.
 #pragma unroll 1
         for (int sweep = kUnits ? 1 : 0; sweep < 2; ++sweep) {
-            const int np = sweep ? segments * kSegChunks : nch;
+            const int np = sweep ? total : nch;
 #pragma unroll 1
-            for (int p = 0; p < np + (sweep ? 0 : kSlots); ++p) {
-                const int r = p / kSegChunks, at = p % kSegChunks, slot = sweep ? ring_slot(r, at) : at;
-                if (p >= kSlots && p - kSlots < np) bar_sync(kBarFree + slot, (sweep ? kGrad : kChain) + kPrep);
-                if (p >= np) continue;
+            for (int u = 0; u < 2 * (np + (sweep ? 3 : kSlots)); ++u) {
+                const int p = u >> 1, m = sweep ? p - 3 : -1;
                 int bh, s;
+                if (m < 0 ? (u & 1) != 0 : ((u & 1) == 0) != (m % kSegChunks == 0)) {
+                    if (m < 0) continue;
+                    const int r = m / kSegChunks, c = kSegChunks - 1 - m % kSegChunks, slot = ring_slot(r, c);
+                    segment(r, bh, s);
+                    bar_sync(kBarDone + slot, kPrep + kChain);
+                    if (m) bar_sync(kBarTaken, kGrad + kPrep);
+                    stage_tokens<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, slot, s * kSeg + c * kC, row_of(bh), ptid);
+                    continue;
+                }
+                if (!sweep && p >= kSlots) bar_sync(kBarDone + p % kSlots, kPrep + kChain);
+                if (p >= np) continue;
+                const int r = p / kSegChunks, at = p % kSegChunks, slot = sweep ? ring_slot(r, at) : at;
+                if (sweep && p >= kSlots) bar_sync(kBarReady + (p & 1), kGrad + kPrep);
                 segment(sweep ? r : 0, bh, s);
                 const size_t row0 = row_of(bh);
                 const int t0 = sweep ? s * kSeg + at * kC : p * kC;
@@ -1113,7 +1155,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 float rr[2][4];
                 load_rows(rr, static_cast<const T *>(a.v) + (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col, step, a.T - t0 - 2 * t4);
                 big_s = forward_step<DK, kPrep + kChain>(ss, big_s, smem + slot * TL::bytes, kBarFull + slot, rr, pub, r < 0 || c + 1 < kSegChunks, lane);
-                if (r < 0) bar_arrive(kBarFree + slot, kPrep + kChain);
+                if (r < 0) bar_arrive(kBarDone + slot, kPrep + kChain);
             }
             if (r < 0) continue;
 #pragma unroll 1
@@ -1126,7 +1168,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 load_cotangents<T>(yr, yi, a.d_o, a.d_o_im, at, step, left);
                 big_g = backward_step<DK, kExact>(sg, big_g, smem + slot * TL::bytes, yr, yi, a.d_o_im != nullptr, pr, pub, lane);
                 store_rows(static_cast<T *>(a.dv) + at, pr, step, left);
-                bar_arrive(kBarDone + slot, kGrad + kChain);
+                bar_arrive(kBarDone + slot, kPrep + kChain);
             }
             if (!kUnits && r + 1 == segments) state_to_memory<DK>(sg, a.dS0 + state_at, NB);
         }
