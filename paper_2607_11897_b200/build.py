@@ -1,4 +1,4 @@
-"""Build ``libsfda.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Build ``libsfda.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and the small extension beside it.
 
 A build is current when the hash of its sources, kept in a small file beside the library, equals the hash of the
 sources in the tree: file times say nothing once a source file has been put back to an earlier state."""
@@ -10,6 +10,7 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsfda.so")
+HOST = os.path.join(HERE, "_host.so")          # native marshalling of the decode calls (CPython extension)
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 
 FLAGS = [
@@ -24,7 +25,7 @@ def sources():
 
 
 def _deps():
-    return sorted(sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))
+    return sorted(sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cpp"))
                   + glob.glob(os.path.join(HERE, "..", "include", "*.h")))
 
 
@@ -47,12 +48,26 @@ def _current(lib: str, extra_flags=()) -> bool:
 
 
 def is_stale() -> bool:
-    """True when ``libsfda.so`` is missing or was not built from the sources now in the tree."""
-    return not _current(LIB)
+    """True when a library is missing or was not built from the sources now in the tree."""
+    return not (_current(LIB) and os.path.exists(HOST))
 
 
 def _stale() -> bool:
     return is_stale()
+
+
+def _host_command(out: str):
+    """g++ command of the extension; its torch and CUDA symbols come from the libraries torch has loaded."""
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+            "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+            "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+            "-isystem", os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"), "-isystem", sysconfig.get_paths()["include"],
+            os.path.join(CSRC, "sfda_host.cpp"), "-o", out, "-L" + os.path.join(root, "lib"),
+            "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -68,6 +83,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd = [NVCC] + FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", src, "-o", obj]
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
         objs.append(obj)
+    host = HOST + ".tmp.%d" % os.getpid()
+    cmd = _host_command(host)
+    procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     for cmd, p in procs:
         out, _ = p.communicate()
         if verbose and out:
@@ -77,6 +95,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + ".tmp.%d" % os.getpid()
     link = [NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs
     subprocess.run(link, check=True)
+    os.replace(host, HOST)
     os.replace(tmp, LIB)
     with open(LIB + ".srchash", "w") as f:
         f.write(source_hash() + "\n")
