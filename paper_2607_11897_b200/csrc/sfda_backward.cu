@@ -37,7 +37,7 @@ using namespace c16;
 constexpr int kSeg = 64;                    // tokens between checkpoints
 constexpr int kSegChunks = kSeg / kC;
 static_assert(kSegChunks == kSlots, "a segment's operand tiles fill the ring");
-constexpr int kGradWarps = 8, kGrad = 32 * kGradWarps;
+constexpr int kGradWarps = 8, kGrad = 32 * kGradWarps, kPrepWarps = 8, kPrep = 32 * kPrepWarps;   // of the walk with gradients
 constexpr int kBarGrad = kBarAux, kBarPrep = 14, kBarReady = 10, kBarTaken = 12, kBarStaged = 13, kBarTri = 15;   // READY: + parity
 
 struct BwdArgsDev {
@@ -886,11 +886,11 @@ __device__ __forceinline__ float4 *kept(float *keep, int bh, int pitch, int s, i
 // cotangent's chain needs neither S nor U: so S walks forward and G backward at the same time, each in blocks of value
 // columns (NB), both kept every 64 tokens; then every segment's gradients are a unit of their own (kUnits below).
 template <int DK, int DVT, int NB, typename T>
-__global__ void __launch_bounds__(ChainRoles<NB>::threads, 1) sfda_backward_chain_kernel(const BwdArgsDev a)
+__global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_backward_chain_kernel(const BwdArgsDev a)
 {
     using TL = Tile<DK>;
     using L = ChainSmem<DK, NB>;
-    constexpr int kChain = 2 * NB;
+    constexpr int kChain = 2 * NB, kPrepWarps = ChainRoles<DK, NB>::prep_warps, kPrep = ChainRoles<DK, NB>::kPrep;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
     const bool back = blockIdx.z != 0;
@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(ChainRoles<NB>::threads, 1) sfda_backward_chai
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::slow);
     __syncthreads();
 
-    const ChainRoles<NB> role(tid);
+    const ChainRoles<DK, NB> role(tid);
     if (role.prep >= 0) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
         const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
@@ -1217,7 +1217,7 @@ cudaError_t launch_chains(const BwdArgsDev &a, int pairs, cudaStream_t stream, i
     auto kern = sfda_backward_chain_kernel<DK, DV, NB, T>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainSmem<DK, NB>::bytes);
     if (e != cudaSuccess) return e;
-    kern<<<dim3((unsigned)pairs, DV / NB, 2), ChainRoles<NB>::threads, ChainSmem<DK, NB>::bytes, stream>>>(a);
+    kern<<<dim3((unsigned)pairs, DV / NB, 2), ChainRoles<DK, NB>::threads, ChainSmem<DK, NB>::bytes, stream>>>(a);
     if (launches) ++*launches;
     return cudaGetLastError();
 }

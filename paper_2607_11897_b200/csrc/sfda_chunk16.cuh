@@ -865,23 +865,27 @@ __device__ __forceinline__ void store_lower(unsigned char *tile, const float2 *A
 }
 
 // ---- kernels that run a chain and nothing else: PREP, SOLVE, CHAIN -----------------------------------
-constexpr int kPrepWarps = 8, kPrep = 32 * kPrepWarps, kSolve = 128;
+constexpr int kSolve = 128;
 constexpr int kBarPlanes = kBarFree;                             // + slot: planes ready (a chain alone needs no FREE)
 
 // Which warp does what.  A warp runs on scheduler (warp % 4), and mma.sync holds its scheduler: measured, 8.2 cycles each
 // and 0.7 more for every other instruction issued meanwhile.  With 32 columns the two chain warps would share theirs
-// with a quarter of PREP each (7.2 k cycles per chunk); so PREP goes to schedulers 2 and 3, chain and SOLVE to 0 and 1.
-template <int NB>
+// with a quarter of PREP each (7.2 k cycles per chunk at 64 key pairs); so PREP goes to schedulers 2 and 3.  With 64 key
+// pairs it needs eight warps there (four: 8.2 k, eight: 6.3 k) and SOLVE stays beside the chain; with 32 pairs four do,
+// and SOLVE joins them (5.2 k -> 4.9 k).
+template <int DK, int NB>
 struct ChainRoles {
+    static constexpr bool few = NB == 32 && DK == 64;
+    static constexpr int prep_warps = few ? 4 : 8, kPrep = 32 * prep_warps;
     static constexpr int threads = NB == 32 ? 512 : kPrep + kSolve + 2 * NB;
     int prep = -1, solve = -1, chain = -1;                       // thread index inside the role, or -1
     __device__ explicit ChainRoles(int tid)
     {
         if constexpr (NB == 32) {
-            const int w = tid >> 5, lane = tid & 31;
-            if (w & 2) prep = ((w >> 2) * 2 + (w & 1)) * 32 + lane;
-            else if (w < 2) chain = tid;
-            else if (w < 12) solve = (((w >> 2) - 1) * 2 + (w & 1)) * 32 + lane;
+            const int w = tid >> 5, at = ((w >> 2) * 2 + (w & 1)) * 32 + (tid & 31);   // among the warps of two schedulers
+            if (w < 2) chain = tid;
+            else if (w & 2) (few && w >= 8 ? solve : prep) = few && w >= 8 ? at - kPrep : at;
+            else if (!few && w < 12) solve = at - 64;
         } else {
             if (tid < kPrep) prep = tid;
             else if (tid < kPrep + kSolve) solve = tid - kPrep;
@@ -892,7 +896,7 @@ struct ChainRoles {
 
 template <int DK, int NB>
 struct ChainSmem {
-    using PM = PrepMap<DK, kPrepWarps>;
+    using PM = PrepMap<DK, ChainRoles<DK, NB>::prep_warps>;
     static constexpr int kb = kSlots * Tile<DK>::bytes;          // Kb planes, a slot each
     static constexpr int gram = kb + kSlots * Tile<DK>::BIG;     // the two Gram matrices, a slot each
     static constexpr int gram_bytes = 2 * 16 * 17 * 8;

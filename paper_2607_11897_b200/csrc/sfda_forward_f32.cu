@@ -27,11 +27,11 @@ struct FwdArgsDev {
 };
 
 template <int DK, int NB, typename T>
-__global__ void __launch_bounds__(ChainRoles<NB>::threads, 1) sfda_forward_f32_kernel(const FwdArgsDev a)
+__global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f32_kernel(const FwdArgsDev a)
 {
     using TL = Tile<DK>;
     using L = ChainSmem<DK, NB>;
-    constexpr int kChain = 2 * NB;
+    constexpr int kChain = 2 * NB, kPrepWarps = ChainRoles<DK, NB>::prep_warps, kPrep = ChainRoles<DK, NB>::kPrep;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
     const size_t row0 = (size_t)b * a.T * a.H + h;               // row of token t: row0 + t H
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(ChainRoles<NB>::threads, 1) sfda_forward_f32_k
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::slow);
     __syncthreads();
 
-    const ChainRoles<NB> role(tid);
+    const ChainRoles<DK, NB> role(tid);
     if (role.prep >= 0) {
         // register shares with all 128 value columns: 256 x 88 + 128 x 72 + 256 x 112 of the launch's 640 x 96
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
@@ -148,7 +148,7 @@ cudaError_t launch_nb(const ForwardArgs &x, cudaStream_t stream)
     a.q = x.q; a.k = x.k; a.v = x.v; a.alpha = x.alpha; a.theta = x.theta; a.beta = x.beta; a.S0 = x.S0;
     a.o = x.o; a.o_im = x.o_im; a.S_T = x.S_T;
     a.T = x.T; a.H = x.H; a.dv = x.d_v;
-    kern<<<dim3((unsigned)(x.B * x.H), (unsigned)(x.d_v / NB)), ChainRoles<NB>::threads, ChainSmem<DK, NB>::bytes, stream>>>(a);
+    kern<<<dim3((unsigned)(x.B * x.H), (unsigned)(x.d_v / NB)), ChainRoles<DK, NB>::threads, ChainSmem<DK, NB>::bytes, stream>>>(a);
     return cudaGetLastError();
 }
 
