@@ -1492,7 +1492,7 @@ cudaError_t launch_forward_ws(const ForwardArgs &a, void *scratch, size_t scratc
                               bool clear_status)
 {
     Maps maps;
-    if (!make_map(&maps.v, a.v, a.B, a.T, a.H) || !make_map(&maps.o, a.o, a.B, a.T, a.H, false, true) ||
+    if (!make_map(&maps.v, a.v, a.zero_v ? 1 : a.B, a.zero_v ? 1 : a.T, a.zero_v ? 1 : a.H) || !make_map(&maps.o, a.o, a.B, a.T, a.H, false, true) ||
         !make_map(&maps.oim, a.o_im ? a.o_im : a.o, a.B, a.T, a.H, false, true) || !make_map(&maps.q, a.q, a.B, a.T, a.H) ||
         !make_map(&maps.k, a.k, a.B, a.T, a.H) || !make_map(&maps.al, a.alpha, a.B, a.T, a.H, true) ||
         !make_map(&maps.th, a.theta, a.B, a.T, a.H, true))

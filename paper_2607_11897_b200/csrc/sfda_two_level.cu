@@ -133,6 +133,7 @@ two_level_scan_kernel(const float *__restrict__ Bst, const float *__restrict__ P
 constexpr int kCorrThreads = 256;
 constexpr int kCorrTokens = 128;
 constexpr int kCorrTilesPerCta = 8;   // tiles of 128 tokens per CTA: conj(S_in) is converted once for all of them
+constexpr int kCorrDLd = 40;     // row stride (bf16) of the staged corrections
 constexpr int kCorrLd = 72;      // row stride (bf16) of the shared tiles: 144 bytes, conflict-free for ldmatrix
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const __nv_bfloat16 *p)
@@ -179,83 +180,90 @@ two_level_correct_kernel(const __nv_bfloat16 *__restrict__ g_re, const __nv_bflo
     const int arow = 16 * warp + (lane & 7) + 8 * ((lane >> 3) & 1), acol = 8 * (lane >> 4);   // ldmatrix x4 addresses
     const int brow = lane & 7, bcol = 8 * ((lane >> 3) & 1);                                     // ldmatrix x2
     const int gq = lane >> 2, tg = lane & 3;
+    // Corrections of 32 channels as bf16 [128 tokens][32] (Re, then Im) behind the operand tiles, so that the
+    // read-modify-write of the outputs runs on whole 16-byte pieces of a row.
+    constexpr int kPieces = kCorrTokens * 4 / kCorrThreads;              // 16-byte pieces per thread and plane
+    __nv_bfloat16 *Dre = Bim + DV * kCorrLd, *Dim = Dre + kCorrTokens * kCorrDLd;
+    // g tile: 128 rows of 128 bytes (Re and Im), 16 bytes per copy; rows past the slice are zero
+    uint4 gv[8];
+    auto fetch_g = [&](int t0) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const int idx = tid + x * kCorrThreads, r = idx >> 3, ch = idx & 7;
+            gv[x] = gv[4 + x] = make_uint4(0u, 0u, 0u, 0u);
+            if (t0 + r < Ts) {
+                const size_t src = (((size_t)bq * Ts + t0 + r) * H + h) * DV + 8 * ch;
+                gv[x] = __ldcs(reinterpret_cast<const uint4 *>(g_re + src));
+                gv[4 + x] = __ldcs(reinterpret_cast<const uint4 *>(g_im + src));
+            }
+        }
+    };
+    const int first = blockIdx.x * kCorrTilesPerCta, end = min(first + kCorrTilesPerCta, (Ts + kCorrTokens - 1) / kCorrTokens);
+    fetch_g(first * kCorrTokens);
     // this CTA's tiles of 128 tokens
 #pragma unroll 1
-    for (int tile = blockIdx.x * kCorrTilesPerCta; tile < (blockIdx.x + 1) * kCorrTilesPerCta; ++tile) {
-    const int t0 = tile * kCorrTokens;
-    if (t0 >= Ts) break;
-    const int rows = min(kCorrTokens, Ts - t0);
-
-    // g tile: 128 rows of 128 bytes (Re and Im), 16 bytes per copy; rows past the slice are zero
-    for (int idx = tid; idx < kCorrTokens * 8; idx += kCorrThreads) {
-        const int r = idx >> 3, ch = idx & 7;
-        const size_t src = (((size_t)bq * Ts + t0 + r) * H + h) * DV + 8 * ch;
-        uint4 vr = make_uint4(0u, 0u, 0u, 0u), vi = vr;
-        if (r < rows) {
-            vr = *reinterpret_cast<const uint4 *>(g_re + src);
-            vi = *reinterpret_cast<const uint4 *>(g_im + src);
+    for (int tile = first; tile < end; ++tile) {
+        const int t0 = tile * kCorrTokens, rows = min(kCorrTokens, Ts - t0);
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const int idx = tid + x * kCorrThreads, r = idx >> 3, ch = idx & 7;
+            *reinterpret_cast<uint4 *>(Are + r * kCorrLd + 8 * ch) = gv[x];
+            *reinterpret_cast<uint4 *>(Aim + r * kCorrLd + 8 * ch) = gv[4 + x];
         }
-        *reinterpret_cast<uint4 *>(Are + r * kCorrLd + 8 * ch) = vr;
-        *reinterpret_cast<uint4 *>(Aim + r * kCorrLd + 8 * ch) = vi;
-    }
-    __syncthreads();
-
-    // Corrections of one half of the channels as bf16 [128 tokens][64 channels] (Re, then Im) behind the operand
-    // tiles, so that the read-modify-write of the outputs runs on whole 16-byte pieces of a row with every load of a
-    // thread in flight at once.
-    constexpr int kDLd = 64 + 8;
-    __nv_bfloat16 *Dre = Bim + DV * kCorrLd, *Dim = Dre + kCorrTokens * kDLd;
-    constexpr int kPieces = kCorrTokens * 8 / kCorrThreads;              // 16-byte pieces per thread, plane and half
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-        float dre[8][4], dim[8][4];
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) dre[nt][x] = dim[nt][x] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-            uint32_t are[4], aim[4], aren[4];
-            ldsm_x4(are, Are + arow * kCorrLd + 16 * ks + acol);
-            ldsm_x4(aim, Aim + arow * kCorrLd + 16 * ks + acol);
-#pragma unroll
-            for (int x = 0; x < 4; ++x) aren[x] = are[x] ^ 0x80008000u;      // -g_re
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {
-                uint32_t bre[2], bim[2];
-                const int c = 64 * half + 8 * nt + brow;
-                ldsm_x2(bre, Bre + c * kCorrLd + 16 * ks + bcol);
-                ldsm_x2(bim, Bim + c * kCorrLd + 16 * ks + bcol);
-                mma_bf16(dre[nt], are, bre);
-                mma_bf16(dre[nt], aim, bim);
-                mma_bf16(dim[nt], aim, bre);
-                mma_bf16(dim[nt], aren, bim);
-            }
-        }
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int hr = 0; hr < 2; ++hr) {
-                const int r = 16 * warp + gq + 8 * hr, c = 8 * nt + 2 * tg;
-                *reinterpret_cast<__nv_bfloat162 *>(Dre + r * kDLd + c) = __floats2bfloat162_rn(dre[nt][2 * hr], dre[nt][2 * hr + 1]);
-                *reinterpret_cast<__nv_bfloat162 *>(Dim + r * kDLd + c) = __floats2bfloat162_rn(dim[nt][2 * hr], dim[nt][2 * hr + 1]);
-            }
         __syncthreads();
-        auto add_plane = [&](__nv_bfloat16 *dst, const __nv_bfloat16 *D) {
-            uint4 cur[kPieces];
+        // a quarter of the channels at a time; what it needs from memory, and before the last one the next tile of g, is
+        // requested in front of its products
+#pragma unroll 1
+        for (int part = 0; part < 4; ++part) {
+            uint4 cur[2 * kPieces];
+            __nv_bfloat16 *dst[kPieces];
 #pragma unroll
             for (int x = 0; x < kPieces; ++x) {
-                const int idx = tid + x * kCorrThreads, r = idx >> 3, ch = idx & 7;
-                cur[x] = make_uint4(0u, 0u, 0u, 0u);
-                if (r < rows)
-                    cur[x] = *reinterpret_cast<const uint4 *>(dst + (((size_t)bq * Ts + t0 + r) * H + h) * DV + 64 * half + 8 * ch);
+                const int idx = tid + x * kCorrThreads, r = idx >> 2, ch = idx & 3;
+                const size_t at = (((size_t)bq * Ts + t0 + r) * H + h) * DV + 32 * part + 8 * ch;
+                dst[x] = o + at;
+                if (r < rows) {
+                    cur[x] = *reinterpret_cast<const uint4 *>(dst[x]);
+                    if (o_im) cur[kPieces + x] = *reinterpret_cast<const uint4 *>(o_im + at);
+                }
+            }
+            if (part == 3 && tile + 1 < end) fetch_g(t0 + kCorrTokens);
+            float dre[4][4], dim[4][4];
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) dre[nt][x] = dim[nt][x] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                uint32_t are[4], aim[4], aren[4];
+                ldsm_x4(are, Are + arow * kCorrLd + 16 * ks + acol);
+                ldsm_x4(aim, Aim + arow * kCorrLd + 16 * ks + acol);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) aren[x] = are[x] ^ 0x80008000u;      // -g_re
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    uint32_t bre[2], bim[2];
+                    const int c = 32 * part + 8 * nt + brow;
+                    ldsm_x2(bre, Bre + c * kCorrLd + 16 * ks + bcol);
+                    ldsm_x2(bim, Bim + c * kCorrLd + 16 * ks + bcol);
+                    mma_bf16(dre[nt], are, bre);
+                    mma_bf16(dre[nt], aim, bim);
+                    mma_bf16(dim[nt], aim, bre);
+                    mma_bf16(dim[nt], aren, bim);
+                }
             }
 #pragma unroll
-            for (int x = 0; x < kPieces; ++x) {
-                const int idx = tid + x * kCorrThreads, r = idx >> 3, ch = idx & 7;
-                if (r >= rows) continue;
-                const uint4 dl = *reinterpret_cast<const uint4 *>(D + r * kDLd + 8 * ch);
-                const uint32_t *pc = reinterpret_cast<const uint32_t *>(&cur[x]), *pd = reinterpret_cast<const uint32_t *>(&dl);
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int hr = 0; hr < 2; ++hr) {
+                    const int r = 16 * warp + gq + 8 * hr, c = 8 * nt + 2 * tg;
+                    *reinterpret_cast<__nv_bfloat162 *>(Dre + r * kCorrDLd + c) = __floats2bfloat162_rn(dre[nt][2 * hr], dre[nt][2 * hr + 1]);
+                    *reinterpret_cast<__nv_bfloat162 *>(Dim + r * kCorrDLd + c) = __floats2bfloat162_rn(dim[nt][2 * hr], dim[nt][2 * hr + 1]);
+                }
+            __syncthreads();
+            auto add = [&](const uint4 &a4, const __nv_bfloat16 *D) {
+                const uint4 dl = *reinterpret_cast<const uint4 *>(D);
+                const uint32_t *pc = reinterpret_cast<const uint32_t *>(&a4), *pd = reinterpret_cast<const uint32_t *>(&dl);
                 uint32_t out[4];
 #pragma unroll
                 for (int y = 0; y < 4; ++y) {
@@ -264,14 +272,17 @@ two_level_correct_kernel(const __nv_bfloat16 *__restrict__ g_re, const __nv_bflo
                     const __nv_bfloat162 sum = __floats2bfloat162_rn(a2.x + b2.x, a2.y + b2.y);
                     out[y] = *reinterpret_cast<const uint32_t *>(&sum);
                 }
-                *reinterpret_cast<uint4 *>(dst + (((size_t)bq * Ts + t0 + r) * H + h) * DV + 64 * half + 8 * ch) =
-                    make_uint4(out[0], out[1], out[2], out[3]);
+                return make_uint4(out[0], out[1], out[2], out[3]);
+            };
+#pragma unroll
+            for (int x = 0; x < kPieces; ++x) {
+                const int idx = tid + x * kCorrThreads, r = idx >> 2, ch = idx & 3;
+                if (r >= rows) continue;
+                *reinterpret_cast<uint4 *>(dst[x]) = add(cur[x], Dre + r * kCorrDLd + 8 * ch);
+                if (o_im) *reinterpret_cast<uint4 *>(o_im + (dst[x] - o)) = add(cur[kPieces + x], Dim + r * kCorrDLd + 8 * ch);
             }
-        };
-        add_plane(o, Dre);
-        if (o_im) add_plane(o_im, Dim);
-        __syncthreads();                           // the next half overwrites the corrections
-    }
+            __syncthreads();                           // the next quarter overwrites the corrections, the next tile g
+        }
     }
 }
 
@@ -289,7 +300,8 @@ bool forward_two_level_supported(const ForwardArgs &a, int n)
 }
 
 // Workspace: the chunk forward's own scratch for the [B n][T / n] problem, five sets of B n H states (initial states
-// of pass 1a, B, [I | 0], P, true initial states), a zero v and the outputs of pass 1b (Re and Im: g).
+// of pass 1a, B, [I | 0], P, true initial states), the zeros that stand for v in pass 1b (256 bytes of the place of a v
+// are used) and the outputs of pass 1b (Re and Im: g).
 size_t forward_two_level_bytes(const ForwardArgs &a, int n)
 {
     const size_t states = (size_t)a.B * n * a.H * a.d_k * a.d_v * 4;
@@ -313,7 +325,7 @@ cudaError_t launch_forward_two_level(const ForwardArgs &a, int n, void *workspac
     void *g_re = w;                                     w += tokens;
     void *g_im = w;
 
-    cudaError_t e = cudaMemsetAsync(v_zero, 0, tokens, stream);
+    cudaError_t e = cudaMemsetAsync(v_zero, 0, 256, stream);
     if (e != cudaSuccess) return e;
     const unsigned fill_grid = (unsigned)((n_states * per + 255) / 256 < 4096 ? (n_states * per + 255) / 256 : 4096);
     two_level_init_kernel<<<fill_grid, 256, 0, stream>>>(S_a, a.S0, n, a.H, per, n_states);
@@ -328,8 +340,22 @@ cudaError_t launch_forward_two_level(const ForwardArgs &a, int n, void *workspac
     s.S0 = S_a; s.S_T = B_st;
     if ((e = launch_forward_ws(s, fwd_ws, fwd_bytes, stream, launches)) != cudaSuccess) return e;
     // pass 1b: P of every slice, and g_t = P_t^* q_t in the first d_k / 2 channels of its outputs
-    // (same scratch block: the status word keeps a timeout of pass 1a, so that the caller's one read sees either)
-    s.v = v_zero; s.S0 = S_id; s.S_T = P_st; s.o = g_re; s.o_im = g_im;
+    // (same scratch block: the status word keeps a timeout of pass 1a, so that the caller's one read sees either).  The
+    // first slice needs neither; with one batch element the others lie together in memory and it is left out.
+    s.v = v_zero; s.zero_v = 1; s.S0 = S_id; s.S_T = P_st; s.o = g_re; s.o_im = g_im;
+    if (a.B == 1) {
+        const size_t rows = (size_t)s.T * a.H;
+        s.B = n - 1;
+        s.q = static_cast<const char *>(a.q) + rows * a.d_k * 2;
+        s.k = static_cast<const char *>(a.k) + rows * a.d_k * 2;
+        s.alpha = a.alpha + rows * (a.d_k / 2);
+        s.theta = a.theta + rows * (a.d_k / 2);
+        s.beta = a.beta + rows;
+        s.S0 = S_id + a.H * per;
+        s.S_T = P_st + a.H * per;
+        s.o = static_cast<char *>(g_re) + rows * a.d_v * 2;
+        s.o_im = static_cast<char *>(g_im) + rows * a.d_v * 2;
+    }
     if ((e = launch_forward_ws(s, fwd_ws, fwd_bytes, stream, launches, false)) != cudaSuccess) return e;
     // scan over the slices
     two_level_scan_kernel<128, 128><<<dim3((unsigned)(a.B * a.H), 128 / kScanCols), kScanThreads, 0, stream>>>(
@@ -337,7 +363,7 @@ cudaError_t launch_forward_two_level(const ForwardArgs &a, int n, void *workspac
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (launches) ++*launches;
     // correction: o += S_in^* g for every slice but the first
-    const size_t csmem = (size_t)((2 * kCorrTokens + 2 * 128) * kCorrLd + 2 * kCorrTokens * (64 + 8)) * 2;
+    const size_t csmem = (size_t)((2 * kCorrTokens + 2 * 128) * kCorrLd + 2 * kCorrTokens * kCorrDLd) * 2;
     if ((e = cudaFuncSetAttribute(two_level_correct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem)) != cudaSuccess)
         return e;
     const int ctiles = (s.T + kCorrTokens - 1) / kCorrTokens;
