@@ -134,7 +134,7 @@ __device__ __forceinline__ float join_half(uint32_t h, uint32_t l, int half)
 struct SlowOut {
     float2 qb, zb, fb;
 };
-__device__ __noinline__ SlowOut slow_corrections(const float4 *vals, int M, const float2 *uy, const float *alpha, const float *beta,
+__device__ __forceinline__ SlowOut slow_corrections(const float4 *vals, int M, const float2 *uy, const float *alpha, const float *beta,
                                                  size_t row0, int H, int t0, int T_, int tl, int key, float2 x1, float2 x2, float2 x3)
 {
     auto at = [&](int mat, int i, int t) {
@@ -174,7 +174,7 @@ __device__ __noinline__ SlowOut slow_corrections(const float4 *vals, int M, cons
 // dalpha of one (token tl, key) from its definition, by one warp: S_{t-1} and the cotangent of Lambda_t S_{t-1} rebuilt
 // from the boundary matrices, value column by value column.
 template <int DK, int NB>
-__device__ __noinline__ float small_alpha(const float4 *vals, const uint4 *frag, const uint4 *pS, const uint4 *pG, const float *sc,
+__device__ __forceinline__ float small_alpha(const float4 *vals, const uint4 *frag, const uint4 *pS, const uint4 *pG, const float *sc,
                                           const float *yscal, const float *alpha, const float *theta, const float *beta,
                                           size_t row0, int H, int t0, int T_, int tl, int kt, int kl, int lane)
 {
@@ -415,79 +415,58 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 xi[i] = fmaf(f, pi[i] - mi[i], xi[i]);
             }
         };
-        // the ring's operands are requested two steps ahead: they come from L2
-        uint4 n[2][2];
+        // the ring's operands are requested a step ahead (more of them in registers cost more in spills than they hid)
         const uint4 *p = pS + warp * 64 + lane;
+        uint4 n0 = p[0], n1 = p[32];
+#pragma unroll 1
+        for (int w = 0; w < NCW; ++w) {
+            const uint4 s0 = n0, s1 = n1;
+            p = w + 1 < NCW ? p + KT * 64 : pG + warp * 64 + lane;
+            n0 = p[0];
+            n1 = p[32];
+            {
+                const uint4 *fy = frag + w * 128 + lane;
+                const uint4 h = fy[0], l = fy[32];
+                const uint32_t ah[4] = {h.x, h.y, h.z, h.w}, al[4] = {l.x, l.y, l.z, l.w};
+                float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mr[4] = {0.f, 0.f, 0.f, 0.f};
+                mma3x<kExact>(pr, ah, al, s0.x, s0.y, s0.z, s0.w);
+                mma3x<kExact>(pi, ah, al, s1.x, s1.y, s1.z, s1.w);
+                if (has_im) {
+                    const uint4 h2 = fy[64], l2 = fy[96];
+                    const uint32_t bh[4] = {h2.x, h2.y, h2.z, h2.w}, bl[4] = {l2.x, l2.y, l2.z, l2.w};
+                    mma3x<kExact>(mr, bh, bl, s1.x, s1.y, s1.z, s1.w);
+                    mma3x<kExact>(pi, bh, bl, s0.x, s0.y, s0.z, s0.w);
+                }
+                const float f = sc[4 * w] * yscal[w];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            n[e][0] = p[e * KT * 64];
-            n[e][1] = p[e * KT * 64 + 32];
+                for (int i = 0; i < 4; ++i) {
+                    x1r[i] = fmaf(f, pr[i] - mr[i], x1r[i]);
+                    x1i[i] = fmaf(f, pi[i], x1i[i]);
+                }
+            }
+            conj_product(frag + (NCW + w) * 128 + lane, s0, s1, sc[4 * w] * sc[4 * w + 3], x2r, x2i);
         }
 #pragma unroll 1
-        for (int w2 = 0; w2 < NCW; w2 += 2) {
-            p += 2 * KT * 64;
-            if (w2 + 2 >= NCW) p = pG + warp * 64 + lane;
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int w = w2 + e;
-                const uint4 s0 = n[e][0], s1 = n[e][1];
-                n[e][0] = p[e * KT * 64];
-                n[e][1] = p[e * KT * 64 + 32];
-                {
-                    const uint4 *fy = frag + w * 128 + lane;
-                    const uint4 h = fy[0], l = fy[32];
-                    const uint32_t ah[4] = {h.x, h.y, h.z, h.w}, al[4] = {l.x, l.y, l.z, l.w};
-                    float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mr[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma3x<kExact>(pr, ah, al, s0.x, s0.y, s0.z, s0.w);
-                    mma3x<kExact>(pi, ah, al, s1.x, s1.y, s1.z, s1.w);
-                    if (has_im) {
-                        const uint4 h2 = fy[64], l2 = fy[96];
-                        const uint32_t bh[4] = {h2.x, h2.y, h2.z, h2.w}, bl[4] = {l2.x, l2.y, l2.z, l2.w};
-                        mma3x<kExact>(mr, bh, bl, s1.x, s1.y, s1.z, s1.w);
-                        mma3x<kExact>(pi, bh, bl, s0.x, s0.y, s0.z, s0.w);
-                    }
-                    const float f = sc[4 * w] * yscal[w];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        x1r[i] = fmaf(f, pr[i] - mr[i], x1r[i]);
-                        x1i[i] = fmaf(f, pi[i], x1i[i]);
-                    }
-                }
-                conj_product(frag + (NCW + w) * 128 + lane, s0, s1, sc[4 * w] * sc[4 * w + 3], x2r, x2i);
+        for (int w = 0; w < NCW; ++w) {
+            const uint4 g0 = n0, g1 = n1;
+            if (w + 1 < NCW) {
+                p += KT * 64;
+                n0 = p[0];
+                n1 = p[32];
             }
-        }
-#pragma unroll 1
-        for (int w2 = 0; w2 < NCW; w2 += 2) {
-            p += 2 * KT * 64;
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int w = w2 + e;
-                const uint4 g0 = n[e][0], g1 = n[e][1];
-                if (w2 + 2 < NCW) {
-                    n[e][0] = p[e * KT * 64];
-                    n[e][1] = p[e * KT * 64 + 32];
-                }
-                conj_product(frag + (2 * NCW + w) * 128 + lane, g0, g1, sc[4 * w + 2] * sc[4 * w + 1], x3r, x3i);
-            }
+            conj_product(frag + (2 * NCW + w) * 128 + lane, g0, g1, sc[4 * w + 2] * sc[4 * w + 1], x3r, x3i);
         }
     }
-    // what the elements need besides, requested here: it comes from L2 and memory
-    float4 vk[4], vp[4], last[2];
-    float2 al2[2];
-    float be2[2];
+    // what the elements need besides, requested here: it comes from L2 and memory (prod alpha up to the token and after it)
+    float2 va[4], al2[2];
     if (warp < KT) {
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int t = t0 + g + 8 * r;
-            const size_t row = row0 + (size_t)t * a.H;
             const float4 *p = vals + ((g + 8 * r) * M + 8 * warp + 2 * t4) * 2;
-            vk[2 * r] = p[0];
-            vp[2 * r] = p[1];
-            vk[2 * r + 1] = p[2];
-            vp[2 * r + 1] = p[3];
-            last[r] = vals[(15 * M + 8 * warp + 2 * t4 + r) * 2 + 1];              // a_C, -, e^{i phi_C} of key r
-            al2[r] = t < a.T ? *reinterpret_cast<const float2 *>(a.alpha + row * M + 8 * warp + 2 * t4) : make_float2(1.f, 1.f);
-            be2[r] = t < a.T ? a.beta[row] : 0.f;
+            va[2 * r] = *reinterpret_cast<const float2 *>(p + 1);
+            va[2 * r + 1] = *reinterpret_cast<const float2 *>(p + 3);
+            al2[r] = t < a.T ? *reinterpret_cast<const float2 *>(a.alpha + (row0 + (size_t)t * a.H) * M + 8 * warp + 2 * t4) : make_float2(1.f, 1.f);
         }
     }
     bar_sync(kBarTri, kPrep + kGrad);
@@ -495,15 +474,19 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     if (warp < KT) {
         const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
         const bool fast = reinterpret_cast<const int *>(inv)[6] != 0;
-        float z1r[4], z1i[4], z2r[4], z2i[4], z3r[4], z3i[4];
+        const unsigned char *slot_at = smem + slot * TL::bytes;
+        // from here on x1, x2, x3 become S_t yb_t, Lambda_t S_{t-1} b_t, G_t conj(u_t) in the rotated frame
         if (fast) {
             // B operand: tokens as k, the warp's eight keys; heads in registers 0, 1 and tails in 2, 3
-            const uint32_t tile = (uint32_t)__cvta_generic_to_shared(smem) + slot * TL::bytes + (uint32_t)((lane & 15) * TL::LDB + warp * 16 + (lane >> 4) * TL::PL);
-            auto tri_product = [&](int sum, const uint32_t(&br)[4], const uint32_t(&bi)[4], float (&zr)[4], float (&zi)[4]) {
+            const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot_at) + (uint32_t)((lane & 15) * TL::LDB + warp * 16 + (lane >> 4) * TL::PL);
+            auto tri_product = [&](int sum, uint32_t at, float (&zr)[4], float (&zi)[4]) {
                 const uint4 *p = tri + sum * 128 + lane;
                 const uint4 h = p[0], l = p[32], h2 = p[64], l2 = p[96];
                 const uint32_t rh[4] = {h.x, h.y, h.z, h.w}, rl[4] = {l.x, l.y, l.z, l.w};
                 const uint32_t ih[4] = {h2.x, h2.y, h2.z, h2.w}, il[4] = {l2.x, l2.y, l2.z, l2.w};
+                uint32_t br[4], bi[4];
+                ldsm_t(br, tile + at);
+                ldsm_t(bi, tile + at + 2 * TL::PL);
                 float nr[4], ni[4];
                 mma_f16_z(zr, rl, br[0], br[1]);
                 mma_f16_z(zi, rl, bi[0], bi[1]);
@@ -523,27 +506,54 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                     zi[i] += ni[i];
                 }
             };
-            uint32_t br[4], bi[4];
-            ldsm_t(br, tile + TL::oY);
-            ldsm_t(bi, tile + TL::oY + 2 * TL::PL);
-            tri_product(0, br, bi, z1r, z1i);
-            tri_product(1, br, bi, z2r, z2i);
-            ldsm_t(br, tile + TL::oQ);
-            ldsm_t(bi, tile + TL::oQ + 2 * TL::PL);
-            tri_product(2, br, bi, z3r, z3i);
+            const float4 gm = reinterpret_cast<const float4 *>(slot_at + TL::oG)[4 * warp + t4];   // gamma_C of the two keys
+            const float n2[2] = {gm.x * gm.x + gm.y * gm.y, gm.z * gm.z + gm.w * gm.w};
+            float zr[4], zi[4];
+            // a_t (X + conj(gamma_C) Z / |gamma_C|^2), the scale f of Z included
+            auto fold = [&](float f, float (&xr)[4], float (&xi)[4]) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int e = i & 1;
+                    const float w = __fdividef(f, n2[e]);
+                    const float2 z = cmulc(e ? make_float2(gm.z, gm.w) : make_float2(gm.x, gm.y), make_float2(w * zr[i], w * zi[i]));
+                    xr[i] = va[i].x * (xr[i] + z.x);
+                    xi[i] = va[i].x * (xi[i] + z.y);
+                }
+            };
+            tri_product(0, TL::oY, zr, zi);
+            fold(tscal[0] * inv[1], x1r, x1i);
+            tri_product(1, TL::oY, zr, zi);
+            fold(tscal[1] * inv[1], x2r, x2i);
             float wr[4], wi[4];
-            ldsm_t(br, tile + TL::oW);
-            ldsm_t(bi, tile + TL::oW + 2 * TL::PL);
-            tri_product(3, br, bi, wr, wi);
-            const float f0 = tscal[0] * inv[1], f1 = tscal[1] * inv[1], f2 = tscal[2] * inv[2], f3 = tscal[3] * inv[0];
+            tri_product(2, TL::oQ, zr, zi);
+            tri_product(3, TL::oW, wr, wi);
+            const float f2 = tscal[2] * inv[2], f3 = tscal[3] * inv[0];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                z1r[i] *= f0;
-                z1i[i] *= f0;
-                z2r[i] *= f1;
-                z2i[i] *= f1;
-                z3r[i] = fmaf(f2, z3r[i], f3 * wr[i]);
-                z3i[i] = fmaf(f2, z3i[i], f3 * wi[i]);
+                const int e = i & 1;
+                const float s = va[i].y * rsqrtf(n2[e]), down = __frcp_rn(va[i].x);      // 1 / a_t: at most 2^16
+                const float2 z = cmulc(e ? make_float2(gm.z, gm.w) : make_float2(gm.x, gm.y), make_float2(x3r[i], x3i[i]));
+                x3r[i] = fmaf(s, z.x, down * fmaf(f2, zr[i], f3 * wr[i]));
+                x3i[i] = fmaf(s, z.y, down * fmaf(f2, zi[i], f3 * wi[i]));
+            }
+        } else {
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i) {                          // (no function and no indexed registers: both cost the common path)
+                auto pick = [&](const float(&v)[4]) { return i == 0 ? v[0] : i == 1 ? v[1] : i == 2 ? v[2] : v[3]; };
+                auto put = [&](float(&v)[4], float x) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) v[j] = i == j ? x : v[j];
+                };
+                const int tl = g + 8 * (i >> 1), key = 8 * warp + 2 * t4 + (i & 1);
+                const float4 lv = vals[(15 * M + key) * 2 + 1];    // -, -, e^{i phi_C}
+                const SlowOut o = slow_corrections(vals, M, uy, a.alpha, a.beta, row0, a.H, t0, a.T, tl, key, make_float2(pick(x1r), pick(x1i)),
+                                                   make_float2(pick(x2r), pick(x2i)), cmulc(make_float2(lv.z, lv.w), make_float2(pick(x3r), pick(x3i))));
+                put(x1r, o.qb.x);
+                put(x1i, o.qb.y);
+                put(x2r, o.zb.x);
+                put(x2i, o.zb.y);
+                put(x3r, o.fb.x);
+                put(x3i, o.fb.y);
             }
         }
         // the staged operands are needed further only where a slow path rebuilds something from them
@@ -552,33 +562,45 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         float2 dqv[4], dkv[4], dd[4];
         float al[4], dbp[2] = {0.f, 0.f};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = i >> 1, e = i & 1, tl = g + 8 * r, key = 8 * warp + 2 * t4 + e;
-            const float4 x = vk[i], y = vp[i];
-            const float2 kp = make_float2(x.x, x.y), qp = make_float2(x.z, x.w), ph = make_float2(y.z, y.w), pc = make_float2(last[e].z, last[e].w);
-            const float be = be2[r];
-            al[i] = e ? al2[r].y : al2[r].x;
-            const float2 x3 = cmulc(pc, make_float2(x3r[i], x3i[i]));
-            float2 qb, zb, fb;
+        for (int r = 0; r < 2; ++r) {
+            // rotated key and query of the two keys: from the planes (W = a k', Q = a q'), or as they were kept
+            const int tl = g + 8 * r;
+            const float4 *p = vals + (tl * M + 8 * warp + 2 * t4) * 2;
+            float2 kr, ki, qr, qi;
             if (fast) {
-                const float up = __fdividef(y.x, last[e].x), down = __frcp_rn(y.x);   // a_t / a_C, 1 / a_t: at most 2^16
-                const float2 c1 = cmulc(pc, make_float2(z1r[i], z1i[i])), c2 = cmulc(pc, make_float2(z2r[i], z2i[i]));
-                qb = make_float2(fmaf(y.x, x1r[i], up * c1.x), fmaf(y.x, x1i[i], up * c1.y));
-                zb = make_float2(fmaf(y.x, x2r[i], up * c2.x), fmaf(y.x, x2i[i], up * c2.y));
-                fb = make_float2(fmaf(y.y, x3.x, down * z3r[i]), fmaf(y.y, x3.y, down * z3i[i]));
+                const unsigned char *pw = slot_at + tl * TL::LDB + 2 * (8 * warp + 2 * t4);
+                auto both = [&](int off, float2 f) {
+                    const float2 h = unpack_f16(*reinterpret_cast<const uint32_t *>(pw + off)), l = unpack_f16(*reinterpret_cast<const uint32_t *>(pw + off + TL::PL));
+                    return make_float2(f.x * (h.x + l.x), f.y * (h.y + l.y));
+                };
+                const float2 fw = make_float2(__fdividef(inv[0], va[2 * r].x), __fdividef(inv[0], va[2 * r + 1].x));
+                const float2 fq = make_float2(__fdividef(inv[2], va[2 * r].x), __fdividef(inv[2], va[2 * r + 1].x));
+                kr = both(TL::oW, fw);
+                ki = both(TL::oW + 2 * TL::PL, fw);
+                qr = both(TL::oQ, fq);
+                qi = both(TL::oQ + 2 * TL::PL, fq);
             } else {
-                const SlowOut o = slow_corrections(vals, M, uy, a.alpha, a.beta, row0, a.H, t0, a.T, tl, key, make_float2(x1r[i], x1i[i]),
-                                                   make_float2(x2r[i], x2i[i]), x3);
-                qb = o.qb;
-                zb = o.zb;
-                fb = o.fb;
+                const float4 u = p[0], v = p[2];
+                kr = make_float2(u.x, v.x);
+                ki = make_float2(u.y, v.y);
+                qr = make_float2(u.z, v.z);
+                qi = make_float2(u.w, v.w);
             }
-            const float2 dkp = make_float2(be * fb.x - zb.x, be * fb.y - zb.y);
-            dqv[i] = cmul(ph, qb);
-            dkv[i] = cmul(ph, dkp);
-            dbp[r] += fb.x * kp.x + fb.y * kp.y;
-            const float2 p = cmulc(qb, qp), s = cmulc(kp, make_float2(be * fb.x, be * fb.y)), z = cmulc(zb, kp);
-            dd[i] = make_float2(p.x - s.x - z.x, p.y - s.y - z.y);
+            const float be = reinterpret_cast<const float *>(slot_at + TL::oB)[tl];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int i = 2 * r + e;
+                const float2 ph = *(reinterpret_cast<const float2 *>(p + 1 + 2 * e) + 1);          // e^{i phi}
+                const float2 kp = e ? make_float2(kr.y, ki.y) : make_float2(kr.x, ki.x), qp = e ? make_float2(qr.y, qi.y) : make_float2(qr.x, qi.x);
+                const float2 qb = make_float2(x1r[i], x1i[i]), zb = make_float2(x2r[i], x2i[i]), fb = make_float2(x3r[i], x3i[i]);
+                al[i] = e ? al2[r].y : al2[r].x;
+                const float2 dkp = make_float2(be * fb.x - zb.x, be * fb.y - zb.y);
+                dqv[i] = cmul(ph, qb);
+                dkv[i] = cmul(ph, dkp);
+                dbp[r] += fb.x * kp.x + fb.y * kp.y;
+                const float2 y = cmulc(qb, qp), s = cmulc(kp, make_float2(be * fb.x, be * fb.y)), z = cmulc(zb, kp);
+                dd[i] = make_float2(y.x - s.x - z.x, y.y - s.y - z.y);
+            }
         }
         // D: sums over the tokens behind, down to each token (tokens 8-15 in i = 2, 3, tokens 0-7 in i = 0, 1)
         if (first) {

@@ -176,8 +176,8 @@ struct Tile {
     static constexpr int PL = 16 * LDB, BIG = 4 * PL;
     static constexpr int LDS = 48, PS = 16 * LDS, SMALL = 4 * PS;
     static constexpr int oW = 0, oY = BIG, oQ = 2 * BIG, oM = 3 * BIG, oA = oM + SMALL, oG = oA + SMALL, oS = oG + 8 * M;
-    // oG: gamma_C float2 [M]; oS: inverse scales of W, Y, Q, M, A, Kb, then whether the chunk is fast
-    static constexpr int bytes = (oS + 32 + 127) / 128 * 128;
+    // oG: gamma_C float2 [M]; oS: inverse scales of W, Y, Q, M, A, Kb, then whether the chunk is fast; oB: beta [16]
+    static constexpr int oB = oS + 32, bytes = (oB + 64 + 127) / 128 * 128;
 };
 
 // ---- CHAIN --------------------------------------------------------------------------------------
@@ -579,6 +579,10 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
     float4 kk[TPT], qq[TPT];
     float2 av[TPT], yf[TPT], bi[TPT];
     float mw = 0.f, my = 0.f, mq = 0.f, mb = 0.f;
+    if (pair == 0) {
+#pragma unroll
+        for (int x = 0; x < TPT; ++x) reinterpret_cast<float *>(slot + TL::oB)[grp * TPT + x] = in.be[x];
+    }
 #pragma unroll
     for (int x = 0; x < TPT; ++x) {
         const int t = grp * TPT + x;
