@@ -51,6 +51,8 @@ struct BwdArgsDev {
     unsigned char *ring;      // the CTAs' scratch rings, ring_bytes apart
     size_t ring_bytes;
     int T, H, NS, pitch, units;
+    long long work;           // of all pairs' walks, in the units of walk_cut
+    unsigned *flags;          // per CTA: the piece it hands on is written (null where none is)
 };
 
 // One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
@@ -82,7 +84,8 @@ struct BwdSmem {
     static constexpr int scal = tri + 4 * 4 * 512;                // inverse scales [slot][NCW] (S, U, G, B), [NCW] Yb, [4] tri
     static constexpr int db = scal + kSlots * NCW * 16 + 48;      // dbeta: [8][16] floats
     static constexpr int word = db + 8 * 16 * 4;                  // tensor-memory address
-    static constexpr int bytes = word + 16;
+    static constexpr int job = word + 16;                         // the walk's current piece: pair, first and last position, gave up
+    static constexpr int bytes = job + 16;
     static_assert(bytes <= 232448, "shared memory");
     static constexpr int columns = (NB + 63) / 64 * DK < 32 ? 32 : (NB + 63) / 64 * DK;   // S and G
 };
@@ -708,6 +711,26 @@ __device__ __forceinline__ void read_piece(const float4 *p, float (&x)[16])
     }
 }
 
+// A kept state back into tensor memory (NaN if the CTA that writes it was given up); this thread's largest entry
+template <int DK>
+__device__ __forceinline__ float state_from_kept(uint32_t st, const float4 *p, bool gave_up)
+{
+    float largest = 0.f;
+#pragma unroll 1
+    for (int n = 0; n < Tile<DK>::KS; ++n, p += 128) {
+        float x[16];
+        read_piece(p, x);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            if (gave_up) x[i] = __int_as_float(0x7fc00000);
+            largest = fmaxf(largest, fabsf(x[i]));
+        }
+        tm_store(st + 16 * n, x);
+    }
+    tm_wait_store();
+    return largest;
+}
+
 // The split state of a step of keys_product as the B operand (value channel, key) of the gradients' products
 __device__ __forceinline__ void publish_state(uint4 *p, int kk, const uint32_t (&rh)[4], const uint32_t (&rl)[4], const uint32_t (&ih)[4], const uint32_t (&il)[4])
 {
@@ -1000,10 +1023,41 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_backward_
 }
 
 // ---- the walk with gradients ------------------------------------------------------------------------------
-// kUnits == false: one CTA per pair walks the sequence forward (keeping S), then its segments last to first.
+// kUnits == false: a pair is walked forward (keeping S), then its segments last to first: 2 NS positions.  The pairs'
+// positions, one pair after the other, are cut into as many equal pieces as there are CTAs, so that no SM is idle while
+// others work through a last round of whole pairs.  A pair that a cut falls into is begun by the CTA before the cut, as the
+// first thing it does, and finished by the next one, as its last: S or G goes from one to the other through the place of
+// the kept final state, and a CTA only waits for what the CTA before it in the grid does first.  256 pairs of 8192 tokens
+// on 148 SMs, with the forward and the passes around it: 30.5 ms as two rounds of whole pairs, 27.5 ms cut.
 // kUnits == true: S and G are kept already; a CTA takes units (pair, segment) blockIdx.x, + gridDim.x, ...
 // Either way the second sweep is a list of segments, each of kSegChunks chunks (a ragged last one is completed with
 // neutral tokens), pipelined over its borders.
+
+// a position's share of the work: 12.6k cycles per chunk in the first sweep, 44.6k on the way back (d_k = d_v = 128)
+constexpr int kSweepCost = 2, kBackCost = 7;
+
+// Where CTA c's piece begins: pair * 2 NS + position
+__device__ __forceinline__ long long walk_cut(long long work, int c, int ctas, int NS)
+{
+    const long long x = work * c / ctas;
+    const int whole = (kSweepCost + kBackCost) * NS, pair = (int)(x / whole), rest = (int)(x - (long long)pair * whole);
+    return (long long)pair * 2 * NS + (rest < kSweepCost * NS ? rest / kSweepCost : NS + (rest - kSweepCost * NS) / kBackCost);
+}
+
+// The j-th part of CTA c's piece: the pair that the next CTA finishes, whole pairs, the pair that the CTA before has begun.
+// (pair, first position, position behind the last), or pair -1 behind the last part.
+__device__ __forceinline__ int3 walk_part(long long work, int c, int ctas, int NS, int j)
+{
+    const int len = 2 * NS;
+    const long long from = walk_cut(work, c, ctas, NS), to = walk_cut(work, c + 1, ctas, NS);
+    const int head = (int)(to % len), tail = (int)(from % len);
+    const int first = (int)((from + len - 1) / len), last = (int)(to / len);
+    if (head && j-- == 0) return make_int3(last, 0, head);
+    if (j < last - first) return make_int3(first + j, 0, len);
+    if (tail && j == last - first) return make_int3(first - 1, tail, len);
+    return make_int3(-1, 0, 0);
+}
+
 template <int DK, int NB, typename T, bool kUnits>
 __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kernel(const BwdArgsDev a)
 {
@@ -1016,7 +1070,36 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     const int tid = threadIdx.x, NS = a.NS, nch = (a.T + kC - 1) / kC;
     unsigned char *ring = a.ring + blockIdx.x * a.ring_bytes;
     float2 *rgs = reinterpret_cast<float2 *>(ring + SC::oRg);
-    const int segments = kUnits ? (a.units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : NS;
+    volatile int *job = reinterpret_cast<volatile int *>(smem + L::job);
+    // The next part of the walk, for all threads at once (a part leaves none of its barriers pending).
+    auto next_part = [&](int j) {
+        if constexpr (kUnits) return j == 0;
+        bar_sync(0, kGrad + kPrep + kChain);
+        if (tid == 0) {
+            // the first part is what the next CTA waits for
+            if (j == 1 && a.flags) asm volatile("fence.acq_rel.gpu;\n\tst.relaxed.gpu.global.u32 [%0], 1;" ::"l"(a.flags + blockIdx.x) : "memory");
+            const int3 p = walk_part(a.work, blockIdx.x, gridDim.x, NS, j);
+            int gave_up = 0;
+            if (p.x >= 0 && p.y) {                                       // about a second at most
+                uint32_t seen;
+                const uint32_t t0 = (uint32_t)clock();
+                do {
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.flags + blockIdx.x - 1) : "memory");
+                    if (seen) break;
+                    __nanosleep(200);
+                } while ((uint32_t)clock() - t0 < 0x80000000u);
+                gave_up = !seen;
+                __threadfence();
+            }
+            job[0] = p.x;
+            job[1] = p.y;
+            job[2] = p.z;
+            job[3] = gave_up;
+        }
+        bar_sync(0, kGrad + kPrep + kChain);
+        return job[0] >= 0;
+    };
+    auto segments_of = [&] { return kUnits ? (a.units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : max(0, job[2] - max(job[1], NS)); };
     // the r-th segment of this CTA's list: pair and segment; row of token t of a pair: row0 + t H
     auto segment = [&](int r, int &bh, int &s) {
         if constexpr (kUnits) {
@@ -1024,8 +1107,8 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
             bh = u / NS;
             s = u - bh * NS;
         } else {
-            bh = blockIdx.x;
-            s = NS - 1 - r;
+            bh = job[0];
+            s = 2 * NS - 1 - max(job[1], NS) - r;
         }
     };
     auto row_of = [&](int bh) { return (size_t)(bh / a.H) * a.T * a.H + bh % a.H; };
@@ -1037,19 +1120,22 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
 
     // register shares: 256 x (88 + 64 + 88) of 768 x 80 with 128 value columns; 256 x (104 + 80) + 128 x 112 of 640 x 96
     // with 64
-    const int total = segments * kSegChunks;
     if (tid < kGrad) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
         if constexpr (NB == 64) asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
         float2 carry[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll 1
-        for (int n = 0; n < total; ++n) {
-            const int r = n / kSegChunks, at = n % kSegChunks, c = kSegChunks - 1 - at, slot = ring_slot(r, c);
-            int bh, s;
-            segment(r, bh, s);
-            chunk_gradients<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, rgs + (r & 1) * NCW * M, slot, at == 0, n + 1 == total,
-                                       s * kSeg + c * kC, row_of(bh), carry, tid);
-            if (n + kSlots < total) bar_arrive(kBarReady + (n & 1), kGrad + kPrep);
+        for (int j = 0; next_part(j); ++j) {
+            const int total = segments_of() * kSegChunks;
+#pragma unroll 1
+            for (int n = 0; n < total; ++n) {
+                const int r = n / kSegChunks, at = n % kSegChunks, c = kSegChunks - 1 - at, slot = ring_slot(r, c);
+                int bh, s;
+                segment(r, bh, s);
+                chunk_gradients<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, rgs + (r & 1) * NCW * M, slot, at == 0, n + 1 == total,
+                                           s * kSeg + c * kC, row_of(bh), carry, tid);
+                if (n + kSlots < total) bar_arrive(kBarReady + (n & 1), kGrad + kPrep);
+            }
         }
     } else if (tid < kGrad + kPrep) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
@@ -1063,8 +1149,11 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
         // and chunk p (in the order it goes forward) is prepared once those of chunk p - 4 are written.  The chain needs
         // a whole segment prepared before it can come back, so that a segment's first chunk is staged second.
 #pragma unroll 1
-        for (int sweep = kUnits ? 1 : 0; sweep < 2; ++sweep) {
-            const int np = sweep ? total : nch;
+        for (int j = 0; next_part(j);)
+#pragma unroll 1
+        for (int sweep = kUnits ? 1 : 0; sweep < 2; j += sweep++) {
+            const int c0 = sweep ? 0 : min(job[1], NS) * kSegChunks;
+            const int np = sweep ? segments_of() * kSegChunks : min(nch, job[2] * kSegChunks) - c0;
 #pragma unroll 1
             for (int u = 0; u < 2 * (np + (sweep ? 3 : kSlots)); ++u) {
                 const int p = u >> 1, m = sweep ? p - 3 : -1;
@@ -1084,7 +1173,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 if (sweep && p >= kSlots) bar_sync(kBarReady + (p & 1), kGrad + kPrep);
                 segment(sweep ? r : 0, bh, s);
                 const size_t row0 = row_of(bh);
-                const int t0 = sweep ? s * kSeg + at * kC : p * kC;
+                const int t0 = sweep ? s * kSeg + at * kC : (c0 + p) * kC;
                 const bool needq = sweep;
                 unsigned char *tile = smem + slot * TL::bytes;
                 float *inv = reinterpret_cast<float *>(tile + TL::oS);
@@ -1117,17 +1206,21 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
         const size_t step = (size_t)a.H * NB;
         float big_s = 0.f, big_g = 0.f;
 #pragma unroll 1
-        for (int r = kUnits ? 0 : -1; r < segments; ++r) {               // -1: the first sweep over the whole sequence
+        for (int j = 0; next_part(j); ++j)
+#pragma unroll 1
+        for (int r = kUnits ? 0 : -1, segments = segments_of(); r < segments; ++r) {   // -1: the first sweep
             int bh, s;
             segment(max(r, 0), bh, s);
             const size_t state_at = ((size_t)bh * DK + 4 * t4) * NB + col, row0 = row_of(bh);
+            const int from = kUnits ? 0 : job[1], to = kUnits ? 0 : job[2], c0 = r < 0 ? from * kSegChunks : 0;
             if (r < 0) {
-                big_s = state_from_memory<DK>(ss, a.S0 ? a.S0 + state_at : nullptr, NB);
+                if (from >= NS) continue;
+                big_s = from ? state_from_kept<DK>(ss, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), job[3])
+                             : state_from_memory<DK>(ss, a.S0 ? a.S0 + state_at : nullptr, NB);
             } else {
-                if (!kUnits && r == 0) {
-                    keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), ss);
-                    big_g = state_from_memory<DK>(sg, a.dS_T ? a.dS_T + state_at : nullptr, NB);
-                }
+                if (!kUnits && r == 0)
+                    big_g = from > NS ? state_from_kept<DK>(sg, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), job[3])
+                                      : state_from_memory<DK>(sg, a.dS_T ? a.dS_T + state_at : nullptr, NB);
                 // rowdot(conj S, G) at the segment's end, this warp's columns; then S at its start
                 float2 *rg = rgs + ((r & 1) * NCW + w) * M + 2 * t4;
                 const float4 *end = kept<DK>(a.keep_s, bh, a.pitch, s + 1, NB, 16 * w, lane), *start = kept<DK>(a.keep_s, bh, a.pitch, s, NB, 16 * w, lane);
@@ -1168,7 +1261,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 tm_wait_store();
             }
 #pragma unroll 1
-            for (int c = 0; c < (r < 0 ? nch : kSegChunks); ++c) {
+            for (int c = c0, n = r < 0 ? min(nch, to * kSegChunks) : kSegChunks; c < n; ++c) {
                 const int slot = r < 0 ? c % kSlots : ring_slot(r, c), t0 = (r < 0 ? 0 : s * kSeg) + c * kC;
                 if (r < 0 && c % kSegChunks == 0) keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, c / kSegChunks, NB, 16 * w, lane), ss);
                 unsigned char *scr = ring + (size_t)slot * SC::slot;
@@ -1179,7 +1272,10 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 big_s = forward_step<DK, kPrep + kChain>(ss, big_s, smem + slot * TL::bytes, kBarFull + slot, rr, pub, r < 0 || c + 1 < kSegChunks, lane);
                 if (r < 0) bar_arrive(kBarDone + slot, kPrep + kChain);
             }
-            if (r < 0) continue;
+            if (r < 0) {                                                 // the final state, or where the next CTA begins
+                keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), ss);
+                continue;
+            }
 #pragma unroll 1
             for (int c = kSegChunks - 1; c >= 0; --c) {
                 const int slot = ring_slot(r, c), t0 = s * kSeg + c * kC, left = a.T - t0 - 2 * t4;
@@ -1192,7 +1288,10 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 store_rows(static_cast<T *>(a.dv) + at, pr, step, left);
                 bar_arrive(kBarDone + slot, kPrep + kChain);
             }
-            if (!kUnits && r + 1 == segments) state_to_memory<DK>(sg, a.dS0 + state_at, NB);
+            if (!kUnits && r + 1 == segments) {
+                if (to == 2 * NS) state_to_memory<DK>(sg, a.dS0 + state_at, NB);
+                else keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), sg);
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1262,8 +1361,16 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     a.keep_g = ws + (size_t)pairs * a.pitch * state;
     a.ring_bytes = SC::bytes;
     if (cols == DV) {
+        const int grid = pairs < kBwdTargetCtas ? pairs : kBwdTargetCtas;
         a.ring = reinterpret_cast<unsigned char *>(a.keep_g);
-        return launch_walk<DK, DV, T, false>(a, pairs, stream, launches);
+        a.work = (long long)pairs * a.NS * (kSweepCost + kBackCost);
+        a.flags = nullptr;
+        if (pairs % grid) {                                      // behind the rings: a pair has room for one, a CTA uses it
+            a.flags = reinterpret_cast<unsigned *>(a.ring + (size_t)grid * SC::bytes);
+            const cudaError_t e = cudaMemsetAsync(a.flags, 0, grid * sizeof(unsigned), stream);
+            if (e != cudaSuccess) return e;
+        }
+        return launch_walk<DK, DV, T, false>(a, grid, stream, launches);
     }
     float *rings = a.keep_g + (size_t)pairs * a.pitch * state;
     a.ring = reinterpret_cast<unsigned char *>(rings);

@@ -47,3 +47,14 @@ def test_fp32_backward(B, H, T, d_k, d_v, alpha, im):
     if alpha.startswith("u(0.0"):
         inp["alpha"][:, ::17, :, ::5] = 0.0
     check_backward(cfg, inp, upstream(cfg, T, want_im=im), all_pairs(cfg)[:4] + all_pairs(cfg)[-2:], BWD_TOL)
+
+
+@pytest.mark.parametrize("B,H,T,d_k,d_v,im", [
+    (1, 149, 300, 128, 128, True), (5, 37, 200, 128, 64, False), (2, 100, 64, 64, 128, True), (1, 256, 130, 128, 128, False),
+    (3, 99, 449, 64, 64, True)])
+def test_backward_of_pairs_shared_by_two_blocks(B, H, T, d_k, d_v, im):
+    """More pairs than SMs: nearly every pair is begun by one block and finished by the next, from a different place on."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16s", B=B, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="u(0.9,1)", s0_std=0.5,
+                                      seed=500 + T + H)
+    pairs = all_pairs(cfg)
+    check_backward(cfg, workloads.forward_inputs(cfg), upstream(cfg, T, want_im=im), pairs[::19] + pairs[-2:], BWD_TOL)
