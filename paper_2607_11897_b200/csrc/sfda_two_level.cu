@@ -127,13 +127,19 @@ two_level_scan_kernel(const float *__restrict__ Bst, const float *__restrict__ P
 }
 
 // ---- correction o += S_in^* g on the tensor cores (mma.sync m16n8k16, bf16 operands, fp32 accumulation) -------------
-// CTA = 128 tokens of one (slice, head); warp = 16 tokens x 128 channels in two halves of 64.  The A operand is the
-// tile of g (tokens x 64 coordinates, Re and Im), the B operand conj(S_in) as [channel][coordinate]:
+// CTA = 8 tiles of 128 tokens of one (slice, head); warp = 16 channels of 32 tokens at a time.  The A operand is the tile of
+// g (tokens x 64 coordinates, Re and Im), the B operand conj(S_in) as [channel][coordinate], a warp's 16 channels in its
+// registers for all of its tiles:
 //   Re += g_re S_re + g_im S_im,   Im += g_im S_re - g_re S_im.
+// 16 heads x 131072 tokens in 16 slices: 2.5 GB at 3.8 TB/s; the whole forward 2.96 ms.  The next outputs requested a step
+// ahead do not help (3.00 ms): the schedulers are held by mma.sync (a third of the time) and by the instructions around
+// it.  B read from shared memory for each 32 channels of all tokens, outputs in 64-byte pieces: 2.99 ms; 4 or 16 tiles per
+// CTA: 2.98 ms.
 constexpr int kCorrThreads = 256;
 constexpr int kCorrTokens = 128;
 constexpr int kCorrTilesPerCta = 8;   // tiles of 128 tokens per CTA: conj(S_in) is converted once for all of them
-constexpr int kCorrDLd = 40;     // row stride (bf16) of the staged corrections
+constexpr int kCorrDLd = 136;    // row stride (bf16) of the staged corrections
+constexpr int kCorrPart = 32;    // tokens at a time
 constexpr int kCorrLd = 72;      // row stride (bf16) of the shared tiles: 144 bytes, conflict-free for ldmatrix
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const __nv_bfloat16 *p)
@@ -177,13 +183,13 @@ two_level_correct_kernel(const __nv_bfloat16 *__restrict__ g_re, const __nv_bflo
         Bre[c * kCorrLd + l] = __float2bfloat16_rn(Sp[(size_t)(2 * l) * DV + c]);
         Bim[c * kCorrLd + l] = __float2bfloat16_rn(Sp[(size_t)(2 * l + 1) * DV + c]);
     }
-    const int arow = 16 * warp + (lane & 7) + 8 * ((lane >> 3) & 1), acol = 8 * (lane >> 4);   // ldmatrix x4 addresses
-    const int brow = lane & 7, bcol = 8 * ((lane >> 3) & 1);                                     // ldmatrix x2
+    const int arow = (lane & 7) + 8 * ((lane >> 3) & 1), acol = 8 * (lane >> 4);   // ldmatrix x4 addresses
+    const int brow = 16 * warp + (lane & 7), bcol = 8 * ((lane >> 3) & 1);                                     // ldmatrix x2
     const int gq = lane >> 2, tg = lane & 3;
-    // Corrections of 32 channels as bf16 [128 tokens][32] (Re, then Im) behind the operand tiles, so that the
-    // read-modify-write of the outputs runs on whole 16-byte pieces of a row.
-    constexpr int kPieces = kCorrTokens * 4 / kCorrThreads;              // 16-byte pieces per thread and plane
-    __nv_bfloat16 *Dre = Bim + DV * kCorrLd, *Dim = Dre + kCorrTokens * kCorrDLd;
+    // Corrections of 32 tokens as bf16 [32][128 channels] (Re, then Im) behind the operand tiles, so that the
+    // read-modify-write of the outputs runs on whole 256-byte rows.
+    constexpr int kPieces = kCorrPart * DV / 8 / kCorrThreads;              // 16-byte pieces per thread and plane
+    __nv_bfloat16 *Dre = Bim + DV * kCorrLd, *Dim = Dre + kCorrPart * kCorrDLd;
     // g tile: 128 rows of 128 bytes (Re and Im), 16 bytes per copy; rows past the slice are zero
     uint4 gv[8];
     auto fetch_g = [&](int t0) {
@@ -200,6 +206,15 @@ two_level_correct_kernel(const __nv_bfloat16 *__restrict__ g_re, const __nv_bflo
     };
     const int first = blockIdx.x * kCorrTilesPerCta, end = min(first + kCorrTilesPerCta, (Ts + kCorrTokens - 1) / kCorrTokens);
     fetch_g(first * kCorrTokens);
+    __syncthreads();
+    uint32_t bre[4][2][2], bim[4][2][2];             // this warp's 16 channels of S_in^T, for all its tiles
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            ldsm_x2(bre[ks][nt], Bre + (8 * nt + brow) * kCorrLd + 16 * ks + bcol);
+            ldsm_x2(bim[ks][nt], Bim + (8 * nt + brow) * kCorrLd + 16 * ks + bcol);
+        }
     // this CTA's tiles of 128 tokens
 #pragma unroll 1
     for (int tile = first; tile < end; ++tile) {
@@ -211,7 +226,7 @@ two_level_correct_kernel(const __nv_bfloat16 *__restrict__ g_re, const __nv_bflo
             *reinterpret_cast<uint4 *>(Aim + r * kCorrLd + 8 * ch) = gv[4 + x];
         }
         __syncthreads();
-        // a quarter of the channels at a time; what it needs from memory, and before the last one the next tile of g, is
+        // 32 tokens at a time; what it needs from memory, and before the last one the next tile of g, is
         // requested in front of its products
 #pragma unroll 1
         for (int part = 0; part < 4; ++part) {
@@ -219,8 +234,8 @@ two_level_correct_kernel(const __nv_bfloat16 *__restrict__ g_re, const __nv_bflo
             __nv_bfloat16 *dst[kPieces];
 #pragma unroll
             for (int x = 0; x < kPieces; ++x) {
-                const int idx = tid + x * kCorrThreads, r = idx >> 2, ch = idx & 3;
-                const size_t at = (((size_t)bq * Ts + t0 + r) * H + h) * DV + 32 * part + 8 * ch;
+                const int idx = tid + x * kCorrThreads, r = kCorrPart * part + (idx >> 4), ch = idx & 15;
+                const size_t at = (((size_t)bq * Ts + t0 + r) * H + h) * DV + 8 * ch;
                 dst[x] = o + at;
                 if (r < rows) {
                     cur[x] = *reinterpret_cast<const uint4 *>(dst[x]);
@@ -228,38 +243,38 @@ two_level_correct_kernel(const __nv_bfloat16 *__restrict__ g_re, const __nv_bflo
                 }
             }
             if (part == 3 && tile + 1 < end) fetch_g(t0 + kCorrTokens);
-            float dre[4][4], dim[4][4];
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt)
+            for (int half = 0; half < kCorrPart / 16; ++half) {
+                float dre[2][4], dim[2][4];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) dre[nt][x] = dim[nt][x] = 0.f;
+                for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                uint32_t are[4], aim[4], aren[4];
-                ldsm_x4(are, Are + arow * kCorrLd + 16 * ks + acol);
-                ldsm_x4(aim, Aim + arow * kCorrLd + 16 * ks + acol);
+                    for (int x = 0; x < 4; ++x) dre[nt][x] = dim[nt][x] = 0.f;
 #pragma unroll
-                for (int x = 0; x < 4; ++x) aren[x] = are[x] ^ 0x80008000u;      // -g_re
+                for (int ks = 0; ks < 4; ++ks) {
+                    uint32_t are[4], aim[4], aren[4];
+                    const int at = (kCorrPart * part + 16 * half + arow) * kCorrLd + 16 * ks + acol;
+                    ldsm_x4(are, Are + at);
+                    ldsm_x4(aim, Aim + at);
 #pragma unroll
-                for (int nt = 0; nt < 4; ++nt) {
-                    uint32_t bre[2], bim[2];
-                    const int c = 32 * part + 8 * nt + brow;
-                    ldsm_x2(bre, Bre + c * kCorrLd + 16 * ks + bcol);
-                    ldsm_x2(bim, Bim + c * kCorrLd + 16 * ks + bcol);
-                    mma_bf16(dre[nt], are, bre);
-                    mma_bf16(dre[nt], aim, bim);
-                    mma_bf16(dim[nt], aim, bre);
-                    mma_bf16(dim[nt], aren, bim);
+                    for (int x = 0; x < 4; ++x) aren[x] = are[x] ^ 0x80008000u;      // -g_re
+#pragma unroll
+                    for (int nt = 0; nt < 2; ++nt) {
+                        mma_bf16(dre[nt], are, bre[ks][nt]);
+                        mma_bf16(dim[nt], aim, bre[ks][nt]);
+                        mma_bf16(dre[nt], aim, bim[ks][nt]);
+                        mma_bf16(dim[nt], aren, bim[ks][nt]);
+                    }
                 }
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int hr = 0; hr < 2; ++hr) {
+                        const int r = 16 * half + gq + 8 * hr, c = 16 * warp + 8 * nt + 2 * tg;
+                        *reinterpret_cast<__nv_bfloat162 *>(Dre + r * kCorrDLd + c) = __floats2bfloat162_rn(dre[nt][2 * hr], dre[nt][2 * hr + 1]);
+                        *reinterpret_cast<__nv_bfloat162 *>(Dim + r * kCorrDLd + c) = __floats2bfloat162_rn(dim[nt][2 * hr], dim[nt][2 * hr + 1]);
+                    }
             }
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                for (int hr = 0; hr < 2; ++hr) {
-                    const int r = 16 * warp + gq + 8 * hr, c = 8 * nt + 2 * tg;
-                    *reinterpret_cast<__nv_bfloat162 *>(Dre + r * kCorrDLd + c) = __floats2bfloat162_rn(dre[nt][2 * hr], dre[nt][2 * hr + 1]);
-                    *reinterpret_cast<__nv_bfloat162 *>(Dim + r * kCorrDLd + c) = __floats2bfloat162_rn(dim[nt][2 * hr], dim[nt][2 * hr + 1]);
-                }
             __syncthreads();
             auto add = [&](const uint4 &a4, const __nv_bfloat16 *D) {
                 const uint4 dl = *reinterpret_cast<const uint4 *>(D);
@@ -276,8 +291,8 @@ two_level_correct_kernel(const __nv_bfloat16 *__restrict__ g_re, const __nv_bflo
             };
 #pragma unroll
             for (int x = 0; x < kPieces; ++x) {
-                const int idx = tid + x * kCorrThreads, r = idx >> 2, ch = idx & 3;
-                if (r >= rows) continue;
+                const int idx = tid + x * kCorrThreads, r = idx >> 4, ch = idx & 15;
+                if (kCorrPart * part + r >= rows) continue;
                 *reinterpret_cast<uint4 *>(dst[x]) = add(cur[x], Dre + r * kCorrDLd + 8 * ch);
                 if (o_im) *reinterpret_cast<uint4 *>(o_im + (dst[x] - o)) = add(cur[kPieces + x], Dim + r * kCorrDLd + 8 * ch);
             }
@@ -363,7 +378,7 @@ cudaError_t launch_forward_two_level(const ForwardArgs &a, int n, void *workspac
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (launches) ++*launches;
     // correction: o += S_in^* g for every slice but the first
-    const size_t csmem = (size_t)((2 * kCorrTokens + 2 * 128) * kCorrLd + 2 * kCorrTokens * kCorrDLd) * 2;
+    const size_t csmem = (size_t)((2 * kCorrTokens + 2 * 128) * kCorrLd + 2 * kCorrPart * kCorrDLd) * 2;
     if ((e = cudaFuncSetAttribute(two_level_correct_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem)) != cudaSuccess)
         return e;
     const int ctiles = (s.T + kCorrTokens - 1) / kCorrTokens;
