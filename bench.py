@@ -518,7 +518,7 @@ def main():
                 t_sweep.append({"T": Ts, "skipped": "not enough free device memory for this point"})
             torch.cuda.empty_cache()
 
-    # backward pass (sfda_backward) on the headline inputs: token-level fp32 adjoint, a first correct path
+    # backward pass (sfda_backward) on the headline inputs: chunked, on the tensor cores at fp32 precision
     bwd = None
     if rank == 0 and not args.no_backward:
         g = torch.Generator(device=dev)
@@ -552,7 +552,7 @@ def main():
         bwd = {"workload": cfg.name + " (gradients of all inputs)", "ms_per_call": b_ms,
                "tokens_per_s": cfg.B * cfg.T / (b_ms * 1e-3), "algorithmic_bytes": bb,
                "achieved_gbs": bb / (b_ms * 1e-3) / 1e9, "workspace_bytes": int(bws.numel()),
-               "note": "token-level adjoint in fp32 on the CUDA cores, one CTA per (batch, head) pair"}
+               "note": "16-token chunks, split-fp16 tensor-core products at fp32 precision; the walks of all pairs cut into one piece per SM"}
         del d_o, d_oi, dS_T, dq, dk, dv_, dal, dth, dbe, dS0, bws
 
     # forward of the write-decoupled variant (token-level fp32 reference path) on the headline inputs

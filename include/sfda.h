@@ -485,8 +485,9 @@ SFDA_API int sfda_forward_fused(const void *q, const void *k_raw, const void *v,
  *               start of every 64 tokens and room for 64 states; with few sequences more); clobbered.
  *
  * d_k, d_v in {64, 128}; no chunk argument (the derivative does not depend on the chunking).  fp32 precision on the
- * tensor cores in chunks of 16 tokens, as the fp32 forward.  One launch, one CTA per (batch, head) pair; when B * H is
- * at most half of the 148 SMs of a B200, two: the chains of the state and of its cotangent by themselves, then every
+ * tensor cores in chunks of 16 tokens, as the fp32 forward.  One launch, one CTA per (batch, head) pair, or one per SM
+ * with an equal piece of the pairs' walks where there are more pairs than the 148 SMs of a B200; when B * H is at most
+ * half of them two launches: the chains of the state and of its cotangent by themselves, then every
  * segment of 64 tokens as a unit of its own.  The result is deterministic either way.
  */
 SFDA_API size_t sfda_backward_workspace_bytes(int B, int T, int H, int d_k, int d_v, int dtype);
