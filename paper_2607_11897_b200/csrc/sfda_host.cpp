@@ -1,8 +1,10 @@
 // Native marshalling of the decode calls: checks the tensors, takes their addresses and the current stream, calls the
 // C ABI.  One token of one sequence keeps the GPU busy for 2.4 us; the same checks in Python with ctypes took 15 us.
-// Same errors as the Python wrappers: ValueError for layout and place, TypeError for the element type.
+// Errors as in the Python wrappers of the other calls: ValueError for layout and place, TypeError for the element type;
+// what torch itself throws (a tensor without storage, no driver) comes back as the Python exception torch makes of it.
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 namespace {
@@ -56,6 +58,7 @@ bool stream_of(PyObject *obj, void **out)
 // step(q, k, v, alpha, theta, beta, S, o, o_im, stream); step_fused the same with four floats after beta
 PyObject *call(PyObject *const *args, Py_ssize_t n, bool fused)
 {
+    HANDLE_TH_ERRORS
     static const char *const plain[] = {"q", "k", "v", "alpha", "theta", "beta", "S", "o", "o_im"};
     static const char *const raw[] = {"q", "k_raw", "v", "a_raw", "b_raw", "c_raw", "S", "o", "o_im"};
     const char *const *name = fused ? raw : plain;
@@ -100,6 +103,7 @@ PyObject *call(PyObject *const *args, Py_ssize_t n, bool fused)
                     dv, dt, stream);
     }
     return PyLong_FromLong(rc);
+    END_HANDLE_TH_ERRORS
 }
 
 PyObject *step(PyObject *, PyObject *const *args, Py_ssize_t n) { return call(args, n, false); }

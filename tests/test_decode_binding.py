@@ -1,0 +1,35 @@
+"""The native marshalling of the decode calls, away from the arithmetic: what it does with tensors that torch refuses
+to give an address for."""
+import subprocess
+import sys
+
+import pytest
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+
+import paper_2607_11897_b200 as sfda
+
+ROOT = __file__.rsplit("/tests/", 1)[0]
+
+
+def decode_tensors(B=1, H=2, d_k=64, d_v=64, device="cuda"):
+    f = lambda *shape: torch.empty(*shape, device=device)  # noqa: E731
+    return (f(B, H, d_k), f(B, H, d_k), f(B, H, d_v), f(B, H, d_k // 2), f(B, H, d_k // 2), f(B, H)), f(B, H, d_k, d_v), f(B, H, d_v)
+
+
+def call_with_fake_tensors(fused):
+    with FakeTensorMode():
+        x, S, o = decode_tensors()
+        if fused:
+            sfda.sfda_step_fused(*x, 0.0, 1.0, 3.0, 1e-6, S, o, None)
+        else:
+            sfda.sfda_step(*x, S, o, None)
+
+
+@pytest.mark.parametrize("fused", [False, True])
+def test_tensors_without_storage_raise_a_python_exception(fused):
+    """In a process of its own: a C++ exception that leaves the extension would end it."""
+    code = ("import tests.test_decode_binding as t\n"
+            "try:\n    t.call_with_fake_tensors(%r)\nexcept RuntimeError as e:\n    print('raised')\n" % fused)
+    p = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=600)
+    assert p.returncode == 0 and "raised" in p.stdout, (p.returncode, p.stdout, p.stderr[-2000:])
