@@ -88,20 +88,21 @@ PyObject *call(PyObject *const *args, Py_ssize_t n, bool fused)
     }
     if (!stream_of(args[9 + skip], &stream)) return nullptr;
     const int B = (int)q.size(0), H = (int)q.size(1), dk = (int)q.size(2), dv = (int)v.size(-1), dt = type == at::kBFloat16;
-    int rc;
-    if (fused) {
-        float f[4];
-        for (int i = 0; i < 4; ++i) {
-            const double x = PyFloat_AsDouble(args[6 + i]);
-            if (x == -1.0 && PyErr_Occurred()) return nullptr;
-            f[i] = (float)x;
-        }
-        rc = g_step_fused(p[0], p[1], p[2], (const float *)p[3], (const float *)p[4], (const float *)p[5], f[0], f[1], f[2], f[3],
-                          (float *)p[6], p[7], p[8], B, H, dk, dv, dt, stream);
-    } else {
-        rc = g_step(p[0], p[1], p[2], (const float *)p[3], (const float *)p[4], (const float *)p[5], (float *)p[6], p[7], p[8], B, H, dk,
-                    dv, dt, stream);
+    float f[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int i = 0; i < skip; ++i) {
+        const double x = PyFloat_AsDouble(args[6 + i]);
+        if (x == -1.0 && PyErr_Occurred()) return nullptr;
+        f[i] = (float)x;
     }
+    // The launch runs without the interpreter's lock, as a call through ctypes does: it blocks while the launch queue is
+    // full, and what empties the queue may be a host callback that needs the lock.
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    const float *alpha = static_cast<const float *>(p[3]), *theta = static_cast<const float *>(p[4]), *beta = static_cast<const float *>(p[5]);
+    float *S = static_cast<float *>(p[6]);
+    rc = fused ? g_step_fused(p[0], p[1], p[2], alpha, theta, beta, f[0], f[1], f[2], f[3], S, p[7], p[8], B, H, dk, dv, dt, stream)
+               : g_step(p[0], p[1], p[2], alpha, theta, beta, S, p[7], p[8], B, H, dk, dv, dt, stream);
+    Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
     END_HANDLE_TH_ERRORS
 }

@@ -1,7 +1,10 @@
 """The native marshalling of the decode calls, away from the arithmetic: what it does with tensors that torch refuses
 to give an address for."""
+import ctypes
 import subprocess
 import sys
+import threading
+import time
 
 import pytest
 import torch
@@ -33,3 +36,38 @@ def test_tensors_without_storage_raise_a_python_exception(fused):
             "try:\n    t.call_with_fake_tensors(%r)\nexcept RuntimeError as e:\n    print('raised')\n" % fused)
     p = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=600)
     assert p.returncode == 0 and "raised" in p.stdout, (p.returncode, p.stdout, p.stderr[-2000:])
+
+
+SLOW_STEP = """#include <unistd.h>
+extern "C" int slow_step(...) { usleep(400000); return 0; }
+"""
+
+
+@pytest.mark.gpu
+def test_other_python_threads_run_while_a_call_blocks(tmp_path):
+    """A stand-in for a launch that waits for room in the queue: the other thread must not stop meanwhile."""
+    from paper_2607_11897_b200 import binding
+    lib = sfda.load()
+    (tmp_path / "slow.cpp").write_text(SLOW_STEP)
+    subprocess.run(["g++", "-shared", "-fPIC", "-o", str(tmp_path / "slow.so"), str(tmp_path / "slow.cpp")], check=True)
+    slow = ctypes.cast(ctypes.CDLL(str(tmp_path / "slow.so")).slow_step, ctypes.c_void_p).value
+    x, S, o = decode_tensors()
+    sfda.sfda_step(*x, S, o, None)
+    ticks, stop = [], threading.Event()
+
+    def count():
+        while not stop.wait(0.01):
+            ticks.append(time.monotonic())
+    thread = threading.Thread(target=count)
+    binding._host.bind(slow, slow)
+    thread.start()
+    try:
+        t0 = time.monotonic()
+        sfda.sfda_step(*x, S, o, None)
+        t1 = time.monotonic()
+    finally:
+        binding._host.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.sfda_step, lib.sfda_step_fused)))
+        stop.set()
+        thread.join()
+    assert t1 - t0 >= 0.4
+    assert sum(t0 + 0.05 < t < t1 - 0.05 for t in ticks) >= 10, "the other thread stood still during the call"
