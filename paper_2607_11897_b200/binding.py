@@ -1,12 +1,15 @@
 """ctypes marshalling for ``include/sfda.h``.  Same names, same argument order."""
 import ctypes
 import os
+import threading
 
 import torch
 
 SFDA_F32, SFDA_BF16 = 0, 1
 _HERE = os.path.dirname(os.path.abspath(__file__))
-_LIB = None
+_LIB = None                      # the library in use
+_host, _BOUND = None, None       # the extension, and the library whose decode calls it has
+_LOCK = threading.Lock()
 
 _vp, _ci, _sz = ctypes.c_void_p, ctypes.c_int, ctypes.c_size_t
 
@@ -26,39 +29,47 @@ def load():
     the sources now in the tree is rebuilt first: an out-of-date kernel must never be what a test or a benchmark runs."""
     global _LIB
     if _LIB is None:
-        path = lib_path()
-        from . import build as _build
-        if os.path.abspath(path) == os.path.abspath(_build.LIB) and os.path.exists(path) and _build.is_stale():
-            if int(os.environ.get("LOCAL_RANK", "0")) == 0:
-                _build.build(force=True)
-            else:                                   # several ranks on one node: the first one builds, the others wait for it
-                import time
-                for _ in range(1800):
-                    if not _build.is_stale():
-                        break
-                    time.sleep(1.0)
-        _LIB = load_library(path)
-        _host.bind(ctypes.cast(_LIB.sfda_step, _vp).value, ctypes.cast(_LIB.sfda_step_fused, _vp).value)
+        with _LOCK:
+            if _LIB is None:
+                path = lib_path()
+                from . import build as _build
+                if os.path.abspath(path) == os.path.abspath(_build.LIB) and os.path.exists(path) and _build.is_stale():
+                    if int(os.environ.get("LOCAL_RANK", "0")) == 0:
+                        _build.build(force=True)
+                    else:                           # several ranks on one node: the first one builds, the others wait for it
+                        import time
+                        for _ in range(1800):
+                            if not _build.is_stale():
+                                break
+                            time.sleep(1.0)
+                _LIB = load_library(path)
     return _LIB
 
 
-class _HostModule:
-    """The native marshalling of the decode calls; a build of its own beside the library, loaded on first use."""
-
-    def __getattr__(self, name):
-        import importlib.machinery
-        import importlib.util
-        path = os.path.join(_HERE, "_host.so")
-        if not os.path.exists(path):
-            raise ImportError("%s is missing: run `python -m paper_2607_11897_b200.build` first" % path)
-        loader = importlib.machinery.ExtensionFileLoader(__package__ + "._host", path)
-        module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
-        loader.exec_module(module)
-        globals()["_host"] = module
-        return getattr(module, name)
+def _load_host():
+    """The extension module with the native marshalling of the decode calls, a build of its own beside the library."""
+    import importlib.machinery
+    import importlib.util
+    path = os.path.join(_HERE, "_host.so")
+    if not os.path.exists(path):
+        raise ImportError("%s is missing: run `python -m paper_2607_11897_b200.build` first" % path)
+    loader = importlib.machinery.ExtensionFileLoader(__package__ + "._host", path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
+    loader.exec_module(module)
+    return module
 
 
-_host = _HostModule()
+def _bind_decode():
+    """Give the extension the decode calls of the library in use: on the first of them, again after one that failed,
+    and when another build of the library has been put in its place.  ``_BOUND`` is set last, so that a thread which
+    finds it set finds the addresses bound too."""
+    global _host, _BOUND
+    lib = load()
+    with _LOCK:
+        if _host is None:
+            _host = _load_host()
+        _host.bind(ctypes.cast(lib.sfda_step, _vp).value, ctypes.cast(lib.sfda_step_fused, _vp).value)
+        _BOUND = lib
 
 
 def load_library(path):
@@ -278,8 +289,8 @@ def sfda_chunk_factors(k, alpha, theta, beta, Gamma, Y, M, W, phase_turns, chunk
 
 def sfda_step(q, k, v, alpha, theta, beta, S, o, o_im, stream=None):
     """``sfda_step`` of ``include/sfda.h``; S is updated in place."""
-    if _LIB is None:
-        load()
+    if _BOUND is None or _BOUND is not _LIB:
+        _bind_decode()
     rc = _host.step(q, k, v, alpha, theta, beta, S, o, o_im, stream)
     if rc != 0:
         raise SfdaError(rc, "sfda_step")
@@ -353,8 +364,8 @@ def sfda_forward_fused(q, k_raw, v, a_raw, b_raw, c_raw, alpha_min, alpha_max, t
 
 def sfda_step_fused(q, k_raw, v, a_raw, b_raw, c_raw, alpha_min, alpha_max, theta_max, eps, S, o, o_im, stream=None):
     """``sfda_step_fused`` of ``include/sfda.h``: one decode step on the raw inputs; S is updated in place."""
-    if _LIB is None:
-        load()
+    if _BOUND is None or _BOUND is not _LIB:
+        _bind_decode()
     rc = _host.step_fused(q, k_raw, v, a_raw, b_raw, c_raw, alpha_min, alpha_max, theta_max, eps, S, o, o_im, stream)
     if rc != 0:
         raise SfdaError(rc, "sfda_step_fused")

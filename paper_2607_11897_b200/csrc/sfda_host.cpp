@@ -67,6 +67,10 @@ PyObject *call(PyObject *const *args, Py_ssize_t n, bool fused)
         PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
         return nullptr;
     }
+    if (!g_step || !g_step_fused) {
+        PyErr_SetString(PyExc_RuntimeError, "bind has not been called");
+        return nullptr;
+    }
     if (!THPVariable_Check(args[0]) || !THPVariable_Check(args[2])) {
         PyErr_SetString(PyExc_TypeError, "q and v must be tensors");
         return nullptr;

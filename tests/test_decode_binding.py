@@ -47,7 +47,6 @@ extern "C" int slow_step(...) { usleep(400000); return 0; }
 def test_other_python_threads_run_while_a_call_blocks(tmp_path):
     """A stand-in for a launch that waits for room in the queue: the other thread must not stop meanwhile."""
     from paper_2607_11897_b200 import binding
-    lib = sfda.load()
     (tmp_path / "slow.cpp").write_text(SLOW_STEP)
     subprocess.run(["g++", "-shared", "-fPIC", "-o", str(tmp_path / "slow.so"), str(tmp_path / "slow.cpp")], check=True)
     slow = ctypes.cast(ctypes.CDLL(str(tmp_path / "slow.so")).slow_step, ctypes.c_void_p).value
@@ -59,15 +58,89 @@ def test_other_python_threads_run_while_a_call_blocks(tmp_path):
         while not stop.wait(0.01):
             ticks.append(time.monotonic())
     thread = threading.Thread(target=count)
-    binding._host.bind(slow, slow)
     thread.start()
+    binding._host.bind(slow, slow)
     try:
         t0 = time.monotonic()
         sfda.sfda_step(*x, S, o, None)
         t1 = time.monotonic()
     finally:
-        binding._host.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.sfda_step, lib.sfda_step_fused)))
+        binding._bind_decode()
         stop.set()
         thread.join()
     assert t1 - t0 >= 0.4
     assert sum(t0 + 0.05 < t < t1 - 0.05 for t in ticks) >= 10, "the other thread stood still during the call"
+
+
+def in_a_new_process(body):
+    code = "import threading\nimport tests.test_decode_binding as t\nfrom paper_2607_11897_b200 import binding\n" + body
+    p = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=600)
+    assert p.returncode == 0 and "done" in p.stdout, (p.returncode, p.stdout, p.stderr[-2000:])
+
+
+def test_an_unbound_extension_raises():
+    """The extension by itself, before anybody gave it the library's addresses."""
+    in_a_new_process("""
+host = binding._load_host() if hasattr(binding, "_load_host") else binding._host
+x, S, o = t.decode_tensors(device="cpu")
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+class Stream:
+    cuda_stream = 0
+with FakeTensorMode():
+    x, S, o = t.decode_tensors()
+    try:
+        host.step(*x, S, o, None, Stream())
+    except RuntimeError as e:
+        assert "bind" in str(e), e
+        print("done")
+""")
+
+
+def test_the_first_calls_of_two_threads_both_find_the_library_bound():
+    """The second thread calls while the first is still loading the extension."""
+    in_a_new_process("""
+import time
+held, slow = [], threading.Event()
+real = binding._load_host
+def load_host():
+    slow.set()
+    time.sleep(0.5)
+    return real()
+binding._load_host = load_host
+def call():
+    try:
+        t.call_with_fake_tensors(False)
+    except RuntimeError as e:
+        held.append("bind" not in str(e))
+a = threading.Thread(target=call)
+a.start()
+slow.wait()
+b = threading.Thread(target=call)
+b.start()
+a.join(); b.join()
+assert held == [True, True], held
+print("done")
+""")
+
+
+def test_a_call_after_a_failed_load_of_the_extension_tries_again():
+    in_a_new_process("""
+real = binding._load_host
+def missing():
+    raise ImportError("not there yet")
+binding._load_host = missing
+for fused in (False, True):
+    try:
+        t.call_with_fake_tensors(fused)
+    except ImportError:
+        pass
+    else:
+        raise AssertionError("no error")
+binding._load_host = real
+try:
+    t.call_with_fake_tensors(True)
+except RuntimeError as e:
+    assert "bind" not in str(e), e
+print("done")
+""")
