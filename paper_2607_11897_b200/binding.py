@@ -33,26 +33,37 @@ def load():
             if _LIB is None:
                 path = lib_path()
                 from . import build as _build
-                if os.path.abspath(path) == os.path.abspath(_build.LIB) and os.path.exists(path) and _build.is_stale():
-                    if int(os.environ.get("LOCAL_RANK", "0")) == 0:
-                        _build.build(force=True)
-                    else:                           # several ranks on one node: the first one builds, the others wait for it
-                        import time
-                        for _ in range(1800):
-                            if not _build.is_stale():
-                                break
-                            time.sleep(1.0)
+                if os.path.abspath(path) == os.path.abspath(_build.LIB) and os.path.exists(path):
+                    _rebuild_if(_build.is_stale, _build.build_library)
                 _LIB = load_library(path)
     return _LIB
 
 
+def _rebuild_if(stale, build):
+    """Several ranks on one node: the first one builds, the others wait for it."""
+    if not stale():
+        return
+    if int(os.environ.get("LOCAL_RANK", "0")) == 0:
+        build()
+        return
+    import time
+    for _ in range(1800):
+        if not stale():
+            break
+        time.sleep(1.0)
+
+
 def _load_host():
-    """The extension module with the native marshalling of the decode calls, a build of its own beside the library."""
+    """The extension module with the native marshalling of the decode calls, a build of its own beside the library that
+    nothing else needs.  One built for another torch or interpreter is rebuilt first, like an out-of-date library."""
     import importlib.machinery
     import importlib.util
+
+    from . import build as _build
     path = os.path.join(_HERE, "_host.so")
     if not os.path.exists(path):
         raise ImportError("%s is missing: run `python -m paper_2607_11897_b200.build` first" % path)
+    _rebuild_if(_build.host_is_stale, _build.build_host)
     loader = importlib.machinery.ExtensionFileLoader(__package__ + "._host", path)
     module = importlib.util.module_from_spec(importlib.util.spec_from_loader(loader.name, loader))
     loader.exec_module(module)

@@ -1,11 +1,13 @@
 """Build ``libsfda.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and the small extension beside it.
 
 A build is current when the hash of its sources, kept in a small file beside the library, equals the hash of the
-sources in the tree: file times say nothing once a source file has been put back to an earlier state."""
+sources in the tree: file times say nothing once a source file has been put back to an earlier state.  The extension's
+hash also covers the torch and the interpreter that it was built against; the library depends on neither."""
 import glob
 import hashlib
 import os
 import subprocess
+import sys
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -25,7 +27,7 @@ def sources():
 
 
 def _deps():
-    return sorted(sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cpp"))
+    return sorted(sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))
                   + glob.glob(os.path.join(HERE, "..", "include", "*.h")))
 
 
@@ -39,21 +41,27 @@ def source_hash(extra_flags=()) -> str:
     return h.hexdigest()
 
 
-def _current(lib: str, extra_flags=()) -> bool:
+def _recorded(target: str):
+    """The hash kept beside a build, or None where there is no such build."""
     try:
-        with open(lib + ".srchash") as f:
-            return os.path.exists(lib) and f.read().strip() == source_hash(extra_flags)
+        with open(target + ".srchash") as f:
+            return f.read().strip() if os.path.exists(target) else None
     except OSError:
-        return False
+        return None
+
+
+def _record(target: str, value: str) -> None:
+    with open(target + ".srchash", "w") as f:
+        f.write(value + "\n")
+
+
+def _current(lib: str, extra_flags=()) -> bool:
+    return _recorded(lib) == source_hash(extra_flags)
 
 
 def is_stale() -> bool:
-    """True when a library is missing or was not built from the sources now in the tree."""
-    return not (_current(LIB) and os.path.exists(HOST))
-
-
-def _stale() -> bool:
-    return is_stale()
+    """True when the library is missing or was not built from the sources now in the tree."""
+    return not _current(LIB)
 
 
 def _host_command(out: str):
@@ -70,35 +78,71 @@ def _host_command(out: str):
             "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every ``csrc/*.cu`` into ``libsfda.so`` when missing or stale."""
-    if not force and not _stale():
-        return LIB
-    objdir = os.path.join(HERE, "build")
-    os.makedirs(objdir, exist_ok=True)
-    objs = []
-    procs = []
-    for src in sources():
-        obj = os.path.join(objdir, os.path.basename(src)[:-3] + ".o")
-        cmd = [NVCC] + FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", src, "-o", obj]
-        procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-        objs.append(obj)
-    host = HOST + ".tmp.%d" % os.getpid()
-    cmd = _host_command(host)
-    procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+def host_hash() -> str:
+    """SHA-256 over the extension's source, its build command and the torch and interpreter whose ABI it is built for."""
+    import sysconfig
+
+    import torch
+    h = hashlib.sha256(" ".join(_host_command("") + [torch.__version__, sys.version, str(sysconfig.get_config_var("SOABI"))]).encode())
+    with open(os.path.join(CSRC, "sfda_host.cpp"), "rb") as f:
+        h.update(f.read())
+    return h.hexdigest()
+
+
+def host_is_stale() -> bool:
+    """True when the extension is missing or was built from another source or for another torch or interpreter."""
+    return _recorded(HOST) != host_hash()
+
+
+def _start(cmd):
+    return cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+
+
+def _finish(procs, verbose=False):
     for cmd, p in procs:
         out, _ = p.communicate()
         if verbose and out:
             print(out)
         if p.returncode != 0:
-            raise RuntimeError("nvcc failed: %s\n%s" % (" ".join(cmd), out))
-    tmp = LIB + ".tmp.%d" % os.getpid()
-    link = [NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs
-    subprocess.run(link, check=True)
-    os.replace(host, HOST)
-    os.replace(tmp, LIB)
-    with open(LIB + ".srchash", "w") as f:
-        f.write(source_hash() + "\n")
+            raise RuntimeError("build failed: %s\n%s" % (" ".join(cmd), out))
+
+
+def build_host() -> str:
+    """Compile the extension."""
+    tmp = HOST + ".tmp.%d" % os.getpid()
+    _finish([_start(_host_command(tmp))])
+    os.replace(tmp, HOST)
+    _record(HOST, host_hash())
+    return HOST
+
+
+def build_library(verbose: bool = False) -> str:
+    """Compile every ``csrc/*.cu`` into ``libsfda.so``."""
+    objdir = os.path.join(HERE, "build")
+    os.makedirs(objdir, exist_ok=True)
+    _link(objdir, LIB, [], verbose)
+    return LIB
+
+
+def _link(objdir, lib, extra_flags, verbose=False):
+    procs, objs = [], []
+    for src in sources():
+        obj = os.path.join(objdir, os.path.basename(src)[:-3] + ".o")
+        procs.append(_start([NVCC] + FLAGS + list(extra_flags) + (["-Xptxas", "-v"] if verbose else []) + ["-c", src, "-o", obj]))
+        objs.append(obj)
+    _finish(procs, verbose)
+    tmp = lib + ".tmp.%d" % os.getpid()
+    subprocess.run([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs, check=True)
+    os.replace(tmp, lib)
+    _record(lib, source_hash(extra_flags))
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    """Build the library and the extension where they are missing or stale; returns the library's path."""
+    if force or is_stale():
+        build_library(verbose)
+    if force or host_is_stale():
+        build_host()
     return LIB
 
 
@@ -110,21 +154,7 @@ def build_variant(name: str, extra_flags):
     if _current(lib, extra_flags):
         return lib
     os.makedirs(objdir, exist_ok=True)
-    procs, objs = [], []
-    for src in sources():
-        obj = os.path.join(objdir, os.path.basename(src)[:-3] + ".o")
-        cmd = [NVCC] + FLAGS + list(extra_flags) + ["-c", src, "-o", obj]
-        procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-        objs.append(obj)
-    for cmd, p in procs:
-        out, _ = p.communicate()
-        if p.returncode != 0:
-            raise RuntimeError("nvcc failed: %s\n%s" % (" ".join(cmd), out))
-    tmp = lib + ".tmp.%d" % os.getpid()
-    subprocess.run([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs, check=True)
-    os.replace(tmp, lib)
-    with open(lib + ".srchash", "w") as f:
-        f.write(source_hash(extra_flags) + "\n")
+    _link(objdir, lib, extra_flags)
     return lib
 
 

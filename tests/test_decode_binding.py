@@ -144,3 +144,29 @@ except RuntimeError as e:
     assert "bind" not in str(e), e
 print("done")
 """)
+
+
+def test_only_the_decode_calls_need_the_extension():
+    in_a_new_process("""
+from paper_2607_11897_b200 import build
+build.HOST = binding.__dict__["_HERE"] + "/no_such_host.so"
+binding._load_host = lambda: (_ for _ in ()).throw(ImportError("missing"))
+import paper_2607_11897_b200 as sfda
+assert sfda.sfda_plan(256, 64) and not build.is_stale() and build.host_is_stale()
+print("done")
+""")
+
+
+def test_an_extension_for_another_torch_or_interpreter_is_stale(monkeypatch):
+    import torch
+
+    from paper_2607_11897_b200 import build
+    build.build()
+    assert not build.host_is_stale()
+    with monkeypatch.context() as m:
+        m.setattr(torch, "__version__", "0.0.1")
+        assert build.host_is_stale()
+    with monkeypatch.context() as m:
+        m.setattr(sys, "version", "2.0")
+        assert build.host_is_stale()
+    assert not build.host_is_stale()
