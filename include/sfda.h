@@ -219,11 +219,11 @@ SFDA_API int sfda_forward_two_level(const void *q, const void *k, const void *v,
                                     void *workspace, size_t workspace_bytes, void *stream);
 
 /*
- * After work enqueued by sfda_forward with a non-empty workspace: waits for `stream`
- * and reads the status word the tensor-core kernel keeps at the start of the
+ * After work enqueued by sfda_forward with a non-empty workspace, or by sfda_backward: waits for `stream`
+ * and reads the status word the kernel keeps at the start of the
  * workspace.  Returns SFDA_OK, or SFDA_ERR_TIMEOUT when a bounded device-side wait
- * (on a TMA copy or a tensor-core commit) ran out, in which case the kernel returned
- * early and o, o_im, S_T of that call are invalid; *detail (host, may be NULL) gets
+ * (on a TMA copy, a tensor-core commit or another CTA) ran out, in which case the forward's kernel returned
+ * early and o, o_im, S_T of that call are invalid (sfda_backward says what becomes of its gradients); *detail (host, may be NULL) gets
  * the raw word.  Synchronises the stream.  Host only.
  */
 SFDA_API int sfda_workspace_status(const void *workspace, void *stream, uint32_t *detail);
@@ -482,13 +482,19 @@ SFDA_API int sfda_forward_fused(const void *q, const void *k_raw, const void *v,
  *               to its two real numbers), dv [B][T][H][d_v] dtype, dalpha, dtheta [B][T][H][m] float,
  *               dbeta [B][T][H] float, dS0 [B][H][d_k][d_v] float.  All are required and overwritten.
  *  workspace:   sfda_backward_workspace_bytes(...) bytes of device scratch (per (batch, head) pair the state at the
- *               start of every 64 tokens and room for 64 states; with few sequences more); clobbered.
+ *               start of every 64 tokens and room for 64 states; with few sequences more); clobbered.  It begins with
+ *               the status word that sfda_workspace_status reads.
  *
  * d_k, d_v in {64, 128}; no chunk argument (the derivative does not depend on the chunking).  fp32 precision on the
  * tensor cores in chunks of 16 tokens, as the fp32 forward.  One launch, one CTA per (batch, head) pair, or one per SM
  * with an equal piece of the pairs' walks where there are more pairs than the 148 SMs of a B200; when B * H is at most
  * half of them two launches: the chains of the state and of its cotangent by themselves, then every
  * segment of 64 tokens as a unit of its own.  The result is deterministic either way.
+ *
+ * With more pairs than SMs and no multiple of them, a pair that a cut falls into is begun by one CTA and finished by the
+ * next, which waits for it: a cooperative launch, as for sfda_forward's time slices.  The wait is bounded (about a second,
+ * more for long sequences; longer than any inputs take).  Where it runs out sfda_workspace_status returns
+ * SFDA_ERR_TIMEOUT, and every gradient that the waiting CTA had still to write is NaN; the others are valid.
  */
 SFDA_API size_t sfda_backward_workspace_bytes(int B, int T, int H, int d_k, int d_v, int dtype);
 SFDA_API int sfda_backward(const void *q, const void *k, const void *v,
@@ -496,6 +502,18 @@ SFDA_API int sfda_backward(const void *q, const void *k, const void *v,
                            const void *d_o, const void *d_o_im, const float *dS_T,
                            void *dq, void *dk, void *dv, float *dalpha, float *dtheta, float *dbeta, float *dS0,
                            int B, int T, int H, int d_k, int d_v, int dtype,
+                           void *workspace, size_t workspace_bytes, void *stream);
+
+/*
+ * Diagnostic: sfda_backward whose CTAs never announce what they hand over, with the wait limit set to `wait_ticks`
+ * SM-clock ticks (2^16..2^26), so that every wait runs out (see sfda_forward_withheld_handoff).  SFDA_ERR_SHAPE where no
+ * pair would be cut, SFDA_ERR_VALUE for wait_ticks out of range.  Nothing in the library calls this.
+ */
+SFDA_API int sfda_backward_withheld_handoff(const void *q, const void *k, const void *v,
+                           const float *alpha, const float *theta, const float *beta, const float *S0,
+                           const void *d_o, const void *d_o_im, const float *dS_T,
+                           void *dq, void *dk, void *dv, float *dalpha, float *dtheta, float *dbeta, float *dS0,
+                           int B, int T, int H, int d_k, int d_v, int dtype, unsigned wait_ticks,
                            void *workspace, size_t workspace_bytes, void *stream);
 
 /* Number of kernels the last sfda_forward* / sfda_step / sfda_chunk_factors / sfda_frontend call of

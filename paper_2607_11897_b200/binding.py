@@ -118,6 +118,7 @@ def load_library(path):
     lib.sfda_backward_workspace_bytes.restype = _sz
     lib.sfda_backward_workspace_bytes.argtypes = [_ci] * 6
     lib.sfda_backward.argtypes = [_vp] * 17 + [_ci] * 6 + [_vp, _sz, _vp]
+    lib.sfda_backward_withheld_handoff.argtypes = [_vp] * 17 + [_ci] * 6 + [ctypes.c_uint, _vp, _sz, _vp]
     lib.sfda_forward_two_level_workspace_bytes.restype = _sz
     lib.sfda_forward_two_level_workspace_bytes.argtypes = [_ci] * 8
     lib.sfda_forward_two_level.argtypes = [_vp] * 10 + [_ci] * 8 + [_vp, _sz, _vp]
@@ -389,6 +390,19 @@ def sfda_backward_workspace_bytes(B, T, H, d_k, d_v, dtype) -> int:
 def sfda_backward(q, k, v, alpha, theta, beta, S0, d_o, d_o_im, dS_T, dq, dk, dv, dalpha, dtheta, dbeta, dS0,
                   workspace, stream=None):
     """``sfda_backward`` of ``include/sfda.h``: gradients of a real loss through the recurrence."""
+    _backward_common("sfda_backward", (), q, k, v, alpha, theta, beta, S0, d_o, d_o_im, dS_T, dq, dk, dv, dalpha, dtheta, dbeta,
+                     dS0, workspace, stream)
+
+
+def sfda_backward_withheld_handoff(q, k, v, alpha, theta, beta, S0, d_o, d_o_im, dS_T, dq, dk, dv, dalpha, dtheta, dbeta, dS0,
+                                   wait_ticks, workspace, stream=None):
+    """``sfda_backward_withheld_handoff`` of ``include/sfda.h``: the diagnostic launch whose waits all run out."""
+    _backward_common("sfda_backward_withheld_handoff", (int(wait_ticks),), q, k, v, alpha, theta, beta, S0, d_o, d_o_im, dS_T, dq,
+                     dk, dv, dalpha, dtheta, dbeta, dS0, workspace, stream)
+
+
+def _backward_common(name, more, q, k, v, alpha, theta, beta, S0, d_o, d_o_im, dS_T, dq, dk, dv, dalpha, dtheta, dbeta, dS0,
+                     workspace, stream):
     B, T, H, d_k = q.shape
     d_v = v.shape[-1]
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (d_o, "d_o"), (d_o_im, "d_o_im"), (dq, "dq"), (dk, "dk"), (dv, "dv")):
@@ -398,12 +412,12 @@ def sfda_backward(q, k, v, alpha, theta, beta, S0, d_o, d_o_im, dS_T, dq, dk, dv
         _check(t, n, torch.float32)
     _check(workspace, "workspace")
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    rc = load().sfda_backward(_ptr(q), _ptr(k), _ptr(v), _ptr(alpha), _ptr(theta), _ptr(beta), _ptr(S0), _ptr(d_o),
-                              _ptr(d_o_im), _ptr(dS_T), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dalpha), _ptr(dtheta),
-                              _ptr(dbeta), _ptr(dS0), B, T, H, d_k, d_v, _dtype_code(q), _ptr(workspace), ws_bytes,
-                              _stream(stream))
+    rc = getattr(load(), name)(_ptr(q), _ptr(k), _ptr(v), _ptr(alpha), _ptr(theta), _ptr(beta), _ptr(S0), _ptr(d_o),
+                               _ptr(d_o_im), _ptr(dS_T), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dalpha), _ptr(dtheta),
+                               _ptr(dbeta), _ptr(dS0), B, T, H, d_k, d_v, _dtype_code(q), *more, _ptr(workspace), ws_bytes,
+                               _stream(stream))
     if rc != 0:
-        raise SfdaError(rc, "sfda_backward")
+        raise SfdaError(rc, name)
 
 
 def sfda_forward_two_level_workspace_bytes(B, T, H, d_k, d_v, chunk, dtype, n_slices=0) -> int:

@@ -681,10 +681,11 @@ size_t sfda_backward_workspace_bytes(int B, int T, int H, int d_k, int d_v, int 
     return sfda::backward_workspace_bytes(B, T, H, d_k, d_v);
 }
 
-int sfda_backward(const void *q, const void *k, const void *v, const float *alpha, const float *theta,
-                  const float *beta, const float *S0, const void *d_o, const void *d_o_im, const float *dS_T,
-                  void *dq, void *dk, void *dv, float *dalpha, float *dtheta, float *dbeta, float *dS0, int B, int T,
-                  int H, int d_k, int d_v, int dtype, void *workspace, size_t workspace_bytes, void *stream)
+static int backward_common(const void *q, const void *k, const void *v, const float *alpha, const float *theta,
+                           const float *beta, const float *S0, const void *d_o, const void *d_o_im, const float *dS_T,
+                           void *dq, void *dk, void *dv, float *dalpha, float *dtheta, float *dbeta, float *dS0, int B, int T,
+                           int H, int d_k, int d_v, int dtype, bool withhold, unsigned wait_ticks, void *workspace,
+                           size_t workspace_bytes, void *stream)
 {
     g_last_launches = 0;
     if (!q || !k || !v || !alpha || !theta || !beta || !d_o || !dq || !dk || !dv || !dalpha || !dtheta || !dbeta ||
@@ -697,15 +698,38 @@ int sfda_backward(const void *q, const void *k, const void *v, const float *alph
                           workspace};
     for (const void *p : ptrs)
         if (p && !aligned16(p)) return SFDA_ERR_ALIGN;
+    if (withhold && (wait_ticks < (1u << 16) || wait_ticks > (1u << 26))) return SFDA_ERR_VALUE;
+    if (withhold && !sfda::backward_hands_over(B, H, d_v)) return SFDA_ERR_SHAPE;
     if (!workspace || workspace_bytes < sfda::backward_workspace_bytes(B, T, H, d_k, d_v)) return SFDA_ERR_WORKSPACE;
     sfda::BackwardArgs a;
     a.q = q; a.k = k; a.v = v; a.d_o = d_o; a.d_o_im = d_o_im;
     a.alpha = alpha; a.theta = theta; a.beta = beta; a.S0 = S0; a.dS_T = dS_T;
     a.dq = dq; a.dk = dk; a.dv = dv; a.dalpha = dalpha; a.dtheta = dtheta; a.dbeta = dbeta; a.dS0 = dS0;
     a.B = B; a.T = T; a.H = H; a.d_k = d_k; a.d_v = d_v; a.dtype = dtype;
+    a.withhold = withhold;
+    a.wait_ticks = withhold ? wait_ticks : 0;
     return sfda::launch_backward(a, workspace, static_cast<cudaStream_t>(stream), &g_last_launches) == cudaSuccess
                ? SFDA_OK
                : SFDA_ERR_CUDA;
+}
+
+int sfda_backward(const void *q, const void *k, const void *v, const float *alpha, const float *theta,
+                  const float *beta, const float *S0, const void *d_o, const void *d_o_im, const float *dS_T,
+                  void *dq, void *dk, void *dv, float *dalpha, float *dtheta, float *dbeta, float *dS0, int B, int T,
+                  int H, int d_k, int d_v, int dtype, void *workspace, size_t workspace_bytes, void *stream)
+{
+    return backward_common(q, k, v, alpha, theta, beta, S0, d_o, d_o_im, dS_T, dq, dk, dv, dalpha, dtheta, dbeta, dS0, B,
+                           T, H, d_k, d_v, dtype, false, 0, workspace, workspace_bytes, stream);
+}
+
+int sfda_backward_withheld_handoff(const void *q, const void *k, const void *v, const float *alpha, const float *theta,
+                                   const float *beta, const float *S0, const void *d_o, const void *d_o_im,
+                                   const float *dS_T, void *dq, void *dk, void *dv, float *dalpha, float *dtheta,
+                                   float *dbeta, float *dS0, int B, int T, int H, int d_k, int d_v, int dtype,
+                                   unsigned wait_ticks, void *workspace, size_t workspace_bytes, void *stream)
+{
+    return backward_common(q, k, v, alpha, theta, beta, S0, d_o, d_o_im, dS_T, dq, dk, dv, dalpha, dtheta, dbeta, dS0, B,
+                           T, H, d_k, d_v, dtype, true, wait_ticks, workspace, workspace_bytes, stream);
 }
 
 int sfda_last_launch_count(void) { return g_last_launches; }

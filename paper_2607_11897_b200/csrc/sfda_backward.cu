@@ -58,8 +58,17 @@ struct BwdArgsDev {
     size_t ring_bytes;
     int T, H, NS, pitch, units;
     long long work;           // of all pairs' walks, in the units of walk_cut
+    unsigned *status;         // first word of the workspace: 1 where a wait for a piece ran out
     unsigned *flags;          // per CTA: the piece it hands on is written (null where none is)
+    unsigned long long wait_ticks;   // SM-clock ticks after which a wait gives up
+    int withhold;             // diagnostic: pieces are never announced
 };
+
+// The head of the workspace: the status word and, 256 bytes behind it, the flags of at most kBwdTargetCtas CTAs.
+constexpr int kBwdTargetCtas = 148;
+constexpr size_t kHeadBytes = 1024;
+constexpr unsigned long long kChunkTicks = 1ull << 23;           // more than any chunk takes
+static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags follow the status block");
 
 // One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
 // S_0, G_C as B operands [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U, Bc as A operands
@@ -72,7 +81,7 @@ struct BwdScratch {
     static constexpr int oV = oB + NCW * 2048, slot = oV + 16 * M * 32;
     static constexpr int oRg = slot * kSlots, oSlow = oRg + 2 * NCW * M * 8;
     static constexpr size_t bytes = (oSlow + PrepMap<DK, kPrepWarps>::slow_bytes + 255) / 256 * 256;
-    static_assert(bytes + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "ring and final state must fit a pair's scratch");
+    static_assert(kHeadBytes + bytes + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "head, ring and final state must fit a pair's scratch");
 };
 
 template <int DK, int NB>
@@ -717,9 +726,9 @@ __device__ __forceinline__ void read_piece(const float4 *p, float (&x)[16])
     }
 }
 
-// A kept state back into tensor memory (NaN if the CTA that writes it was given up); this thread's largest entry
+// A kept state back into tensor memory; this thread's largest entry
 template <int DK>
-__device__ __forceinline__ float state_from_kept(uint32_t st, const float4 *p, bool gave_up)
+__device__ __forceinline__ float state_from_kept(uint32_t st, const float4 *p)
 {
     float largest = 0.f;
 #pragma unroll 1
@@ -727,10 +736,7 @@ __device__ __forceinline__ float state_from_kept(uint32_t st, const float4 *p, b
         float x[16];
         read_piece(p, x);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            if (gave_up) x[i] = __int_as_float(0x7fc00000);
-            largest = fmaxf(largest, fabsf(x[i]));
-        }
+        for (int i = 0; i < 16; ++i) largest = fmaxf(largest, fabsf(x[i]));
         tm_store(st + 16 * n, x);
     }
     tm_wait_store();
@@ -1035,6 +1041,10 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_backward_
 // first thing it does, and finished by the next one, as its last: S or G goes from one to the other through the place of
 // the kept final state, and a CTA only waits for what the CTA before it in the grid does first.  256 pairs of 8192 tokens
 // on 148 SMs, with the forward and the passes around it: 30.5 ms as two rounds of whole pairs, 27.5 ms cut.
+// The launch is cooperative, so that both CTAs run, and the wait is bounded by what the other's part can take at most: a
+// chunk takes 57 k cycles, and up to 6.4 M where every alpha is below 1/16.  Where it runs out all the same, the status
+// word is set and the part is not walked: its gradients become NaN.  (Signs of life instead of a bound, one store per
+// segment, cost 1.3 % of the walk, in the chain's warps as in the gradients'.)
 // kUnits == true: S and G are kept already; a CTA takes units (pair, segment) blockIdx.x, + gridDim.x, ...
 // Either way the second sweep is a list of segments, each of kSegChunks chunks (a ragged last one is completed with
 // neutral tokens), pipelined over its borders.
@@ -1064,6 +1074,24 @@ __device__ __forceinline__ int3 walk_part(long long work, int c, int ctas, int N
     return make_int3(-1, 0, 0);
 }
 
+// NaN for every gradient of the first `tokens` tokens of pair bh and for dS0, by all threads of the CTA
+template <int DK, int NB, typename T>
+__device__ __forceinline__ void give_up(const BwdArgsDev &a, int bh, int tokens, int tid, int threads)
+{
+    const float nan = __int_as_float(0x7fc00000);
+    const size_t row0 = (size_t)(bh / a.H) * a.T * a.H + bh % a.H;
+    for (int i = tid; i < tokens * DK; i += threads) {
+        const size_t row = row0 + (size_t)(i / DK) * a.H;
+        const int x = i % DK;
+        st_val(static_cast<T *>(a.dq), row * DK + x, nan);
+        st_val(static_cast<T *>(a.dk), row * DK + x, nan);
+        if (x < DK / 2) a.dalpha[row * (DK / 2) + x] = a.dtheta[row * (DK / 2) + x] = nan;
+        if (x == 0) a.dbeta[row] = nan;
+    }
+    for (int i = tid; i < tokens * NB; i += threads) st_val(static_cast<T *>(a.dv), (row0 + (size_t)(i / NB) * a.H) * NB + i % NB, nan);
+    for (int i = tid; i < DK * NB; i += threads) a.dS0[(size_t)bh * DK * NB + i] = nan;
+}
+
 template <int DK, int NB, typename T, bool kUnits>
 __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kernel(const BwdArgsDev a)
 {
@@ -1083,18 +1111,25 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
         bar_sync(0, kGrad + kPrep + kChain);
         if (tid == 0) {
             // the first part is what the next CTA waits for
-            if (j == 1 && a.flags) asm volatile("fence.acq_rel.gpu;\n\tst.relaxed.gpu.global.u32 [%0], 1;" ::"l"(a.flags + blockIdx.x) : "memory");
+            if (j == 1 && a.flags && !a.withhold) asm volatile("fence.acq_rel.gpu;\n\tst.relaxed.gpu.global.u32 [%0], 1;" ::"l"(a.flags + blockIdx.x) : "memory");
             const int3 p = walk_part(a.work, blockIdx.x, gridDim.x, NS, j);
             int gave_up = 0;
-            if (p.x >= 0 && p.y) {                                       // about a second at most
-                uint32_t seen;
-                const uint32_t t0 = (uint32_t)clock();
-                do {
+            if (p.x >= 0 && p.y) {
+                uint32_t seen, before = (uint32_t)clock();
+                unsigned long long spent = 0;
+                while (true) {
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.flags + blockIdx.x - 1) : "memory");
                     if (seen) break;
+                    const uint32_t now = (uint32_t)clock();
+                    spent += min(now - before, 1u << 16);                // (a pause of the whole SM counts as one look)
+                    before = now;
+                    if (spent >= a.wait_ticks) {
+                        gave_up = 1;
+                        atomicOr(a.status, 1u);
+                        break;
+                    }
                     __nanosleep(200);
-                } while ((uint32_t)clock() - t0 < 0x80000000u);
-                gave_up = !seen;
+                }
                 __threadfence();
             }
             job[0] = p.x;
@@ -1103,7 +1138,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
             job[3] = gave_up;
         }
         bar_sync(0, kGrad + kPrep + kChain);
-        return job[0] >= 0;
+        return job[0] >= 0 && !job[3];                                   // (only the last part can be given up)
     };
     auto segments_of = [&] { return kUnits ? (a.units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : max(0, job[2] - max(job[1], NS)); };
     // the r-th segment of this CTA's list: pair and segment; row of token t of a pair: row0 + t H
@@ -1118,6 +1153,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
         }
     };
     auto row_of = [&](int bh) { return (size_t)(bh / a.H) * a.T * a.H + bh % a.H; };
+    if (!a.flags && blockIdx.x == 0 && tid == 0) *a.status = 0;          // nothing waits (else the launcher has cleared it)
     if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::word), L::columns);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -1221,11 +1257,11 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
             const int from = kUnits ? 0 : job[1], to = kUnits ? 0 : job[2], c0 = r < 0 ? from * kSegChunks : 0;
             if (r < 0) {
                 if (from >= NS) continue;
-                big_s = from ? state_from_kept<DK>(ss, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), job[3])
+                big_s = from ? state_from_kept<DK>(ss, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane))
                              : state_from_memory<DK>(ss, a.S0 ? a.S0 + state_at : nullptr, NB);
             } else {
                 if (!kUnits && r == 0)
-                    big_g = from > NS ? state_from_kept<DK>(sg, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), job[3])
+                    big_g = from > NS ? state_from_kept<DK>(sg, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane))
                                       : state_from_memory<DK>(sg, a.dS_T ? a.dS_T + state_at : nullptr, NB);
                 // rowdot(conj S, G) at the segment's end, this warp's columns; then S at its start
                 float2 *rg = rgs + ((r & 1) * NCW + w) * M + 2 * t4;
@@ -1300,6 +1336,9 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
             }
         }
     }
+    if constexpr (!kUnits) {
+        if (job[3]) give_up<DK, NB, T>(a, job[0], min(a.T, (2 * NS - max(job[1], NS)) * kSeg), tid, kGrad + kPrep + kChain);
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (tid < 32) tm_free(tmem, L::columns);
@@ -1308,8 +1347,6 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
 // Blocks of value columns of the two chains: all of them while the (batch, head) pairs alone fill the SMs (then there is
 // only the walk with gradients, one CTA per pair); with few sequences 64 or 32.  (A fixed count rather than the
 // device's: the workspace size must not depend on where it is asked for.)
-constexpr int kBwdTargetCtas = 148;
-
 int bwd_cols(int B, int H, int d_v)
 {
     int cols = d_v;
@@ -1331,9 +1368,19 @@ template <int DK, int DV, typename T, bool kUnits>
 cudaError_t launch_walk(const BwdArgsDev &a, int grid, cudaStream_t stream, int *launches)
 {
     auto kern = sfda_backward_kernel<DK, DV, T, kUnits>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BwdSmem<DK, DV>::bytes);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BwdSmem<DK, DV>::bytes);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kGrad + kPrep + 2 * DV, BwdSmem<DK, DV>::bytes, stream>>>(a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kGrad + kPrep + 2 * DV);
+    cfg.dynamicSmemBytes = BwdSmem<DK, DV>::bytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = a.flags ? 1 : 0;                   // CTAs that wait for one another run together (one per SM)
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if ((e = cudaLaunchKernelEx(&cfg, kern, a)) != cudaSuccess) return e;
     if (launches) ++*launches;
     return cudaGetLastError();
 }
@@ -1355,7 +1402,7 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     using SC = BwdScratch<DK, DV>;
     const size_t state = (size_t)DK * DV;
     const int pairs = x.B * x.H, cols = bwd_cols(x.B, x.H, DV);
-    float *ws = static_cast<float *>(workspace);
+    float *ws = reinterpret_cast<float *>(static_cast<char *>(workspace) + kHeadBytes);
     BwdArgsDev a;
     a.q = x.q; a.k = x.k; a.v = x.v; a.d_o = x.d_o; a.d_o_im = x.d_o_im;
     a.alpha = x.alpha; a.theta = x.theta; a.beta = x.beta; a.S0 = x.S0; a.dS_T = x.dS_T;
@@ -1366,21 +1413,31 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     a.pitch = a.NS + 1;
     a.keep_g = ws + (size_t)pairs * a.pitch * state;
     a.ring_bytes = SC::bytes;
+    a.status = static_cast<unsigned *>(workspace);
+    a.flags = nullptr;
+    a.wait_ticks = x.wait_ticks ? x.wait_ticks : 1ull << 31;     // about a second, more for long sequences
+    if (!x.wait_ticks && (unsigned long long)a.NS * kSegChunks * kChunkTicks > a.wait_ticks) a.wait_ticks = (unsigned long long)a.NS * kSegChunks * kChunkTicks;
+    a.withhold = x.withhold;
     if (cols == DV) {
-        const int grid = pairs < kBwdTargetCtas ? pairs : kBwdTargetCtas;
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        const int most = sms < kBwdTargetCtas ? sms : kBwdTargetCtas, grid = pairs < most ? pairs : most;
         a.ring = reinterpret_cast<unsigned char *>(a.keep_g);
         a.work = (long long)pairs * a.NS * (kSweepCost + kBackCost);
-        a.flags = nullptr;
-        if (pairs % grid) {                                      // behind the rings: a pair has room for one, a CTA uses it
-            a.flags = reinterpret_cast<unsigned *>(a.ring + (size_t)grid * SC::bytes);
-            const cudaError_t e = cudaMemsetAsync(a.flags, 0, grid * sizeof(unsigned), stream);
-            if (e != cudaSuccess) return e;
+        if (pairs % grid) {
+            a.flags = a.status + 64;
+            if ((e = cudaMemsetAsync(a.status, 0, kHeadBytes, stream)) != cudaSuccess) return e;
+        } else if (a.withhold) {
+            return cudaErrorInvalidValue;                        // no pair is cut
         }
         return launch_walk<DK, DV, T, false>(a, grid, stream, launches);
     }
+    if (a.withhold) return cudaErrorInvalidValue;
     float *rings = a.keep_g + (size_t)pairs * a.pitch * state;
     a.ring = reinterpret_cast<unsigned char *>(rings);
-    const size_t room = (bwd_workspace(x.B, x.T, x.H, DK, DV) - (size_t)(rings - ws)) * sizeof(float) / SC::bytes;
+    const size_t room = (bwd_workspace(x.B, x.T, x.H, DK, DV) * sizeof(float) - kHeadBytes - (size_t)(rings - ws) * sizeof(float)) / SC::bytes;
     int grid = a.units < kBwdTargetCtas ? a.units : kBwdTargetCtas;
     if ((size_t)grid > room) grid = (int)room;
     // both chains of all pairs at once: the columns are cut while that still fits the SMs
@@ -1394,6 +1451,12 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
 }
 
 }  // namespace
+
+bool backward_hands_over(int B, int H, int d_v)
+{
+    const long long pairs = (long long)B * H;
+    return bwd_cols(B, H, d_v) == d_v && pairs > kBwdTargetCtas && pairs % kBwdTargetCtas != 0;
+}
 
 size_t backward_workspace_bytes(int B, int T, int H, int d_k, int d_v)
 {

@@ -78,6 +78,10 @@ struct BackwardArgs {
     void *dq, *dk, *dv;
     float *dalpha, *dtheta, *dbeta, *dS0;
     int B, T, H, d_k, d_v, dtype;
+    // diagnostic launches: wait limit in SM-clock ticks (0: about a second), and hand-overs between CTAs that are written
+    // but never announced
+    uint32_t wait_ticks = 0;
+    int withhold = 0;
 };
 
 struct DecoupledArgs {
@@ -119,8 +123,9 @@ cudaError_t launch_step(const StepArgs &a, cudaStream_t stream, int *launches);
 bool forward_two_level_supported(const ForwardArgs &a, int n);
 size_t forward_two_level_bytes(const ForwardArgs &a, int n);
 cudaError_t launch_forward_two_level(const ForwardArgs &a, int n, void *workspace, cudaStream_t stream, int *launches);
-// Reverse-mode derivative, token by token in fp32 (every supported d_k, d_v and dtype); the workspace holds the
-// checkpointed states.
+// Reverse-mode derivative at fp32 precision (every supported d_k, d_v and dtype); the workspace begins with the status
+// word and holds the kept states and scratch rings.
+bool backward_hands_over(int B, int H, int d_v);   // pairs are cut between CTAs
 size_t backward_workspace_bytes(int B, int T, int H, int d_k, int d_v);
 cudaError_t launch_backward(const BackwardArgs &a, void *workspace, cudaStream_t stream, int *launches);
 // Forward of the write-decoupled variant, token by token in fp32 (every supported d_k, d_v and dtype).

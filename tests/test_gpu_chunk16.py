@@ -9,6 +9,7 @@ import workloads
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 if torch.cuda.is_available():
+    import paper_2607_11897_b200 as sfda
     from tests.test_gpu_parity import all_pairs, check_backward, check_forward, upstream
 
 # Operands keep 22 bits and the products of their tails (2^-22) are left out; sums are fp32 over at most 128 terms,
@@ -58,3 +59,84 @@ def test_backward_of_pairs_shared_by_two_blocks(B, H, T, d_k, d_v, im):
                                       seed=500 + T + H)
     pairs = all_pairs(cfg)
     check_backward(cfg, workloads.forward_inputs(cfg), upstream(cfg, T, want_im=im), pairs[::19] + pairs[-2:], BWD_TOL)
+
+
+GRADS = ("dq", "dk", "dv", "dalpha", "dtheta", "dbeta", "dS0")
+
+
+def backward_tensors(cfg, inp, up):
+    dev = lambda x: None if x is None else torch.from_numpy(np.ascontiguousarray(x)).cuda()  # noqa: E731
+    x = [dev(inp[n]) for n in ("q", "k", "v", "alpha", "theta", "beta", "S0")]
+    u = [dev(up[n]) for n in ("do_re", "do_im", "dS_T")]
+    ws = torch.ones(sfda.sfda_backward_workspace_bytes(cfg.B, cfg.T, cfg.H, cfg.d_k, cfg.d_v, 0) // 4, device="cuda")   # plausible leftovers
+    return x, u, [torch.zeros_like(t) for t in x], ws
+
+
+@pytest.mark.parametrize("H,T,d_k", [(149, 300, 128), (200, 64, 64), (256, 130, 64)])
+def test_a_wait_for_another_blocks_piece_that_runs_out(H, T, d_k):
+    """Nothing is announced: every block that finishes another's pair gives up.  The call's status says so, a gradient is NaN or
+    that of the ordinary call, and whatever depends on the missing piece is NaN.  200 pairs of one segment are cut at the
+    turning point, 256 of three segments within both sweeps as well."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16w", B=1, T=T, H=H, d_k=d_k, d_v=64, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=600 + H)
+    x, u, out, ws = backward_tensors(cfg, workloads.forward_inputs(cfg), upstream(cfg, T))
+    with pytest.raises(sfda.SfdaError) as e:
+        sfda.sfda_backward_withheld_handoff(*x, *u, *out, 1 << 20, ws)
+        sfda.sfda_workspace_status(ws)
+    assert e.value.status == -7
+    lost = [t.clone() for t in out]
+    sfda.sfda_backward(*x, *u, *out, ws)
+    assert sfda.sfda_workspace_status(ws) == 0
+    NS = (T + 63) // 64
+    cut = set()                                        # pairs that a cut of the walks falls into, and where
+    for c in range(1, 148):
+        at = H * NS * 9 * c // 148
+        pair, rest = divmod(at, 9 * NS)
+        pos = rest // 2 if rest < 2 * NS else NS + (rest - 2 * NS) // 7
+        if pos:
+            cut.add((pair, pos))
+    for name, a, b in zip(GRADS, lost, out):
+        assert torch.isfinite(b).all(), name
+        gone = torch.isnan(a)
+        assert torch.equal(torch.where(gone, b, a), b), name
+        for h in range(H):
+            at = [pos for pair, pos in cut if pair == h]
+            g = gone[0, h] if name == "dS0" else gone[0, :, h]
+            if not at:
+                assert not g.any(), (name, h)
+            elif name == "dS0":
+                assert g.all(), (name, h)
+            else:                                      # the segments that the second block had still to write
+                left = 64 * (2 * NS - max(max(at), NS))
+                assert g[:left].all() and not g[left:].any(), (name, h, at)
+    for ticks, code in ((1 << 10, -8), (1 << 30, -8)):
+        with pytest.raises(sfda.SfdaError) as e:
+            sfda.sfda_backward_withheld_handoff(*x, *u, *out, ticks, ws)
+        assert e.value.status == code
+
+
+def test_nothing_is_handed_over_where_no_pair_is_cut():
+    cfg = workloads.CONFIGS[0].scaled(name="c16n", B=1, T=64, H=2, d_k=64, d_v=64, chunk=64, s0_std=0.5, seed=610)
+    x, u, out, ws = backward_tensors(cfg, workloads.forward_inputs(cfg), upstream(cfg, 1))
+    with pytest.raises(sfda.SfdaError) as e:
+        sfda.sfda_backward_withheld_handoff(*x, *u, *out, 1 << 20, ws)
+    assert e.value.status == -2
+    sfda.sfda_backward(*x, *u, *out, ws)
+    assert sfda.sfda_workspace_status(ws) == 0         # also where nothing waits
+
+
+def test_backward_of_cut_pairs_is_deterministic_beside_other_work():
+    cfg = workloads.CONFIGS[0].scaled(name="c16d", B=1, T=200, H=201, d_k=128, d_v=128, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=611)
+    x, u, out, ws = backward_tensors(cfg, workloads.forward_inputs(cfg), upstream(cfg, 2))
+    sfda.sfda_backward(*x, *u, *out, ws)
+    want = [t.clone() for t in out]
+    side, m = torch.cuda.Stream(), torch.randn(4096, 4096, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(4):
+        with torch.cuda.stream(side):
+            for _ in range(6):
+                m = torch.tanh(m @ m)
+        sfda.sfda_backward(*x, *u, *out, ws)
+        assert sfda.sfda_workspace_status(ws) == 0
+        for name, a, b in zip(GRADS, out, want):
+            assert torch.equal(a, b), name
+    torch.cuda.synchronize()
