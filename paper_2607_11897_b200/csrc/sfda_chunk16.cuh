@@ -78,6 +78,56 @@ __device__ __forceinline__ float2 unpack_f16(uint32_t x)
     asm("{\n.reg .b16 a, b;\nmov.b32 {a, b}, %2;\ncvt.f32.f16 %0, a;\ncvt.f32.f16 %1, b;\n}" : "=f"(r.x), "=f"(r.y) : "r"(x));
     return r;
 }
+// re += Re(conj(b) a), im += Im(conj(b) a) for split complex operands (h: head, l: tail) and NT column tiles of b, tile n in
+// registers 2 n and 2 n + 1.  An accumulator's next product is at least four instructions away, b's tails come first (their
+// registers are free after a third of the products).  Two accumulators less by negating b's imaginary part: 543 us
+// instead of 422 for the fp32 forward at B = 2, T = 2001, H = 16.
+//
+// The tensor core truncates its sums: with all 24 products of a 64-key sum in one accumulator the outputs were 1.7 times as
+// far from 64-bit arithmetic as with sums rounded to nearest (5.3e-7, the CUDA-core kernel 3.1e-7).  So 16 keys at a time
+// start from zero, small terms first, and are added with fp32 additions: 2.1e-7.  (415 -> 422 us at those sizes.)
+template <int NT>
+__device__ __forceinline__ void add_products(float (&re)[NT][4], float (&im)[NT][4], const uint32_t (&arh)[4], const uint32_t (&arl)[4],
+                                             const uint32_t (&aih)[4], const uint32_t (&ail)[4], const uint32_t (&brh)[2 * NT],
+                                             const uint32_t (&brl)[2 * NT], const uint32_t (&bih)[2 * NT], const uint32_t (&bil)[2 * NT])
+{
+    float x[NT][4], y[NT][4], z[NT][4], x2[NT][4];                 // Ar Br (+ Ai Bi), Ai Br, Ar Bi; one tile: Ai Bi by itself
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t(&ar)[4] = k == 1 ? arl : arh;
+        const uint32_t(&ai)[4] = k == 1 ? ail : aih;
+        const uint32_t(&br)[2 * NT] = k == 0 ? brl : brh;
+        const uint32_t(&bi)[2 * NT] = k == 0 ? bil : bih;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            if (k == 0) mma_f16_z(x[n], ar, br[2 * n], br[2 * n + 1]);
+            else mma_f16(x[n], ar, br[2 * n], br[2 * n + 1]);
+        }
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            if (k == 0) mma_f16_z(y[n], ai, br[2 * n], br[2 * n + 1]);
+            else mma_f16(y[n], ai, br[2 * n], br[2 * n + 1]);
+        }
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            if (NT > 1) mma_f16(x[n], ai, bi[2 * n], bi[2 * n + 1]);
+            else if (k == 0) mma_f16_z(x2[n], ai, bi[2 * n], bi[2 * n + 1]);
+            else mma_f16(x2[n], ai, bi[2 * n], bi[2 * n + 1]);
+        }
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            if (k == 0) mma_f16_z(z[n], ar, bi[2 * n], bi[2 * n + 1]);
+            else mma_f16(z[n], ar, bi[2 * n], bi[2 * n + 1]);
+        }
+    }
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            re[n][i] += NT > 1 ? x[n][i] : x[n][i] + x2[n][i];
+            im[n][i] += y[n][i] - z[n][i];
+        }
+}
 // head and tail of two values (already scaled)
 __device__ __forceinline__ void split_f16(float x, float y, uint32_t &h, uint32_t &l)
 {
@@ -182,17 +232,17 @@ struct Tile {
 
 // ---- CHAIN --------------------------------------------------------------------------------------
 // acc[x] = products conj(X_x)^T S of NX tiles with the state at `st`, value channels in rows, tokens in columns, for
-// each of two token tiles: [0] = Xr Sr + Xi Si, [1] = Xr Si, [2] = Xi Sr (Im = [1] - [2]); scaled by s and the tiles'
-// scales.  pub(kk, rh, rl, ih, il) sees the split state of every step.
+// each of two token tiles: [0] = Re = Xr Sr + Xi Si, [1] = Im = Xr Si - Xi Sr; scaled by s and the tiles' scales.
+// pub(kk, rh, rl, ih, il) sees the split state of every step.
 template <int DK, int NX, typename Pub>
-__device__ __forceinline__ void keys_product(float (&acc)[NX][3][2][4], uint32_t st, float s, const uint32_t (&tile)[NX],
+__device__ __forceinline__ void keys_product(float (&acc)[NX][2][2][4], uint32_t st, float s, const uint32_t (&tile)[NX],
                                              int lane, Pub pub)
 {
     using TL = Tile<DK>;
 #pragma unroll
     for (int x = 0; x < NX; ++x)
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+        for (int c = 0; c < 2; ++c)
 #pragma unroll
             for (int n = 0; n < 2; ++n)
 #pragma unroll
@@ -213,25 +263,20 @@ __device__ __forceinline__ void keys_product(float (&acc)[NX][3][2][4], uint32_t
         for (int t = 0; t < NX; ++t) {
             uint32_t brh[4], brl[4], bih[4], bil[4];
             const uint32_t p = tile[t] + at;
-            ldsm(brh, p);
-            ldsm(bih, p + 2 * TL::PL);
             ldsm(brl, p + TL::PL);
             ldsm(bil, p + 3 * TL::PL);
-            // an accumulator's next product is four instructions away
+            ldsm(brh, p);
+            ldsm(bih, p + 2 * TL::PL);
+            if constexpr (NX == 1) {                              // (a column tile at a time: eight registers fewer)
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const uint32_t(&ar)[4] = k == 0 ? rl : rh;
-                const uint32_t(&ai)[4] = k == 0 ? il : ih;
-                const uint32_t(&br)[4] = k == 1 ? brl : brh;
-                const uint32_t(&bi)[4] = k == 1 ? bil : bih;
-#pragma unroll
-                for (int n = 0; n < 2; ++n) mma_f16(acc[t][0][n], ar, br[2 * n], br[2 * n + 1]);
-#pragma unroll
-                for (int n = 0; n < 2; ++n) mma_f16(acc[t][1][n], ai, br[2 * n], br[2 * n + 1]);
-#pragma unroll
-                for (int n = 0; n < 2; ++n) mma_f16(acc[t][0][n], ai, bi[2 * n], bi[2 * n + 1]);
-#pragma unroll
-                for (int n = 0; n < 2; ++n) mma_f16(acc[t][2][n], ar, bi[2 * n], bi[2 * n + 1]);
+                for (int n = 0; n < 2; ++n) {
+                    const uint32_t h0[2] = {brh[2 * n], brh[2 * n + 1]}, l0[2] = {brl[2 * n], brl[2 * n + 1]};
+                    const uint32_t h1[2] = {bih[2 * n], bih[2 * n + 1]}, l1[2] = {bil[2 * n], bil[2 * n + 1]};
+                    add_products<1>(reinterpret_cast<float(&)[1][4]>(acc[t][0][n]), reinterpret_cast<float(&)[1][4]>(acc[t][1][n]), rh, rl,
+                                    ih, il, h0, l0, h1, l1);
+                }
+            } else {
+                add_products<2>(acc[t][0], acc[t][1], rh, rl, ih, il, brh, brl, bih, bil);
             }
         }
         if (more) tm_wait_load(x);
@@ -734,11 +779,11 @@ __device__ __forceinline__ void gram_tiles(uint32_t x, uint32_t kb, float f, flo
     uint32_t pa = x + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
     // B registers of both halves of a k-step for the heads (lanes 0-15) and the tails (lanes 16-31)
     uint32_t pb = kb + (uint32_t)((8 * nt0 + (lane & 7)) * TL::LDB + ((lane >> 3) & 1) * 16 + (lane >> 4) * TL::PL);
-    float re[NT][4], im[NT][4], ni[NT][4];
+    float re[NT][4], im[NT][4];                     // im: of a conj(b), negated at the end
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) re[n][i] = im[n][i] = ni[n][i] = 0.f;
+        for (int i = 0; i < 4; ++i) re[n][i] = im[n][i] = 0.f;
 #pragma unroll 1
     for (int kk = 0; kk < TL::KS; ++kk, pa += 32, pb += 32) {
         uint32_t rh[4], rl[4], ih[4], il[4], br[NT][4], bi[NT][4];
@@ -751,26 +796,23 @@ __device__ __forceinline__ void gram_tiles(uint32_t x, uint32_t kb, float f, flo
             ldsm(br[n], pb + n * 8 * TL::LDB);
             ldsm(bi[n], pb + n * 8 * TL::LDB + 2 * TL::PL);
         }
+        uint32_t brh[2 * NT], brl[2 * NT], bih[2 * NT], bil[2 * NT];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const uint32_t(&ar)[4] = k == 0 ? rl : rh;
-            const uint32_t(&ai)[4] = k == 0 ? il : ih;
-            const int o = k == 1 ? 2 : 0;
+        for (int n = 0; n < NT; ++n)
 #pragma unroll
-            for (int n = 0; n < NT; ++n) mma_f16(re[n], ar, br[n][o], br[n][o + 1]);
-#pragma unroll
-            for (int n = 0; n < NT; ++n) mma_f16(im[n], ar, bi[n][o], bi[n][o + 1]);
-#pragma unroll
-            for (int n = 0; n < NT; ++n) mma_f16(re[n], ai, bi[n][o], bi[n][o + 1]);
-#pragma unroll
-            for (int n = 0; n < NT; ++n) mma_f16(ni[n], ai, br[n][o], br[n][o + 1]);
-        }
+            for (int i = 0; i < 2; ++i) {
+                brh[2 * n + i] = br[n][i];
+                brl[2 * n + i] = br[n][2 + i];
+                bih[2 * n + i] = bi[n][i];
+                bil[2 * n + i] = bi[n][2 + i];
+            }
+        add_products<NT>(re, im, rh, rl, ih, il, brh, brl, bih, bil);
     }
     out += g * 17 + 8 * nt0 + 2 * t4;
 #pragma unroll
     for (int n = 0; n < NT; ++n)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) out[8 * 17 * (i >> 1) + 8 * n + (i & 1)] = make_float2(f * re[n][i], f * (im[n][i] - ni[n][i]));
+        for (int i = 0; i < 4; ++i) out[8 * 17 * (i >> 1) + 8 * n + (i & 1)] = make_float2(f * re[n][i], -f * im[n][i]);
 }
 
 // Inverse of I + N (16 x 16 complex, [17] float2 rows, only the strictly lower part of N is read) by one warp, in place:

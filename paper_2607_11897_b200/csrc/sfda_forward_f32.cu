@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
             bar_sync(kBarFull + slot, 64 + kChain);
             const uint32_t tile = base + slot * TL::bytes;
             const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
-            float acc[2][3][2][4];
+            float acc[2][2][2][4];
             const uint32_t tiles[2] = {tile + TL::oW, tile + TL::oQ};
             keys_product<DK, 2>(acc, st, ss, tiles, lane, [](int, const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4]) {});
             const float fw = isv * inv[0], fq = isv * inv[2];
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
-                    ri[n][i] = -fw * (acc[0][1][n][i] - acc[0][2][n][i]);
+                    ri[n][i] = -fw * acc[0][1][n][i];
                 }
             TokFrag fr;
             float iu;
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     rr[n][i] = fmaf(fq, acc[1][0][n][i], rr[n][i]);
-                    ri[n][i] = -fmaf(fq, acc[1][1][n][i] - acc[1][2][n][i], ri[n][i]);
+                    ri[n][i] = -fmaf(fq, acc[1][1][n][i], ri[n][i]);
                 }
             store_rows(static_cast<T *>(a.o) + at, rr, step, left);
             if (a.o_im) store_rows(static_cast<T *>(a.o_im) + at, ri, step, left);

@@ -10,7 +10,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 if torch.cuda.is_available():
     import paper_2607_11897_b200 as sfda
-    from tests.test_gpu_parity import all_pairs, check_backward, check_forward, upstream
+    from tests.test_gpu_parity import all_pairs, check_backward, check_forward, oracle_pairs, run_forward, upstream
 
 # Operands keep 22 bits and the products of their tails (2^-22) are left out; sums are fp32 over at most 128 terms,
 # carried over chunks by a contraction.  That is a few 1e-7 of a tensor's largest entry (8e-7 measured); ten times that.
@@ -140,3 +140,19 @@ def test_backward_of_cut_pairs_is_deterministic_beside_other_work():
         for name, a, b in zip(GRADS, out, want):
             assert torch.equal(a, b), name
     torch.cuda.synchronize()
+
+
+def distance(got, want):
+    return np.linalg.norm(got - want) / np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("B,H,d_k,d_v,T", [(1, 2, 128, 128, 700), (1, 2, 64, 64, 333), (5, 16, 128, 64, 200), (5, 32, 128, 128, 100)])
+def test_fp32_forward_is_as_close_to_64_bits_as_the_cuda_core_kernel(B, H, d_k, d_v, T):
+    """Relative 2-norm; both differ from 64-bit arithmetic by roundings alone (3e-7), 5 % for their scatter."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16p", B=B, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="sigmoid(n(3,1))", s0_std=0.02, seed=700 + T)
+    inp = workloads.forward_inputs(cfg)
+    pairs = all_pairs(cfg)[:4]
+    want = oracle_pairs(inp, pairs)
+    pick = lambda out: [np.stack([x[b, :, h] if i < 2 else x[b, h] for b, h in pairs]) for i, x in enumerate(out[:3])]  # noqa: E731
+    for a, b, w in zip(pick(run_forward(cfg, inp)), pick(run_forward(cfg, inp, simt=True)), want):
+        assert distance(a, w) <= 1.05 * distance(b, w)
