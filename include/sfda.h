@@ -140,7 +140,9 @@ SFDA_API int sfda_forward_partition(int B, int T, int H, int d_k, int d_v, int c
  * bf16 inputs with d_k = d_v = 128 and chunk >= 64 take the tensor-core path
  * (bf16 operands, fp32 accumulation and state); everything else runs at fp32
  * precision (products of operands split into two fp16 parts, 22 bits, summed in
- * fp32; any alpha in [0, 1]).  The bf16 tensor-core path forms 1/gamma_t inside a chunk and so
+ * fp32; any alpha in [0, 1]).  Those 22 bits count from the largest entry of a value channel (over the keys, or over
+ * 16 tokens) and of the keys and queries of 16 tokens; an entry 2^-16 and more below that has an absolute error of
+ * 2^-39 of it.  The bf16 tensor-core path forms 1/gamma_t inside a chunk and so
  * additionally assumes prod_{t in chunk} alpha_{t,j} >= exp(-80) for every
  * coordinate j; beyond that results lose accuracy but stay finite.
  */
@@ -486,7 +488,8 @@ SFDA_API int sfda_forward_fused(const void *q, const void *k_raw, const void *v,
  *               the status word that sfda_workspace_status reads.
  *
  * d_k, d_v in {64, 128}; no chunk argument (the derivative does not depend on the chunking).  fp32 precision on the
- * tensor cores in chunks of 16 tokens, as the fp32 forward.  One launch, one CTA per (batch, head) pair, or one per SM
+ * tensor cores in chunks of 16 tokens, as the fp32 forward; the sums over the value columns (dq, dk, dalpha, dtheta,
+ * dbeta) count their 22 bits from the largest entries of 16 columns.  One launch, one CTA per (batch, head) pair, or one per SM
  * with an equal piece of the pairs' walks where there are more pairs than the 148 SMs of a B200; when B * H is at most
  * half of them two launches: the chains of the state and of its cotangent by themselves, then every
  * segment of 64 tokens as a unit of its own.  The result is deterministic either way.

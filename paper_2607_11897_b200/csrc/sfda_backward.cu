@@ -117,16 +117,22 @@ __device__ __forceinline__ void mma3x(float (&d)[4], const uint32_t (&ah)[4], co
     mma_f16(d, ah, bh0, bh1);
 }
 
-// the [value x token] operand as the A operand (token, value) of products over the value columns
-__device__ __forceinline__ void publish_frag(uint4 *p, const TokFrag &f, int lane)
+// the [value x token] operand as the A operand (token, value) of products over the value columns, at their
+// shared scale, whose inverse is returned
+__device__ __forceinline__ float publish_frag(uint4 *p, const TokFrag &f, const RowScale &r, int lane)
 {
-    auto put = [&](int plane, const uint32_t(&x)[4]) {
+    bool own;
+    const float all = shared_scale(r, own);                      // (nearly always some row has another)
+    auto put = [&](int plane, const uint32_t(&v)[4]) {
+        uint32_t x[4] = {v[0], v[1], v[2], v[3]};
+        to_shared_scale(x, r, all);
         p[plane * 32 + lane] = make_uint4(transpose8x8(x[0]), transpose8x8(x[2]), transpose8x8(x[1]), transpose8x8(x[3]));
     };
     put(0, f.rh);
     put(1, f.rl);
     put(2, f.ih);
     put(3, f.il);
+    return all;
 }
 
 __device__ __forceinline__ void st_val4(float *p, float4 x) { *reinterpret_cast<float4 *>(p) = x; }
@@ -289,6 +295,16 @@ __device__ __forceinline__ void stage_tokens(const BwdArgsDev &a, unsigned char 
         for (int p = 0; p < 4; ++p) {
             frag[((NCW + w) * 4 + p) * 32 + lane] = x[p];
             frag[((2 * NCW + w) * 4 + p) * 32 + lane] = x[4 + p];
+        }
+        if (__any_sync(0xffffffffu, m > 3.402823466e38f)) {              // an infinity does not decide the others' scale
+            m = 0.f;
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float ax = fabsf(y[c][i].x), ay = fabsf(y[c][i].y);
+                    m = fmaxf(m, fmaxf(ax <= 3.402823466e38f ? ax : 0.f, ay <= 3.402823466e38f ? ay : 0.f));
+                }
         }
         float inv;
         const float s = scale_for(warp_max(m), inv);
@@ -726,17 +742,16 @@ __device__ __forceinline__ void read_piece(const float4 *p, float (&x)[16])
     }
 }
 
-// A kept state back into tensor memory; this thread's largest entry
+// A kept state back into tensor memory; the largest entries of this thread's rows
 template <int DK>
-__device__ __forceinline__ float state_from_kept(uint32_t st, const float4 *p)
+__device__ __forceinline__ float2 state_from_kept(uint32_t st, const float4 *p)
 {
-    float largest = 0.f;
+    float2 largest = make_float2(0.f, 0.f);
 #pragma unroll 1
     for (int n = 0; n < Tile<DK>::KS; ++n, p += 128) {
         float x[16];
         read_piece(p, x);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) largest = fmaxf(largest, fabsf(x[i]));
+        largest = max_abs(reinterpret_cast<const float(&)[4][4]>(x), largest);
         tm_store(st + 16 * n, x);
     }
     tm_wait_store();
@@ -744,13 +759,34 @@ __device__ __forceinline__ float state_from_kept(uint32_t st, const float4 *p)
 }
 
 // The split state of a step of keys_product as the B operand (value channel, key) of the gradients' products
-__device__ __forceinline__ void publish_state(uint4 *p, int kk, const uint32_t (&rh)[4], const uint32_t (&rl)[4], const uint32_t (&ih)[4], const uint32_t (&il)[4])
+__device__ __forceinline__ void publish_split(uint4 *p, int kk, const uint32_t (&rh)[4], const uint32_t (&rl)[4], const uint32_t (&ih)[4], const uint32_t (&il)[4])
 {
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
         p[(4 * kk + 2 * e) * 32] = make_uint4(transpose8x8(rh[2 * e]), transpose8x8(rh[2 * e + 1]), transpose8x8(rl[2 * e]), transpose8x8(rl[2 * e + 1]));
         p[(4 * kk + 2 * e + 1) * 32] = make_uint4(transpose8x8(ih[2 * e]), transpose8x8(ih[2 * e + 1]), transpose8x8(il[2 * e]), transpose8x8(il[2 * e + 1]));
     }
+}
+
+// The same at the shared scale of all channels
+__device__ __forceinline__ void publish_state(uint4 *p, int kk, const uint32_t (&rh)[4], const uint32_t (&rl)[4], const uint32_t (&ih)[4], const uint32_t (&il)[4],
+                                              const RowScale &r, float all, bool own)
+{
+    if (!own) {
+        publish_split(p, kk, rh, rl, ih, il);
+        return;
+    }
+    uint32_t x[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        x[0][i] = rh[i];
+        x[1][i] = rl[i];
+        x[2][i] = ih[i];
+        x[3][i] = il[i];
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) to_shared_scale(x[c], r, all);
+    publish_split(p, kk, x[0], x[1], x[2], x[3]);
 }
 
 // Where a chain warp leaves a chunk's operands for the gradients; ps = NULL: nowhere
@@ -760,71 +796,73 @@ struct Publish {
 };
 
 // forward through one chunk whose tile is at `slot` (shared memory): U = M (V - W^* S), S <- gamma_C S + Y U unless
-// `update` is false.  rr: the chunk's rows of v.  Returns the largest magnitude of S.
+// `update` is false.  rr: the chunk's rows of v.  Returns the largest magnitudes of S.
 template <int DK, int BARN>
-__device__ __forceinline__ float forward_step(uint32_t st, float big, unsigned char *slot, int bar, float (&rr)[2][4], const Publish &pub, bool update, int lane)
+__device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned char *slot, int bar, float (&rr)[2][4], const Publish &pub, bool update, int lane)
 {
     using TL = Tile<DK>;
-    float isv;
-    const float sv = scale_for(warp_max(big), isv);
+    const RowScale sr = row_scale<4>(big);
+    bool own = false;
+    const float all = pub.ps ? shared_scale(sr, own) : 0.f;
     bar_sync(bar, BARN);
     const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot);
     const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
     float acc[1][2][2][4], ri[2][4];
     const uint32_t tiles[1] = {tile + TL::oW};
-    keys_product<DK, 1>(acc, st, sv, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
-        if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il);
+    keys_product<DK, 1>(acc, st, sr, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+        if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il, sr, all, own);
     });
-    const float fw = isv * inv[0];
+    const float fw[2] = {sr.inv[0] * inv[0], sr.inv[1] * inv[0]};
 #pragma unroll
     for (int n = 0; n < 2; ++n)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
-            ri[n][i] = -fw * acc[0][1][n][i];
+            rr[n][i] = fmaf(-fw[i >> 1], acc[0][0][n][i], rr[n][i]);
+            ri[n][i] = -fw[i >> 1] * acc[0][1][n][i];
         }
     TokFrag fr;
     {
         TokFrag fb;
-        const float ir = make_frag(fr, rr, ri);
+        const RowScale r = make_frag(fr, rr, ri);
         load_small<false>(fb, tile + TL::oM, lane);
-        product_small<false>(rr, ri, fr, fb, ir * inv[3]);
+        product_small<false>(rr, ri, fr, fb, r.inv, inv[3]);
     }
-    const float iu = make_frag(fr, rr, ri);
+    const RowScale ru = make_frag(fr, rr, ri);
     if (pub.ps) {
-        publish_frag(pub.pt, fr, lane);
+        const float all_u = publish_frag(pub.pt, fr, ru, lane);
         if (lane == 0) {
-            pub.scale[0] = isv;
-            pub.scale[1] = iu;
+            pub.scale[0] = all;
+            pub.scale[1] = all_u;
         }
     }
-    return update ? state_update<DK>(st, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(slot + TL::oG), lane) : big;
+    return update ? state_update<DK>(st, fr, ru.inv, inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(slot + TL::oG), lane) : big;
 }
 
 // backward through one chunk: Bc = M^H (Y^* G + (A D_beta)^H Yb^*), G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc.  yr, yi: the
-// chunk's rows of Yb^* (yi only with has_im).  Leaves Re Bc (the rows of dv) in pr; returns the largest magnitude of G.
+// chunk's rows of Yb^* (yi only with has_im).  Leaves Re Bc (the rows of dv) in pr; returns the largest magnitudes of G.
 template <int DK, bool kExact>
-__device__ __forceinline__ float backward_step(uint32_t sg, float big, unsigned char *slot, float (&yr)[2][4], float (&yi)[2][4], bool has_im,
+__device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigned char *slot, float (&yr)[2][4], float (&yi)[2][4], bool has_im,
                                                float (&pr)[2][4], const Publish &pub, int lane)
 {
     using TL = Tile<DK>;
     const int t4 = lane & 3;
     TokFrag fy;
-    const float iy = make_frag(fy, yr, yi);
+    const RowScale ry = make_frag(fy, yr, yi);
     const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot);
     const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
-    float ig;
-    const float sv = scale_for(warp_max(big), ig);
+    const RowScale sr = row_scale<4>(big);
+    bool own = false;
+    const float all = pub.ps ? shared_scale(sr, own) : 0.f;
     float acc[1][2][2][4];
     const uint32_t tiles[1] = {tile + TL::oY};
-    keys_product<DK, 1>(acc, sg, sv, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
-        if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il);
+    keys_product<DK, 1>(acc, sg, sr, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+        if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il, sr, all, own);
     });
     float pi[2][4];
     {
         TokFrag fb;
         load_small<true>(fb, tile + TL::oA, lane);
-        const float fg = ig * inv[1], fa = iy * inv[4];
+        const float fg[2] = {sr.inv[0] * inv[1], sr.inv[1] * inv[1]}, fa[2] = {ry.inv[0] * inv[4], ry.inv[1] * inv[4]};
 #pragma unroll
         for (int n = 0; n < 2; ++n) {
             float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f}, ni[4] = {0.f, 0.f, 0.f, 0.f};
@@ -836,27 +874,27 @@ __device__ __forceinline__ float backward_step(uint32_t sg, float big, unsigned 
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                pr[n][i] = fmaf(fa, re[i], fg * acc[0][0][n][i]);
-                pi[n][i] = fmaf(fa, im[i] - ni[i], fg * acc[0][1][n][i]);
+                pr[n][i] = fmaf(fa[i >> 1], re[i], fg[i >> 1] * acc[0][0][n][i]);
+                pi[n][i] = fmaf(fa[i >> 1], im[i] - ni[i], fg[i >> 1] * acc[0][1][n][i]);
             }
         }
     }
     TokFrag fp;
     {
         TokFrag fb;
-        const float ip = make_frag(fp, pr, pi);
+        const RowScale r = make_frag(fp, pr, pi);
         load_small<true>(fb, tile + TL::oM, lane);
-        product_small<true>(pr, pi, fp, fb, ip * inv[3]);
+        product_small<true>(pr, pi, fp, fb, r.inv, inv[3]);
     }
-    const float ib = make_frag(fp, pr, pi);
+    const RowScale rb = make_frag(fp, pr, pi);
     if (pub.ps) {
-        publish_frag(pub.pt, fp, lane);
+        const float all_b = publish_frag(pub.pt, fp, rb, lane);
         if (lane == 0) {
-            pub.scale[0] = ig;
-            pub.scale[1] = ib;
+            pub.scale[0] = all;
+            pub.scale[1] = all_b;
         }
     }
-    const float fq = iy * inv[2], fw = -ib * inv[0];
+    const float fq[2] = {ry.inv[0] * inv[2], ry.inv[1] * inv[2]}, fw[2] = {-rb.inv[0] * inv[0], -rb.inv[1] * inv[0]};
     const float4 *gamma = reinterpret_cast<const float4 *>(slot + TL::oG) + t4;
     uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
     uint32_t nih[4], nil[4];
@@ -865,7 +903,7 @@ __device__ __forceinline__ float backward_step(uint32_t sg, float big, unsigned 
         nih[i] = fp.ih[i] ^ 0x80008000u;
         nil[i] = fp.il[i] ^ 0x80008000u;
     }
-    big = 0.f;
+    big = make_float2(0.f, 0.f);
 #pragma unroll 1
     for (int np = 0; np < TL::KS; ++np, at += 32, gamma += 8) {
         float x[16];
@@ -900,8 +938,8 @@ __device__ __forceinline__ float backward_step(uint32_t sg, float big, unsigned 
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float cr = (i & 1) ? gm.z : gm.x, ci = (i & 1) ? gm.w : gm.y, u = x[8 * n + i], v = x[8 * n + 4 + i];
-                x[8 * n + i] = fmaf(fq, qr[n][i], cr * u + ci * v);
-                x[8 * n + 4 + i] = fmaf(fq, qi[n][i], cr * v - ci * u);
+                x[8 * n + i] = fmaf(fq[i >> 1], qr[n][i], cr * u + ci * v);
+                x[8 * n + 4 + i] = fmaf(fq[i >> 1], qi[n][i], cr * v - ci * u);
             }
         }
         tokens_product<DK>(qr, qi, fp, nih, nil, at + TL::oW);
@@ -909,10 +947,10 @@ __device__ __forceinline__ float backward_step(uint32_t sg, float big, unsigned 
         for (int n = 0; n < 2; ++n)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                x[8 * n + i] = fmaf(fw, qr[n][i], x[8 * n + i]);
-                x[8 * n + 4 + i] = fmaf(fw, qi[n][i], x[8 * n + 4 + i]);
-                big = fmaxf(big, fmaxf(fabsf(x[8 * n + i]), fabsf(x[8 * n + 4 + i])));
+                x[8 * n + i] = fmaf(fw[i >> 1], qr[n][i], x[8 * n + i]);
+                x[8 * n + 4 + i] = fmaf(fw[i >> 1], qi[n][i], x[8 * n + 4 + i]);
             }
+        big = max_abs(reinterpret_cast<const float(&)[4][4]>(x), big);
         tm_store(sg + 16 * np, x);
     }
     tm_wait_store();
@@ -1006,7 +1044,7 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_backward_
         const size_t state_at = ((size_t)bh * DK + 4 * t4) * DVT + col, step = (size_t)a.H * DVT;
         const Publish none = {nullptr, nullptr, nullptr};
         const float *from = back ? a.dS_T : a.S0;
-        float big = state_from_memory<DK>(st, from ? from + state_at : nullptr, DVT);
+        float2 big = state_from_memory<DK>(st, from ? from + state_at : nullptr, DVT);
 #pragma unroll 1
         for (int c = 0; c < nch; ++c) {
             const int slot = c % kSlots, cc = back ? nch - 1 - c : c, left = a.T - cc * kC - 2 * t4;
@@ -1248,7 +1286,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
         const uint32_t ss = tmem + ((uint32_t)(w & 3) << 21) + (w >> 2) * 16 * KT, sg = ss + 8 * KT;   // S and G
         float *scal = reinterpret_cast<float *>(smem + L::scal);
         const size_t step = (size_t)a.H * NB;
-        float big_s = 0.f, big_g = 0.f;
+        float2 big_s = make_float2(0.f, 0.f), big_g = big_s;
 #pragma unroll 1
         for (int j = 0; next_part(j); ++j)
 #pragma unroll 1
@@ -1269,16 +1307,15 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 float2 *rg = rgs + ((r & 1) * NCW + w) * M + 2 * t4;
                 const float4 *end = kept<DK>(a.keep_s, bh, a.pitch, s + 1, NB, 16 * w, lane), *start = kept<DK>(a.keep_s, bh, a.pitch, s, NB, 16 * w, lane);
                 const float4 *kg = kept<DK>(a.keep_g, bh, a.pitch, s, NB, 16 * w, lane);
-                big_s = 0.f;
-                if (kUnits) big_g = 0.f;
+                big_s = make_float2(0.f, 0.f);
+                if (kUnits) big_g = make_float2(0.f, 0.f);
 #pragma unroll 1
                 for (int n = 0; n < TL::KS; ++n, rg += 16, end += 128, start += 128, kg += 128) {
                     float x[16], y[16];
                     if constexpr (kUnits) {
                         read_piece(kg, x);
                         tm_store(sg + 16 * n, x);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) big_g = fmaxf(big_g, fabsf(x[i]));
+                        big_g = max_abs(reinterpret_cast<const float(&)[4][4]>(x), big_g);
                         read_piece(end, y);
                     } else {
                         tm_load(x, sg + 16 * n);
@@ -1299,8 +1336,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                     }
                     read_piece(start, y);
                     tm_store(ss + 16 * n, y);
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) big_s = fmaxf(big_s, fabsf(y[i]));
+                    big_s = max_abs(reinterpret_cast<const float(&)[4][4]>(y), big_s);
                 }
                 tm_wait_store();
             }

@@ -4,8 +4,9 @@
 //
 // Why split fp16: measured per SM and clock, mma.sync does 970 multiply-adds in fp16 and 484 in TF32, so three fp16
 // products (323 effective) are twice as fast as 3 x TF32 (161) and 2.5 times the fp32 pipe (128), at the same 22 bits.
-// fp16's exponent range is covered by scaling every operand tile by a power of two that puts its largest magnitude
-// at 2^14: entries down to 2^-16 of the largest keep all 22 bits, smaller ones an absolute error of 2^-39 of it.
+// fp16's exponent range is covered by powers of two: a chunk's tile of keys or queries is scaled so that its largest
+// magnitude comes to lie at 2^14, a state, R, U and what else has value channels for rows channel by channel (RowScale).
+// Entries down to 2^-16 of that largest one keep all 22 bits, smaller ones an absolute error of 2^-39 of it.
 //
 // Why chunks of 16: the state-sized products cost the same per token at any chunk size, the products inside a chunk
 // grow with it, and inside 16 tokens the decays divide safely unless a coordinate loses more than 2^-16, which is
@@ -143,23 +144,48 @@ __device__ __forceinline__ float scale_for(float largest, float &inv)
     return __uint_as_float((uint32_t)(141 - e) << 23);
 }
 __device__ __forceinline__ float warp_max(float x) { return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x))); }   // x >= 0
+// Largest magnitudes of a fragment's two rows (value channels: lane >> 2, + 8) in this thread.
 template <int N>
-__device__ __forceinline__ float max_abs(const float (&x)[N][4])
+__device__ __forceinline__ float2 max_abs(const float (&x)[N][4], float2 m = make_float2(0.f, 0.f))
 {
-    float m = 0.f;
 #pragma unroll
-    for (int n = 0; n < N; ++n)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) m = fmaxf(m, fabsf(x[n][i]));
+    for (int n = 0; n < N; ++n) {
+        m.x = fmaxf(m.x, fmaxf(fabsf(x[n][0]), fabsf(x[n][1])));
+        m.y = fmaxf(m.y, fmaxf(fabsf(x[n][2]), fabsf(x[n][3])));
+    }
     return m;
 }
-// A-operand registers (16 x 16) of two neighbouring accumulator tiles, scaled and split
-__device__ __forceinline__ void split_tiles(const float *x, const float *y, float s, uint32_t (&h)[4], uint32_t (&l)[4])
+// Scales of a fragment's rows, given the largest magnitudes in this thread.  Value channels do not interact, so every row has
+// a scale of its own: an entry's precision does not depend on other channels, and one that is not finite spoils none.
+// kStep: exponents go in steps of 1 or 4 (the largest entry of a row comes to lie in [2^14, 2^15) or [2^11, 2^15)); with
+// steps neighbouring channels mostly share a scale all the same, which the gradients' sums over the channels are for.
+struct RowScale {
+    float inv[2];
+};
+template <int kStep>
+__device__ __forceinline__ RowScale row_scale(float2 m)
 {
-    split_f16(x[0] * s, x[1] * s, h[0], l[0]);
-    split_f16(x[2] * s, x[3] * s, h[1], l[1]);
-    split_f16(y[0] * s, y[1] * s, h[2], l[2]);
-    split_f16(y[2] * s, y[3] * s, h[3], l[3]);
+    // both rows' leading 16 bits (all the exponent) at once through the row's four lanes
+    uint32_t x = __byte_perm(__float_as_uint(m.x), __float_as_uint(m.y), 0x7632);
+    x = __vmaxu2(x, __shfl_xor_sync(0xffffffffu, x, 1));
+    x = __vmaxu2(x, __shfl_xor_sync(0xffffffffu, x, 2));
+    RowScale r;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t e = max((i ? x >> 23 : (x << 16) >> 23), 27u);
+        r.inv[i] = __uint_as_float(kStep == 1 ? (e - 14u) << 23 : ((e + kStep & ~(uint32_t)(kStep - 1)) - 15u) << 23);
+    }
+    return r;
+}
+__device__ __forceinline__ float scale_of(float inv) { return __uint_as_float(0x7f000000u - __float_as_uint(inv)); }   // 1 / a power of two
+// A-operand registers (16 x 16) of two neighbouring accumulator tiles, scaled and split
+__device__ __forceinline__ void split_tiles(const float *x, const float *y, const RowScale &r, uint32_t (&h)[4], uint32_t (&l)[4])
+{
+    const float s0 = scale_of(r.inv[0]), s1 = scale_of(r.inv[1]);
+    split_f16(x[0] * s0, x[1] * s0, h[0], l[0]);
+    split_f16(x[2] * s1, x[3] * s1, h[1], l[1]);
+    split_f16(y[0] * s0, y[1] * s0, h[2], l[2]);
+    split_f16(y[2] * s1, y[3] * s1, h[3], l[3]);
 }
 // cos / sin of a phase in 2^-32 turns: the quadrant is the two leading bits, the rest lies in [-pi/4, pi/4], where the
 // Taylor polynomials to x^9 and x^10 are off by 2e-9 (half the code of sincospif, and code is what costs here)
@@ -235,7 +261,7 @@ struct Tile {
 // each of two token tiles: [0] = Re = Xr Sr + Xi Si, [1] = Im = Xr Si - Xi Sr; scaled by s and the tiles' scales.
 // pub(kk, rh, rl, ih, il) sees the split state of every step.
 template <int DK, int NX, typename Pub>
-__device__ __forceinline__ void keys_product(float (&acc)[NX][2][2][4], uint32_t st, float s, const uint32_t (&tile)[NX],
+__device__ __forceinline__ void keys_product(float (&acc)[NX][2][2][4], uint32_t st, const RowScale &s, const uint32_t (&tile)[NX],
                                              int lane, Pub pub)
 {
     using TL = Tile<DK>;
@@ -308,9 +334,9 @@ __device__ __forceinline__ void load_small(TokFrag &b, uint32_t tile, int lane)
     }
 }
 
-// out = a b (kConj: a conj(b)) over 16 tokens, both complex, unscaled by f
+// out = a b (kConj: a conj(b)) over 16 tokens, both complex, unscaled by f and the rows' inv
 template <bool kConj>
-__device__ __forceinline__ void product_small(float (&re)[2][4], float (&im)[2][4], const TokFrag &a, const TokFrag &b, float f)
+__device__ __forceinline__ void product_small(float (&re)[2][4], float (&im)[2][4], const TokFrag &a, const TokFrag &b, const float (&inv)[2], float f)
 {
     float rr[2][4], ii[2][4], ir[2][4], ri[2][4];
 #pragma unroll
@@ -338,19 +364,36 @@ __device__ __forceinline__ void product_small(float (&re)[2][4], float (&im)[2][
     for (int n = 0; n < 2; ++n)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            re[n][i] = f * (kConj ? rr[n][i] + ii[n][i] : rr[n][i] - ii[n][i]);
-            im[n][i] = f * (kConj ? ir[n][i] - ri[n][i] : ir[n][i] + ri[n][i]);
+            re[n][i] = (inv[i >> 1] * f) * (kConj ? rr[n][i] + ii[n][i] : rr[n][i] - ii[n][i]);
+            im[n][i] = (inv[i >> 1] * f) * (kConj ? ir[n][i] - ri[n][i] : ir[n][i] + ri[n][i]);
         }
 }
 
-// scale and split a [value x 16 tokens] matrix; returns the inverse scale
-__device__ __forceinline__ float make_frag(TokFrag &f, const float (&re)[2][4], const float (&im)[2][4])
+// scale and split a [value x 16 tokens] matrix
+__device__ __forceinline__ RowScale make_frag(TokFrag &f, const float (&re)[2][4], const float (&im)[2][4])
 {
-    float inv;
-    const float s = scale_for(warp_max(fmaxf(max_abs(re), max_abs(im))), inv);
-    split_tiles(re[0], re[1], s, f.rh, f.rl);
-    split_tiles(im[0], im[1], s, f.ih, f.il);
-    return inv;
+    const RowScale r = row_scale<1>(max_abs(im, max_abs(re)));
+    split_tiles(re[0], re[1], r, f.rh, f.rl);
+    split_tiles(im[0], im[1], r, f.ih, f.il);
+    return r;
+}
+// The inverse of the scale for sums over a warp's channels: that of its largest row (2^114 or an infinity's aside); own: some
+// row has another.
+__device__ __forceinline__ float shared_scale(const RowScale &r, bool &own)
+{
+    const float all = warp_max(fmaxf(r.inv[0], r.inv[1]));
+    own = __any_sync(0xffffffffu, r.inv[0] != all || r.inv[1] != all);
+    return all;
+}
+// Split operands from the rows' scales to the shared one (a power of two: exact unless bits fall off the end)
+__device__ __forceinline__ void to_shared_scale(uint32_t (&x)[4], const RowScale &r, float all)
+{
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float f = r.inv[i & 1] * scale_of(all);
+        const uint32_t f2 = pack_f16(f, f);
+        asm("mul.rn.f16x2 %0, %0, %1;" : "+r"(x[i]) : "r"(f2));
+    }
 }
 
 // re, im (two key tiles of eight) = a X with tokens as k: X the tile at `at` (B operand by transposed loads);
@@ -420,19 +463,18 @@ __device__ __forceinline__ void store_rows(T *p, const float (&x)[2][4], size_t 
 }
 
 // The thread's fragment of a state [d_k][dv] (paired rows) at `p` (its key pair 2 (lane & 3), its column); returns the
-// largest magnitude.  p = NULL: zeros.
+// largest magnitudes of its two rows.  p = NULL: zeros.
 template <int DK>
-__device__ __forceinline__ float state_from_memory(uint32_t st, const float *p, int dv)
+__device__ __forceinline__ float2 state_from_memory(uint32_t st, const float *p, int dv)
 {
-    float largest = 0.f;
+    float2 largest = make_float2(0.f, 0.f);
 #pragma unroll 1
     for (int n = 0; n < Tile<DK>::KS; ++n) {
         float x[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {                            // [key tile][Re / Im][column half][key]
+        for (int i = 0; i < 16; ++i)                              // [key tile][Re / Im][column half][key]
             x[i] = p ? p[(size_t)(32 * n + 16 * (i >> 3) + 2 * (i & 1) + ((i >> 2) & 1)) * dv + 8 * ((i >> 1) & 1)] : 0.f;
-            largest = fmaxf(largest, fabsf(x[i]));
-        }
+        largest = max_abs(reinterpret_cast<const float(&)[4][4]>(x), largest);
         tm_store(st + 16 * n, x);
     }
     tm_wait_store();
@@ -451,9 +493,9 @@ __device__ __forceinline__ void state_to_memory(uint32_t st, float *p, int dv)
     }
 }
 
-// S <- gamma_C S + f a Y, the state at `st`; returns the thread's largest magnitude of the new state
+// S <- gamma_C S + f inv a Y, the state at `st`, inv per row; returns the largest magnitudes of the new state's rows
 template <int DK>
-__device__ __forceinline__ float state_update(uint32_t st, const TokFrag &a, float f, uint32_t tile, const float4 *gamma, int lane)
+__device__ __forceinline__ float2 state_update(uint32_t st, const TokFrag &a, const float (&inv)[2], float f, uint32_t tile, const float4 *gamma, int lane)
 {
     using TL = Tile<DK>;
     uint32_t nih[4], nil[4];
@@ -464,7 +506,8 @@ __device__ __forceinline__ float state_update(uint32_t st, const TokFrag &a, flo
     }
     uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
     gamma += lane & 3;
-    float largest = 0.f;
+    const float fr[2] = {inv[0] * f, inv[1] * f};
+    float2 largest = make_float2(0.f, 0.f);
 #pragma unroll 1
     for (int np = 0; np < TL::KS; ++np, at += 32, gamma += 8, st += 16) {
         float x[16], re[2][4], im[2][4];
@@ -477,11 +520,11 @@ __device__ __forceinline__ float state_update(uint32_t st, const TokFrag &a, flo
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float gr = (i & 1) ? g.z : g.x, gi = (i & 1) ? g.w : g.y, u = x[8 * n + i], v = x[8 * n + 4 + i];
-                x[8 * n + i] = fmaf(f, re[n][i], gr * u - gi * v);
-                x[8 * n + 4 + i] = fmaf(f, im[n][i], gr * v + gi * u);
-                largest = fmaxf(largest, fmaxf(fabsf(x[8 * n + i]), fabsf(x[8 * n + 4 + i])));
+                x[8 * n + i] = fmaf(fr[i >> 1], re[n][i], gr * u - gi * v);
+                x[8 * n + 4 + i] = fmaf(fr[i >> 1], im[n][i], gr * v + gi * u);
             }
         }
+        largest = max_abs(reinterpret_cast<const float(&)[4][4]>(x), largest);
         tm_store(st, x);
     }
     tm_wait_store();

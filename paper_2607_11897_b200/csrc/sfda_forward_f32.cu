@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
         const int col = c0 + 16 * w + g;                         // and col + 8
         const uint32_t st = tmem + ((uint32_t)(w & 3) << 21) + (w >> 2) * 8 * TL::KT;    // this warp's lanes and columns
         const size_t state_at = ((size_t)bh * DK + 4 * t4) * a.dv + col;
-        float largest = state_from_memory<DK>(st, a.S0 ? a.S0 + state_at : nullptr, a.dv);
+        float2 largest = state_from_memory<DK>(st, a.S0 ? a.S0 + state_at : nullptr, a.dv);
         const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
         const size_t step = (size_t)a.H * a.dv;
         size_t at = (row0 + (size_t)(2 * t4) * a.H) * a.dv + col;
@@ -94,39 +94,38 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
             const int slot = c % kSlots, left = a.T - c * kC - 2 * t4;
             float rr[2][4], ri[2][4];
             load_rows(rr, static_cast<const T *>(a.v) + at, step, left);
-            float isv;
-            const float ss = scale_for(warp_max(largest), isv);
+            const RowScale sr = row_scale<4>(largest);
             bar_sync(kBarFull + slot, 64 + kChain);
             const uint32_t tile = base + slot * TL::bytes;
             const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
             float acc[2][2][2][4];
             const uint32_t tiles[2] = {tile + TL::oW, tile + TL::oQ};
-            keys_product<DK, 2>(acc, st, ss, tiles, lane, [](int, const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4]) {});
-            const float fw = isv * inv[0], fq = isv * inv[2];
+            keys_product<DK, 2>(acc, st, sr, tiles, lane, [](int, const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4]) {});
+            const float fw[2] = {sr.inv[0] * inv[0], sr.inv[1] * inv[0]}, fq[2] = {sr.inv[0] * inv[2], sr.inv[1] * inv[2]};
 #pragma unroll
             for (int n = 0; n < 2; ++n)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    rr[n][i] = fmaf(-fw, acc[0][0][n][i], rr[n][i]);
-                    ri[n][i] = -fw * acc[0][1][n][i];
+                    rr[n][i] = fmaf(-fw[i >> 1], acc[0][0][n][i], rr[n][i]);
+                    ri[n][i] = -fw[i >> 1] * acc[0][1][n][i];
                 }
             TokFrag fr;
-            float iu;
+            RowScale ru;
 #pragma unroll 1
             for (int pass = 0; pass < 2; ++pass) {               // U = M R, then (A^{qk} D_beta) U
                 TokFrag fb;
-                iu = make_frag(fr, rr, ri);
+                ru = make_frag(fr, rr, ri);
                 load_small<false>(fb, tile + (pass ? TL::oA : TL::oM), lane);
-                product_small<false>(rr, ri, fr, fb, iu * inv[3 + pass]);
+                product_small<false>(rr, ri, fr, fb, ru.inv, inv[3 + pass]);
             }
-            largest = state_update<DK>(st, fr, iu * inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
+            largest = state_update<DK>(st, fr, ru.inv, inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
             if (c + kSlots < nch) bar_arrive(kBarDone + slot, kPrep + kChain);
 #pragma unroll
             for (int n = 0; n < 2; ++n)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    rr[n][i] = fmaf(fq, acc[1][0][n][i], rr[n][i]);
-                    ri[n][i] = -fmaf(fq, acc[1][1][n][i], ri[n][i]);
+                    rr[n][i] = fmaf(fq[i >> 1], acc[1][0][n][i], rr[n][i]);
+                    ri[n][i] = -fmaf(fq[i >> 1], acc[1][1][n][i], ri[n][i]);
                 }
             store_rows(static_cast<T *>(a.o) + at, rr, step, left);
             if (a.o_im) store_rows(static_cast<T *>(a.o_im) + at, ri, step, left);

@@ -5,12 +5,13 @@ import numpy as np
 import pytest
 
 import workloads
+from oracle import backward
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 if torch.cuda.is_available():
     import paper_2607_11897_b200 as sfda
-    from tests.test_gpu_parity import all_pairs, check_backward, check_forward, oracle_pairs, run_forward, upstream
+    from tests.test_gpu_parity import all_pairs, check_backward, check_forward, oracle_pairs, run_backward, run_forward, upstream
 
 # Operands keep 22 bits and the products of their tails (2^-22) are left out; sums are fp32 over at most 128 terms,
 # carried over chunks by a contraction.  That is a few 1e-7 of a tensor's largest entry (8e-7 measured); ten times that.
@@ -156,3 +157,41 @@ def test_fp32_forward_is_as_close_to_64_bits_as_the_cuda_core_kernel(B, H, d_k, 
     pick = lambda out: [np.stack([x[b, :, h] if i < 2 else x[b, h] for b, h in pairs]) for i, x in enumerate(out[:3])]  # noqa: E731
     for a, b, w in zip(pick(run_forward(cfg, inp)), pick(run_forward(cfg, inp, simt=True)), want):
         assert distance(a, w) <= 1.05 * distance(b, w)
+
+
+@pytest.mark.parametrize("B,H,d_k,d_v,T", [(1, 2, 128, 128, 100), (1, 2, 64, 64, 33), (5, 16, 128, 64, 50), (5, 32, 128, 128, 70)])
+def test_every_value_channel_has_its_own_precision(B, H, d_k, d_v, T):
+    """Value channels do not interact: one 2^-36 below its neighbours is as exact as they are.  Error per channel against
+    that channel's own size: a few roundings of 22-bit operands and fp32 sums, 3e-7 measured; five times that."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16c", B=B, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=720 + T)
+    inp, up = workloads.forward_inputs(cfg), upstream(cfg, T)
+    down, back = np.exp2(-(np.arange(d_v) * 7 % 37)).astype(np.float32), np.exp2(np.arange(d_v) * 5 % 23).astype(np.float32)
+    for n in ("v", "S0"):
+        inp[n] *= down
+    for n in up:
+        up[n] = up[n] * back
+    pairs = all_pairs(cfg)[:2] + all_pairs(cfg)[-2:]
+    o, o_im, S_T = run_forward(cfg, inp)
+    grads = run_backward(cfg, inp, up)
+    s = workloads.sequences(inp, pairs)
+    pick = lambda x, state=False: np.stack([x[b, h] if state else x[b, :, h] for b, h in pairs]).astype(np.float64)  # noqa: E731
+    w = oracle_pairs(inp, pairs)
+    g = backward.sfda_backward(s["q"], s["k"], s["v"], s["alpha"], s["theta"], s["beta"], s["S0"], pick(up["do_re"]), pick(up["do_im"]),
+                               pick(up["dS_T"], True))
+    for name, got, want in (("o", pick(o), w[0]), ("o_im", pick(o_im), w[1]), ("S_T", pick(S_T, True), w[2]),
+                            ("dv", pick(grads["dv"]), g[2]), ("dS0", pick(grads["dS0"], True), g[6])):
+        e = np.sqrt(((got - want) ** 2).sum((0, 1)) / (want ** 2).sum((0, 1)))
+        assert e.max() <= 1.5e-6, (name, e.max(), e.argmax())
+
+
+@pytest.mark.parametrize("what,where", [("v", (0, 17, 0, 5)), ("S0", (0, 0, 3, 5)), ("dS_T", (0, 0, 3, 5)), ("do_re", (0, 17, 0, 5))])
+def test_an_infinite_channel_leaves_the_others_alone(what, where):
+    """... in all that belongs to a channel alone: outputs, states, dv and dS0 are those of the call without it."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16i", B=1, T=40, H=1, d_k=128, d_v=128, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=730)
+    inp, up = workloads.forward_inputs(cfg), upstream(cfg, 5)
+    run = lambda: list(run_forward(cfg, inp)) + [run_backward(cfg, inp, up)[n] for n in ("dv", "dS0")]  # noqa: E731
+    want = run()
+    (inp if what in inp else up)[what][where] = np.inf
+    others = np.arange(128) != 5
+    for a, b in zip(run(), want):
+        assert np.array_equal(a[..., others], b[..., others])
