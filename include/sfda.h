@@ -142,7 +142,8 @@ SFDA_API int sfda_forward_partition(int B, int T, int H, int d_k, int d_v, int c
  * precision (products of operands split into two fp16 parts, 22 bits, summed in
  * fp32; any alpha in [0, 1]).  Those 22 bits count from the largest entry of a value channel (over the keys, or over
  * 16 tokens) and of the keys and queries of 16 tokens; an entry 2^-16 and more below that has an absolute error of
- * 2^-39 of it.  The bf16 tensor-core path forms 1/gamma_t inside a chunk and so
+ * 2^-39 of it.  An input that is not finite makes NaN of what depends on it in the recurrence, and of nothing else.
+ * The bf16 tensor-core path forms 1/gamma_t inside a chunk and so
  * additionally assumes prod_{t in chunk} alpha_{t,j} >= exp(-80) for every
  * coordinate j; beyond that results lose accuracy but stay finite.
  */

@@ -118,14 +118,21 @@ __device__ __forceinline__ void mma3x(float (&d)[4], const uint32_t (&ah)[4], co
 }
 
 // the [value x token] operand as the A operand (token, value) of products over the value columns, at their
-// shared scale, whose inverse is returned
-__device__ __forceinline__ float publish_frag(uint4 *p, const TokFrag &f, const RowScale &r, int lane)
+// shared scale, whose inverse is returned; NaN at the tokens `off`
+__device__ __forceinline__ float publish_frag(uint4 *p, const TokFrag &f, const RowScale &r, bool odd, uint32_t off, int lane)
 {
     bool own;
     const float all = shared_scale(r, own);                      // (nearly always some row has another)
     auto put = [&](int plane, const uint32_t(&v)[4]) {
         uint32_t x[4] = {v[0], v[1], v[2], v[3]};
         to_shared_scale(x, r, all);
+        if (plane == 0 && odd) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t m = off >> (8 * (i >> 1) + 2 * (lane & 3) + 16 * (i & 1));
+                x[i] |= (m & 1 ? 0x7e00u : 0u) | (m & 2 ? 0x7e000000u : 0u);
+            }
+        }
         p[plane * 32 + lane] = make_uint4(transpose8x8(x[0]), transpose8x8(x[2]), transpose8x8(x[1]), transpose8x8(x[3]));
     };
     put(0, f.rh);
@@ -700,7 +707,8 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             float x = dbp[r];
             x += __shfl_xor_sync(0xffffffffu, x, 1);
             x += __shfl_xor_sync(0xffffffffu, x, 2);
-            if (t4 == 0) db[warp * 16 + g + 8 * r] = x;
+            // (a query that was taken out is missing from its own token's sum)
+            if (t4 == 0) db[warp * 16 + g + 8 * r] = reinterpret_cast<const uint32_t *>(inv)[7] >> (16 + g + 8 * r) & 1 ? __int_as_float(0x7fc00000) : x;
         }
         if (!last_one && keep) bar_arrive(kBarTaken, kGrad + kPrep);
     } else if (!last_one) {
@@ -796,58 +804,79 @@ struct Publish {
 };
 
 // forward through one chunk whose tile is at `slot` (shared memory): U = M (V - W^* S), S <- gamma_C S + Y U unless
-// `update` is false.  rr: the chunk's rows of v.  Returns the largest magnitudes of S.
-template <int DK, int BARN>
-__device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned char *slot, int bar, float (&rr)[2][4], const Publish &pub, bool update, int lane)
+// `update` is false.  load(rr): the chunk's rows of v.  Returns the largest magnitudes of S.
+template <int DK, int BARN, typename Load>
+__device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned char *slot, int bar, Load load, const Publish &pub, bool update, int lane)
 {
     using TL = Tile<DK>;
+    float rr[2][4], ri[2][4];
+    load(rr);
+    uint32_t off;                                                // tokens whose v is not finite; below, all behind them too
     const RowScale sr = row_scale<4>(big);
     bool own = false;
     const float all = pub.ps ? shared_scale(sr, own) : 0.f;
     bar_sync(bar, BARN);
     const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot);
     const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
-    float acc[1][2][2][4], ri[2][4];
     const uint32_t tiles[1] = {tile + TL::oW};
-    keys_product<DK, 1>(acc, st, sr, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
-        if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il, sr, all, own);
-    });
-    const float fw[2] = {sr.inv[0] * inv[0], sr.inv[1] * inv[0]};
-#pragma unroll
-    for (int n = 0; n < 2; ++n)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            rr[n][i] = fmaf(-fw[i >> 1], acc[0][0][n][i], rr[n][i]);
-            ri[n][i] = -fw[i >> 1] * acc[0][1][n][i];
-        }
     TokFrag fr;
+    {
+        float acc[1][2][2][4];
+        keys_product<DK, 1>(acc, st, sr, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+            if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il, sr, all, own);
+        });
+        const float fw[2] = {sr.inv[0] * inv[0], sr.inv[1] * inv[0]};
+        off = take_out(rr);
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                rr[n][i] = fmaf(-fw[i >> 1], acc[0][0][n][i], rr[n][i]);
+                ri[n][i] = -fw[i >> 1] * acc[0][1][n][i];
+            }
+    }
     {
         TokFrag fb;
         const RowScale r = make_frag(fr, rr, ri);
         load_small<false>(fb, tile + TL::oM, lane);
         product_small<false>(rr, ri, fr, fb, r.inv, inv[3]);
     }
-    const RowScale ru = make_frag(fr, rr, ri);
+    RowScale ru = make_frag(fr, rr, ri);
+    const uint32_t out = reinterpret_cast<const uint32_t *>(inv)[7];
+    const bool odd = __any_sync(0xffffffffu, (off | out) != 0);
+    if (odd) {
+        off = every_lanes(off, lane);
+        off = from_first(off & 0xffffu) | from_first(off >> 16) << 16 | both(from_first(out & 0xffffu));
+    }
     if (pub.ps) {
-        const float all_u = publish_frag(pub.pt, fr, ru, lane);
+        const float all_u = publish_frag(pub.pt, fr, ru, odd, off, lane);
         if (lane == 0) {
             pub.scale[0] = all;
             pub.scale[1] = all_u;
         }
     }
+    if (odd) put_nan(ru.inv, off);
     return update ? state_update<DK>(st, fr, ru.inv, inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(slot + TL::oG), lane) : big;
 }
 
-// backward through one chunk: Bc = M^H (Y^* G + (A D_beta)^H Yb^*), G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc.  yr, yi: the
-// chunk's rows of Yb^* (yi only with has_im).  Leaves Re Bc (the rows of dv) in pr; returns the largest magnitudes of G.
-template <int DK, bool kExact>
-__device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigned char *slot, float (&yr)[2][4], float (&yi)[2][4], bool has_im,
-                                               float (&pr)[2][4], const Publish &pub, int lane)
+// backward through one chunk: Bc = M^H (Y^* G + (A D_beta)^H Yb^*), G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc.  load(yr, yi):
+// the chunk's rows of Yb^* (yi zero without has_im).  Leaves Re Bc (the rows of dv) in pr; returns the largest magnitudes of G.
+template <int DK, bool kExact, typename Load>
+__device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigned char *slot, Load load, bool has_im, float (&pr)[2][4],
+                                                const Publish &pub, int lane)
 {
     using TL = Tile<DK>;
     const int t4 = lane & 3;
+    uint32_t off;                                                // tokens whose cotangents are not finite; below, all before them too
     TokFrag fy;
-    const RowScale ry = make_frag(fy, yr, yi);
+    RowScale ry;
+    {
+        float yr[2][4], yi[2][4];
+        load(yr, yi);
+        off = take_out(yr);
+        if (has_im) off |= take_out(yi);
+        ry = make_frag(fy, yr, yi);
+    }
     const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot);
     const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
     const RowScale sr = row_scale<4>(big);
@@ -887,8 +916,16 @@ __device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigne
         product_small<true>(pr, pi, fp, fb, r.inv, inv[3]);
     }
     const RowScale rb = make_frag(fp, pr, pi);
+    const uint32_t out = reinterpret_cast<const uint32_t *>(inv)[7];
+    const bool odd = __any_sync(0xffffffffu, (off | out) != 0);
+    if (odd) {
+        off = every_lanes(off, lane);
+        off = to_last(off & 0xffffu) | to_last(off >> 16) << 16 | both(to_last((out | out >> 16) & 0xffffu));
+        put_nan(pr, off, lane);
+        put_nan(ry.inv, off);
+    }
     if (pub.ps) {
-        const float all_b = publish_frag(pub.pt, fp, rb, lane);
+        const float all_b = publish_frag(pub.pt, fp, rb, odd, off, lane);
         if (lane == 0) {
             pub.scale[0] = all;
             pub.scale[1] = all_b;
@@ -1011,7 +1048,8 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_backward_
             PrepRaw<L::PM::TPT, T> next;
             prep_fetch<DK, kPrepWarps, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, nx * kC, a.T, back, role.prep);
             float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes);
-            if (!prep_planes<DK, kPrepWarps, kBarAux, T>(in, nullptr, smem + slot * TL::bytes, smem + L::kb + slot * TL::BIG, smem + L::scan, back, role.prep))
+            if (!prep_chunk<DK, kPrepWarps, kBarAux, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, at * kC, a.T, nullptr, smem + slot * TL::bytes,
+                                                        smem + L::kb + slot * TL::BIG, smem + L::scan, back, role.prep))
                 slow_gram<DK, kPrepWarps, kBarAux, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, at * kC, a.T, smem + L::slow, smem + L::scan,
                                                       gk, gk + 16 * 17, back, role.prep);
             bar_arrive(kBarPlanes + slot, kPrep + 64);
@@ -1052,15 +1090,14 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_backward_
             const size_t at = (row0 + (size_t)(cc * kC + 2 * t4) * a.H) * DVT + col;
             if (!back) {
                 if (cc % kSegChunks == 0) keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, cc / kSegChunks, DVT, col0, lane), st);
-                float rr[2][4];
-                load_rows(rr, static_cast<const T *>(a.v) + at, step, left);
-                big = forward_step<DK, 64 + kChain>(st, big, tile, kBarFull + slot, rr, none, true, lane);
+                auto rows = [&](float(&x)[2][4]) { load_rows(x, static_cast<const T *>(a.v) + at, step, left); };
+                big = forward_step<DK, 64 + kChain>(st, big, tile, kBarFull + slot, rows, none, true, lane);
             } else {
                 if (c == 0 || cc % kSegChunks == kSegChunks - 1) keep_state<DK>(kept<DK>(a.keep_g, bh, a.pitch, cc / kSegChunks, DVT, col0, lane), st);
-                float yr[2][4], yi[2][4], pr[2][4];
-                load_cotangents<T>(yr, yi, a.d_o, a.d_o_im, at, step, left);
+                float pr[2][4];
+                auto rows = [&](float(&x)[2][4], float(&y)[2][4]) { load_cotangents<T>(x, y, a.d_o, a.d_o_im, at, step, left); };
                 bar_sync(kBarFull + slot, 64 + kChain);
-                big = backward_step<DK, sizeof(T) == 2>(st, big, tile, yr, yi, a.d_o_im != nullptr, pr, none, lane);
+                big = backward_step<DK, sizeof(T) == 2>(st, big, tile, rows, a.d_o_im != nullptr, pr, none, lane);
             }
             if (c + kSlots < nch) bar_arrive(kBarDone + slot, kPrep + kChain);
         }
@@ -1260,7 +1297,8 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 PrepRaw<L::PM::TPT, T> in;
                 prep_fetch<DK, kPrepWarps, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, needq, ptid);
                 float4 *vals = sweep ? reinterpret_cast<float4 *>(ring + (size_t)slot * SC::slot + SC::oV) : nullptr;
-                const bool fast = prep_planes<DK, kPrepWarps, kBarPrep, T>(in, vals, tile, smem + L::kb, smem + L::scan, needq, ptid);
+                const bool fast = prep_chunk<DK, kPrepWarps, kBarPrep, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, vals, tile, smem + L::kb,
+                                                                          smem + L::scan, needq, ptid);
                 if (!fast)
                     slow_gram<DK, kPrepWarps, kBarPrep, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T, ring + SC::oSlow,
                                                            smem + L::scan, gram, gram + 16 * 17, needq, ptid);
@@ -1347,9 +1385,10 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 unsigned char *scr = ring + (size_t)slot * SC::slot;
                 Publish pub = {nullptr, nullptr, nullptr};
                 if (r >= 0) pub = {reinterpret_cast<uint4 *>(scr + SC::oS) + w * KT * 64 + lane, reinterpret_cast<uint4 *>(scr + SC::oU) + w * 128, scal + (slot * NCW + w) * 4};
-                float rr[2][4];
-                load_rows(rr, static_cast<const T *>(a.v) + (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col, step, a.T - t0 - 2 * t4);
-                big_s = forward_step<DK, kPrep + kChain>(ss, big_s, smem + slot * TL::bytes, kBarFull + slot, rr, pub, r < 0 || c + 1 < kSegChunks, lane);
+                auto rows = [&](float(&x)[2][4]) {
+                    load_rows(x, static_cast<const T *>(a.v) + (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col, step, a.T - t0 - 2 * t4);
+                };
+                big_s = forward_step<DK, kPrep + kChain>(ss, big_s, smem + slot * TL::bytes, kBarFull + slot, rows, pub, r < 0 || c + 1 < kSegChunks, lane);
                 if (r < 0) bar_arrive(kBarDone + slot, kPrep + kChain);
             }
             if (r < 0) {                                                 // the final state, or where the next CTA begins
@@ -1362,9 +1401,9 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 const size_t at = (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col;
                 unsigned char *scr = ring + (size_t)slot * SC::slot;
                 const Publish pub = {reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64 + lane, reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, scal + (slot * NCW + w) * 4 + 2};
-                float yr[2][4], yi[2][4], pr[2][4];
-                load_cotangents<T>(yr, yi, a.d_o, a.d_o_im, at, step, left);
-                big_g = backward_step<DK, kExact>(sg, big_g, smem + slot * TL::bytes, yr, yi, a.d_o_im != nullptr, pr, pub, lane);
+                float pr[2][4];
+                auto rows = [&](float(&x)[2][4], float(&y)[2][4]) { load_cotangents<T>(x, y, a.d_o, a.d_o_im, at, step, left); };
+                big_g = backward_step<DK, kExact>(sg, big_g, smem + slot * TL::bytes, rows, a.d_o_im != nullptr, pr, pub, lane);
                 store_rows(static_cast<T *>(a.dv) + at, pr, step, left);
                 bar_arrive(kBarDone + slot, kPrep + kChain);
             }

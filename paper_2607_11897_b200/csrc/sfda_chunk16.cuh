@@ -144,14 +144,20 @@ __device__ __forceinline__ float scale_for(float largest, float &inv)
     return __uint_as_float((uint32_t)(141 - e) << 23);
 }
 __device__ __forceinline__ float warp_max(float x) { return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x))); }   // x >= 0
+__device__ __forceinline__ float max_nan(float x, float y)     // NaN where either is
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(y));
+    return r;
+}
 // Largest magnitudes of a fragment's two rows (value channels: lane >> 2, + 8) in this thread.
 template <int N>
 __device__ __forceinline__ float2 max_abs(const float (&x)[N][4], float2 m = make_float2(0.f, 0.f))
 {
 #pragma unroll
     for (int n = 0; n < N; ++n) {
-        m.x = fmaxf(m.x, fmaxf(fabsf(x[n][0]), fabsf(x[n][1])));
-        m.y = fmaxf(m.y, fmaxf(fabsf(x[n][2]), fabsf(x[n][3])));
+        m.x = max_nan(m.x, max_nan(fabsf(x[n][0]), fabsf(x[n][1])));
+        m.y = max_nan(m.y, max_nan(fabsf(x[n][2]), fabsf(x[n][3])));
     }
     return m;
 }
@@ -205,6 +211,53 @@ __device__ __forceinline__ void cos_sin(uint32_t turns, float &c, float &s)
     s = q & 2 ? -ss : ss;
 }
 
+// ---- inputs that are not finite -------------------------------------------------------------------
+// The products over a chunk's tokens multiply by the zeros of triangular matrices, and zero times NaN is NaN: a token that
+// is not finite would reach the outputs of the tokens before it, and the gradients of those behind it.  So it goes in as
+// zeros (PREP: the keys' side for all channels, CHAIN: v and the cotangents channel by channel), and what it does reach in
+// the recurrence becomes NaN explicitly: a channel's outputs from the token on and its state behind it, or, on the way
+// back, its cotangents up to the token.  PREP sees it in the maxima that the scales need anyway and then does the chunk
+// over; CHAIN takes its few values out as they come and asks only after the products whether there was one.  (PREP
+// looking at its inputs first: 528 us instead of 444 for the fp32 forward at B = 2, T = 2001, H = 16; CHAIN branching in
+// front of its products: 472 us, doing a step over: 567 us.)
+// Tokens that are not finite in this thread's share of the two rows become zero; their bits, for every_lanes
+__device__ __forceinline__ uint32_t take_out(float (&x)[2][4])
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool on = fabsf(x[n][i]) <= 3.402823466e38f;
+            m |= on ? 0u : 1u << (8 * n + (i & 1) + 16 * (i >> 1));
+            x[n][i] = on ? x[n][i] : 0.f;
+        }
+    return m;
+}
+// bit t: the row lane >> 2, bit 16 + t: the row + 8
+__device__ __forceinline__ uint32_t every_lanes(uint32_t m, int lane)
+{
+    m <<= 2 * (lane & 3);
+    m |= __shfl_xor_sync(0xffffffffu, m, 1);
+    return m | __shfl_xor_sync(0xffffffffu, m, 2);
+}
+__device__ __forceinline__ uint32_t from_first(uint32_t m) { return m ? 0xffffu & ~((m & (0u - m)) - 1u) : 0u; }    // 16 tokens
+__device__ __forceinline__ uint32_t to_last(uint32_t m) { return m ? 0xffffffffu >> __clz(m) : 0u; }
+__device__ __forceinline__ uint32_t both(uint32_t m) { return m | m << 16; }
+__device__ __forceinline__ void put_nan(float (&x)[2][4], uint32_t m, int lane)
+{
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (m >> (8 * n + 2 * (lane & 3) + (i & 1) + 16 * (i >> 1)) & 1) x[n][i] = __int_as_float(0x7fc00000);
+}
+__device__ __forceinline__ void put_nan(float (&inv)[2], uint32_t m)      // the rows' scales: a state update with them is NaN
+{
+    if (m & 0xffffu) inv[0] = __int_as_float(0x7fc00000);
+    if (m >> 16) inv[1] = __int_as_float(0x7fc00000);
+}
+
 // ---- the state in tensor memory: 16 columns of the thread's lane = two key tiles, [re 4, im 4] each ------------------
 __device__ __forceinline__ void tm_load(float (&x)[16], uint32_t addr)
 {
@@ -252,7 +305,8 @@ struct Tile {
     static constexpr int PL = 16 * LDB, BIG = 4 * PL;
     static constexpr int LDS = 48, PS = 16 * LDS, SMALL = 4 * PS;
     static constexpr int oW = 0, oY = BIG, oQ = 2 * BIG, oM = 3 * BIG, oA = oM + SMALL, oG = oA + SMALL, oS = oG + 8 * M;
-    // oG: gamma_C float2 [M]; oS: inverse scales of W, Y, Q, M, A, Kb, then whether the chunk is fast; oB: beta [16]
+    // oG: gamma_C float2 [M]; oS: inverse scales of W, Y, Q, M, A, Kb, then whether the chunk is fast, then its tokens that
+    // are not finite (bit t: k, alpha, theta or beta, bit 16 + t: q); oB: beta [16]
     static constexpr int oB = oS + 32, bytes = (oB + 64 + 127) / 128 * 128;
 };
 
@@ -539,7 +593,7 @@ template <int DK, int PW>
 struct PrepMap {
     static constexpr int M = DK / 2, PAIRS = M / 2, NG = 32 * PW / PAIRS, TPT = kC / NG;
     static_assert(NG * PAIRS == 32 * PW && TPT * NG == kC && TPT >= 1, "token groups must tile the chunk");
-    static constexpr int scan_bytes = NG * PAIRS * 16 + 4 * PW * 4;          // products, phase sums, the warps' maxima
+    static constexpr int scan_bytes = NG * PAIRS * 16 + 5 * PW * 4;          // products, phase sums, the warps' maxima and tokens taken out
     static constexpr int slow_bytes = kC * (M + 4) * 8 * 3;                 // k', q', alpha of a chunk that is not fast
 };
 
@@ -593,6 +647,36 @@ __device__ __forceinline__ void prep_fetch(PrepRaw<PrepMap<DK, PW>::TPT, T> &in,
     }
 }
 
+// The rare path: a thread's tokens that are not finite in any of the warp's keys become zeros (alpha 1); the bits of the
+// warp's tokens are returned
+template <int TPT, typename T>
+__device__ __forceinline__ uint32_t take_out(PrepRaw<TPT, T> &in, int t)
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int x = 0; x < TPT; ++x) {
+        const float4 k = in.k[x].get(), q = in.q[x].get();
+        const float zk = fmaf(k.x, 0.f, fmaf(k.y, 0.f, fmaf(k.z, 0.f, k.w * 0.f))), zq = fmaf(q.x, 0.f, fmaf(q.y, 0.f, fmaf(q.z, 0.f, q.w * 0.f)));
+        const float za = fmaf(in.al[x].x, 0.f, fmaf(in.al[x].y, 0.f, fmaf(in.th[x].x, 0.f, fmaf(in.th[x].y, 0.f, fmaf(in.be[x], 0.f, zk)))));
+        if (za != 0.f) m |= 1u << (t + x);
+        if (zq != 0.f) m |= 0x10000u << (t + x);
+    }
+    m = __reduce_or_sync(0xffffffffu, m);
+    if (m) {
+#pragma unroll
+        for (int x = 0; x < TPT; ++x) {
+            if (m >> (t + x) & 1) {
+                in.k[x].zero();
+                in.al[x] = make_float2(1.f, 1.f);
+                in.th[x] = make_float2(0.f, 0.f);
+                in.be[x] = 0.f;
+            }
+            if (m >> (16 + t + x) & 1) in.q[x].zero();
+        }
+    }
+    return m;
+}
+
 // two keys of one token into the four planes
 __device__ __forceinline__ void put_planes(unsigned char *p, int pl, float r0, float i0, float r1, float i1)
 {
@@ -612,11 +696,11 @@ __device__ __forceinline__ void put_planes(unsigned char *p, int pl, float r0, f
 //
 // The division by gamma_i is bounded by 2^16 inside a fast chunk (every coordinate keeps at least 2^-16 over the 16
 // tokens): Kb's entries then reach 2^16, the smaller ones keep an absolute error of 2^-39 of that, 2^-23 beside the
-// unit-sized entries of W they meet.  Stronger decays take slow_gram.  Returns whether the chunk is fast (the same
-// value in every thread).
-template <int DK, int PW, int BAR, typename T>
-__device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, T> &in, float4 *vals, unsigned char *slot,
-                                            unsigned char *kb, unsigned char *scan, bool needq, int tid)
+// unit-sized entries of W they meet.  Stronger decays take slow_gram.  Returns whether the chunk is fast, or -1 where it
+// is not finite -- unless kAgain: this has been seen to, by leaving out the tokens `out` (the same value in every thread).
+template <int DK, int PW, int BAR, bool kAgain, typename T>
+__device__ __forceinline__ int prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, T> &in, float4 *vals, unsigned char *slot,
+                                           unsigned char *kb, unsigned char *scan, bool needq, int tid, uint32_t out)
 {
     using PM = PrepMap<DK, PW>;
     using TL = Tile<DK>;
@@ -630,7 +714,7 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
     uint2 u[TPT];
 #pragma unroll
     for (int x = 0; x < TPT; ++x) {
-        p[x] = in.al[x];
+        p[x] = make_float2(fmaf(in.th[x].x, 0.f, in.al[x].x), fmaf(in.th[x].y, 0.f, in.al[x].y));   // (NaN where theta is not finite)
         u[x] = make_uint2(phase_to_turns(in.th[x].x), phase_to_turns(in.th[x].y));
         if (x) {
             p[x] = make_float2(p[x - 1].x * p[x].x, p[x - 1].y * p[x].y);
@@ -694,19 +778,22 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
                 o[3] = make_float4(av[x].y, sf[x].y, c1, s1);
             }
             qq[x] = make_float4(av[x].x * qq[x].x, av[x].x * qq[x].y, av[x].y * qq[x].z, av[x].y * qq[x].w);
-            mq = fmaxf(fmaxf(mq, fmaxf(fabsf(qq[x].x), fabsf(qq[x].y))), fmaxf(fabsf(qq[x].z), fabsf(qq[x].w)));
+            mq = max_nan(max_nan(mq, max_nan(fabsf(qq[x].x), fabsf(qq[x].y))), max_nan(fabsf(qq[x].z), fabsf(qq[x].w)));
         }
         bi[x] = fast ? make_float2(__fdividef(in.be[x], av[x].x), __fdividef(in.be[x], av[x].y)) : make_float2(0.f, 0.f);
         const float n0 = fabsf(kk[x].x) + fabsf(kk[x].y), n1 = fabsf(kk[x].z) + fabsf(kk[x].w);   // bounds both parts
-        mw = fmaxf(mw, fmaxf(av[x].x * n0, av[x].y * n1));
-        my = fmaxf(my, fmaxf(fabsf(yf[x].x) * n0, fabsf(yf[x].y) * n1));
-        mb = fmaxf(mb, fmaxf(fabsf(bi[x].x) * n0, fabsf(bi[x].y) * n1));
+        mw = max_nan(mw, max_nan(av[x].x * n0, av[x].y * n1));
+        my = max_nan(my, max_nan(fabsf(yf[x].x) * n0, fabsf(yf[x].y) * n1));
+        mb = max_nan(mb, max_nan(fabsf(bi[x].x) * n0, fabsf(bi[x].y) * n1));
     }
     uint32_t m[4] = {__float_as_uint(mw), __float_as_uint(my), __float_as_uint(mq), __float_as_uint(mb)};   // all >= 0
 #pragma unroll
     for (int i = 0; i < 4; ++i)
         m[i] = __reduce_max_sync(0xffffffffu, m[i]);
-    if (lane == 0) *reinterpret_cast<uint4 *>(red + 4 * warp) = make_uint4(m[0], m[1], m[2], m[3]);
+    if (lane == 0) {
+        *reinterpret_cast<uint4 *>(red + 4 * warp) = make_uint4(m[0], m[1], m[2], m[3]);
+        if (kAgain) red[4 * PW + warp] = out;
+    }
     bar_sync(BAR, 32 * PW);
 #pragma unroll 2
     for (int w = 0; w < PW; ++w) {
@@ -716,6 +803,7 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
         m[2] = max(m[2], r.z);
         m[3] = max(m[3], r.w);
     }
+    if (!kAgain && max(max(m[0], m[1]), max(m[2], m[3])) >= 0x7f800000u) return -1;
     float iw, iy, iq, ib;
     const float sw = scale_for(__uint_as_float(m[0]), iw), sy = scale_for(__uint_as_float(m[1]), iy);
     const float sq = scale_for(__uint_as_float(m[2]), iq), sb = scale_for(__uint_as_float(m[3]), ib);
@@ -726,6 +814,10 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
         inv[2] = iq;
         inv[5] = ib;
         reinterpret_cast<int *>(inv)[6] = fast;
+        uint32_t all = 0;
+        if (kAgain)
+            for (int w = 0; w < PW; ++w) all |= red[4 * PW + w];
+        reinterpret_cast<uint32_t *>(inv)[7] = all;
     }
 #pragma unroll
     for (int x = 0; x < TPT; ++x) {
@@ -743,6 +835,27 @@ __device__ __forceinline__ bool prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, 
     return fast;
 }
 
+// prep_planes for a chunk that is not finite: once more, without the tokens that are not
+template <int DK, int PW, int BAR, typename T>
+__device__ __noinline__ bool prep_again(const T *q, const T *k, const float *alpha, const float *theta, const float *beta, size_t row0, int H, int t0,
+                                        int T_, float4 *vals, unsigned char *slot, unsigned char *kb, unsigned char *scan, bool needq, int tid)
+{
+    using PM = PrepMap<DK, PW>;
+    PrepRaw<PM::TPT, T> in;
+    prep_fetch<DK, PW, T>(in, q, k, alpha, theta, beta, row0, H, t0, T_, needq, tid);
+    const uint32_t out = take_out<PM::TPT, T>(in, tid / PM::PAIRS * PM::TPT);
+    return prep_planes<DK, PW, BAR, true, T>(in, vals, slot, kb, scan, needq, tid, out) != 0;
+}
+// the chunk at t0, whose inputs are in `in`
+template <int DK, int PW, int BAR, typename T>
+__device__ __forceinline__ bool prep_chunk(const PrepRaw<PrepMap<DK, PW>::TPT, T> &in, const T *q, const T *k, const float *alpha, const float *theta,
+                                           const float *beta, size_t row0, int H, int t0, int T_, float4 *vals, unsigned char *slot,
+                                           unsigned char *kb, unsigned char *scan, bool needq, int tid)
+{
+    const int fast = prep_planes<DK, PW, BAR, false, T>(in, vals, slot, kb, scan, needq, tid, 0);
+    return fast < 0 ? prep_again<DK, PW, BAR, T>(q, k, alpha, theta, beta, row0, H, t0, T_, vals, slot, kb, scan, needq, tid) : fast != 0;
+}
+
 // The Gram matrices of a chunk whose decays are too strong to divide by: every pair's decay as a running product.  Called
 // by all 32 PW threads after prep_planes returned false; `slow` is a scratch of PrepMap::slow_bytes nobody else uses.
 // Reads its inputs again: passed on, they would not stay in registers on the common path.
@@ -756,6 +869,7 @@ __device__ __noinline__ void slow_gram(const T *q, const T *k, const float *alph
     prep_fetch<DK, PW, T>(in, q, k, alpha, theta, beta, row0, H, t0, T_, needq, tid);
     constexpr int M = PM::M, PAIRS = PM::PAIRS, TPT = PM::TPT, LD = M + 4;
     const int pair = tid % PAIRS, grp = tid / PAIRS, lane = tid & 31, warp = tid >> 5;
+    take_out<PM::TPT, T>(in, grp * TPT);
     const uint2 *su = reinterpret_cast<const uint2 *>(scan + PM::NG * PAIRS * 8);
     float2 *sk = reinterpret_cast<float2 *>(slow), *sq = sk + kC * LD, *sa = sq + kC * LD;   // sa: (alpha, beta)
     uint2 ub = make_uint2(0u, 0u);

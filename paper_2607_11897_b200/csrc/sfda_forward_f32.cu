@@ -56,7 +56,8 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
             PrepRaw<L::PM::TPT, T> next;
             prep_fetch<DK, kPrepWarps, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, (c + 1) * kC, a.T, true, role.prep);
             float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes);
-            if (!prep_planes<DK, kPrepWarps, kBarAux, T>(in, nullptr, smem + slot * TL::bytes, smem + L::kb + slot * TL::BIG, smem + L::scan, true, role.prep))
+            if (!prep_chunk<DK, kPrepWarps, kBarAux, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, nullptr, smem + slot * TL::bytes,
+                                                        smem + L::kb + slot * TL::BIG, smem + L::scan, true, role.prep))
                 slow_gram<DK, kPrepWarps, kBarAux, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, c * kC, a.T, smem + L::slow, smem + L::scan,
                                                    gk, gk + 16 * 17, true, role.prep);
             bar_arrive(kBarPlanes + slot, kPrep + 64);
@@ -102,6 +103,7 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
             const uint32_t tiles[2] = {tile + TL::oW, tile + TL::oQ};
             keys_product<DK, 2>(acc, st, sr, tiles, lane, [](int, const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4]) {});
             const float fw[2] = {sr.inv[0] * inv[0], sr.inv[1] * inv[0]}, fq[2] = {sr.inv[0] * inv[2], sr.inv[1] * inv[2]};
+            uint32_t off = take_out(rr);                         // tokens whose v is not finite; below, all behind them too
 #pragma unroll
             for (int n = 0; n < 2; ++n)
 #pragma unroll
@@ -118,6 +120,13 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
                 load_small<false>(fb, tile + (pass ? TL::oA : TL::oM), lane);
                 product_small<false>(rr, ri, fr, fb, ru.inv, inv[3 + pass]);
             }
+            const uint32_t out = reinterpret_cast<const uint32_t *>(inv)[7];
+            const bool odd = __any_sync(0xffffffffu, (off | out) != 0);
+            if (odd) {
+                off = every_lanes(off, lane);
+                off = from_first(off & 0xffffu) | from_first(off >> 16) << 16 | both(from_first(out & 0xffffu));
+                put_nan(ru.inv, off);
+            }
             largest = state_update<DK>(st, fr, ru.inv, inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG), lane);
             if (c + kSlots < nch) bar_arrive(kBarDone + slot, kPrep + kChain);
 #pragma unroll
@@ -127,6 +136,10 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_forward_f
                     rr[n][i] = fmaf(fq[i >> 1], acc[1][0][n][i], rr[n][i]);
                     ri[n][i] = -fmaf(fq[i >> 1], acc[1][1][n][i], ri[n][i]);
                 }
+            if (odd) {
+                put_nan(rr, off | both(out >> 16), lane);
+                put_nan(ri, off | both(out >> 16), lane);
+            }
             store_rows(static_cast<T *>(a.o) + at, rr, step, left);
             if (a.o_im) store_rows(static_cast<T *>(a.o_im) + at, ri, step, left);
         }

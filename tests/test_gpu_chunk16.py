@@ -195,3 +195,46 @@ def test_an_infinite_channel_leaves_the_others_alone(what, where):
     others = np.arange(128) != 5
     for a, b in zip(run(), want):
         assert np.array_equal(a[..., others], b[..., others])
+
+
+# Which tokens' results an input that is not finite at token t leaves alone, by what depends on what in the recurrence and
+# its adjoint: < t, > t or all of them.
+UNTOUCHED = {
+    "q": dict(o="!", S_T="all", dq="all", dk=">", dv=">", dbeta=">", dalpha=">", dtheta=">"),
+    "k": dict(o="<", dq="<", dv=">"),
+    "alpha": dict(o="<", dq="<", dv=">"),
+    "theta": dict(o="<", dq="<", dv=">"),
+    "beta": dict(o="<", dq="<", dv=">"),
+    "v": dict(o="<", dq="<", dk="<", dv="all", dbeta="<", dS0="all"),
+    "do_re": dict(o="all", S_T="all", dq="!", dk=">", dv=">", dbeta=">", dalpha=">", dtheta=">")}
+
+
+@pytest.mark.parametrize("B,H,d_k,d_v", [(1, 2, 128, 128), (1, 2, 64, 64), (5, 16, 64, 128), (5, 32, 128, 128)])
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("what", sorted(UNTOUCHED))
+def test_a_token_that_is_not_finite_reaches_only_what_depends_on_it(what, value, B, H, d_k, d_v):
+    cfg = workloads.CONFIGS[0].scaled(name="c16f", B=B, T=100, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=740)
+    inp, up = workloads.forward_inputs(cfg), upstream(cfg, 6)
+
+    def run():
+        o, _, S_T = run_forward(cfg, inp)
+        return dict(run_backward(cfg, inp, up), o=o, S_T=S_T)
+    want, t = run(), 37
+    x = inp[what] if what in inp else up[what]
+    x[(0, t, 0) + (5,) * (x.ndim - 3)] = value
+    got = run()
+    token = np.arange(cfg.T)
+    for name, tokens in UNTOUCHED[what].items():
+        w, g = want[name], got[name]
+        assert np.array_equal(w[0, 1] if name in ("S_T", "dS0") else w[0, :, 1], g[0, 1] if name in ("S_T", "dS0") else g[0, :, 1])   # another head
+        if name in ("S_T", "dS0"):
+            w, g = w[0, 0], g[0, 0]
+        else:
+            keep = {"<": token < t, ">": token > t, "!": token != t, "all": token >= 0}[tokens]
+            w, g = w[0, keep, 0], g[0, keep, 0]
+        assert np.abs(g - w).max() <= 2e-6 * np.abs(w).max(), (what, name)      # (zeros in the token's place may move a scale)
+    # ... and everything that does depend on it shows it
+    for name in ("o", "dq", "dk", "dbeta"):
+        assert not np.isfinite(got[name][0, t, 0]).all() or (what, name) in (("q", "dq"), ("do_re", "o")), (what, name)
+    if what != "q":
+        assert not np.isfinite(got["S_T"][0, 0]).all() or what == "do_re"
