@@ -67,7 +67,7 @@ struct BwdArgsDev {
 // The head of the workspace: the status word and, 256 bytes behind it, the flags of at most kBwdTargetCtas CTAs.
 constexpr int kBwdTargetCtas = 148;
 constexpr size_t kHeadBytes = 1024;
-constexpr unsigned long long kChunkTicks = 1ull << 23;           // more than any chunk takes
+constexpr unsigned long long kChunkTicks = 1ull << 22;           // more than any chunk takes
 static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags follow the status block");
 
 // One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
@@ -202,61 +202,114 @@ __device__ __forceinline__ SlowOut slow_corrections(const float4 *vals, int M, c
     return o;
 }
 
-// dalpha of one (token tl, key) from its definition, by one warp: S_{t-1} and the cotangent of Lambda_t S_{t-1} rebuilt
-// from the boundary matrices, value column by value column.
+// dalpha and dtheta from their definition instead of from D, by a warp for the keys of its tile:  Re H and alpha Im H with
+// H = sum_c conj(S'_c) Z'_c over the value columns, where e^{i phi_{t-1}} S' is the state before token t and e^{i phi_t} Z'
+// the cotangent of Lambda_t S_{t-1}.  Written out over S_0, the tokens before t, G_C and the tokens from t on, every sum
+// over the columns is one that the chunk's products have already made (X1, X2, X3 before they are corrected, U Yb^T, U B^T)
+// or sum_c conj(S_0) G_C, made here; decays come as running products.  x: the thread's tokens g, g + 8 and keys 2 t4, + 1.
+// redo: bit 2 r + e says that this element is wanted; it goes to the caller's arrays.
+// (Rebuilding both matrices per element, column by column, took 6.4 M cycles a chunk where every alpha is small.)
 template <int DK, int NB>
-__device__ __forceinline__ float small_alpha(const float4 *vals, const uint4 *frag, const uint4 *pS, const uint4 *pG, const float *sc,
-                                          const float *yscal, const float *alpha, const float *theta, const float *beta,
-                                          size_t row0, int H, int t0, int T_, int tl, int kt, int kl, int lane)
+__device__ __forceinline__ void from_definition(const BwdArgsDev &a, const float4 *vals, const float2 *uy, const uint4 *pS, const uint4 *pG, const float *sc,
+                                                const float (&x1r)[4], const float (&x1i)[4], const float (&x2r)[4], const float (&x2i)[4],
+                                                const float (&x3r)[4], const float (&x3i)[4], unsigned redo, size_t row0, int t0, int kt, int lane)
 {
     constexpr int NCW = NB / 16, M = DK / 2, KT = M / 8;
-    const int key = 8 * kt + kl;
-    float sum = 0.f, cst = 1.f, snt = 0.f;
-    for (int val = lane; val < NB; val += 32) {
-        const int w = val >> 4, vl = val & 15, hf = vl & 1;
-        auto state = [&](const uint4 *base, float inv) {
-            const uint32_t *p = reinterpret_cast<const uint32_t *>(base + ((w * KT + kt) * 2) * 32 + 4 * kl + ((vl & 7) >> 1)) + (vl >> 3);
-            return make_float2(inv * join_half(p[0], p[2], hf), inv * join_half(p[128], p[130], hf));
-        };
-        auto token = [&](int mat, int tok, float inv) {
-            const uint32_t *p = reinterpret_cast<const uint32_t *>(frag + (mat * NCW + w) * 128 + 4 * (tok & 7) + ((vl & 7) >> 1)) + (tok >> 3) + 2 * (vl >> 3);
-            return make_float2(inv * join_half(p[0], p[128], hf), inv * join_half(p[256], p[384], hf));
-        };
-        float2 s = state(pS, sc[4 * w]), z = state(pG, sc[4 * w + 2]);
-        for (int j = 0; j < tl; ++j) {               // S_{t-1}
-            const size_t rj = row0 + (size_t)(t0 + j) * H;
-            const float4 x = vals[(j * M + key) * 2], y = vals[(j * M + key) * 2 + 1];
-            float sn, cs;
-            sincosf(theta[rj * M + key], &sn, &cs);
-            const float aj = alpha[rj * M + key], bj = beta[rj];
-            const float2 kj = cmul(make_float2(y.z, y.w), make_float2(bj * x.x, bj * x.y)), u = token(2, j, sc[4 * w + 1]);
-            s = cmul(make_float2(aj * cs, aj * sn), s);
-            const float2 p = cmul(kj, u);
-            s = make_float2(s.x + p.x, s.y + p.y);
+    const int g = lane >> 2, t4 = lane & 3, key = 8 * kt + 2 * t4, left = a.T - t0;
+    float2 r0 = make_float2(0.f, 0.f);                            // of key g: four channels of every warp per lane
+#pragma unroll 1
+    for (int w = 0; w < NCW; ++w) {
+        const uint4 sr = pS[(w * KT + kt) * 64 + lane], si = pS[(w * KT + kt) * 64 + 32 + lane];
+        const uint4 gr = pG[(w * KT + kt) * 64 + lane], gi = pG[(w * KT + kt) * 64 + 32 + lane];
+        float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            auto at = [&](const uint4 &v) { return join_half(c < 2 ? v.x : v.y, c < 2 ? v.z : v.w, c & 1); };
+            const float2 p = cmulc(make_float2(at(sr), at(si)), make_float2(at(gr), at(gi)));
+            sum = make_float2(sum.x + p.x, sum.y + p.y);
         }
-        for (int l = min(15, T_ - 1 - t0); l >= tl; --l) {     // the cotangent of Lambda_t S_{t-1}
-            const size_t rl = row0 + (size_t)(t0 + l) * H;
-            const float4 x = vals[(l * M + key) * 2], y = vals[(l * M + key) * 2 + 1];
-            const float2 ph = make_float2(y.z, y.w), ql = cmul(ph, make_float2(x.z, x.w)), kj = cmul(ph, make_float2(x.x, x.y));
-            const float2 yb = token(0, l, yscal[w]), bc = token(1, l, sc[4 * w + 3]);
-            const float2 p = cmulc(yb, ql), m = cmul(kj, bc);
-            z = make_float2(z.x + p.x - m.x, z.y + p.y - m.y);
-            float sn, cs;
-            sincosf(theta[rl * M + key], &sn, &cs);
-            if (l > tl) {
-                const float aj = alpha[rl * M + key];
-                z = cmulc(make_float2(aj * cs, aj * sn), z);
-            } else {
-                cst = cs;
-                snt = sn;
-            }
-        }
-        const float2 lb = cmulc(s, z);
-        sum += lb.x * cst + lb.y * snt;              // Re(conj(lambda bar) e^{i theta})
+        const float f = sc[4 * w] * sc[4 * w + 2];
+        r0 = make_float2(fmaf(f, sum.x, r0.x), fmaf(f, sum.y, r0.y));
     }
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-    return sum;
+    for (int d = 1; d < 4; d <<= 1) {
+        r0.x += __shfl_xor_sync(0xffffffffu, r0.x, d);
+        r0.y += __shfl_xor_sync(0xffffffffu, r0.y, d);
+    }
+    // an element (token, key 2 t4 + e) of another thread's tile
+    auto other = [&](const float(&re)[4], const float(&im)[4], int t, int e) {
+        const int src = 4 * (t & 7) + t4;
+        const float u = t < 8 ? re[e] : re[2 + e], v = t < 8 ? im[e] : im[2 + e];
+        return make_float2(__shfl_sync(0xffffffffu, u, src), __shfl_sync(0xffffffffu, v, src));
+    };
+    float2 s0[2], wt[16][2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) s0[e] = make_float2(__shfl_sync(0xffffffffu, r0.x, 4 * (2 * t4 + e)), __shfl_sync(0xffffffffu, r0.y, 4 * (2 * t4 + e)));
+#pragma unroll 1
+    for (int r = 0; r < 2; ++r) {
+        const int t = g + 8 * r;
+        float pw[2] = {1.f, 1.f}, pz[2] = {1.f, 1.f};
+        float2 h[2], sx[2], su[2];                                // with S_0, with G_C and u_i, with u_i and the tokens from t on
+#pragma unroll
+        for (int e = 0; e < 2; ++e) h[e] = sx[e] = su[e] = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int i = 14; i >= 0; --i) {                           // prod alpha behind i up to t - 1, beta_i conj(k'_i)
+            const float2 x3[2] = {other(x3r, x3i, i, 0), other(x3r, x3i, i, 1)};
+            if (i >= t || i >= left) continue;
+            const size_t row = row0 + (size_t)(t0 + i) * a.H;
+            const float be = a.beta[row];
+            const float2 al = *reinterpret_cast<const float2 *>(a.alpha + row * M + key);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float4 v = vals[(i * M + key + e) * 2];
+                const float2 w = make_float2(pw[e] * be * v.x, -pw[e] * be * v.y), p = cmul(w, x3[e]);
+                wt[i][e] = w;
+                sx[e] = make_float2(sx[e].x + p.x, sx[e].y + p.y);
+                pw[e] *= e ? al.y : al.x;
+            }
+        }
+#pragma unroll 1
+        for (int l = 0; l < 16; ++l) {                            // prod alpha behind t up to l
+            const float2 x1[2] = {other(x1r, x1i, l, 0), other(x1r, x1i, l, 1)}, x2[2] = {other(x2r, x2i, l, 0), other(x2r, x2i, l, 1)};
+            if (l < t || l >= left) continue;
+            if (l > t) {
+                const float2 al = *reinterpret_cast<const float2 *>(a.alpha + (row0 + (size_t)(t0 + l) * a.H) * M + key);
+                pz[0] *= al.x;
+                pz[1] *= al.y;
+            }
+            float2 q[2], k[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float4 v = vals[(l * M + key + e) * 2];
+                k[e] = make_float2(pz[e] * v.x, pz[e] * v.y);
+                q[e] = make_float2(pz[e] * v.z, pz[e] * v.w);
+                const float2 p = cmulc(x1[e], q[e]), m = cmulc(x2[e], k[e]);
+                h[e] = make_float2(h[e].x + p.x - m.x, h[e].y + p.y - m.y);
+            }
+#pragma unroll 1
+            for (int i = 0; i < t; ++i) {
+                const float2 *u = uy + i * 17 + l;
+                const float2 y = make_float2(u[0].x + u[544].x, u[0].y + u[544].y), b = make_float2(u[272].x + u[816].x, u[272].y + u[816].y);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float2 p = cmulc(y, q[e]), m = cmulc(b, k[e]), x = cmul(wt[i][e], make_float2(p.x - m.x, p.y - m.y));
+                    su[e] = make_float2(su[e].x + x.x, su[e].y + x.y);
+                }
+            }
+        }
+        if (t >= left) continue;
+        const size_t row = row0 + (size_t)(t0 + t) * a.H;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float4 v = vals[(15 * M + key + e) * 2 + 1];    // -, -, e^{i phi_C}
+            const float2 end = make_float2(pz[e] * v.z, -pz[e] * v.w), z0 = cmul(end, s0[e]), zx = cmul(end, sx[e]);
+            const float hr = fmaf(pw[e], h[e].x + z0.x, su[e].x + zx.x), hi = fmaf(pw[e], h[e].y + z0.y, su[e].y + zx.y);
+            if (redo >> (2 * r + e) & 1) {
+                a.dalpha[row * M + key + e] = hr;
+                a.dtheta[row * M + key + e] = a.alpha[row * M + key + e] * hi;
+            }
+        }
+    }
 }
 
 // ---- PREP, second task: what the gradients of a chunk need of its tokens -----------------------------------
@@ -513,6 +566,28 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     bar_sync(kBarTri, kPrep + kGrad);
 
     if (warp < KT) {
+        if (first) {                                               // D at the segment's end
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                carry[e] = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int w = 0; w < NCW; ++w) {
+                    const float2 x = rg[w * M + 8 * warp + 2 * t4 + e];
+                    carry[e] = make_float2(carry[e].x + x.x, carry[e].y + x.y);
+                }
+            }
+        }
+        // D / alpha loses digits where alpha is small, and D takes up all that is not finite up to the segment's end: those
+        // elements come from the definition
+        constexpr float kSmall = 0.0625f;
+        unsigned redo = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float x = i & 1 ? al2[i >> 1].y : al2[i >> 1].x, d = (carry[i & 1].x + carry[i & 1].y) * 0.f;
+            if (x < kSmall || d != 0.f) redo |= 1u << i;
+        }
+        const bool some = __any_sync(0xffffffffu, redo != 0);
+        if (some) from_definition<DK, NB>(a, vals, uy, pS, pG, sc, x1r, x1i, x2r, x2i, x3r, x3i, redo, row0, t0, warp, lane);
         const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
         const bool fast = reinterpret_cast<const int *>(inv)[6] != 0;
         const unsigned char *slot_at = smem + slot * TL::bytes;
@@ -597,9 +672,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 put(x3i, o.fb.y);
             }
         }
-        // the staged operands are needed further only where a slow path rebuilds something from them
-        const bool keep = !fast || __any_sync(0xffffffffu, fminf(fminf(al2[0].x, al2[0].y), fminf(al2[1].x, al2[1].y)) < 0.0625f);
-        if (!last_one && !keep) bar_arrive(kBarTaken, kGrad + kPrep);
+        if (!last_one) bar_arrive(kBarTaken, kGrad + kPrep);
         float2 dqv[4], dkv[4], dd[4];
         float al[4], dbp[2] = {0.f, 0.f};
 #pragma unroll
@@ -644,17 +717,6 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             }
         }
         // D: sums over the tokens behind, down to each token (tokens 8-15 in i = 2, 3, tokens 0-7 in i = 0, 1)
-        if (first) {
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                carry[e] = make_float2(0.f, 0.f);
-#pragma unroll 1
-                for (int w = 0; w < NCW; ++w) {
-                    const float2 x = rg[w * M + 8 * warp + 2 * t4 + e];
-                    carry[e] = make_float2(carry[e].x + x.x, carry[e].y + x.y);
-                }
-            }
-        }
 #pragma unroll
         for (int d = 4; d < 32; d <<= 1)
 #pragma unroll
@@ -671,25 +733,6 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         float dal[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) dal[i] = __fdividef(dd[i].x, al[i]);
-        // small alpha: from the definition, one (token, key) at a time
-        if (__any_sync(0xffffffffu, fminf(fminf(al[0], al[1]), fminf(al[2], al[3])) < 0.0625f)) {
-#pragma unroll 1
-            for (int i = 0; i < 4; ++i) {
-                unsigned todo = __ballot_sync(0xffffffffu, (i == 0 ? al[0] : i == 1 ? al[1] : i == 2 ? al[2] : al[3]) < 0.0625f);
-                while (todo) {
-                    const int src = __ffs(todo) - 1;
-                    todo &= todo - 1;
-                    const float sum = small_alpha<DK, NB>(vals, frag, pS, pG, sc, yscal, a.alpha, a.theta, a.beta, row0, a.H, t0, a.T,
-                                                          (src >> 2) + 8 * (i >> 1), warp, 2 * (src & 3) + (i & 1), lane);
-                    if (lane == src) {
-                        if (i == 0) dal[0] = sum;
-                        else if (i == 1) dal[1] = sum;
-                        else if (i == 2) dal[2] = sum;
-                        else dal[3] = sum;
-                    }
-                }
-            }
-        }
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int t = t0 + g + 8 * r;
@@ -698,7 +741,11 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 const size_t ak = row * DK + 2 * (8 * warp + 2 * t4), am = row * M + 8 * warp + 2 * t4;
                 const float4 q4 = make_float4(dqv[2 * r].x, dqv[2 * r].y, dqv[2 * r + 1].x, dqv[2 * r + 1].y);
                 const float4 k4 = make_float4(dkv[2 * r].x, dkv[2 * r].y, dkv[2 * r + 1].x, dkv[2 * r + 1].y);
-                const float2 a2 = make_float2(dal[2 * r], dal[2 * r + 1]), th2 = make_float2(dd[2 * r].y, dd[2 * r + 1].y);
+                float2 a2 = make_float2(dal[2 * r], dal[2 * r + 1]), th2 = make_float2(dd[2 * r].y, dd[2 * r + 1].y);
+                if (some) {                                        // (written by this thread, above)
+                    if (redo >> 2 * r & 1) a2.x = a.dalpha[am], th2.x = a.dtheta[am];
+                    if (redo >> 2 * r & 2) a2.y = a.dalpha[am + 1], th2.y = a.dtheta[am + 1];
+                }
                 st_val4(static_cast<T *>(a.dq) + ak, q4);
                 st_val4(static_cast<T *>(a.dk) + ak, k4);
                 *reinterpret_cast<float2 *>(a.dalpha + am) = a2;
@@ -710,7 +757,6 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             // (a query that was taken out is missing from its own token's sum)
             if (t4 == 0) db[warp * 16 + g + 8 * r] = reinterpret_cast<const uint32_t *>(inv)[7] >> (16 + g + 8 * r) & 1 ? __int_as_float(0x7fc00000) : x;
         }
-        if (!last_one && keep) bar_arrive(kBarTaken, kGrad + kPrep);
     } else if (!last_one) {
         bar_arrive(kBarTaken, kGrad + kPrep);
     }
@@ -1117,7 +1163,7 @@ __global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_backward_
 // the kept final state, and a CTA only waits for what the CTA before it in the grid does first.  256 pairs of 8192 tokens
 // on 148 SMs, with the forward and the passes around it: 30.5 ms as two rounds of whole pairs, 27.5 ms cut.
 // The launch is cooperative, so that both CTAs run, and the wait is bounded by what the other's part can take at most: a
-// chunk takes 57 k cycles, and up to 6.4 M where every alpha is below 1/16.  Where it runs out all the same, the status
+// chunk takes 60 k cycles, and 250 k where every alpha is below 1/16.  Where it runs out all the same, the status
 // word is set and the part is not walked: its gradients become NaN.  (Signs of life instead of a bound, one store per
 // segment, cost 1.3 % of the walk, in the chain's warps as in the gradients'.)
 // kUnits == true: S and G are kept already; a CTA takes units (pair, segment) blockIdx.x, + gridDim.x, ...
