@@ -522,20 +522,20 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 const uint4 *fy = frag + w * 128 + lane;
                 const uint4 h = fy[0], l = fy[32];
                 const uint32_t ah[4] = {h.x, h.y, h.z, h.w}, al[4] = {l.x, l.y, l.z, l.w};
-                float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mr[4] = {0.f, 0.f, 0.f, 0.f};
+                float pr[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f}, mr[4] = {0.f, 0.f, 0.f, 0.f}, mi[4] = {0.f, 0.f, 0.f, 0.f};
                 mma3x<kExact>(pr, ah, al, s0.x, s0.y, s0.z, s0.w);
                 mma3x<kExact>(pi, ah, al, s1.x, s1.y, s1.z, s1.w);
                 if (has_im) {
                     const uint4 h2 = fy[64], l2 = fy[96];
                     const uint32_t bh[4] = {h2.x, h2.y, h2.z, h2.w}, bl[4] = {l2.x, l2.y, l2.z, l2.w};
                     mma3x<kExact>(mr, bh, bl, s1.x, s1.y, s1.z, s1.w);
-                    mma3x<kExact>(pi, bh, bl, s0.x, s0.y, s0.z, s0.w);
+                    mma3x<kExact>(mi, bh, bl, s0.x, s0.y, s0.z, s0.w);
                 }
                 const float f = sc[4 * w] * yscal[w];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     x1r[i] = fmaf(f, pr[i] - mr[i], x1r[i]);
-                    x1i[i] = fmaf(f, pi[i], x1i[i]);
+                    x1i[i] = fmaf(f, pi[i] + mi[i], x1i[i]);
                 }
             }
             conj_product(frag + (NCW + w) * 128 + lane, s0, s1, sc[4 * w] * sc[4 * w + 3], x2r, x2i);
@@ -623,14 +623,19 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 }
             };
             const float4 gm = reinterpret_cast<const float4 *>(slot_at + TL::oG)[4 * warp + t4];   // gamma_C of the two keys
+            // 1 / |gamma_C|^2 and 1 / |gamma_C|, the latter with a Newton step (the instruction is good to 23 bits)
             const float n2[2] = {gm.x * gm.x + gm.y * gm.y, gm.z * gm.z + gm.w * gm.w};
+            const float i2[2] = {__frcp_rn(n2[0]), __frcp_rn(n2[1])};
+            float i1[2] = {rsqrtf(n2[0]), rsqrtf(n2[1])};
+#pragma unroll
+            for (int e = 0; e < 2; ++e) i1[e] = fmaf(0.5f * i1[e], fmaf(-n2[e] * i1[e], i1[e], 1.f), i1[e]);
             float zr[4], zi[4];
             // a_t (X + conj(gamma_C) Z / |gamma_C|^2), the scale f of Z included
             auto fold = [&](float f, float (&xr)[4], float (&xi)[4]) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int e = i & 1;
-                    const float w = __fdividef(f, n2[e]);
+                    const float w = f * i2[e];
                     const float2 z = cmulc(e ? make_float2(gm.z, gm.w) : make_float2(gm.x, gm.y), make_float2(w * zr[i], w * zi[i]));
                     xr[i] = va[i].x * (xr[i] + z.x);
                     xi[i] = va[i].x * (xi[i] + z.y);
@@ -647,7 +652,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int e = i & 1;
-                const float s = va[i].y * rsqrtf(n2[e]), down = __frcp_rn(va[i].x);      // 1 / a_t: at most 2^16
+                const float s = va[i].y * i1[e], down = __frcp_rn(va[i].x);      // 1 / a_t: at most 2^16
                 const float2 z = cmulc(e ? make_float2(gm.z, gm.w) : make_float2(gm.x, gm.y), make_float2(x3r[i], x3i[i]));
                 x3r[i] = fmaf(s, z.x, down * fmaf(f2, zr[i], f3 * wr[i]));
                 x3i[i] = fmaf(s, z.y, down * fmaf(f2, zi[i], f3 * wi[i]));
