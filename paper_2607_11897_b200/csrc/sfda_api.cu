@@ -105,7 +105,7 @@ int check_param_scalars(float alpha_min, float alpha_max, float theta_max, float
     return ok ? SFDA_OK : SFDA_ERR_VALUE;
 }
 
-// workspace of sfda_forward_fused on the CUDA-core shapes: alpha, theta, beta and the normalised key
+// workspace of sfda_forward_fused on the shapes of the fp32 forward: alpha, theta, beta and the normalised key
 size_t staged_frontend_bytes(size_t rows, int d_k, int dtype)
 {
     return 2 * round256(rows * (d_k / 2) * 4) + round256(rows * 4) + round256(rows * d_k * elem_bytes(dtype));
@@ -658,7 +658,7 @@ int sfda_forward_fused(const void *q, const void *k_raw, const void *v, const fl
         return sfda::launch_forward_ws(a, workspace, workspace_bytes, s, &g_last_launches) == cudaSuccess ? SFDA_OK
                                                                                                           : SFDA_ERR_CUDA;
     }
-    // other shapes: the parameterisation as a kernel of its own into the workspace, then the CUDA-core forward
+    // other shapes: the parameterisation as a kernel of its own into the workspace, then the fp32 forward
     const size_t rows = (size_t)B * T * H;
     if (!workspace || workspace_bytes < staged_frontend_bytes(rows, d_k, dtype)) return SFDA_ERR_WORKSPACE;
     char *w = static_cast<char *>(workspace);

@@ -7,9 +7,9 @@
 // One CTA per (batch, head) pair and block of value columns; sfda_chunk16.cuh describes the arithmetic (split fp16 on
 // the tensor cores) and the two roles, which are pipelined over a ring of operand tiles.
 //
-// What bounds it: the schedulers' issue slots, which mma.sync holds (see ChainRoles).  Measured in cycles per 16 tokens:
-// 6.4 k with 32 value columns per CTA (B = 2, T = 2001, H = 16, d = 128, fp32: 422 us; the unrolled first version 665 us,
-// the CUDA-core kernel 3154 us), 11.4 k with 128 columns; B = 1, T = 256, H = 2, d = 64: 43 us (61, 201).
+// What bounds it: the schedulers' issue slots, which mma.sync holds (see ChainRoles), and the latency of the chain.
+// B = 2, T = 2001, H = 16, d = 128, fp32: 457 us, 6.9 k cycles per 16 tokens with 32 value columns per CTA (the unrolled first
+// version 665 us, the CUDA-core kernel 3154 us); B = 1, T = 256, H = 2, d = 64: 39 us (61, 201).
 #include "sfda_chunk16.cuh"
 #include "sfda_internal.h"
 
@@ -165,7 +165,8 @@ cudaError_t launch_nb(const ForwardArgs &x, cudaStream_t stream)
 }
 
 // Value columns per CTA: all of them when the (batch, head) pairs fill the SMs, halved (down to 32) while the grid
-// still fits: every block of columns repeats the chunk preparation, which runs beside the chain.
+// still fits: every block of columns repeats the chunk preparation, which runs beside the chain.  (148: the SMs of a B200.
+// On another device the blocks are merely not the best ones.)
 template <int DK, typename T>
 cudaError_t launch_typed(const ForwardArgs &x, cudaStream_t stream)
 {

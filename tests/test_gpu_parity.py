@@ -1163,12 +1163,14 @@ def run_backward(cfg, inp, up):
                        u["dS_T"], out["dq"], out["dk"], out["dv"], out["dalpha"], out["dtheta"], out["dbeta"],
                        out["dS0"], ws)
     torch.cuda.synchronize()
-    assert sfda.last_launch_count() == (2 if blocks > 1 else 1)   # the sweeps, then the sum of the blocks' shares
+    assert sfda.last_launch_count() == (2 if blocks > 1 else 1)   # few sequences: the chains, then the segments; else the walk
+    assert sfda.sfda_workspace_status(ws) == 0
     return {k: v.float().cpu().numpy() for k, v in out.items()}
 
 
 def backward_column_blocks(B, H, d_v):
-    """Column blocks per state: the value columns are halved (down to 32 per CTA) while the grid fits 148 SMs."""
+    """More than 1 for few sequences: the rule that the workspace's size (it has room for a share per block) and the choice of
+    two launches follow: value columns are halved (down to 32) while the grid fits 148 SMs."""
     cols = d_v
     while cols > 32 and B * H * (d_v // (cols // 2)) <= 148:
         cols //= 2
@@ -1214,8 +1216,9 @@ def test_backward_matches_oracle(d_k, d_v, T, dtype):
 
 @pytest.mark.parametrize("B,H,d_v,blocks", [(5, 8, 128, 2), (19, 8, 128, 1), (10, 8, 64, 1), (3, 3, 64, 2)])
 def test_backward_column_blocks(B, H, d_v, blocks):
-    """Few sequences split the value columns over more CTAs (shares summed by a second kernel); many do not."""
-    assert backward_column_blocks(B, H, d_v) == blocks
+    """Few sequences run as chains and segments (two launches), many as one walk; run_backward checks which against
+    the library's launch count, and the workspace's size."""
+    assert backward_column_blocks(B, H, d_v) == blocks             # (which side of the rule this case is for)
     cfg = workloads.CONFIGS[0].scaled(name="bwd_blocks", B=B, T=70, H=H, d_k=64, d_v=d_v, dtype="bf16", s0_std=0.5,
                                       seed=85 + B)
     inp = workloads.forward_inputs(cfg)
