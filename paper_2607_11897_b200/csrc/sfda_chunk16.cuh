@@ -178,8 +178,9 @@ __device__ __forceinline__ RowScale row_scale(float2 m)
     RowScale r;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        const uint32_t e = max((i ? x >> 23 : (x << 16) >> 23), 27u);
-        r.inv[i] = __uint_as_float(kStep == 1 ? (e - 14u) << 23 : ((e + kStep & ~(uint32_t)(kStep - 1)) - 15u) << 23);
+        // exponent + 1; that of an infinity or NaN counts as the smallest, so that it does not decide a shared scale
+        const uint32_t e = max((i ? x >> 23 : (x << 16) >> 23) + 1u & 255u, 28u);
+        r.inv[i] = __uint_as_float(kStep == 1 ? (e - 15u) << 23 : ((e + (kStep - 1) & ~(uint32_t)(kStep - 1)) - 15u) << 23);
     }
     return r;
 }
@@ -431,8 +432,7 @@ __device__ __forceinline__ RowScale make_frag(TokFrag &f, const float (&re)[2][4
     split_tiles(im[0], im[1], r, f.ih, f.il);
     return r;
 }
-// The inverse of the scale for sums over a warp's channels: that of its largest row (2^114 or an infinity's aside); own: some
-// row has another.
+// The inverse of the scale for sums over a warp's channels: that of its largest row; own: some row has another.
 __device__ __forceinline__ float shared_scale(const RowScale &r, bool &own)
 {
     const float all = warp_max(fmaxf(r.inv[0], r.inv[1]));

@@ -197,6 +197,19 @@ def test_an_infinite_channel_leaves_the_others_alone(what, where):
         assert np.array_equal(a[..., others], b[..., others])
 
 
+@pytest.mark.parametrize("what", ["S0", "dS_T"])
+def test_an_infinite_state_entry_makes_no_sum_over_the_channels_finite_and_wrong(what):
+    cfg = workloads.CONFIGS[0].scaled(name="c16j", B=1, T=40, H=2, d_k=128, d_v=128, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=731)
+    inp, up = workloads.forward_inputs(cfg), upstream(cfg, 5)
+    want = run_backward(cfg, inp, up)
+    (inp if what in inp else up)[what][0, 0, 3, 5] = np.inf
+    got = run_backward(cfg, inp, up)
+    for name in ("dq", "dk", "dalpha", "dtheta", "dbeta"):
+        on = np.isfinite(got[name])
+        assert np.abs(got[name] - want[name])[on].max() <= 2e-6 * np.abs(want[name]).max(), name
+        assert on[0, :, 1].all() and (not on[0, :, 0].all() or (what, name) == ("dS_T", "dq"))
+
+
 # Which tokens' results an input that is not finite at token t leaves alone, by what depends on what in the recurrence and
 # its adjoint: < t, > t or all of them.
 UNTOUCHED = {
