@@ -11,13 +11,14 @@
 //              G_0 = conj(gamma_C) G_C + Q^T Yb^* - W^T Bc
 //   gradients  dq_t = S_t yb_t,   f_t = G_t conj(u_t),   z_t = Lambda_t S_{t-1} (beta_t p_t),
 //              dk_t = beta_t f_t - z_t,   dbeta_t = Re(f_t^* k_t),
-//              D_t = D_{t+1} + q_t conj(dq_t) - beta_t conj(k_t) f_t - k_t conj(z_t)    (D_{T+1} = rowdot(S_T, G_T)),
+//              D_t = D_{t+1} + q_t conj(dq_t) - beta_t conj(k_t) f_t - k_t conj(z_t)    (behind a chunk: rowdot(S_C, G_C)),
 //              dalpha_t = Re D_t / alpha_t,   dtheta_t = Im D_t
 //
 // where S_t, G_t inside a chunk are S_0, G_C plus rank-16 corrections, so dq, f, z come from three products with the
 // boundary matrices (S_0 Yb^T, S_0 B^T, G_C U^H), two 16 x 16 matrices U Yb^T, U B^T and triangular products with the
 // decayed keys and queries.  Where alpha_t < 1/16 the division would lose digits: dalpha comes from its definition,
-// sum_c conj(S_{t-1,jc}) Zb_jc, rebuilt for that (token, coordinate) alone.
+// sum_c conj(S_{t-1,jc}) Zb_jc, written out over the chunk's own products (from_definition).  D is made anew behind every
+// chunk from sum_c conj(S_0) G_C: it runs over at most 16 tokens (over 64: dalpha 5.4e-7 from 64 bits instead of 3.3e-7).
 //
 // A (batch, head) pair is walked forward once, keeping the state every 64 tokens, then per segment of 64 tokens, last to
 // first: forward again from the kept state, backward through it; the walks of all pairs are cut into one equal piece per
@@ -28,10 +29,11 @@
 // (a tile is complete), DONE (the chain came back through the chunk); READY (the gradients are through with the slot),
 // STAGED and TAKEN (the tokens are there, and free again).
 //
-// What bounds it: 57 k cycles per 16 tokens of a pair at d_k = d_v = 128, 12.6 k of them in the first sweep.  mma.sync
-// holds 29 % of the tensor pipe's time, issue slots are 33 % used: the rest is the latency of the two chains (about 11 k
-// cycles a step each, alone) under roles that share the schedulers.  B = 8, T = 8192, H = 32, bf16: 24.7 ms (the
-// token-level adjoint on the CUDA cores: 145 ms); B = 4, T = 4096, H = 16: chains 1.5 ms, units 2.5 ms.
+// What bounds it: about 60 k cycles per 16 tokens of a pair at d_k = d_v = 128 (57 k, 12.6 k of them in the first sweep, with
+// mma.sync holding 29 % of the tensor pipe's time and issue slots 33 % used, before sums over the keys were rounded to
+// nearest and channels had scales of their own): the latency of the two chains under roles that share the schedulers.
+// Training step on raw inputs, B = 8, T = 8192, H = 32, bf16: 29.4 ms (the token-level adjoint on the CUDA cores: 148 ms);
+// B = 4, T = 4096, H = 16: 4.5 ms (21.8).
 #include "sfda_chunk16.cuh"
 #include "sfda_internal.h"
 
@@ -73,13 +75,13 @@ static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags 
 // One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
 // S_0, G_C as B operands [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U, Bc as A operands
 // [chain warp][plane][lane] uint4; then the chunk's rotated keys and queries, decays and phases, 8 floats per
-// (token, key).  Behind the ring: rowdot(S, G) [2][chain warp][key] and slow_gram's scratch.
+// (token, key).  Behind the ring: slow_gram's scratch.
 template <int DK, int NB>
 struct BwdScratch {
     static constexpr int NCW = NB / 16, KT = DK / 16, M = DK / 2;
     static constexpr int oS = 0, oU = oS + NCW * KT * 1024, oG = oU + NCW * 2048, oB = oG + NCW * KT * 1024;
     static constexpr int oV = oB + NCW * 2048, slot = oV + 16 * M * 32;
-    static constexpr int oRg = slot * kSlots, oSlow = oRg + 2 * NCW * M * 8;
+    static constexpr int oSlow = slot * kSlots;
     static constexpr size_t bytes = (oSlow + PrepMap<DK, kPrepWarps>::slow_bytes + 255) / 256 * 256;
     static_assert(kHeadBytes + bytes + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "head, ring and final state must fit a pair's scratch");
 };
@@ -206,45 +208,23 @@ __device__ __forceinline__ SlowOut slow_corrections(const float4 *vals, int M, c
 // H = sum_c conj(S'_c) Z'_c over the value columns, where e^{i phi_{t-1}} S' is the state before token t and e^{i phi_t} Z'
 // the cotangent of Lambda_t S_{t-1}.  Written out over S_0, the tokens before t, G_C and the tokens from t on, every sum
 // over the columns is one that the chunk's products have already made (X1, X2, X3 before they are corrected, U Yb^T, U B^T)
-// or sum_c conj(S_0) G_C, made here; decays come as running products.  x: the thread's tokens g, g + 8 and keys 2 t4, + 1.
+// or r0 = sum_c conj(S_0) G_C; decays come as running products.  x: the thread's tokens g, g + 8 and keys 2 t4, + 1.
 // redo: bit 2 r + e says that this element is wanted; it goes to the caller's arrays.
 // (Rebuilding both matrices per element, column by column, took 6.4 M cycles a chunk where every alpha is small.)
-template <int DK, int NB>
-__device__ __forceinline__ void from_definition(const BwdArgsDev &a, const float4 *vals, const float2 *uy, const uint4 *pS, const uint4 *pG, const float *sc,
+template <int DK>
+__device__ __forceinline__ void from_definition(const BwdArgsDev &a, const float4 *vals, const float2 *uy, const float2 (&r0)[2],
                                                 const float (&x1r)[4], const float (&x1i)[4], const float (&x2r)[4], const float (&x2i)[4],
                                                 const float (&x3r)[4], const float (&x3i)[4], unsigned redo, size_t row0, int t0, int kt, int lane)
 {
-    constexpr int NCW = NB / 16, M = DK / 2, KT = M / 8;
+    constexpr int M = DK / 2;
     const int g = lane >> 2, t4 = lane & 3, key = 8 * kt + 2 * t4, left = a.T - t0;
-    float2 r0 = make_float2(0.f, 0.f);                            // of key g: four channels of every warp per lane
-#pragma unroll 1
-    for (int w = 0; w < NCW; ++w) {
-        const uint4 sr = pS[(w * KT + kt) * 64 + lane], si = pS[(w * KT + kt) * 64 + 32 + lane];
-        const uint4 gr = pG[(w * KT + kt) * 64 + lane], gi = pG[(w * KT + kt) * 64 + 32 + lane];
-        float2 sum = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            auto at = [&](const uint4 &v) { return join_half(c < 2 ? v.x : v.y, c < 2 ? v.z : v.w, c & 1); };
-            const float2 p = cmulc(make_float2(at(sr), at(si)), make_float2(at(gr), at(gi)));
-            sum = make_float2(sum.x + p.x, sum.y + p.y);
-        }
-        const float f = sc[4 * w] * sc[4 * w + 2];
-        r0 = make_float2(fmaf(f, sum.x, r0.x), fmaf(f, sum.y, r0.y));
-    }
-#pragma unroll
-    for (int d = 1; d < 4; d <<= 1) {
-        r0.x += __shfl_xor_sync(0xffffffffu, r0.x, d);
-        r0.y += __shfl_xor_sync(0xffffffffu, r0.y, d);
-    }
     // an element (token, key 2 t4 + e) of another thread's tile
     auto other = [&](const float(&re)[4], const float(&im)[4], int t, int e) {
         const int src = 4 * (t & 7) + t4;
         const float u = t < 8 ? re[e] : re[2 + e], v = t < 8 ? im[e] : im[2 + e];
         return make_float2(__shfl_sync(0xffffffffu, u, src), __shfl_sync(0xffffffffu, v, src));
     };
-    float2 s0[2], wt[16][2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) s0[e] = make_float2(__shfl_sync(0xffffffffu, r0.x, 4 * (2 * t4 + e)), __shfl_sync(0xffffffffu, r0.y, 4 * (2 * t4 + e)));
+    float2 wt[16][2];
 #pragma unroll 1
     for (int r = 0; r < 2; ++r) {
         const int t = g + 8 * r;
@@ -302,7 +282,7 @@ __device__ __forceinline__ void from_definition(const BwdArgsDev &a, const float
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const float4 v = vals[(15 * M + key + e) * 2 + 1];    // -, -, e^{i phi_C}
-            const float2 end = make_float2(pz[e] * v.z, -pz[e] * v.w), z0 = cmul(end, s0[e]), zx = cmul(end, sx[e]);
+            const float2 end = make_float2(pz[e] * v.z, -pz[e] * v.w), z0 = cmul(end, r0[e]), zx = cmul(end, sx[e]);
             const float hr = fmaf(pw[e], h[e].x + z0.x, su[e].x + zx.x), hi = fmaf(pw[e], h[e].y + z0.y, su[e].y + zx.y);
             if (redo >> (2 * r + e) & 1) {
                 a.dalpha[row * M + key + e] = hr;
@@ -460,8 +440,8 @@ __device__ __forceinline__ void stage_tokens(const BwdArgsDev &a, unsigned char 
 
 // ---- GRAD: the gradients of one chunk -----------------------------------------------------------------
 template <int DK, int NB, typename T>
-__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, const float2 *rg, int slot,
-                                                bool first, bool last_one, int t0, size_t row0, float2 (&carry)[2], int tid)
+__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, int slot, bool last_one, int t0,
+                                                size_t row0, int tid)
 {
     using L = BwdSmem<DK, NB>;
     using SC = BwdScratch<DK, NB>;
@@ -485,6 +465,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     // keys 2 t4, + 1); every chain warp's 16 columns come with scales of their own
     float x1r[4] = {0.f, 0.f, 0.f, 0.f}, x1i[4] = {0.f, 0.f, 0.f, 0.f}, x2r[4] = {0.f, 0.f, 0.f, 0.f};
     float x2i[4] = {0.f, 0.f, 0.f, 0.f}, x3r[4] = {0.f, 0.f, 0.f, 0.f}, x3i[4] = {0.f, 0.f, 0.f, 0.f};
+    float2 r0[2];
     if (warp < KT) {
         auto conj_product = [&](const uint4 *fx, const uint4 &b0, const uint4 &b1, float f, float (&xr)[4], float (&xi)[4]) {
             const uint4 h = fx[0], l = fx[32], h2 = fx[64], l2 = fx[96];
@@ -540,15 +521,33 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             }
             conj_product(frag + (NCW + w) * 128 + lane, s0, s1, sc[4 * w] * sc[4 * w + 3], x2r, x2i);
         }
+        // ... and sum_c conj(S_0) G_C: S with Re and Im in the rows, the diagonal of what that gives with Re G and Im G
+        const uint4 *ps = pS + warp * 64 + lane;
+        float sre[2] = {0.f, 0.f}, sim[2] = {0.f, 0.f};
 #pragma unroll 1
-        for (int w = 0; w < NCW; ++w) {
-            const uint4 g0 = n0, g1 = n1;
+        for (int w = 0; w < NCW; ++w, ps += KT * 64) {
+            const uint4 g0 = n0, g1 = n1, s0 = ps[0], s1 = ps[32];
             if (w + 1 < NCW) {
                 p += KT * 64;
                 n0 = p[0];
                 n1 = p[32];
             }
             conj_product(frag + (2 * NCW + w) * 128 + lane, g0, g1, sc[4 * w + 2] * sc[4 * w + 1], x3r, x3i);
+            const uint32_t ah[4] = {s0.x, s1.x, s0.y, s1.y}, al[4] = {s0.z, s1.z, s0.w, s1.w};
+            float d1[4] = {0.f, 0.f, 0.f, 0.f}, d2[4] = {0.f, 0.f, 0.f, 0.f};
+            mma3x<false>(d1, ah, al, g0.x, g0.y, g0.z, g0.w);
+            mma3x<false>(d2, ah, al, g1.x, g1.y, g1.z, g1.w);
+            const float f = sc[4 * w] * sc[4 * w + 2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                sre[e] = fmaf(f, d1[e] + d2[2 + e], sre[e]);
+                sim[e] = fmaf(f, d2[e] - d1[2 + e], sim[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int src = 4 * (2 * t4 + e) + t4;                 // row = column = 2 t4 + e
+            r0[e] = make_float2(__shfl_sync(0xffffffffu, sre[e], src), __shfl_sync(0xffffffffu, sim[e], src));
         }
     }
     // what the elements need besides, requested here: it comes from L2 and memory (prod alpha up to the token and after it)
@@ -566,18 +565,41 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     bar_sync(kBarTri, kPrep + kGrad);
 
     if (warp < KT) {
-        if (first) {                                               // D at the segment's end
+        // D behind the chunk, sum_c conj(S_C) G_C = conj(gamma_C) (sum_c conj(S_0) G_C) + sum_t conj(Y_t) X3_t
+        float2 carry[2];
+        {
+            const unsigned char *py = smem + slot * TL::bytes + TL::oY + g * TL::LDB + 2 * (8 * warp + 2 * t4);
+            float2 yr[2], yi[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                auto both = [&](int off) {
+                    const uint32_t *h = reinterpret_cast<const uint32_t *>(py + 8 * r * TL::LDB + off);
+                    const float2 x = unpack_f16(h[0]), y = unpack_f16(h[TL::PL / 4]);
+                    return make_float2(x.x + y.x, x.y + y.y);
+                };
+                yr[r] = both(0);
+                yi[r] = both(2 * TL::PL);
+            }
+            const float f = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS)[1];
+            const float4 gm = reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG)[4 * warp + t4];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                carry[e] = make_float2(0.f, 0.f);
-#pragma unroll 1
-                for (int w = 0; w < NCW; ++w) {
-                    const float2 x = rg[w * M + 8 * warp + 2 * t4 + e];
-                    carry[e] = make_float2(carry[e].x + x.x, carry[e].y + x.y);
+                float2 d = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const float2 x = cmulc(e ? make_float2(yr[r].y, yi[r].y) : make_float2(yr[r].x, yi[r].x), make_float2(x3r[2 * r + e], x3i[2 * r + e]));
+                    d = make_float2(d.x + x.x, d.y + x.y);
                 }
+#pragma unroll
+                for (int i = 4; i < 32; i <<= 1) {
+                    d.x += __shfl_xor_sync(0xffffffffu, d.x, i);
+                    d.y += __shfl_xor_sync(0xffffffffu, d.y, i);
+                }
+                const float2 z = cmulc(e ? make_float2(gm.z, gm.w) : make_float2(gm.x, gm.y), r0[e]);
+                carry[e] = make_float2(fmaf(f, d.x, z.x), fmaf(f, d.y, z.y));
             }
         }
-        // D / alpha loses digits where alpha is small, and D takes up all that is not finite up to the segment's end: those
+        // D / alpha loses digits where alpha is small, and D takes up all that is not finite up to the chunk's end: those
         // elements come from the definition
         constexpr float kSmall = 0.0625f;
         unsigned redo = 0;
@@ -587,7 +609,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             if (x < kSmall || d != 0.f) redo |= 1u << i;
         }
         const bool some = __any_sync(0xffffffffu, redo != 0);
-        if (some) from_definition<DK, NB>(a, vals, uy, pS, pG, sc, x1r, x1i, x2r, x2i, x3r, x3i, redo, row0, t0, warp, lane);
+        if (some) from_definition<DK>(a, vals, uy, r0, x1r, x1i, x2r, x2i, x3r, x3i, redo, row0, t0, warp, lane);
         const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
         const bool fast = reinterpret_cast<const int *>(inv)[6] != 0;
         const unsigned char *slot_at = smem + slot * TL::bytes;
@@ -733,7 +755,6 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         for (int e = 0; e < 2; ++e) {
             dd[2 + e] = make_float2(dd[2 + e].x + carry[e].x, dd[2 + e].y + carry[e].y);
             dd[e] = make_float2(dd[e].x + __shfl_sync(0xffffffffu, dd[2 + e].x, t4), dd[e].y + __shfl_sync(0xffffffffu, dd[2 + e].y, t4));
-            carry[e] = make_float2(__shfl_sync(0xffffffffu, dd[e].x, t4), __shfl_sync(0xffffffffu, dd[e].y, t4));
         }
         float dal[4];
 #pragma unroll
@@ -1229,7 +1250,6 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, NS = a.NS, nch = (a.T + kC - 1) / kC;
     unsigned char *ring = a.ring + blockIdx.x * a.ring_bytes;
-    float2 *rgs = reinterpret_cast<float2 *>(ring + SC::oRg);
     volatile int *job = reinterpret_cast<volatile int *>(smem + L::job);
     // The next part of the walk, for all threads at once (a part leaves none of its barriers pending).
     auto next_part = [&](int j) {
@@ -1291,7 +1311,6 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     if (tid < kGrad) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
         if constexpr (NB == 64) asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
-        float2 carry[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll 1
         for (int j = 0; next_part(j); ++j) {
             const int total = segments_of() * kSegChunks;
@@ -1300,8 +1319,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 const int r = n / kSegChunks, at = n % kSegChunks, c = kSegChunks - 1 - at, slot = ring_slot(r, c);
                 int bh, s;
                 segment(r, bh, s);
-                chunk_gradients<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, rgs + (r & 1) * NCW * M, slot, at == 0, n + 1 == total,
-                                           s * kSeg + c * kC, row_of(bh), carry, tid);
+                chunk_gradients<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, slot, n + 1 == total, s * kSeg + c * kC, row_of(bh), tid);
                 if (n + kSlots < total) bar_arrive(kBarReady + (n & 1), kGrad + kPrep);
             }
         }
@@ -1392,40 +1410,20 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 if (!kUnits && r == 0)
                     big_g = from > NS ? state_from_kept<DK>(sg, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane))
                                       : state_from_memory<DK>(sg, a.dS_T ? a.dS_T + state_at : nullptr, NB);
-                // rowdot(conj S, G) at the segment's end, this warp's columns; then S at its start
-                float2 *rg = rgs + ((r & 1) * NCW + w) * M + 2 * t4;
-                const float4 *end = kept<DK>(a.keep_s, bh, a.pitch, s + 1, NB, 16 * w, lane), *start = kept<DK>(a.keep_s, bh, a.pitch, s, NB, 16 * w, lane);
-                const float4 *kg = kept<DK>(a.keep_g, bh, a.pitch, s, NB, 16 * w, lane);
+                const float4 *start = kept<DK>(a.keep_s, bh, a.pitch, s, NB, 16 * w, lane), *kg = kept<DK>(a.keep_g, bh, a.pitch, s, NB, 16 * w, lane);
                 big_s = make_float2(0.f, 0.f);
                 if (kUnits) big_g = make_float2(0.f, 0.f);
 #pragma unroll 1
-                for (int n = 0; n < TL::KS; ++n, rg += 16, end += 128, start += 128, kg += 128) {
-                    float x[16], y[16];
+                for (int n = 0; n < TL::KS; ++n, start += 128, kg += 128) {
+                    float x[16];
                     if constexpr (kUnits) {
                         read_piece(kg, x);
                         tm_store(sg + 16 * n, x);
                         big_g = max_abs(reinterpret_cast<const float(&)[4][4]>(x), big_g);
-                        read_piece(end, y);
-                    } else {
-                        tm_load(x, sg + 16 * n);
-                        read_piece(end, y);
-                        tm_wait_load(x);
                     }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {                        // (tile, key)
-                        const int o = 8 * (u >> 1) + (u & 1);
-                        float re = y[o] * x[o] + y[o + 4] * x[o + 4] + y[o + 2] * x[o + 2] + y[o + 6] * x[o + 6];
-                        float im = y[o] * x[o + 4] - y[o + 4] * x[o] + y[o + 2] * x[o + 6] - y[o + 6] * x[o + 2];
-#pragma unroll
-                        for (int d = 4; d < 32; d <<= 1) {
-                            re += __shfl_xor_sync(0xffffffffu, re, d);
-                            im += __shfl_xor_sync(0xffffffffu, im, d);
-                        }
-                        if (g == 0) rg[8 * (u >> 1) + (u & 1)] = make_float2(re, im);
-                    }
-                    read_piece(start, y);
-                    tm_store(ss + 16 * n, y);
-                    big_s = max_abs(reinterpret_cast<const float(&)[4][4]>(y), big_s);
+                    read_piece(start, x);
+                    tm_store(ss + 16 * n, x);
+                    big_s = max_abs(reinterpret_cast<const float(&)[4][4]>(x), big_s);
                 }
                 tm_wait_store();
             }
