@@ -798,11 +798,11 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
 
 // ---- CHAIN helpers -----------------------------------------------------------------------------------
 // the state's 16-column pieces to and from the checkpoint [piece][4][lane] float4
-template <int DK>
+template <int KN>
 __device__ __forceinline__ void keep_state(float4 *p, uint32_t st)
 {
 #pragma unroll 1
-    for (int n = 0; n < Tile<DK>::KS; ++n, p += 128) {
+    for (int n = 0; n < KN; ++n, p += 128) {
         float x[16];
         tm_load(x, st + 16 * n);
         tm_wait_load(x);
@@ -875,43 +875,59 @@ struct Publish {
     float *scale;             // two inverse scales
 };
 
+// The products over the keys of both halves, scaled by f and added
+__device__ __forceinline__ void whole_sum(float (&acc)[2][2][4], const float (&f)[2], const Half &hf)
+{
+    float x[16], y[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = y[i] = f[(i & 3) >> 1] * acc[i >> 3][(i >> 2) & 1][i & 3];
+    add_other(x, y, hf);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i >> 3][(i >> 2) & 1][i & 3] = x[i];
+}
+
 // forward through one chunk whose tile is at `slot` (shared memory): U = M (V - W^* S), S <- gamma_C S + Y U unless
-// `update` is false.  load(rr): the chunk's rows of v.  Returns the largest magnitudes of S.
-template <int DK, int BARN, typename Load>
-__device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned char *slot, int bar, Load load, const Publish &pub, bool update, int lane)
+// `update` is false.  wait(): until the tile is there; load(rr): the chunk's rows of v.  KSP = 2: by one of two warps, for half
+// of the keys.  Returns the largest magnitudes of S.
+template <int DK, int KSP, typename Load, typename Wait>
+__device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned char *slot, Wait wait, Load load, const Publish &pub, bool update, int lane,
+                                               const Half &hf = Half())
 {
     using TL = Tile<DK>;
+    constexpr int KN = TL::KS / KSP;
     float rr[2][4], ri[2][4];
     load(rr);
     uint32_t off;                                                // tokens whose v is not finite; below, all behind them too
     const RowScale sr = row_scale<4>(big);
     bool own = false;
     const float all = pub.ps ? shared_scale(sr, own) : 0.f;
-    bar_sync(bar, BARN);
-    const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot);
+    const bool ok = wait();
+    const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot), keys = KSP > 1 ? 32 * KN * hf.half : 0;
     const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
-    const uint32_t tiles[1] = {tile + TL::oW};
+    const uint32_t tiles[1] = {tile + TL::oW + keys};
     TokFrag fr;
     {
         float acc[1][2][2][4];
-        keys_product<DK, 1>(acc, st, sr, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+        keys_product<DK, 1, KN>(acc, st, sr, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
             if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il, sr, all, own);
         });
         const float fw[2] = {sr.inv[0] * inv[0], sr.inv[1] * inv[0]};
         off = take_out(rr);
+        if (!ok) off = 0xffffffffu;
+        if constexpr (KSP > 1) whole_sum(acc[0], fw, hf);
 #pragma unroll
         for (int n = 0; n < 2; ++n)
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                rr[n][i] = fmaf(-fw[i >> 1], acc[0][0][n][i], rr[n][i]);
-                ri[n][i] = -fw[i >> 1] * acc[0][1][n][i];
+                rr[n][i] = KSP > 1 ? rr[n][i] - acc[0][0][n][i] : fmaf(-fw[i >> 1], acc[0][0][n][i], rr[n][i]);
+                ri[n][i] = KSP > 1 ? -acc[0][1][n][i] : -fw[i >> 1] * acc[0][1][n][i];
             }
     }
     {
         TokFrag fb;
         const RowScale r = make_frag(fr, rr, ri);
         load_small<false>(fb, tile + TL::oM, lane);
-        product_small<false>(rr, ri, fr, fb, r.inv, inv[3]);
+        product_small<false, 2>(rr, ri, fr, fb, r.inv, inv[3]);
     }
     RowScale ru = make_frag(fr, rr, ri);
     const uint32_t out = reinterpret_cast<const uint32_t *>(inv)[7];
@@ -928,16 +944,17 @@ __device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned
         }
     }
     if (odd) put_nan(ru.inv, off);
-    return update ? state_update<DK>(st, fr, ru.inv, inv[1], tile + TL::oY, reinterpret_cast<const float4 *>(slot + TL::oG), lane) : big;
+    return update ? state_update<DK, KN>(st, fr, ru.inv, inv[1], tile + TL::oY + keys, reinterpret_cast<const float4 *>(slot + TL::oG) + keys / 4, lane) : big;
 }
 
 // backward through one chunk: Bc = M^H (Y^* G + (A D_beta)^H Yb^*), G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc.  load(yr, yi):
 // the chunk's rows of Yb^* (yi zero without has_im).  Leaves Re Bc (the rows of dv) in pr; returns the largest magnitudes of G.
-template <int DK, bool kExact, typename Load>
-__device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigned char *slot, Load load, bool has_im, float (&pr)[2][4],
-                                                const Publish &pub, int lane)
+template <int DK, int KSP, bool kExact, typename Load>
+__device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigned char *slot, bool ok, Load load, bool has_im, float (&pr)[2][4],
+                                                const Publish &pub, int lane, const Half &hf = Half())
 {
     using TL = Tile<DK>;
+    constexpr int KN = TL::KS / KSP;
     const int t4 = lane & 3;
     uint32_t off;                                                // tokens whose cotangents are not finite; below, all before them too
     TokFrag fy;
@@ -947,23 +964,29 @@ __device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigne
         load(yr, yi);
         off = take_out(yr);
         if (has_im) off |= take_out(yi);
+        if (!ok) off = 0xffffffffu;
         ry = make_frag(fy, yr, yi);
     }
-    const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot);
+    const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot), keys = KSP > 1 ? 32 * KN * hf.half : 0;
     const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
     const RowScale sr = row_scale<4>(big);
     bool own = false;
     const float all = pub.ps ? shared_scale(sr, own) : 0.f;
     float acc[1][2][2][4];
-    const uint32_t tiles[1] = {tile + TL::oY};
-    keys_product<DK, 1>(acc, sg, sr, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
+    const uint32_t tiles[1] = {tile + TL::oY + keys};
+    keys_product<DK, 1, KN>(acc, sg, sr, tiles, lane, [&](int kk, const uint32_t(&rh)[4], const uint32_t(&rl)[4], const uint32_t(&ih)[4], const uint32_t(&il)[4]) {
         if (pub.ps) publish_state(pub.ps, kk, rh, rl, ih, il, sr, all, own);
     });
     float pi[2][4];
     {
         TokFrag fb;
         load_small<true>(fb, tile + TL::oA, lane);
-        const float fg[2] = {sr.inv[0] * inv[1], sr.inv[1] * inv[1]}, fa[2] = {ry.inv[0] * inv[4], ry.inv[1] * inv[4]};
+        float fg[2] = {sr.inv[0] * inv[1], sr.inv[1] * inv[1]};
+        if constexpr (KSP > 1) {
+            whole_sum(acc[0], fg, hf);
+            fg[0] = fg[1] = 1.f;
+        }
+        const float fa[2] = {ry.inv[0] * inv[4], ry.inv[1] * inv[4]};
 #pragma unroll
         for (int n = 0; n < 2; ++n) {
             float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f}, ni[4] = {0.f, 0.f, 0.f, 0.f};
@@ -985,7 +1008,7 @@ __device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigne
         TokFrag fb;
         const RowScale r = make_frag(fp, pr, pi);
         load_small<true>(fb, tile + TL::oM, lane);
-        product_small<true>(pr, pi, fp, fb, r.inv, inv[3]);
+        product_small<true, 2>(pr, pi, fp, fb, r.inv, inv[3]);
     }
     const RowScale rb = make_frag(fp, pr, pi);
     const uint32_t out = reinterpret_cast<const uint32_t *>(inv)[7];
@@ -1004,8 +1027,8 @@ __device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigne
         }
     }
     const float fq[2] = {ry.inv[0] * inv[2], ry.inv[1] * inv[2]}, fw[2] = {-rb.inv[0] * inv[0], -rb.inv[1] * inv[0]};
-    const float4 *gamma = reinterpret_cast<const float4 *>(slot + TL::oG) + t4;
-    uint32_t at = tile + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
+    const float4 *gamma = reinterpret_cast<const float4 *>(slot + TL::oG) + t4 + keys / 4;
+    uint32_t at = tile + keys + (uint32_t)(((lane & 7) + (((lane >> 3) & 1) << 3)) * TL::LDB + (lane >> 4) * 16);
     uint32_t nih[4], nil[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1014,7 +1037,7 @@ __device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigne
     }
     big = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int np = 0; np < TL::KS; ++np, at += 32, gamma += 8) {
+    for (int np = 0; np < KN; ++np, at += 32, gamma += 8) {
         float x[16];
         tm_load(x, sg + 16 * np);
         uint32_t qh[4], ql[4], jh[4], jl[4];
@@ -1089,96 +1112,61 @@ __device__ __forceinline__ float4 *kept(float *keep, int bh, int pitch, int s, i
 // With less than half as many sequences as SMs the walk of one CTA per sequence leaves the device idle.  But the
 // cotangent's chain needs neither S nor U: so S walks forward and G backward at the same time, each in blocks of value
 // columns (NB), both kept every 64 tokens; then every segment's gradients are a unit of their own (kUnits below).
-template <int DK, int DVT, int NB, typename T>
-__global__ void __launch_bounds__(ChainRoles<DK, NB>::threads, 1) sfda_backward_chain_kernel(const BwdArgsDev a)
+template <int DK, int NB, int CL, typename T>
+__global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_backward_chain_kernel(const BwdArgsDev a)
 {
     using TL = Tile<DK>;
-    using L = ChainSmem<DK, NB>;
-    constexpr int kChain = 2 * NB, kPrepWarps = ChainRoles<DK, NB>::prep_warps, kPrep = ChainRoles<DK, NB>::kPrep;
+    using L = Chain<DK, NB, CL>;
+    constexpr int KN = L::KN, DVT = NB * CL;
     extern __shared__ __align__(128) unsigned char smem[];
-    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB;
+    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, rank = CL > 1 ? blockIdx.y : 0, c0 = rank * NB;
     const bool back = blockIdx.z != 0;
     const size_t row0 = (size_t)b * a.T * a.H + h;
     const int nch = (a.T + kC - 1) / kC;
-    if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::slow), L::columns);
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    chain_begin<DK, NB, CL>(smem, tid);
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::slow);
     __syncthreads();
 
-    const ChainRoles<DK, NB> role(tid);
-    if (role.prep >= 0) {
+    if (tid < L::kPrep) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
-        const T *q = static_cast<const T *>(a.q), *k = static_cast<const T *>(a.k);
-        PrepRaw<L::PM::TPT, T> in;
-        prep_fetch<DK, kPrepWarps, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, (back ? nch - 1 : 0) * kC, a.T, back, role.prep);
-#pragma unroll 1
-        for (int c = 0; c < nch; ++c) {
-            const int slot = c % kSlots, at = back ? nch - 1 - c : c, nx = back ? max(at - 1, 0) : at + 1;
-            if (c >= kSlots) bar_sync(kBarDone + slot, kPrep + kChain);
-            PrepRaw<L::PM::TPT, T> next;
-            prep_fetch<DK, kPrepWarps, T>(next, q, k, a.alpha, a.theta, a.beta, row0, a.H, nx * kC, a.T, back, role.prep);
-            float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes);
-            if (!prep_chunk<DK, kPrepWarps, kBarAux, T>(in, q, k, a.alpha, a.theta, a.beta, row0, a.H, at * kC, a.T, nullptr, smem + slot * TL::bytes,
-                                                        smem + L::kb + slot * TL::BIG, smem + L::scan, back, role.prep))
-                slow_gram<DK, kPrepWarps, kBarAux, T>(q, k, a.alpha, a.theta, a.beta, row0, a.H, at * kC, a.T, smem + L::slow, smem + L::scan,
-                                                      gk, gk + 16 * 17, back, role.prep);
-            bar_arrive(kBarPlanes + slot, kPrep + 64);
-            in = next;
-        }
-    } else if (role.solve >= 0) {
+        chain_prep<DK, NB, CL, T>(smem, static_cast<const T *>(a.q), static_cast<const T *>(a.k), a.alpha, a.theta, a.beta, row0, a.H, a.T, nch, back, back,
+                                  rank, tid);
+    } else if (tid < L::kPrep + L::kSolve) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-        const int lane = tid & 31, w = role.solve >> 5, out = w >> 1;
-        const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
-#pragma unroll 1
-        for (int c = w & 1; c < nch; c += 2) {
-            const int slot = c % kSlots;
-            unsigned char *tile = smem + slot * TL::bytes;
-            float *inv = reinterpret_cast<float *>(tile + TL::oS);
-            float2 *gm = reinterpret_cast<float2 *>(smem + L::gram + slot * L::gram_bytes) + out * 16 * 17;
-            bar_sync(kBarPlanes + slot, kPrep + 64);
-            if (back || !out) {
-                if (reinterpret_cast<const int *>(inv)[6])
-                    gram_tiles<DK, 2>(base + slot * TL::bytes + (out ? TL::oQ : TL::oW), base + L::kb + slot * TL::BIG, inv[out ? 2 : 0] * inv[5], gm, 0, lane);
-                __syncwarp();
-                if (!out) invert_unit_lower16(gm, lane);
-                store_lower(tile + (out ? TL::oA : TL::oM), gm, inv + 3 + out, lane);
-            }
-            bar_arrive(kBarFull + slot, 64 + kChain);
-        }
-    } else if (role.chain >= 0) {
+        chain_solve<DK, NB, CL>(smem, nch, back, rank, tid - L::kPrep);
+    } else {
         if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
-        const int lane = tid & 31, w = role.chain >> 5, g = lane >> 2, t4 = lane & 3, col0 = c0 + 16 * w, col = col0 + g;
-        const uint32_t st = tmem + ((uint32_t)(w & 3) << 21) + (w >> 2) * 8 * TL::KT;
-        const size_t state_at = ((size_t)bh * DK + 4 * t4) * DVT + col, step = (size_t)a.H * DVT;
+        const int lane = tid & 31, w = (tid - L::kPrep - L::kSolve) >> 5, half = L::KSP > 1 ? w & 1 : 0, g = lane >> 2, t4 = lane & 3;
+        const int col0 = c0 + 16 * (w / L::KSP), col = col0 + g;
+        const uint32_t st = tmem + ((uint32_t)(w & 3) << 21) + (w >> 2) * 16 * KN, full = (uint32_t)__cvta_generic_to_shared(smem + L::bars);
+        const size_t state_at = ((size_t)bh * DK + 32 * KN * half + 4 * t4) * DVT + col, step = (size_t)a.H * DVT;
         const Publish none = {nullptr, nullptr, nullptr};
         const float *from = back ? a.dS_T : a.S0;
-        float2 big = state_from_memory<DK>(st, from ? from + state_at : nullptr, DVT);
+        float2 big = state_from_memory<KN>(st, from ? from + state_at : nullptr, DVT);
 #pragma unroll 1
         for (int c = 0; c < nch; ++c) {
             const int slot = c % kSlots, cc = back ? nch - 1 - c : c, left = a.T - cc * kC - 2 * t4;
             unsigned char *tile = smem + slot * TL::bytes;
             const size_t at = (row0 + (size_t)(cc * kC + 2 * t4) * a.H) * DVT + col;
+            const Half hf = L::KSP > 1 ? chain_half<DK, NB, CL>(smem, w, c, lane) : Half();
+            auto wait = [&] { return mbar_wait(full + 8 * slot, (c / kSlots) & 1); };
+            auto kept_at = [&](float *keep) { return kept<DK>(keep, bh, a.pitch, cc / kSegChunks, DVT, col0, lane) + 128 * KN * half; };
             if (!back) {
-                if (cc % kSegChunks == 0) keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, cc / kSegChunks, DVT, col0, lane), st);
+                if (cc % kSegChunks == 0) keep_state<KN>(kept_at(a.keep_s), st);
                 auto rows = [&](float(&x)[2][4]) { load_rows(x, static_cast<const T *>(a.v) + at, step, left); };
-                big = forward_step<DK, 64 + kChain>(st, big, tile, kBarFull + slot, rows, none, true, lane);
+                big = forward_step<DK, L::KSP>(st, big, tile, wait, rows, none, true, lane, hf);
             } else {
-                if (c == 0 || cc % kSegChunks == kSegChunks - 1) keep_state<DK>(kept<DK>(a.keep_g, bh, a.pitch, cc / kSegChunks, DVT, col0, lane), st);
+                if (c == 0 || cc % kSegChunks == kSegChunks - 1) keep_state<KN>(kept_at(a.keep_g), st);
                 float pr[2][4];
                 auto rows = [&](float(&x)[2][4], float(&y)[2][4]) { load_cotangents<T>(x, y, a.d_o, a.d_o_im, at, step, left); };
-                bar_sync(kBarFull + slot, 64 + kChain);
-                big = backward_step<DK, sizeof(T) == 2>(st, big, tile, rows, a.d_o_im != nullptr, pr, none, lane);
+                const bool ok = wait();
+                big = backward_step<DK, L::KSP, sizeof(T) == 2>(st, big, tile, ok, rows, a.d_o_im != nullptr, pr, none, lane, hf);
             }
-            if (c + kSlots < nch) bar_arrive(kBarDone + slot, kPrep + kChain);
+            if (c + kSlots < nch) warp_arrive(full + 8 * (kSlots + slot), c % CL, lane);
         }
-        if (back) state_to_memory<DK>(st, a.dS0 + state_at, DVT);
-        else keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, a.NS, DVT, col0, lane), st);
+        if (back) state_to_memory<KN>(st, a.dS0 + state_at, DVT);
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (tid < 32) tm_free(tmem, L::columns);
+    chain_end<DK, NB, CL>(tmem, tid);
 }
 
 // ---- the walk with gradients ------------------------------------------------------------------------------
@@ -1405,11 +1393,11 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
             if (r < 0) {
                 if (from >= NS) continue;
                 big_s = from ? state_from_kept<DK>(ss, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane))
-                             : state_from_memory<DK>(ss, a.S0 ? a.S0 + state_at : nullptr, NB);
+                             : state_from_memory<TL::KS>(ss, a.S0 ? a.S0 + state_at : nullptr, NB);
             } else {
                 if (!kUnits && r == 0)
                     big_g = from > NS ? state_from_kept<DK>(sg, kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane))
-                                      : state_from_memory<DK>(sg, a.dS_T ? a.dS_T + state_at : nullptr, NB);
+                                      : state_from_memory<TL::KS>(sg, a.dS_T ? a.dS_T + state_at : nullptr, NB);
                 const float4 *start = kept<DK>(a.keep_s, bh, a.pitch, s, NB, 16 * w, lane), *kg = kept<DK>(a.keep_g, bh, a.pitch, s, NB, 16 * w, lane);
                 big_s = make_float2(0.f, 0.f);
                 if (kUnits) big_g = make_float2(0.f, 0.f);
@@ -1430,18 +1418,22 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
 #pragma unroll 1
             for (int c = c0, n = r < 0 ? min(nch, to * kSegChunks) : kSegChunks; c < n; ++c) {
                 const int slot = r < 0 ? c % kSlots : ring_slot(r, c), t0 = (r < 0 ? 0 : s * kSeg) + c * kC;
-                if (r < 0 && c % kSegChunks == 0) keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, c / kSegChunks, NB, 16 * w, lane), ss);
+                if (r < 0 && c % kSegChunks == 0) keep_state<TL::KS>(kept<DK>(a.keep_s, bh, a.pitch, c / kSegChunks, NB, 16 * w, lane), ss);
                 unsigned char *scr = ring + (size_t)slot * SC::slot;
                 Publish pub = {nullptr, nullptr, nullptr};
                 if (r >= 0) pub = {reinterpret_cast<uint4 *>(scr + SC::oS) + w * KT * 64 + lane, reinterpret_cast<uint4 *>(scr + SC::oU) + w * 128, scal + (slot * NCW + w) * 4};
                 auto rows = [&](float(&x)[2][4]) {
                     load_rows(x, static_cast<const T *>(a.v) + (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col, step, a.T - t0 - 2 * t4);
                 };
-                big_s = forward_step<DK, kPrep + kChain>(ss, big_s, smem + slot * TL::bytes, kBarFull + slot, rows, pub, r < 0 || c + 1 < kSegChunks, lane);
+                auto full = [&] {
+                    bar_sync(kBarFull + slot, kPrep + kChain);
+                    return true;
+                };
+                big_s = forward_step<DK, 1>(ss, big_s, smem + slot * TL::bytes, full, rows, pub, r < 0 || c + 1 < kSegChunks, lane);
                 if (r < 0) bar_arrive(kBarDone + slot, kPrep + kChain);
             }
             if (r < 0) {                                                 // the final state, or where the next CTA begins
-                keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), ss);
+                keep_state<TL::KS>(kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), ss);
                 continue;
             }
 #pragma unroll 1
@@ -1452,13 +1444,13 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 const Publish pub = {reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64 + lane, reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, scal + (slot * NCW + w) * 4 + 2};
                 float pr[2][4];
                 auto rows = [&](float(&x)[2][4], float(&y)[2][4]) { load_cotangents<T>(x, y, a.d_o, a.d_o_im, at, step, left); };
-                big_g = backward_step<DK, kExact>(sg, big_g, smem + slot * TL::bytes, rows, a.d_o_im != nullptr, pr, pub, lane);
+                big_g = backward_step<DK, 1, kExact>(sg, big_g, smem + slot * TL::bytes, true, rows, a.d_o_im != nullptr, pr, pub, lane);
                 store_rows(static_cast<T *>(a.dv) + at, pr, step, left);
                 bar_arrive(kBarDone + slot, kPrep + kChain);
             }
             if (!kUnits && r + 1 == segments) {
-                if (to == 2 * NS) state_to_memory<DK>(sg, a.dS0 + state_at, NB);
-                else keep_state<DK>(kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), sg);
+                if (to == 2 * NS) state_to_memory<TL::KS>(sg, a.dS0 + state_at, NB);
+                else keep_state<TL::KS>(kept<DK>(a.keep_s, bh, a.pitch, NS, NB, 16 * w, lane), sg);
             }
         }
     }
@@ -1511,15 +1503,12 @@ cudaError_t launch_walk(const BwdArgsDev &a, int grid, cudaStream_t stream, int 
     return cudaGetLastError();
 }
 
-template <int DK, int DV, int NB, typename T>
+template <int DK, int NB, int CL, typename T>
 cudaError_t launch_chains(const BwdArgsDev &a, int pairs, cudaStream_t stream, int *launches)
 {
-    auto kern = sfda_backward_chain_kernel<DK, DV, NB, T>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ChainSmem<DK, NB>::bytes);
-    if (e != cudaSuccess) return e;
-    kern<<<dim3((unsigned)pairs, DV / NB, 2), ChainRoles<DK, NB>::threads, ChainSmem<DK, NB>::bytes, stream>>>(a);
+    using L = Chain<DK, NB, CL>;
     if (launches) ++*launches;
-    return cudaGetLastError();
+    return launch_clusters(sfda_backward_chain_kernel<DK, NB, CL, T>, a, dim3((unsigned)pairs, CL, 2), L::threads, L::bytes, stream);
 }
 
 template <int DK, int DV, typename T>
@@ -1566,13 +1555,11 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     const size_t room = (bwd_workspace(x.B, x.T, x.H, DK, DV) * sizeof(float) - kHeadBytes - (size_t)(rings - ws) * sizeof(float)) / SC::bytes;
     int grid = a.units < kBwdTargetCtas ? a.units : kBwdTargetCtas;
     if ((size_t)grid > room) grid = (int)room;
-    // both chains of all pairs at once: the columns are cut while that still fits the SMs
-    int nb = DV;
-    while (nb > 32 && 2LL * pairs * (DV / (nb / 2)) <= kBwdTargetCtas) nb /= 2;
+    const int nb = chain_columns(2LL * pairs, DV);               // both chains of all pairs at once
     cudaError_t e;
-    if (nb == DV) e = launch_chains<DK, DV, DV, T>(a, pairs, stream, launches);
-    else if (nb == 32) e = launch_chains<DK, DV, 32, T>(a, pairs, stream, launches);
-    else e = launch_chains<DK, DV, 64, T>(a, pairs, stream, launches);
+    if (nb == DV) e = launch_chains<DK, DV, 1, T>(a, pairs, stream, launches);
+    else if (nb == 32) e = launch_chains<DK, 32, DV / 32, T>(a, pairs, stream, launches);
+    else e = launch_chains<DK, 64, DV / 64, T>(a, pairs, stream, launches);
     return e == cudaSuccess ? launch_walk<DK, DV, T, true>(a, grid, stream, launches) : e;
 }
 

@@ -245,13 +245,15 @@ __device__ __forceinline__ uint32_t every_lanes(uint32_t m, int lane)
 __device__ __forceinline__ uint32_t from_first(uint32_t m) { return m ? 0xffffu & ~((m & (0u - m)) - 1u) : 0u; }    // 16 tokens
 __device__ __forceinline__ uint32_t to_last(uint32_t m) { return m ? 0xffffffffu >> __clz(m) : 0u; }
 __device__ __forceinline__ uint32_t both(uint32_t m) { return m | m << 16; }
-__device__ __forceinline__ void put_nan(float (&x)[2][4], uint32_t m, int lane)
+// (t0: the first tile's first token, 0 or 8)
+template <int NT>
+__device__ __forceinline__ void put_nan(float (&x)[NT][4], uint32_t m, int lane, int t0 = 0)
 {
 #pragma unroll
-    for (int n = 0; n < 2; ++n)
+    for (int n = 0; n < NT; ++n)
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            if (m >> (8 * n + 2 * (lane & 3) + (i & 1) + 16 * (i >> 1)) & 1) x[n][i] = __int_as_float(0x7fc00000);
+            if (m >> (t0 + 8 * n + 2 * (lane & 3) + (i & 1) + 16 * (i >> 1)) & 1) x[n][i] = __int_as_float(0x7fc00000);
 }
 __device__ __forceinline__ void put_nan(float (&inv)[2], uint32_t m)      // the rows' scales: a state update with them is NaN
 {
@@ -314,8 +316,8 @@ struct Tile {
 // ---- CHAIN --------------------------------------------------------------------------------------
 // acc[x] = products conj(X_x)^T S of NX tiles with the state at `st`, value channels in rows, tokens in columns, for
 // each of two token tiles: [0] = Re = Xr Sr + Xi Si, [1] = Im = Xr Si - Xi Sr; scaled by s and the tiles' scales.
-// pub(kk, rh, rl, ih, il) sees the split state of every step.
-template <int DK, int NX, typename Pub>
+// KN: steps of 16 keys (all of them, or a warp's share).  pub(kk, rh, rl, ih, il) sees the split state of every step.
+template <int DK, int NX, int KN, typename Pub>
 __device__ __forceinline__ void keys_product(float (&acc)[NX][2][2][4], uint32_t st, const RowScale &s, const uint32_t (&tile)[NX],
                                              int lane, Pub pub)
 {
@@ -333,11 +335,11 @@ __device__ __forceinline__ void keys_product(float (&acc)[NX][2][2][4], uint32_t
     tm_load(x, st);
     tm_wait_load(x);
 #pragma unroll 1
-    for (int kk = 0; kk < TL::KS; ++kk, at += 32) {
+    for (int kk = 0; kk < KN; ++kk, at += 32) {
         uint32_t rh[4], rl[4], ih[4], il[4];
         split_tiles(x, x + 8, s, rh, rl);
         split_tiles(x + 4, x + 12, s, ih, il);
-        const bool more = kk + 1 < TL::KS;
+        const bool more = kk + 1 < KN;
         if (more) tm_load(x, st + 16 * (kk + 1));
         pub(kk, rh, rl, ih, il);
 #pragma unroll
@@ -389,11 +391,11 @@ __device__ __forceinline__ void load_small(TokFrag &b, uint32_t tile, int lane)
     }
 }
 
-// out = a b (kConj: a conj(b)) over 16 tokens, both complex, unscaled by f and the rows' inv
-template <bool kConj>
-__device__ __forceinline__ void product_small(float (&re)[2][4], float (&im)[2][4], const TokFrag &a, const TokFrag &b, const float (&inv)[2], float f)
+// out = a b (kConj: a conj(b)) over 16 tokens, both complex, unscaled by f and the rows' inv; NT column tiles of b
+template <bool kConj, int NT>
+__device__ __forceinline__ void product_small(float (&re)[NT][4], float (&im)[NT][4], const TokFrag &a, const TokFrag &b, const float (&inv)[2], float f)
 {
-    float rr[2][4], ii[2][4], ir[2][4], ri[2][4];
+    float rr[NT][4], ii[NT][4], ir[NT][4], ri[NT][4];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const uint32_t(&ar)[4] = k == 0 ? a.rl : a.rh;
@@ -401,7 +403,7 @@ __device__ __forceinline__ void product_small(float (&re)[2][4], float (&im)[2][
         const uint32_t(&br)[4] = k == 1 ? b.rl : b.rh;
         const uint32_t(&bi)[4] = k == 1 ? b.il : b.ih;
 #pragma unroll
-        for (int n = 0; n < 2; ++n) {
+        for (int n = 0; n < NT; ++n) {
             if (k == 0) {
                 mma_f16_z(rr[n], ar, br[2 * n], br[2 * n + 1]);
                 mma_f16_z(ii[n], ai, bi[2 * n], bi[2 * n + 1]);
@@ -416,7 +418,7 @@ __device__ __forceinline__ void product_small(float (&re)[2][4], float (&im)[2][
         }
     }
 #pragma unroll
-    for (int n = 0; n < 2; ++n)
+    for (int n = 0; n < NT; ++n)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             re[n][i] = (inv[i >> 1] * f) * (kConj ? rr[n][i] + ii[n][i] : rr[n][i] - ii[n][i]);
@@ -501,11 +503,11 @@ __device__ __forceinline__ void load_rows(float (&x)[2][4], const T *p, size_t s
             x[n][e + 2] = on ? ld_val(r, 8) : 0.f;
         }
 }
-template <typename T>
-__device__ __forceinline__ void store_rows(T *p, const float (&x)[2][4], size_t step, int left)
+template <typename T, int NT>
+__device__ __forceinline__ void store_rows(T *p, const float (&x)[NT][4], size_t step, int left)
 {
 #pragma unroll
-    for (int n = 0; n < 2; ++n, p += 8 * step)
+    for (int n = 0; n < NT; ++n, p += 8 * step)
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             T *r = p + (e ? step : 0);
@@ -518,12 +520,12 @@ __device__ __forceinline__ void store_rows(T *p, const float (&x)[2][4], size_t 
 
 // The thread's fragment of a state [d_k][dv] (paired rows) at `p` (its key pair 2 (lane & 3), its column); returns the
 // largest magnitudes of its two rows.  p = NULL: zeros.
-template <int DK>
+template <int KN>
 __device__ __forceinline__ float2 state_from_memory(uint32_t st, const float *p, int dv)
 {
     float2 largest = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int n = 0; n < Tile<DK>::KS; ++n) {
+    for (int n = 0; n < KN; ++n) {
         float x[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i)                              // [key tile][Re / Im][column half][key]
@@ -534,11 +536,11 @@ __device__ __forceinline__ float2 state_from_memory(uint32_t st, const float *p,
     tm_wait_store();
     return largest;
 }
-template <int DK>
+template <int KN>
 __device__ __forceinline__ void state_to_memory(uint32_t st, float *p, int dv)
 {
 #pragma unroll 1
-    for (int n = 0; n < Tile<DK>::KS; ++n) {
+    for (int n = 0; n < KN; ++n) {
         float x[16];
         tm_load(x, st + 16 * n);
         tm_wait_load(x);
@@ -548,7 +550,7 @@ __device__ __forceinline__ void state_to_memory(uint32_t st, float *p, int dv)
 }
 
 // S <- gamma_C S + f inv a Y, the state at `st`, inv per row; returns the largest magnitudes of the new state's rows
-template <int DK>
+template <int DK, int KN>
 __device__ __forceinline__ float2 state_update(uint32_t st, const TokFrag &a, const float (&inv)[2], float f, uint32_t tile, const float4 *gamma, int lane)
 {
     using TL = Tile<DK>;
@@ -563,7 +565,7 @@ __device__ __forceinline__ float2 state_update(uint32_t st, const TokFrag &a, co
     const float fr[2] = {inv[0] * f, inv[1] * f};
     float2 largest = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int np = 0; np < TL::KS; ++np, at += 32, gamma += 8, st += 16) {
+    for (int np = 0; np < KN; ++np, at += 32, gamma += 8, st += 16) {
         float x[16], re[2][4], im[2][4];
         tm_load(x, st);
         tokens_product<DK>(re, im, a, nih, nil, at);
@@ -1067,47 +1069,231 @@ __device__ __forceinline__ void store_lower(unsigned char *tile, const float2 *A
     if (lane == 0) *inv_out = inv;
 }
 
-// ---- kernels that run a chain and nothing else: PREP, SOLVE, CHAIN -----------------------------------
-constexpr int kSolve = 128;
-constexpr int kBarPlanes = kBarFree;                             // + slot: planes ready (a chain alone needs no FREE)
-
-// Which warp does what.  A warp runs on scheduler (warp % 4), and mma.sync holds its scheduler: measured, 8.2 cycles each
-// and 0.7 more for every other instruction issued meanwhile.  With 32 columns the two chain warps would share theirs
-// with a quarter of PREP each (7.2 k cycles per chunk at 64 key pairs); so PREP goes to schedulers 2 and 3.  With 64 key
-// pairs it needs eight warps there (four: 8.2 k, eight: 6.3 k) and SOLVE stays beside the chain; with 32 pairs four do,
-// and SOLVE joins them (5.2 k -> 4.9 k).
-template <int DK, int NB>
-struct ChainRoles {
-    static constexpr bool few = NB == 32 && DK == 64;
-    static constexpr int prep_warps = few ? 4 : 8, kPrep = 32 * prep_warps;
-    static constexpr int threads = NB == 32 ? 512 : kPrep + kSolve + 2 * NB;
-    int prep = -1, solve = -1, chain = -1;                       // thread index inside the role, or -1
-    __device__ explicit ChainRoles(int tid)
-    {
-        if constexpr (NB == 32) {
-            const int w = tid >> 5, at = ((w >> 2) * 2 + (w & 1)) * 32 + (tid & 31);   // among the warps of two schedulers
-            if (w < 2) chain = tid;
-            else if (w & 2) (few && w >= 8 ? solve : prep) = few && w >= 8 ? at - kPrep : at;
-            else if (!few && w < 12) solve = at - 64;
-        } else {
-            if (tid < kPrep) prep = tid;
-            else if (tid < kPrep + kSolve) solve = tid - kPrep;
-            else chain = tid - kPrep - kSolve;
-        }
+// ---- a cluster's shared memory ---------------------------------------------------------------------
+// Barriers in shared memory: FULL (a slot's tile is complete) in every CTA, EMPTY (all CTAs are through with it) in the CTA
+// that makes the slot's tiles.  Waits are bounded; where one runs out (never, unless a CTA is gone) the results become NaN.
+constexpr uint32_t kWaitTries = 1u << 20;
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count)); }
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)       // by whole warps
+{
+#pragma unroll 1
+    for (uint32_t i = 0; i < kWaitTries; ++i) {
+        uint32_t ok;
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (__all_sync(0xffffffffu, ok)) return true;            // (the warp leaves together: what follows is for whole warps)
     }
-};
+    return false;
+}
+__device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank)       // the same place in another CTA of the cluster
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void warp_arrive(uint32_t bar, uint32_t rank, int lane)   // once for the warp, when all of it is here
+{
+    __syncwarp();
+    if (lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(in_cta(bar, rank)) : "memory");
+    __syncwarp();
+}
+// `bytes` from this CTA's shared memory to the same place in another's, counted by the barrier there
+__device__ __forceinline__ void copy_to_cta(uint32_t from, uint32_t bytes, uint32_t bar, uint32_t rank)
+{
+    const uint32_t to = in_cta(from, rank), there = in_cta(bar, rank);
+    asm volatile("mbarrier.arrive.expect_tx.release.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(there), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(to), "r"(from), "r"(bytes), "r"(there) : "memory");
+}
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-template <int DK, int NB>
-struct ChainSmem {
-    using PM = PrepMap<DK, ChainRoles<DK, NB>::prep_warps>;
-    static constexpr int kb = kSlots * Tile<DK>::bytes;          // Kb planes, a slot each
-    static constexpr int gram = kb + kSlots * Tile<DK>::BIG;     // the two Gram matrices, a slot each
+// ---- kernels that run a chain and nothing else: PREP, SOLVE, CHAIN -----------------------------------
+// A pair's CTAs (blocks of NB value columns) are a cluster of CL: the tile of chunk c is made by CTA c % CL alone and copied
+// to the others' shared memory, so that the preparation, which does not depend on the columns, is done once per pair.  It
+// had been half of what a CTA of 32 columns issued (13.4 k of 27.6 k issue cycles per chunk; mma.sync holds its scheduler
+// for 8.2 cycles, and 0.7 more for every other instruction issued meanwhile).  With 32 columns two warps share a block of
+// 16, half of the keys each (KSP), and add up their parts of the products over the keys: every scheduler has one chain
+// warp, with less work.  fp32 forward, B = 2, T = 2001, H = 16, d = 128: 457 -> 334 us (one warp per block of 16 columns 431,
+// eight PREP warps instead of four 371, the planes handed out with the rest of a tile 387).
+template <int DK, int NB, int CL>
+struct Chain {
+    static constexpr int KSP = NB == 32 ? 2 : 1, KN = Tile<DK>::KS / KSP;
+    static constexpr int prep_warps = NB == 32 ? 4 : 8, kPrep = 32 * prep_warps, kSolve = 128, warps = NB / 16 * KSP, kChain = 32 * warps;
+    static constexpr int threads = kPrep + kSolve + kChain;
+    static_assert(kSlots % CL == 0, "a slot's tiles are made by one CTA");
+    using PM = PrepMap<DK, prep_warps>;
+    static constexpr int own = kSlots / CL;                      // slots whose tiles this CTA makes
+    static constexpr int kb = kSlots * Tile<DK>::bytes;          // Kb planes, one for each of them,
+    static constexpr int gram = kb + own * Tile<DK>::BIG;        // the two Gram matrices likewise
     static constexpr int gram_bytes = 2 * 16 * 17 * 8;
-    static constexpr int scan = gram + kSlots * gram_bytes;
-    static constexpr int slow = scan + (PM::scan_bytes + 127) / 128 * 128;
-    static constexpr int bytes = slow + PM::slow_bytes;          // its first word also passes the tensor-memory address on
-    static constexpr int columns = (NB + 63) / 64 * DK / 2 < 32 ? 32 : (NB + 63) / 64 * DK / 2;
+    static constexpr int scan = gram + own * gram_bytes;
+    static constexpr int slow = scan + (PM::scan_bytes + 127) / 128 * 128;   // its first word also passes the tensor-memory address on
+    static constexpr int part = slow + (PM::slow_bytes + 127) / 128 * 128;   // KSP: [chunk parity][warp][6][lane] float4
+    static constexpr int bars = part + (KSP - 1) * 2 * warps * 3072;
+    static constexpr int bytes = bars + 2 * kSlots * 8;
+    static_assert(bytes <= 232448, "shared memory");
+    // 8 KT / KSP columns for every four warps
+    static constexpr int need = (warps + 3) / 4 * Tile<DK>::KT * 8 / KSP, columns = need < 32 ? 32 : need;
 };
+constexpr int kBarPlanes = kBarFree, kBarPair = 2, kBarHalf = 4;  // planes ready: + slot; SOLVE: + parity; chain halves: + block
+
+template <int DK, int NB, int CL>
+__device__ __forceinline__ void chain_begin(unsigned char *smem, int tid)
+{
+    using L = Chain<DK, NB, CL>;
+    if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::slow), L::columns);
+    if (tid == 32) {
+        const uint32_t bars = (uint32_t)__cvta_generic_to_shared(smem + L::bars);
+        for (int i = 0; i < kSlots; ++i) {
+            mbar_init(bars + 8 * i, 2);
+            mbar_init(bars + 8 * (kSlots + i), CL * L::warps);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if constexpr (CL > 1) cluster_sync();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+// Every CTA's copies have arrived when its chain is through; nobody leaves before the others are.
+template <int DK, int NB, int CL>
+__device__ __forceinline__ void chain_end(uint32_t tmem, int tid)
+{
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if constexpr (CL > 1) cluster_sync();
+    if (tid < 32) tm_free(tmem, Chain<DK, NB, CL>::columns);
+}
+
+// PREP of the chunks of rank `rank`, in the order of the chain (back: last to first)
+template <int DK, int NB, int CL, typename T>
+__device__ __forceinline__ void chain_prep(unsigned char *smem, const T *q, const T *k, const float *alpha, const float *theta, const float *beta,
+                                           size_t row0, int H, int T_, int nch, bool back, bool needq, int rank, int tid)
+{
+    using L = Chain<DK, NB, CL>;
+    constexpr int PW = L::prep_warps;
+    const uint32_t empty = (uint32_t)__cvta_generic_to_shared(smem + L::bars) + 8 * kSlots;
+    PrepRaw<L::PM::TPT, T> in;
+    prep_fetch<DK, PW, T>(in, q, k, alpha, theta, beta, row0, H, max(back ? nch - 1 - rank : rank, 0) * kC, T_, needq, tid);
+    bool ok = true;
+#pragma unroll 1
+    for (int c = rank; c < nch; c += CL) {
+        const int slot = c % kSlots, at = back ? nch - 1 - c : c, nx = back ? max(at - CL, 0) : at + CL;
+        if (c >= kSlots) ok = ok && mbar_wait(empty + 8 * slot, (c / kSlots - 1) & 1);
+        PrepRaw<L::PM::TPT, T> next;
+        prep_fetch<DK, PW, T>(next, q, k, alpha, theta, beta, row0, H, nx * kC, T_, needq, tid);
+        unsigned char *tile = smem + slot * Tile<DK>::bytes, *kb = smem + L::kb + slot / CL * Tile<DK>::BIG;
+        float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot / CL * L::gram_bytes);
+        if (!prep_chunk<DK, PW, kBarAux, T>(in, q, k, alpha, theta, beta, row0, H, at * kC, T_, nullptr, tile, kb, smem + L::scan, needq, tid))
+            slow_gram<DK, PW, kBarAux, T>(q, k, alpha, theta, beta, row0, H, at * kC, T_, smem + L::slow, smem + L::scan, gk, gk + 16 * 17, needq, tid);
+        if (!ok && tid == 0) reinterpret_cast<uint32_t *>(tile + Tile<DK>::oS)[7] = 0xffffffffu;
+        if constexpr (CL > 1) fence_async_smem();
+        bar_arrive(kBarPlanes + slot, L::kPrep + 64);
+        in = next;
+    }
+}
+
+// SOLVE: warps 0, 1 the system's inverse of this CTA's even / odd chunks, warps 2, 3 the outputs' Gram matrix of them
+// (needq); they also hand the tile out, its large planes first.  (With a single slot to make tiles in, warps 0 and 2 do it
+// alone: two chunks would meet at the slot's barrier.)
+template <int DK, int NB, int CL>
+__device__ __forceinline__ void chain_solve(unsigned char *smem, int nch, bool needq, int rank, int tid)
+{
+    using L = Chain<DK, NB, CL>;
+    using TL = Tile<DK>;
+    constexpr int pairs = L::own > 1 ? 2 : 1;
+    const int lane = tid & 31, w = tid >> 5, out = w >> 1;
+    const bool other = CL > 1 && lane < CL && lane != rank;      // a lane per CTA to hand out to
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem), full = base + L::bars;
+    if ((w & 1) >= pairs) return;
+#pragma unroll 1
+    for (int c = rank + CL * (w & 1); c < nch; c += pairs * CL) {
+        const int slot = c % kSlots;
+        unsigned char *tile = smem + slot * TL::bytes;
+        float *inv = reinterpret_cast<float *>(tile + TL::oS);
+        float2 *gm = reinterpret_cast<float2 *>(smem + L::gram + slot / CL * L::gram_bytes) + out * 16 * 17;
+        const uint32_t bar = full + 8 * slot, from = base + slot * TL::bytes;
+        bar_sync(kBarPlanes + slot, L::kPrep + 64);
+        if (out && other) copy_to_cta(from, TL::oM, bar, lane);
+        __syncwarp();
+        if (needq || !out) {
+            if (reinterpret_cast<const int *>(inv)[6])
+                gram_tiles<DK, 2>(base + slot * TL::bytes + (out ? TL::oQ : TL::oW), base + L::kb + slot / CL * TL::BIG, inv[out ? 2 : 0] * inv[5], gm, 0, lane);
+            __syncwarp();
+            if (!out) invert_unit_lower16(gm, lane);
+            store_lower(tile + (out ? TL::oA : TL::oM), gm, inv + 3 + out, lane);
+        }
+        if constexpr (CL > 1) fence_async_smem();
+        if (out) {
+            bar_arrive(kBarPair + (w & 1), 64);
+        } else {
+            bar_sync(kBarPair + (w & 1), 64);
+            if (other) copy_to_cta(from + TL::oM, TL::bytes - TL::oM, bar, lane);
+        }
+        warp_arrive(bar, rank, lane);
+    }
+}
+
+// A chain warp's place: its half of the keys (KSP = 2), and where the halves exchange their parts
+struct Half {
+    int half, bar;
+    float4 *mine;             // this chunk's (offset by the lane); the other half's lies `other` float4 further
+    int other;
+};
+// x += the other half's x; N a multiple of 4.  `out` goes to the other half, which sends its own in return.
+template <int N>
+__device__ __forceinline__ void add_other(float (&x)[N], const float (&out)[N], const Half &h)
+{
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i) h.mine[32 * i] = make_float4(out[4 * i], out[4 * i + 1], out[4 * i + 2], out[4 * i + 3]);
+    bar_sync(h.bar, 64);
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i) {
+        const float4 v = h.mine[h.other + 32 * i];
+        x[4 * i] += v.x;
+        x[4 * i + 1] += v.y;
+        x[4 * i + 2] += v.z;
+        x[4 * i + 3] += v.w;
+    }
+}
+template <int DK, int NB, int CL>
+__device__ __forceinline__ Half chain_half(unsigned char *smem, int w, int c, int lane)
+{
+    using L = Chain<DK, NB, CL>;
+    const int half = w & 1, block = w >> 1;
+    float4 *p = reinterpret_cast<float4 *>(smem + L::part) + ((c & 1) * L::warps + w) * 192 + lane;
+    return {half, kBarHalf + block, p, half ? -192 : 192};
+}
+
+// Value columns per CTA for `walks` sequences that a chain kernel takes at once: all of them, halved (down to 32) while the
+// clusters fit the SMs together: 74 of two, 32 of four (a GPC has 16 to 20 SMs).  (Those of a B200; on another device the
+// blocks are merely not the best ones.)
+inline int chain_columns(long long walks, int d_v)
+{
+    int nb = d_v;
+    while (nb > 32 && walks <= (d_v == nb ? 74 : 32)) nb /= 2;
+    return nb;
+}
+template <typename Args>
+cudaError_t launch_clusters(void (*kern)(Args), const Args &a, dim3 grid, int threads, int bytes, cudaStream_t stream)
+{
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = bytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = grid.y;                           // the blocks of columns of a pair
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = grid.y > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
 
 }  // namespace c16
 }  // namespace sfda
