@@ -62,6 +62,17 @@ def test_backward_of_pairs_shared_by_two_blocks(B, H, T, d_k, d_v, im):
     check_backward(cfg, workloads.forward_inputs(cfg), upstream(cfg, T, want_im=im), pairs[::19] + pairs[-2:], BWD_TOL)
 
 
+@pytest.mark.parametrize("H,d_k,d_v,T", [(32, 128, 128, 83), (33, 128, 128, 65), (74, 64, 128, 49), (75, 64, 128, 33), (74, 128, 64, 65),
+                                          (16, 128, 128, 67), (17, 64, 128, 81), (37, 128, 128, 50), (38, 64, 64, 97)])
+def test_blocks_of_columns_in_clusters(H, d_k, d_v, T):
+    """As many pairs as just fit in clusters of four or two blocks of columns, and one more (forward 32 and 74 pairs, backward
+    half as many); lengths at which ranks of the cluster make no, one or several of the tiles.  Bounds as above."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16k", B=1, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=900 + T + H)
+    inp, pairs = workloads.forward_inputs(cfg), all_pairs(cfg)
+    check_forward(cfg, inp, pairs[:2] + pairs[-2:], TOL)
+    check_backward(cfg, inp, upstream(cfg, T), pairs[:2] + pairs[-2:], BWD_TOL)
+
+
 GRADS = ("dq", "dk", "dv", "dalpha", "dtheta", "dbeta", "dS0")
 
 
