@@ -32,8 +32,8 @@
 // What bounds it: about 60 k cycles per 16 tokens of a pair at d_k = d_v = 128 (57 k, 12.6 k of them in the first sweep, with
 // mma.sync holding 29 % of the tensor pipe's time and issue slots 33 % used, before sums over the keys were rounded to
 // nearest and channels had scales of their own): the latency of the two chains under roles that share the schedulers.
-// Training step on raw inputs, B = 8, T = 8192, H = 32, bf16: 29.4 ms (the token-level adjoint on the CUDA cores: 148 ms);
-// B = 4, T = 4096, H = 16: 4.5 ms (21.8).
+// Training step on raw inputs, B = 8, T = 8192, H = 32, bf16: 28.2 ms (the token-level adjoint on the CUDA cores: 148 ms);
+// B = 4, T = 4096, H = 16: 4.3 ms (21.8).
 #include "sfda_chunk16.cuh"
 #include "sfda_internal.h"
 
@@ -74,13 +74,15 @@ static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags 
 
 // One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
 // S_0, G_C as B operands [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U, Bc as A operands
-// [chain warp][plane][lane] uint4; then the chunk's rotated keys and queries, decays and phases, 8 floats per
-// (token, key).  Behind the ring: slow_gram's scratch.
+// [chain warp][plane][lane] uint4; then the chunk's decays and phases, 4 floats per (token, key).  Behind the ring:
+// slow_gram's scratch.  The rotated keys and queries, which only the rare paths want, are not kept (Rotated): 704 KB instead
+// of 768 for d_k = d_v = 128, of which every chunk writes and reads 176 instead of 192.  Training step at the headline sizes
+// 29.5 -> 28.2 ms, B = 4, T = 4096, H = 16: 4.43 -> 4.29 ms, B = 2, T = 333, H = 4, d = 64: 195 -> 187 us.
 template <int DK, int NB>
 struct BwdScratch {
     static constexpr int NCW = NB / 16, KT = DK / 16, M = DK / 2;
     static constexpr int oS = 0, oU = oS + NCW * KT * 1024, oG = oU + NCW * 2048, oB = oG + NCW * KT * 1024;
-    static constexpr int oV = oB + NCW * 2048, slot = oV + 16 * M * 32;
+    static constexpr int oV = oB + NCW * 2048, slot = oV + 16 * M * 16;
     static constexpr int oSlow = slot * kSlots;
     static constexpr size_t bytes = (oSlow + PrepMap<DK, kPrepWarps>::slow_bytes + 255) / 256 * 256;
     static_assert(kHeadBytes + bytes + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "head, ring and final state must fit a pair's scratch");
@@ -154,20 +156,37 @@ __device__ __forceinline__ void st_val4(__nv_bfloat16 *p, float4 x)
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) { return make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }   // conj(a) b
 
-// one 16-bit half of the head and of the tail, added
-__device__ __forceinline__ float join_half(uint32_t h, uint32_t l, int half)
-{
-    const float2 x = unpack_f16(h), y = unpack_f16(l);
-    return half ? x.y + y.y : x.x + y.x;
-}
-
 // ---- the gradients where decays are too strong to divide by, or alpha too small -----------------------------
+// The rotated key and query (k'_t, q'_t) of a token of the chunk, as PREP made them: from the caller's arrays and the phases in
+// `vals`; zero behind the sequence and where PREP took a token out (`out`, see Tile).
+template <typename T>
+struct Rotated {
+    const T *k, *q;                                              // the pair's first row
+    const float4 *vals;
+    int M, left;
+    size_t step;                                                 // from one token to the next
+    uint32_t out;
+    __device__ Rotated(const BwdArgsDev &a, const float4 *v, int m, size_t row0, int t0, uint32_t o)
+        : k(static_cast<const T *>(a.k) + (row0 + (size_t)t0 * a.H) * 2 * m), q(static_cast<const T *>(a.q) + (row0 + (size_t)t0 * a.H) * 2 * m), vals(v), M(m),
+          left(a.T - t0), step((size_t)a.H * 2 * m), out(o) {}
+    __device__ __forceinline__ float4 operator()(int t, int key) const
+    {
+        const float4 v = vals[t * M + key];                      // -, -, cos, sin
+        const size_t at = t * step + 2 * key;
+        const bool on = t < left && !(out >> t & 1), onq = t < left && !(out >> (16 + t) & 1);
+        const float kx = on ? ld_val(k, at) : 0.f, ky = on ? ld_val(k, at + 1) : 0.f;
+        const float qx = onq ? ld_val(q, at) : 0.f, qy = onq ? ld_val(q, at + 1) : 0.f;
+        return make_float4(kx * v.z + ky * v.w, ky * v.z - kx * v.w, qx * v.z + qy * v.w, qy * v.z - qx * v.w);
+    }
+};
+
 // The corrections of one (token, key) where the decays are too strong to divide by: running products, token by token.
 // uy: U Yb^T and U B^T (two halves each); x1, x2, x3: the products with the boundary matrices.
 struct SlowOut {
     float2 qb, zb, fb;
 };
-__device__ __forceinline__ SlowOut slow_corrections(const float4 *vals, int M, const float2 *uy, const float *alpha, const float *beta,
+template <typename T>
+__device__ __forceinline__ SlowOut slow_corrections(const Rotated<T> &rotated, int M, const float2 *uy, const float *alpha, const float *beta,
                                                  size_t row0, int H, int t0, int T_, int tl, int key, float2 x1, float2 x2, float2 x3)
 {
     auto at = [&](int mat, int i, int t) {
@@ -179,7 +198,7 @@ __device__ __forceinline__ SlowOut slow_corrections(const float4 *vals, int M, c
     o.qb = o.zb = o.fb = make_float2(0.f, 0.f);
     for (int j = tl; j >= 0; --j) {
         const size_t rj = row0 + (size_t)(t0 + j) * H;
-        const float4 kj = vals[(j * M + key) * 2];
+        const float4 kj = rotated(j, key);
         const float bj = t0 + j < T_ ? w * beta[rj] : 0.f;
         const float2 kk = make_float2(bj * kj.x, bj * kj.y);
         const float2 p = cmul(kk, at(0, j, tl)), s = cmul(kk, at(1, j, tl));
@@ -191,7 +210,7 @@ __device__ __forceinline__ SlowOut slow_corrections(const float4 *vals, int M, c
     o.zb = make_float2(fmaf(w, x2.x, o.zb.x), fmaf(w, x2.y, o.zb.y));
     w = 1.f;
     for (int l = tl; l < 16; ++l) {
-        const float4 kl = vals[(l * M + key) * 2];
+        const float4 kl = rotated(l, key);
         const float2 p = cmulc(at(0, tl, l), make_float2(w * kl.z, w * kl.w));
         o.fb = make_float2(o.fb.x + p.x, o.fb.y + p.y);
         if (l > tl) {
@@ -211,8 +230,8 @@ __device__ __forceinline__ SlowOut slow_corrections(const float4 *vals, int M, c
 // or r0 = sum_c conj(S_0) G_C; decays come as running products.  x: the thread's tokens g, g + 8 and keys 2 t4, + 1.
 // redo: bit 2 r + e says that this element is wanted; it goes to the caller's arrays.
 // (Rebuilding both matrices per element, column by column, took 6.4 M cycles a chunk where every alpha is small.)
-template <int DK>
-__device__ __forceinline__ void from_definition(const BwdArgsDev &a, const float4 *vals, const float2 *uy, const float2 (&r0)[2],
+template <int DK, typename T>
+__device__ __forceinline__ void from_definition(const BwdArgsDev &a, const Rotated<T> &rotated, const float2 *uy, const float2 (&r0)[2],
                                                 const float (&x1r)[4], const float (&x1i)[4], const float (&x2r)[4], const float (&x2i)[4],
                                                 const float (&x3r)[4], const float (&x3i)[4], unsigned redo, size_t row0, int t0, int kt, int lane)
 {
@@ -241,7 +260,7 @@ __device__ __forceinline__ void from_definition(const BwdArgsDev &a, const float
             const float2 al = *reinterpret_cast<const float2 *>(a.alpha + row * M + key);
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const float4 v = vals[(i * M + key + e) * 2];
+                const float4 v = rotated(i, key + e);
                 const float2 w = make_float2(pw[e] * be * v.x, -pw[e] * be * v.y), p = cmul(w, x3[e]);
                 wt[i][e] = w;
                 sx[e] = make_float2(sx[e].x + p.x, sx[e].y + p.y);
@@ -260,7 +279,7 @@ __device__ __forceinline__ void from_definition(const BwdArgsDev &a, const float
             float2 q[2], k[2];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const float4 v = vals[(l * M + key + e) * 2];
+                const float4 v = rotated(l, key + e);
                 k[e] = make_float2(pz[e] * v.x, pz[e] * v.y);
                 q[e] = make_float2(pz[e] * v.z, pz[e] * v.w);
                 const float2 p = cmulc(x1[e], q[e]), m = cmulc(x2[e], k[e]);
@@ -281,7 +300,7 @@ __device__ __forceinline__ void from_definition(const BwdArgsDev &a, const float
         const size_t row = row0 + (size_t)(t0 + t) * a.H;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const float4 v = vals[(15 * M + key + e) * 2 + 1];    // -, -, e^{i phi_C}
+            const float4 v = rotated.vals[15 * M + key + e];       // -, -, e^{i phi_C}
             const float2 end = make_float2(pz[e] * v.z, -pz[e] * v.w), z0 = cmul(end, r0[e]), zx = cmul(end, sx[e]);
             const float hr = fmaf(pw[e], h[e].x + z0.x, su[e].x + zx.x), hi = fmaf(pw[e], h[e].y + z0.y, su[e].y + zx.y);
             if (redo >> (2 * r + e) & 1) {
@@ -556,9 +575,9 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int t = t0 + g + 8 * r;
-            const float4 *p = vals + ((g + 8 * r) * M + 8 * warp + 2 * t4) * 2;
-            va[2 * r] = *reinterpret_cast<const float2 *>(p + 1);
-            va[2 * r + 1] = *reinterpret_cast<const float2 *>(p + 3);
+            const float4 *p = vals + (g + 8 * r) * M + 8 * warp + 2 * t4;
+            va[2 * r] = *reinterpret_cast<const float2 *>(p);
+            va[2 * r + 1] = *reinterpret_cast<const float2 *>(p + 1);
             al2[r] = t < a.T ? *reinterpret_cast<const float2 *>(a.alpha + (row0 + (size_t)t * a.H) * M + 8 * warp + 2 * t4) : make_float2(1.f, 1.f);
         }
     }
@@ -609,8 +628,10 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             if (x < kSmall || d != 0.f) redo |= 1u << i;
         }
         const bool some = __any_sync(0xffffffffu, redo != 0);
-        if (some) from_definition<DK>(a, vals, uy, r0, x1r, x1i, x2r, x2i, x3r, x3i, redo, row0, t0, warp, lane);
         const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
+        const uint32_t out = reinterpret_cast<const uint32_t *>(inv)[7];
+        if (some)
+            from_definition<DK, T>(a, Rotated<T>(a, vals, M, row0, t0, out), uy, r0, x1r, x1i, x2r, x2i, x3r, x3i, redo, row0, t0, warp, lane);
         const bool fast = reinterpret_cast<const int *>(inv)[6] != 0;
         const unsigned char *slot_at = smem + slot * TL::bytes;
         // from here on x1, x2, x3 become S_t yb_t, Lambda_t S_{t-1} b_t, G_t conj(u_t) in the rotated frame
@@ -680,6 +701,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 x3i[i] = fmaf(s, z.y, down * fmaf(f2, zi[i], f3 * wi[i]));
             }
         } else {
+            const Rotated<T> rotated(a, vals, M, row0, t0, out);
 #pragma unroll 1
             for (int i = 0; i < 4; ++i) {                          // (no function and no indexed registers: both cost the common path)
                 auto pick = [&](const float(&v)[4]) { return i == 0 ? v[0] : i == 1 ? v[1] : i == 2 ? v[2] : v[3]; };
@@ -688,8 +710,8 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                     for (int j = 0; j < 4; ++j) v[j] = i == j ? x : v[j];
                 };
                 const int tl = g + 8 * (i >> 1), key = 8 * warp + 2 * t4 + (i & 1);
-                const float4 lv = vals[(15 * M + key) * 2 + 1];    // -, -, e^{i phi_C}
-                const SlowOut o = slow_corrections(vals, M, uy, a.alpha, a.beta, row0, a.H, t0, a.T, tl, key, make_float2(pick(x1r), pick(x1i)),
+                const float4 lv = vals[15 * M + key];              // -, -, e^{i phi_C}
+                const SlowOut o = slow_corrections(rotated, M, uy, a.alpha, a.beta, row0, a.H, t0, a.T, tl, key, make_float2(pick(x1r), pick(x1i)),
                                                    make_float2(pick(x2r), pick(x2i)), cmulc(make_float2(lv.z, lv.w), make_float2(pick(x3r), pick(x3i))));
                 put(x1r, o.qb.x);
                 put(x1i, o.qb.y);
@@ -704,9 +726,9 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         float al[4], dbp[2] = {0.f, 0.f};
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            // rotated key and query of the two keys: from the planes (W = a k', Q = a q'), or as they were kept
+            // rotated key and query of the two keys: from the planes (W = a k', Q = a q'), or made again
             const int tl = g + 8 * r;
-            const float4 *p = vals + (tl * M + 8 * warp + 2 * t4) * 2;
+            const float4 *p = vals + tl * M + 8 * warp + 2 * t4;
             float2 kr, ki, qr, qi;
             if (fast) {
                 const unsigned char *pw = slot_at + tl * TL::LDB + 2 * (8 * warp + 2 * t4);
@@ -721,7 +743,8 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 qr = both(TL::oQ, fq);
                 qi = both(TL::oQ + 2 * TL::PL, fq);
             } else {
-                const float4 u = p[0], v = p[2];
+                const Rotated<T> rotated(a, vals, M, row0, t0, out);
+                const float4 u = rotated(tl, 8 * warp + 2 * t4), v = rotated(tl, 8 * warp + 2 * t4 + 1);
                 kr = make_float2(u.x, v.x);
                 ki = make_float2(u.y, v.y);
                 qr = make_float2(u.z, v.z);
@@ -731,7 +754,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const int i = 2 * r + e;
-                const float2 ph = *(reinterpret_cast<const float2 *>(p + 1 + 2 * e) + 1);          // e^{i phi}
+                const float2 ph = *(reinterpret_cast<const float2 *>(p + e) + 1);          // e^{i phi}
                 const float2 kp = e ? make_float2(kr.y, ki.y) : make_float2(kr.x, ki.x), qp = e ? make_float2(qr.y, qi.y) : make_float2(qr.x, qi.x);
                 const float2 qb = make_float2(x1r[i], x1i[i]), zb = make_float2(x2r[i], x2i[i]), fb = make_float2(x3r[i], x3i[i]);
                 al[i] = e ? al2[r].y : al2[r].x;
@@ -781,7 +804,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             x += __shfl_xor_sync(0xffffffffu, x, 1);
             x += __shfl_xor_sync(0xffffffffu, x, 2);
             // (a query that was taken out is missing from its own token's sum)
-            if (t4 == 0) db[warp * 16 + g + 8 * r] = reinterpret_cast<const uint32_t *>(inv)[7] >> (16 + g + 8 * r) & 1 ? __int_as_float(0x7fc00000) : x;
+            if (t4 == 0) db[warp * 16 + g + 8 * r] = out >> (16 + g + 8 * r) & 1 ? __int_as_float(0x7fc00000) : x;
         }
     } else if (!last_one) {
         bar_arrive(kBarTaken, kGrad + kPrep);
@@ -1233,7 +1256,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     using TL = Tile<DK>;
     using L = BwdSmem<DK, NB>;
     using SC = BwdScratch<DK, NB>;
-    constexpr int kChain = 2 * NB, NCW = NB / 16, M = DK / 2, KT = TL::KT;
+    constexpr int kChain = 2 * NB, NCW = NB / 16, KT = TL::KT;
     constexpr bool kExact = sizeof(T) == 2;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, NS = a.NS, nch = (a.T + kC - 1) / kC;

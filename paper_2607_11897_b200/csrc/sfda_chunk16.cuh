@@ -692,8 +692,8 @@ __device__ __forceinline__ void put_planes(unsigned char *p, int pl, float r0, f
 }
 
 // Operand planes of one chunk: W, Y (and Q, with needq) into the slot, Kb_i = beta_i k_i / gamma_i into `kb` for the Gram products.
-// `vals` (or NULL) receives what the gradients need again, two float4 per (token, key): rotated key and query; prod
-// alpha up to the token and after it, e^{i phi}.  Called by all 32 PW threads (BAR: their barrier); the planes are
+// `vals` (or NULL) receives what the gradients need again, a float4 per (token, key): prod alpha up to the token and after
+// it, e^{i phi}.  Called by all 32 PW threads (BAR: their barrier); the planes are
 // complete for other threads only after a barrier of the caller's.
 //
 // The division by gamma_i is bounded by 2^16 inside a fast chunk (every coordinate keeps at least 2^-16 over the 16
@@ -773,11 +773,9 @@ __device__ __forceinline__ int prep_planes(const PrepRaw<PrepMap<DK, PW>::TPT, T
             r = in.q[x].get();
             qq[x] = make_float4(r.x * c0 + r.y * s0, r.y * c0 - r.x * s0, r.z * c1 + r.w * s1, r.w * c1 - r.z * s1);
             if (vals) {
-                float4 *o = vals + (t * M + 2 * pair) * 2;
-                o[0] = make_float4(kk[x].x, kk[x].y, qq[x].x, qq[x].y);
-                o[1] = make_float4(av[x].x, sf[x].x, c0, s0);
-                o[2] = make_float4(kk[x].z, kk[x].w, qq[x].z, qq[x].w);
-                o[3] = make_float4(av[x].y, sf[x].y, c1, s1);
+                float4 *o = vals + t * M + 2 * pair;
+                o[0] = make_float4(av[x].x, sf[x].x, c0, s0);
+                o[1] = make_float4(av[x].y, sf[x].y, c1, s1);
             }
             qq[x] = make_float4(av[x].x * qq[x].x, av[x].x * qq[x].y, av[x].y * qq[x].z, av[x].y * qq[x].w);
             mq = max_nan(max_nan(mq, max_nan(fabsf(qq[x].x), fabsf(qq[x].y))), max_nan(fabsf(qq[x].z), fabsf(qq[x].w)));
