@@ -26,14 +26,14 @@
 // unit of its own.  The CHAIN warps leave S_0, U, G_C, Bc of a chunk in a scratch ring as the operand registers of the
 // gradients' products.  PREP warps prepare the chunks' operand tiles and stage what the gradients need of the tokens;
 // GRAD warps turn all that into gradients one chunk behind the chain.  They meet at hardware barriers, one per slot: FULL
-// (a tile is complete), DONE (the chain came back through the chunk); READY (the gradients are through with the slot),
+// (a tile is complete), DONE (the chain came back through the chunk), GFREE (G_C's place is free again); READY (the gradients are through with the slot),
 // STAGED and TAKEN (the tokens are there, and free again).
 //
 // What bounds it: about 60 k cycles per 16 tokens of a pair at d_k = d_v = 128 (57 k, 12.6 k of them in the first sweep, with
 // mma.sync holding 29 % of the tensor pipe's time and issue slots 33 % used, before sums over the keys were rounded to
 // nearest and channels had scales of their own): the latency of the two chains under roles that share the schedulers.
-// Training step on raw inputs, B = 8, T = 8192, H = 32, bf16: 28.2 ms (the token-level adjoint on the CUDA cores: 148 ms);
-// B = 4, T = 4096, H = 16: 4.3 ms (21.8).
+// Training step on raw inputs, B = 8, T = 8192, H = 32, bf16: 28.3 ms (the token-level adjoint on the CUDA cores: 148 ms);
+// B = 4, T = 4096, H = 16: 4.2 ms (21.8).
 #include "sfda_chunk16.cuh"
 #include "sfda_internal.h"
 
@@ -72,21 +72,28 @@ constexpr size_t kHeadBytes = 1024;
 constexpr unsigned long long kChunkTicks = 1ull << 22;           // more than any chunk takes
 static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags follow the status block");
 
-// One slot of the scratch ring (global memory, one ring per CTA), all of it in the order of the consumer's registers:
-// S_0, G_C as B operands [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U, Bc as A operands
-// [chain warp][plane][lane] uint4; then the chunk's decays and phases, 4 floats per (token, key).  Behind the ring:
-// slow_gram's scratch.  The rotated keys and queries, which only the rare paths want, are not kept (Rotated): 704 KB instead
-// of 768 for d_k = d_v = 128, of which every chunk writes and reads 176 instead of 192.  Training step at the headline sizes
-// 29.5 -> 28.2 ms, B = 4, T = 4096, H = 16: 4.43 -> 4.29 ms, B = 2, T = 333, H = 4, d = 64: 195 -> 187 us.
+// The scratch ring (global memory, one per CTA), all of it in the order of the consumer's registers.  A slot for every chunk
+// of a segment: S_0 as B operand [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U as A operand [chain warp]
+// [plane][lane] uint4; the chunk's decays and phases, 4 floats per (token, key).  Behind the slots slow_gram's scratch and four
+// or two places in turn for G_C and Bc likewise.  With two the chain that comes back waits until the gradients have used up
+// what lies there (GFREE); see ring_places.  The rotated keys and queries, which only the rare paths want, are not kept (Rotated):
+// 704 KB with four places for d_k = d_v = 128 instead of 768, of which every chunk writes and reads 176 instead of 192.
+// Training step at the headline sizes 29.5 -> 28.2 ms, B = 4, T = 4096, H = 16: 4.43 -> 4.29 ms.
 template <int DK, int NB>
 struct BwdScratch {
     static constexpr int NCW = NB / 16, KT = DK / 16, M = DK / 2;
-    static constexpr int oS = 0, oU = oS + NCW * KT * 1024, oG = oU + NCW * 2048, oB = oG + NCW * KT * 1024;
-    static constexpr int oV = oB + NCW * 2048, slot = oV + 16 * M * 16;
-    static constexpr int oSlow = slot * kSlots;
-    static constexpr size_t bytes = (oSlow + PrepMap<DK, kPrepWarps>::slow_bytes + 255) / 256 * 256;
-    static_assert(kHeadBytes + bytes + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "head, ring and final state must fit a pair's scratch");
+    static constexpr int oS = 0, oU = oS + NCW * KT * 1024, oV = oU + NCW * 2048, slot = oV + 16 * M * 16;
+    static constexpr int oSlow = slot * kSlots, oG = (oSlow + PrepMap<DK, kPrepWarps>::slow_bytes + 255) / 256 * 256;
+    static constexpr int oB = oG + NCW * KT * 1024, place = NCW * KT * 1024 + NCW * 2048;
+    static constexpr size_t bytes(int places) { return (size_t)oG + (size_t)places * place; }
+    static_assert(place % 256 == 0 && kHeadBytes + bytes(4) + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "head, ring and final state must fit a pair's scratch");
 };
+// Two for the units: B = 2, T = 333, H = 4, d = 64 has 48 segments, for which the workspace has room for 60 rings instead of 42 (one
+// round instead of two, 187 -> 158 us), and B = 4, T = 4096, H = 16 has its rings in 80 MB of L2 instead of 104 (4.29 -> 4.22 ms).  Four for the walk, whose gradients have all of the way forward to catch up in: 28.2 ms at the headline sizes, 28.8 with
+// two.
+constexpr int ring_places(bool units) { return units ? 2 : 4; }
+// Which of the places chunk c of a segment has: they take turns in the order in which the chain comes back
+__device__ __forceinline__ int back_place(int c, int places) { return (kSegChunks - 1 - c) & (places - 1); }
 
 template <int DK, int NB>
 struct BwdSmem {
@@ -104,7 +111,8 @@ struct BwdSmem {
     static constexpr int db = scal + kSlots * NCW * 16 + 48;      // dbeta: [8][16] floats
     static constexpr int word = db + 8 * 16 * 4;                  // tensor-memory address
     static constexpr int job = word + 16;                         // the walk's current piece: pair, first and last position, gave up
-    static constexpr int bytes = job + 16;
+    static constexpr int gfree = job + 16;                        // GFREE: two barriers in shared memory
+    static constexpr int bytes = gfree + 16;
     static_assert(bytes <= 232448, "shared memory");
     static constexpr int columns = (NB + 63) / 64 * DK < 32 ? 32 : (NB + 63) / 64 * DK;   // S and G
 };
@@ -146,11 +154,13 @@ __device__ __forceinline__ float publish_frag(uint4 *p, const TokFrag &f, const 
     return all;
 }
 
-__device__ __forceinline__ void st_val4(float *p, float4 x) { *reinterpret_cast<float4 *>(p) = x; }
+// Gradients and kept states pass through L2 first to go (4.30 -> 4.25 ms for the training step at B = 4, T = 4096, H = 16): the rings
+// want to stay in it.
+__device__ __forceinline__ void st_val4(float *p, float4 x) { __stcs(reinterpret_cast<float4 *>(p), x); }
 __device__ __forceinline__ void st_val4(__nv_bfloat16 *p, float4 x)
 {
     const __nv_bfloat162 lo = __floats2bfloat162_rn(x.x, x.y), hi = __floats2bfloat162_rn(x.z, x.w);
-    *reinterpret_cast<uint2 *>(p) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+    __stcs(reinterpret_cast<uint2 *>(p), make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi)));
 }
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
@@ -314,7 +324,7 @@ __device__ __forceinline__ void from_definition(const BwdArgsDev &a, const Rotat
 // ---- PREP, second task: what the gradients of a chunk need of its tokens -----------------------------------
 // Yb, Bc, U into shared memory (STAGED), U Yb^T and U B^T, and the triangular factors of the corrections (TRI).
 template <int DK, int NB, typename T>
-__device__ __forceinline__ void stage_tokens(const BwdArgsDev &a, unsigned char *smem, const unsigned char *scr, int slot, int t0, size_t row0, int tid)
+__device__ __forceinline__ void stage_tokens(const BwdArgsDev &a, unsigned char *smem, const unsigned char *ring, int slot, int place, int t0, size_t row0, int tid)
 {
     using L = BwdSmem<DK, NB>;
     using SC = BwdScratch<DK, NB>;
@@ -330,7 +340,8 @@ __device__ __forceinline__ void stage_tokens(const BwdArgsDev &a, unsigned char 
     // operands over the value columns: Yb from the caller's arrays, Bc and U from the ring
     if (warp < NCW) {
         const int w = warp;
-        const uint4 *pB = reinterpret_cast<const uint4 *>(scr + SC::oB) + w * 128 + lane, *pU = reinterpret_cast<const uint4 *>(scr + SC::oU) + w * 128 + lane;
+        const uint4 *pB = reinterpret_cast<const uint4 *>(ring + SC::oB + place * SC::place) + w * 128 + lane;
+        const uint4 *pU = reinterpret_cast<const uint4 *>(ring + slot * SC::slot + SC::oU) + w * 128 + lane;
         uint4 x[8];
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
@@ -459,7 +470,7 @@ __device__ __forceinline__ void stage_tokens(const BwdArgsDev &a, unsigned char 
 
 // ---- GRAD: the gradients of one chunk -----------------------------------------------------------------
 template <int DK, int NB, typename T>
-__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *scr, int slot, bool last_one, int t0,
+__device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned char *smem, unsigned char *ring, int slot, int place, bool gfree, bool last_one, int t0,
                                                 size_t row0, int tid)
 {
     using L = BwdSmem<DK, NB>;
@@ -475,7 +486,8 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     float *scal = reinterpret_cast<float *>(smem + L::scal), *yscal = scal + kSlots * NCW * 4, *tscal = yscal + 8;
     const float *sc = scal + slot * NCW * 4;
     float *db = reinterpret_cast<float *>(smem + L::db);
-    const uint4 *pS = reinterpret_cast<const uint4 *>(scr + SC::oS), *pG = reinterpret_cast<const uint4 *>(scr + SC::oG);
+    const unsigned char *scr = ring + slot * SC::slot;
+    const uint4 *pS = reinterpret_cast<const uint4 *>(scr + SC::oS), *pG = reinterpret_cast<const uint4 *>(ring + SC::oG + place * SC::place);
     const float4 *vals = reinterpret_cast<const float4 *>(scr + SC::oV);
 
     bar_sync(kBarStaged, kPrep + kGrad);
@@ -569,6 +581,8 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
             r0[e] = make_float2(__shfl_sync(0xffffffffu, sre[e], src), __shfl_sync(0xffffffffu, sim[e], src));
         }
     }
+    __syncwarp();
+    if (gfree && lane == 0) mbar_arrive((uint32_t)__cvta_generic_to_shared(smem + L::gfree) + 8 * place);   // (Bc has been staged, G_C is in X3 and r0)
     // what the elements need besides, requested here: it comes from L2 and memory (prod alpha up to the token and after it)
     float2 va[4], al2[2];
     if (warp < KT) {
@@ -797,8 +811,8 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 }
                 st_val4(static_cast<T *>(a.dq) + ak, q4);
                 st_val4(static_cast<T *>(a.dk) + ak, k4);
-                *reinterpret_cast<float2 *>(a.dalpha + am) = a2;
-                *reinterpret_cast<float2 *>(a.dtheta + am) = th2;
+                __stcs(reinterpret_cast<float2 *>(a.dalpha + am), a2);
+                __stcs(reinterpret_cast<float2 *>(a.dtheta + am), th2);
             }
             float x = dbp[r];
             x += __shfl_xor_sync(0xffffffffu, x, 1);
@@ -830,14 +844,14 @@ __device__ __forceinline__ void keep_state(float4 *p, uint32_t st)
         tm_load(x, st + 16 * n);
         tm_wait_load(x);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) p[32 * j] = make_float4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
+        for (int j = 0; j < 4; ++j) __stcs(p + 32 * j, make_float4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]));
     }
 }
 __device__ __forceinline__ void read_piece(const float4 *p, float (&x)[16])
 {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const float4 v = p[32 * j];
+        const float4 v = __ldcs(p + 32 * j);
         x[4 * j] = v.x;
         x[4 * j + 1] = v.y;
         x[4 * j + 2] = v.z;
@@ -1261,6 +1275,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, NS = a.NS, nch = (a.T + kC - 1) / kC;
     unsigned char *ring = a.ring + blockIdx.x * a.ring_bytes;
+    constexpr int places = ring_places(kUnits);
     volatile int *job = reinterpret_cast<volatile int *>(smem + L::job);
     // The next part of the walk, for all threads at once (a part leaves none of its barriers pending).
     auto next_part = [&](int j) {
@@ -1312,6 +1327,11 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     auto row_of = [&](int bh) { return (size_t)(bh / a.H) * a.T * a.H + bh % a.H; };
     if (!a.flags && blockIdx.x == 0 && tid == 0) *a.status = 0;          // nothing waits (else the launcher has cleared it)
     if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::word), L::columns);
+    if (places == 2 && tid == 32) {
+        const uint32_t bar = (uint32_t)__cvta_generic_to_shared(smem + L::gfree);
+        mbar_init(bar, kGradWarps);
+        mbar_init(bar + 8, kGradWarps);
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1330,7 +1350,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 const int r = n / kSegChunks, at = n % kSegChunks, c = kSegChunks - 1 - at, slot = ring_slot(r, c);
                 int bh, s;
                 segment(r, bh, s);
-                chunk_gradients<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, slot, n + 1 == total, s * kSeg + c * kC, row_of(bh), tid);
+                chunk_gradients<DK, NB, T>(a, smem, ring, slot, back_place(c, places), places == 2, n + 1 == total, s * kSeg + c * kC, row_of(bh), tid);
                 if (n + kSlots < total) bar_arrive(kBarReady + (n & 1), kGrad + kPrep);
             }
         }
@@ -1361,7 +1381,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                     segment(r, bh, s);
                     bar_sync(kBarDone + slot, kPrep + kChain);
                     if (m) bar_sync(kBarTaken, kGrad + kPrep);
-                    stage_tokens<DK, NB, T>(a, smem, ring + (size_t)slot * SC::slot, slot, s * kSeg + c * kC, row_of(bh), ptid);
+                    stage_tokens<DK, NB, T>(a, smem, ring, slot, back_place(c, places), s * kSeg + c * kC, row_of(bh), ptid);
                     continue;
                 }
                 if (!sweep && p >= kSlots) bar_sync(kBarDone + p % kSlots, kPrep + kChain);
@@ -1463,11 +1483,14 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
             for (int c = kSegChunks - 1; c >= 0; --c) {
                 const int slot = ring_slot(r, c), t0 = s * kSeg + c * kC, left = a.T - t0 - 2 * t4;
                 const size_t at = (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col;
-                unsigned char *scr = ring + (size_t)slot * SC::slot;
+                const int n = r * kSegChunks + kSegChunks - 1 - c;
+                unsigned char *scr = ring + (n & (places - 1)) * SC::place;
                 const Publish pub = {reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64 + lane, reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, scal + (slot * NCW + w) * 4 + 2};
+                bool ok = true;
+                if constexpr (places == 2) ok = mbar_wait((uint32_t)__cvta_generic_to_shared(smem + L::gfree) + 8 * (n & 1), ((n >> 1) + 1) & 1);
                 float pr[2][4];
                 auto rows = [&](float(&x)[2][4], float(&y)[2][4]) { load_cotangents<T>(x, y, a.d_o, a.d_o_im, at, step, left); };
-                big_g = backward_step<DK, 1, kExact>(sg, big_g, smem + slot * TL::bytes, true, rows, a.d_o_im != nullptr, pr, pub, lane);
+                big_g = backward_step<DK, 1, kExact>(sg, big_g, smem + slot * TL::bytes, ok, rows, a.d_o_im != nullptr, pr, pub, lane);
                 store_rows(static_cast<T *>(a.dv) + at, pr, step, left);
                 bar_arrive(kBarDone + slot, kPrep + kChain);
             }
@@ -1550,7 +1573,7 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     a.keep_s = ws;
     a.pitch = a.NS + 1;
     a.keep_g = ws + (size_t)pairs * a.pitch * state;
-    a.ring_bytes = SC::bytes;
+    a.ring_bytes = SC::bytes(ring_places(cols != DV));
     a.status = static_cast<unsigned *>(workspace);
     a.flags = nullptr;
     a.wait_ticks = x.wait_ticks ? x.wait_ticks : 1ull << 31;     // about a second, more for long sequences
@@ -1575,9 +1598,9 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     if (a.withhold) return cudaErrorInvalidValue;
     float *rings = a.keep_g + (size_t)pairs * a.pitch * state;
     a.ring = reinterpret_cast<unsigned char *>(rings);
-    const size_t room = (bwd_workspace(x.B, x.T, x.H, DK, DV) * sizeof(float) - kHeadBytes - (size_t)(rings - ws) * sizeof(float)) / SC::bytes;
+    const size_t room = bwd_workspace(x.B, x.T, x.H, DK, DV) * sizeof(float) - kHeadBytes - (size_t)(rings - ws) * sizeof(float);
     int grid = a.units < kBwdTargetCtas ? a.units : kBwdTargetCtas;
-    if ((size_t)grid > room) grid = (int)room;
+    if ((size_t)grid * a.ring_bytes > room) grid = (int)(room / a.ring_bytes);
     const int nb = chain_columns(2LL * pairs, DV);               // both chains of all pairs at once
     cudaError_t e;
     if (nb == DV) e = launch_chains<DK, DV, 1, T>(a, pairs, stream, launches);

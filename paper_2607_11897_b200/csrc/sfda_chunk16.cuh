@@ -1089,6 +1089,7 @@ __device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank)       /
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
 __device__ __forceinline__ void warp_arrive(uint32_t bar, uint32_t rank, int lane)   // once for the warp, when all of it is here
 {
     __syncwarp();
