@@ -89,8 +89,8 @@ struct BwdScratch {
     static_assert(place % 256 == 0 && kHeadBytes + bytes(4) + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "head, ring and final state must fit a pair's scratch");
 };
 // Two for the units: B = 2, T = 333, H = 4, d = 64 has 48 segments, for which the workspace has room for 60 rings instead of 42 (one
-// round instead of two, 187 -> 158 us), and B = 4, T = 4096, H = 16 has its rings in 80 MB of L2 instead of 104 (4.29 -> 4.22 ms).  Four for the walk, whose gradients have all of the way forward to catch up in: 28.2 ms at the headline sizes, 28.8 with
-// two.
+// round instead of two, 187 -> 158 us), and B = 4, T = 4096, H = 16 has its rings in 80 MB of L2 instead of 104 (4.29 -> 4.22 ms).
+// Four for the walk, whose gradients have all of the way forward to catch up in: 28.2 ms at the headline sizes, 28.8 with two.
 constexpr int ring_places(bool units) { return units ? 2 : 4; }
 // Which of the places chunk c of a segment has: they take turns in the order in which the chain comes back
 __device__ __forceinline__ int back_place(int c, int places) { return (kSegChunks - 1 - c) & (places - 1); }
@@ -1186,7 +1186,7 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_backward_c
             unsigned char *tile = smem + slot * TL::bytes;
             const size_t at = (row0 + (size_t)(cc * kC + 2 * t4) * a.H) * DVT + col;
             const Half hf = L::KSP > 1 ? chain_half<DK, NB, CL>(smem, w, c, lane) : Half();
-            auto wait = [&] { return mbar_wait(full + 8 * slot, (c / kSlots) & 1); };
+            auto wait = [&] { return chain_wait<DK, NB, CL>(full, c); };
             auto kept_at = [&](float *keep) { return kept<DK>(keep, bh, a.pitch, cc / kSegChunks, DVT, col0, lane) + 128 * KN * half; };
             if (!back) {
                 if (cc % kSegChunks == 0) keep_state<KN>(kept_at(a.keep_s), st);
@@ -1199,7 +1199,7 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_backward_c
                 const bool ok = wait();
                 big = backward_step<DK, L::KSP, sizeof(T) == 2>(st, big, tile, ok, rows, a.d_o_im != nullptr, pr, none, lane, hf);
             }
-            if (c + kSlots < nch) warp_arrive(full + 8 * (kSlots + slot), c % CL, lane);
+            chain_release<DK, NB, CL>(full, c, nch, lane);
         }
         if (back) state_to_memory<KN>(st, a.dS0 + state_at, DVT);
     }

@@ -1179,7 +1179,8 @@ __device__ __forceinline__ void chain_prep(unsigned char *smem, const T *q, cons
 #pragma unroll 1
     for (int c = rank; c < nch; c += CL) {
         const int slot = c % kSlots, at = back ? nch - 1 - c : c, nx = back ? max(at - CL, 0) : at + CL;
-        if (c >= kSlots) ok = ok && mbar_wait(empty + 8 * slot, (c / kSlots - 1) & 1);
+        if (CL == 1 && c >= kSlots) bar_sync(kBarDone + slot, L::kPrep + L::kChain);
+        if (CL > 1 && c >= kSlots) ok = ok && mbar_wait(empty + 8 * slot, (c / kSlots - 1) & 1);
         PrepRaw<L::PM::TPT, T> next;
         prep_fetch<DK, PW, T>(next, q, k, alpha, theta, beta, row0, H, nx * kC, T_, needq, tid);
         unsigned char *tile = smem + slot * Tile<DK>::bytes, *kb = smem + L::kb + slot / CL * Tile<DK>::BIG;
@@ -1223,7 +1224,11 @@ __device__ __forceinline__ void chain_solve(unsigned char *smem, int nch, bool n
             if (!out) invert_unit_lower16(gm, lane);
             store_lower(tile + (out ? TL::oA : TL::oM), gm, inv + 3 + out, lane);
         }
-        if constexpr (CL > 1) fence_async_smem();
+        if constexpr (CL == 1) {
+            bar_arrive(kBarFull + slot, 64 + L::kChain);
+            continue;
+        }
+        fence_async_smem();
         if (out) {
             bar_arrive(kBarPair + (w & 1), 64);
         } else {
@@ -1232,6 +1237,26 @@ __device__ __forceinline__ void chain_solve(unsigned char *smem, int nch, bool n
         }
         warp_arrive(bar, rank, lane);
     }
+}
+
+// CHAIN: until chunk c's tile is there; and when the warp is through with it.  (A CTA by itself has hardware barriers for FULL and
+// EMPTY: a warp that waits at one in shared memory resumes a few hundred cycles late, 36.3 us instead of 34.8 for the forward of
+// B = 20, T = 104, H = 7, d_k = 64, d_v = 128.)
+template <int DK, int NB, int CL>
+__device__ __forceinline__ bool chain_wait(uint32_t full, int c)
+{
+    const int slot = c % kSlots;
+    if constexpr (CL > 1) return mbar_wait(full + 8 * slot, (c / kSlots) & 1);
+    bar_sync(kBarFull + slot, 64 + Chain<DK, NB, CL>::kChain);
+    return true;
+}
+template <int DK, int NB, int CL>
+__device__ __forceinline__ void chain_release(uint32_t full, int c, int nch, int lane)
+{
+    const int slot = c % kSlots;
+    if (c + kSlots >= nch) return;
+    if constexpr (CL > 1) warp_arrive(full + 8 * (kSlots + slot), c % CL, lane);
+    else bar_arrive(kBarDone + slot, Chain<DK, NB, CL>::kPrep + Chain<DK, NB, CL>::kChain);
 }
 
 // A chain warp's place: its half of the keys (KSP = 2), and where the halves exchange their parts

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
             float rr[2][4], ri[2][4];
             load_rows(rr, static_cast<const T *>(a.v) + at, step, left);
             const RowScale sr = row_scale<4>(largest);
-            const bool ok = mbar_wait(base + L::bars + 8 * slot, (c / kSlots) & 1);
+            const bool ok = chain_wait<DK, NB, CL>(base + L::bars, c);
             const uint32_t tile = base + slot * TL::bytes;
             const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
             float acc[2][2][2][4];
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
                 put_nan(ru.inv, off);
             }
             largest = state_update<DK, KN>(st, fr, ru.inv, inv[1], tile + TL::oY + keys, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG) + 8 * KN * half, lane);
-            if (c + kSlots < nch) warp_arrive(base + L::bars + 8 * (kSlots + slot), c % CL, lane);
+            chain_release<DK, NB, CL>(base + L::bars, c, nch, lane);
 #pragma unroll
             for (int n = 0; n < NT; ++n)
 #pragma unroll
