@@ -143,6 +143,8 @@ SFDA_API int sfda_forward_partition(int B, int T, int H, int d_k, int d_v, int c
  * fp32; any alpha in [0, 1]).  Those 22 bits count from the largest entry of a value channel (over the keys, or over
  * 16 tokens) and of the keys and queries of 16 tokens; an entry 2^-16 and more below that has an absolute error of
  * 2^-39 of it.  An input that is not finite makes NaN of what depends on it in the recurrence, and of nothing else.
+ * On that path the CTAs of a (batch, head) pair may wait for one another (about a second at most); where such a wait runs
+ * out, all outputs and the final state of the waiting CTA's pair are NaN (there is no workspace to report it in).
  * The bf16 tensor-core path forms 1/gamma_t inside a chunk and so
  * additionally assumes prod_{t in chunk} alpha_{t,j} >= exp(-80) for every
  * coordinate j; beyond that results lose accuracy but stay finite.
@@ -499,6 +501,10 @@ SFDA_API int sfda_forward_fused(const void *q, const void *k_raw, const void *v,
  * next, which waits for it: a cooperative launch, as for sfda_forward's time slices.  The wait is bounded (about a second,
  * more for long sequences; longer than any inputs take).  Where it runs out sfda_workspace_status returns
  * SFDA_ERR_TIMEOUT, and every gradient that the waiting CTA had still to write is NaN; the others are valid.
+ * With few pairs a pair's CTAs (a thread-block cluster) wait for one another's preparation of the chunks, and the roles
+ * of a unit for a place in its scratch; these waits are bounded by about a second each.  Where one runs out the status is
+ * SFDA_ERR_TIMEOUT as well, and every gradient that depends on what was waited for is NaN: all of the pair's (dv, dS0
+ * only if it was the cotangent's chain), or those of all segments that the CTA had.
  */
 SFDA_API size_t sfda_backward_workspace_bytes(int B, int T, int H, int d_k, int d_v, int dtype);
 SFDA_API int sfda_backward(const void *q, const void *k, const void *v,

@@ -60,8 +60,9 @@ struct BwdArgsDev {
     size_t ring_bytes;
     int T, H, NS, pitch, units;
     long long work;           // of all pairs' walks, in the units of walk_cut
-    unsigned *status;         // first word of the workspace: 1 where a wait for a piece ran out
-    unsigned *flags;          // per CTA: the piece it hands on is written (null where none is)
+    unsigned *status;         // first word of the workspace: 1 where a wait ran out
+    unsigned *flags;          // per CTA of the walk: the piece it hands on is written (null where none is); of the chains: a wait ran out
+    int chain_ctas;           // CTAs of the chains that write such a flag
     unsigned long long wait_ticks;   // SM-clock ticks after which a wait gives up
     int withhold;             // diagnostic: pieces are never announced
 };
@@ -70,7 +71,7 @@ struct BwdArgsDev {
 constexpr int kBwdTargetCtas = 148;
 constexpr size_t kHeadBytes = 1024;
 constexpr unsigned long long kChunkTicks = 1ull << 22;           // more than any chunk takes
-static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags follow the status block");
+static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags follow the status block");   // (the chains: at most 2 x 74)
 
 // The scratch ring (global memory, one per CTA), all of it in the order of the consumer's registers.  A slot for every chunk
 // of a segment: S_0 as B operand [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U as A operand [chain warp]
@@ -111,8 +112,8 @@ struct BwdSmem {
     static constexpr int db = scal + kSlots * NCW * 16 + 48;      // dbeta: [8][16] floats
     static constexpr int word = db + 8 * 16 * 4;                  // tensor-memory address
     static constexpr int job = word + 16;                         // the walk's current piece: pair, first and last position, gave up
-    static constexpr int gfree = job + 16;                        // GFREE: two barriers in shared memory
-    static constexpr int bytes = gfree + 16;
+    static constexpr int gfree = job + 16;                        // GFREE: two barriers in shared memory, and the flag of a wait that ran out
+    static constexpr int bytes = gfree + 32;
     static_assert(bytes <= 232448, "shared memory");
     static constexpr int columns = (NB + 63) / 64 * DK < 32 ? 32 : (NB + 63) / 64 * DK;   // S and G
 };
@@ -938,7 +939,7 @@ __device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned
     const RowScale sr = row_scale<4>(big);
     bool own = false;
     const float all = pub.ps ? shared_scale(sr, own) : 0.f;
-    const bool ok = wait();
+    wait();
     const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot), keys = KSP > 1 ? 32 * KN * hf.half : 0;
     const float *inv = reinterpret_cast<const float *>(slot + TL::oS);
     const uint32_t tiles[1] = {tile + TL::oW + keys};
@@ -950,7 +951,6 @@ __device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned
         });
         const float fw[2] = {sr.inv[0] * inv[0], sr.inv[1] * inv[0]};
         off = take_out(rr);
-        if (!ok) off = 0xffffffffu;
         if constexpr (KSP > 1) whole_sum(acc[0], fw, hf);
 #pragma unroll
         for (int n = 0; n < 2; ++n)
@@ -987,7 +987,7 @@ __device__ __forceinline__ float2 forward_step(uint32_t st, float2 big, unsigned
 // backward through one chunk: Bc = M^H (Y^* G + (A D_beta)^H Yb^*), G <- conj(gamma_C) G + Q^T Yb^* - W^T Bc.  load(yr, yi):
 // the chunk's rows of Yb^* (yi zero without has_im).  Leaves Re Bc (the rows of dv) in pr; returns the largest magnitudes of G.
 template <int DK, int KSP, bool kExact, typename Load>
-__device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigned char *slot, bool ok, Load load, bool has_im, float (&pr)[2][4],
+__device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigned char *slot, Load load, bool has_im, float (&pr)[2][4],
                                                 const Publish &pub, int lane, const Half &hf = Half())
 {
     using TL = Tile<DK>;
@@ -1001,7 +1001,6 @@ __device__ __forceinline__ float2 backward_step(uint32_t sg, float2 big, unsigne
         load(yr, yi);
         off = take_out(yr);
         if (has_im) off |= take_out(yi);
-        if (!ok) off = 0xffffffffu;
         ry = make_frag(fy, yr, yi);
     }
     const uint32_t tile = (uint32_t)__cvta_generic_to_shared(slot), keys = KSP > 1 ? 32 * KN * hf.half : 0;
@@ -1162,12 +1161,14 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_backward_c
     const int nch = (a.T + kC - 1) / kC;
     chain_begin<DK, NB, CL>(smem, tid);
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::slow);
+    const Wait limit = chain_limit<DK, NB, CL>(smem, (uint32_t)a.wait_ticks);
+    if (tid == 0 && blockIdx.x + blockIdx.y + blockIdx.z == 0) *a.status = 0;     // (set, if at all, by the launch behind this one)
     __syncthreads();
 
     if (tid < L::kPrep) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
         chain_prep<DK, NB, CL, T>(smem, static_cast<const T *>(a.q), static_cast<const T *>(a.k), a.alpha, a.theta, a.beta, row0, a.H, a.T, nch, back, back,
-                                  rank, tid);
+                                  rank, limit, tid);
     } else if (tid < L::kPrep + L::kSolve) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
         chain_solve<DK, NB, CL>(smem, nch, back, rank, tid - L::kPrep);
@@ -1186,7 +1187,7 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_backward_c
             unsigned char *tile = smem + slot * TL::bytes;
             const size_t at = (row0 + (size_t)(cc * kC + 2 * t4) * a.H) * DVT + col;
             const Half hf = L::KSP > 1 ? chain_half<DK, NB, CL>(smem, w, c, lane) : Half();
-            auto wait = [&] { return chain_wait<DK, NB, CL>(full, c); };
+            auto wait = [&] { chain_wait<DK, NB, CL>(full, c, limit, lane); };
             auto kept_at = [&](float *keep) { return kept<DK>(keep, bh, a.pitch, cc / kSegChunks, DVT, col0, lane) + 128 * KN * half; };
             if (!back) {
                 if (cc % kSegChunks == 0) keep_state<KN>(kept_at(a.keep_s), st);
@@ -1196,14 +1197,22 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_backward_c
                 if (c == 0 || cc % kSegChunks == kSegChunks - 1) keep_state<KN>(kept_at(a.keep_g), st);
                 float pr[2][4];
                 auto rows = [&](float(&x)[2][4], float(&y)[2][4]) { load_cotangents<T>(x, y, a.d_o, a.d_o_im, at, step, left); };
-                const bool ok = wait();
-                big = backward_step<DK, L::KSP, sizeof(T) == 2>(st, big, tile, ok, rows, a.d_o_im != nullptr, pr, none, lane, hf);
+                wait();
+                big = backward_step<DK, L::KSP, sizeof(T) == 2>(st, big, tile, rows, a.d_o_im != nullptr, pr, none, lane, hf);
             }
-            chain_release<DK, NB, CL>(full, c, nch, lane);
+            chain_release<DK, NB, CL>(full, c, nch, limit, lane);
         }
         if (back) state_to_memory<KN>(st, a.dS0 + state_at, DVT);
     }
-    chain_end<DK, NB, CL>(tmem, tid);
+    // where a wait ran out the kept states become NaN, so that all gradients that depend on them do (dv not on S), and dS0
+    const bool gave_up = chain_end<DK, NB, CL>(smem, tmem, limit, tid);
+    if (CL > 1 && tid == 0) a.flags[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = gave_up;
+    if (gave_up) {
+        const float nan = __int_as_float(0x7fc00000);
+        float *keep = (back ? a.keep_g : a.keep_s) + ((size_t)bh * a.pitch * DVT + c0) * DK;
+        for (size_t i = tid; i < (size_t)a.NS * NB * DK; i += L::threads) keep[i / (NB * DK) * DVT * DK + i % (NB * DK)] = nan;
+        for (int i = tid; back && i < DK * NB; i += L::threads) a.dS0[((size_t)bh * DK + i / NB) * DVT + c0 + i % NB] = nan;
+    }
 }
 
 // ---- the walk with gradients ------------------------------------------------------------------------------
@@ -1246,12 +1255,12 @@ __device__ __forceinline__ int3 walk_part(long long work, int c, int ctas, int N
     return make_int3(-1, 0, 0);
 }
 
-// NaN for every gradient of the first `tokens` tokens of pair bh and for dS0, by all threads of the CTA
+// NaN for every gradient of `tokens` tokens from t0 on of pair bh and, with `state`, for dS0, by all threads of the CTA
 template <int DK, int NB, typename T>
-__device__ __forceinline__ void give_up(const BwdArgsDev &a, int bh, int tokens, int tid, int threads)
+__device__ __forceinline__ void give_up(const BwdArgsDev &a, int bh, int t0, int tokens, bool state, int tid, int threads)
 {
     const float nan = __int_as_float(0x7fc00000);
-    const size_t row0 = (size_t)(bh / a.H) * a.T * a.H + bh % a.H;
+    const size_t row0 = (size_t)(bh / a.H) * a.T * a.H + bh % a.H + (size_t)t0 * a.H;
     for (int i = tid; i < tokens * DK; i += threads) {
         const size_t row = row0 + (size_t)(i / DK) * a.H;
         const int x = i % DK;
@@ -1261,7 +1270,7 @@ __device__ __forceinline__ void give_up(const BwdArgsDev &a, int bh, int tokens,
         if (x == 0) a.dbeta[row] = nan;
     }
     for (int i = tid; i < tokens * NB; i += threads) st_val(static_cast<T *>(a.dv), (row0 + (size_t)(i / NB) * a.H) * NB + i % NB, nan);
-    for (int i = tid; i < DK * NB; i += threads) a.dS0[(size_t)bh * DK * NB + i] = nan;
+    for (int i = tid; state && i < DK * NB; i += threads) a.dS0[(size_t)bh * DK * NB + i] = nan;
 }
 
 template <int DK, int NB, typename T, bool kUnits>
@@ -1325,12 +1334,15 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
         }
     };
     auto row_of = [&](int bh) { return (size_t)(bh / a.H) * a.T * a.H + bh % a.H; };
-    if (!a.flags && blockIdx.x == 0 && tid == 0) *a.status = 0;          // nothing waits (else the launcher has cleared it)
+    // the status word: cleared by the launcher where pieces are handed over, by the chains before units
+    if (!kUnits && !a.flags && blockIdx.x == 0 && tid == 0) *a.status = 0;
+    const Wait limit = {(uint32_t)__cvta_generic_to_shared(smem + L::gfree + 16), (uint32_t)a.wait_ticks};   // (of GFREE)
     if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::word), L::columns);
     if (places == 2 && tid == 32) {
         const uint32_t bar = (uint32_t)__cvta_generic_to_shared(smem + L::gfree);
         mbar_init(bar, kGradWarps);
         mbar_init(bar + 8, kGradWarps);
+        *reinterpret_cast<uint32_t *>(smem + L::gfree + 16) = 0;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -1342,6 +1354,8 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     if (tid < kGrad) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
         if constexpr (NB == 64) asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+        if (kUnits && blockIdx.x == 0 && tid < a.chain_ctas && a.flags[tid]) atomicOr(a.status, 1u);
+        __syncwarp();
 #pragma unroll 1
         for (int j = 0; next_part(j); ++j) {
             const int total = segments_of() * kSegChunks;
@@ -1350,7 +1364,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 const int r = n / kSegChunks, at = n % kSegChunks, c = kSegChunks - 1 - at, slot = ring_slot(r, c);
                 int bh, s;
                 segment(r, bh, s);
-                chunk_gradients<DK, NB, T>(a, smem, ring, slot, back_place(c, places), places == 2, n + 1 == total, s * kSeg + c * kC, row_of(bh), tid);
+                chunk_gradients<DK, NB, T>(a, smem, ring, slot, back_place(c, places), places == 2 && !limit.withheld(), n + 1 == total, s * kSeg + c * kC, row_of(bh), tid);
                 if (n + kSlots < total) bar_arrive(kBarReady + (n & 1), kGrad + kPrep);
             }
         }
@@ -1468,10 +1482,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 auto rows = [&](float(&x)[2][4]) {
                     load_rows(x, static_cast<const T *>(a.v) + (row0 + (size_t)(t0 + 2 * t4) * a.H) * NB + col, step, a.T - t0 - 2 * t4);
                 };
-                auto full = [&] {
-                    bar_sync(kBarFull + slot, kPrep + kChain);
-                    return true;
-                };
+                auto full = [&] { bar_sync(kBarFull + slot, kPrep + kChain); };
                 big_s = forward_step<DK, 1>(ss, big_s, smem + slot * TL::bytes, full, rows, pub, r < 0 || c + 1 < kSegChunks, lane);
                 if (r < 0) bar_arrive(kBarDone + slot, kPrep + kChain);
             }
@@ -1486,11 +1497,11 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 const int n = r * kSegChunks + kSegChunks - 1 - c;
                 unsigned char *scr = ring + (n & (places - 1)) * SC::place;
                 const Publish pub = {reinterpret_cast<uint4 *>(scr + SC::oG) + w * KT * 64 + lane, reinterpret_cast<uint4 *>(scr + SC::oB) + w * 128, scal + (slot * NCW + w) * 4 + 2};
-                bool ok = true;
-                if constexpr (places == 2) ok = mbar_wait((uint32_t)__cvta_generic_to_shared(smem + L::gfree) + 8 * (n & 1), ((n >> 1) + 1) & 1);
+                // (where this wait runs out the place is overwritten while it is read, and all of the CTA's gradients become NaN)
+                if constexpr (places == 2) cluster_wait<1>(limit.flag - 16 + 8 * (n & 1), ((n >> 1) + 1) & 1, limit, lane);
                 float pr[2][4];
                 auto rows = [&](float(&x)[2][4], float(&y)[2][4]) { load_cotangents<T>(x, y, a.d_o, a.d_o_im, at, step, left); };
-                big_g = backward_step<DK, 1, kExact>(sg, big_g, smem + slot * TL::bytes, ok, rows, a.d_o_im != nullptr, pr, pub, lane);
+                big_g = backward_step<DK, 1, kExact>(sg, big_g, smem + slot * TL::bytes, rows, a.d_o_im != nullptr, pr, pub, lane);
                 store_rows(static_cast<T *>(a.dv) + at, pr, step, left);
                 bar_arrive(kBarDone + slot, kPrep + kChain);
             }
@@ -1501,10 +1512,18 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
         }
     }
     if constexpr (!kUnits) {
-        if (job[3]) give_up<DK, NB, T>(a, job[0], min(a.T, (2 * NS - max(job[1], NS)) * kSeg), tid, kGrad + kPrep + kChain);
+        if (job[3]) give_up<DK, NB, T>(a, job[0], 0, min(a.T, (2 * NS - max(job[1], NS)) * kSeg), true, tid, kGrad + kPrep + kChain);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (places == 2 && limit.raised()) {
+        if (tid == 0) atomicOr(a.status, 1u);
+        for (int r = 0; r < segments_of(); ++r) {
+            int bh, s;
+            segment(r, bh, s);
+            give_up<DK, NB, T>(a, bh, s * kSeg, min(kSeg, a.T - s * kSeg), false, tid, kGrad + kPrep + kChain);
+        }
+    }
     if (tid < 32) tm_free(tmem, L::columns);
 }
 
@@ -1541,7 +1560,7 @@ cudaError_t launch_walk(const BwdArgsDev &a, int grid, cudaStream_t stream, int 
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = a.flags ? 1 : 0;                   // CTAs that wait for one another run together (one per SM)
+    attr[0].val.cooperative = !kUnits && a.flags ? 1 : 0;                 // CTAs that wait for one another run together (one per SM)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if ((e = cudaLaunchKernelEx(&cfg, kern, a)) != cudaSuccess) return e;
@@ -1576,6 +1595,7 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     a.ring_bytes = SC::bytes(ring_places(cols != DV));
     a.status = static_cast<unsigned *>(workspace);
     a.flags = nullptr;
+    a.chain_ctas = 0;
     a.wait_ticks = x.wait_ticks ? x.wait_ticks : 1ull << 31;     // about a second, more for long sequences
     if (!x.wait_ticks && (unsigned long long)a.NS * kSegChunks * kChunkTicks > a.wait_ticks) a.wait_ticks = (unsigned long long)a.NS * kSegChunks * kChunkTicks;
     a.withhold = x.withhold;
@@ -1602,6 +1622,9 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     int grid = a.units < kBwdTargetCtas ? a.units : kBwdTargetCtas;
     if ((size_t)grid * a.ring_bytes > room) grid = (int)(room / a.ring_bytes);
     const int nb = chain_columns(2LL * pairs, DV);               // both chains of all pairs at once
+    a.flags = a.status + 64;
+    a.chain_ctas = nb == DV ? 0 : 2 * pairs * (DV / nb);         // (those of clusters)
+    a.wait_ticks = wait_limit();
     cudaError_t e;
     if (nb == DV) e = launch_chains<DK, DV, 1, T>(a, pairs, stream, launches);
     else if (nb == 32) e = launch_chains<DK, 32, DV / 32, T>(a, pairs, stream, launches);

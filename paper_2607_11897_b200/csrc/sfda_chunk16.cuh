@@ -25,6 +25,7 @@
 // fragment in consecutive columns of its lane -- and passes through registers 16 columns at a time, requested one step
 // ahead; that also frees the 64 registers per thread it took.
 #pragma once
+#include <cstdlib>
 #include "sfda_common.cuh"
 
 namespace sfda {
@@ -1069,18 +1070,44 @@ __device__ __forceinline__ void store_lower(unsigned char *tile, const float2 *A
 
 // ---- a cluster's shared memory ---------------------------------------------------------------------
 // Barriers in shared memory: FULL (a slot's tile is complete) in every CTA, EMPTY (all CTAs are through with it) in the CTA
-// that makes the slot's tiles.  Waits are bounded; where one runs out (never, unless a CTA is gone) the results become NaN.
-constexpr uint32_t kWaitTries = 1u << 20;
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count)); }
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)       // by whole warps
-{
-#pragma unroll 1
-    for (uint32_t i = 0; i < kWaitTries; ++i) {
-        uint32_t ok;
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (__all_sync(0xffffffffu, ok)) return true;            // (the warp leaves together: what follows is for whole warps)
+// that makes the slot's tiles.  Every wait has a limit (never reached, unless a CTA is stuck).  The warp that gives up raises
+// a flag in all CTAs of the cluster and nobody waits any more: tiles may be overwritten while they are read.  So all
+// results of the pair are replaced by NaN at the end, what was computed before the wait included.
+constexpr uint32_t kWaitTicks = 1u << 31;                        // of the SM's clock, about a second
+#ifdef SFDA_WS_CHAOS
+// Development builds only: with SFDA_WITHHOLD in the environment some arrivals at these barriers are withheld and the limit is
+// short, so that waits run out.
+constexpr bool kWithhold = true;
+inline uint32_t wait_limit() { return getenv("SFDA_WITHHOLD") ? 1u << 18 : kWaitTicks; }
+#else
+constexpr bool kWithhold = false;
+inline uint32_t wait_limit() { return kWaitTicks; }
+#endif
+struct Wait {
+    uint32_t flag, limit;                                        // the CTA's flag (shared memory); SM-clock ticks
+    __device__ __forceinline__ bool raised() const
+    {
+        uint32_t x;
+        asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(x) : "r"(flag) : "memory");
+        return x != 0;
     }
+    __device__ __forceinline__ bool withheld() const { return kWithhold && limit != kWaitTicks; }
+};
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count)); }
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// By whole warps, which leave together (what follows is for whole warps); false: given up, by this warp or another.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const Wait &w)
+{
+    const uint32_t start = (uint32_t)clock(), limit = kWithhold ? w.limit : kWaitTicks;
+    do {
+        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    } while (!__any_sync(0xffffffffu, (uint32_t)clock() - start >= limit || w.raised()));
     return false;
 }
 __device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank)       // the same place in another CTA of the cluster
@@ -1088,6 +1115,15 @@ __device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank)       /
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
+}
+// A warp of a cluster of CL waits; where the wait runs out every CTA learns of it.
+template <int CL>
+__device__ __forceinline__ bool cluster_wait(uint32_t bar, uint32_t parity, const Wait &w, int lane)
+{
+    if (mbar_wait(bar, parity, w)) return true;
+    if (lane < CL) asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], 1;" ::"r"(in_cta(w.flag, lane)) : "memory");
+    __syncwarp();
+    return false;
 }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory"); }
 __device__ __forceinline__ void warp_arrive(uint32_t bar, uint32_t rank, int lane)   // once for the warp, when all of it is here
@@ -1130,7 +1166,8 @@ struct Chain {
     static constexpr int slow = scan + (PM::scan_bytes + 127) / 128 * 128;   // its first word also passes the tensor-memory address on
     static constexpr int part = slow + (PM::slow_bytes + 127) / 128 * 128;   // KSP: [chunk parity][warp][6][lane] float4
     static constexpr int bars = part + (KSP - 1) * 2 * warps * 3072;
-    static constexpr int bytes = bars + 2 * kSlots * 8;
+    static constexpr int sent = bars + 2 * kSlots * 8;           // per slot: tiles handed out; then the flag of a wait that ran out
+    static constexpr int flag = sent + kSlots * 4, bytes = flag + 16;
     static_assert(bytes <= 232448, "shared memory");
     // 8 KT / KSP columns for every four warps
     static constexpr int need = (warps + 3) / 4 * Tile<DK>::KT * 8 / KSP, columns = need < 32 ? 32 : need;
@@ -1144,10 +1181,13 @@ __device__ __forceinline__ void chain_begin(unsigned char *smem, int tid)
     if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::slow), L::columns);
     if (tid == 32) {
         const uint32_t bars = (uint32_t)__cvta_generic_to_shared(smem + L::bars);
+        uint32_t *sent = reinterpret_cast<uint32_t *>(smem + L::sent);
         for (int i = 0; i < kSlots; ++i) {
             mbar_init(bars + 8 * i, 2);
             mbar_init(bars + 8 * (kSlots + i), CL * L::warps);
+            sent[i] = 0;
         }
+        sent[kSlots] = 0;                                        // the flag
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1155,20 +1195,43 @@ __device__ __forceinline__ void chain_begin(unsigned char *smem, int tid)
     if constexpr (CL > 1) cluster_sync();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-// Every CTA's copies have arrived when its chain is through; nobody leaves before the others are.
 template <int DK, int NB, int CL>
-__device__ __forceinline__ void chain_end(uint32_t tmem, int tid)
+__device__ __forceinline__ Wait chain_limit(const unsigned char *smem, uint32_t limit)
 {
+    return {(uint32_t)__cvta_generic_to_shared(smem + Chain<DK, NB, CL>::flag), limit};
+}
+// Nobody leaves before the others are through.  Every CTA's copies have arrived when its chain is; where a wait has run out
+// (the answer, the same in all CTAs) that is waited for here: the last tile sent into a slot is the last phase of its FULL.
+template <int DK, int NB, int CL>
+__device__ __forceinline__ bool chain_end(unsigned char *smem, uint32_t tmem, const Wait &wait, int tid)
+{
+    using L = Chain<DK, NB, CL>;
+    bool gave_up = false;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if constexpr (CL > 1) cluster_sync();
-    if (tid < 32) tm_free(tmem, Chain<DK, NB, CL>::columns);
+    if constexpr (CL > 1) {
+        cluster_sync();
+        gave_up = wait.raised();
+        if (gave_up) {
+            const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
+            if (tid < kSlots) {
+                uint32_t sent;
+                asm volatile("ld.relaxed.cluster.shared::cluster.u32 %0, [%1];" : "=r"(sent) : "r"(in_cta(base + L::sent + 4 * tid, tid % CL)) : "memory");
+#pragma unroll 1
+                for (uint32_t i = 0; sent && i < 1u << 20 && !mbar_try(base + L::bars + 8 * tid, (sent - 1) & 1);) ++i;
+            }
+            __syncwarp();
+            cluster_sync();
+        }
+    }
+    if (tid < 32) tm_free(tmem, L::columns);
+    return gave_up;
 }
 
 // PREP of the chunks of rank `rank`, in the order of the chain (back: last to first)
 template <int DK, int NB, int CL, typename T>
 __device__ __forceinline__ void chain_prep(unsigned char *smem, const T *q, const T *k, const float *alpha, const float *theta, const float *beta,
-                                           size_t row0, int H, int T_, int nch, bool back, bool needq, int rank, int tid)
+                                           size_t row0, int H, int T_, int nch, bool back, bool needq, int rank, const Wait &wait, int tid)
 {
     using L = Chain<DK, NB, CL>;
     constexpr int PW = L::prep_warps;
@@ -1180,14 +1243,16 @@ __device__ __forceinline__ void chain_prep(unsigned char *smem, const T *q, cons
     for (int c = rank; c < nch; c += CL) {
         const int slot = c % kSlots, at = back ? nch - 1 - c : c, nx = back ? max(at - CL, 0) : at + CL;
         if (CL == 1 && c >= kSlots) bar_sync(kBarDone + slot, L::kPrep + L::kChain);
-        if (CL > 1 && c >= kSlots) ok = ok && mbar_wait(empty + 8 * slot, (c / kSlots - 1) & 1);
+        if (CL > 1) {                                            // a tile goes out only into a slot that all are through with
+            if (c >= kSlots) ok = ok && cluster_wait<CL>(empty + 8 * slot, (c / kSlots - 1) & 1, wait, tid & 31) && !wait.raised();
+            if (ok && tid == 0) reinterpret_cast<uint32_t *>(smem + L::sent)[slot] = c / kSlots + 1;
+        }
         PrepRaw<L::PM::TPT, T> next;
         prep_fetch<DK, PW, T>(next, q, k, alpha, theta, beta, row0, H, nx * kC, T_, needq, tid);
         unsigned char *tile = smem + slot * Tile<DK>::bytes, *kb = smem + L::kb + slot / CL * Tile<DK>::BIG;
         float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot / CL * L::gram_bytes);
         if (!prep_chunk<DK, PW, kBarAux, T>(in, q, k, alpha, theta, beta, row0, H, at * kC, T_, nullptr, tile, kb, smem + L::scan, needq, tid))
             slow_gram<DK, PW, kBarAux, T>(q, k, alpha, theta, beta, row0, H, at * kC, T_, smem + L::slow, smem + L::scan, gk, gk + 16 * 17, needq, tid);
-        if (!ok && tid == 0) reinterpret_cast<uint32_t *>(tile + Tile<DK>::oS)[7] = 0xffffffffu;
         if constexpr (CL > 1) fence_async_smem();
         bar_arrive(kBarPlanes + slot, L::kPrep + 64);
         in = next;
@@ -1204,7 +1269,6 @@ __device__ __forceinline__ void chain_solve(unsigned char *smem, int nch, bool n
     using TL = Tile<DK>;
     constexpr int pairs = L::own > 1 ? 2 : 1;
     const int lane = tid & 31, w = tid >> 5, out = w >> 1;
-    const bool other = CL > 1 && lane < CL && lane != rank;      // a lane per CTA to hand out to
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem), full = base + L::bars;
     if ((w & 1) >= pairs) return;
 #pragma unroll 1
@@ -1215,6 +1279,8 @@ __device__ __forceinline__ void chain_solve(unsigned char *smem, int nch, bool n
         float2 *gm = reinterpret_cast<float2 *>(smem + L::gram + slot / CL * L::gram_bytes) + out * 16 * 17;
         const uint32_t bar = full + 8 * slot, from = base + slot * TL::bytes;
         bar_sync(kBarPlanes + slot, L::kPrep + 64);
+        const bool send = CL > 1 && reinterpret_cast<const uint32_t *>(smem + L::sent)[slot] == c / kSlots + 1;
+        const bool other = send && lane < CL && lane != rank;    // a lane per CTA to hand out to
         if (out && other) copy_to_cta(from, TL::oM, bar, lane);
         __syncwarp();
         if (needq || !out) {
@@ -1235,7 +1301,7 @@ __device__ __forceinline__ void chain_solve(unsigned char *smem, int nch, bool n
             bar_sync(kBarPair + (w & 1), 64);
             if (other) copy_to_cta(from + TL::oM, TL::bytes - TL::oM, bar, lane);
         }
-        warp_arrive(bar, rank, lane);
+        if (send) warp_arrive(bar, rank, lane);
     }
 }
 
@@ -1243,18 +1309,18 @@ __device__ __forceinline__ void chain_solve(unsigned char *smem, int nch, bool n
 // EMPTY: a warp that waits at one in shared memory resumes a few hundred cycles late, 36.3 us instead of 34.8 for the forward of
 // B = 20, T = 104, H = 7, d_k = 64, d_v = 128.)
 template <int DK, int NB, int CL>
-__device__ __forceinline__ bool chain_wait(uint32_t full, int c)
+__device__ __forceinline__ void chain_wait(uint32_t full, int c, const Wait &wait, int lane)
 {
     const int slot = c % kSlots;
-    if constexpr (CL > 1) return mbar_wait(full + 8 * slot, (c / kSlots) & 1);
-    bar_sync(kBarFull + slot, 64 + Chain<DK, NB, CL>::kChain);
-    return true;
+    if constexpr (CL > 1) cluster_wait<CL>(full + 8 * slot, (c / kSlots) & 1, wait, lane);
+    else bar_sync(kBarFull + slot, 64 + Chain<DK, NB, CL>::kChain);
 }
 template <int DK, int NB, int CL>
-__device__ __forceinline__ void chain_release(uint32_t full, int c, int nch, int lane)
+__device__ __forceinline__ void chain_release(uint32_t full, int c, int nch, const Wait &wait, int lane)
 {
     const int slot = c % kSlots;
     if (c + kSlots >= nch) return;
+    if (CL > 1 && wait.withheld() && c % CL == 0) return;        // (the others learn of it by the flag)
     if constexpr (CL > 1) warp_arrive(full + 8 * (kSlots + slot), c % CL, lane);
     else bar_arrive(kBarDone + slot, Chain<DK, NB, CL>::kPrep + Chain<DK, NB, CL>::kChain);
 }

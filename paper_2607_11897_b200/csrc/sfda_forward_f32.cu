@@ -26,6 +26,7 @@ struct FwdArgsDev {
     void *o, *o_im;
     float *S_T;
     int T, H, dv;
+    uint32_t wait_ticks;                                         // limit of the waits on another CTA
 };
 
 template <int DK, int NB, int CL, typename T>
@@ -40,13 +41,14 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
     const int nch = (a.T + kC - 1) / kC;
     chain_begin<DK, NB, CL>(smem, tid);
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::slow);
+    const Wait wait = chain_limit<DK, NB, CL>(smem, a.wait_ticks);
     __syncthreads();
 
     // register shares with all 128 value columns: 256 x 88 + 128 x 72 + 256 x 112 of the launch's 640 x 96
     if (tid < L::kPrep) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
         chain_prep<DK, NB, CL, T>(smem, static_cast<const T *>(a.q), static_cast<const T *>(a.k), a.alpha, a.theta, a.beta, row0, a.H, a.T, nch, false, true,
-                                  rank, tid);
+                                  rank, wait, tid);
     } else if (tid < L::kPrep + L::kSolve) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
         chain_solve<DK, NB, CL>(smem, nch, true, rank, tid - L::kPrep);
@@ -66,7 +68,7 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
             float rr[2][4], ri[2][4];
             load_rows(rr, static_cast<const T *>(a.v) + at, step, left);
             const RowScale sr = row_scale<4>(largest);
-            const bool ok = chain_wait<DK, NB, CL>(base + L::bars, c);
+            chain_wait<DK, NB, CL>(base + L::bars, c, wait, lane);
             const uint32_t tile = base + slot * TL::bytes;
             const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
             float acc[2][2][2][4];
@@ -74,7 +76,6 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
             keys_product<DK, 2, KN>(acc, st, sr, tiles, lane, [](int, const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4], const uint32_t(&)[4]) {});
             const float fw[2] = {sr.inv[0] * inv[0], sr.inv[1] * inv[0]}, fq[2] = {sr.inv[0] * inv[2], sr.inv[1] * inv[2]};
             uint32_t off = take_out(rr);                         // tokens whose v is not finite; below, all behind them too
-            if (!ok) off = 0xffffffffu;
             // R in rr, ri; the outputs' part from S in pr, pi: all tokens, or the eight of this half
             constexpr int NT = 2 / L::KSP;
             float pr[NT][4], pi[NT][4];
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
                 put_nan(ru.inv, off);
             }
             largest = state_update<DK, KN>(st, fr, ru.inv, inv[1], tile + TL::oY + keys, reinterpret_cast<const float4 *>(smem + slot * TL::bytes + TL::oG) + 8 * KN * half, lane);
-            chain_release<DK, NB, CL>(base + L::bars, c, nch, lane);
+            chain_release<DK, NB, CL>(base + L::bars, c, nch, wait, lane);
 #pragma unroll
             for (int n = 0; n < NT; ++n)
 #pragma unroll
@@ -148,7 +149,15 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
         }
         if (a.S_T) state_to_memory<KN>(st, a.S_T + state_at, a.dv);
     }
-    chain_end<DK, NB, CL>(tmem, tid);
+    if (chain_end<DK, NB, CL>(smem, tmem, wait, tid)) {          // NaN for all of this CTA's results
+        const float nan = __int_as_float(0x7fc00000);
+        for (size_t i = tid; i < (size_t)a.T * NB; i += L::threads) {
+            const size_t at = (row0 + i / NB * a.H) * a.dv + c0 + i % NB;
+            st_val(static_cast<T *>(a.o), at, nan);
+            if (a.o_im) st_val(static_cast<T *>(a.o_im), at, nan);
+        }
+        for (int i = tid; a.S_T && i < DK * NB; i += L::threads) a.S_T[((size_t)bh * DK + i / NB) * a.dv + c0 + i % NB] = nan;
+    }
 }
 
 template <int DK, int NB, int CL, typename T>
@@ -159,6 +168,7 @@ cudaError_t launch_nb(const ForwardArgs &x, cudaStream_t stream)
     a.q = x.q; a.k = x.k; a.v = x.v; a.alpha = x.alpha; a.theta = x.theta; a.beta = x.beta; a.S0 = x.S0;
     a.o = x.o; a.o_im = x.o_im; a.S_T = x.S_T;
     a.T = x.T; a.H = x.H; a.dv = x.d_v;
+    a.wait_ticks = wait_limit();
     return launch_clusters(sfda_forward_f32_kernel<DK, NB, CL, T>, a, dim3((unsigned)(x.B * x.H), CL), L::threads, L::bytes, stream);
 }
 

@@ -283,3 +283,75 @@ def test_small_alpha_does_not_take_a_hundred_times_as_long():
     usual = ms()
     x[3].fill_(0.01)
     assert ms() <= 6 * usual
+
+
+# ------------------------------------------------------------------------------------------------
+# bounded waits between the CTAs of a cluster and between the roles of a unit that run out
+# ------------------------------------------------------------------------------------------------
+def all_nan(*tensors):
+    return all(bool(torch.isnan(t).all()) for t in tensors)
+
+
+@pytest.fixture
+def withheld(monkeypatch):
+    """Runs a function on the development build with some of the arrivals withheld, so that waits run out after 2^18 ticks."""
+    from paper_2607_11897_b200 import binding, build as cuda_build
+    dev, plain = binding.load_library(cuda_build.build_variant("chaos", ["-DSFDA_WS_CHAOS"])), binding.load()
+
+    def run(fn):
+        with monkeypatch.context() as m:
+            m.setenv("SFDA_WITHHOLD", "1")
+            m.setattr(binding, "_LIB", dev)
+            return fn()
+    assert binding.load() is plain
+    return run
+
+
+@pytest.mark.parametrize("H,T,d_k,d_v", [(2, 64, 128, 128), (2, 81, 128, 128), (2, 200, 64, 64), (40, 200, 128, 128)])
+def test_forward_waits_that_run_out_leave_nothing_but_nan(withheld, H, T, d_k, d_v):
+    """A CTA that never hears that a tile has been used overwrites it while others may read it: from the fifth chunk on,
+    all results of the pair are NaN, those of earlier tokens too; shorter sequences never wait."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16w", B=1, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=T + H)
+    inp = workloads.forward_inputs(cfg)
+    want = run_forward(cfg, inp)
+    got = withheld(lambda: run_forward(cfg, inp))
+    for x, y in zip(got, want):
+        if T <= 64:
+            assert np.array_equal(x, y)
+        else:
+            assert np.isnan(x).all()
+    for x, y in zip(run_forward(cfg, inp), want):                # the context is intact
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("H,T,d_k,d_v", [(2, 60, 128, 128), (2, 200, 128, 128), (3, 200, 64, 64), (20, 130, 64, 128), (38, 200, 128, 128)])
+def test_backward_waits_that_run_out_are_reported(withheld, H, T, d_k, d_v):
+    """SFDA_ERR_TIMEOUT and NaN in every gradient: of the units where the scratch's places are never given back (a segment alone
+    has waits), of the whole pair where the chains wait in vain as well (more than four chunks, in clusters: up to 37 pairs)."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16v", B=1, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=T + H)
+    x, u, out, ws = backward_tensors(cfg, workloads.forward_inputs(cfg), upstream(cfg, T))
+
+    def run():
+        sfda.sfda_backward(*x, *u, *out, ws)
+        torch.cuda.synchronize()
+        return [t.clone() for t in out]
+
+    want = run()
+    assert sfda.sfda_workspace_status(ws) == 0
+
+    def run_out():
+        grads = run()
+        with pytest.raises(sfda.SfdaError) as e:
+            sfda.sfda_workspace_status(ws)
+        assert e.value.status == -7
+        return grads
+
+    got = withheld(run_out)
+    assert all_nan(*got[:6])
+    if T > 64 and H <= 37:
+        assert all_nan(got[6])
+    else:                                                        # dS0 comes from the chains, which waited for nothing
+        assert torch.equal(got[6], want[6])
+    for a, b in zip(run(), want):                                # the context and the workspace are intact
+        assert torch.equal(a, b)
+    assert sfda.sfda_workspace_status(ws) == 0
