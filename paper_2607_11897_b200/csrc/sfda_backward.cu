@@ -1148,14 +1148,14 @@ __device__ __forceinline__ float4 *kept(float *keep, int bh, int pitch, int s, i
 // With less than half as many sequences as SMs the walk of one CTA per sequence leaves the device idle.  But the
 // cotangent's chain needs neither S nor U: so S walks forward and G backward at the same time, each in blocks of value
 // columns (NB), both kept every 64 tokens; then every segment's gradients are a unit of their own (kUnits below).
-template <int DK, int NB, int CL, typename T>
+template <int DK, int NB, int CL, int DVT, typename T>
 __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_backward_chain_kernel(const BwdArgsDev a)
 {
     using TL = Tile<DK>;
     using L = Chain<DK, NB, CL>;
-    constexpr int KN = L::KN, DVT = NB * CL;
+    constexpr int KN = L::KN;
     extern __shared__ __align__(128) unsigned char smem[];
-    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, rank = CL > 1 ? blockIdx.y : 0, c0 = rank * NB;
+    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, rank = blockIdx.y % CL, c0 = blockIdx.y * NB;
     const bool back = blockIdx.z != 0;
     const size_t row0 = (size_t)b * a.T * a.H + h;
     const int nch = (a.T + kC - 1) / kC;
@@ -1568,12 +1568,12 @@ cudaError_t launch_walk(const BwdArgsDev &a, int grid, cudaStream_t stream, int 
     return cudaGetLastError();
 }
 
-template <int DK, int NB, int CL, typename T>
+template <int DK, int NB, int CL, int DV, typename T>
 cudaError_t launch_chains(const BwdArgsDev &a, int pairs, cudaStream_t stream, int *launches)
 {
     using L = Chain<DK, NB, CL>;
     if (launches) ++*launches;
-    return launch_clusters(sfda_backward_chain_kernel<DK, NB, CL, T>, a, dim3((unsigned)pairs, CL, 2), L::threads, L::bytes, stream);
+    return launch_clusters(sfda_backward_chain_kernel<DK, NB, CL, DV, T>, a, dim3((unsigned)pairs, DV / NB, 2), CL, L::threads, L::bytes, stream);
 }
 
 template <int DK, int DV, typename T>
@@ -1621,14 +1621,15 @@ cudaError_t launch_typed(const BackwardArgs &x, void *workspace, cudaStream_t st
     const size_t room = bwd_workspace(x.B, x.T, x.H, DK, DV) * sizeof(float) - kHeadBytes - (size_t)(rings - ws) * sizeof(float);
     int grid = a.units < kBwdTargetCtas ? a.units : kBwdTargetCtas;
     if ((size_t)grid * a.ring_bytes > room) grid = (int)(room / a.ring_bytes);
-    const int nb = chain_columns(2LL * pairs, DV);               // both chains of all pairs at once
+    const Blocks b = chain_blocks(2LL * pairs, DV);              // both chains of all pairs at once
     a.flags = a.status + 64;
-    a.chain_ctas = nb == DV ? 0 : 2 * pairs * (DV / nb);         // (those of clusters)
+    a.chain_ctas = b.cluster > 1 ? 2 * pairs * (DV / b.columns) : 0;
     a.wait_ticks = wait_limit();
     cudaError_t e;
-    if (nb == DV) e = launch_chains<DK, DV, 1, T>(a, pairs, stream, launches);
-    else if (nb == 32) e = launch_chains<DK, 32, DV / 32, T>(a, pairs, stream, launches);
-    else e = launch_chains<DK, 64, DV / 64, T>(a, pairs, stream, launches);
+    if (b.columns == DV) e = launch_chains<DK, DV, 1, DV, T>(a, pairs, stream, launches);
+    else if (b.columns == 64) e = launch_chains<DK, 64, DV / 64, DV, T>(a, pairs, stream, launches);
+    else if (b.cluster == 2) e = launch_chains<DK, 32, 2, DV, T>(a, pairs, stream, launches);
+    else e = launch_chains<DK, 32, DV / 32, DV, T>(a, pairs, stream, launches);
     return e == cudaSuccess ? launch_walk<DK, DV, T, true>(a, grid, stream, launches) : e;
 }
 

@@ -1144,7 +1144,7 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 __device__ __forceinline__ void cluster_sync() { asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // ---- kernels that run a chain and nothing else: PREP, SOLVE, CHAIN -----------------------------------
-// A pair's CTAs (blocks of NB value columns) are a cluster of CL: the tile of chunk c is made by CTA c % CL alone and copied
+// A pair's CTAs (blocks of NB value columns) are clusters of CL (mostly one cluster): the tile of chunk c is made by CTA c % CL alone and copied
 // to the others' shared memory, so that the preparation, which does not depend on the columns, is done once per pair.  It
 // had been half of what a CTA of 32 columns issued (13.4 k of 27.6 k issue cycles per chunk; mma.sync holds its scheduler
 // for 8.2 cycles, and 0.7 more for every other instruction issued meanwhile).  With 32 columns two warps share a block of
@@ -1356,17 +1356,25 @@ __device__ __forceinline__ Half chain_half(unsigned char *smem, int w, int c, in
     return {half, kBarHalf + block, p, half ? -192 : 192};
 }
 
-// Value columns per CTA for `walks` sequences that a chain kernel takes at once: all of them, halved (down to 32) while the
-// clusters fit the SMs together: 74 of two, 32 of four (a GPC has 16 to 20 SMs).  (Those of a B200; on another device the
-// blocks are merely not the best ones.)
-inline int chain_columns(long long walks, int d_v)
+// Value columns per CTA for `walks` sequences that a chain kernel takes at once, and CTAs per cluster: all columns, halved (down
+// to 32) while the CTAs fit the SMs.  Clusters of two fit all SMs (74), of clusters of four 33 at a time (asked of the driver; 32
+// here, as other parts may have lost other SMs).  So 33 to 37 sequences of 128 columns have two clusters of two each, and every
+// chunk is prepared twice: 37 sequences of 520 tokens 126 us at d_k = 128, 74 us at 64, with blocks of 64 columns 138 and 95,
+// with CTAs that prepare everything for themselves 125 and 76.  (Only where every decay is too strong to divide by are 64 columns
+// better, 166 us instead of 207; without clusters 303.)  On a device with other SMs the blocks are merely not the best ones.
+struct Blocks {
+    int columns, cluster;
+};
+inline Blocks chain_blocks(long long walks, int d_v)
 {
-    int nb = d_v;
-    while (nb > 32 && walks <= (d_v == nb ? 74 : 32)) nb /= 2;
-    return nb;
+    Blocks b = {d_v, 1};
+    while (b.columns > 32 && walks * (2 * d_v / b.columns) <= 148) b.columns /= 2;
+    b.cluster = d_v / b.columns;
+    if (b.cluster == 4 && walks > 32) b.cluster = 2;
+    return b;
 }
 template <typename Args>
-cudaError_t launch_clusters(void (*kern)(Args), const Args &a, dim3 grid, int threads, int bytes, cudaStream_t stream)
+cudaError_t launch_clusters(void (*kern)(Args), const Args &a, dim3 grid, int cluster, int threads, int bytes, cudaStream_t stream)
 {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
@@ -1378,10 +1386,10 @@ cudaError_t launch_clusters(void (*kern)(Args), const Args &a, dim3 grid, int th
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1;
-    attr[0].val.clusterDim.y = grid.y;                           // the blocks of columns of a pair
+    attr[0].val.clusterDim.y = cluster;                          // neighbouring blocks of columns of a pair
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = grid.y > 1 ? 1 : 0;
+    cfg.numAttrs = cluster > 1 ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 

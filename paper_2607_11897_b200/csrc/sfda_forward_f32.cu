@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
     using L = Chain<DK, NB, CL>;
     constexpr int KN = L::KN;
     extern __shared__ __align__(128) unsigned char smem[];
-    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB, rank = CL > 1 ? blockIdx.y : 0;
+    const int tid = threadIdx.x, bh = blockIdx.x, h = bh % a.H, b = bh / a.H, c0 = blockIdx.y * NB, rank = blockIdx.y % CL;
     const size_t row0 = (size_t)b * a.T * a.H + h;               // row of token t: row0 + t H
     const int nch = (a.T + kC - 1) / kC;
     chain_begin<DK, NB, CL>(smem, tid);
@@ -169,18 +169,16 @@ cudaError_t launch_nb(const ForwardArgs &x, cudaStream_t stream)
     a.o = x.o; a.o_im = x.o_im; a.S_T = x.S_T;
     a.T = x.T; a.H = x.H; a.dv = x.d_v;
     a.wait_ticks = wait_limit();
-    return launch_clusters(sfda_forward_f32_kernel<DK, NB, CL, T>, a, dim3((unsigned)(x.B * x.H), CL), L::threads, L::bytes, stream);
+    return launch_clusters(sfda_forward_f32_kernel<DK, NB, CL, T>, a, dim3((unsigned)(x.B * x.H), x.d_v / NB), CL, L::threads, L::bytes, stream);
 }
 
-// Value columns per CTA: all of them when the (batch, head) pairs fill the SMs, halved (down to 32) while the clusters
-// still fit.
 template <int DK, typename T>
 cudaError_t launch_typed(const ForwardArgs &x, cudaStream_t stream)
 {
-    const int nb = chain_columns((long long)x.B * x.H, x.d_v);
-    if (nb == 128) return launch_nb<DK, 128, 1, T>(x, stream);
-    if (nb == 64) return x.d_v == 128 ? launch_nb<DK, 64, 2, T>(x, stream) : launch_nb<DK, 64, 1, T>(x, stream);
-    return x.d_v == 128 ? launch_nb<DK, 32, 4, T>(x, stream) : launch_nb<DK, 32, 2, T>(x, stream);
+    const Blocks b = chain_blocks((long long)x.B * x.H, x.d_v);
+    if (b.columns == 128) return launch_nb<DK, 128, 1, T>(x, stream);
+    if (b.columns == 64) return b.cluster == 2 ? launch_nb<DK, 64, 2, T>(x, stream) : launch_nb<DK, 64, 1, T>(x, stream);
+    return b.cluster == 4 ? launch_nb<DK, 32, 4, T>(x, stream) : launch_nb<DK, 32, 2, T>(x, stream);
 }
 
 }  // namespace
