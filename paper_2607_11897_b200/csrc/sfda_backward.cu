@@ -77,7 +77,7 @@ static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags 
 // of a segment: S_0 as B operand [chain warp][key tile][Re / Im][lane] uint4 (two heads, two tails); U as A operand [chain warp]
 // [plane][lane] uint4; the chunk's decays and phases, 4 floats per (token, key).  Behind the slots slow_gram's scratch and four
 // or two places in turn for G_C and Bc likewise.  With two the chain that comes back waits until the gradients have used up
-// what lies there (GFREE); see ring_places.  The rotated keys and queries, which only the rare paths want, are not kept (Rotated):
+// what lies there (GFREE); see ring_places.  The rotated keys and queries, which only the rare paths want, are made again there (Rotated):
 // 704 KB with four places for d_k = d_v = 128 instead of 768, of which every chunk writes and reads 176 instead of 192.
 // Training step at the headline sizes 29.5 -> 28.2 ms, B = 4, T = 4096, H = 16: 4.43 -> 4.29 ms.
 template <int DK, int NB>
@@ -168,26 +168,30 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) { return make_float2(
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) { return make_float2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }   // conj(a) b
 
 // ---- the gradients where decays are too strong to divide by, or alpha too small -----------------------------
-// The rotated key and query (k'_t, q'_t) of a token of the chunk, as PREP made them: from the caller's arrays and the phases in
-// `vals`; zero behind the sequence and where PREP took a token out (`out`, see Tile).
-template <typename T>
+// The rotated keys and queries (k'_t, q'_t) of a warp's eight keys, as PREP made them: from the caller's arrays and the phases in
+// `vals`; zero behind the sequence and where PREP took a token out (`out`, see Tile).  They lie where the warp has read its key
+// tile of S_0: tokens 0-7 in the first chain warp's kilobyte, 8-15 in the second's.  Made again at each use, element
+// by element in the loops below, they cost a quarter: 200 sequences of 1000 tokens with alpha ~ U(0, 1) 14.2 ms, 10.9 ms so (11.3
+// when PREP wrote them for every chunk), a not finite token in each 9.8 and 8.4 (8.3); 148 of 333 with alpha = 0.01 3.31 and 2.60 (2.65).
+template <int DK>
 struct Rotated {
-    const T *k, *q;                                              // the pair's first row
-    const float4 *vals;
-    int M, left;
-    size_t step;                                                 // from one token to the next
-    uint32_t out;
-    __device__ Rotated(const BwdArgsDev &a, const float4 *v, int m, size_t row0, int t0, uint32_t o)
-        : k(static_cast<const T *>(a.k) + (row0 + (size_t)t0 * a.H) * 2 * m), q(static_cast<const T *>(a.q) + (row0 + (size_t)t0 * a.H) * 2 * m), vals(v), M(m),
-          left(a.T - t0), step((size_t)a.H * 2 * m), out(o) {}
-    __device__ __forceinline__ float4 operator()(int t, int key) const
+    float4 *at;
+    __device__ __forceinline__ float4 &operator()(int t, int key) const { return at[(t >> 3) * Tile<DK>::KT * 64 + (t & 7) * 8 + (key & 7)]; }
+    template <typename T>
+    __device__ __forceinline__ void make(const BwdArgsDev &a, const float4 *vals, size_t row0, int t0, uint32_t out, int warp, int lane) const
     {
-        const float4 v = vals[t * M + key];                      // -, -, cos, sin
-        const size_t at = t * step + 2 * key;
-        const bool on = t < left && !(out >> t & 1), onq = t < left && !(out >> (16 + t) & 1);
-        const float kx = on ? ld_val(k, at) : 0.f, ky = on ? ld_val(k, at + 1) : 0.f;
-        const float qx = onq ? ld_val(q, at) : 0.f, qy = onq ? ld_val(q, at + 1) : 0.f;
-        return make_float4(kx * v.z + ky * v.w, ky * v.z - kx * v.w, qx * v.z + qy * v.w, qy * v.z - qx * v.w);
+#pragma unroll 1
+        for (int i = lane; i < 128; i += 32) {
+            const int t = i >> 3, key = 8 * warp + (i & 7);
+            const size_t x = (row0 + (size_t)(t0 + t) * a.H) * DK + 2 * key;
+            const bool on = t0 + t < a.T;
+            const float4 v = vals[t * (DK / 2) + key];           // -, -, cos, sin
+            float2 k = make_float2(0.f, 0.f), q = k;
+            if (on && !(out >> t & 1)) k = make_float2(ld_val(static_cast<const T *>(a.k), x), ld_val(static_cast<const T *>(a.k), x + 1));
+            if (on && !(out >> (16 + t) & 1)) q = make_float2(ld_val(static_cast<const T *>(a.q), x), ld_val(static_cast<const T *>(a.q), x + 1));
+            (*this)(t, key) = make_float4(k.x * v.z + k.y * v.w, k.y * v.z - k.x * v.w, q.x * v.z + q.y * v.w, q.y * v.z - q.x * v.w);
+        }
+        __syncwarp();
     }
 };
 
@@ -196,14 +200,15 @@ struct Rotated {
 struct SlowOut {
     float2 qb, zb, fb;
 };
-template <typename T>
-__device__ __forceinline__ SlowOut slow_corrections(const Rotated<T> &rotated, int M, const float2 *uy, const float *alpha, const float *beta,
+template <int DK>
+__device__ __forceinline__ SlowOut slow_corrections(const Rotated<DK> &rotated, const float2 *uy, const float *alpha, const float *beta,
                                                  size_t row0, int H, int t0, int T_, int tl, int key, float2 x1, float2 x2, float2 x3)
 {
     auto at = [&](int mat, int i, int t) {
         const float2 x = uy[mat * 272 + i * 17 + t], y = uy[544 + mat * 272 + i * 17 + t];
         return make_float2(x.x + y.x, x.y + y.y);
     };
+    constexpr int M = DK / 2;
     SlowOut o;
     float w = 1.f;
     o.qb = o.zb = o.fb = make_float2(0.f, 0.f);
@@ -241,8 +246,8 @@ __device__ __forceinline__ SlowOut slow_corrections(const Rotated<T> &rotated, i
 // or r0 = sum_c conj(S_0) G_C; decays come as running products.  x: the thread's tokens g, g + 8 and keys 2 t4, + 1.
 // redo: bit 2 r + e says that this element is wanted; it goes to the caller's arrays.
 // (Rebuilding both matrices per element, column by column, took 6.4 M cycles a chunk where every alpha is small.)
-template <int DK, typename T>
-__device__ __forceinline__ void from_definition(const BwdArgsDev &a, const Rotated<T> &rotated, const float2 *uy, const float2 (&r0)[2],
+template <int DK>
+__device__ __forceinline__ void from_definition(const BwdArgsDev &a, const Rotated<DK> &rotated, const float4 *vals, const float2 *uy, const float2 (&r0)[2],
                                                 const float (&x1r)[4], const float (&x1i)[4], const float (&x2r)[4], const float (&x2i)[4],
                                                 const float (&x3r)[4], const float (&x3i)[4], unsigned redo, size_t row0, int t0, int kt, int lane)
 {
@@ -311,7 +316,7 @@ __device__ __forceinline__ void from_definition(const BwdArgsDev &a, const Rotat
         const size_t row = row0 + (size_t)(t0 + t) * a.H;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const float4 v = rotated.vals[15 * M + key + e];       // -, -, e^{i phi_C}
+            const float4 v = vals[15 * M + key + e];               // -, -, e^{i phi_C}
             const float2 end = make_float2(pz[e] * v.z, -pz[e] * v.w), z0 = cmul(end, r0[e]), zx = cmul(end, sx[e]);
             const float hr = fmaf(pw[e], h[e].x + z0.x, su[e].x + zx.x), hi = fmaf(pw[e], h[e].y + z0.y, su[e].y + zx.y);
             if (redo >> (2 * r + e) & 1) {
@@ -487,7 +492,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
     float *scal = reinterpret_cast<float *>(smem + L::scal), *yscal = scal + kSlots * NCW * 4, *tscal = yscal + 8;
     const float *sc = scal + slot * NCW * 4;
     float *db = reinterpret_cast<float *>(smem + L::db);
-    const unsigned char *scr = ring + slot * SC::slot;
+    unsigned char *scr = ring + slot * SC::slot;
     const uint4 *pS = reinterpret_cast<const uint4 *>(scr + SC::oS), *pG = reinterpret_cast<const uint4 *>(ring + SC::oG + place * SC::place);
     const float4 *vals = reinterpret_cast<const float4 *>(scr + SC::oV);
 
@@ -645,9 +650,11 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         const bool some = __any_sync(0xffffffffu, redo != 0);
         const float *inv = reinterpret_cast<const float *>(smem + slot * TL::bytes + TL::oS);
         const uint32_t out = reinterpret_cast<const uint32_t *>(inv)[7];
-        if (some)
-            from_definition<DK, T>(a, Rotated<T>(a, vals, M, row0, t0, out), uy, r0, x1r, x1i, x2r, x2i, x3r, x3i, redo, row0, t0, warp, lane);
         const bool fast = reinterpret_cast<const int *>(inv)[6] != 0;
+        const Rotated<DK> rotated = {reinterpret_cast<float4 *>(scr + SC::oS) + warp * 64};
+        if (some || !fast) rotated.template make<T>(a, vals, row0, t0, out, warp, lane);
+        if (some)
+            from_definition<DK>(a, rotated, vals, uy, r0, x1r, x1i, x2r, x2i, x3r, x3i, redo, row0, t0, warp, lane);
         const unsigned char *slot_at = smem + slot * TL::bytes;
         // from here on x1, x2, x3 become S_t yb_t, Lambda_t S_{t-1} b_t, G_t conj(u_t) in the rotated frame
         if (fast) {
@@ -716,7 +723,6 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 x3i[i] = fmaf(s, z.y, down * fmaf(f2, zi[i], f3 * wi[i]));
             }
         } else {
-            const Rotated<T> rotated(a, vals, M, row0, t0, out);
 #pragma unroll 1
             for (int i = 0; i < 4; ++i) {                          // (no function and no indexed registers: both cost the common path)
                 auto pick = [&](const float(&v)[4]) { return i == 0 ? v[0] : i == 1 ? v[1] : i == 2 ? v[2] : v[3]; };
@@ -726,7 +732,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 };
                 const int tl = g + 8 * (i >> 1), key = 8 * warp + 2 * t4 + (i & 1);
                 const float4 lv = vals[15 * M + key];              // -, -, e^{i phi_C}
-                const SlowOut o = slow_corrections(rotated, M, uy, a.alpha, a.beta, row0, a.H, t0, a.T, tl, key, make_float2(pick(x1r), pick(x1i)),
+                const SlowOut o = slow_corrections<DK>(rotated, uy, a.alpha, a.beta, row0, a.H, t0, a.T, tl, key, make_float2(pick(x1r), pick(x1i)),
                                                    make_float2(pick(x2r), pick(x2i)), cmulc(make_float2(lv.z, lv.w), make_float2(pick(x3r), pick(x3i))));
                 put(x1r, o.qb.x);
                 put(x1i, o.qb.y);
@@ -741,7 +747,7 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
         float al[4], dbp[2] = {0.f, 0.f};
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            // rotated key and query of the two keys: from the planes (W = a k', Q = a q'), or made again
+            // rotated key and query of the two keys: from the planes (W = a k', Q = a q'), or as above
             const int tl = g + 8 * r;
             const float4 *p = vals + tl * M + 8 * warp + 2 * t4;
             float2 kr, ki, qr, qi;
@@ -758,7 +764,6 @@ __device__ __forceinline__ void chunk_gradients(const BwdArgsDev &a, unsigned ch
                 qr = both(TL::oQ, fq);
                 qi = both(TL::oQ + 2 * TL::PL, fq);
             } else {
-                const Rotated<T> rotated(a, vals, M, row0, t0, out);
                 const float4 u = rotated(tl, 8 * warp + 2 * t4), v = rotated(tl, 8 * warp + 2 * t4 + 1);
                 kr = make_float2(u.x, v.x);
                 ki = make_float2(u.y, v.y);
