@@ -1215,7 +1215,9 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_backward_c
     if (gave_up) {
         const float nan = __int_as_float(0x7fc00000);
         float *keep = (back ? a.keep_g : a.keep_s) + ((size_t)bh * a.pitch * DVT + c0) * DK;
+#pragma unroll 1
         for (size_t i = tid; i < (size_t)a.NS * NB * DK; i += L::threads) keep[i / (NB * DK) * DVT * DK + i % (NB * DK)] = nan;
+#pragma unroll 1
         for (int i = tid; back && i < DK * NB; i += L::threads) a.dS0[((size_t)bh * DK + i / NB) * DVT + c0 + i % NB] = nan;
     }
 }
@@ -1266,6 +1268,7 @@ __device__ __forceinline__ void give_up(const BwdArgsDev &a, int bh, int t0, int
 {
     const float nan = __int_as_float(0x7fc00000);
     const size_t row0 = (size_t)(bh / a.H) * a.T * a.H + bh % a.H + (size_t)t0 * a.H;
+#pragma unroll 1
     for (int i = tid; i < tokens * DK; i += threads) {
         const size_t row = row0 + (size_t)(i / DK) * a.H;
         const int x = i % DK;
@@ -1274,7 +1277,9 @@ __device__ __forceinline__ void give_up(const BwdArgsDev &a, int bh, int t0, int
         if (x < DK / 2) a.dalpha[row * (DK / 2) + x] = a.dtheta[row * (DK / 2) + x] = nan;
         if (x == 0) a.dbeta[row] = nan;
     }
+#pragma unroll 1
     for (int i = tid; i < tokens * NB; i += threads) st_val(static_cast<T *>(a.dv), (row0 + (size_t)(i / NB) * a.H) * NB + i % NB, nan);
+#pragma unroll 1
     for (int i = tid; state && i < DK * NB; i += threads) a.dS0[(size_t)bh * DK * NB + i] = nan;
 }
 
@@ -1354,6 +1359,20 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *reinterpret_cast<const uint32_t *>(smem + L::word);
 
+    // Where a wait for GFREE ran out: NaN for all gradients of this CTA's segments.  By the gradients' warps with 128 value columns, by
+    // all threads with 64: at the end of the kernel it costs the former's code 1 % (training step at B = 4, T = 4096, H = 16 4.22 -> 4.17
+    // ms), among the gradients it costs the latter's 2 % (fp32 segments of 64 / 64 at B H = 8, T = 333 101 us instead of 99).
+    auto give_up_units = [&](int threads) {
+        if (places != 2 || !limit.raised()) return;
+        if (tid == 0) atomicOr(a.status, 1u);
+#pragma unroll 1
+        for (int r = 0; r < segments_of(); ++r) {
+            int bh, s;
+            segment(r, bh, s);
+            give_up<DK, NB, T>(a, bh, s * kSeg, min(kSeg, a.T - s * kSeg), false, tid, threads);
+        }
+    };
+
     // register shares: 256 x (88 + 64 + 88) of 768 x 80 with 128 value columns; 256 x (104 + 80) + 128 x 112 of 640 x 96
     // with 64
     if (tid < kGrad) {
@@ -1372,6 +1391,10 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
                 chunk_gradients<DK, NB, T>(a, smem, ring, slot, back_place(c, places), places == 2 && !limit.withheld(), n + 1 == total, s * kSeg + c * kC, row_of(bh), tid);
                 if (n + kSlots < total) bar_arrive(kBarReady + (n & 1), kGrad + kPrep);
             }
+        }
+        if constexpr (NB == 128) {                               // (the chain is through with what these warps have used)
+            bar_sync(kBarGrad, kGrad);
+            give_up_units(kGrad);
         }
     } else if (tid < kGrad + kPrep) {
         if constexpr (NB == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
@@ -1521,14 +1544,7 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (places == 2 && limit.raised()) {
-        if (tid == 0) atomicOr(a.status, 1u);
-        for (int r = 0; r < segments_of(); ++r) {
-            int bh, s;
-            segment(r, bh, s);
-            give_up<DK, NB, T>(a, bh, s * kSeg, min(kSeg, a.T - s * kSeg), false, tid, kGrad + kPrep + kChain);
-        }
-    }
+    if constexpr (NB == 64) give_up_units(kGrad + kPrep + kChain);
     if (tid < 32) tm_free(tmem, L::columns);
 }
 

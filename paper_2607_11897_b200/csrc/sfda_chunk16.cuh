@@ -1243,16 +1243,14 @@ __device__ __forceinline__ void chain_prep(unsigned char *smem, const T *q, cons
     for (int c = rank; c < nch; c += CL) {
         const int slot = c % kSlots, at = back ? nch - 1 - c : c, nx = back ? max(at - CL, 0) : at + CL;
         if (CL == 1 && c >= kSlots) bar_sync(kBarDone + slot, L::kPrep + L::kChain);
-        if (CL > 1) {                                            // a tile goes out only into a slot that all are through with
-            if (c >= kSlots) ok = ok && cluster_wait<CL>(empty + 8 * slot, (c / kSlots - 1) & 1, wait, tid & 31) && !wait.raised();
-            if (ok && tid == 0) reinterpret_cast<uint32_t *>(smem + L::sent)[slot] = c / kSlots + 1;
-        }
+        if (CL > 1 && c >= kSlots) ok = ok && cluster_wait<CL>(empty + 8 * slot, (c / kSlots - 1) & 1, wait, tid & 31) && !wait.raised();
         PrepRaw<L::PM::TPT, T> next;
         prep_fetch<DK, PW, T>(next, q, k, alpha, theta, beta, row0, H, nx * kC, T_, needq, tid);
         unsigned char *tile = smem + slot * Tile<DK>::bytes, *kb = smem + L::kb + slot / CL * Tile<DK>::BIG;
         float2 *gk = reinterpret_cast<float2 *>(smem + L::gram + slot / CL * L::gram_bytes);
         if (!prep_chunk<DK, PW, kBarAux, T>(in, q, k, alpha, theta, beta, row0, H, at * kC, T_, nullptr, tile, kb, smem + L::scan, needq, tid))
             slow_gram<DK, PW, kBarAux, T>(q, k, alpha, theta, beta, row0, H, at * kC, T_, smem + L::slow, smem + L::scan, gk, gk + 16 * 17, needq, tid);
+        if (CL > 1 && ok && tid == 0) reinterpret_cast<uint32_t *>(smem + L::sent)[slot] = c / kSlots + 1;   // only into a slot that all are through with
         if constexpr (CL > 1) fence_async_smem();
         bar_arrive(kBarPlanes + slot, L::kPrep + 64);
         in = next;

@@ -151,11 +151,13 @@ __global__ void __launch_bounds__(Chain<DK, NB, CL>::threads, 1) sfda_forward_f3
     }
     if (chain_end<DK, NB, CL>(smem, tmem, wait, tid)) {          // NaN for all of this CTA's results
         const float nan = __int_as_float(0x7fc00000);
+#pragma unroll 1
         for (size_t i = tid; i < (size_t)a.T * NB; i += L::threads) {
             const size_t at = (row0 + i / NB * a.H) * a.dv + c0 + i % NB;
             st_val(static_cast<T *>(a.o), at, nan);
             if (a.o_im) st_val(static_cast<T *>(a.o_im), at, nan);
         }
+#pragma unroll 1
         for (int i = tid; a.S_T && i < DK * NB; i += L::threads) a.S_T[((size_t)bh * DK + i / NB) * a.dv + c0 + i % NB] = nan;
     }
 }
