@@ -174,10 +174,15 @@ cudaError_t launch_nb(const ForwardArgs &x, cudaStream_t stream)
     return launch_clusters(sfda_forward_f32_kernel<DK, NB, CL, T>, a, dim3((unsigned)(x.B * x.H), x.d_v / NB), CL, L::threads, L::bytes, stream);
 }
 
+// A sequence of one chunk, or of up to four where the blocks have 64 columns anyway, takes blocks of 64 without a cluster: there is
+// little or nothing to share, and a cluster's start, its two meetings and the copies cost 1 to 2 us.  74 sequences, d_v = 128:
+// 14.2 -> 12.5 us at T = 16, 20.6 -> 18.9 at 48, 24.1 -> 23.0 at 64; one sequence of 16 tokens 11.8 -> 11.6; with blocks of 32 columns
+// clusters are better from two chunks on (T = 48: 16.5 us, 18.6 without).
 template <int DK, typename T>
 cudaError_t launch_typed(const ForwardArgs &x, cudaStream_t stream)
 {
-    const Blocks b = chain_blocks((long long)x.B * x.H, x.d_v);
+    Blocks b = chain_blocks((long long)x.B * x.H, x.d_v);
+    if (b.cluster > 1 && x.T <= (b.columns == 64 ? 4 * kC : kC)) b = {64, 1};
     if (b.columns == 128) return launch_nb<DK, 128, 1, T>(x, stream);
     if (b.columns == 64) return b.cluster == 2 ? launch_nb<DK, 64, 2, T>(x, stream) : launch_nb<DK, 64, 1, T>(x, stream);
     return b.cluster == 4 ? launch_nb<DK, 32, 4, T>(x, stream) : launch_nb<DK, 32, 2, T>(x, stream);
