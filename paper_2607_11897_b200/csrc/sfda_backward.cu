@@ -1584,9 +1584,11 @@ cudaError_t launch_walk(const BwdArgsDev &a, int grid, cudaStream_t stream, int 
     attr[0].val.cooperative = !kUnits && a.flags ? 1 : 0;                 // CTAs that wait for one another run together (one per SM)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if ((e = cudaLaunchKernelEx(&cfg, kern, a)) != cudaSuccess) return e;
+    e = cudaLaunchKernelEx(&cfg, kern, a);
+    const cudaError_t last = cudaGetLastError();                 // (cleared also where the launch was refused)
+    if (e != cudaSuccess) return e;
     if (launches) ++*launches;
-    return cudaGetLastError();
+    return last;
 }
 
 template <int DK, int NB, int CL, int DV, typename T>

@@ -1179,7 +1179,7 @@ __device__ __forceinline__ void chain_begin(unsigned char *smem, int tid)
 {
     using L = Chain<DK, NB, CL>;
     if (tid < 32) tm_alloc(reinterpret_cast<uint32_t *>(smem + L::slow), L::columns);
-    if (tid == 32) {
+    if (CL > 1 && tid == 32) {                                   // (without a cluster nothing uses them)
         const uint32_t bars = (uint32_t)__cvta_generic_to_shared(smem + L::bars);
         uint32_t *sent = reinterpret_cast<uint32_t *>(smem + L::sent);
         for (int i = 0; i < kSlots; ++i) {
@@ -1388,7 +1388,9 @@ cudaError_t launch_clusters(void (*kern)(Args), const Args &a, dim3 grid, int cl
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = cluster > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, a);
+    const cudaError_t launched = cudaLaunchKernelEx(&cfg, kern, a);
+    const cudaError_t last = cudaGetLastError();                 // (a refused launch is this call's error, not a later one's)
+    return launched != cudaSuccess ? launched : last;
 }
 
 }  // namespace c16
