@@ -66,11 +66,47 @@ def test_backward_of_pairs_shared_by_two_blocks(B, H, T, d_k, d_v, im):
                                           (16, 128, 128, 67), (17, 64, 128, 81), (37, 128, 128, 50), (38, 64, 64, 97)])
 def test_blocks_of_columns_in_clusters(H, d_k, d_v, T):
     """As many pairs as just fit in clusters of four or two blocks of columns, and one more (forward 32 and 74 pairs, backward
-    half as many); lengths at which ranks of the cluster make no, one or several of the tiles.  Bounds as above."""
+    half as many); lengths at which ranks of the cluster make one or several of the tiles.  Bounds as above."""
     cfg = workloads.CONFIGS[0].scaled(name="c16k", B=1, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=900 + T + H)
     inp, pairs = workloads.forward_inputs(cfg), all_pairs(cfg)
     check_forward(cfg, inp, pairs[:2] + pairs[-2:], TOL)
     check_backward(cfg, inp, upstream(cfg, T), pairs[:2] + pairs[-2:], BWD_TOL)
+
+
+@pytest.mark.parametrize("H,d_k,d_v,T,alpha", [
+    (16, 128, 128, 17, "u(0.9,1)"), (32, 64, 128, 33, "u(0.9,1)"), (37, 64, 64, 17, "u(0.9,1)"), (40, 128, 128, 16, "u(0.9,1)"),
+    (40, 128, 128, 260, "u(0.9,1)"), (20, 64, 128, 257, "u(0.9,1)"), (35, 128, 128, 270, "u(0.0,1)"), (18, 128, 128, 250, "u(0.0,1)"),
+    (40, 64, 128, 150, "u(0.0,1)"), (20, 128, 64, 200, "u(0.0,1)")])
+def test_clusters_with_few_and_with_many_tiles(H, d_k, d_v, T, alpha):
+    """One to three chunks, so that ranks of a cluster make no tile, and more than a dozen, so that every barrier of the ring is used
+    in both parities; decays too strong to divide by and zeros.  Bounds as above."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16r", B=1, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha=alpha, s0_std=0.5, seed=950 + T + H)
+    inp, pairs = workloads.forward_inputs(cfg), all_pairs(cfg)
+    if alpha.startswith("u(0.0"):
+        inp["alpha"][:, ::17, :, ::5] = 0.0
+    check_forward(cfg, inp, pairs[:2] + pairs[-2:], TOL)
+    check_backward(cfg, inp, upstream(cfg, T), pairs[:2] + pairs[-2:], BWD_TOL)
+
+
+@pytest.mark.parametrize("H,d_k,d_v", [(40, 128, 128), (35, 64, 128), (20, 128, 128), (18, 64, 128)])
+@pytest.mark.parametrize("what", ["v", "k"])
+def test_a_token_that_is_not_finite_in_a_cluster(what, H, d_k, d_v):
+    """Tiles that are made a second time, without that token: chunks before it and other pairs as in the call without it."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16q", B=1, T=230, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha="u(0.9,1)", s0_std=0.5, seed=960 + H)
+    inp, up = workloads.forward_inputs(cfg), upstream(cfg, 9)
+    run = lambda: (*run_forward(cfg, inp), run_backward(cfg, inp, up))  # noqa: E731
+    o, o_im, S_T, grads = run()
+    inp[what][0, 100, 1] = np.nan
+    p, p_im, R_T, bad = run()
+    others = np.arange(H) != 1
+    for x, y in ((o, p), (o_im, p_im)):
+        assert np.array_equal(x[0][:, others], y[0][:, others]) and np.array_equal(x[0, :96, 1], y[0, :96, 1])
+        assert np.isnan(y[0, 100:, 1]).all()
+    assert np.array_equal(S_T[0, others], R_T[0, others]) and np.isnan(R_T[0, 1]).all()
+    for name in GRADS[:6]:
+        assert np.array_equal(grads[name][0][:, others], bad[name][0][:, others]), name
+    assert np.array_equal(grads["dq"][0, :96, 1], bad["dq"][0, :96, 1]) and np.isnan(bad["dq"][0, 100:, 1]).all()
+    assert np.array_equal(grads["dS0"][0, others], bad["dS0"][0, others])
 
 
 GRADS = ("dq", "dk", "dv", "dalpha", "dtheta", "dbeta", "dS0")
