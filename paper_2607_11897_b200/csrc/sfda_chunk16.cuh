@@ -36,7 +36,20 @@ constexpr int kSlots = 4;                    // operand tiles in flight
 constexpr int kBarAux = 1, kBarFull = 2, kBarDone = 6, kBarFree = 10;   // hardware barriers; the last three: + slot
 
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+#ifdef SFDA_WS_CHAOS
+__device__ __forceinline__ void pause(uint32_t salt)              // of a warp (see chaos)
+{
+    chaos(salt);
+    __syncwarp();
+}
+#else
+__device__ __forceinline__ void pause(uint32_t) {}
+#endif
+__device__ __forceinline__ void bar_arrive(int id, int n)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+    pause(id);
+}
 
 // ---- tensor-core primitives ---------------------------------------------------------------------
 __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
@@ -1120,7 +1133,10 @@ __device__ __forceinline__ uint32_t in_cta(uint32_t addr, uint32_t rank)       /
 template <int CL>
 __device__ __forceinline__ bool cluster_wait(uint32_t bar, uint32_t parity, const Wait &w, int lane)
 {
-    if (mbar_wait(bar, parity, w)) return true;
+    if (mbar_wait(bar, parity, w)) {
+        pause(bar);
+        return true;
+    }
     if (lane < CL) asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], 1;" ::"r"(in_cta(w.flag, lane)) : "memory");
     __syncwarp();
     return false;
@@ -1131,6 +1147,7 @@ __device__ __forceinline__ void warp_arrive(uint32_t bar, uint32_t rank, int lan
     __syncwarp();
     if (lane == 0) asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(in_cta(bar, rank)) : "memory");
     __syncwarp();
+    pause(bar + rank);
 }
 // `bytes` from this CTA's shared memory to the same place in another's, counted by the barrier there
 __device__ __forceinline__ void copy_to_cta(uint32_t from, uint32_t bytes, uint32_t bar, uint32_t rank)

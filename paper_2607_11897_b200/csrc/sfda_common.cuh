@@ -43,4 +43,18 @@ __device__ __forceinline__ void turns_to_cos_sin(uint32_t turns, float *c, float
 // cumulative sums over a chunk stay small enough that differences of two of them keep fp32 precision.
 __device__ __forceinline__ float log_decay(float alpha) { return fmaxf(logf(alpha), -30.0f); }
 
+// Development builds only (-DSFDA_WS_CHAOS): a pseudo-random pause of 0.1 to 1.1 us after one in eight barrier
+// arrivals and completed waits.  The results do not depend on timing, so a build with the pauses must reproduce
+// the plain build bit for bit; an ordering hazard between the roles shows as a difference.
+#ifdef SFDA_WS_CHAOS
+__device__ __forceinline__ void chaos(uint32_t salt)
+{
+    uint32_t x = (uint32_t)clock() * 2654435761u + salt * 40503u + (threadIdx.x >> 5) * 9176u;
+    x ^= x >> 13; x *= 0x5bd1e995u; x ^= x >> 15;
+    if ((x & 7u) == 0u) __nanosleep(100u + ((x >> 8) & 1023u));
+}
+#else
+__device__ __forceinline__ void chaos(uint32_t) {}
+#endif
+
 }  // namespace sfda

@@ -256,19 +256,6 @@ __device__ __forceinline__ ChunkInfo ring_get(const Misc &mi, int j)
 
 static_assert(sizeof(ChunkCursor) == 48, "the cursor is handed over as three 16-byte words");
 
-// Development builds only (-DSFDA_WS_CHAOS): a pseudo-random pause of 0.1 to 1.1 us after one in eight barrier
-// arrivals and completed waits.  The results do not depend on timing, so a build with the pauses must reproduce
-// the plain build bit for bit; an ordering hazard between the roles shows as a difference.
-#ifdef SFDA_WS_CHAOS
-__device__ __forceinline__ void chaos(uint32_t salt)
-{
-    uint32_t x = (uint32_t)clock() * 2654435761u + salt * 40503u + (threadIdx.x >> 5) * 9176u;
-    x ^= x >> 13; x *= 0x5bd1e995u; x ^= x >> 15;
-    if ((x & 7u) == 0u) __nanosleep(100u + ((x >> 8) & 1023u));
-}
-#else
-__device__ __forceinline__ void chaos(uint32_t) {}
-#endif
 __device__ __forceinline__ void mbar_arrive(unsigned long long *bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");

@@ -350,18 +350,40 @@ def all_nan(*tensors):
 
 
 @pytest.fixture
-def withheld(monkeypatch):
-    """Runs a function on the development build with some of the arrivals withheld, so that waits run out after 2^18 ticks."""
+def perturbed(monkeypatch):
+    """Runs a function on the development build, whose roles pause for 0.1 to 1.1 us after one in eight arrivals and waits."""
     from paper_2607_11897_b200 import binding, build as cuda_build
     dev, plain = binding.load_library(cuda_build.build_variant("chaos", ["-DSFDA_WS_CHAOS"])), binding.load()
 
     def run(fn):
         with monkeypatch.context() as m:
-            m.setenv("SFDA_WITHHOLD", "1")
             m.setattr(binding, "_LIB", dev)
             return fn()
     assert binding.load() is plain
     return run
+
+
+@pytest.fixture
+def withheld(perturbed, monkeypatch):
+    """Runs a function on the development build with some of the arrivals withheld, so that waits run out after 2^18 ticks."""
+    def run(fn):
+        with monkeypatch.context() as m:
+            m.setenv("SFDA_WITHHOLD", "1")
+            return perturbed(fn)
+    return run
+
+
+@pytest.mark.parametrize("H,T,d_k,d_v,alpha", [(2, 333, 128, 128, "u(0.9,1)"), (35, 200, 64, 128, "u(0.3,1)"), (20, 260, 128, 128, "u(0.9,1)"),
+                                               (60, 150, 128, 64, "u(0.0,1)"), (5, 400, 64, 64, "u(0.9,1)"), (160, 130, 128, 128, "u(0.9,1)")])
+def test_results_do_not_depend_on_the_timing_of_the_roles(perturbed, H, T, d_k, d_v, alpha):
+    """Tiles handed from CTA to CTA of a cluster and from role to role, places given back: bit for bit as without the pauses."""
+    cfg = workloads.CONFIGS[0].scaled(name="c16t", B=1, T=T, H=H, d_k=d_k, d_v=d_v, chunk=64, alpha=alpha, s0_std=0.5, seed=970 + H)
+    inp, up = workloads.forward_inputs(cfg), upstream(cfg, 11)
+    run = lambda: (*run_forward(cfg, inp), *run_backward(cfg, inp, up).values())  # noqa: E731
+    want = run()
+    for _ in range(2):
+        for x, y in zip(perturbed(run), want):
+            assert np.array_equal(x, y)
 
 
 @pytest.mark.parametrize("H,T,d_k,d_v", [(2, 64, 128, 128), (2, 81, 128, 128), (2, 200, 64, 64), (40, 200, 128, 128)])
