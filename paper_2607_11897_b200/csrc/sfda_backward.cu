@@ -26,8 +26,9 @@
 // unit of its own.  The CHAIN warps leave S_0, U, G_C, Bc of a chunk in a scratch ring as the operand registers of the
 // gradients' products.  PREP warps prepare the chunks' operand tiles and stage what the gradients need of the tokens;
 // GRAD warps turn all that into gradients one chunk behind the chain.  They meet at hardware barriers, one per slot: FULL
-// (a tile is complete), DONE (the chain came back through the chunk), GFREE (G_C's place is free again); READY (the gradients are through with the slot),
-// STAGED and TAKEN (the tokens are there, and free again).
+// (a tile is complete), DONE (the chain came back through the chunk); READY (the gradients are through with the slot),
+// STAGED and TAKEN (the tokens are there, and free again).  In the units also at two barriers in shared memory, one per place
+// of G_C: GFREE (the place is free again).
 //
 // What bounds it: about 60 k cycles per 16 tokens of a pair at d_k = d_v = 128 (57 k, 12.6 k of them in the first sweep, with
 // mma.sync holding 29 % of the tensor pipe's time and issue slots 33 % used, before sums over the keys were rounded to
@@ -78,7 +79,7 @@ static_assert(256 + kBwdTargetCtas * sizeof(unsigned) <= kHeadBytes, "the flags 
 // [plane][lane] uint4; the chunk's decays and phases, 4 floats per (token, key).  Behind the slots slow_gram's scratch and four
 // or two places in turn for G_C and Bc likewise.  With two the chain that comes back waits until the gradients have used up
 // what lies there (GFREE); see ring_places.  The rotated keys and queries, which only the rare paths want, are made again there (Rotated):
-// 704 KB with four places for d_k = d_v = 128 instead of 768, of which every chunk writes and reads 176 instead of 192.
+// 704 KB (and 25 of slow_gram's scratch) with four places for d_k = d_v = 128 instead of 768, of which every chunk writes and reads 176 instead of 192.
 // Training step at the headline sizes 29.5 -> 28.2 ms, B = 4, T = 4096, H = 16: 4.43 -> 4.29 ms.
 template <int DK, int NB>
 struct BwdScratch {
@@ -89,7 +90,7 @@ struct BwdScratch {
     static constexpr size_t bytes(int places) { return (size_t)oG + (size_t)places * place; }
     static_assert(place % 256 == 0 && kHeadBytes + bytes(4) + DK * NB * 4 <= (size_t)kSeg * DK * NB * 4, "head, ring and final state must fit a pair's scratch");
 };
-// Two for the units: B = 2, T = 333, H = 4, d = 64 has 48 segments, for which the workspace has room for 60 rings instead of 42 (one
+// Two for the units: B = 2, T = 333, H = 4, d = 64 has 48 segments, for which the workspace has room for 59 rings (47 with four places, 41 before; one
 // round instead of two, 187 -> 158 us), and B = 4, T = 4096, H = 16 has its rings in 80 MB of L2 instead of 104 (4.29 -> 4.22 ms).
 // Four for the walk, whose gradients have all of the way forward to catch up in: 28.2 ms at the headline sizes, 28.8 with two.
 constexpr int ring_places(bool units) { return units ? 2 : 4; }
@@ -1548,8 +1549,9 @@ __global__ void __launch_bounds__(kGrad + kPrep + 2 * NB, 1) sfda_backward_kerne
     if (tid < 32) tm_free(tmem, L::columns);
 }
 
-// Blocks of value columns of the two chains: all of them while the (batch, head) pairs alone fill the SMs (then there is
-// only the walk with gradients, one CTA per pair); with few sequences 64 or 32.  (A fixed count rather than the
+// All value columns while the (batch, head) pairs alone fill the SMs: then there is only the walk with gradients.  Fewer with few
+// sequences: the chains by themselves, then units; how many fewer only says how large the workspace is (the chains' blocks are
+// those of chain_blocks).  (A fixed count rather than the
 // device's: the workspace size must not depend on where it is asked for.)
 int bwd_cols(int B, int H, int d_v)
 {

@@ -13,10 +13,11 @@
 // checked per chunk (a slow exact path takes over then).
 //
 // Roles in a CTA: PREP warps make the operand tiles of a chunk into a ring of shared-memory slots, SOLVE warps the two
-// Gram matrices and the inverse of the triangular system, and each CHAIN warp owns 16 value columns of the state, for
-// all keys, in the accumulator layout of m16n8 with the value channel as the row.  That layout is also the A-operand
-// layout of the next product, so a chain warp goes R = V - W^* S -> U = M R -> S = gamma_C S + Y U with no exchange
-// with other warps at all.
+// Gram matrices and the inverse of the triangular system, and each CHAIN warp owns 16 value columns of the state in the
+// accumulator layout of m16n8 with the value channel as the row.  That layout is also the A-operand layout of the next product,
+// so a chain warp that has all keys goes R = V - W^* S -> U = M R -> S = gamma_C S + Y U with no exchange with other warps at
+// all.  In blocks of 32 columns two warps have half of the keys each and exchange their parts of W^* S (and Q^* S) through
+// shared memory once per chunk.  Blocks of columns of one pair are clusters, whose CTAs make the tiles in turn for all (Chain).
 //
 // Code counts: mma.sync holds its scheduler (sfda_forward_f32.cu), so every other instruction adds to the time, and
 // unrolled code streams from the instruction caches (the first version was 93 KB for the forward).  So the operands of
@@ -1166,7 +1167,7 @@ __device__ __forceinline__ void cluster_sync() { asm volatile("barrier.cluster.a
 // had been half of what a CTA of 32 columns issued (13.4 k of 27.6 k issue cycles per chunk; mma.sync holds its scheduler
 // for 8.2 cycles, and 0.7 more for every other instruction issued meanwhile).  With 32 columns two warps share a block of
 // 16, half of the keys each (KSP), and add up their parts of the products over the keys: every scheduler has one chain
-// warp, with less work.  fp32 forward, B = 2, T = 2001, H = 16, d = 128: 457 -> 334 us (one warp per block of 16 columns 431,
+// warp, with less work.  fp32 forward, B = 2, T = 2001, H = 16, d = 128: 457 -> 334 us, 326 now (at 334: one warp per block of 16 columns 431,
 // eight PREP warps instead of four 371, the planes handed out with the rest of a tile 387).
 template <int DK, int NB, int CL>
 struct Chain {

@@ -9,7 +9,7 @@
 // over a ring of operand tiles.
 //
 // What bounds it: with few pairs the latency of the chain (B = 2, T = 2001, H = 16, d = 128, fp32: 5.0 k cycles of a chunk's 5.1 k are
-// left without any preparation), with many the schedulers' issue slots, which mma.sync holds.  334 us at those sizes (457
+// left without any preparation), with many the schedulers' issue slots, which mma.sync holds.  326 us at those sizes (457
 // while each of a pair's four CTAs prepared every chunk for itself and a warp had all keys of its 16 columns; the unrolled
 // first version 665, the CUDA-core kernel 3154); B = 1, T = 256, H = 2, d = 64: 37 us (39, 61, 201).
 #include "sfda_chunk16.cuh"
